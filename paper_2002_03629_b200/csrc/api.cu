@@ -1,6 +1,7 @@
 // C ABI of the sampler library: model construction (masking, rounding, tile
 // metadata), argument checks, kernel selection and launch, status read-back.
 #include <algorithm>
+#include <atomic>
 #include <cstdio>
 #include <cstring>
 #include <new>
@@ -168,6 +169,8 @@ int common_scratch(js_model *m, int T)
     if ((rc = dev_alloc<JsCtl>(m, &m->ctl, 1, true)) != JS_OK) return rc;
     CU_TRY(cudaHostAlloc((void **)&m->h_result, sizeof(JsCtl), cudaHostAllocMapped));
     CU_TRY(cudaHostGetDevicePointer((void **)&m->d_result, m->h_result, 0));
+    CU_TRY(cudaHostAlloc((void **)&m->h_words, sizeof(unsigned long long) * JS_MAX_CLUSTERS, cudaHostAllocMapped));
+    CU_TRY(cudaHostGetDevicePointer((void **)&m->d_words, m->h_words, 0));
     if ((rc = dev_alloc<int>(m, &m->smp_changed, 2 * (size_t)m->rows, true)) != JS_OK) return rc;
     if ((rc = dev_alloc<int>(m, &m->smp_state, 2 * (size_t)m->rows, true)) != JS_OK) return rc;
     if ((rc = dev_alloc<int>(m, &m->perm, 2 * (size_t)m->rows, true)) != JS_OK) return rc;
@@ -186,6 +189,15 @@ bool noise_kind_ok(const js_model *m, int nk)
 }
 
 const int NOT_REPORTED = -1000000;
+
+inline void cpu_relax()
+{
+#if defined(__x86_64__)
+    __builtin_ia32_pause();
+#elif defined(__aarch64__)
+    asm volatile("yield");
+#endif
+}
 
 // model-owned fields of the launch arguments; the control block is cleared if the last call left it dirty
 int prep_args(js_model *m, RunArgs &r, cudaStream_t st)
@@ -208,20 +220,67 @@ int prep_args(js_model *m, RunArgs &r, cudaStream_t st)
     if (!m->ctl_clean) CU_TRY(cudaMemsetAsync(m->ctl, 0, sizeof(JsCtl), st));
     m->ctl_clean = false;
     r.result = m->d_result;
+    r.words = m->d_words;
     m->h_result->status = NOT_REPORTED;
     return JS_OK;
 }
 
-// waits for the launch and reads what the kernel reported through mapped host memory
+// Waits for the launch and reads what the kernel reported through mapped host memory.  The kernel writes the
+// status word last, when the outputs are complete and the control block is cleared, so polling it is enough; going
+// through the driver's stream synchronisation instead costs 3.2 us more (launch + wait of an empty kernel on B200:
+// 10.1 us against 6.9 us).  The stream itself is asked now and then, for a launch that ended without reporting.
 int wait_result(js_model *m, cudaStream_t st, JsCtl &h)
 {
-    CU_TRY(cudaStreamSynchronize(st));
+    volatile int *status = &m->h_result->status;
+    for (unsigned i = 1; *status == NOT_REPORTED; ++i) {
+        if ((i & 0x3fffu) == 0) {
+            const cudaError_t e = cudaStreamQuery(st);
+            if (e == cudaErrorNotReady) continue;
+            CU_TRY(e);
+            break;
+        }
+        cpu_relax();
+    }
+    std::atomic_thread_fence(std::memory_order_acquire);
     h = *m->h_result;
     if (h.status == NOT_REPORTED) {
         snprintf(g_cuda_err, sizeof g_cuda_err, "the kernel ended without reporting");
         return JS_ERR_CUDA;
     }
     m->ctl_clean = h.status >= 0;
+    return JS_OK;
+}
+
+// The same for kernels whose clusters report one by one (cluster_report in made_driver.cuh).
+int wait_words(js_model *m, int n, cudaStream_t st, JsCtl &h)
+{
+    memset(&h, 0, sizeof h);
+    h.frontier = INT_MAX;
+    volatile unsigned long long *words = m->h_words;
+    for (int c = 0; c < n; ++c) {
+        for (unsigned i = 1; words[c] == 0; ++i) {
+            if ((i & 0x3fffu) == 0) {
+                const cudaError_t e = cudaStreamQuery(st);
+                if (e == cudaErrorNotReady) continue;
+                CU_TRY(e);
+                if (words[c] == 0) {
+                    snprintf(g_cuda_err, sizeof g_cuda_err, "the kernel ended without reporting");
+                    return JS_ERR_CUDA;
+                }
+            }
+            cpu_relax();
+        }
+        const unsigned long long w = words[c];
+        const int state = (int)(w & 3);
+        if (state == 3) h.status = JS_ERR_TIMEOUT;
+        else if (state == 2 && h.status == JS_OK) h.status = JS_NOT_CONVERGED;
+        h.iterations = std::max(h.iterations, (int)(w >> 2 & 0xfffff));
+        h.frontier = std::min(h.frontier, (int)(w >> 22 & 0xfffff));
+        h.tiles_issued += w >> 42;
+    }
+    std::atomic_thread_fence(std::memory_order_acquire);
+    h.iters_max = h.iterations;
+    m->ctl_clean = h.status >= 0;        // these kernels touch the control block only to give up
     return JS_OK;
 }
 
@@ -321,7 +380,14 @@ int run_jacobi_gs_tc(js_model *m, RunArgs &r, cudaStream_t st)
         if ((rc = wait_result(m, st, h)) != JS_OK) return rc;
         flops += (long long)h.mma_flops;
         if (h.status < 0) { fill_stats(m, h, 0); return h.status; }
-        const int any = *m->h_any;
+        // the bookkeeping kernel runs after the sweep that has just reported
+        volatile int *any_word = m->h_any;
+        for (unsigned i = 1; *any_word < 0; ++i) {
+            if ((i & 0x3fffu) == 0 && cudaStreamQuery(st) != cudaErrorNotReady) break;
+            cpu_relax();
+        }
+        std::atomic_thread_fence(std::memory_order_acquire);
+        const int any = *any_word;
         if (any < 0) {
             snprintf(g_cuda_err, sizeof g_cuda_err, "the bookkeeping kernel did not report");
             return JS_ERR_CUDA;
@@ -349,6 +415,15 @@ int run_made(js_model *m, RunArgs &r, cudaStream_t st)
     if (r.kmode == KM_JACOBI_GS && sweeps_usable(m, r)) return run_jacobi_gs_tc(m, r, st);
     int rc = prep_args(m, r, st);
     if (rc != JS_OK) return rc;
+    if (js_small_serves(m, r)) {
+        int clusters = 0;
+        const int rl = js_launch_made_small(m, r, st, &clusters);
+        if (rl != 0) return launch_failed(rl);
+        JsCtl h;
+        if ((rc = wait_words(m, clusters, st, h)) != JS_OK) return rc;
+        fill_stats(m, h, 1);
+        return h.status;
+    }
 
     int used_path = 1;
     int rc_launch;
@@ -411,6 +486,7 @@ int js_made_create(const js_made_desc *d, js_model **out)
     int rc = made_build(m, d);
     if (rc == JS_OK) rc = common_scratch(m, d->T);
     if (rc == JS_OK && js_tc_prepare(m) < 0) rc = JS_ERR_CUDA;
+    if (rc == JS_OK && js_small_prepare(m) < 0) rc = JS_ERR_CUDA;
     if (rc != JS_OK) { js_model_destroy(m); return rc; }
     *out = m;
     return JS_OK;
@@ -446,6 +522,7 @@ void js_model_destroy(js_model *m)
     if (!m) return;
     for (void *p : m->allocs) cudaFree(p);
     if (m->h_result) cudaFreeHost(m->h_result);
+    if (m->h_words) cudaFreeHost(m->h_words);
     if (m->h_nflag) cudaFreeHost(m->h_nflag);
     if (m->h_any) cudaFreeHost(m->h_any);
     if (m->ev_main) cudaEventDestroy(m->ev_main);

@@ -53,6 +53,17 @@ struct SweepDev {
     int n_stages, ring_bytes, smem_bytes, slots;
 };
 
+// Small fp32 masked MLPs (made_small.cu): how a cluster of CS CTAs shares the units, and the packed weights.
+#define SMALL_KENDS 16
+struct SmallDev {
+    int CS, cs_log2, sms;
+    int nc[JS_MAXL + 1], ncs[JS_MAXL + 1];          // own outputs per CTA and layer, row stride of the packed weights
+    int w_off[JS_MAXL + 1], b_off[JS_MAXL + 1], d_off[JS_MAXL + 1];     // float offsets inside a CTA's pack
+    int kend[JS_MAXL + 1][SMALL_KENDS];             // last live input of every block of 32 own outputs
+    int pack_floats;
+    const float *pack;                              // [CS][pack_floats]
+};
+
 // Device view of a masked-convolution stack (tensor-core kernel only).
 struct ConvDev {
     int height, width, in_ch, ch, n_conv, C, T;
@@ -68,6 +79,8 @@ struct ConvDev {
     const CUtensorMap *tmW;             // [n_conv+1] 2-D maps of the packed weights
 };
 
+#define JS_MAX_CLUSTERS 4096          // most clusters a call of the cluster kernels may have
+
 struct js_model {
     int kind = 0;                 // 0 masked MLP, 1 masked-conv stack
     int max_batch = 0;
@@ -79,6 +92,7 @@ struct js_model {
     JsCtl *ctl = nullptr;
     JsCtl *h_result = nullptr;    // pinned host memory, mapped: the kernels report here
     JsCtl *d_result = nullptr;    // the same memory as the device sees it
+    unsigned long long *h_words = nullptr, *d_words = nullptr;      // JS_MAX_CLUSTERS reports, mapped like h_result
     bool ctl_clean = false;       // the last call left the control block zeroed
     // host-buffer entry point: device staging, copy stream, "noise has arrived" word
     float *st_noise = nullptr;
@@ -95,6 +109,8 @@ struct js_model {
     int max_grid_generic = 0;
     TcDev tc{};
     int tc_ok = 0, tc_max_grid = 0;
+    SmallDev small{};
+    int small_ok = 0;
     ConvDev conv{};
     int conv_max_grid = 0;
     SweepDev sweep{};
@@ -106,6 +122,9 @@ struct js_model {
 
 int js_tc_prepare(js_model *m);
 int js_launch_made_tc(const js_model *m, const RunArgs &r, cudaStream_t stream);
+int js_small_prepare(js_model *m);
+bool js_small_serves(const js_model *m, const RunArgs &r);
+int js_launch_made_small(const js_model *m, const RunArgs &r, cudaStream_t stream, int *clusters);
 int js_conv_build(js_model *m, const js_conv_desc *d);
 int js_launch_conv_tc(const js_model *m, const RunArgs &r, cudaStream_t stream);
 int js_sweep_prepare(js_model *m);

@@ -11,6 +11,7 @@
 // iterate with fin_x final positions makes hidden units of degree <= fin_x final.
 #pragma once
 #include <limits.h>
+#include <stddef.h>
 
 #include "js_common.cuh"
 
@@ -201,9 +202,34 @@ __device__ DriverResult made_driver(E &e, int T_, const RunArgs &r)
     return res;
 }
 
-// Every CTA adds its statistics; the last one to leave copies the control block to the caller's
-// mapped host memory (so that the host needs no device-to-host copy) and zeroes it, ready for
-// the next launch (so that the host needs no memset either, unless a call ended abnormally).
+// Every CTA adds its statistics; the last one to leave zeroes the control block, ready for the next launch
+// (so that the host needs no memset, unless a call ended abnormally), and copies it to the caller's mapped
+// host memory (so that the host needs no device-to-host copy).  The status word is written last, behind a
+// system-wide fence: the host may poll it, and finds the outputs, the report and the cleared block complete.
+__device__ __forceinline__ void ctl_report(const RunArgs &r, int status)
+{
+    JsCtl *c = r.ctl;
+    // word-wise through volatile pointers: the block was written by other CTAs
+    constexpr int NW = sizeof(JsCtl) / 4;
+    unsigned w[NW];
+    volatile unsigned *cw = reinterpret_cast<volatile unsigned *>(c);
+#pragma unroll
+    for (int i = 0; i < NW; ++i) w[i] = cw[i];
+    JsCtl *o = reinterpret_cast<JsCtl *>(w);
+    const int final_status = o->abort != 0 ? JS_ERR_TIMEOUT : status;
+#pragma unroll
+    for (int i = 0; i < NW; ++i) cw[i] = 0u;
+    if (r.result) {
+        volatile unsigned *rw = reinterpret_cast<volatile unsigned *>(r.result);
+        constexpr int SW = offsetof(JsCtl, status) / 4;
+#pragma unroll
+        for (int i = 0; i < NW; ++i)
+            if (i != SW) rw[i] = w[i];
+        __threadfence_system();
+        rw[SW] = (unsigned)final_status;
+    }
+}
+
 __device__ __forceinline__ void driver_finish(const RunArgs &r, const DriverResult &res, unsigned long long issued,
                                               unsigned long long skipped, unsigned long long mma_flops = 0,
                                               unsigned long long weight_bytes = 0)
@@ -222,17 +248,24 @@ __device__ __forceinline__ void driver_finish(const RunArgs &r, const DriverResu
     __threadfence();
     if (atomicAdd(&c->exit_count, 1u) != gridDim.x - 1) return;
     __threadfence();
-    // word-wise through volatile pointers: the block was written by other CTAs
-    constexpr int NW = sizeof(JsCtl) / 4;
-    unsigned w[NW];
-    volatile unsigned *cw = reinterpret_cast<volatile unsigned *>(c);
-    for (int i = 0; i < NW; ++i) w[i] = cw[i];
-    JsCtl *o = reinterpret_cast<JsCtl *>(w);
-    o->status = o->abort != 0 ? JS_ERR_TIMEOUT : res.status;     // res.status is the same in every CTA
-    if (r.result) {
-        volatile unsigned *rw = reinterpret_cast<volatile unsigned *>(r.result);
-        for (int i = 0; i < NW; ++i) rw[i] = w[i];
-        __threadfence_system();
-    }
-    for (int i = 0; i < NW; ++i) cw[i] = 0u;
+    ctl_report(r, res.status);     // res.status is the same in every CTA
+}
+
+// Report of a cluster that solved its samples by itself (kernels without a grid-wide step): one 64-bit word in
+// mapped host memory per cluster, written when the cluster's outputs are complete; the host polls and combines
+// them (js_cluster_word / combine_words in api.cu).  No counter is shared on the device: summing up in the control
+// block and copying it out cost 4 us of fences and round trips at the end of a 15 us kernel.
+//   bits 0-1 state (1 done, 2 iteration cap reached, 3 a wait gave up), 2-21 iterations, 22-41 frontier, 42-63 tiles
+__device__ __forceinline__ void cluster_report(unsigned long long *words, int cluster, bool alive, int status,
+                                               int iterations, int frontier, unsigned tiles)
+{
+    const unsigned long long state = !alive ? 3ull : status == JS_OK ? 1ull : 2ull;
+    const unsigned long long w = state | (unsigned long long)min(iterations, 0xfffff) << 2 |
+                                 (unsigned long long)min(frontier, 0xfffff) << 22 |
+                                 (unsigned long long)min(tiles, 0x3fffffu) << 42;
+    // The cluster's outputs first (its barrier made them visible to this thread).  They lie in device memory, which
+    // the host only reaches through later work on the GPU, so the device-wide fence is the one they need; the
+    // system-wide one costs 3 us here.
+    __threadfence();
+    *reinterpret_cast<volatile unsigned long long *>(words + cluster) = w;
 }
