@@ -120,6 +120,12 @@ __device__ void gemm_phase(Smem &s, const MadeDev &m, int l, const T *Asrc, T *o
     }
 }
 
+// place in a[0] (rows of n[0] >= T values) of element i = sample * T + position
+__device__ __forceinline__ size_t a0_at(const MadeDev &m, size_t i)
+{
+    return m.n[0] == m.T ? i : i / m.T * m.n[0] + i % m.T;
+}
+
 // x = init (or zeros), a[0] = lut[x]; also clears the per-sample bookkeeping.
 template <typename T>
 __device__ void init_phase(const MadeDev &m, const RunArgs &r, const uint8_t *src)
@@ -129,7 +135,7 @@ __device__ void init_phase(const MadeDev &m, const RunArgs &r, const uint8_t *sr
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         const uint8_t v = src ? src[i] : (uint8_t)0;
         if (r.x) r.x[i] = v;
-        a0[i] = from_f32<T>(m.lut[v]);
+        a0[a0_at(m, i)] = from_f32<T>(m.lut[v]);
     }
     if (blockIdx.x == 0) {
         for (int i = threadIdx.x; i < 2 * r.batch; i += blockDim.x) {
@@ -159,7 +165,7 @@ __device__ void sample_phase(const MadeDev &m, const RunArgs &r, const float *z,
             const int xn = js_sample_binary(r.nk, z[at], r.noise[at]);
             if (xn != r.x[at]) {
                 r.x[at] = (uint8_t)xn;
-                a0[at] = from_f32<T>(m.lut[xn]);
+                a0[a0_at(m, at)] = from_f32<T>(m.lut[xn]);
                 if (flag) note_change(r, parity, b, d);
             }
         }
@@ -174,7 +180,7 @@ __device__ void sample_phase(const MadeDev &m, const RunArgs &r, const float *z,
         const int bi = js_warp_sample_cat(r.nk, z + at * C, r.noise + (r.nk == JS_NOISE_GUMBEL ? at * C : at), C, lane);
         if (lane == 0 && bi != r.x[at]) {
             r.x[at] = (uint8_t)bi;
-            a0[at] = from_f32<T>(m.lut[bi]);
+            a0[a0_at(m, at)] = from_f32<T>(m.lut[bi]);
             if (flag) note_change(r, parity, b, d);
         }
     }
@@ -189,7 +195,7 @@ __device__ void init_phase_real(const MadeDev &m, const RunArgs &r, const float 
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         const float v = src ? src[i] : 0.0f;
         if (r.xr) r.xr[i] = v;
-        a0[i] = from_f32<T>(v);
+        a0[a0_at(m, i)] = from_f32<T>(v);
     }
     if (blockIdx.x == 0) {
         for (int i = threadIdx.x; i < 2 * r.batch; i += blockDim.x) {
@@ -224,7 +230,7 @@ __device__ void sample_real_phase(const MadeDev &m, const RunArgs &r, const floa
         const float xn = fmaf(expf(z[2 * at + 1]), r.noise[at], z[2 * at]);
         const float xo = r.xr[at];
         r.xr[at] = xn;
-        a0[at] = from_f32<T>(xn);
+        a0[a0_at(m, at)] = from_f32<T>(xn);
         if (flag && !(fabsf(xn - xo) <= r.eps)) note_change(r, parity, b, d);     // a NaN difference is a change
     }
 }
@@ -331,7 +337,7 @@ __device__ void jgs_output_phase(const MadeDev &m, const RunArgs &r, int j, int 
                 const size_t at = (size_t)b * m.T + t;
                 const int xn = js_sample_binary(r.nk, z, r.noise[at]);
                 r.x[at] = (uint8_t)xn;
-                ((T *)m.a[0])[at] = from_f32<T>(m.lut[xn]);
+                ((T *)m.a[0])[a0_at(m, at)] = from_f32<T>(m.lut[xn]);
             }
         } else if (lane == 0) {
             m.logits[(size_t)b * m.n[L + 1] + unit] = z;
@@ -355,7 +361,7 @@ __device__ void jgs_commit_phase(const MadeDev &m, const RunArgs &r, int j, int 
         const int bi = js_warp_sample_cat(r.nk, m.logits + at * C, r.noise + (r.nk == JS_NOISE_GUMBEL ? at * C : at), C, lane);
         if (lane == 0) {
             r.x[at] = (uint8_t)bi;
-            ((T *)m.a[0])[at] = from_f32<T>(m.lut[bi]);
+            ((T *)m.a[0])[a0_at(m, at)] = from_f32<T>(m.lut[bi]);
         }
     }
 }
@@ -371,7 +377,7 @@ __device__ void jgs_copy_or_compare(const MadeDev &m, const RunArgs &r, bool com
             if (r.x[i] != r.x_old[i]) note_change(r, parity, (int)(i / m.T), (int)(i % m.T));
         } else {
             r.x_old[i] = r.x[i];
-            ((T *)m.a_old[0])[i] = ((const T *)m.a[0])[i];
+            ((T *)m.a_old[0])[a0_at(m, i)] = ((const T *)m.a[0])[a0_at(m, i)];
         }
     }
 }

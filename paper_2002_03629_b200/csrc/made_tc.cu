@@ -121,7 +121,7 @@ struct TcEngine {
     {
         const size_t n = (size_t)r.batch * m.T;
         __nv_bfloat16 *a0 = (__nv_bfloat16 *)m.a[0];
-        if (n % 16 == 0 && ((uintptr_t)src & 15u) == 0) {
+        if (n % 16 == 0 && m.n[0] == m.T && ((uintptr_t)src & 15u) == 0) {
             // sixteen positions per step (the buffers are 16-byte aligned)
             for (size_t i = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * 16; i < n; i += (size_t)gridDim.x * blockDim.x * 16) {
                 const uint4 xv = src ? __ldcg(reinterpret_cast<const uint4 *>(src + i)) : make_uint4(0u, 0u, 0u, 0u);
@@ -140,7 +140,7 @@ struct TcEngine {
             for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
                 const uint8_t v = src ? src[i] : (uint8_t)0;
                 if (r.x) r.x[i] = v;
-                a0[i] = __float2bfloat16_rn(m.lut[v]);
+                a0[i / m.T * m.n[0] + i % m.T] = __float2bfloat16_rn(m.lut[v]);
             }
         }
         for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < (size_t)t.n_pflags;
@@ -227,7 +227,7 @@ struct TcEngine {
             const size_t n = (size_t)live * m.T;
             for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
                 const int row = (int)(i / m.T), d = (int)(i % m.T);
-                a0[i] = __float2bfloat16_rn(m.lut[r.x[(size_t)pn[row] * m.T + d]]);
+                a0[(size_t)row * m.n[0] + d] = __float2bfloat16_rn(m.lut[r.x[(size_t)pn[row] * m.T + d]]);
             }
         }
         return barrier() ? 1 : -1;
@@ -616,17 +616,35 @@ struct TcEngine {
                 bulk_load(smem_u32(nz_row()), r.noise + at, (uint32_t)ncols * 4u, &sh.nzbar[q]);
                 bulk_load(smem_u32(xs_row()), r.x + at, (uint32_t)ncols, &sh.nzbar[q]);
             }
-        } else if (smp >= 0) {
-            // widths that are not multiples of 16: plain loads (8 positions at a time)
-            const size_t at = (size_t)smp * m.T + n0;
-            uint8_t *nz = nz_row(), *xs = xs_row();
-            for (int c = 0; c < ncols; c += 8) {
-                const float4 v0 = ld_nc_f4_now(r.noise + at + c), v1 = ld_nc_f4_now(r.noise + at + c + 4);
-                const uint2 xv = __ldcg(reinterpret_cast<const uint2 *>(r.x + at + c));
-                *reinterpret_cast<float4 *>(nz + c * 4) = v0;
-                *reinterpret_cast<float4 *>(nz + c * 4 + 16) = v1;
-                *reinterpret_cast<uint2 *>(xs + c) = xv;
+        } else {
+            // Rows that do not start on 16 bytes: the warp takes its 32 rows in turn, lane = column (coalesced whatever the
+            // length of a row), four rows' loads in flight together.
+            uint8_t *nz = staging + (size_t)(q * 32) * BIN_NZ_ROW, *xs = staging + BIN_NZ_BYTES + (size_t)(q * 32) * BIN_XS_ROW;
+#pragma unroll 1
+            for (int r0 = 0; r0 < 32; r0 += 4) {
+                float nv[4][4];
+                uint8_t xv[4][4];
+#pragma unroll
+                for (int rr = 0; rr < 4; ++rr) {
+                    const int s = __shfl_sync(0xffffffffu, smp, r0 + rr);
+                    const size_t at = (size_t)max(s, 0) * m.T + n0;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const int c = 32 * k + lane;
+                        const bool in = s >= 0 && c < ncols;
+                        nv[rr][k] = in ? __ldg(r.noise + at + c) : 0.0f;
+                        xv[rr][k] = in ? __ldcg(r.x + at + c) : (uint8_t)0;
+                    }
+                }
+#pragma unroll
+                for (int rr = 0; rr < 4; ++rr)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        *reinterpret_cast<float *>(nz + (r0 + rr) * BIN_NZ_ROW + 4 * (32 * k + lane)) = nv[rr][k];
+                        xs[(r0 + rr) * BIN_XS_ROW + 32 * k + lane] = xv[rr][k];
+                    }
             }
+            __syncwarp();
         }
     }
 
@@ -717,13 +735,22 @@ struct TcEngine {
                 bulk_store((__nv_bfloat16 *)m.a[0] + (size_t)rw * m.T + n0, smem_u32(nz), (uint32_t)ncols * 2u);
                 bulk_commit();
             }
-        } else if (changed) {
-            uint8_t *xg = r.x + (size_t)smp * m.T + n0;
-            __nv_bfloat16 *ag = (__nv_bfloat16 *)m.a[0] + (size_t)rw * m.T + n0;
-            for (int c = 0; c < ncols; c += 8) {
-                *reinterpret_cast<uint2 *>(xg + c) = *reinterpret_cast<const uint2 *>(xs + c);
-                *reinterpret_cast<uint4 *>(ag + c) = *reinterpret_cast<const uint4 *>(nz + c * 2);
+        } else {
+            // changed rows, one after the other, lane = column; the encodings' rows start on 16 bytes (n[0])
+            const uint8_t *nzw = staging + (size_t)((warp & 3) * 32) * BIN_NZ_ROW;
+            const uint8_t *xsw = staging + BIN_NZ_BYTES + (size_t)((warp & 3) * 32) * BIN_XS_ROW;
+            __syncwarp();
+            for (unsigned todo = __ballot_sync(0xffffffffu, changed); todo != 0u; todo &= todo - 1u) {
+                const int rr = __ffs((int)todo) - 1;
+                const int s = __shfl_sync(0xffffffffu, smp, rr), rwr = __shfl_sync(0xffffffffu, rw, rr);
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (32 * k + lane < ncols) r.x[(size_t)s * m.T + n0 + 32 * k + lane] = xsw[rr * BIN_XS_ROW + 32 * k + lane];
+                if (8 * lane < ncols && lane < 16)
+                    *reinterpret_cast<uint4 *>((__nv_bfloat16 *)m.a[0] + (size_t)rwr * m.n[0] + n0 + 8 * lane) =
+                        *reinterpret_cast<const uint4 *>(nzw + rr * BIN_NZ_ROW + 16 * lane);
             }
+            __syncwarp();
         }
         if (flag) {
             if (changed) raise_flag(parity, smp);
@@ -822,7 +849,7 @@ struct TcEngine {
         bool ch = false;
         if (commit && xold != bi) {
             r.x[(size_t)sample * m.T + d] = (uint8_t)bi;
-            ((__nv_bfloat16 *)m.a[0])[(size_t)row * m.T + d] = __float2bfloat16_rn(sh.lut_s[bi]);
+            ((__nv_bfloat16 *)m.a[0])[(size_t)row * m.n[0] + d] = __float2bfloat16_rn(sh.lut_s[bi]);
             ch = true;
         }
         if (flag && ch) {
@@ -902,7 +929,7 @@ struct TcEngine {
         bool ch = false;
         if (commit && xold != bi) {
             r.x[(size_t)sample * m.T + d] = (uint8_t)bi;
-            ((__nv_bfloat16 *)m.a[0])[(size_t)row * m.T + d] = __float2bfloat16_rn(sh.lut_s[bi]);
+            ((__nv_bfloat16 *)m.a[0])[(size_t)row * m.n[0] + d] = __float2bfloat16_rn(sh.lut_s[bi]);
             ch = true;
         }
         if (flag && ch) {
