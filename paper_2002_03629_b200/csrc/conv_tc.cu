@@ -25,9 +25,8 @@ constexpr int BM = TC_BM, BK = TC_BK;
 constexpr int NTH = 320;          // warp 0 loads, warp 1 MMA, warps 2-9 epilogue: two per tensor-memory lane quadrant
 constexpr int ACC_COLS = 256;
 constexpr int A_BYTES = BM * BK * 2;
-constexpr int STAGE_BYTES = A_BYTES + 256 * BK * 2;   // A tile + up to 256 weight rows
-constexpr int N_STAGES = 3;
-constexpr int RING_BYTES = N_STAGES * STAGE_BYTES;    // 144 KB
+constexpr int RING_BYTES = 144 * 1024;                // cut anew for every layer: A tile + up to 256 weight rows per stage
+constexpr int MAX_STAGES = 6;                         // 64 weight rows: 24 KB; 128: 32 KB, 4 stages; 256: 48 KB, 3 stages
 constexpr int STAGING_BYTES = 32 * 1024;
 constexpr int SMEM_BYTES = RING_BYTES + STAGING_BYTES + 1024;
 constexpr int MAX_IMAGES = 256;
@@ -38,12 +37,8 @@ enum { EPI_HIDDEN = 0, EPI_LOGITS = 1, EPI_CAT = 3 };
 // the working set - the view a one-row block has in Algorithm 2.
 enum { SRC_NEW = 0, SRC_OLD = 1, SRC_MIXED = 2 };
 
-// the five taps a causal 3x3 kernel keeps, in the order the packed weights use
-__device__ __constant__ int c_tap_ky[5] = {0, 0, 0, 1, 1};
-__device__ __constant__ int c_tap_kx[5] = {0, 1, 2, 0, 1};
-
 struct ConvShared {
-    uint64_t full[N_STAGES], empty[N_STAGES], tfull[2], tempty[2];
+    uint64_t full[MAX_STAGES], empty[MAX_STAGES], tfull[2], tempty[2];
     uint32_t tmem_base;
     float bias_s[4][256];
     float xbest[2][4][32];    // head: the upper class half's best score and class, by tile parity and quadrant
@@ -64,7 +59,8 @@ struct ConvEngine {
     unsigned long long issued = 0, skipped = 0, mma_flops = 0, weight_bytes = 0;
     int warp, lane;
     int stage = 0;
-    uint32_t sphase = 0;
+    uint32_t spar = 0;             // bit s: parity of the next use of ring stage s
+    int cur_stages = 1, cur_stage_bytes = 0;      // ring geometry of the current layer
     int acc = 0;
     uint32_t aphase = 0;
     bool dead = false;
@@ -146,11 +142,20 @@ struct ConvEngine {
         return 0;
     }
 
-    __device__ uint8_t *stage_a(int s) const { return ring + (size_t)s * STAGE_BYTES; }
-    __device__ uint8_t *stage_b(int s) const { return ring + (size_t)s * STAGE_BYTES + A_BYTES; }
+    // The ring is cut anew for every layer (it is drained at every phase boundary, and the parity of a stage's
+    // barriers is kept per stage).
+    __device__ void ring_for_width(int bn)
+    {
+        cur_stage_bytes = A_BYTES + bn * BK * 2;
+        cur_stages = min(MAX_STAGES, RING_BYTES / cur_stage_bytes);
+        stage = 0;
+    }
+    __device__ uint8_t *stage_a(int s) const { return ring + (size_t)s * cur_stage_bytes; }
+    __device__ uint8_t *stage_b(int s) const { return ring + (size_t)s * cur_stage_bytes + A_BYTES; }
     __device__ void advance_stage()
     {
-        if (++stage == N_STAGES) { stage = 0; sphase ^= 1u; }
+        spar ^= 1u << stage;
+        if (++stage == cur_stages) stage = 0;
     }
     __device__ void advance_acc()
     {
@@ -196,22 +201,27 @@ struct ConvEngine {
         const int bn = head ? 256 : m.ch;
         const CUtensorMap *ma_new = m.tmAct + l, *ma_old = m.tmActOld + l, *mw = m.tmW + l;
         const uint32_t bytes = A_BYTES + bn * BK * 2;
-        const int kcs = head ? m.ch / BK : m.cin_pad[l] / BK;
-        trace(0);
+        const int kcs = head ? m.ch / BK : m.cin_pad[l] / BK, kcs_log2 = kcs == 2 ? 1 : 0;       // 64 or 128 channels
+        const int nkb = kblocks(l);
+        ring_for_width(bn);
+        if (lane == 0) trace(0);
         for (int id = blockIdx.x; id < ntiles && !dead; id += gridDim.x) {
             int n, yt, c;
             locate(id, nyl, yt_lo, per, n, yt, c);
             const int y0 = yt * m.R;
-            const int ntaps = head ? 1 : 5;
-            for (int tap = 0; tap < ntaps && !dead; ++tap) {
-                const int dy = head ? 0 : c_tap_ky[tap] - 1, dx = head ? 0 : c_tap_kx[tap] - 1;
-                const CUtensorMap *ma = (src == SRC_OLD || (src == SRC_MIXED && dy < 0)) ? ma_old : ma_new;
-                for (int kc = 0; kc < kcs; ++kc) {
-                    if (!mbar_wait(&sh.empty[stage], sphase ^ 1u, r.ctl)) { dead = true; break; }
-                    mbar_expect_tx(&sh.full[stage], bytes);
-                    tma_load_4d(smem_u32(stage_a(stage)), ma, &sh.full[stage], kc * BK, dx, y0 + dy, n);
-                    tma_load_2d(smem_u32(stage_b(stage)), mw, &sh.full[stage], kc * BK,
-                                head ? c * 256 : tap * m.ch);
+            for (int kb = 0; kb < nkb;) {
+                const int run = mbar_wait_run(sh.empty, stage, cur_stages, ~spar, nkb - kb, r.ctl);
+                if (run == 0) { dead = true; break; }
+                for (int i = 0; i < run; ++i, ++kb) {
+                    const int tap = kb >> kcs_log2, kc = kb & (kcs - 1);
+                    // taps in the order of the packed weights: the three of the row above, then left and centre
+                    const int dy = head || tap >= 3 ? 0 : -1, dx = head ? 0 : tap >= 3 ? tap - 4 : tap - 1;
+                    const CUtensorMap *ma = (src == SRC_OLD || (src == SRC_MIXED && dy < 0)) ? ma_old : ma_new;
+                    if (elect_one()) {
+                        mbar_expect_tx(&sh.full[stage], bytes);
+                        tma_load_4d(smem_u32(stage_a(stage)), ma, &sh.full[stage], kc * BK, dx, y0 + dy, n);
+                        tma_load_2d(smem_u32(stage_b(stage)), mw, &sh.full[stage], kc * BK, head ? c * 256 : tap * m.ch);
+                    }
                     advance_stage();
                 }
             }
@@ -223,28 +233,36 @@ struct ConvEngine {
         const bool head = (l == m.n_conv);
         const uint32_t idesc = instr_desc_bf16(head ? 256 : m.ch);
         const int nkb = kblocks(l);
+        ring_for_width(head ? 256 : m.ch);
+        bool first = true;
         for (int id = blockIdx.x; id < ntiles && !dead; id += gridDim.x) {
-            if (!mbar_wait(&sh.tempty[acc], aphase ^ 1u, r.ctl)) { dead = true; break; }
+            if (!__all_sync(0xffffffffu, mbar_wait(&sh.tempty[acc], aphase ^ 1u, r.ctl))) { dead = true; break; }
             tc_fence_after();
             const uint32_t d_tmem = tmem_base + (uint32_t)(acc * ACC_COLS);
-            for (int kb = 0; kb < nkb; ++kb) {
-                if (!mbar_wait(&sh.full[stage], sphase, r.ctl)) { dead = true; break; }
+            for (int kb = 0; kb < nkb;) {
+                const int run = mbar_wait_run(sh.full, stage, cur_stages, spar, nkb - kb, r.ctl);
+                if (run == 0) { dead = true; break; }
                 tc_fence_after();
-                if (kb == 0 && id == (int)blockIdx.x) trace(1);
-                const uint64_t adesc = smem_desc_sw128(smem_u32(stage_a(stage)));
-                const uint64_t bdesc = smem_desc_sw128(smem_u32(stage_b(stage)));
+                if (first && lane == 0) trace(1);
+                first = false;
+                for (int i = 0; i < run; ++i, ++kb) {
+                    const uint64_t adesc = smem_desc_sw128(smem_u32(stage_a(stage)));
+                    const uint64_t bdesc = smem_desc_sw128(smem_u32(stage_b(stage)));
+                    if (elect_one()) {
 #pragma unroll
-                for (int k = 0; k < BK / 16; ++k)
-                    umma_bf16(d_tmem, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), idesc,
-                              (kb > 0 || k > 0) ? 1u : 0u);
-                umma_commit(&sh.empty[stage]);
-                advance_stage();
+                        for (int k = 0; k < BK / 16; ++k)
+                            umma_bf16(d_tmem, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), idesc,
+                                      (kb > 0 || k > 0) ? 1u : 0u);
+                        umma_commit(&sh.empty[stage]);
+                    }
+                    advance_stage();
+                }
             }
             if (dead) break;
-            umma_commit(&sh.tfull[acc]);
+            if (elect_one()) umma_commit(&sh.tfull[acc]);
             advance_acc();
         }
-        trace(2);
+        if (lane == 0) trace(2);
     }
 
     __device__ void release_acc()
@@ -490,9 +508,9 @@ struct ConvEngine {
         if (ntiles == 0) return false;
         phase_no++;
         if (warp == 0) {
-            if (lane == 0) producer(l, yt_lo, nyl, ntiles, src);
+            producer(l, yt_lo, nyl, ntiles, src);
         } else if (warp == 1) {
-            if (lane == 0) mma_issuer(l, ntiles);
+            mma_issuer(l, ntiles);
         } else {
             epilogue(l, kind, w, flag, parity, zout, yt_lo, nyl, ntiles, src);
         }
@@ -577,7 +595,7 @@ conv_tc_kernel(const __grid_constant__ ConvDev m, const __grid_constant__ RunArg
     uint8_t *ring = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const int warp = threadIdx.x >> 5;
     if (threadIdx.x == 0) {
-        for (int s = 0; s < N_STAGES; ++s) { mbar_init(&sh.full[s], 1); mbar_init(&sh.empty[s], 1); }
+        for (int s = 0; s < MAX_STAGES; ++s) { mbar_init(&sh.full[s], 1); mbar_init(&sh.empty[s], 1); }
         for (int a = 0; a < 2; ++a) { mbar_init(&sh.tfull[a], 1); mbar_init(&sh.tempty[a], 8); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async();

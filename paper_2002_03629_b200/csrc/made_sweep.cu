@@ -255,11 +255,49 @@ struct SweepEngine {
 
     __device__ uint8_t *stage_a(int s) const { return ring + (size_t)s * STAGE_BYTES; }
     __device__ uint8_t *stage_b(int s) const { return ring + (size_t)s * STAGE_BYTES + A_BYTES; }
-    __device__ uint32_t stage_parity() const { return (spar >> stage) & 1u; }
     __device__ void advance_stage()
     {
         spar ^= 1u << stage;
         if (++stage == sw.n_stages) stage = 0;
+    }
+
+    // K blocks [kb, kb_end) of layer l through the ring (whole warp, one elected lane issues): activations from the previous
+    // iterate below the block's start, else from the job's own buffer F, and a box of weight rows from row0 on
+    __device__ void load_blocks(int l, int kb, int kb_end, int kb_old, int rt, int slot, const CUtensorMap *mw, int row0, uint32_t bytes)
+    {
+        while (kb < kb_end) {
+            const int run = mbar_wait_run(sh.empty, stage, sw.n_stages, ~spar, kb_end - kb, r.ctl);
+            if (run == 0) { dead = true; return; }
+            for (int i = 0; i < run; ++i, ++kb) {
+                if (elect_one()) {
+                    mbar_expect_tx(&sh.full[stage], bytes);
+                    if (kb < kb_old) tma_load_2d(smem_u32(stage_a(stage)), sw.tmAold + l, &sh.full[stage], kb * BK, rt * BM);
+                    else tma_load_3d(smem_u32(stage_a(stage)), sw.tmF + l, &sh.full[stage], (kb - kb_old) * BK, 0, slot);
+                    tma_load_2d(smem_u32(stage_b(stage)), mw, &sh.full[stage], kb * BK, row0);
+                }
+                advance_stage();
+            }
+        }
+    }
+    // the MMAs of n K blocks into the accumulator d (which they start)
+    __device__ void mma_blocks(int n, uint32_t d, uint32_t idesc)
+    {
+        for (int kb = 0; kb < n;) {
+            const int run = mbar_wait_run(sh.full, stage, sw.n_stages, spar, n - kb, r.ctl);
+            if (run == 0) { dead = true; return; }
+            tc_fence_after();
+            for (int i = 0; i < run; ++i, ++kb) {
+                const uint64_t adesc = smem_desc_sw128(smem_u32(stage_a(stage)));
+                const uint64_t bdesc = smem_desc_sw128(smem_u32(stage_b(stage)));
+                if (elect_one()) {
+#pragma unroll
+                    for (int k = 0; k < BK / 16; ++k)
+                        umma_bf16(d, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), idesc, (kb > 0 || k > 0) ? 1u : 0u);
+                    umma_commit(&sh.empty[stage]);
+                }
+                advance_stage();
+            }
+        }
     }
 
     // ------------------------------------------------------------------ roles
@@ -270,10 +308,10 @@ struct SweepEngine {
         for (int t0 = a; t0 < b && !dead; t0 += sw.G) {
             const int t1 = min(t0 + sw.G, b), hi = min(t1, b - 1);
             // the previous group's activations (or the job's start values) are in F
-            if (!mbar_wait_idle(&sh.gdone, gd_par, r.ctl)) { dead = true; break; }
+            if (!__all_sync(0xffffffffu, mbar_wait_idle(&sh.gdone, gd_par, r.ctl))) { dead = true; break; }
             gd_par ^= 1u;
             fence_proxy_async();
-            trace(0);
+            if (lane == 0) trace(0);
             const int s0 = base_start(a, t0);
             if (t0 == s0) {
                 // the base GEMMs of the next GPB groups: NB units at a time over the full K blocks of the prefix
@@ -281,17 +319,7 @@ struct SweepEngine {
                     const Base bs = base_of(l, s0, b);
                     for (int c = 0; c * NB < bs.nb && bs.kbs > 0 && !dead; ++c) {
                         mma_flops += 2ull * BM * BK * NB * (unsigned long long)bs.kbs;
-                        for (int kb = 0; kb < bs.kbs; ++kb) {
-                            if (!mbar_wait(&sh.empty[stage], stage_parity() ^ 1u, r.ctl)) { dead = true; break; }
-                            mbar_expect_tx(&sh.full[stage], A_BYTES + NB * BK * 2);
-                            if (kb < kb_old[l])
-                                tma_load_2d(smem_u32(stage_a(stage)), sw.tmAold + l, &sh.full[stage], kb * BK, rt * BM);
-                            else
-                                tma_load_3d(smem_u32(stage_a(stage)), sw.tmF + l, &sh.full[stage], (kb - kb_old[l]) * BK, 0, slot);
-                            tma_load_2d(smem_u32(stage_b(stage)), sw.tmW16 + 2 * (m.L + 1) + l, &sh.full[stage], kb * BK,
-                                        bs.ub0 + c * NB);
-                            advance_stage();
-                        }
+                        load_blocks(l, 0, bs.kbs, kb_old[l], rt, slot, sw.tmW16 + 2 * (m.L + 1) + l, bs.ub0 + c * NB, A_BYTES + NB * BK * 2);
                     }
                 }
             }
@@ -301,18 +329,8 @@ struct SweepEngine {
                 const uint32_t bytes = A_BYTES + (uint32_t)g.npad * BK * 2;
                 const int kbs = base_of(l, s0, b).kbs;
                 mma_flops += 2ull * BM * BK * (unsigned long long)g.npad * (unsigned long long)(g.kb_n - kbs);
-                for (int kb = kbs; kb < g.kb_n; ++kb) {
-                    if (!mbar_wait(&sh.empty[stage], stage_parity() ^ 1u, r.ctl)) { dead = true; break; }
-                    mbar_expect_tx(&sh.full[stage], bytes);
-                    if (kb < kb_old[l])
-                        tma_load_2d(smem_u32(stage_a(stage)), sw.tmAold + l, &sh.full[stage], kb * BK, rt * BM);
-                    else
-                        tma_load_3d(smem_u32(stage_a(stage)), sw.tmF + l, &sh.full[stage], (kb - kb_old[l]) * BK, 0, slot);
-                    // one box of 16 or of 32 weight rows (a load per 16 rows cost a fifth of the K loop)
-                    tma_load_2d(smem_u32(stage_b(stage)), sw.tmW16 + (g.npad == 32 ? m.L + 1 : 0) + l, &sh.full[stage],
-                                kb * BK, g.u0);
-                    advance_stage();
-                }
+                // one box of 16 or of 32 weight rows (a load per 16 rows cost a fifth of the K loop)
+                load_blocks(l, kbs, g.kb_n, kb_old[l], rt, slot, sw.tmW16 + (g.npad == 32 ? m.L + 1 : 0) + l, g.u0, bytes);
             }
             group_no++;
         }
@@ -323,7 +341,7 @@ struct SweepEngine {
         for (int t0 = a; t0 < b && !dead; t0 += sw.G) {
             const int t1 = min(t0 + sw.G, b), hi = min(t1, b - 1);
             // the epilogue has read the previous group's accumulators
-            if (!mbar_wait_idle(&sh.tempty, te_par ^ 1u, r.ctl)) { dead = true; break; }
+            if (!__all_sync(0xffffffffu, mbar_wait_idle(&sh.tempty, te_par ^ 1u, r.ctl))) { dead = true; break; }
             te_par ^= 1u;
             tc_fence_after();
             bool any = false;
@@ -334,23 +352,12 @@ struct SweepEngine {
                     const Base bs = base_of(l, s0, b);
                     for (int c = 0; c * NB < bs.nb && bs.kbs > 0 && !dead; ++c) {
                         // the epilogue has copied this accumulator's previous chunk away
-                        if (!mbar_wait(&sh.bempty[bbuf], ((bb_par >> bbuf) & 1u) ^ 1u, r.ctl)) { dead = true; break; }
+                        if (!__all_sync(0xffffffffu, mbar_wait(&sh.bempty[bbuf], ((bb_par >> bbuf) & 1u) ^ 1u, r.ctl))) { dead = true; break; }
                         tc_fence_after();
                         const uint32_t d_base = tmem_base + (uint32_t)(BASE_COL + bbuf * NB);
-                        for (int kb = 0; kb < bs.kbs; ++kb) {
-                            if (!mbar_wait(&sh.full[stage], stage_parity(), r.ctl)) { dead = true; break; }
-                            tc_fence_after();
-                            const uint64_t adesc = smem_desc_sw128(smem_u32(stage_a(stage)));
-                            const uint64_t bdesc = smem_desc_sw128(smem_u32(stage_b(stage)));
-#pragma unroll
-                            for (int k = 0; k < BK / 16; ++k)
-                                umma_bf16(d_base, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), idescb,
-                                          (kb > 0 || k > 0) ? 1u : 0u);
-                            umma_commit(&sh.empty[stage]);
-                            advance_stage();
-                        }
+                        mma_blocks(bs.kbs, d_base, idescb);
                         if (dead) break;
-                        umma_commit(&sh.bfull[bbuf]);
+                        if (elect_one()) umma_commit(&sh.bfull[bbuf]);
                         bb_par ^= 1u << bbuf;
                         bbuf ^= 1;
                     }
@@ -363,24 +370,15 @@ struct SweepEngine {
                 const uint32_t idesc = instr_desc_bf16(g.npad);
                 const uint32_t d_tmem = tmem_base + (uint32_t)(l * NUP);
                 const int kbs = base_of(l, s0, b).kbs;
-                for (int kb = kbs; kb < g.kb_n; ++kb) {
-                    if (!mbar_wait(&sh.full[stage], stage_parity(), r.ctl)) { dead = true; break; }
-                    tc_fence_after();
-                    const uint64_t adesc = smem_desc_sw128(smem_u32(stage_a(stage)));
-                    const uint64_t bdesc = smem_desc_sw128(smem_u32(stage_b(stage)));
-#pragma unroll
-                    for (int k = 0; k < BK / 16; ++k)
-                        umma_bf16(d_tmem, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), idesc,
-                                  (kb > kbs || k > 0) ? 1u : 0u);
-                    umma_commit(&sh.empty[stage]);
-                    advance_stage();
-                    any = true;
-                }
+                mma_blocks(g.kb_n - kbs, d_tmem, idesc);
+                any = any || g.kb_n > kbs;
             }
             if (dead) break;
-            if (any) umma_commit(&sh.tfull);
-            else mbar_arrive(&sh.tfull);          // a group with empty prefixes (the very first positions)
-            trace(1);
+            if (elect_one()) {
+                if (any) umma_commit(&sh.tfull);
+                else mbar_arrive(&sh.tfull);      // a group with empty prefixes (the very first positions)
+                trace(1);
+            }
             group_no++;
         }
     }
@@ -773,9 +771,9 @@ made_sweep_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ Swe
         __syncthreads();
         if (sh.stop) break;
         if (warp == 0) {
-            if (e.lane == 0) e.producer(rt, blockIdx.x, a, b);
+            e.producer(rt, blockIdx.x, a, b);
         } else if (warp == 1) {
-            if (e.lane == 0) e.mma_issuer(a, b);
+            e.mma_issuer(a, b);
         } else {
             bool row_changed = false;
             e.template epilogue<LT>(rt, blockIdx.x, a, b, row_changed);

@@ -3,7 +3,7 @@
 // One persistent cooperative kernel runs the whole solver.  Every layer of the
 // masked network is a GEMM  D[128 samples x BN units] = A[128 x K] * W[BN x K]^T
 // on the 5th-generation tensor cores: operands arrive in shared memory by TMA
-// (128-byte swizzle, K-major), one elected thread issues tcgen05.mma with the
+// (128-byte swizzle, K-major), one warp issues tcgen05.mma with the
 // fp32 accumulator in tensor memory, and four epilogue warps read it back with
 // tcgen05.ld.  Masked (all-zero) K blocks beyond a tile's last live input are
 // never loaded; adding exact zeros would not change the fp32 sum, so h_t stays
@@ -251,7 +251,6 @@ struct TcEngine {
     }
     __device__ uint8_t *stage_a(int s) const { return ring + (size_t)s * cur_stage_bytes; }
     __device__ uint8_t *stage_b(int s) const { return ring + (size_t)s * cur_stage_bytes + A_BYTES; }
-    __device__ uint32_t stage_parity() const { return (spar >> stage) & 1u; }
     __device__ void advance_stage()
     {
         spar ^= 1u << stage;
@@ -320,13 +319,14 @@ struct TcEngine {
         e_end = so[blockIdx.x + 1];
     }
 
+    // (the whole warp walks the units; one elected lane issues)
     __device__ void producer(int l, int nt_lo, int nt_hi, int MT)
     {
         const TcLayer &ly = t.lay[l];
         const CUtensorMap *ma = t.tmA + l, *mw = t.tmW + l;
         const uint32_t bytes = A_BYTES + ly.bn * BK * 2;
         ring_for_layer(l);
-        trace(0);
+        if (lane == 0) trace(0);
         int e, e_end;
         unit_list(l, MT, e, e_end);
         Unit u;
@@ -334,19 +334,24 @@ struct TcEngine {
             issued++;
             mma_flops += 2ull * BM * BK * (unsigned long long)ly.bn * (unsigned long long)(u.kb1 - u.kb0);
             if (u.mt == 0) weight_bytes += 2ull * BK * (unsigned long long)ly.bn * (unsigned long long)(u.kb1 - u.kb0);
-            for (int kb = u.kb0; kb < u.kb1; ++kb) {
-                if (!mbar_wait(&sh.empty[stage], stage_parity() ^ 1u, r.ctl)) { dead = true; break; }
-                mbar_expect_tx(&sh.full[stage], bytes);
-                tma_load_2d(smem_u32(stage_a(stage)), ma, &sh.full[stage], kb * BK, u.mt * BM);
-                tma_load_2d(smem_u32(stage_b(stage)), mw, &sh.full[stage], 0, kb * ly.npad + u.nt * ly.bn);
-                advance_stage();
+            for (int kb = u.kb0; kb < u.kb1;) {
+                const int run = mbar_wait_run(sh.empty, stage, cur_stages, ~spar, u.kb1 - kb, r.ctl);
+                if (run == 0) { dead = true; break; }
+                for (int i = 0; i < run; ++i, ++kb) {
+                    if (elect_one()) {
+                        mbar_expect_tx(&sh.full[stage], bytes);
+                        tma_load_2d(smem_u32(stage_a(stage)), ma, &sh.full[stage], kb * BK, u.mt * BM);
+                        tma_load_2d(smem_u32(stage_b(stage)), mw, &sh.full[stage], 0, kb * ly.npad + u.nt * ly.bn);
+                    }
+                    advance_stage();
+                }
             }
         }
         // The next phase starts with a round trip to HBM for its first weight blocks, while every
         // CTA waits.  Ask L2 for them now: weights depend on nothing, and this thread is idle until
         // the grid barrier.  (The same tile range is assumed for the next layer; a wrong guess only
         // wastes the hint.)
-        {
+        if (lane == 0) {
             const int ln = (l == m.L) ? 0 : l + 1;
             const TcLayer &nx = t.lay[ln];
             int e2, e2_end, lo2 = 0, hi2 = nx.nt;
@@ -368,27 +373,33 @@ struct TcEngine {
         Unit u;
         bool first = true;
         while (!dead && next_unit(l, e, e_end, nt_lo, nt_hi, MT, u)) {
-            if (!mbar_wait(&sh.tempty[acc], aphase ^ 1u, r.ctl)) { dead = true; break; }
+            if (!__all_sync(0xffffffffu, mbar_wait(&sh.tempty[acc], aphase ^ 1u, r.ctl))) { dead = true; break; }
             tc_fence_after();
             const uint32_t d_tmem = tmem_base + (uint32_t)(acc * ACC_COLS);
-            for (int kb = u.kb0; kb < u.kb1; ++kb) {
-                if (!mbar_wait(&sh.full[stage], stage_parity(), r.ctl)) { dead = true; break; }
+            for (int kb = u.kb0; kb < u.kb1;) {
+                const int run = mbar_wait_run(sh.full, stage, cur_stages, spar, u.kb1 - kb, r.ctl);
+                if (run == 0) { dead = true; break; }
                 tc_fence_after();
-                if (first) { trace(1); first = false; }
-                const uint64_t adesc = smem_desc_sw128(smem_u32(stage_a(stage)));
-                const uint64_t bdesc = smem_desc_sw128(smem_u32(stage_b(stage)));
+                if (first && lane == 0) trace(1);
+                first = false;
+                for (int i = 0; i < run; ++i, ++kb) {
+                    const uint64_t adesc = smem_desc_sw128(smem_u32(stage_a(stage)));
+                    const uint64_t bdesc = smem_desc_sw128(smem_u32(stage_b(stage)));
+                    if (elect_one()) {
 #pragma unroll
-                for (int k = 0; k < BK / 16; ++k)       // 16 bf16 = 32 bytes per instruction along K
-                    umma_bf16(d_tmem, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), idesc,
-                              (kb > u.kb0 || k > 0) ? 1u : 0u);
-                umma_commit(&sh.empty[stage]);          // frees the stage once these MMAs have read it
-                advance_stage();
+                        for (int k = 0; k < BK / 16; ++k)       // 16 bf16 = 32 bytes per instruction along K
+                            umma_bf16(d_tmem, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), idesc,
+                                      (kb > u.kb0 || k > 0) ? 1u : 0u);
+                        umma_commit(&sh.empty[stage]);          // frees the stage once these MMAs have read it
+                    }
+                    advance_stage();
+                }
             }
             if (dead) break;
-            umma_commit(&sh.tfull[acc]);                // accumulator complete
+            if (elect_one()) umma_commit(&sh.tfull[acc]);       // accumulator complete
             advance_acc();
         }
-        trace(2);
+        if (lane == 0) trace(2);
     }
 
     // ---- partial sums.  Layout of a slot: [column / 4][128 rows] float4, written and read with
@@ -1081,9 +1092,9 @@ struct TcEngine {
         if (nlive == 0) return false;
         phase_no++;
         if (warp == 0) {
-            if (lane == 0) producer(l, nt_lo, nt_hi, MT);
+            producer(l, nt_lo, nt_hi, MT);
         } else if (warp == 1) {
-            if (lane == 0) mma_issuer(l, nt_lo, nt_hi, MT);
+            mma_issuer(l, nt_lo, nt_hi, MT);
         } else {
             epilogue(l, kind, w, flag, parity, zout, nt_lo, nt_hi, MT);
         }

@@ -37,6 +37,18 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity)
         : "memory");
     return ok != 0;
 }
+__device__ __forceinline__ bool mbar_test_wait(uint64_t *bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
 __device__ __forceinline__ uint64_t global_ns()
 {
     uint64_t t;
@@ -77,6 +89,41 @@ __device__ __forceinline__ bool mbar_wait_idle(uint64_t *bar, uint32_t parity, J
     }
     atomicExch(&ctl->abort, 1);
     return false;
+}
+
+// one lane of a converged warp, known as such to the compiler (uniform operands stay in uniform registers: the four
+// MMAs of a K block take 230 cycles to issue instead of 290)
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.b32 %0, 1, 0, P;\n\t}" : "=r"(p));
+    return p != 0;
+}
+
+// Warp-wide bounded wait on a ring of mbarriers: how many stages from `stage` on, one after the other and at most
+// `most`, have completed the phase whose parity bit `par` holds (bit s: stage s); 0 if the wait gave up.  Lane i looks
+// at the i-th stage.  A wait costs its thread about 150 cycles even on a barrier that completed long ago, and as much again
+// for the loop around it: with one wait per K block the MMA thread needed 525 cycles per K block for MMAs that take
+// 256 (N = 128), and the loading thread 330.  One look at all stages spreads that over the stages that are ready.
+__device__ __forceinline__ int mbar_wait_run(uint64_t *bars, int stage, int n_stages, uint32_t par, int most, JsCtl *ctl)
+{
+    const int lane = threadIdx.x & 31;
+    int s = stage + lane;
+    if (s >= n_stages) s -= n_stages;
+    const bool look = lane < n_stages && lane < most;
+    if (!look) s = 0;
+    uint64_t t0 = 0;
+    for (unsigned i = 1;; ++i) {
+        const unsigned ready = __ballot_sync(0xffffffffu, look && mbar_test_wait(&bars[s], (par >> s) & 1u));
+        const int run = __ffs((int)~ready) - 1;
+        if (run > 0) return run;
+        if ((i & 31u) == 0u) {
+            if (t0 == 0) t0 = global_ns();
+            if (__any_sync(0xffffffffu, ld_volatile_i32(&ctl->abort) != 0 || global_ns() - t0 > MBAR_WAIT_NS)) break;
+        }
+    }
+    if (lane == 0) atomicExch(&ctl->abort, 1);
+    return 0;
 }
 
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, uint64_t *bar, int c0, int c1)
