@@ -425,13 +425,14 @@ int run_made(js_model *m, RunArgs &r, cudaStream_t st)
     if (r.kmode == KM_JACOBI_GS && sweeps_usable(m, r)) return run_jacobi_gs_tc(m, r, st);
     int rc = prep_args(m, r, st);
     if (rc != JS_OK) return rc;
-    if (js_small_serves(m, r)) {
+    const bool cluster = m->opt_path == 0 && js_cluster_serves(m, r);
+    if (cluster || js_small_serves(m, r)) {
         int clusters = 0;
-        const int rl = js_launch_made_small(m, r, st, &clusters);
+        const int rl = cluster ? js_launch_made_cluster(m, r, st, &clusters) : js_launch_made_small(m, r, st, &clusters);
         if (rl != 0) return launch_failed(rl);
         JsCtl h;
         if ((rc = wait_words(m, clusters, st, h)) != JS_OK) return rc;
-        fill_stats(m, h, 1);
+        fill_stats(m, h, cluster ? 0 : 1);
         return h.status;
     }
 
@@ -496,6 +497,7 @@ int js_made_create(const js_made_desc *d, js_model **out)
     int rc = made_build(m, d);
     if (rc == JS_OK) rc = common_scratch(m, d->T);
     if (rc == JS_OK && js_tc_prepare(m) < 0) rc = JS_ERR_CUDA;
+    if (rc == JS_OK && js_cluster_prepare(m) < 0) rc = JS_ERR_CUDA;
     if (rc == JS_OK && js_small_prepare(m) < 0) rc = JS_ERR_CUDA;
     if (rc != JS_OK) { js_model_destroy(m); return rc; }
     *out = m;
@@ -632,7 +634,8 @@ int jacobi_sample_host(const js_model *cm, int batch, const float *noise_host, i
     r.block = block; r.max_iters = max_iters;
     r.x = m->st_x; r.out_iters = m->st_iters;
     // only the tensor-core kernel of the masked MLPs waits for the noise by itself
-    const bool overlap = m->kind == 0 && m->tc_ok && m->opt_path == 0 && (r.kmode == KM_JACOBI || r.kmode == KM_GS_JACOBI);
+    const bool overlap = m->kind == 0 && m->tc_ok && m->opt_path == 0 && (r.kmode == KM_JACOBI || r.kmode == KM_GS_JACOBI) &&
+                         !js_cluster_serves(m, r);
     if (overlap) {
         r.noise_ready = m->d_nflag;
         r.noise_stamp = m->n_uploads;

@@ -64,6 +64,23 @@ struct SmallDev {
     const float *pack;                              // [CS][pack_floats]
 };
 
+// Binary bf16 models on the cluster kernel (made_cluster.cu): tiles of 64 units per layer.
+#define CL_MAXL 3             // hidden layers
+#define CL_TILES 48           // tiles (and K blocks) per layer
+struct ClTiles {
+    unsigned char kbe[CL_MAXL + 1][CL_TILES];       // K blocks a tile reads
+    short dmin[CL_MAXL + 1][CL_TILES], dmax[CL_MAXL + 1][CL_TILES];
+};
+struct ClusterDev {
+    int CS, cs_log2, max_clusters;
+    int nt[CL_MAXL + 1], nkb[CL_MAXL + 1], npad[CL_MAXL + 1];
+    int own_out;                 // most output tiles of one CTA
+    int early_ok;                // encodings may be sent as soon as they are sampled
+    int n_stages;
+    ClTiles tiles;
+    const CUtensorMap *tmW;      // tile-major weights, box 64 x 64
+};
+
 // Device view of a masked-convolution stack (tensor-core kernel only).
 struct ConvDev {
     int height, width, in_ch, ch, n_conv, C, T;
@@ -109,6 +126,9 @@ struct js_model {
     int max_grid_generic = 0;
     TcDev tc{};
     int tc_ok = 0, tc_max_grid = 0;
+    const void *tc_weights[JS_MAXL + 1] = {};       // tile-major weights of the tensor-core kernels
+    ClusterDev cluster{};
+    int cluster_ok = 0;
     SmallDev small{};
     int small_ok = 0;
     ConvDev conv{};
@@ -125,6 +145,10 @@ int js_launch_made_tc(const js_model *m, const RunArgs &r, cudaStream_t stream);
 int js_small_prepare(js_model *m);
 bool js_small_serves(const js_model *m, const RunArgs &r);
 int js_launch_made_small(const js_model *m, const RunArgs &r, cudaStream_t stream, int *clusters);
+bool js_encode_map_2d(CUtensorMap *out, const void *base, int rows, int cols, int box_rows);
+int js_cluster_prepare(js_model *m);
+bool js_cluster_serves(const js_model *m, const RunArgs &r);
+int js_launch_made_cluster(const js_model *m, const RunArgs &r, cudaStream_t stream, int *clusters);
 int js_conv_build(js_model *m, const js_conv_desc *d);
 int js_launch_conv_tc(const js_model *m, const RunArgs &r, cudaStream_t stream);
 int js_sweep_prepare(js_model *m);

@@ -1219,7 +1219,7 @@ static EncodeTiledFn get_encode_fn()
 }
 
 // 2-D bf16 row-major tensor [rows][cols], box = 64 columns x box_rows rows, 128-byte swizzle
-static bool encode_map(CUtensorMap *out, const void *base, int rows, int cols, int box_rows)
+bool js_encode_map_2d(CUtensorMap *out, const void *base, int rows, int cols, int box_rows)
 {
     EncodeTiledFn fn = get_encode_fn();
     if (!fn) return false;
@@ -1312,7 +1312,7 @@ int js_tc_prepare(js_model *mo)
         const int ring_cap = t.ring_bytes + (l < L ? t.aux_bytes - STAGING_BYTES : 0);
         t.lay[l].n_stages = std::min(MAX_STAGES, ring_cap / t.lay[l].stage_bytes);
         kb_all[l] = kb;
-        if (!encode_map(&mapsA[l], v.a[l], mo->rows, K, BM)) return 0;
+        if (!js_encode_map_2d(&mapsA[l], v.a[l], mo->rows, K, BM)) return 0;
         {
             const int nkb = (K + BK - 1) / BK, npad = nt * bn;
             void *wp = nullptr;
@@ -1320,8 +1320,9 @@ int js_tc_prepare(js_model *mo)
             mo->allocs.push_back(wp);
             tile_major_weights<<<1184, 256>>>((const __nv_bfloat16 *)v.W[l], (__nv_bfloat16 *)wp, N, K, npad, nkb);
             if (cudaGetLastError() != cudaSuccess) return JS_ERR_CUDA;
+            mo->tc_weights[l] = wp;
             t.lay[l].npad = npad;
-            if (!encode_map(&mapsW[l], wp, nkb * npad, BK, bn)) return 0;
+            if (!js_encode_map_2d(&mapsW[l], wp, nkb * npad, BK, bn)) return 0;
         }
     }
     if (cudaDeviceSynchronize() != cudaSuccess) return JS_ERR_CUDA;     // the tile-major copies are complete
