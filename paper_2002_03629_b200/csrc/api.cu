@@ -73,7 +73,9 @@ int made_build(js_model *m, const js_made_desc *d)
     // Rows of activations and weights start on 16 bytes in a bf16 model (TMA needs it): widths that are not multiples
     // of 8 get padding units with zero weights and biases, whose activation is zero and which nothing reads.  Models
     // with such widths used to be left to the CUDA-core kernels (T = 729, H = 1000 x 2, batch 100: 1.6 ms a call).
-    for (int l = 0; l <= L + 1; ++l) v.n[l] = d->prec == JS_BF16 && l <= L ? (wn[l] + 7) / 8 * 8 : wn[l];
+    // In fp32 models widths become multiples of 4 for the same reason (asynchronous 16-byte copies).
+    const int unit = d->prec == JS_BF16 ? 8 : 4;
+    for (int l = 0; l <= L + 1; ++l) v.n[l] = l <= L ? (wn[l] + unit - 1) / unit * unit : wn[l];
     const size_t esz = d->prec == JS_BF16 ? 2 : 4;
 
     // degrees
@@ -448,16 +450,24 @@ int run_made(js_model *m, RunArgs &r, cudaStream_t st)
         used_path = 0;
         rc_launch = js_launch_made_tc(m, r, st);
     } else {
-        if (m->max_grid_generic <= 0) m->max_grid_generic = js_made_generic_max_grid(v.prec);
+        if (m->max_grid_generic <= 0) {
+            m->max_grid_generic = js_made_generic_max_grid(v.prec);
+            int dev = 0;
+            cudaGetDevice(&dev);
+            cudaDeviceGetAttribute(&m->sms, cudaDevAttrMultiProcessorCount, dev);
+        }
         if (m->max_grid_generic <= 0) {
             snprintf(g_cuda_err, sizeof g_cuda_err, "occupancy query failed");
             return JS_ERR_CUDA;
         }
+        // smallest tiles of the products (16 x 32); the phases that take a warp or a thread per element.  Two CTAs per SM keep
+        // the grid barrier short; the micro-steps of Jacobi-GS, a warp per inner product, want every warp they can get.
         long long tiles = 1;
         for (int l = 0; l <= v.L; ++l)
-            tiles = std::max<long long>(tiles, (long long)((r.batch + JS_GT - 1) / JS_GT) * ((v.n[l + 1] + JS_GT - 1) / JS_GT));
-        const long long elems = ((long long)r.batch * v.T * (v.C > 1 ? 32 : 1) + 255) / 256;
-        const int grid = (int)std::min<long long>(m->max_grid_generic, std::max(tiles, elems));
+            tiles = std::max<long long>(tiles, (long long)((r.batch + 15) / 16) * ((v.n[l + 1] + 31) / 32));
+        const long long elems = ((long long)r.batch * v.T * (v.C > 1 ? 32 : 1) + 127) / 128;
+        const long long most = r.kmode == KM_JACOBI_GS ? m->max_grid_generic : std::min(m->max_grid_generic, 2 * m->sms);
+        const int grid = (int)std::min<long long>(most, std::max(tiles, elems));
         rc_launch = js_launch_made_generic(v, r, std::max(grid, 1), st);
     }
     if (rc_launch != 0) return launch_failed(rc_launch);

@@ -75,6 +75,7 @@ struct ClusterDev {
     int CS, cs_log2, max_clusters;
     int nt[CL_MAXL + 1], nkb[CL_MAXL + 1], npad[CL_MAXL + 1];
     int own_out;                 // most output tiles of one CTA
+    int kblocks;                 // K blocks of weights a CTA reads per pass
     int early_ok;                // encodings may be sent as soon as they are sampled
     int n_stages;
     ClTiles tiles;
@@ -123,7 +124,7 @@ struct js_model {
     uint8_t *x_old = nullptr, *x_tmp = nullptr;
     unsigned long long *trace = nullptr;
     int opt_frontier_skip = 1, opt_seq_skip = 2, opt_spin_limit = 1 << 22, opt_path = 0, opt_compact = 1, opt_trace = 0;
-    int max_grid_generic = 0;
+    int max_grid_generic = 0, sms = 1;
     TcDev tc{};
     int tc_ok = 0, tc_max_grid = 0;
     const void *tc_weights[JS_MAXL + 1] = {};       // tile-major weights of the tensor-core kernels

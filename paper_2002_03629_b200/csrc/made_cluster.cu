@@ -799,6 +799,7 @@ int js_cluster_prepare(js_model *mo)
     c.cs_log2 = c.CS == 1 ? 0 : c.CS == 2 ? 1 : c.CS == 4 ? 2 : 3;
     c.own_out = (c.nt[v.L] + c.CS - 1) / c.CS;
     std::vector<CUtensorMap> maps(v.L + 1);
+    c.kblocks = 0;
     for (int l = 0; l <= v.L; ++l) {
         const std::vector<int> &din = mo->host_deg[l], &dout = mo->host_deg[l + 1];
         const int N = v.n[l + 1], K = v.n[l];
@@ -808,12 +809,14 @@ int js_cluster_prepare(js_model *mo)
             int ke = K;
             while (ke > 0 && !(l == v.L ? din[ke - 1] < hi : din[ke - 1] <= hi)) --ke;
             c.tiles.kbe[l][t] = (unsigned char)std::max(1, (ke + BK - 1) / BK);
+            c.kblocks += c.tiles.kbe[l][t];
             c.tiles.dmin[l][t] = (short)lo;
             c.tiles.dmax[l][t] = (short)hi;
         }
         c.npad[l] = mo->tc.lay[l].npad;
         if (!js_encode_map_2d(&maps[l], mo->tc_weights[l], c.nkb[l] * c.npad[l], BK, TM)) return 0;
     }
+    c.kblocks = (c.kblocks + c.CS - 1) / c.CS;
     // Encodings may be sent before the pass has ended everywhere if each CTA's last output tile reads hidden units of every
     // CTA, in a layer above the first: a CTA issues its MMAs in order, so all of them have then done the first layer.
     c.early_ok = v.L >= 2 && c.nt[v.L] >= c.CS ? 1 : 0;
@@ -874,7 +877,10 @@ bool js_cluster_serves(const js_model *mo, const RunArgs &r)
     int st = 0;
     const int R = cluster_rows(mo, r.batch, &st);
     if (R == 0) return false;
-    return (r.batch + R - 1) / R <= std::min(JS_MAX_CLUSTERS, mo->cluster.max_clusters);
+    // A CTA streams its share of the weights every pass, 0.22 us per K block where the ring is short of room: measured at
+    // 4 passes of T = 1936, H = 2048 x 3 (259 K blocks): 262 us against 246 us grid-wide; T = 1296, H = 2048 x 2 (150): 170
+    // against 222 us.
+    return mo->cluster.kblocks <= 230 && (r.batch + R - 1) / R <= std::min(JS_MAX_CLUSTERS, mo->cluster.max_clusters);
 }
 
 int js_launch_made_cluster(const js_model *mo, const RunArgs &r, cudaStream_t stream, int *clusters)

@@ -15,109 +15,249 @@
 
 namespace {
 
-constexpr int GT = JS_GT;      // 64x64 output tile
-constexpr int KC = 32;         // k chunk staged in shared memory
-constexpr int NTHREADS = 256;
+constexpr int KC = 32;         // inputs per step of a product
+constexpr int NTHREADS = 128;
+constexpr int ROWF = KC + 4;   // row stride in shared memory: the 16-byte pieces of eight rows lie in different banks
+constexpr int STAGES = 3;
 
 struct Smem {
-    alignas(16) float As[KC][GT + 4];       // read as float4: rows of GT + 4 floats keep every group of four on 16 bytes
-    alignas(16) float Bs[KC][GT + 4];
-    int list[4096];            // Jacobi-GS: units to evaluate in this micro-step
+    union {
+        alignas(16) float tile[STAGES][(32 + 64) * ROWF];      // activation rows, then weight rows, of a step
+        int list[4096];        // Jacobi-GS: units to evaluate in this micro-step
+    };
     int list_n;
     int wcnt[NTHREADS / 32];
 };
 
-// One 64x64 tile of  out = A[batch][K] * W[N][K]^T  over k in [0, kend).
-template <typename T>
-__device__ void gemm_tile(Smem &s, const T *A, int lda, const T *__restrict__ W, int ldw,
-                          int M, int N, int kend, int m0, int n0, float (&acc)[4][4])
+__device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+// One tile of  out = A[rows][K] * W[N][K]^T  over k in [0, kend): 8 MR rows x 16 NR columns, 128 threads of MR x NR outputs
+// (row lr + 8 i, column 4 NR warp + lc + 4 j).  Operand rows are copied as they lie in memory, 16 bytes at a time, three
+// steps of 32 inputs in flight; a thread reads four inputs of a row at once.  lr takes bits 0, 3, 4 of the lane and lc bits
+// 1, 2: a 16-byte shared-memory load whose address does not depend on bit 0, or not on bit 1, takes two cycles for a warp
+// instead of four.  Every output is one chain of fused multiply-adds over k in ascending order, whatever the tile's form.
+template <typename T, int MR, int NR>
+__device__ __forceinline__ void gemm_tile(Smem &s, const T *A, int lda, const T *__restrict__ W, int ldw, int N, int kend,
+                                          int m0, int n0, int lr, int wc, float (&acc)[MR][NR])
 {
-    const int tid = threadIdx.x;
-    const int ty = tid >> 4, tx = tid & 15;
+    constexpr int BMt = 8 * MR, BNt = 16 * NR, EPP = 16 / sizeof(T);      // values per 16-byte piece
+    constexpr int PIECES = (BMt + BNt) * KC / EPP, PER = (PIECES + NTHREADS - 1) / NTHREADS;
+    const int steps = (kend + KC - 1) / KC;
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < MR; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.0f;
-    // the operands of the next K step are fetched into registers while the current one is multiplied
-    // (the sums themselves are taken in the same order as without the prefetch)
-    constexpr int PER = (GT * KC) / NTHREADS;
-    float av[PER], bv[PER];
-    auto fetch = [&](int k0) {
+        for (int j = 0; j < NR; ++j) acc[i][j] = 0.0f;
+    // piece e of this thread at step c: its source, how many values of it lie below kend, its place in a stage
+    auto piece = [&](int e, int c, const T *&src, int &vals, int &at) {
+        const int idx = threadIdx.x + e * NTHREADS, row = idx / (KC / EPP), k = (idx % (KC / EPP)) * EPP;
+        const bool is_a = row < BMt;
+        const int n = n0 + row - BMt;
+        vals = (PIECES % NTHREADS == 0 || idx < PIECES) && (is_a || n < N) ? max(0, min(EPP, kend - (c * KC + k))) : 0;
+        src = is_a ? A + (size_t)(m0 + row) * lda : W + (size_t)(vals > 0 ? n : 0) * ldw;
+        src += vals > 0 ? c * KC + k : 0;
+        at = row * ROWF + k;
+    };
+    uint4 reg[sizeof(T) == 2 ? PER : 1];
+    auto fetch = [&](int c) {                       // fp32: asynchronous copies; bf16: into registers, converted by put()
 #pragma unroll
-        for (int it = 0; it < PER; ++it) {
-            const int idx = tid + it * NTHREADS;
-            const int kk = idx % KC, row = idx / KC;
-            const int k = k0 + kk;
-            av[it] = 0.0f;
-            bv[it] = 0.0f;
-            if (k < kend) {
-                if (m0 + row < M) av[it] = to_f32<T>(A[(size_t)(m0 + row) * lda + k]);
-                if (n0 + row < N) bv[it] = to_f32<T>(W[(size_t)(n0 + row) * ldw + k]);
+        for (int e = 0; e < PER; ++e) {
+            const T *src;
+            int vals, at;
+            piece(e, c, src, vals, at);
+            if constexpr (sizeof(T) == 4) {
+                if (PIECES % NTHREADS == 0 || threadIdx.x + e * NTHREADS < PIECES)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr(&s.tile[c % STAGES][at])), "l"(src), "r"(vals * 4)
+                                 : "memory");
+            } else {
+                reg[e] = vals > 0 ? __ldcg(reinterpret_cast<const uint4 *>(src)) : make_uint4(0, 0, 0, 0);
+            }
+        }
+        if constexpr (sizeof(T) == 4) asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    auto put = [&](int c) {
+        if constexpr (sizeof(T) == 2) {
+#pragma unroll
+            for (int e = 0; e < PER; ++e) {
+                const T *src;
+                int vals, at;
+                piece(e, c, src, vals, at);
+                if (!(PIECES % NTHREADS == 0 || threadIdx.x + e * NTHREADS < PIECES)) continue;
+                const uint32_t w[4] = {reg[e].x, reg[e].y, reg[e].z, reg[e].w};
+                float v[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) v[i] = i < vals ? __uint_as_float((i & 1) ? (w[i / 2] & 0xffff0000u) : (w[i / 2] << 16)) : 0.0f;
+                float4 *dst = reinterpret_cast<float4 *>(&s.tile[c % STAGES][at]);
+                dst[0] = make_float4(v[0], v[1], v[2], v[3]);
+                dst[1] = make_float4(v[4], v[5], v[6], v[7]);
             }
         }
     };
-    if (kend > 0) fetch(0);
-    for (int k0 = 0; k0 < kend; k0 += KC) {
-#pragma unroll
-        for (int it = 0; it < PER; ++it) {
-            const int idx = tid + it * NTHREADS;
-            const int kk = idx % KC, row = idx / KC;
-            s.As[kk][row] = av[it];
-            s.Bs[kk][row] = bv[it];
+    __syncthreads();                                // the stages are free
+    if constexpr (sizeof(T) == 4) {
+        for (int c = 0; c < STAGES - 1; ++c) {
+            if (c < steps) fetch(c);
+            else asm volatile("cp.async.commit_group;" ::: "memory");
         }
+    } else if (steps > 0) {
+        fetch(0);
+    }
+    for (int c = 0; c < steps; ++c) {
+        if constexpr (sizeof(T) == 4) asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
+        else put(c);
         __syncthreads();
-        if (k0 + KC < kend) fetch(k0 + KC);
-#pragma unroll 8
-        for (int kk = 0; kk < KC; ++kk) {
-            // (rows of As / Bs are GT + 4 floats: every row and every group of four starts on 16 bytes)
-            const float4 a4 = *reinterpret_cast<const float4 *>(&s.As[kk][ty * 4]);
-            const float4 b4 = *reinterpret_cast<const float4 *>(&s.Bs[kk][tx * 4]);
-            const float a[4] = {a4.x, a4.y, a4.z, a4.w}, b[4] = {b4.x, b4.y, b4.z, b4.w};
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+        if constexpr (sizeof(T) == 4) {
+            if (c + STAGES - 1 < steps) fetch(c + STAGES - 1);
+            else asm volatile("cp.async.commit_group;" ::: "memory");
+        } else if (c + 1 < steps) {
+            fetch(c + 1);
         }
-        __syncthreads();
+        const float *ta = &s.tile[c % STAGES][lr * ROWF], *tb = &s.tile[c % STAGES][(BMt + wc) * ROWF];
+#pragma unroll
+        for (int k = 0; k < KC; k += 4) {
+            float4 a[MR], b[NR];
+#pragma unroll
+            for (int i = 0; i < MR; ++i) a[i] = *reinterpret_cast<const float4 *>(ta + 8 * i * ROWF + k);
+#pragma unroll
+            for (int j = 0; j < NR; ++j) b[j] = *reinterpret_cast<const float4 *>(tb + 4 * j * ROWF + k);
+#pragma unroll
+            for (int i = 0; i < MR; ++i)
+#pragma unroll
+                for (int j = 0; j < NR; ++j) acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
+#pragma unroll
+            for (int i = 0; i < MR; ++i)
+#pragma unroll
+                for (int j = 0; j < NR; ++j) acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
+#pragma unroll
+            for (int i = 0; i < MR; ++i)
+#pragma unroll
+                for (int j = 0; j < NR; ++j) acc[i][j] = fmaf(a[i].z, b[j].z, acc[i][j]);
+#pragma unroll
+            for (int i = 0; i < MR; ++i)
+#pragma unroll
+                for (int j = 0; j < NR; ++j) acc[i][j] = fmaf(a[i].w, b[j].w, acc[i][j]);
+        }
     }
 }
 
-// Layer l over the window: hidden layers store act(pre) into `out`; the output
-// layer (l == L) stores fp32 logits into `zout` [batch][T*C].
-template <typename T>
-__device__ void gemm_phase(Smem &s, const MadeDev &m, int l, const T *Asrc, T *out, float *zout, int batch,
-                           const Win &w, unsigned long long &issued, unsigned long long &skipped)
+__device__ __forceinline__ size_t a0_at(const MadeDev &m, size_t i);
+
+// What becomes of an output tile: logits to memory, or, with one or two outputs per position, sampled on the spot.
+struct OutArgs {
+    float *zout;               // logits [batch][T*C], or NULL: sample
+    bool flag;
+    int parity;
+};
+
+// Change flags of many positions: the per-sample word by a plain store, the batch-level words once per warp (an atomic per
+// changed position on two words for the whole batch took longer than the forward pass).
+struct Changes {
+    int first = INT_MAX;
+    __device__ __forceinline__ void note(const RunArgs &r, int parity, int b, int d)
+    {
+        r.smp_changed[parity * r.batch + b] = 1;
+        first = min(first, d);
+    }
+    __device__ __forceinline__ void flush(const RunArgs &r, int parity)
+    {
+        const int f = __reduce_min_sync(0xffffffffu, first);
+        if (f != INT_MAX && (threadIdx.x & 31) == 0) {
+            atomicMin(&r.ctl->agg_minfirst[parity], f);
+            atomicOr(&r.ctl->agg_any[parity], 1);
+        }
+        first = INT_MAX;
+    }
+};
+
+// Layer l over the window in tiles of one form, longest inner products first, dealt to the CTAs back and forth.
+template <typename T, int MR, int NR>
+__device__ void gemm_tiles(Smem &s, const MadeDev &m, const RunArgs &r, int l, const T *Asrc, T *out, const OutArgs &oa, const Win &w,
+                           unsigned long long &issued, unsigned long long &skipped)
 {
-    const int N = m.n[l + 1], K = m.n[l];
-    const int mt = (batch + GT - 1) / GT, nt = (N + GT - 1) / GT;
+    constexpr int BMt = 8 * MR, BNt = 16 * NR;
+    const int N = m.n[l + 1], K = m.n[l], batch = r.batch;
+    const int mt = (batch + BMt - 1) / BMt, nt = (N + BNt - 1) / BNt, G = (int)gridDim.x;
     const bool is_out = (l == m.L);
-    const T *Wl = (const T *)m.W[l];
-    for (int tile = blockIdx.x; tile < mt * nt; tile += gridDim.x) {
-        const int tn = tile / mt, tm = tile % mt;
-        const int dmin = m.t_dmin[l][tn], dmax = m.t_dmax[l][tn];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lr = (lane & 1) | ((lane >> 3) << 1), wc = 4 * NR * warp + ((lane >> 1) & 3);
+    Changes chg;
+    for (int round = 0; round * G < mt * nt; ++round) {
+        const int tile = round * G + ((round & 1) ? G - 1 - (int)blockIdx.x : (int)blockIdx.x);
+        if (tile >= mt * nt) continue;
+        const int tn = nt - 1 - tile / mt, tm = tile % mt, m0 = tm * BMt, n0 = tn * BNt, meta = n0 / JS_GT;
+        const int dmin = m.t_dmin[l][meta], dmax = m.t_dmax[l][meta];
         bool live;
         if (is_out) live = (dmax - 1 >= w.olo) && (dmin - 1 < w.ohi);
         else live = (dmax > w.hdeg_lo) && (dmin <= w.hdeg_hi);
         if (!live) { if (threadIdx.x == 0) skipped++; continue; }
         if (threadIdx.x == 0) issued++;
-        float acc[4][4];
-        const int m0 = tm * GT, n0 = tn * GT;
-        gemm_tile<T>(s, Asrc, K, Wl, K, batch, N, m.t_kend[l][tn], m0, n0, acc);
-        const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
+        float acc[MR][NR];
+        gemm_tile<T, MR, NR>(s, Asrc, K, (const T *)m.W[l], K, N, m.t_kend[l][meta], m0, n0, lr, wc, acc);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int row = m0 + ty * 4 + i;
-            if (row >= batch) continue;
+        for (int i = 0; i < MR; ++i) {
+            const int row = m0 + lr + 8 * i;
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int col = n0 + tx * 4 + j;
-                if (col >= N) continue;
-                const float pre = acc[i][j] + m.bias[l][col];
-                if (is_out) zout[(size_t)row * N + col] = pre;
-                else out[(size_t)row * N + col] = from_f32<T>(js_act_fn(m.act, pre));
+            for (int j = 0; j < NR; ++j) {
+                const int col = n0 + wc + 4 * j;
+                const float pre = acc[i][j] + (col < N ? __ldg(&m.bias[l][col]) : 0.0f);
+                if (!is_out) {
+                    if (row < batch && col < N) out[(size_t)row * N + col] = from_f32<T>(js_act_fn(m.act, pre));
+                    continue;
+                }
+                if (oa.zout) {
+                    if (row < batch && col < N) oa.zout[(size_t)row * N + col] = pre;
+                    continue;
+                }
+                // Continuous states with logistic conditionals (Section 5.3.1, Appendix C.3 of arXiv 2002.03629): logit 2t is the
+                // location m_t, logit 2t+1 (the neighbouring column: lane bit 1) the log-scale l_t, and the position's
+                // reserved noise e_t = logit(u_t) gives x_t = m_t + exp(l_t) e_t (inverse CDF of the logistic law).  A position
+                // counts as changed when it moved by more than eps, so "no position changed" is the stopping rule
+                // max_t |x^k_t - x^{k-1}_t| <= eps  of Section 2.2.1 in the maximum norm.
+                const float scale = r.real ? __shfl_xor_sync(0xffffffffu, pre, 2) : 0.0f;
+                const int d = r.real ? col >> 1 : col;
+                if (row >= batch || col >= N || d < w.plo || d >= w.phi || (r.real && (col & 1))) continue;
+                const size_t at = (size_t)row * m.T + d;
+                if (r.real) {
+                    // a sample whose stopping test has fired keeps the iterate it stopped at (with eps > 0 a further
+                    // update would still move it)
+                    if (oa.flag && r.smp_state[row] != 0) continue;
+                    const float xn = fmaf(expf(scale), r.noise[at], pre), xo = r.xr[at];
+                    r.xr[at] = xn;
+                    ((T *)m.a[0])[a0_at(m, at)] = from_f32<T>(xn);
+                    if (oa.flag && !(fabsf(xn - xo) <= r.eps)) chg.note(r, oa.parity, row, d);     // a NaN difference is a change
+                } else {
+                    const int xn = js_sample_binary(r.nk, pre, r.noise[at]);
+                    if (xn != r.x[at]) {
+                        r.x[at] = (uint8_t)xn;
+                        ((T *)m.a[0])[a0_at(m, at)] = from_f32<T>(m.lut[xn]);
+                        if (oa.flag) chg.note(r, oa.parity, row, d);
+                    }
+                }
             }
         }
     }
+    if (oa.flag) chg.flush(r, oa.parity);
+}
+
+// Layer l over the window: hidden layers store act(pre) into `out`; the output layer (l == L) see OutArgs.
+// The tile's form: 32 x 64 needs the fewest shared-memory reads per multiply-add, smaller ones spread a layer over more SMs and
+// shorten its longest tile.  Estimate of a layer in cycles: its longest tile alone (issue: 18, 10, 6 cycles per input), or
+// what an SM's share of the tiles takes from shared memory (16, 12, 8 cycles per tile and input, inner products half the
+// longest on average).  Measured on 256 samples, 1024 units, 1024 inputs: 100 us per layer with the former 64 x 64 tiles
+// (staged through registers, transposed), see DESIGN for what it is now.
+template <typename T>
+__device__ void gemm_phase(Smem &s, const MadeDev &m, const RunArgs &r, int l, const T *Asrc, T *out, const OutArgs &oa, const Win &w,
+                           unsigned long long &issued, unsigned long long &skipped)
+{
+    const int N = m.n[l + 1];
+    const float sms = 148.0f;
+    auto cost = [&](int bm, int bn, float alone, float share) {
+        const float tiles = (float)((r.batch + bm - 1) / bm) * (float)((N + bn - 1) / bn);
+        return fmaxf(alone, fmaxf(1.0f, tiles / sms) * share * 0.5f);
+    };
+    const float c44 = cost(32, 64, 18.0f, 16.0f), c24 = cost(16, 64, 10.0f, 12.0f), c22 = cost(16, 32, 6.0f, 8.0f);
+    if (c22 <= c24 && c22 <= c44) gemm_tiles<T, 2, 2>(s, m, r, l, Asrc, out, oa, w, issued, skipped);
+    else if (c24 <= c44) gemm_tiles<T, 2, 4>(s, m, r, l, Asrc, out, oa, w, issued, skipped);
+    else gemm_tiles<T, 4, 4>(s, m, r, l, Asrc, out, oa, w, issued, skipped);
 }
 
 // place in a[0] (rows of n[0] >= T values) of element i = sample * T + position
@@ -149,31 +289,18 @@ __device__ void init_phase(const MadeDev &m, const RunArgs &r, const uint8_t *sr
     }
 }
 
-// Sample positions [plo, phi) of every sample from the logits scratch, compare
-// with the current iterate, store the new symbol and its encoding.
+// Sample C-way positions [plo, phi) of every sample from the logits scratch, compare with the current iterate, store the
+// new symbol and its encoding: a warp per position.
 template <typename T>
 __device__ void sample_phase(const MadeDev &m, const RunArgs &r, const float *z, int plo, int phi, bool flag,
                              int parity)
 {
     const int T_ = m.T, C = m.C, np = phi - plo;
     T *a0 = (T *)m.a[0];
-    if (C == 1) {
-        const size_t n = (size_t)r.batch * np;
-        for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-            const int b = (int)(i / np), d = plo + (int)(i % np);
-            const size_t at = (size_t)b * T_ + d;
-            const int xn = js_sample_binary(r.nk, z[at], r.noise[at]);
-            if (xn != r.x[at]) {
-                r.x[at] = (uint8_t)xn;
-                a0[a0_at(m, at)] = from_f32<T>(m.lut[xn]);
-                if (flag) note_change(r, parity, b, d);
-            }
-        }
-        return;
-    }
     const int lane = threadIdx.x & 31;
     const size_t warps = ((size_t)gridDim.x * blockDim.x) >> 5;
     const size_t n = (size_t)r.batch * np;
+    Changes chg;
     for (size_t i = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += warps) {
         const int b = (int)(i / np), d = plo + (int)(i % np);
         const size_t at = (size_t)b * T_ + d;
@@ -181,9 +308,10 @@ __device__ void sample_phase(const MadeDev &m, const RunArgs &r, const float *z,
         if (lane == 0 && bi != r.x[at]) {
             r.x[at] = (uint8_t)bi;
             a0[a0_at(m, at)] = from_f32<T>(m.lut[bi]);
-            if (flag) note_change(r, parity, b, d);
+            if (flag) chg.note(r, parity, b, d);
         }
     }
+    if (flag) chg.flush(r, parity);
 }
 
 // Continuous states: x = start values (or zeros), a[0] = x (rounded like any activation in a bf16 model).
@@ -207,44 +335,6 @@ __device__ void init_phase_real(const MadeDev &m, const RunArgs &r, const float 
             r.ctl->agg_minfirst[0] = r.ctl->agg_minfirst[1] = INT_MAX;
         }
     }
-}
-
-// Continuous states with logistic conditionals (Section 5.3.1, Appendix C.3 of arXiv 2002.03629): logit 2t
-// is the location m_t, logit 2t+1 the log-scale l_t, and the position's reserved noise e_t = logit(u_t) gives
-// x_t = m_t + exp(l_t) e_t (inverse CDF of the logistic law).  A position counts as changed when it moved by
-// more than eps, so "no position changed" is the stopping rule  max_t |x^k_t - x^{k-1}_t| <= eps  of
-// Section 2.2.1 in the maximum norm.
-template <typename T>
-__device__ void sample_real_phase(const MadeDev &m, const RunArgs &r, const float *z, int plo, int phi, bool flag,
-                                  int parity)
-{
-    const int T_ = m.T, np = phi - plo;
-    T *a0 = (T *)m.a[0];
-    const size_t n = (size_t)r.batch * np;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const int b = (int)(i / np), d = plo + (int)(i % np);
-        // a sample whose stopping test has fired keeps the iterate it stopped at (with eps > 0 a further
-        // update would still move it)
-        if (flag && r.smp_state[b] != 0) continue;
-        const size_t at = (size_t)b * T_ + d;
-        const float xn = fmaf(expf(z[2 * at + 1]), r.noise[at], z[2 * at]);
-        const float xo = r.xr[at];
-        r.xr[at] = xn;
-        a0[a0_at(m, at)] = from_f32<T>(xn);
-        if (flag && !(fabsf(xn - xo) <= r.eps)) note_change(r, parity, b, d);     // a NaN difference is a change
-    }
-}
-
-template <typename T>
-__device__ bool forward_pass(Smem &s, const MadeDev &m, const RunArgs &r, T *const *acts, float *zout, const Win &w,
-                             unsigned &epoch, unsigned long long &issued, unsigned long long &skipped)
-{
-    for (int l = 0; l <= m.L; ++l) {
-        gemm_phase<T>(s, m, l, (const T *)acts[l], l < m.L ? acts[l + 1] : (T *)nullptr, zout, r.batch, w, issued,
-                      skipped);
-        if (!grid_barrier(r.ctl, epoch, r.spin_limit)) return false;
-    }
-    return true;
 }
 
 // ---- Jacobi-GS micro-steps (Algorithm 2): warp-per-dot-product evaluation of
@@ -307,7 +397,7 @@ __device__ void jgs_hidden_phase(Smem &s, const MadeDev &m, const RunArgs &r, in
             const int unit = s.list[it / r.batch], b = (int)(it % r.batch);
             const int g = m.deg[l + 1][unit];
             const float pre = mixed_dot<T>(m, l, unit, (g - 1) / B, B, (const T *)m.a_old[l] + (size_t)b * m.n[l],
-                                           (const T *)m.a[l] + (size_t)b * m.n[l], m.t_kend[l][unit / GT]) +
+                                           (const T *)m.a[l] + (size_t)b * m.n[l], m.t_kend[l][unit / JS_GT]) +
                               m.bias[l][unit];
             if (lane == 0) ((T *)m.a[l + 1])[(size_t)b * N + unit] = from_f32<T>(js_act_fn(m.act, pre));
         }
@@ -330,7 +420,7 @@ __device__ void jgs_output_phase(const MadeDev &m, const RunArgs &r, int j, int 
         if (t >= m.T) continue;
         const int unit = t * C + c;
         const float z = mixed_dot<T>(m, L, unit, blk, B, (const T *)m.a_old[L] + (size_t)b * m.n[L],
-                                     (const T *)m.a[L] + (size_t)b * m.n[L], m.t_kend[L][unit / GT]) +
+                                     (const T *)m.a[L] + (size_t)b * m.n[L], m.t_kend[L][unit / JS_GT]) +
                         m.bias[L][unit];
         if (C == 1) {
             if (lane == 0) {
@@ -371,15 +461,17 @@ __device__ void jgs_commit_phase(const MadeDev &m, const RunArgs &r, int j, int 
 template <typename T>
 __device__ void jgs_copy_or_compare(const MadeDev &m, const RunArgs &r, bool compare, int parity)
 {
+    Changes chg;
     const size_t n = (size_t)r.batch * m.T;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         if (compare) {
-            if (r.x[i] != r.x_old[i]) note_change(r, parity, (int)(i / m.T), (int)(i % m.T));
+            if (r.x[i] != r.x_old[i]) chg.note(r, parity, (int)(i / m.T), (int)(i % m.T));
         } else {
             r.x_old[i] = r.x[i];
             ((T *)m.a_old[0])[a0_at(m, i)] = ((const T *)m.a[0])[a0_at(m, i)];
         }
     }
+    if (compare) chg.flush(r, parity);
 }
 
 // ------------------------------------------------------------------ engine
@@ -406,14 +498,19 @@ struct GenericEngine {
             init_phase<T>(m, r, src);
     }
     __device__ int compact(int) { return 0; }      // the CUDA-core path keeps the batch as it is
-    // one forward pass over the window; then either the logits go to zout (teacher forcing) or
-    // positions [w.plo, w.phi) are sampled and committed
+    // One forward pass over the window; then either the logits go to zout (teacher forcing) or positions [w.plo, w.phi) are
+    // sampled and committed: in the output tiles themselves where a position has one logit or a location and a log-scale,
+    // from the logits scratch where it has more.
     __device__ bool step(const Win &w, bool flag, int parity, float *zout)
     {
-        if (zout) return forward_pass<T>(s, m, r, acts, zout, w, epoch, issued, skipped);
-        if (!forward_pass<T>(s, m, r, acts, m.logits, w, epoch, issued, skipped)) return false;
-        if (r.real) sample_real_phase<T>(m, r, m.logits, w.plo, w.phi, flag, parity);
-        else sample_phase<T>(m, r, m.logits, w.plo, w.phi, flag, parity);
+        const bool fused = !zout && (m.C == 1 || r.real);
+        for (int l = 0; l <= m.L; ++l) {
+            const OutArgs oa = {zout ? zout : fused ? (float *)nullptr : m.logits, fused && flag && l == m.L, parity};
+            gemm_phase<T>(s, m, r, l, (const T *)acts[l], l < m.L ? acts[l + 1] : (T *)nullptr, oa, w, issued, skipped);
+            if (!barrier()) return false;
+        }
+        if (zout || fused) return true;
+        sample_phase<T>(m, r, m.logits, w.plo, w.phi, flag, parity);
         return barrier();
     }
     // one outer iteration of Algorithm 2
@@ -425,7 +522,7 @@ struct GenericEngine {
         // hidden activations of the previous outer iterate
         const Win w = make_win(fin_h, T_, T_, T_);
         for (int l = 0; l < m.L; ++l) {
-            gemm_phase<T>(s, m, l, acts_old[l], acts_old[l + 1], nullptr, r.batch, w, issued, skipped);
+            gemm_phase<T>(s, m, r, l, acts_old[l], acts_old[l + 1], OutArgs{nullptr, false, 0}, w, issued, skipped);
             if (!barrier()) return false;
         }
         const int jmax = min(B, T_);

@@ -161,7 +161,7 @@ made_small_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ Sma
             a0[t * RS + rr] = REAL ? v : v != 0.0f ? lut1 : lut0;
         }
     for (int l = 0; l <= L; ++l)                         // padding rows are multiplied by zero weights: keep them finite
-        for (int i = m.n[l] * RS + tid; i < pad_k(m.n[l]) * RS; i += NTH) sm[lo_.a[l] + i] = 0.0f;
+        for (int i = (l == 0 ? T : m.n[l]) * RS + tid; i < pad_k(m.n[l]) * RS; i += NTH) sm[lo_.a[l] + i] = 0.0f;
     for (int i = tid; i < 2 * RMAX; i += NTH) {
         sh.chg[i / RMAX][i % RMAX] = 0;
         if (i < RMAX) { sh.done[i] = 0; sh.count[i] = 0; }
