@@ -450,23 +450,18 @@ int run_made(js_model *m, RunArgs &r, cudaStream_t st)
         used_path = 0;
         rc_launch = js_launch_made_tc(m, r, st);
     } else {
-        if (m->max_grid_generic <= 0) {
-            m->max_grid_generic = js_made_generic_max_grid(v.prec);
-            int dev = 0;
-            cudaGetDevice(&dev);
-            cudaDeviceGetAttribute(&m->sms, cudaDevAttrMultiProcessorCount, dev);
-        }
-        if (m->max_grid_generic <= 0) {
+        const bool jgs = r.kmode == KM_JACOBI_GS;
+        int &most = m->max_grid_generic[jgs];
+        if (most <= 0) most = js_made_generic_max_grid(v.prec, jgs);
+        if (most <= 0) {
             snprintf(g_cuda_err, sizeof g_cuda_err, "occupancy query failed");
             return JS_ERR_CUDA;
         }
-        // smallest tiles of the products (16 x 32); the phases that take a warp or a thread per element.  Two CTAs per SM keep
-        // the grid barrier short; the micro-steps of Jacobi-GS, a warp per inner product, want every warp they can get.
+        // smallest tiles of the products (16 x 32); the phases that take a warp or a thread per element
         long long tiles = 1;
         for (int l = 0; l <= v.L; ++l)
             tiles = std::max<long long>(tiles, (long long)((r.batch + 15) / 16) * ((v.n[l + 1] + 31) / 32));
         const long long elems = ((long long)r.batch * v.T * (v.C > 1 ? 32 : 1) + 127) / 128;
-        const long long most = r.kmode == KM_JACOBI_GS ? m->max_grid_generic : std::min(m->max_grid_generic, 2 * m->sms);
         const int grid = (int)std::min<long long>(most, std::max(tiles, elems));
         rc_launch = js_launch_made_generic(v, r, std::max(grid, 1), st);
     }

@@ -222,4 +222,4 @@ template <> __device__ __forceinline__ __nv_bfloat16 from_f32<__nv_bfloat16>(flo
 
 // host-side launchers implemented by the kernel files
 int js_launch_made_generic(const MadeDev &m, const RunArgs &r, int grid_limit, cudaStream_t stream);
-int js_made_generic_max_grid(int prec);
+int js_made_generic_max_grid(int prec, bool jgs);

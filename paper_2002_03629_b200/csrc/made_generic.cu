@@ -15,127 +15,128 @@
 
 namespace {
 
-constexpr int KC = 32;         // inputs per step of a product
+constexpr int KC = 64;         // inputs per step of a product
 constexpr int NTHREADS = 128;
 constexpr int ROWF = KC + 4;   // row stride in shared memory: the 16-byte pieces of eight rows lie in different banks
-constexpr int STAGES = 3;
+// Two instances: the products' (three tile forms, four stages of activation rows and weight rows, two CTAs per SM), and
+// Jacobi-GS's, whose micro-steps are a warp per inner product and want many warps per SM (smallest tiles, two stages).
+template <bool JGS> struct Conf {
+    static constexpr int STAGES = JGS ? 2 : 4, STAGE_F = (JGS ? 16 + 32 : 32 + 64) * ROWF, CTAS = JGS ? 6 : 2;
+    static constexpr int SMEM_BYTES = STAGES * STAGE_F * (int)sizeof(float);
+};
 
 struct Smem {
-    union {
-        alignas(16) float tile[STAGES][(32 + 64) * ROWF];      // activation rows, then weight rows, of a step
-        int list[4096];        // Jacobi-GS: units to evaluate in this micro-step
-    };
-    int list_n;
-    int wcnt[NTHREADS / 32];
+    float *tile;               // the stages
+    int *list;                 // Jacobi-GS: units to evaluate in this micro-step (shares the stages' memory)
+    int *list_n, *wcnt;
 };
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 // One tile of  out = A[rows][K] * W[N][K]^T  over k in [0, kend): 8 MR rows x 16 NR columns, 128 threads of MR x NR outputs
 // (row lr + 8 i, column 4 NR warp + lc + 4 j).  Operand rows are copied as they lie in memory, 16 bytes at a time, three
-// steps of 32 inputs in flight; a thread reads four inputs of a row at once.  lr takes bits 0, 3, 4 of the lane and lc bits
-// 1, 2: a 16-byte shared-memory load whose address does not depend on bit 0, or not on bit 1, takes two cycles for a warp
-// instead of four.  Every output is one chain of fused multiply-adds over k in ascending order, whatever the tile's form.
-template <typename T, int MR, int NR>
-__device__ __forceinline__ void gemm_tile(Smem &s, const T *A, int lda, const T *__restrict__ W, int ldw, int N, int kend,
+// steps of 64 inputs in flight; a thread reads four inputs of a row at once, the next four while it multiplies.  lr takes bits
+// 0, 3, 4 of the lane and lc bits 1, 2: a 16-byte shared-memory load whose address does not depend on bit 0, or not on bit 1,
+// takes two cycles for a warp instead of four.  Every output is one chain of fused multiply-adds over k in ascending order,
+// whatever the tile's form.  (Steps of 32 inputs, two in flight, with the copies' addresses worked out piece by piece: 57
+// cycles per input of a 16 x 64 tile instead of 14.)
+template <typename T, int MR, int NR, int STAGES, int STAGE_F>
+__device__ __forceinline__ void gemm_tile(float *tile, const T *A, int lda, const T *__restrict__ W, int ldw, int N, int kend,
                                           int m0, int n0, int lr, int wc, float (&acc)[MR][NR])
 {
-    constexpr int BMt = 8 * MR, BNt = 16 * NR, EPP = 16 / sizeof(T);      // values per 16-byte piece
-    constexpr int PIECES = (BMt + BNt) * KC / EPP, PER = (PIECES + NTHREADS - 1) / NTHREADS;
+    constexpr int BMt = 8 * MR, EPP = 16 / sizeof(T);      // values per 16-byte piece
+    constexpr int PPR = KC / EPP, RPE = NTHREADS / PPR;    // pieces per row, rows per round of the 128 threads
+    constexpr int EA = BMt / RPE, EW = 16 * NR / RPE;      // rounds for the activations, for the weights
+    static_assert(BMt % RPE == 0 && (16 * NR) % RPE == 0, "a round lies in one operand");
     const int steps = (kend + KC - 1) / KC;
 #pragma unroll
     for (int i = 0; i < MR; ++i)
 #pragma unroll
         for (int j = 0; j < NR; ++j) acc[i][j] = 0.0f;
-    // piece e of this thread at step c: its source, how many values of it lie below kend, its place in a stage
-    auto piece = [&](int e, int c, const T *&src, int &vals, int &at) {
-        const int idx = threadIdx.x + e * NTHREADS, row = idx / (KC / EPP), k = (idx % (KC / EPP)) * EPP;
-        const bool is_a = row < BMt;
-        const int n = n0 + row - BMt;
-        vals = (PIECES % NTHREADS == 0 || idx < PIECES) && (is_a || n < N) ? max(0, min(EPP, kend - (c * KC + k))) : 0;
-        src = is_a ? A + (size_t)(m0 + row) * lda : W + (size_t)(vals > 0 ? n : 0) * ldw;
-        src += vals > 0 ? c * KC + k : 0;
-        at = row * ROWF + k;
-    };
-    uint4 reg[sizeof(T) == 2 ? PER : 1];
-    auto fetch = [&](int c) {                       // fp32: asynchronous copies; bf16: into registers, converted by put()
+    const int prow = threadIdx.x / PPR, pk = (threadIdx.x % PPR) * EPP;       // this thread's piece: row (+ RPE e), inputs
+    const T *pa = A + (size_t)(m0 + prow) * lda + pk;
+    const uint32_t dst0 = smem_addr(tile) + 4u * (uint32_t)(prow * ROWF + pk);
+    // (weight rows beyond the last column: the last one again, their outputs are not stored)
+    auto w_src = [&](int e) { return W + (size_t)min(n0 + prow + RPE * e, N - 1) * ldw + pk; };
+    uint4 reg[sizeof(T) == 2 ? EA + EW : 1];
+    auto fetch = [&](int c, int st) {               // fp32: asynchronous copies; bf16: into registers, converted by put()
+        const int vals = max(0, min(EPP, kend - (c * KC + pk))), off = vals > 0 ? c * KC : -pk;
 #pragma unroll
-        for (int e = 0; e < PER; ++e) {
-            const T *src;
-            int vals, at;
-            piece(e, c, src, vals, at);
-            if constexpr (sizeof(T) == 4) {
-                if (PIECES % NTHREADS == 0 || threadIdx.x + e * NTHREADS < PIECES)
-                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr(&s.tile[c % STAGES][at])), "l"(src), "r"(vals * 4)
-                                 : "memory");
-            } else {
+        for (int e = 0; e < EA + EW; ++e) {
+            const T *src = (e < EA ? pa + (size_t)(RPE * e) * lda : w_src(e - EA)) + off;
+            if constexpr (sizeof(T) == 4)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst0 + 4u * (uint32_t)(st * STAGE_F + RPE * e * ROWF)),
+                             "l"(src), "r"(vals * 4) : "memory");
+            else
                 reg[e] = vals > 0 ? __ldcg(reinterpret_cast<const uint4 *>(src)) : make_uint4(0, 0, 0, 0);
-            }
         }
-        if constexpr (sizeof(T) == 4) asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    auto put = [&](int c) {
-        if constexpr (sizeof(T) == 2) {
+    auto commit = [] { asm volatile("cp.async.commit_group;" ::: "memory"); };
+    auto put = [&](int c, int st) {
+        const int vals = kend - (c * KC + pk);
 #pragma unroll
-            for (int e = 0; e < PER; ++e) {
-                const T *src;
-                int vals, at;
-                piece(e, c, src, vals, at);
-                if (!(PIECES % NTHREADS == 0 || threadIdx.x + e * NTHREADS < PIECES)) continue;
-                const uint32_t w[4] = {reg[e].x, reg[e].y, reg[e].z, reg[e].w};
-                float v[8];
+        for (int e = 0; e < EA + EW; ++e) {
+            const uint32_t w[4] = {reg[sizeof(T) == 2 ? e : 0].x, reg[sizeof(T) == 2 ? e : 0].y, reg[sizeof(T) == 2 ? e : 0].z, reg[sizeof(T) == 2 ? e : 0].w};
+            float v[8];
 #pragma unroll
-                for (int i = 0; i < 8; ++i) v[i] = i < vals ? __uint_as_float((i & 1) ? (w[i / 2] & 0xffff0000u) : (w[i / 2] << 16)) : 0.0f;
-                float4 *dst = reinterpret_cast<float4 *>(&s.tile[c % STAGES][at]);
-                dst[0] = make_float4(v[0], v[1], v[2], v[3]);
-                dst[1] = make_float4(v[4], v[5], v[6], v[7]);
-            }
+            for (int i = 0; i < 8; ++i) v[i] = i < vals ? __uint_as_float((i & 1) ? (w[i / 2] & 0xffff0000u) : (w[i / 2] << 16)) : 0.0f;
+            float4 *dst = reinterpret_cast<float4 *>(tile + st * STAGE_F + (prow + RPE * e) * ROWF + pk);
+            dst[0] = make_float4(v[0], v[1], v[2], v[3]);
+            dst[1] = make_float4(v[4], v[5], v[6], v[7]);
         }
     };
     __syncthreads();                                // the stages are free
     if constexpr (sizeof(T) == 4) {
+#pragma unroll
         for (int c = 0; c < STAGES - 1; ++c) {
-            if (c < steps) fetch(c);
-            else asm volatile("cp.async.commit_group;" ::: "memory");
+            if (c < steps) fetch(c, c);
+            commit();
         }
     } else if (steps > 0) {
-        fetch(0);
+        fetch(0, 0);
     }
+    int st = 0;
     for (int c = 0; c < steps; ++c) {
         if constexpr (sizeof(T) == 4) asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
-        else put(c);
+        else put(c, st);
         __syncthreads();
         if constexpr (sizeof(T) == 4) {
-            if (c + STAGES - 1 < steps) fetch(c + STAGES - 1);
-            else asm volatile("cp.async.commit_group;" ::: "memory");
+            if (c + STAGES - 1 < steps) fetch(c + STAGES - 1, st == 0 ? STAGES - 1 : st - 1);
+            commit();
         } else if (c + 1 < steps) {
-            fetch(c + 1);
+            fetch(c + 1, 0);
         }
-        const float *ta = &s.tile[c % STAGES][lr * ROWF], *tb = &s.tile[c % STAGES][(BMt + wc) * ROWF];
+        const float *ta = tile + st * STAGE_F + lr * ROWF, *tb = tile + st * STAGE_F + (BMt + wc) * ROWF;
+        float4 a[2][MR], b[2][NR];
+        auto read = [&](int k, int u) {
+#pragma unroll
+            for (int i = 0; i < MR; ++i) a[u][i] = *reinterpret_cast<const float4 *>(ta + 8 * i * ROWF + k);
+#pragma unroll
+            for (int j = 0; j < NR; ++j) b[u][j] = *reinterpret_cast<const float4 *>(tb + 4 * j * ROWF + k);
+        };
+        read(0, 0);
 #pragma unroll
         for (int k = 0; k < KC; k += 4) {
-            float4 a[MR], b[NR];
-#pragma unroll
-            for (int i = 0; i < MR; ++i) a[i] = *reinterpret_cast<const float4 *>(ta + 8 * i * ROWF + k);
-#pragma unroll
-            for (int j = 0; j < NR; ++j) b[j] = *reinterpret_cast<const float4 *>(tb + 4 * j * ROWF + k);
+            const int u = (k >> 2) & 1;
+            if (k + 4 < KC) read(k + 4, u ^ 1);
 #pragma unroll
             for (int i = 0; i < MR; ++i)
 #pragma unroll
-                for (int j = 0; j < NR; ++j) acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
+                for (int j = 0; j < NR; ++j) acc[i][j] = fmaf(a[u][i].x, b[u][j].x, acc[i][j]);
 #pragma unroll
             for (int i = 0; i < MR; ++i)
 #pragma unroll
-                for (int j = 0; j < NR; ++j) acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
+                for (int j = 0; j < NR; ++j) acc[i][j] = fmaf(a[u][i].y, b[u][j].y, acc[i][j]);
 #pragma unroll
             for (int i = 0; i < MR; ++i)
 #pragma unroll
-                for (int j = 0; j < NR; ++j) acc[i][j] = fmaf(a[i].z, b[j].z, acc[i][j]);
+                for (int j = 0; j < NR; ++j) acc[i][j] = fmaf(a[u][i].z, b[u][j].z, acc[i][j]);
 #pragma unroll
             for (int i = 0; i < MR; ++i)
 #pragma unroll
-                for (int j = 0; j < NR; ++j) acc[i][j] = fmaf(a[i].w, b[j].w, acc[i][j]);
+                for (int j = 0; j < NR; ++j) acc[i][j] = fmaf(a[u][i].w, b[u][j].w, acc[i][j]);
         }
+        if (++st == STAGES) st = 0;
     }
 }
 
@@ -169,7 +170,7 @@ struct Changes {
 };
 
 // Layer l over the window in tiles of one form, longest inner products first, dealt to the CTAs back and forth.
-template <typename T, int MR, int NR>
+template <typename T, int MR, int NR, bool JGS>
 __device__ void gemm_tiles(Smem &s, const MadeDev &m, const RunArgs &r, int l, const T *Asrc, T *out, const OutArgs &oa, const Win &w,
                            unsigned long long &issued, unsigned long long &skipped)
 {
@@ -190,21 +191,46 @@ __device__ void gemm_tiles(Smem &s, const MadeDev &m, const RunArgs &r, int l, c
         else live = (dmax > w.hdeg_lo) && (dmin <= w.hdeg_hi);
         if (!live) { if (threadIdx.x == 0) skipped++; continue; }
         if (threadIdx.x == 0) issued++;
-        float acc[MR][NR];
-        gemm_tile<T, MR, NR>(s, Asrc, K, (const T *)m.W[l], K, N, m.t_kend[l][meta], m0, n0, lr, wc, acc);
+        // what the epilogue needs from memory is asked for before the product: biases, and where positions are sampled in the
+        // tile their noise and present values (one after the other behind the product they cost 2 us an output)
+        float acc[MR][NR], bv[NR], nz[MR][NR], xo[MR][NR];
+        const bool sample = is_out && !oa.zout;
+        auto position = [&](int j) { return r.real ? (n0 + wc + 4 * j) >> 1 : n0 + wc + 4 * j; };
+        auto mine = [&](int i, int j) {
+            const int row = m0 + lr + 8 * i, col = n0 + wc + 4 * j, d = position(j);
+            return row < batch && col < N && d >= w.plo && d < w.phi && !(r.real && (col & 1));
+        };
+#pragma unroll
+        for (int j = 0; j < NR; ++j) bv[j] = n0 + wc + 4 * j < N ? __ldg(&m.bias[l][n0 + wc + 4 * j]) : 0.0f;
+        bool frozen[MR];
+        if (sample)
+#pragma unroll
+            for (int i = 0; i < MR; ++i) {
+                const int row = m0 + lr + 8 * i;
+                // a sample whose stopping test has fired keeps the iterate it stopped at (with eps > 0 a further update
+                // would still move it)
+                frozen[i] = r.real && oa.flag && row < batch && r.smp_state[row] != 0;
+#pragma unroll
+                for (int j = 0; j < NR; ++j) {
+                    const bool in = mine(i, j);
+                    const size_t at = (size_t)(in ? row : 0) * m.T + (in ? position(j) : 0);
+                    nz[i][j] = in ? __ldg(r.noise + at) : 0.0f;
+                    xo[i][j] = !in ? 0.0f : r.real ? r.xr[at] : (float)r.x[at];
+                }
+            }
+        gemm_tile<T, MR, NR, Conf<JGS>::STAGES, Conf<JGS>::STAGE_F>(s.tile, Asrc, K, (const T *)m.W[l], K, N, m.t_kend[l][meta], m0, n0, lr, wc, acc);
 #pragma unroll
         for (int i = 0; i < MR; ++i) {
             const int row = m0 + lr + 8 * i;
 #pragma unroll
             for (int j = 0; j < NR; ++j) {
                 const int col = n0 + wc + 4 * j;
-                const float pre = acc[i][j] + (col < N ? __ldg(&m.bias[l][col]) : 0.0f);
-                if (!is_out) {
-                    if (row < batch && col < N) out[(size_t)row * N + col] = from_f32<T>(js_act_fn(m.act, pre));
-                    continue;
-                }
-                if (oa.zout) {
-                    if (row < batch && col < N) oa.zout[(size_t)row * N + col] = pre;
+                const float pre = acc[i][j] + bv[j];
+                if (!sample) {
+                    if (row < batch && col < N) {
+                        if (is_out) oa.zout[(size_t)row * N + col] = pre;
+                        else out[(size_t)row * N + col] = from_f32<T>(js_act_fn(m.act, pre));
+                    }
                     continue;
                 }
                 // Continuous states with logistic conditionals (Section 5.3.1, Appendix C.3 of arXiv 2002.03629): logit 2t is the
@@ -213,20 +239,17 @@ __device__ void gemm_tiles(Smem &s, const MadeDev &m, const RunArgs &r, int l, c
                 // counts as changed when it moved by more than eps, so "no position changed" is the stopping rule
                 // max_t |x^k_t - x^{k-1}_t| <= eps  of Section 2.2.1 in the maximum norm.
                 const float scale = r.real ? __shfl_xor_sync(0xffffffffu, pre, 2) : 0.0f;
-                const int d = r.real ? col >> 1 : col;
-                if (row >= batch || col >= N || d < w.plo || d >= w.phi || (r.real && (col & 1))) continue;
+                if (!mine(i, j) || frozen[i]) continue;
+                const int d = position(j);
                 const size_t at = (size_t)row * m.T + d;
                 if (r.real) {
-                    // a sample whose stopping test has fired keeps the iterate it stopped at (with eps > 0 a further
-                    // update would still move it)
-                    if (oa.flag && r.smp_state[row] != 0) continue;
-                    const float xn = fmaf(expf(scale), r.noise[at], pre), xo = r.xr[at];
+                    const float xn = fmaf(expf(scale), nz[i][j], pre);
                     r.xr[at] = xn;
                     ((T *)m.a[0])[a0_at(m, at)] = from_f32<T>(xn);
-                    if (oa.flag && !(fabsf(xn - xo) <= r.eps)) chg.note(r, oa.parity, row, d);     // a NaN difference is a change
+                    if (oa.flag && !(fabsf(xn - xo[i][j]) <= r.eps)) chg.note(r, oa.parity, row, d);     // a NaN difference is a change
                 } else {
-                    const int xn = js_sample_binary(r.nk, pre, r.noise[at]);
-                    if (xn != r.x[at]) {
+                    const int xn = js_sample_binary(r.nk, pre, nz[i][j]);
+                    if ((float)xn != xo[i][j]) {
                         r.x[at] = (uint8_t)xn;
                         ((T *)m.a[0])[a0_at(m, at)] = from_f32<T>(m.lut[xn]);
                         if (oa.flag) chg.note(r, oa.parity, row, d);
@@ -240,24 +263,28 @@ __device__ void gemm_tiles(Smem &s, const MadeDev &m, const RunArgs &r, int l, c
 
 // Layer l over the window: hidden layers store act(pre) into `out`; the output layer (l == L) see OutArgs.
 // The tile's form: 32 x 64 needs the fewest shared-memory reads per multiply-add, smaller ones spread a layer over more SMs and
-// shorten its longest tile.  Estimate of a layer in cycles: its longest tile alone (issue: 18, 10, 6 cycles per input), or
+// shorten its longest tile.  Estimate of a layer in cycles: its longest tile alone (issue: 20, 12, 8 cycles per input), or
 // what an SM's share of the tiles takes from shared memory (16, 12, 8 cycles per tile and input, inner products half the
-// longest on average).  Measured on 256 samples, 1024 units, 1024 inputs: 100 us per layer with the former 64 x 64 tiles
-// (staged through registers, transposed), see DESIGN for what it is now.
-template <typename T>
+// longest on average).  (Before, 64 x 64 tiles only, staged through registers: 100 us per layer of 1024 units and inputs on
+// 256 samples, 64 of 148 SMs at work.)
+template <typename T, bool JGS>
 __device__ void gemm_phase(Smem &s, const MadeDev &m, const RunArgs &r, int l, const T *Asrc, T *out, const OutArgs &oa, const Win &w,
                            unsigned long long &issued, unsigned long long &skipped)
 {
-    const int N = m.n[l + 1];
-    const float sms = 148.0f;
-    auto cost = [&](int bm, int bn, float alone, float share) {
-        const float tiles = (float)((r.batch + bm - 1) / bm) * (float)((N + bn - 1) / bn);
-        return fmaxf(alone, fmaxf(1.0f, tiles / sms) * share * 0.5f);
-    };
-    const float c44 = cost(32, 64, 18.0f, 16.0f), c24 = cost(16, 64, 10.0f, 12.0f), c22 = cost(16, 32, 6.0f, 8.0f);
-    if (c22 <= c24 && c22 <= c44) gemm_tiles<T, 2, 2>(s, m, r, l, Asrc, out, oa, w, issued, skipped);
-    else if (c24 <= c44) gemm_tiles<T, 2, 4>(s, m, r, l, Asrc, out, oa, w, issued, skipped);
-    else gemm_tiles<T, 4, 4>(s, m, r, l, Asrc, out, oa, w, issued, skipped);
+    if constexpr (JGS) {
+        gemm_tiles<T, 2, 2, true>(s, m, r, l, Asrc, out, oa, w, issued, skipped);
+    } else {
+        const int N = m.n[l + 1];
+        const float sms = 148.0f;
+        auto cost = [&](int bm, int bn, float alone, float share) {
+            const float tiles = (float)((r.batch + bm - 1) / bm) * (float)((N + bn - 1) / bn);
+            return fmaxf(alone, fmaxf(1.0f, tiles / sms) * share * 0.5f);
+        };
+        const float c44 = cost(32, 64, 20.0f, 16.0f), c24 = cost(16, 64, 12.0f, 12.0f), c22 = cost(16, 32, 8.0f, 8.0f);
+        if (c22 <= c24 && c22 <= c44) gemm_tiles<T, 2, 2, false>(s, m, r, l, Asrc, out, oa, w, issued, skipped);
+        else if (c24 <= c44) gemm_tiles<T, 2, 4, false>(s, m, r, l, Asrc, out, oa, w, issued, skipped);
+        else gemm_tiles<T, 4, 4, false>(s, m, r, l, Asrc, out, oa, w, issued, skipped);
+    }
 }
 
 // place in a[0] (rows of n[0] >= T values) of element i = sample * T + position
@@ -368,7 +395,7 @@ __device__ void jgs_hidden_phase(Smem &s, const MadeDev &m, const RunArgs &r, in
     const size_t warps = ((size_t)gridDim.x * blockDim.x) >> 5;
     for (int ubase = 0; ubase < N; ubase += 4096) {
         const int uend = min(N, ubase + 4096);
-        if (threadIdx.x == 0) s.list_n = 0;
+        if (threadIdx.x == 0) *s.list_n = 0;
         __syncthreads();
         for (int base = ubase; base < uend; base += NTHREADS) {
             const int i = base + threadIdx.x;
@@ -380,18 +407,18 @@ __device__ void jgs_hidden_phase(Smem &s, const MadeDev &m, const RunArgs &r, in
             const unsigned bal = __ballot_sync(0xffffffffu, pred);
             if (lane == 0) s.wcnt[warp] = __popc(bal);
             __syncthreads();
-            int off = s.list_n;
+            int off = *s.list_n;
             for (int w2 = 0; w2 < warp; ++w2) off += s.wcnt[w2];
             if (pred) s.list[off + __popc(bal & ((1u << lane) - 1u))] = i;
             __syncthreads();
             if (threadIdx.x == 0) {
                 int tot = 0;
                 for (int w2 = 0; w2 < NTHREADS / 32; ++w2) tot += s.wcnt[w2];
-                s.list_n += tot;
+                *s.list_n += tot;
             }
             __syncthreads();
         }
-        const int cnt = s.list_n;
+        const int cnt = *s.list_n;
         const size_t items = (size_t)cnt * r.batch;
         for (size_t it = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; it < items; it += warps) {
             const int unit = s.list[it / r.batch], b = (int)(it % r.batch);
@@ -475,9 +502,9 @@ __device__ void jgs_copy_or_compare(const MadeDev &m, const RunArgs &r, bool com
 }
 
 // ------------------------------------------------------------------ engine
-template <typename T>
+template <typename T, bool JGS>
 struct GenericEngine {
-    static constexpr bool has_jgs = true;
+    static constexpr bool has_jgs = JGS;
     Smem &s;
     const MadeDev &m;
     const RunArgs &r;
@@ -506,7 +533,7 @@ struct GenericEngine {
         const bool fused = !zout && (m.C == 1 || r.real);
         for (int l = 0; l <= m.L; ++l) {
             const OutArgs oa = {zout ? zout : fused ? (float *)nullptr : m.logits, fused && flag && l == m.L, parity};
-            gemm_phase<T>(s, m, r, l, (const T *)acts[l], l < m.L ? acts[l + 1] : (T *)nullptr, oa, w, issued, skipped);
+            gemm_phase<T, JGS>(s, m, r, l, (const T *)acts[l], l < m.L ? acts[l + 1] : (T *)nullptr, oa, w, issued, skipped);
             if (!barrier()) return false;
         }
         if (zout || fused) return true;
@@ -522,7 +549,7 @@ struct GenericEngine {
         // hidden activations of the previous outer iterate
         const Win w = make_win(fin_h, T_, T_, T_);
         for (int l = 0; l < m.L; ++l) {
-            gemm_phase<T>(s, m, r, l, acts_old[l], acts_old[l + 1], OutArgs{nullptr, false, 0}, w, issued, skipped);
+            gemm_phase<T, JGS>(s, m, r, l, acts_old[l], acts_old[l + 1], OutArgs{nullptr, false, 0}, w, issued, skipped);
             if (!barrier()) return false;
         }
         const int jmax = min(B, T_);
@@ -545,25 +572,36 @@ struct GenericEngine {
     }
 };
 
-template <typename T>
-__global__ void __launch_bounds__(NTHREADS) made_generic_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ RunArgs r)
+template <typename T, bool JGS>
+__global__ void __launch_bounds__(NTHREADS, Conf<JGS>::CTAS) made_generic_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ RunArgs r)
 {
-    __shared__ Smem s;
-    GenericEngine<T> e(s, m, r);
+    extern __shared__ __align__(16) float sm[];
+    __shared__ int list_n, wcnt[NTHREADS / 32];
+    Smem s = {sm, reinterpret_cast<int *>(sm), &list_n, wcnt};
+    GenericEngine<T, JGS> e(s, m, r);
     const DriverResult res = made_driver(e, m.T, r);
     driver_finish(r, res, e.issued, e.skipped);
 }
 
 }  // namespace
 
-int js_made_generic_max_grid(int prec)
+static const void *generic_kernel_of(int prec, bool jgs)
 {
+    if (prec == JS_BF16) return jgs ? (const void *)made_generic_kernel<__nv_bfloat16, true> : (const void *)made_generic_kernel<__nv_bfloat16, false>;
+    return jgs ? (const void *)made_generic_kernel<float, true> : (const void *)made_generic_kernel<float, false>;
+}
+static int generic_smem(bool jgs) { return jgs ? Conf<true>::SMEM_BYTES : Conf<false>::SMEM_BYTES; }
+
+// most CTAs that are resident at a time (a cooperative launch); jgs: of the instance that serves Jacobi-GS
+int js_made_generic_max_grid(int prec, bool jgs)
+{
+    static_assert(Conf<true>::SMEM_BYTES >= 4096 * 4, "the unit list of the micro-steps shares the stages' memory");
     int dev = 0, sms = 0, per_sm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return -1;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return -1;
-    cudaError_t e = prec == JS_BF16
-        ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, made_generic_kernel<__nv_bfloat16>, NTHREADS, 0)
-        : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, made_generic_kernel<float>, NTHREADS, 0);
+    const void *fn = generic_kernel_of(prec, jgs);
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, generic_smem(jgs));
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, NTHREADS, generic_smem(jgs));
     if (e != cudaSuccess || per_sm < 1) return -1;
     return sms * per_sm;
 }
@@ -571,8 +609,7 @@ int js_made_generic_max_grid(int prec)
 int js_launch_made_generic(const MadeDev &m, const RunArgs &r, int grid, cudaStream_t stream)
 {
     void *args[2] = {(void *)&m, (void *)&r};
-    const void *fn = m.prec == JS_BF16 ? (const void *)made_generic_kernel<__nv_bfloat16>
-                                       : (const void *)made_generic_kernel<float>;
-    cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(NTHREADS), args, 0, stream);
+    const bool jgs = r.kmode == KM_JACOBI_GS;
+    cudaError_t e = cudaLaunchCooperativeKernel(generic_kernel_of(m.prec, jgs), dim3(grid), dim3(NTHREADS), args, generic_smem(jgs), stream);
     return e == cudaSuccess ? 0 : (int)e;
 }
