@@ -25,10 +25,14 @@ template <bool JGS> struct Conf {
     static constexpr int SMEM_BYTES = STAGES * STAGE_F * (int)sizeof(float);
 };
 
+// The stages; for the micro-steps of Jacobi-GS the list of units to evaluate.  Named where it is used, not reached through a
+// pointer: the compiler must see that the accesses go to shared memory (as generic loads they took twice the wavefronts
+// and global-memory latency, 57 cycles per input of a 16 x 64 tile).
+extern __shared__ __align__(16) float g_sm[];
+
 struct Smem {
-    float *tile;               // the stages
-    int *list;                 // Jacobi-GS: units to evaluate in this micro-step (shares the stages' memory)
-    int *list_n, *wcnt;
+    int list_n;
+    int wcnt[NTHREADS / 32];
 };
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -38,10 +42,9 @@ __device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)
 // steps of 64 inputs in flight; a thread reads four inputs of a row at once, the next four while it multiplies.  lr takes bits
 // 0, 3, 4 of the lane and lc bits 1, 2: a 16-byte shared-memory load whose address does not depend on bit 0, or not on bit 1,
 // takes two cycles for a warp instead of four.  Every output is one chain of fused multiply-adds over k in ascending order,
-// whatever the tile's form.  (Steps of 32 inputs, two in flight, with the copies' addresses worked out piece by piece: 57
-// cycles per input of a 16 x 64 tile instead of 14.)
+// whatever the tile's form.
 template <typename T, int MR, int NR, int STAGES, int STAGE_F>
-__device__ __forceinline__ void gemm_tile(float *tile, const T *A, int lda, const T *__restrict__ W, int ldw, int N, int kend,
+__device__ __forceinline__ void gemm_tile(const T *A, int lda, const T *__restrict__ W, int ldw, int N, int kend,
                                           int m0, int n0, int lr, int wc, float (&acc)[MR][NR])
 {
     constexpr int BMt = 8 * MR, EPP = 16 / sizeof(T);      // values per 16-byte piece
@@ -49,6 +52,7 @@ __device__ __forceinline__ void gemm_tile(float *tile, const T *A, int lda, cons
     constexpr int EA = BMt / RPE, EW = 16 * NR / RPE;      // rounds for the activations, for the weights
     static_assert(BMt % RPE == 0 && (16 * NR) % RPE == 0, "a round lies in one operand");
     const int steps = (kend + KC - 1) / KC;
+    float *tile = g_sm;
 #pragma unroll
     for (int i = 0; i < MR; ++i)
 #pragma unroll
@@ -218,7 +222,7 @@ __device__ void gemm_tiles(Smem &s, const MadeDev &m, const RunArgs &r, int l, c
                     xo[i][j] = !in ? 0.0f : r.real ? r.xr[at] : (float)r.x[at];
                 }
             }
-        gemm_tile<T, MR, NR, Conf<JGS>::STAGES, Conf<JGS>::STAGE_F>(s.tile, Asrc, K, (const T *)m.W[l], K, N, m.t_kend[l][meta], m0, n0, lr, wc, acc);
+        gemm_tile<T, MR, NR, Conf<JGS>::STAGES, Conf<JGS>::STAGE_F>(Asrc, K, (const T *)m.W[l], K, N, m.t_kend[l][meta], m0, n0, lr, wc, acc);
 #pragma unroll
         for (int i = 0; i < MR; ++i) {
             const int row = m0 + lr + 8 * i;
@@ -390,12 +394,13 @@ __device__ void jgs_hidden_phase(Smem &s, const MadeDev &m, const RunArgs &r, in
 {
     // units of layer l+1 whose degree g satisfies g % B == j, in blocks >= blk_lo.
     // The list is built in index order so that every CTA holds the same list.
+    int *list = reinterpret_cast<int *>(g_sm);
     const int N = m.n[l + 1];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const size_t warps = ((size_t)gridDim.x * blockDim.x) >> 5;
     for (int ubase = 0; ubase < N; ubase += 4096) {
         const int uend = min(N, ubase + 4096);
-        if (threadIdx.x == 0) *s.list_n = 0;
+        if (threadIdx.x == 0) s.list_n = 0;
         __syncthreads();
         for (int base = ubase; base < uend; base += NTHREADS) {
             const int i = base + threadIdx.x;
@@ -407,21 +412,21 @@ __device__ void jgs_hidden_phase(Smem &s, const MadeDev &m, const RunArgs &r, in
             const unsigned bal = __ballot_sync(0xffffffffu, pred);
             if (lane == 0) s.wcnt[warp] = __popc(bal);
             __syncthreads();
-            int off = *s.list_n;
+            int off = s.list_n;
             for (int w2 = 0; w2 < warp; ++w2) off += s.wcnt[w2];
-            if (pred) s.list[off + __popc(bal & ((1u << lane) - 1u))] = i;
+            if (pred) list[off + __popc(bal & ((1u << lane) - 1u))] = i;
             __syncthreads();
             if (threadIdx.x == 0) {
                 int tot = 0;
                 for (int w2 = 0; w2 < NTHREADS / 32; ++w2) tot += s.wcnt[w2];
-                *s.list_n += tot;
+                s.list_n += tot;
             }
             __syncthreads();
         }
-        const int cnt = *s.list_n;
+        const int cnt = s.list_n;
         const size_t items = (size_t)cnt * r.batch;
         for (size_t it = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; it < items; it += warps) {
-            const int unit = s.list[it / r.batch], b = (int)(it % r.batch);
+            const int unit = list[it / r.batch], b = (int)(it % r.batch);
             const int g = m.deg[l + 1][unit];
             const float pre = mixed_dot<T>(m, l, unit, (g - 1) / B, B, (const T *)m.a_old[l] + (size_t)b * m.n[l],
                                            (const T *)m.a[l] + (size_t)b * m.n[l], m.t_kend[l][unit / JS_GT]) +
@@ -510,11 +515,9 @@ struct GenericEngine {
     const RunArgs &r;
     unsigned epoch = 0;
     unsigned long long issued = 0, skipped = 0;
-    T *acts[JS_MAXL + 1], *acts_old[JS_MAXL + 1];
 
     __device__ GenericEngine(Smem &s_, const MadeDev &m_, const RunArgs &r_) : s(s_), m(m_), r(r_)
     {
-        for (int l = 0; l <= m.L; ++l) { acts[l] = (T *)m.a[l]; acts_old[l] = (T *)m.a_old[l]; }
     }
     __device__ bool barrier() { return grid_barrier(r.ctl, epoch, r.spin_limit); }
     __device__ void init(const uint8_t *src)
@@ -533,7 +536,7 @@ struct GenericEngine {
         const bool fused = !zout && (m.C == 1 || r.real);
         for (int l = 0; l <= m.L; ++l) {
             const OutArgs oa = {zout ? zout : fused ? (float *)nullptr : m.logits, fused && flag && l == m.L, parity};
-            gemm_phase<T, JGS>(s, m, r, l, (const T *)acts[l], l < m.L ? acts[l + 1] : (T *)nullptr, oa, w, issued, skipped);
+            gemm_phase<T, JGS>(s, m, r, l, (const T *)m.a[l], l < m.L ? (T *)m.a[l + 1] : (T *)nullptr, oa, w, issued, skipped);
             if (!barrier()) return false;
         }
         if (zout || fused) return true;
@@ -549,7 +552,7 @@ struct GenericEngine {
         // hidden activations of the previous outer iterate
         const Win w = make_win(fin_h, T_, T_, T_);
         for (int l = 0; l < m.L; ++l) {
-            gemm_phase<T, JGS>(s, m, r, l, acts_old[l], acts_old[l + 1], OutArgs{nullptr, false, 0}, w, issued, skipped);
+            gemm_phase<T, JGS>(s, m, r, l, (const T *)m.a_old[l], (T *)m.a_old[l + 1], OutArgs{nullptr, false, 0}, w, issued, skipped);
             if (!barrier()) return false;
         }
         const int jmax = min(B, T_);
@@ -575,9 +578,7 @@ struct GenericEngine {
 template <typename T, bool JGS>
 __global__ void __launch_bounds__(NTHREADS, Conf<JGS>::CTAS) made_generic_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ RunArgs r)
 {
-    extern __shared__ __align__(16) float sm[];
-    __shared__ int list_n, wcnt[NTHREADS / 32];
-    Smem s = {sm, reinterpret_cast<int *>(sm), &list_n, wcnt};
+    __shared__ Smem s;
     GenericEngine<T, JGS> e(s, m, r);
     const DriverResult res = made_driver(e, m.T, r);
     driver_finish(r, res, e.issued, e.skipped);
