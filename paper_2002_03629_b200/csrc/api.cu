@@ -502,6 +502,7 @@ int js_made_create(const js_made_desc *d, js_model **out)
     int rc = made_build(m, d);
     if (rc == JS_OK) rc = common_scratch(m, d->T);
     if (rc == JS_OK && js_tc_prepare(m) < 0) rc = JS_ERR_CUDA;
+    if (rc == JS_OK) rc = js_generic_prepare(m);
     if (rc == JS_OK && js_cluster_prepare(m) < 0) rc = JS_ERR_CUDA;
     if (rc == JS_OK && js_small_prepare(m) < 0) rc = JS_ERR_CUDA;
     if (rc != JS_OK) { js_model_destroy(m); return rc; }

@@ -49,6 +49,7 @@ struct MadeDev {
     const int *t_dmax[JS_MAXL + 1];
     const float *lut;
     float *logits;                    // scratch [rows][T*C]
+    const void *tma_a, *tma_w;        // fp32 models: tensor maps of a[0..L] and W[0..L] (made_generic.cu)
 };
 
 struct RunArgs {

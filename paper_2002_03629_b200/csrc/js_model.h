@@ -147,6 +147,8 @@ int js_small_prepare(js_model *m);
 bool js_small_serves(const js_model *m, const RunArgs &r);
 int js_launch_made_small(const js_model *m, const RunArgs &r, cudaStream_t stream, int *clusters);
 bool js_encode_map_2d(CUtensorMap *out, const void *base, int rows, int cols, int box_rows);
+bool js_encode_map_f32(CUtensorMap *out, const void *base, int rows, int cols, int box_cols, int box_rows);
+int js_generic_prepare(js_model *m);
 int js_cluster_prepare(js_model *m);
 bool js_cluster_serves(const js_model *m, const RunArgs &r);
 int js_launch_made_cluster(const js_model *m, const RunArgs &r, cudaStream_t stream, int *clusters);

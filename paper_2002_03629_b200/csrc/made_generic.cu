@@ -12,18 +12,24 @@
 
 #include "js_common.cuh"
 #include "made_driver.cuh"
+#include "js_model.h"
+#include "tc_common.cuh"
 
 namespace {
 
 constexpr int KC = 64;         // inputs per step of a product
 constexpr int NTHREADS = 128;
 constexpr int ROWF = KC + 4;   // row stride in shared memory: the 16-byte pieces of eight rows lie in different banks
-// Two instances: the products' (three tile forms, four stages of activation rows and weight rows, two CTAs per SM), and
-// Jacobi-GS's, whose micro-steps are a warp per inner product and want many warps per SM (smallest tiles, two stages).
-template <bool JGS> struct Conf {
-    static constexpr int STAGES = JGS ? 2 : 4, STAGE_F = (JGS ? 16 + 32 : 32 + 64) * ROWF, CTAS = JGS ? 6 : 2;
-    static constexpr int SMEM_BYTES = STAGES * STAGE_F * (int)sizeof(float);
+// Instances: fp32 products (three tile forms, operands by TMA: a fifth warp loads), bf16 products (the same forms, operands
+// converted on their way through registers), and for either type Jacobi-GS's, whose micro-steps are a warp per inner product
+// and want many warps per SM (smallest tiles, two stages).
+template <typename T, bool JGS> struct Conf {
+    static constexpr bool TMA = sizeof(T) == 4 && !JGS;
+    static constexpr int STAGES = JGS ? 2 : 4, STAGE_F = TMA ? (32 + 64) * KC : (JGS ? 16 + 32 : 32 + 64) * ROWF, CTAS = JGS ? 6 : 2;
+    static constexpr int SMEM_BYTES = STAGES * STAGE_F * (int)sizeof(float) + (TMA ? 1024 : 0);
+    static constexpr int THREADS = TMA ? NTHREADS + 32 : NTHREADS;
 };
+constexpr int TMA_STAGES = 4, TMA_STAGE_BYTES = (32 + 64) * KC * 4, BOX_K = 32, BOX_A = 16, BOX_W = 32;   // boxes of 128-byte rows
 
 // The stages; for the micro-steps of Jacobi-GS the list of units to evaluate.  Named where it is used, not reached through a
 // pointer: the compiler must see that the accesses go to shared memory (as generic loads they took twice the wavefronts
@@ -33,7 +39,118 @@ extern __shared__ __align__(16) float g_sm[];
 struct Smem {
     int list_n;
     int wcnt[NTHREADS / 32];
+    uint64_t full[TMA_STAGES], empty[TMA_STAGES];
 };
+
+// The ring of the TMA instance; it is drained at the end of every layer.
+struct Ring {
+    int st = 0;
+    uint32_t ph = 0;
+    bool dead = false;
+    __device__ void advance()
+    {
+        if (++st == TMA_STAGES) { st = 0; ph ^= 1u; }
+    }
+};
+__device__ __forceinline__ uint32_t ring_base() { return (smem_u32(g_sm) + 1023u) & ~1023u; }
+__device__ __forceinline__ float4 lds_f4(uint32_t a)
+{
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a));
+    return v;
+}
+
+// The same product with operands by TMA.  A stage holds 64 inputs of the tile's rows: for each half of them the activation
+// rows, then (after both halves) the weight rows, 128 bytes a row, 16-byte pieces permuted by the row number (128-byte swizzle,
+// which keeps the reads of eight rows in different banks).  cp.async, 16 bytes a lane, cost the shared-memory pipe as much as
+// the operand reads (14 wavefronts for 512 bytes).
+template <int MR, int NR>
+__device__ __forceinline__ void tma_tile_load(Smem &s, Ring &rg, const MadeDev &m, int l, int kend, int m0, int n0, JsCtl *ctl)
+{
+    constexpr int BMt = 8 * MR, BNt = 16 * NR;
+    const CUtensorMap *ma = (const CUtensorMap *)m.tma_a + l, *mw = (const CUtensorMap *)m.tma_w + l;
+    const int steps = (kend + KC - 1) / KC;
+    for (int c = 0; c < steps; ++c) {
+        if (!__all_sync(0xffffffffu, mbar_wait(&s.empty[rg.st], rg.ph ^ 1u, ctl))) { rg.dead = true; return; }
+        if (elect_one()) {
+            const uint32_t base = ring_base() + (uint32_t)(rg.st * TMA_STAGE_BYTES);
+            mbar_expect_tx(&s.full[rg.st], (BMt + BNt) * KC * 4);
+#pragma unroll
+            for (int h = 0; h < KC / BOX_K; ++h) {
+#pragma unroll
+                for (int b = 0; b < BMt / BOX_A; ++b)
+                    tma_load_2d(base + (uint32_t)((h * BMt + b * BOX_A) * 128), ma, &s.full[rg.st], c * KC + h * BOX_K, m0 + b * BOX_A);
+#pragma unroll
+                for (int b = 0; b < BNt / BOX_W; ++b)
+                    tma_load_2d(base + (uint32_t)((2 * BMt + h * BNt + b * BOX_W) * 128), mw, &s.full[rg.st], c * KC + h * BOX_K, n0 + b * BOX_W);
+            }
+        }
+        __syncwarp();
+        rg.advance();
+    }
+}
+
+template <int MR, int NR>
+__device__ __forceinline__ void tma_tile(Smem &s, Ring &rg, int kend, int lr, int wc, JsCtl *ctl, float (&acc)[MR][NR])
+{
+    constexpr int BMt = 8 * MR, BNt = 16 * NR;
+    const int steps = (kend + KC - 1) / KC;
+#pragma unroll
+    for (int i = 0; i < MR; ++i)
+#pragma unroll
+        for (int j = 0; j < NR; ++j) acc[i][j] = 0.0f;
+    const uint32_t xa = (uint32_t)(lr & 7) << 4, xb = (uint32_t)(wc & 7) << 4;       // row + 4: the piece's bit 2 flips
+    for (int c = 0; c < steps; ++c) {
+        if (!__all_sync(0xffffffffu, mbar_wait(&s.full[rg.st], rg.ph, ctl))) { rg.dead = true; return; }
+        const uint32_t base = ring_base() + (uint32_t)(rg.st * TMA_STAGE_BYTES);
+        const uint32_t ra = base + (uint32_t)(lr * 128), rb = base + (uint32_t)((2 * BMt + wc) * 128);
+        auto read = [&](int q, float4 (&a)[MR], float4 (&b)[NR]) {      // inputs 4 q .. 4 q + 3 of the step
+            const uint32_t h = (uint32_t)(q >> 3), p = (uint32_t)(q & 7) << 4;
+#pragma unroll
+            for (int i = 0; i < MR; ++i) a[i] = lds_f4(ra + h * (BMt * 128) + (uint32_t)(i * 1024) + (p ^ xa));
+#pragma unroll
+            for (int j = 0; j < NR; ++j) b[j] = lds_f4(rb + h * (BNt * 128) + (uint32_t)(j * 512) + (p ^ xb ^ (uint32_t)((j & 1) << 6)));
+        };
+        auto mul = [&](const float4 (&a)[MR], const float4 (&b)[NR]) {
+#pragma unroll
+            for (int i = 0; i < MR; ++i)
+#pragma unroll
+                for (int j = 0; j < NR; ++j) acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
+#pragma unroll
+            for (int i = 0; i < MR; ++i)
+#pragma unroll
+                for (int j = 0; j < NR; ++j) acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
+#pragma unroll
+            for (int i = 0; i < MR; ++i)
+#pragma unroll
+                for (int j = 0; j < NR; ++j) acc[i][j] = fmaf(a[i].z, b[j].z, acc[i][j]);
+#pragma unroll
+            for (int i = 0; i < MR; ++i)
+#pragma unroll
+                for (int j = 0; j < NR; ++j) acc[i][j] = fmaf(a[i].w, b[j].w, acc[i][j]);
+        };
+        const int nq = min(KC / 4, (kend - c * KC + 3) / 4);             // (weights beyond kend are masked: zeros)
+        if (nq == KC / 4) {
+            float4 a[2][MR], b[2][NR];
+            read(0, a[0], b[0]);
+#pragma unroll
+            for (int q = 0; q < KC / 4; ++q) {
+                if (q + 1 < KC / 4) read(q + 1, a[(q + 1) & 1], b[(q + 1) & 1]);
+                mul(a[q & 1], b[q & 1]);
+            }
+        } else {
+#pragma unroll 1
+            for (int q = 0; q < nq; ++q) {
+                float4 a[MR], b[NR];
+                read(q, a, b);
+                mul(a, b);
+            }
+        }
+        __syncwarp();
+        if ((threadIdx.x & 31) == 0) mbar_arrive(&s.empty[rg.st]);
+        rg.advance();
+    }
+}
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -175,7 +292,7 @@ struct Changes {
 
 // Layer l over the window in tiles of one form, longest inner products first, dealt to the CTAs back and forth.
 template <typename T, int MR, int NR, bool JGS>
-__device__ void gemm_tiles(Smem &s, const MadeDev &m, const RunArgs &r, int l, const T *Asrc, T *out, const OutArgs &oa, const Win &w,
+__device__ void gemm_tiles(Smem &s, Ring &rg, const MadeDev &m, const RunArgs &r, int l, const T *Asrc, T *out, const OutArgs &oa, const Win &w,
                            unsigned long long &issued, unsigned long long &skipped)
 {
     constexpr int BMt = 8 * MR, BNt = 16 * NR;
@@ -184,6 +301,7 @@ __device__ void gemm_tiles(Smem &s, const MadeDev &m, const RunArgs &r, int l, c
     const bool is_out = (l == m.L);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int lr = (lane & 1) | ((lane >> 3) << 1), wc = 4 * NR * warp + ((lane >> 1) & 3);
+    const bool loader = Conf<T, JGS>::TMA && warp == NTHREADS / 32;
     Changes chg;
     for (int round = 0; round * G < mt * nt; ++round) {
         const int tile = round * G + ((round & 1) ? G - 1 - (int)blockIdx.x : (int)blockIdx.x);
@@ -194,6 +312,13 @@ __device__ void gemm_tiles(Smem &s, const MadeDev &m, const RunArgs &r, int l, c
         if (is_out) live = (dmax - 1 >= w.olo) && (dmin - 1 < w.ohi);
         else live = (dmax > w.hdeg_lo) && (dmin <= w.hdeg_hi);
         if (!live) { if (threadIdx.x == 0) skipped++; continue; }
+        if constexpr (Conf<T, JGS>::TMA) {
+            if (rg.dead) break;
+            if (loader) {
+                tma_tile_load<MR, NR>(s, rg, m, l, m.t_kend[l][meta], m0, n0, r.ctl);
+                continue;
+            }
+        }
         if (threadIdx.x == 0) issued++;
         // what the epilogue needs from memory is asked for before the product: biases, and where positions are sampled in the
         // tile their noise and present values (one after the other behind the product they cost 2 us an output)
@@ -222,7 +347,12 @@ __device__ void gemm_tiles(Smem &s, const MadeDev &m, const RunArgs &r, int l, c
                     xo[i][j] = !in ? 0.0f : r.real ? r.xr[at] : (float)r.x[at];
                 }
             }
-        gemm_tile<T, MR, NR, Conf<JGS>::STAGES, Conf<JGS>::STAGE_F>(Asrc, K, (const T *)m.W[l], K, N, m.t_kend[l][meta], m0, n0, lr, wc, acc);
+        if constexpr (Conf<T, JGS>::TMA) {
+            tma_tile<MR, NR>(s, rg, m.t_kend[l][meta], lr, wc, r.ctl, acc);
+            if (rg.dead) break;
+        } else {
+            gemm_tile<T, MR, NR, Conf<T, JGS>::STAGES, Conf<T, JGS>::STAGE_F>(Asrc, K, (const T *)m.W[l], K, N, m.t_kend[l][meta], m0, n0, lr, wc, acc);
+        }
 #pragma unroll
         for (int i = 0; i < MR; ++i) {
             const int row = m0 + lr + 8 * i;
@@ -262,7 +392,7 @@ __device__ void gemm_tiles(Smem &s, const MadeDev &m, const RunArgs &r, int l, c
             }
         }
     }
-    if (oa.flag) chg.flush(r, oa.parity);
+    if (oa.flag && !loader) chg.flush(r, oa.parity);
 }
 
 // Layer l over the window: hidden layers store act(pre) into `out`; the output layer (l == L) see OutArgs.
@@ -272,11 +402,11 @@ __device__ void gemm_tiles(Smem &s, const MadeDev &m, const RunArgs &r, int l, c
 // longest on average).  (Before, 64 x 64 tiles only, staged through registers: 100 us per layer of 1024 units and inputs on
 // 256 samples, 64 of 148 SMs at work.)
 template <typename T, bool JGS>
-__device__ void gemm_phase(Smem &s, const MadeDev &m, const RunArgs &r, int l, const T *Asrc, T *out, const OutArgs &oa, const Win &w,
+__device__ void gemm_phase(Smem &s, Ring &rg, const MadeDev &m, const RunArgs &r, int l, const T *Asrc, T *out, const OutArgs &oa, const Win &w,
                            unsigned long long &issued, unsigned long long &skipped)
 {
     if constexpr (JGS) {
-        gemm_tiles<T, 2, 2, true>(s, m, r, l, Asrc, out, oa, w, issued, skipped);
+        gemm_tiles<T, 2, 2, true>(s, rg, m, r, l, Asrc, out, oa, w, issued, skipped);
     } else {
         const int N = m.n[l + 1];
         const float sms = 148.0f;
@@ -285,9 +415,9 @@ __device__ void gemm_phase(Smem &s, const MadeDev &m, const RunArgs &r, int l, c
             return fmaxf(alone, fmaxf(1.0f, tiles / sms) * share * 0.5f);
         };
         const float c44 = cost(32, 64, 20.0f, 16.0f), c24 = cost(16, 64, 12.0f, 12.0f), c22 = cost(16, 32, 8.0f, 8.0f);
-        if (c22 <= c24 && c22 <= c44) gemm_tiles<T, 2, 2, false>(s, m, r, l, Asrc, out, oa, w, issued, skipped);
-        else if (c24 <= c44) gemm_tiles<T, 2, 4, false>(s, m, r, l, Asrc, out, oa, w, issued, skipped);
-        else gemm_tiles<T, 4, 4, false>(s, m, r, l, Asrc, out, oa, w, issued, skipped);
+        if (c22 <= c24 && c22 <= c44) gemm_tiles<T, 2, 2, false>(s, rg, m, r, l, Asrc, out, oa, w, issued, skipped);
+        else if (c24 <= c44) gemm_tiles<T, 2, 4, false>(s, rg, m, r, l, Asrc, out, oa, w, issued, skipped);
+        else gemm_tiles<T, 4, 4, false>(s, rg, m, r, l, Asrc, out, oa, w, issued, skipped);
     }
 }
 
@@ -515,11 +645,19 @@ struct GenericEngine {
     const RunArgs &r;
     unsigned epoch = 0;
     unsigned long long issued = 0, skipped = 0;
+    Ring rg;
 
     __device__ GenericEngine(Smem &s_, const MadeDev &m_, const RunArgs &r_) : s(s_), m(m_), r(r_)
     {
     }
-    __device__ bool barrier() { return grid_barrier(r.ctl, epoch, r.spin_limit); }
+    __device__ bool barrier()
+    {
+        // activations stored by threads are read by TMA after the barrier
+        if constexpr (Conf<T, JGS>::TMA) fence_proxy_async();
+        const bool ok = grid_barrier(r.ctl, epoch, r.spin_limit);
+        if constexpr (Conf<T, JGS>::TMA) fence_proxy_async();
+        return ok;
+    }
     __device__ void init(const uint8_t *src)
     {
         if (r.real)
@@ -536,7 +674,7 @@ struct GenericEngine {
         const bool fused = !zout && (m.C == 1 || r.real);
         for (int l = 0; l <= m.L; ++l) {
             const OutArgs oa = {zout ? zout : fused ? (float *)nullptr : m.logits, fused && flag && l == m.L, parity};
-            gemm_phase<T, JGS>(s, m, r, l, (const T *)m.a[l], l < m.L ? (T *)m.a[l + 1] : (T *)nullptr, oa, w, issued, skipped);
+            gemm_phase<T, JGS>(s, rg, m, r, l, (const T *)m.a[l], l < m.L ? (T *)m.a[l + 1] : (T *)nullptr, oa, w, issued, skipped);
             if (!barrier()) return false;
         }
         if (zout || fused) return true;
@@ -552,7 +690,7 @@ struct GenericEngine {
         // hidden activations of the previous outer iterate
         const Win w = make_win(fin_h, T_, T_, T_);
         for (int l = 0; l < m.L; ++l) {
-            gemm_phase<T, JGS>(s, m, r, l, (const T *)m.a_old[l], (T *)m.a_old[l + 1], OutArgs{nullptr, false, 0}, w, issued, skipped);
+            gemm_phase<T, JGS>(s, rg, m, r, l, (const T *)m.a_old[l], (T *)m.a_old[l + 1], OutArgs{nullptr, false, 0}, w, issued, skipped);
             if (!barrier()) return false;
         }
         const int jmax = min(B, T_);
@@ -576,11 +714,27 @@ struct GenericEngine {
 };
 
 template <typename T, bool JGS>
-__global__ void __launch_bounds__(NTHREADS, Conf<JGS>::CTAS) made_generic_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ RunArgs r)
+__global__ void __launch_bounds__(Conf<T, JGS>::THREADS, Conf<T, JGS>::CTAS) made_generic_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ RunArgs r)
 {
     __shared__ Smem s;
+    if constexpr (Conf<T, JGS>::TMA) {
+        if (threadIdx.x == 0) {
+            for (int i = 0; i < TMA_STAGES; ++i) { mbar_init(&s.full[i], 1); mbar_init(&s.empty[i], NTHREADS / 32); }
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+            fence_proxy_async();
+        }
+        __syncthreads();
+    }
     GenericEngine<T, JGS> e(s, m, r);
-    const DriverResult res = made_driver(e, m.T, r);
+    DriverResult res = made_driver(e, m.T, r);
+    if constexpr (Conf<T, JGS>::TMA) {
+        // after an aborted wait copies may still be on their way into this CTA's shared memory
+        if (__syncthreads_or(e.rg.dead || !res.alive)) {
+            for (int i = 0; i < 2000; ++i) __nanosleep(1000);
+            res.alive = false;
+        }
+        __syncthreads();
+    }
     driver_finish(r, res, e.issued, e.skipped);
 }
 
@@ -591,18 +745,44 @@ static const void *generic_kernel_of(int prec, bool jgs)
     if (prec == JS_BF16) return jgs ? (const void *)made_generic_kernel<__nv_bfloat16, true> : (const void *)made_generic_kernel<__nv_bfloat16, false>;
     return jgs ? (const void *)made_generic_kernel<float, true> : (const void *)made_generic_kernel<float, false>;
 }
-static int generic_smem(bool jgs) { return jgs ? Conf<true>::SMEM_BYTES : Conf<false>::SMEM_BYTES; }
+static int generic_smem(int prec, bool jgs)
+{
+    if (jgs) return Conf<float, true>::SMEM_BYTES;
+    return prec == JS_BF16 ? Conf<__nv_bfloat16, false>::SMEM_BYTES : Conf<float, false>::SMEM_BYTES;
+}
+static int generic_threads(int prec, bool jgs) { return prec == JS_BF16 || jgs ? NTHREADS : Conf<float, false>::THREADS; }
+
+// Tensor maps of an fp32 model's activations and masked weights: boxes of 32 inputs x 16 or 32 rows, 128-byte swizzle.
+int js_generic_prepare(js_model *mo)
+{
+    MadeDev &v = mo->made;
+    v.tma_a = v.tma_w = nullptr;
+    if (v.prec != JS_F32) return JS_OK;
+    std::vector<CUtensorMap> maps(2 * (v.L + 1));
+    for (int l = 0; l <= v.L; ++l) {
+        if (!js_encode_map_f32(&maps[l], v.a[l], mo->rows, v.n[l], BOX_K, BOX_A) ||
+            !js_encode_map_f32(&maps[v.L + 1 + l], v.W[l], v.n[l + 1], v.n[l], BOX_K, BOX_W))
+            return JS_ERR_CUDA;
+    }
+    void *p = nullptr;
+    if (cudaMalloc(&p, maps.size() * sizeof(CUtensorMap)) != cudaSuccess) return JS_ERR_CUDA;
+    mo->allocs.push_back(p);
+    if (cudaMemcpy(p, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice) != cudaSuccess) return JS_ERR_CUDA;
+    v.tma_a = p;
+    v.tma_w = (const CUtensorMap *)p + v.L + 1;
+    return JS_OK;
+}
 
 // most CTAs that are resident at a time (a cooperative launch); jgs: of the instance that serves Jacobi-GS
 int js_made_generic_max_grid(int prec, bool jgs)
 {
-    static_assert(Conf<true>::SMEM_BYTES >= 4096 * 4, "the unit list of the micro-steps shares the stages' memory");
+    static_assert(Conf<float, true>::SMEM_BYTES >= 4096 * 4, "the unit list of the micro-steps shares the stages' memory");
     int dev = 0, sms = 0, per_sm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return -1;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return -1;
     const void *fn = generic_kernel_of(prec, jgs);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, generic_smem(jgs));
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, NTHREADS, generic_smem(jgs));
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, generic_smem(prec, jgs));
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, generic_threads(prec, jgs), generic_smem(prec, jgs));
     if (e != cudaSuccess || per_sm < 1) return -1;
     return sms * per_sm;
 }
@@ -611,6 +791,6 @@ int js_launch_made_generic(const MadeDev &m, const RunArgs &r, int grid, cudaStr
 {
     void *args[2] = {(void *)&m, (void *)&r};
     const bool jgs = r.kmode == KM_JACOBI_GS;
-    cudaError_t e = cudaLaunchCooperativeKernel(generic_kernel_of(m.prec, jgs), dim3(grid), dim3(NTHREADS), args, generic_smem(jgs), stream);
+    cudaError_t e = cudaLaunchCooperativeKernel(generic_kernel_of(m.prec, jgs), dim3(grid), dim3(generic_threads(m.prec, jgs)), args, generic_smem(m.prec, jgs), stream);
     return e == cudaSuccess ? 0 : (int)e;
 }
