@@ -20,16 +20,20 @@ namespace {
 constexpr int KC = 64;         // inputs per step of a product
 constexpr int NTHREADS = 128;
 constexpr int ROWF = KC + 4;   // row stride in shared memory: the 16-byte pieces of eight rows lie in different banks
-// Instances: fp32 products (three tile forms, operands by TMA: a fifth warp loads), bf16 products (the same forms, operands
-// converted on their way through registers), and for either type Jacobi-GS's, whose micro-steps are a warp per inner product
-// and want many warps per SM (smallest tiles, two stages).
+// The products go by tiles of 16 rows x 32 columns.  What bounds a layer is its longest tile (one chain over all inputs, with
+// every wait of a step in it), so small tiles win although they read shared memory more often: 256 samples through
+// 784 - 1024 - 1024 - 1568, five passes: 298 us, with 16 x 64 tiles 343, with 32 x 64 552; 16 samples: 228, 309, 488.
+constexpr int MR = 2, NR = 2, BMt = 8 * MR, BNt = 16 * NR;
+// Instances: fp32 products (operands by TMA: a fifth warp loads), bf16 products (operands converted on their way through
+// registers), and for either type Jacobi-GS's, whose micro-steps are a warp per inner product and want many warps per SM.
 template <typename T, bool JGS> struct Conf {
     static constexpr bool TMA = sizeof(T) == 4 && !JGS;
-    static constexpr int STAGES = JGS ? 2 : 4, STAGE_F = TMA ? (32 + 64) * KC : (JGS ? 16 + 32 : 32 + 64) * ROWF, CTAS = JGS ? 6 : 2;
+    static constexpr int STAGES = JGS ? 2 : 4, STAGE_F = (BMt + BNt) * (TMA ? 2 * KC : ROWF), CTAS = JGS ? 6 : 2;
     static constexpr int SMEM_BYTES = STAGES * STAGE_F * (int)sizeof(float) + (TMA ? 1024 : 0);
     static constexpr int THREADS = TMA ? NTHREADS + 32 : NTHREADS;
 };
-constexpr int TMA_STAGES = 4, TMA_STAGE_BYTES = (32 + 64) * KC * 4, BOX_K = 32, BOX_A = 16, BOX_W = 32;   // boxes of 128-byte rows
+// TMA instance: stages of TK inputs in boxes of 32 (128-byte rows)
+constexpr int TK = 2 * KC, BOX_K = 32, TMA_STAGES = 4, TMA_STAGE_BYTES = (BMt + BNt) * TK * 4;
 
 // The stages; for the micro-steps of Jacobi-GS the list of units to evaluate.  Named where it is used, not reached through a
 // pointer: the compiler must see that the accesses go to shared memory (as generic loads they took twice the wavefronts
@@ -60,29 +64,22 @@ __device__ __forceinline__ float4 lds_f4(uint32_t a)
     return v;
 }
 
-// The same product with operands by TMA.  A stage holds 64 inputs of the tile's rows: for each half of them the activation
-// rows, then (after both halves) the weight rows, 128 bytes a row, 16-byte pieces permuted by the row number (128-byte swizzle,
-// which keeps the reads of eight rows in different banks).  cp.async, 16 bytes a lane, cost the shared-memory pipe as much as
-// the operand reads (14 wavefronts for 512 bytes).
-template <int MR, int NR>
+// The product with operands by TMA.  A stage holds TK inputs of the tile's rows: for every 32 of them the activation rows,
+// behind all those the weight rows likewise, 128 bytes a row, 16-byte pieces permuted by the row number (128-byte swizzle,
+// which keeps the reads of eight rows in different banks).  cp.async, 16 bytes a lane, cost the shared-memory pipe as much
+// as the operand reads (14 wavefronts for 512 bytes).
 __device__ __forceinline__ void tma_tile_load(Smem &s, Ring &rg, const MadeDev &m, int l, int kend, int m0, int n0, JsCtl *ctl)
 {
-    constexpr int BMt = 8 * MR, BNt = 16 * NR;
     const CUtensorMap *ma = (const CUtensorMap *)m.tma_a + l, *mw = (const CUtensorMap *)m.tma_w + l;
-    const int steps = (kend + KC - 1) / KC;
-    for (int c = 0; c < steps; ++c) {
+    for (int k0 = 0; k0 < kend; k0 += TK) {
         if (!__all_sync(0xffffffffu, mbar_wait(&s.empty[rg.st], rg.ph ^ 1u, ctl))) { rg.dead = true; return; }
         if (elect_one()) {
             const uint32_t base = ring_base() + (uint32_t)(rg.st * TMA_STAGE_BYTES);
-            mbar_expect_tx(&s.full[rg.st], (BMt + BNt) * KC * 4);
-#pragma unroll
-            for (int h = 0; h < KC / BOX_K; ++h) {
-#pragma unroll
-                for (int b = 0; b < BMt / BOX_A; ++b)
-                    tma_load_2d(base + (uint32_t)((h * BMt + b * BOX_A) * 128), ma, &s.full[rg.st], c * KC + h * BOX_K, m0 + b * BOX_A);
-#pragma unroll
-                for (int b = 0; b < BNt / BOX_W; ++b)
-                    tma_load_2d(base + (uint32_t)((2 * BMt + h * BNt + b * BOX_W) * 128), mw, &s.full[rg.st], c * KC + h * BOX_K, n0 + b * BOX_W);
+            const int boxes = min(TK / BOX_K, (kend - k0 + BOX_K - 1) / BOX_K);
+            mbar_expect_tx(&s.full[rg.st], (uint32_t)(boxes * (BMt + BNt) * BOX_K * 4));
+            for (int h = 0; h < boxes; ++h) {
+                tma_load_2d(base + (uint32_t)(h * BMt * 128), ma, &s.full[rg.st], k0 + h * BOX_K, m0);
+                tma_load_2d(base + (uint32_t)(TK / BOX_K * BMt * 128 + h * BNt * 128), mw, &s.full[rg.st], k0 + h * BOX_K, n0);
             }
         }
         __syncwarp();
@@ -90,21 +87,18 @@ __device__ __forceinline__ void tma_tile_load(Smem &s, Ring &rg, const MadeDev &
     }
 }
 
-template <int MR, int NR>
 __device__ __forceinline__ void tma_tile(Smem &s, Ring &rg, int kend, int lr, int wc, JsCtl *ctl, float (&acc)[MR][NR])
 {
-    constexpr int BMt = 8 * MR, BNt = 16 * NR;
-    const int steps = (kend + KC - 1) / KC;
 #pragma unroll
     for (int i = 0; i < MR; ++i)
 #pragma unroll
         for (int j = 0; j < NR; ++j) acc[i][j] = 0.0f;
     const uint32_t xa = (uint32_t)(lr & 7) << 4, xb = (uint32_t)(wc & 7) << 4;       // row + 4: the piece's bit 2 flips
-    for (int c = 0; c < steps; ++c) {
-        if (!__all_sync(0xffffffffu, mbar_wait(&s.full[rg.st], rg.ph, ctl))) { rg.dead = true; return; }
-        const uint32_t base = ring_base() + (uint32_t)(rg.st * TMA_STAGE_BYTES);
-        const uint32_t ra = base + (uint32_t)(lr * 128), rb = base + (uint32_t)((2 * BMt + wc) * 128);
-        auto read = [&](int q, float4 (&a)[MR], float4 (&b)[NR]) {      // inputs 4 q .. 4 q + 3 of the step
+    for (int k0 = 0; k0 < kend; k0 += TK) {
+        if (!mbar_wait(&s.full[rg.st], rg.ph, ctl)) { rg.dead = true; return; }
+        uint32_t ra = ring_base() + (uint32_t)(rg.st * TMA_STAGE_BYTES), rb = ra + (uint32_t)(TK / BOX_K * BMt * 128 + wc * 128);
+        ra += (uint32_t)(lr * 128);
+        auto read = [&](int q, float4 (&a)[MR], float4 (&b)[NR]) {      // inputs 4 q .. 4 q + 3 from ra, rb on
             const uint32_t h = (uint32_t)(q >> 3), p = (uint32_t)(q & 7) << 4;
 #pragma unroll
             for (int i = 0; i < MR; ++i) a[i] = lds_f4(ra + h * (BMt * 128) + (uint32_t)(i * 1024) + (p ^ xa));
@@ -129,22 +123,29 @@ __device__ __forceinline__ void tma_tile(Smem &s, Ring &rg, int kend, int lr, in
 #pragma unroll
                 for (int j = 0; j < NR; ++j) acc[i][j] = fmaf(a[i].w, b[j].w, acc[i][j]);
         };
-        const int nq = min(KC / 4, (kend - c * KC + 3) / 4);             // (weights beyond kend are masked: zeros)
-        if (nq == KC / 4) {
-            float4 a[2][MR], b[2][NR];
-            read(0, a[0], b[0]);
-#pragma unroll
-            for (int q = 0; q < KC / 4; ++q) {
-                if (q + 1 < KC / 4) read(q + 1, a[(q + 1) & 1], b[(q + 1) & 1]);
-                mul(a[q & 1], b[q & 1]);
-            }
-        } else {
+        const int nq = min(TK / 4, (kend - k0 + 3) / 4);                 // (weights beyond kend are masked: zeros)
+        constexpr int QU = 16, AHEAD = 3;                                // reads three quadruples ahead of their use
 #pragma unroll 1
-            for (int q = 0; q < nq; ++q) {
-                float4 a[MR], b[NR];
-                read(q, a, b);
-                mul(a, b);
+        for (int q0 = 0; q0 < nq; q0 += QU) {
+            if (nq - q0 >= QU) {
+                float4 a[AHEAD + 1][MR], b[AHEAD + 1][NR];
+#pragma unroll
+                for (int q = 0; q < AHEAD; ++q) read(q, a[q], b[q]);
+#pragma unroll
+                for (int q = 0; q < QU; ++q) {
+                    if (q + AHEAD < QU) read(q + AHEAD, a[(q + AHEAD) % (AHEAD + 1)], b[(q + AHEAD) % (AHEAD + 1)]);
+                    mul(a[q % (AHEAD + 1)], b[q % (AHEAD + 1)]);
+                }
+            } else {
+#pragma unroll 1
+                for (int q = 0; q < nq - q0; ++q) {
+                    float4 a[MR], b[NR];
+                    read(q, a, b);
+                    mul(a, b);
+                }
             }
+            ra += QU / 8 * BMt * 128;
+            rb += QU / 8 * BNt * 128;
         }
         __syncwarp();
         if ((threadIdx.x & 31) == 0) mbar_arrive(&s.empty[rg.st]);
@@ -158,16 +159,15 @@ __device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)
 // (row lr + 8 i, column 4 NR warp + lc + 4 j).  Operand rows are copied as they lie in memory, 16 bytes at a time, three
 // steps of 64 inputs in flight; a thread reads four inputs of a row at once, the next four while it multiplies.  lr takes bits
 // 0, 3, 4 of the lane and lc bits 1, 2: a 16-byte shared-memory load whose address does not depend on bit 0, or not on bit 1,
-// takes two cycles for a warp instead of four.  Every output is one chain of fused multiply-adds over k in ascending order,
-// whatever the tile's form.
-template <typename T, int MR, int NR, int STAGES, int STAGE_F>
+// takes two cycles for a warp instead of four.  Every output is one chain of fused multiply-adds over k in ascending order.
+template <typename T, int STAGES, int STAGE_F>
 __device__ __forceinline__ void gemm_tile(const T *A, int lda, const T *__restrict__ W, int ldw, int N, int kend,
                                           int m0, int n0, int lr, int wc, float (&acc)[MR][NR])
 {
-    constexpr int BMt = 8 * MR, EPP = 16 / sizeof(T);      // values per 16-byte piece
+    constexpr int EPP = 16 / sizeof(T);      // values per 16-byte piece
     constexpr int PPR = KC / EPP, RPE = NTHREADS / PPR;    // pieces per row, rows per round of the 128 threads
-    constexpr int EA = BMt / RPE, EW = 16 * NR / RPE;      // rounds for the activations, for the weights
-    static_assert(BMt % RPE == 0 && (16 * NR) % RPE == 0, "a round lies in one operand");
+    constexpr int EA = BMt / RPE, EW = BNt / RPE;      // rounds for the activations, for the weights
+    static_assert(BMt % RPE == 0 && BNt % RPE == 0, "a round lies in one operand");
     const int steps = (kend + KC - 1) / KC;
     float *tile = g_sm;
 #pragma unroll
@@ -290,12 +290,12 @@ struct Changes {
     }
 };
 
-// Layer l over the window in tiles of one form, longest inner products first, dealt to the CTAs back and forth.
-template <typename T, int MR, int NR, bool JGS>
-__device__ void gemm_tiles(Smem &s, Ring &rg, const MadeDev &m, const RunArgs &r, int l, const T *Asrc, T *out, const OutArgs &oa, const Win &w,
+// Layer l over the window: hidden layers store act(pre) into `out`; the output layer (l == L) see OutArgs.  Tiles with the
+// longest inner products first, dealt to the CTAs back and forth.
+template <typename T, bool JGS>
+__device__ void gemm_phase(Smem &s, Ring &rg, const MadeDev &m, const RunArgs &r, int l, const T *Asrc, T *out, const OutArgs &oa, const Win &w,
                            unsigned long long &issued, unsigned long long &skipped)
 {
-    constexpr int BMt = 8 * MR, BNt = 16 * NR;
     const int N = m.n[l + 1], K = m.n[l], batch = r.batch;
     const int mt = (batch + BMt - 1) / BMt, nt = (N + BNt - 1) / BNt, G = (int)gridDim.x;
     const bool is_out = (l == m.L);
@@ -315,7 +315,7 @@ __device__ void gemm_tiles(Smem &s, Ring &rg, const MadeDev &m, const RunArgs &r
         if constexpr (Conf<T, JGS>::TMA) {
             if (rg.dead) break;
             if (loader) {
-                tma_tile_load<MR, NR>(s, rg, m, l, m.t_kend[l][meta], m0, n0, r.ctl);
+                tma_tile_load(s, rg, m, l, m.t_kend[l][meta], m0, n0, r.ctl);
                 continue;
             }
         }
@@ -348,10 +348,10 @@ __device__ void gemm_tiles(Smem &s, Ring &rg, const MadeDev &m, const RunArgs &r
                 }
             }
         if constexpr (Conf<T, JGS>::TMA) {
-            tma_tile<MR, NR>(s, rg, m.t_kend[l][meta], lr, wc, r.ctl, acc);
+            tma_tile(s, rg, m.t_kend[l][meta], lr, wc, r.ctl, acc);
             if (rg.dead) break;
         } else {
-            gemm_tile<T, MR, NR, Conf<T, JGS>::STAGES, Conf<T, JGS>::STAGE_F>(Asrc, K, (const T *)m.W[l], K, N, m.t_kend[l][meta], m0, n0, lr, wc, acc);
+            gemm_tile<T, Conf<T, JGS>::STAGES, Conf<T, JGS>::STAGE_F>(Asrc, K, (const T *)m.W[l], K, N, m.t_kend[l][meta], m0, n0, lr, wc, acc);
         }
 #pragma unroll
         for (int i = 0; i < MR; ++i) {
@@ -393,32 +393,6 @@ __device__ void gemm_tiles(Smem &s, Ring &rg, const MadeDev &m, const RunArgs &r
         }
     }
     if (oa.flag && !loader) chg.flush(r, oa.parity);
-}
-
-// Layer l over the window: hidden layers store act(pre) into `out`; the output layer (l == L) see OutArgs.
-// The tile's form: 32 x 64 needs the fewest shared-memory reads per multiply-add, smaller ones spread a layer over more SMs and
-// shorten its longest tile.  Estimate of a layer in cycles: its longest tile alone (issue: 20, 12, 8 cycles per input), or
-// what an SM's share of the tiles takes from shared memory (16, 12, 8 cycles per tile and input, inner products half the
-// longest on average).  (Before, 64 x 64 tiles only, staged through registers: 100 us per layer of 1024 units and inputs on
-// 256 samples, 64 of 148 SMs at work.)
-template <typename T, bool JGS>
-__device__ void gemm_phase(Smem &s, Ring &rg, const MadeDev &m, const RunArgs &r, int l, const T *Asrc, T *out, const OutArgs &oa, const Win &w,
-                           unsigned long long &issued, unsigned long long &skipped)
-{
-    if constexpr (JGS) {
-        gemm_tiles<T, 2, 2, true>(s, rg, m, r, l, Asrc, out, oa, w, issued, skipped);
-    } else {
-        const int N = m.n[l + 1];
-        const float sms = 148.0f;
-        auto cost = [&](int bm, int bn, float alone, float share) {
-            const float tiles = (float)((r.batch + bm - 1) / bm) * (float)((N + bn - 1) / bn);
-            return fmaxf(alone, fmaxf(1.0f, tiles / sms) * share * 0.5f);
-        };
-        const float c44 = cost(32, 64, 20.0f, 16.0f), c24 = cost(16, 64, 12.0f, 12.0f), c22 = cost(16, 32, 8.0f, 8.0f);
-        if (c22 <= c24 && c22 <= c44) gemm_tiles<T, 2, 2, false>(s, rg, m, r, l, Asrc, out, oa, w, issued, skipped);
-        else if (c24 <= c44) gemm_tiles<T, 2, 4, false>(s, rg, m, r, l, Asrc, out, oa, w, issued, skipped);
-        else gemm_tiles<T, 4, 4, false>(s, rg, m, r, l, Asrc, out, oa, w, issued, skipped);
-    }
 }
 
 // place in a[0] (rows of n[0] >= T values) of element i = sample * T + position
@@ -752,7 +726,7 @@ static int generic_smem(int prec, bool jgs)
 }
 static int generic_threads(int prec, bool jgs) { return prec == JS_BF16 || jgs ? NTHREADS : Conf<float, false>::THREADS; }
 
-// Tensor maps of an fp32 model's activations and masked weights: boxes of 32 inputs x 16 or 32 rows, 128-byte swizzle.
+// Tensor maps of an fp32 model's activations and masked weights: boxes of 32 inputs x 16 rows (activations) or 32 rows, 128-byte swizzle.
 int js_generic_prepare(js_model *mo)
 {
     MadeDev &v = mo->made;
@@ -760,8 +734,8 @@ int js_generic_prepare(js_model *mo)
     if (v.prec != JS_F32) return JS_OK;
     std::vector<CUtensorMap> maps(2 * (v.L + 1));
     for (int l = 0; l <= v.L; ++l) {
-        if (!js_encode_map_f32(&maps[l], v.a[l], mo->rows, v.n[l], BOX_K, BOX_A) ||
-            !js_encode_map_f32(&maps[v.L + 1 + l], v.W[l], v.n[l + 1], v.n[l], BOX_K, BOX_W))
+        if (!js_encode_map_f32(&maps[l], v.a[l], mo->rows, v.n[l], BOX_K, BMt) ||
+            !js_encode_map_f32(&maps[v.L + 1 + l], v.W[l], v.n[l + 1], v.n[l], BOX_K, BNt))
             return JS_ERR_CUDA;
     }
     void *p = nullptr;
