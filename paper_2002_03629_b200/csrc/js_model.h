@@ -41,8 +41,9 @@ struct TcDev {
 
 // What the cached sweeps (made_sweep.cu) need beside the tensor-core view.
 struct SweepDev {
-    const CUtensorMap *tmAold;          // [L+1] activations a[l] of the previous iterate, box 64 x 128 (= TcDev::tmA)
-    const CUtensorMap *tmF;             // [L+1] the jobs' buffers F[l], 3-D {column, row, slot}, box 64 x 128 x 1
+    const CUtensorMap *tmAold;          // [3][L+1] activations a[l] of the previous iterate, boxes 64 x 32, 64, 128
+    const CUtensorMap *tmF;             // [3][L+1] the jobs' buffers F[l], 3-D {column, row, slot}, boxes 64 x 32, 64, 128 x 1
+    int rj, rj_idx;                     // sample rows per job (32 << rj_idx)
     const CUtensorMap *tmW16;           // [3][L+1] masked weights W[l]: boxes of 64 x 16, 64 x 32 and 64 x 64 (columns x rows)
     float *S;                           // [slot][L+1][nbs][128 rows] fp32: base sums of a job's next groups
     int nbs;

@@ -7,7 +7,7 @@
 // one block covering every position, the feedforward pass itself with every hidden unit evaluated
 // once (the cached sampler of Section 4.2).
 //
-// Work decomposition.  A job is (128 samples, one block); jobs never talk to each other, so the
+// Work decomposition.  A job is (128, 64 or 32 samples, one block); jobs never talk to each other, so the
 // kernel needs no grid-wide synchronisation at all.  Inside a job the positions are taken in
 // groups of G.  With sorted degrees, everything a group needs from before the group - inputs and
 // hidden units of degree <= t0, the group's first position - is a PREFIX of every layer's units,
@@ -16,9 +16,12 @@
 // the prefix of the activations (from the previous iterate's activations up to the block's start,
 // from the job's own buffer F after it) and 16-row weight boxes, tcgen05.mma accumulates in tensor
 // memory.  What the units of the group contribute to one another is a triangular system of at most
-// 32 x 32 weights per layer, solved position by position with thread = sample row: logit, sample
-// against the fixed noise (Appendix A.3), then the hidden units that the new symbol makes
-// computable.  The group's activations then go to F, where the next group's GEMMs find them.
+// 32 x 32 weights per layer, solved position by position: logit, sample against the fixed noise
+// (Appendix A.3), then the hidden units that the new symbol makes computable.  A warp takes eight sample rows,
+// lane = unit of the group, every layer's running sums in registers; a value that becomes known goes to all lanes by
+// shuffle and is added to 32 running sums by one multiply-add per row.  (With thread = row and the running sums in shared
+// memory a position moved 24 KB through it: 0.6 us for two hidden layers.)  The group's activations then go to F,
+// where the next group's GEMMs find them.
 //
 // Every value is a fixed function of the iterate: the split into prefix and group depends on the
 // block size and the position alone.  Waits are bounded as in the other tensor-core kernels.
@@ -35,7 +38,9 @@
 namespace {
 
 constexpr int BM = TC_BM, BK = TC_BK;
-constexpr int NTH = 192;
+constexpr int NEW = 16;                      // epilogue warps: four per tensor-memory quadrant; eight sample rows each
+constexpr int NEP = 32 * NEW;
+constexpr int NTH = 64 + NEP;
 constexpr int NUP = 32;                      // most units of one layer inside a group
 constexpr int GMAX = 32;                     // most positions per group
 constexpr int A_BYTES = BM * BK * 2;
@@ -44,7 +49,7 @@ constexpr int GPB = 8;                       // groups per base: a base GEMM ser
 constexpr int W_BYTES = NB * BK * 2;
 constexpr int STAGE_BYTES = A_BYTES + W_BYTES;          // 32 KB, a multiple of 1 KB
 constexpr int BASE_COL = 256;                // tensor-memory columns of the two base accumulators (NB each)
-constexpr int XS = BM + 1;                    // row stride of X and Nz: a lane per position writes without bank conflicts
+constexpr int RPW = BM / NEW;                // sample rows per epilogue warp
 constexpr int MAX_STAGES = 10;
 constexpr int SMEM_DYN_MAX = 227 * 1024 - 4 * 1024;
 
@@ -53,10 +58,12 @@ struct SwShared {
     int kbs[JS_MAXL + 1], ub0[JS_MAXL + 1];  // current base: its K blocks per layer (0: none), its first unit
     uint32_t tmem_base;
     int stop;
+    int gave_up[2];                          // an epilogue warp's wait ran out: for a base, for a group
     float lut_s[2];
     // geometry of the current group, per GEMM l (activations a[l] -> a[l+1])
     int kin0[JS_MAXL + 1], nin[JS_MAXL + 1], u0[JS_MAXL + 1], nu[JS_MAXL + 1], kb_n[JS_MAXL + 1];
     int cs[JS_MAXL + 1][GMAX + 2];           // cs[l][i] = units of a[l] with degree <= t0 + i   (l >= 1)
+    uint32_t pk[GMAX];                       // position i completes one unit in every layer: their indices, a byte each; else ~0
     float bias_s[JS_MAXL + 1][NUP];
 };
 
@@ -83,86 +90,6 @@ __device__ __forceinline__ float lds_f(uint32_t a)
 }
 __device__ __forceinline__ void sts_f(uint32_t a, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory"); }
 
-// Position i of the group when every hidden layer gains exactly one unit there (byte l of jn_packed: its index among
-// the group's units of a[l+1]).  The chain  symbol -> unit of a[1] -> ... -> unit of a[L]  is one scalar
-// fused multiply-add and one activation per layer: the unit's running sum and the one weight are
-// loaded beforehand, so no shared-memory round trip sits between two layers.  The additions to the
-// running sums of everything else in the group (32 per layer) come after the chain, the loads of one
-// layer issued before the arithmetic of the layer below: a warp issues in order, and with one warp
-// per scheduler nothing else hides a load.  Every running sum receives exactly the operations, in
-// exactly the order, of the general path (SweepEngine::scatter).  vbase: the thread's row in slot 0 of V.
-template <int L>
-__device__ __forceinline__ void position_one_each(uint32_t wbase, uint32_t vbase, int act, int i, float enc, int row,
-                                               uint32_t jn_packed)
-{
-    const int sw7 = row & 7;
-    int jn[L];
-#pragma unroll
-    for (int l = 0; l < L; ++l) jn[l] = (int)((jn_packed >> (8 * l)) & 255u);
-    float p[L], ws[L], val[L + 1];
-    uint32_t w4[L + 1], pa[L];
-    int kw7[L + 1];                                                 // the weight rows' chunk permutation
-#pragma unroll
-    for (int l = 0; l <= L; ++l) {
-        const int k = l == 0 ? i : jn[l - 1];                      // this position's source in a[l]
-        w4[l] = wbase + 4u * (uint32_t)((l * NUP + k) * NUP);
-        kw7[l] = k & 7;
-    }
-#pragma unroll
-    for (int l = 0; l < L; ++l) {
-        pa[l] = vbase + 4u * (uint32_t)(l * BM * NUP + ((((jn[l] >> 2) ^ sw7) << 2) | (jn[l] & 3)));
-        p[l] = lds_f(pa[l]);
-        ws[l] = lds_f(w4[l] + 4u * (uint32_t)((((jn[l] >> 2) ^ kw7[l]) << 2) | (jn[l] & 3)));
-    }
-    val[0] = enc;
-#pragma unroll
-    for (int l = 0; l < L; ++l)
-        val[l + 1] = __bfloat162float(__float2bfloat16_rn(tc_act_fn(act, fmaf(ws[l], val[l], p[l]))));
-    // half a layer (four 16-byte chunks, 16 targets) at a time, two register buffers in turn
-    constexpr int HC = NUP / 8;
-    float4 w[2][HC], x[2][HC];
-    // a half whose 16 targets all lie below the first unit that may read the source is left out (the
-    // same for every thread: the targets' masked weights are zero)
-    bool live[2 * (L + 1)];
-#pragma unroll
-    for (int l = 0; l <= L; ++l) {
-        const int jmin = l < L ? jn[l] : i + 1;
-        live[2 * l] = jmin < 4 * HC;
-        live[2 * l + 1] = true;
-    }
-#pragma unroll
-    for (int h = 0; h <= 2 * (L + 1); ++h) {
-        if (h < 2 * (L + 1) && live[h]) {
-            // loads of half-step h, issued before the arithmetic of half-step h - 1
-            const int l = h >> 1, cb = (h & 1) * HC;
-            const uint32_t v4 = vbase + 4u * (uint32_t)(l * BM * NUP);
-#pragma unroll
-            for (int c = 0; c < HC; ++c)
-                w[h & 1][c] = lds_f4(w4[l] + 16u * (uint32_t)((cb + c) ^ kw7[l]));
-#pragma unroll
-            for (int c = 0; c < HC; ++c)
-                x[h & 1][c] = lds_f4(v4 + 16u * (uint32_t)((cb + c) ^ sw7));
-        }
-        if (h >= 1 && live[h - 1]) {
-            const int g = h - 1, l = g >> 1, cb = (g & 1) * HC;
-            const uint32_t v4 = vbase + 4u * (uint32_t)(l * BM * NUP);
-            const float s = val[l];
-#pragma unroll
-            for (int c = 0; c < HC; ++c) {
-                float4 xv = x[g & 1][c];
-                const float4 wv = w[g & 1][c];
-                xv.x = fmaf(wv.x, s, xv.x);
-                xv.y = fmaf(wv.y, s, xv.y);
-                xv.z = fmaf(wv.z, s, xv.z);
-                xv.w = fmaf(wv.w, s, xv.w);
-                sts_f4(v4 + 16u * (uint32_t)((cb + c) ^ sw7), xv);
-            }
-        }
-        // the unit's activation replaces its running sum (after both halves of its layer are stored)
-        if (h >= 1 && ((h - 1) & 1) == 1 && (h - 1) / 2 < L) sts_f(pa[(h - 1) / 2 < L ? (h - 1) / 2 : 0], val[(h - 1) / 2 + 1]);
-    }
-}
-
 struct SweepEngine {
     const MadeDev &m;
     const SweepDev &sw;
@@ -171,9 +98,7 @@ struct SweepEngine {
     uint8_t *ring;
     float *V;            // [L+1][128 rows][NUP]: running sums, then activations, of the group's units; a row's
                          // eight 16-byte chunks are permuted by the row number (conflict-free 16-byte accesses)
-    float *X;            // [NUP][XS]: encodings of the group's positions
     float *Wg;           // [L+1][NUP][NUP]: weights between the group's units
-    float *Nz;           // [GMAX][XS]: the group's noise
     int warp, lane;
     int stage = 0;
     uint32_t spar = 0;
@@ -194,11 +119,7 @@ struct SweepEngine {
         // (the threads fence their accesses against the asynchronous proxy before they let the loads go).
         V = reinterpret_cast<float *>(ring);
         uint8_t *p = ring + (size_t)sw.ring_bytes;
-        X = reinterpret_cast<float *>(p);
-        p += (size_t)NUP * XS * 4;
         Wg = reinterpret_cast<float *>(p);
-        p += (size_t)(m.L + 1) * NUP * NUP * 4;
-        Nz = reinterpret_cast<float *>(p);
     }
 
     // optional device timeline (JS_OPT_TRACE, js_get_trace) of the first CTA: one row of stamps per group;
@@ -271,8 +192,8 @@ struct SweepEngine {
             for (int i = 0; i < run; ++i, ++kb) {
                 if (elect_one()) {
                     mbar_expect_tx(&sh.full[stage], bytes);
-                    if (kb < kb_old) tma_load_2d(smem_u32(stage_a(stage)), sw.tmAold + l, &sh.full[stage], kb * BK, rt * BM);
-                    else tma_load_3d(smem_u32(stage_a(stage)), sw.tmF + l, &sh.full[stage], (kb - kb_old) * BK, 0, slot);
+                    if (kb < kb_old) tma_load_2d(smem_u32(stage_a(stage)), sw.tmAold + sw.rj_idx * (m.L + 1) + l, &sh.full[stage], kb * BK, rt * sw.rj);
+                    else tma_load_3d(smem_u32(stage_a(stage)), sw.tmF + sw.rj_idx * (m.L + 1) + l, &sh.full[stage], (kb - kb_old) * BK, 0, slot);
                     tma_load_2d(smem_u32(stage_b(stage)), mw, &sh.full[stage], kb * BK, row0);
                 }
                 advance_stage();
@@ -319,14 +240,14 @@ struct SweepEngine {
                     const Base bs = base_of(l, s0, b);
                     for (int c = 0; c * NB < bs.nb && bs.kbs > 0 && !dead; ++c) {
                         mma_flops += 2ull * BM * BK * NB * (unsigned long long)bs.kbs;
-                        load_blocks(l, 0, bs.kbs, kb_old[l], rt, slot, sw.tmW16 + 2 * (m.L + 1) + l, bs.ub0 + c * NB, A_BYTES + NB * BK * 2);
+                        load_blocks(l, 0, bs.kbs, kb_old[l], rt, slot, sw.tmW16 + 2 * (m.L + 1) + l, bs.ub0 + c * NB, sw.rj * BK * 2 + NB * BK * 2);
                     }
                 }
             }
             for (int l = 0; l <= m.L && !dead; ++l) {
                 const Geo g = geo(l, t0, t1, hi);
                 if (g.nu == 0) continue;
-                const uint32_t bytes = A_BYTES + (uint32_t)g.npad * BK * 2;
+                const uint32_t bytes = (uint32_t)(sw.rj + g.npad) * BK * 2;
                 const int kbs = base_of(l, s0, b).kbs;
                 mma_flops += 2ull * BM * BK * (unsigned long long)g.npad * (unsigned long long)(g.kb_n - kbs);
                 // one box of 16 or of 32 weight rows (a load per 16 rows cost a fifth of the K loop)
@@ -387,7 +308,7 @@ struct SweepEngine {
     // as eight 16-byte chunks, chunk c stored at position c ^ (k & 7)
     __device__ uint32_t wrow(int l, int k) const { return smem_u32(Wg) + 4u * (uint32_t)((l * NUP + k) * NUP); }
 
-    __device__ void ep_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+    __device__ void ep_sync() { asm volatile("bar.sync 1, %0;" ::"n"(NEP) : "memory"); }
 
     // unit j of the group in layer slot l, sample row `row`: its shared-memory address
     __device__ uint32_t vat(int l, int j, int row) const
@@ -395,94 +316,77 @@ struct SweepEngine {
         return smem_u32(V) + 4u * (uint32_t)(((l * BM + row) * NUP) + ((((j >> 2) ^ (row & 7)) << 2) | (j & 3)));
     }
 
-    // source k of a[l] has the value `val`: add its contribution to the running sums of the group's units
-    // of a[l+1] (masked weights are zero where the target may not read the source)
-    // Targets below jmin cannot read this source (their degree is lower, their masked weight zero): their
-    // 16-byte chunks are left alone, which halves the shared-memory traffic that bounds the position loop.
-    __device__ void scatter(int l, int k, float val, int row, int jmin)
-    {
-        const int c0 = jmin >> 2;
-        // the row's 32 running sums as eight 16-byte accesses, all loads before all stores: one warp per
-        // scheduler cannot hide the latency of a load that waits behind a store it might alias
-        const uint32_t w4 = wrow(l, k);
-        const uint32_t v4 = smem_u32(V) + 4u * (uint32_t)((l * BM + row) * NUP);
-        const int sw7 = row & 7, kw7 = k & 7;
-        float4 w[NUP / 4], x[NUP / 4];
-#pragma unroll
-        for (int c = 0; c < NUP / 4; ++c)
-            if (c >= c0) w[c] = lds_f4(w4 + 16u * (uint32_t)(c ^ kw7));
-#pragma unroll
-        for (int c = 0; c < NUP / 4; ++c)
-            if (c >= c0) x[c] = lds_f4(v4 + 16u * (uint32_t)(c ^ sw7));
-#pragma unroll
-        for (int c = 0; c < NUP / 4; ++c) {
-            if (c < c0) continue;
-            x[c].x = fmaf(w[c].x, val, x[c].x);
-            x[c].y = fmaf(w[c].y, val, x[c].y);
-            x[c].z = fmaf(w[c].z, val, x[c].z);
-            x[c].w = fmaf(w[c].w, val, x[c].w);
-        }
-#pragma unroll
-        for (int c = 0; c < NUP / 4; ++c)
-            if (c >= c0) sts_f4(v4 + 16u * (uint32_t)(c ^ sw7), x[c]);
-    }
-
-    // n consecutive values (unit j = 0..n-1 of layer slot l, or the group's encodings when l < 0) of this
-    // thread's row as bf16 to dst[0..n): single elements up to a 16-byte boundary, then eight at a time
-    __device__ float run_val(int l, int j, int row) const { return l < 0 ? X[j * XS + row] : lds_f(vat(l, j, row)); }
-    __device__ void store_run(__nv_bfloat16 *dst, int l, int row, int n)
-    {
-        int j = 0;
-        for (; j < n && (reinterpret_cast<uintptr_t>(dst + j) & 15u) != 0; ++j) dst[j] = __float2bfloat16_rn(run_val(l, j, row));
-        for (; j + 8 <= n; j += 8) {
-            float x[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) x[i] = run_val(l, j + i, row);
-            *reinterpret_cast<uint4 *>(dst + j) = make_uint4(pack_bf16x2(x[0], x[1]), pack_bf16x2(x[2], x[3]),
-                                                             pack_bf16x2(x[4], x[5]), pack_bf16x2(x[6], x[7]));
-        }
-        for (; j < n; ++j) dst[j] = __float2bfloat16_rn(run_val(l, j, row));
-    }
-
     // start of a job: the job's buffer F holds, per layer, the units from the K block that contains
     // the block's first old unit onwards: copies of the old activations up to degree a, zeros after
     __device__ void job_init(int rt, int slot, int a, int b)
     {
-        const int row = (warp & 3) * 32 + lane;
-        const size_t esz = 2;
-        for (int l = 0; l <= m.L; ++l) {
-            const int k_old = cnt(l, a), kb0 = (k_old / BK) * BK;
-            const int ncopy = k_old - kb0;
-            const int cols = min(sw.WF[l], ((cnt(l, min(b, m.T)) - kb0 + BK - 1) / BK) * BK);
-            __nv_bfloat16 *f = sw.F[l] + ((size_t)slot * BM + row) * sw.WF[l];
-            const __nv_bfloat16 *old = (const __nv_bfloat16 *)m.a[l] + (size_t)(rt * BM + row) * m.n[l] + kb0;
-            for (int c = 0; c < cols; c += 8) {
-                uint4 v = make_uint4(0u, 0u, 0u, 0u);
-                if (c + 8 <= ncopy) {
-                    v = __ldcg(reinterpret_cast<const uint4 *>(old + c));
-                } else if (c < ncopy) {
-                    __nv_bfloat16 tmp[8];
-                    for (int i = 0; i < 8; ++i) tmp[i] = c + i < ncopy ? old[c + i] : __float2bfloat16_rn(0.0f);
-                    v = *reinterpret_cast<const uint4 *>(tmp);
+        const int row = (warp & 3) * 32 + lane, part = (warp - 2) >> 2;
+        if (row < sw.rj)
+            for (int l = 0; l <= m.L; ++l) {
+                const int k_old = cnt(l, a), kb0 = (k_old / BK) * BK;
+                const int ncopy = k_old - kb0;
+                const int cols = min(sw.WF[l], ((cnt(l, min(b, m.T)) - kb0 + BK - 1) / BK) * BK);
+                __nv_bfloat16 *f = sw.F[l] + ((size_t)slot * BM + row) * sw.WF[l];
+                const __nv_bfloat16 *old = (const __nv_bfloat16 *)m.a[l] + (size_t)(rt * sw.rj + row) * m.n[l] + kb0;
+                for (int c = 8 * part; c < cols; c += 8 * (NEW / 4)) {
+                    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+                    if (c + 8 <= ncopy) {
+                        v = __ldcg(reinterpret_cast<const uint4 *>(old + c));
+                    } else if (c < ncopy) {
+                        __nv_bfloat16 tmp[8];
+                        for (int i = 0; i < 8; ++i) tmp[i] = c + i < ncopy ? old[c + i] : __float2bfloat16_rn(0.0f);
+                        v = *reinterpret_cast<const uint4 *>(tmp);
+                    }
+                    *reinterpret_cast<uint4 *>(f + c) = v;
                 }
-                *reinterpret_cast<uint4 *>(f + c) = v;
             }
-            (void)esz;
-        }
         fence_proxy_async();
         __syncwarp();
         if (lane == 0) mbar_arrive(&sh.gdone);
     }
 
-    // LT: the number of hidden layers if the one-unit-per-layer path is compiled for it (1 .. 4), else 0
-    template <int LT>
-    __device__ void epilogue(int rt, int slot, int a, int b, bool &row_changed)
+    // The value of unit j of layer slot l (lane j of the running sums S) for the warp's rows, rounded like any activation, in
+    // every lane; it replaces the running sum.  Two rows travel in one shuffle.
+    __device__ __forceinline__ void complete_unit(float (&S)[RPW], int j, float (&val)[RPW]) const
     {
-        const int q = warp & 3, row = q * 32 + lane, tid = threadIdx.x - 64;
-        const int smp = rt * BM + row;
-        const bool valid = smp < r.batch;
-        const int L = m.L;
-        int kb_old[JS_MAXL + 1];
+        uint32_t p[RPW / 2];
+        if (m.act == JS_ACT_RELU) {
+#pragma unroll
+            for (int c = 0; c < RPW / 2; ++c) p[c] = pack_bf16x2(tc_act_fn(JS_ACT_RELU, S[2 * c]), tc_act_fn(JS_ACT_RELU, S[2 * c + 1]));
+        } else {
+#pragma unroll
+            for (int c = 0; c < RPW / 2; ++c) p[c] = pack_bf16x2(tc_act_fn(JS_ACT_GELU_TANH, S[2 * c]), tc_act_fn(JS_ACT_GELU_TANH, S[2 * c + 1]));
+        }
+#pragma unroll
+        for (int c = 0; c < RPW / 2; ++c) {
+            p[c] = __shfl_sync(0xffffffffu, p[c], j);
+            val[2 * c] = __uint_as_float(p[c] << 16);
+            val[2 * c + 1] = __uint_as_float(p[c] & 0xffff0000u);
+        }
+        if (lane == j)
+#pragma unroll
+            for (int rr = 0; rr < RPW; ++rr) S[rr] = val[rr];
+    }
+    // weight from source k of a[l] to this lane's target
+    __device__ __forceinline__ float weight(int l, int k) const
+    {
+        return lds_f(smem_u32(Wg) + 4u * (uint32_t)((l * NUP + k) * NUP + ((((lane >> 2) ^ (k & 7)) << 2) | (lane & 3))));
+    }
+    static __device__ __forceinline__ void add(float (&S)[RPW], float w, const float (&val)[RPW])
+    {
+#pragma unroll
+        for (int rr = 0; rr < RPW; ++rr) S[rr] = fmaf(w, val[rr], S[rr]);
+    }
+
+    template <int L>
+    __device__ void epilogue(int rt, int slot, int a, int b, uint32_t &changed)
+    {
+        const int q = warp & 3, part = (warp - 2) >> 2, row = q * 32 + lane, tid = threadIdx.x - 64;
+        const int r0 = RPW * (warp - 2);                 // this warp's rows in the position loop
+        const bool active = r0 < sw.rj;
+        const float lut0 = sh.lut_s[0], lut1 = sh.lut_s[1];
+        int kb_old[L + 1];
+#pragma unroll
         for (int l = 0; l <= L; ++l) kb_old[l] = cnt(l, a) / BK;
         job_init(rt, slot, a, b);
         for (int t0 = a; t0 < b && !dead; t0 += sw.G) {
@@ -496,91 +400,73 @@ struct SweepEngine {
                 const Base bs = base_of(tid, s0, b);
                 sh.kbs[tid] = bs.kbs; sh.ub0[tid] = bs.ub0;
             }
-            for (int i = tid; i < (L + 1) * (GMAX + 2); i += 128) {
+            for (int i = tid; i < (L + 1) * (GMAX + 2); i += NEP) {
                 const int l = i / (GMAX + 2), k = i % (GMAX + 2);
                 if (l >= 1) sh.cs[l][k] = cnt(l, min(t0 + k, m.T));
+            }
+            // noise and the symbols the positions hold now, lane = position (asked for now, used behind the GEMMs)
+            float nz[RPW];
+            uint32_t xold = 0;                           // bit rr: row rr's symbol; bit 8 + rr: it holds no symbol yet
+#pragma unroll
+            for (int rr = 0; rr < RPW; ++rr) {
+                const int s2 = rt * sw.rj + r0 + rr;
+                const bool in = active && s2 < r.batch && lane < ng;
+                nz[rr] = in ? __ldg(r.noise + (size_t)s2 * m.T + t0 + lane) : 0.0f;
+                const uint32_t xo = in ? r.x[(size_t)s2 * m.T + t0 + lane] : 0u;
+                xold |= (xo & 1u) << rr | (uint32_t)(xo > 1u) << (8 + rr);
             }
             ep_sync();
             if (tid == 0) trace(7);
             {
-                // Every global load of the thread first, the stores to shared memory after them: the compiler
-                // may not move a load across a store it cannot tell apart, and one round trip per layer and
-                // per table would cost more than the group's GEMMs.
-                // thread = (source k = lane, chunk of four targets): four loads (each coalesced over the
-                // warp's sources), one 16-byte store to row k of the source-major table, chunks permuted by
-                // the row number like the running sums (a new activation updates all its targets)
-                constexpr int LB = 3;            // layers per round trip
-                for (int l0 = 0; l0 <= L; l0 += LB) {
-                    __nv_bfloat16 wv[LB][2][4];
-                    float bv[LB];
+                // warp = two targets per layer, lane = source: every load of the thread first (coalesced over the sources),
+                // the stores to the source-major table after them
+                const int j = 2 * (warp - 2);
+                __nv_bfloat16 wv[L + 1][2];
 #pragma unroll
-                    for (int dl = 0; dl < LB; ++dl) {
-                        const int l = min(l0 + dl, L);
-                        const int nu = sh.nu[l], nin = sh.nin[l], u0 = sh.u0[l], kin0 = sh.kin0[l];
-                        const __nv_bfloat16 *Wl = (const __nv_bfloat16 *)m.W[l];
-                        const int K = m.n[l];
+                for (int l = 0; l <= L; ++l) {
+                    const __nv_bfloat16 *Wl = (const __nv_bfloat16 *)m.W[l] + (size_t)(sh.u0[l] + j) * m.n[l] + sh.kin0[l] + lane;
 #pragma unroll
-                        for (int e = 0; e < 2; ++e)
-#pragma unroll
-                            for (int jj = 0; jj < 4; ++jj) {
-                                const int j = 4 * (q + 4 * e) + jj;
-                                wv[dl][e][jj] = (j < nu && lane < nin) ? Wl[(size_t)(u0 + j) * K + kin0 + lane]
-                                                                       : __float2bfloat16_rn(0.0f);
-                            }
-                        bv[dl] = (tid < NUP && tid < nu) ? m.bias[l][u0 + tid] : 0.0f;
-                    }
-#pragma unroll
-                    for (int dl = 0; dl < LB; ++dl) {
-                        const int l = min(l0 + dl, L);           // past the last layer: the last layer again
-#pragma unroll
-                        for (int e = 0; e < 2; ++e)
-                            sts_f4(wrow(l, lane) + 16u * (uint32_t)((q + 4 * e) ^ (lane & 7)),
-                                   make_float4(__bfloat162float(wv[dl][e][0]), __bfloat162float(wv[dl][e][1]),
-                                               __bfloat162float(wv[dl][e][2]), __bfloat162float(wv[dl][e][3])));
-                        if (tid < NUP) sh.bias_s[l][tid] = bv[dl];
-                    }
+                    for (int jj = 0; jj < 2; ++jj)
+                        wv[l][jj] = (j + jj < sh.nu[l] && lane < sh.nin[l]) ? Wl[(size_t)jj * m.n[l]] : __float2bfloat16_rn(0.0f);
                 }
-            }
-            if (tid == 0) trace(8);
-            {
-                // noise and the symbols the group's positions hold now (for the change flags; 255 where there
-                // is none): a warp takes its 32 rows in turn, lane = position, so that a load instruction
-                // touches one line instead of 32; eight rows' loads before their stores
-#pragma unroll 1
-                for (int r0 = 0; r0 < 32; r0 += 8) {
-                    float nv[8];
-                    uint8_t xo[8];
+                float bv = 0.0f;
+                if (tid < (L + 1) * NUP && (tid & 31) < sh.nu[tid >> 5]) bv = __ldg(m.bias[tid >> 5] + sh.u0[tid >> 5] + (tid & 31));
 #pragma unroll
-                    for (int rr = 0; rr < 8; ++rr) {
-                        const int s2 = rt * BM + q * 32 + r0 + rr;
-                        const bool in = s2 < r.batch && lane < ng;
-                        nv[rr] = in ? __ldg(r.noise + (size_t)s2 * m.T + t0 + lane) : 0.0f;
-                        xo[rr] = in ? r.x[(size_t)s2 * m.T + t0 + lane] : (uint8_t)255;
-                    }
+                for (int l = 0; l <= L; ++l) {
+                    const uint32_t at = wrow(l, lane) + 16u * (uint32_t)((j >> 2) ^ (lane & 7)) + 4u * (uint32_t)(j & 3);
+                    sts_f(at, __bfloat162float(wv[l][0]));
+                    sts_f(at + 4u, __bfloat162float(wv[l][1]));
+                }
+                if (tid < (L + 1) * NUP) sh.bias_s[tid >> 5][tid & 31] = bv;
+                if (tid < ng) {
+                    uint32_t pk = 0;
+                    bool one_each = L <= 4;
 #pragma unroll
-                    for (int rr = 0; rr < 8; ++rr) {
-                        Nz[lane * XS + q * 32 + r0 + rr] = nv[rr];
-                        X[lane * XS + q * 32 + r0 + rr] = (float)xo[rr];
+                    for (int l = 0; l < L; ++l) {
+                        const int ca = sh.cs[l + 1][tid];
+                        one_each = one_each && sh.cs[l + 1][tid + 1] - ca == 1;
+                        if (l < 4) pk |= (uint32_t)(ca - sh.u0[l]) << (8 * l);
                     }
+                    sh.pk[tid] = one_each ? pk : ~0u;
                 }
             }
             ep_sync();
             if (tid == 0) trace(2);
             // ---- a new base: its sums go from tensor memory to this job's part of S, chunk by chunk, as the
-            // MMAs deliver them; thread = sample row writes, and later reads, only its own row
+            // MMAs deliver them; a warp takes 32 columns of its quadrant's rows
             if (t0 == s0) {
                 for (int l = 0; l <= L && !dead; ++l) {
                     const Base bs = base_of(l, s0, b);
                     float *Sl = sw.S + (((size_t)slot * (L + 1) + l) * sw.nbs) * BM + row;
                     for (int c = 0; c * NB < bs.nb && bs.kbs > 0; ++c) {
-                        if (!mbar_wait(&sh.bfull[bbuf], (bb_par >> bbuf) & 1u, r.ctl)) { dead = true; break; }
+                        if (!__all_sync(0xffffffffu, mbar_wait(&sh.bfull[bbuf], (bb_par >> bbuf) & 1u, r.ctl))) { dead = true; break; }
                         tc_fence_after();
-#pragma unroll 1
-                        for (int h = 0; h < NB; h += 32) {
+                        static_assert(NB == 32 * (NEW / 4), "32 columns of a chunk per warp");
+                        if (q * 32 < sw.rj) {
                             float v[32];
-                            tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(BASE_COL + bbuf * NB + h), v);
+                            tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(BASE_COL + bbuf * NB + 32 * part), v);
 #pragma unroll
-                            for (int i = 0; i < 32; ++i) Sl[(size_t)(c * NB + h + i) * BM] = v[i];
+                            for (int i = 0; i < 32; ++i) __stcg(Sl + (size_t)(c * NB + 32 * part + i) * BM, v[i]);
                         }
                         tc_fence_before();
                         __syncwarp();
@@ -589,13 +475,16 @@ struct SweepEngine {
                         bbuf ^= 1;
                     }
                 }
-                if (dead) break;
+                if (dead) sh.gave_up[0] = 1;
+                __threadfence_block();
+                ep_sync();                               // a row's sums are read by another warp of its quadrant
+                if (*(volatile int *)&sh.gave_up[0]) { dead = true; break; }     // all leave at the same place
             }
             // ---- the next group's tables (weights between its units, noise, symbols) are touched once per
             // sweep and would come from DRAM, two dependent round trips of 2.5 us each: ask for them now
             if (t1 < b) {
                 const int t2 = min(t1 + sw.G, b), hi2 = min(t2, b - 1);
-                for (int i = tid; i < (L + 1) * NUP; i += 128) {
+                for (int i = tid; i < (L + 1) * NUP; i += NEP) {
                     const int l = i / NUP, j = i % NUP;
                     const Geo g = geo(l, t1, t2, hi2);
                     if (j < g.nu && g.nin > 0) {
@@ -604,133 +493,140 @@ struct SweepEngine {
                         prefetch_l2(pw + g.nin - 1);
                     }
                 }
-                if (valid) {
+                const int row2 = tid & 127, smp = rt * sw.rj + row2, what = tid >> 7;
+                if (row2 < sw.rj && smp < r.batch) {
                     const float *np = r.noise + (size_t)smp * m.T + t1;
-                    prefetch_l2(np);
-                    prefetch_l2(np + (t2 - t1) - 1);
-                    prefetch_l2(r.x + (size_t)smp * m.T + t1);
+                    if (what == 0) prefetch_l2(np);
+                    else if (what == 1) prefetch_l2(np + (t2 - t1) - 1);
+                    else if (what == 2) prefetch_l2(r.x + (size_t)smp * m.T + t1);
                 }
             }
             // ---- prefix sums out of tensor memory
-            if (!mbar_wait(&sh.tfull, tf_par, r.ctl)) { dead = true; break; }
+            if (!__all_sync(0xffffffffu, mbar_wait(&sh.tfull, tf_par, r.ctl))) sh.gave_up[1] = 1;
             tf_par ^= 1u;
             tc_fence_after();
             if (tid == 0) trace(3);
-            for (int l = 0; l <= L; ++l) {
-                float v[32];
-                if (sh.nu[l] > 0 && sh.kb_n[l] > sh.kbs[l]) {
-                    tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(l * NUP), v);
-                } else {
+            if (q * 32 < sw.rj)
+                for (int l = part; l <= L; l += NEW / 4) {
+                    float v[32];
+                    if (sh.nu[l] > 0 && sh.kb_n[l] > sh.kbs[l]) {
+                        tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(l * NUP), v);
+                    } else {
 #pragma unroll
-                    for (int i = 0; i < 32; ++i) v[i] = 0.0f;
+                        for (int i = 0; i < 32; ++i) v[i] = 0.0f;
+                    }
+                    if (sh.kbs[l] > 0 && sh.nu[l] > 0) {
+                        // base + the group's own K blocks (in that order, always)
+                        const float *Sl = sw.S + (((size_t)slot * (L + 1) + l) * sw.nbs + (sh.u0[l] - sh.ub0[l])) * BM + row;
+                        const int nuv = sh.nu[l];
+                        float sv[32];
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) sv[i] = i < nuv ? __ldcg(Sl + (size_t)i * BM) : 0.0f;
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) v[i] = sv[i] + v[i];
+                    }
+                    // running pre-activation of every unit of the group: prefix sum + bias; the group's own
+                    // contributions are added below, each as soon as its source exists
+                    const uint32_t v4 = smem_u32(V) + 4u * (uint32_t)((l * BM + row) * NUP);
+#pragma unroll
+                    for (int c = 0; c < NUP / 4; ++c)
+                        sts_f4(v4 + 16u * (uint32_t)(c ^ (row & 7)),
+                               make_float4(v[4 * c] + sh.bias_s[l][4 * c], v[4 * c + 1] + sh.bias_s[l][4 * c + 1],
+                                           v[4 * c + 2] + sh.bias_s[l][4 * c + 2], v[4 * c + 3] + sh.bias_s[l][4 * c + 3]));
                 }
-                if (sh.kbs[l] > 0 && sh.nu[l] > 0) {
-                    // base + the group's own K blocks (in that order, always)
-                    const float *Sl = sw.S + (((size_t)slot * (L + 1) + l) * sw.nbs + (sh.u0[l] - sh.ub0[l])) * BM + row;
-                    const int nuv = sh.nu[l];
-                    float sv[32];
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) sv[i] = i < nuv ? __ldcg(Sl + (size_t)i * BM) : 0.0f;
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) v[i] = sv[i] + v[i];
-                }
-                // running pre-activation of every unit of the group: prefix sum + bias; the group's own
-                // contributions are added below, each as soon as its source exists
-                const uint32_t v4 = smem_u32(V) + 4u * (uint32_t)((l * BM + row) * NUP);
-#pragma unroll
-                for (int c = 0; c < NUP / 4; ++c)
-                    sts_f4(v4 + 16u * (uint32_t)(c ^ (row & 7)),
-                           make_float4(v[4 * c] + sh.bias_s[l][4 * c], v[4 * c + 1] + sh.bias_s[l][4 * c + 1],
-                                       v[4 * c + 2] + sh.bias_s[l][4 * c + 2], v[4 * c + 3] + sh.bias_s[l][4 * c + 3]));
-            }
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&sh.tempty);
+            ep_sync();
+            if (*(volatile int *)&sh.gave_up[1]) { dead = true; break; }
             if (tid == 0) trace(4);
-            // ---- the group's positions in order, thread = sample row.  A value that becomes known (a
-            // sampled symbol, then the hidden units it completes, layer by layer) is added at once to
-            // the running sums of everything in the group that reads it: the additions of one source
-            // are independent of each other, and each target receives its sources in index order.
-            for (int i = 0; i < ng; ++i) {
-                const int t = t0 + i;
-                // the units this position completes, per hidden layer (looked up before the sampling,
-                // which hides the loads)
-                int jn[LT > 0 ? LT : 1];
-                bool one_each = true;
+            // ---- the group's positions in order.  A value that becomes known (a sampled symbol, then the hidden units it
+            // completes, layer by layer) is added at once to the running sums of everything in the group that reads it; each
+            // target receives its sources in index order.
+            if (active) {
+                float S[L + 1][RPW];
 #pragma unroll
-                for (int l = 0; l < (LT > 0 ? LT : 1); ++l) {
-                    if (LT == 0) break;
-                    const int ca = sh.cs[l + 1][i], cb = sh.cs[l + 1][i + 1];
-                    jn[l] = ca - sh.u0[l];
-                    one_each = one_each && cb - ca == 1;
-                }
-                const float z = lds_f(vat(L, i, row));
-                const uint32_t xa = smem_u32(X) + 4u * (uint32_t)(i * XS + row);
-                const int xn = js_sample_binary(r.nk, z, lds_f(smem_u32(Nz) + 4u * (uint32_t)(i * XS + row)));
-                if (valid && (int)lds_f(xa) != xn) {
-                    r.x[(size_t)smp * m.T + t] = (uint8_t)xn;
-                    row_changed = true;
-                }
-                const float enc = sh.lut_s[xn];
-                sts_f(xa, enc);
-                if (t + 1 > hi) continue;
-                if constexpr (LT > 0) {
-                    if (one_each) {
-                        uint32_t pk = 0;                   // indices below 32, one byte each
+                for (int l = 0; l <= L; ++l)
 #pragma unroll
-                        for (int l = 0; l < LT; ++l) pk |= (uint32_t)jn[l] << (8 * l);
-                        position_one_each<LT>(smem_u32(Wg), smem_u32(V) + 4u * (uint32_t)(row * NUP), m.act, i, enc, row, pk);
-                        continue;
+                    for (int rr = 0; rr < RPW; ++rr) S[l][rr] = lds_f(vat(l, lane, r0 + rr));
+                uint32_t bits = 0;                       // of this lane's position: the rows' symbols
+                uint32_t pk_next = sh.pk[0];
+                for (int i = 0; i < ng; ++i) {
+                    const uint32_t pk = pk_next;
+                    const float w0 = weight(0, i);
+                    if (i + 1 < ng) pk_next = sh.pk[i + 1];
+                    uint32_t mk = 0;
+                    if (r.nk == JS_NOISE_LOGISTIC) {
+#pragma unroll
+                        for (int rr = 0; rr < RPW; ++rr) mk |= (uint32_t)js_sample_binary(JS_NOISE_LOGISTIC, S[L][rr], nz[rr]) << rr;
+                    } else {
+#pragma unroll
+                        for (int rr = 0; rr < RPW; ++rr) mk |= (uint32_t)js_sample_binary(JS_NOISE_UNIFORM_ICDF, S[L][rr], nz[rr]) << rr;
                     }
-                }
-                scatter(0, i, enc, row, L > 0 ? sh.cs[1][i] - sh.u0[0] : i + 1);
-                // the hidden units that position t makes computable: degree t + 1
-                for (int l = 0; l < L; ++l) {
-                    const int j0 = sh.cs[l + 1][i] - sh.u0[l], j1 = sh.cs[l + 1][i + 1] - sh.u0[l];
-                    for (int j = j0; j < j1; ++j) {
-                        const uint32_t pv = vat(l, j, row);
-                        const float val = __bfloat162float(__float2bfloat16_rn(tc_act_fn(m.act, lds_f(pv))));
-                        sts_f(pv, val);
-                        scatter(l + 1, j, val, row, l + 1 < L ? sh.cs[l + 2][i] - sh.u0[l + 1] : i + 1);
-                    }
-                }
-            }
-            if (tid == 0) trace(5);
-            // ---- the group's activations into F, for the GEMMs of the groups that follow
-            if (t1 < b) {
-                // the symbols' encodings by thread = row (their table is position-major); the hidden
-                // units by warp: its 32 rows in turn, lane = unit, so that a store instruction writes one
-                // run of 2-byte values instead of touching 32 lines
-                store_run(sw.F[0] + ((size_t)slot * BM + row) * sw.WF[0] + (t0 - kb_old[0] * BK), -1, row, ng);
-                __syncwarp();
-                for (int l = 1; l <= L; ++l) {
-                    const int n = sh.nin[l];
-                    __nv_bfloat16 *dst = sw.F[l] + ((size_t)slot * BM + q * 32) * sw.WF[l] + (sh.kin0[l] - kb_old[l] * BK) + lane;
-                    if (lane < n) {
-#pragma unroll 1
-                        for (int r0 = 0; r0 < 32; r0 += 8) {
-                            float v[8];
+                    mk = __shfl_sync(0xffffffffu, mk, i);
+                    if (lane == i) bits = mk;
+                    if (t0 + i + 1 > hi) continue;
+                    float val[RPW];
 #pragma unroll
-                            for (int rr = 0; rr < 8; ++rr) v[rr] = lds_f(vat(l - 1, lane, q * 32 + r0 + rr));
+                    for (int rr = 0; rr < RPW; ++rr) val[rr] = (mk >> rr & 1u) ? lut1 : lut0;
+                    if (pk != ~0u) {
+                        float w[L];
 #pragma unroll
-                            for (int rr = 0; rr < 8; ++rr) dst[(size_t)(r0 + rr) * sw.WF[l]] = __float2bfloat16_rn(v[rr]);
+                        for (int l = 0; l < L; ++l) w[l] = weight(l + 1, (int)(pk >> (8 * (l & 3)) & 255u));
+                        add(S[0], w0, val);
+#pragma unroll
+                        for (int l = 0; l < L; ++l) {
+                            complete_unit(S[l], (int)(pk >> (8 * (l & 3)) & 255u), val);
+                            add(S[l + 1], w[l], val);
+                        }
+                    } else {
+                        add(S[0], w0, val);
+#pragma unroll
+                        for (int l = 0; l < L; ++l) {
+                            const int j0 = sh.cs[l + 1][i] - sh.u0[l], j1 = sh.cs[l + 1][i + 1] - sh.u0[l];
+                            for (int j = j0; j < j1; ++j) {
+                                complete_unit(S[l], j, val);
+                                add(S[l + 1], weight(l + 1, j), val);
+                            }
                         }
                     }
                 }
-                fence_proxy_async();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&sh.gdone);
-            } else {
-                fence_proxy_async();          // the next job's loads will overwrite the running sums
+                if (tid == 0) trace(5);
+                // ---- symbols that changed; the group's activations into F, for the GEMMs of the groups that follow
+                if (lane < ng)
+#pragma unroll
+                    for (int rr = 0; rr < RPW; ++rr) {
+                        const int s2 = rt * sw.rj + r0 + rr;
+                        if (s2 < r.batch && (((bits ^ xold) | xold >> 8) >> rr & 1u)) {
+                            r.x[(size_t)s2 * m.T + t0 + lane] = (uint8_t)(bits >> rr & 1u);
+                            changed |= 1u << rr;
+                        }
+                    }
+                if (t1 < b) {
+                    if (lane < ng) {
+                        __nv_bfloat16 *dst = sw.F[0] + ((size_t)slot * BM + r0) * sw.WF[0] + (t0 - kb_old[0] * BK) + lane;
+#pragma unroll
+                        for (int rr = 0; rr < RPW; ++rr) dst[(size_t)rr * sw.WF[0]] = __float2bfloat16_rn((bits >> rr & 1u) ? lut1 : lut0);
+                    }
+#pragma unroll
+                    for (int l = 1; l <= L; ++l)
+                        if (lane < sh.nin[l]) {
+                            __nv_bfloat16 *dst = sw.F[l] + ((size_t)slot * BM + r0) * sw.WF[l] + (sh.kin0[l] - kb_old[l] * BK) + lane;
+#pragma unroll
+                            for (int rr = 0; rr < RPW; ++rr) dst[(size_t)rr * sw.WF[l]] = __float2bfloat16_rn(S[l - 1][rr]);
+                        }
+                }
             }
+            fence_proxy_async();              // F for the next group's loads, which also overwrite the running sums
+            __syncwarp();
+            if (t1 < b && lane == 0) mbar_arrive(&sh.gdone);
             if (tid == 0) trace(6);
             group_no++;
         }
     }
 };
 
-// LT = the model's number of hidden layers where the one-unit-per-layer path of the position loop is
-// compiled for it (1 .. 4), else 0.
+// LT = the model's number of hidden layers
 template <int LT>
 __global__ void __launch_bounds__(NTH, 1)
 made_sweep_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ SweepDev sw, const __grid_constant__ RunArgs r)
@@ -742,11 +638,12 @@ made_sweep_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ Swe
     if (threadIdx.x == 0) {
         for (int s = 0; s < MAX_STAGES; ++s) { mbar_init(&sh.full[s], 1); mbar_init(&sh.empty[s], 1); }
         mbar_init(&sh.tfull, 1);
-        mbar_init(&sh.tempty, 4);
-        mbar_init(&sh.gdone, 4);
-        for (int i = 0; i < 2; ++i) { mbar_init(&sh.bfull[i], 1); mbar_init(&sh.bempty[i], 4); }
+        mbar_init(&sh.tempty, NEW);
+        mbar_init(&sh.gdone, NEW);
+        for (int i = 0; i < 2; ++i) { mbar_init(&sh.bfull[i], 1); mbar_init(&sh.bempty[i], NEW); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async();
+        sh.gave_up[0] = sh.gave_up[1] = 0;
         sh.lut_s[0] = m.lut[0];
         sh.lut_s[1] = m.lut[1];
     }
@@ -758,7 +655,7 @@ made_sweep_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ Swe
     SweepEngine e(m, sw, r, sh, ring);
     e.tmem_base = sh.tmem_base;
     // jobs: (row tile, block), the blocks with the longest prefixes first
-    const int B = r.block, nblk = (m.T + B - 1) / B, MT = (r.batch + BM - 1) / BM;
+    const int B = r.block, nblk = (m.T + B - 1) / B, MT = (r.batch + sw.rj - 1) / sw.rj;
     const int njobs = MT * (nblk - r.blk_lo);
     for (int job = blockIdx.x; job < njobs; job += gridDim.x) {
         const int blk = nblk - 1 - job / MT, rt = job % MT;
@@ -775,10 +672,10 @@ made_sweep_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ Swe
         } else if (warp == 1) {
             e.mma_issuer(a, b);
         } else {
-            bool row_changed = false;
-            e.template epilogue<LT>(rt, blockIdx.x, a, b, row_changed);
-            const int smp = rt * BM + (warp & 3) * 32 + e.lane;
-            if (row_changed && smp < r.batch) r.smp_changed[smp] = 1;
+            uint32_t changed = 0;
+            e.template epilogue<LT>(rt, blockIdx.x, a, b, changed);
+            changed = __reduce_or_sync(0xffffffffu, changed);
+            if (e.lane < RPW && (changed >> e.lane & 1u)) r.smp_changed[rt * sw.rj + RPW * (warp - 2) + e.lane] = 1;
         }
         __syncwarp();
     }
@@ -860,7 +757,9 @@ static SweepKernelFn sweep_kernel_of(int L)
     case 2: return made_sweep_kernel<2>;
     case 3: return made_sweep_kernel<3>;
     case 4: return made_sweep_kernel<4>;
-    default: return made_sweep_kernel<0>;
+    case 5: return made_sweep_kernel<5>;
+    case 6: return made_sweep_kernel<6>;
+    default: return made_sweep_kernel<7>;
     }
 }
 
@@ -900,7 +799,7 @@ int js_sweep_prepare(js_model *mo)
     if (G < 1) return 0;
     s.G = G;
     const int v_bytes = (L + 1) * NUP * BM * 4;            // shares the ring's memory
-    const int fixed = NUP * XS * 4 + (L + 1) * NUP * NUP * 4 + GMAX * XS * 4;
+    const int fixed = (L + 1) * NUP * NUP * 4;
     s.n_stages = std::min(MAX_STAGES, (SMEM_DYN_MAX - 1024 - fixed) / STAGE_BYTES);
     if (s.n_stages < 2) return 0;
     s.ring_bytes = std::max(s.n_stages * STAGE_BYTES, (v_bytes + 1023) / 1024 * 1024);
@@ -912,7 +811,8 @@ int js_sweep_prepare(js_model *mo)
     if (sms < 1) return 0;
     s.slots = sms;
     auto fail = [&]() { cudaGetLastError(); return JS_ERR_CUDA; };
-    std::vector<CUtensorMap> mapsF(L + 1), mapsW(3 * (L + 1));       // weights: boxes of 16, of 32 and of NB rows
+    // activations: boxes of 32, 64 and 128 sample rows; weights: of 16, of 32 and of NB rows
+    std::vector<CUtensorMap> mapsA(3 * (L + 1)), mapsF(3 * (L + 1)), mapsW(3 * (L + 1));
     for (int l = 0; l <= L; ++l) {
         if (l >= 1) {
             void *p = nullptr;
@@ -933,8 +833,12 @@ int js_sweep_prepare(js_model *mo)
         {
             const cuuint64_t dims[3] = {(cuuint64_t)s.WF[l], (cuuint64_t)BM, (cuuint64_t)s.slots};
             const cuuint64_t strides[2] = {(cuuint64_t)s.WF[l] * 2, (cuuint64_t)s.WF[l] * 2 * BM};
-            const cuuint32_t box[3] = {(cuuint32_t)BK, (cuuint32_t)BM, 1};
-            if (!sweep_encode(&mapsF[l], f, 3, dims, strides, box)) return 0;
+            const cuuint64_t dimsA[2] = {(cuuint64_t)v.n[l], (cuuint64_t)mo->rows}, stridesA[1] = {(cuuint64_t)v.n[l] * 2};
+            for (int i = 0; i < 3; ++i) {
+                const cuuint32_t box[3] = {(cuuint32_t)BK, 32u << i, 1};
+                if (!sweep_encode(&mapsF[i * (L + 1) + l], f, 3, dims, strides, box)) return 0;
+                if (!sweep_encode(&mapsA[i * (L + 1) + l], v.a[l], 2, dimsA, stridesA, box)) return 0;
+            }
         }
         for (int big = 0; big < 3; ++big) {
             const cuuint64_t dims[2] = {(cuuint64_t)v.n[l], (cuuint64_t)v.n[l + 1]};
@@ -943,16 +847,19 @@ int js_sweep_prepare(js_model *mo)
             if (!sweep_encode(&mapsW[big * (L + 1) + l], v.W[l], 2, dims, strides, box)) return 0;
         }
     }
-    void *pf = nullptr, *pw = nullptr;
-    if (cudaMalloc(&pf, (L + 1) * sizeof(CUtensorMap)) != cudaSuccess) return fail();
+    void *pf = nullptr, *pw = nullptr, *pa = nullptr;
+    if (cudaMalloc(&pf, 3 * (L + 1) * sizeof(CUtensorMap)) != cudaSuccess) return fail();
     mo->allocs.push_back(pf);
+    if (cudaMalloc(&pa, 3 * (L + 1) * sizeof(CUtensorMap)) != cudaSuccess) return fail();
+    mo->allocs.push_back(pa);
+    if (cudaMemcpy(pa, mapsA.data(), 3 * (L + 1) * sizeof(CUtensorMap), cudaMemcpyHostToDevice) != cudaSuccess) return fail();
     if (cudaMalloc(&pw, 3 * (L + 1) * sizeof(CUtensorMap)) != cudaSuccess) return fail();
     mo->allocs.push_back(pw);
-    if (cudaMemcpy(pf, mapsF.data(), (L + 1) * sizeof(CUtensorMap), cudaMemcpyHostToDevice) != cudaSuccess) return fail();
+    if (cudaMemcpy(pf, mapsF.data(), 3 * (L + 1) * sizeof(CUtensorMap), cudaMemcpyHostToDevice) != cudaSuccess) return fail();
     if (cudaMemcpy(pw, mapsW.data(), 3 * (L + 1) * sizeof(CUtensorMap), cudaMemcpyHostToDevice) != cudaSuccess) return fail();
     s.tmF = (const CUtensorMap *)pf;
     s.tmW16 = (const CUtensorMap *)pw;
-    s.tmAold = mo->tc.tmA;
+    s.tmAold = (const CUtensorMap *)pa;
     {
         // base sums: per slot and layer, room for the units of GPB groups (rounded up to whole chunks)
         int nbs = NB;
@@ -986,9 +893,14 @@ int js_sweep_prepare(js_model *mo)
 // One launch: sweeps of every block >= r.blk_lo (block size r.block) for every row tile.
 int js_launch_made_sweep(const js_model *mo, const RunArgs &r, cudaStream_t stream)
 {
-    const SweepDev &s = mo->sweep;
-    const int nblk = (mo->made.T + r.block - 1) / r.block, MT = (r.batch + BM - 1) / BM;
-    const int njobs = MT * (nblk - r.blk_lo);
+    SweepDev s = mo->sweep;
+    const int nblk = (mo->made.T + r.block - 1) / r.block - r.blk_lo;
+    // Sample rows per job: as few (32, 64) as leave every job an SM of its own.  A position costs a job the chain of its
+    // layers, and beyond 32 rows the issue slots of several warps per scheduler.
+    s.rj_idx = 0;
+    while (s.rj_idx < 2 && (r.batch + (32 << s.rj_idx) - 1) / (32 << s.rj_idx) * nblk > s.slots) s.rj_idx++;
+    s.rj = 32 << s.rj_idx;
+    const int njobs = (r.batch + s.rj - 1) / s.rj * nblk;
     if (njobs < 1) return (int)cudaErrorInvalidValue;
     const int grid = std::min(njobs, s.slots);
     sweep_kernel_of(mo->made.L)<<<grid, NTH, s.smem_bytes, stream>>>(mo->made, s, r);
