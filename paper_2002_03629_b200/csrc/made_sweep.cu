@@ -17,11 +17,17 @@
 // from the job's own buffer F after it) and 16-row weight boxes, tcgen05.mma accumulates in tensor
 // memory.  What the units of the group contribute to one another is a triangular system of at most
 // 32 x 32 weights per layer, solved position by position: logit, sample against the fixed noise
-// (Appendix A.3), then the hidden units that the new symbol makes computable.  A warp takes eight sample rows,
-// lane = unit of the group, every layer's running sums in registers; a value that becomes known goes to all lanes by
-// shuffle and is added to 32 running sums by one multiply-add per row.  (With thread = row and the running sums in shared
-// memory a position moved 24 KB through it: 0.6 us for two hidden layers.)  The group's activations then go to F,
-// where the next group's GEMMs find them.
+// (Appendix A.3), then the hidden units that the new symbol makes computable.  A warp takes four or eight sample
+// rows, lane = unit of the group, every layer's running sums in registers; a value that becomes known
+// goes to all lanes by shuffle and is added to 32 running sums by one multiply-add per row.  (With thread = row and the
+// running sums in shared memory a position moved 24 KB through it: 0.6 us for two hidden layers.)  The group's
+// activations then go to F, where the next group's GEMMs find them.  What those GEMMs read of earlier groups (all full K
+// blocks below the group's first unit) does not wait for that: it is loaded and multiplied while the positions are solved.
+//
+// What bounds it: the chain of the positions.  100 samples of a 784-784-784-784 model, one block (4 jobs of 32 rows): 445 us
+// (1117 with thread = row), per group 5.7 us of positions, 2.6 us from the operands of its late K blocks to the sums, 1.6 us to
+// store its activations.  512 samples of a 4096-wide model in 32 blocks (128 jobs of 128 rows): 1281 us for three outer
+// iterations (1613); a sweep is 230 us, of which the base GEMMs of the longest prefixes take 95 and the positions 75.
 //
 // Every value is a fixed function of the iterate: the split into prefix and group depends on the
 // block size and the position alone.  Waits are bounded as in the other tensor-core kernels.
@@ -38,23 +44,23 @@
 namespace {
 
 constexpr int BM = TC_BM, BK = TC_BK;
-constexpr int NEW = 16;                      // epilogue warps: four per tensor-memory quadrant; eight sample rows each
+constexpr int NEW = 16;                      // epilogue warps: four per tensor-memory quadrant
 constexpr int NEP = 32 * NEW;
 constexpr int NTH = 64 + NEP;
 constexpr int NUP = 32;                      // most units of one layer inside a group
 constexpr int GMAX = 32;                     // most positions per group
+constexpr int WS = NUP + 1;                  // row stride of the table of weights inside a group: read by targets, written by sources
 constexpr int A_BYTES = BM * BK * 2;
 constexpr int NB = 128;                      // units per chunk of a base GEMM
 constexpr int GPB = 8;                       // groups per base: a base GEMM serves the next GPB groups
 constexpr int W_BYTES = NB * BK * 2;
 constexpr int STAGE_BYTES = A_BYTES + W_BYTES;          // 32 KB, a multiple of 1 KB
 constexpr int BASE_COL = 256;                // tensor-memory columns of the two base accumulators (NB each)
-constexpr int RPW = BM / NEW;                // sample rows per epilogue warp
 constexpr int MAX_STAGES = 10;
 constexpr int SMEM_DYN_MAX = 227 * 1024 - 4 * 1024;
 
 struct SwShared {
-    uint64_t full[MAX_STAGES], empty[MAX_STAGES], tfull, tempty, gdone, bfull[2], bempty[2];
+    uint64_t full[MAX_STAGES], empty[MAX_STAGES], tfull, tempty, vread, gdone, bfull[2], bempty[2];
     int kbs[JS_MAXL + 1], ub0[JS_MAXL + 1];  // current base: its K blocks per layer (0: none), its first unit
     uint32_t tmem_base;
     int stop;
@@ -63,7 +69,9 @@ struct SwShared {
     // geometry of the current group, per GEMM l (activations a[l] -> a[l+1])
     int kin0[JS_MAXL + 1], nin[JS_MAXL + 1], u0[JS_MAXL + 1], nu[JS_MAXL + 1], kb_n[JS_MAXL + 1];
     int cs[JS_MAXL + 1][GMAX + 2];           // cs[l][i] = units of a[l] with degree <= t0 + i   (l >= 1)
-    uint32_t pk[GMAX];                       // position i completes one unit in every layer: their indices, a byte each; else ~0
+    uint4 pk[GMAX][2];                       // units of layer slot l (a word each) that position i completes: the first one, + 32 x how
+                                             // many, + 65536 x the byte offset of the first one's weights
+    int most[GMAX];                          // most units of one layer that position i completes
     float bias_s[JS_MAXL + 1][NUP];
 };
 
@@ -88,6 +96,10 @@ __device__ __forceinline__ float lds_f(uint32_t a)
     asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
     return v;
 }
+__device__ __forceinline__ void lds_u4(uint32_t a, uint32_t *v)
+{
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(a));
+}
 __device__ __forceinline__ void sts_f(uint32_t a, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory"); }
 
 struct SweepEngine {
@@ -98,11 +110,11 @@ struct SweepEngine {
     uint8_t *ring;
     float *V;            // [L+1][128 rows][NUP]: running sums, then activations, of the group's units; a row's
                          // eight 16-byte chunks are permuted by the row number (conflict-free 16-byte accesses)
-    float *Wg;           // [L+1][NUP][NUP]: weights between the group's units
+    float *Wg;           // [L+1][NUP][WS]: weights between the group's units, [source][target]
     int warp, lane;
     int stage = 0;
     uint32_t spar = 0;
-    uint32_t tf_par = 0, te_par = 0, gd_par = 0;
+    uint32_t tf_par = 0, te_par = 0, gd_par = 0, vr_par = 0;
     int bbuf = 0;                  // base accumulator in turn; bit b of bb_par: parity of its next use
     uint32_t bb_par = 0;
     bool dead = false;
@@ -200,8 +212,8 @@ struct SweepEngine {
             }
         }
     }
-    // the MMAs of n K blocks into the accumulator d (which they start)
-    __device__ void mma_blocks(int n, uint32_t d, uint32_t idesc)
+    // the MMAs of n K blocks into the accumulator d (which they start or, with `more`, continue)
+    __device__ void mma_blocks(int n, uint32_t d, uint32_t idesc, bool more)
     {
         for (int kb = 0; kb < n;) {
             const int run = mbar_wait_run(sh.full, stage, sw.n_stages, spar, n - kb, r.ctl);
@@ -213,7 +225,7 @@ struct SweepEngine {
                 if (elect_one()) {
 #pragma unroll
                     for (int k = 0; k < BK / 16; ++k)
-                        umma_bf16(d, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), idesc, (kb > 0 || k > 0) ? 1u : 0u);
+                        umma_bf16(d, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), idesc, (more || kb > 0 || k > 0) ? 1u : 0u);
                     umma_commit(&sh.empty[stage]);
                 }
                 advance_stage();
@@ -221,13 +233,57 @@ struct SweepEngine {
         }
     }
 
+    // What the loading and the MMA warp need to know of a group, lane l for layer l (a dependent chain of loads from the
+    // unit counts; one after the other for every layer they took 1 us per group): its K blocks kb0 .. kb_n, of which those
+    // below kb_e hold no unit of the previous group.
+    struct Steps { int kb0, kb_e, kb_n, u0, nu; };
+    __device__ Steps steps_of(int a, int t0, int b) const
+    {
+        Steps g = {0, 0, 0, 0, 0};
+        if (lane > m.L) return g;
+        const int t1 = min(t0 + sw.G, b), s0 = base_start(a, t0);
+        const Geo e = geo(lane, t0, t1, min(t1, b - 1));
+        g.u0 = e.u0;
+        g.nu = e.nu;
+        if (e.nu == 0) return g;
+        g.kb0 = base_of(lane, s0, b).kbs;
+        g.kb_n = e.kb_n;
+        g.kb_e = t0 == s0 ? g.kb0 : max(g.kb0, cnt(lane, t0 - sw.G) / BK);
+        return g;
+    }
+    __device__ Steps of_layer(const Steps &g, int l) const
+    {
+        return {__shfl_sync(0xffffffffu, g.kb0, l), __shfl_sync(0xffffffffu, g.kb_e, l), __shfl_sync(0xffffffffu, g.kb_n, l),
+                __shfl_sync(0xffffffffu, g.u0, l), __shfl_sync(0xffffffffu, g.nu, l)};
+    }
+
     // ------------------------------------------------------------------ roles
+    // the K blocks of a group, those that hold units of the previous group (late) or the others
+    __device__ void load_group(const Steps &all, bool late, int kb_old_l, int rt, int slot)
+    {
+        for (int l = 0; l <= m.L && !dead; ++l) {
+            const Steps g = of_layer(all, l);
+            if (g.nu == 0) continue;
+            const int npad = (g.nu + 15) & ~15, kb = late ? g.kb_e : g.kb0, kb_end = late ? g.kb_n : g.kb_e;
+            mma_flops += 2ull * BM * BK * (unsigned long long)npad * (unsigned long long)(kb_end - kb);
+            // one box of 16 or of 32 weight rows (a load per 16 rows cost a fifth of the K loop)
+            load_blocks(l, kb, kb_end, __shfl_sync(0xffffffffu, kb_old_l, l), rt, slot, sw.tmW16 + (npad == 32 ? m.L + 1 : 0) + l, g.u0,
+                        (uint32_t)(sw.rj + npad) * BK * 2);
+        }
+    }
+
     __device__ void producer(int rt, int slot, int a, int b)
     {
-        int kb_old[JS_MAXL + 1];
-        for (int l = 0; l <= m.L; ++l) kb_old[l] = cnt(l, a) / BK;
+        const int kb_old_l = lane <= m.L ? cnt(lane, a) / BK : 0;
         for (int t0 = a; t0 < b && !dead; t0 += sw.G) {
-            const int t1 = min(t0 + sw.G, b), hi = min(t1, b - 1);
+            const Steps g = steps_of(a, t0, b);
+            if (t0 > a) {
+                // the previous group's running sums are in registers: the ring is free again
+                if (!__all_sync(0xffffffffu, mbar_wait_idle(&sh.vread, vr_par, r.ctl))) { dead = true; break; }
+                vr_par ^= 1u;
+                load_group(g, false, kb_old_l, rt, slot);
+                if (dead) break;
+            }
             // the previous group's activations (or the job's start values) are in F
             if (!__all_sync(0xffffffffu, mbar_wait_idle(&sh.gdone, gd_par, r.ctl))) { dead = true; break; }
             gd_par ^= 1u;
@@ -238,35 +294,38 @@ struct SweepEngine {
                 // the base GEMMs of the next GPB groups: NB units at a time over the full K blocks of the prefix
                 for (int l = 0; l <= m.L && !dead; ++l) {
                     const Base bs = base_of(l, s0, b);
+                    const int kb_old = __shfl_sync(0xffffffffu, kb_old_l, l);
                     for (int c = 0; c * NB < bs.nb && bs.kbs > 0 && !dead; ++c) {
                         mma_flops += 2ull * BM * BK * NB * (unsigned long long)bs.kbs;
-                        load_blocks(l, 0, bs.kbs, kb_old[l], rt, slot, sw.tmW16 + 2 * (m.L + 1) + l, bs.ub0 + c * NB, sw.rj * BK * 2 + NB * BK * 2);
+                        load_blocks(l, 0, bs.kbs, kb_old, rt, slot, sw.tmW16 + 2 * (m.L + 1) + l, bs.ub0 + c * NB, sw.rj * BK * 2 + NB * BK * 2);
                     }
                 }
             }
-            for (int l = 0; l <= m.L && !dead; ++l) {
-                const Geo g = geo(l, t0, t1, hi);
-                if (g.nu == 0) continue;
-                const uint32_t bytes = (uint32_t)(sw.rj + g.npad) * BK * 2;
-                const int kbs = base_of(l, s0, b).kbs;
-                mma_flops += 2ull * BM * BK * (unsigned long long)g.npad * (unsigned long long)(g.kb_n - kbs);
-                // one box of 16 or of 32 weight rows (a load per 16 rows cost a fifth of the K loop)
-                load_blocks(l, kbs, g.kb_n, kb_old[l], rt, slot, sw.tmW16 + (g.npad == 32 ? m.L + 1 : 0) + l, g.u0, bytes);
-            }
+            load_group(g, true, kb_old_l, rt, slot);
             group_no++;
+        }
+    }
+
+    __device__ void mma_group(const Steps &all, bool late)
+    {
+        for (int l = 0; l <= m.L && !dead; ++l) {
+            const Steps g = of_layer(all, l);
+            if (g.nu == 0) continue;
+            mma_blocks(late ? g.kb_n - g.kb_e : g.kb_e - g.kb0, tmem_base + (uint32_t)(l * NUP), instr_desc_bf16((g.nu + 15) & ~15), late && g.kb_e > g.kb0);
         }
     }
 
     __device__ void mma_issuer(int a, int b)
     {
         for (int t0 = a; t0 < b && !dead; t0 += sw.G) {
-            const int t1 = min(t0 + sw.G, b), hi = min(t1, b - 1);
+            const Steps g = steps_of(a, t0, b);
             // the epilogue has read the previous group's accumulators
             if (!__all_sync(0xffffffffu, mbar_wait_idle(&sh.tempty, te_par ^ 1u, r.ctl))) { dead = true; break; }
             te_par ^= 1u;
             tc_fence_after();
-            bool any = false;
             const int s0 = base_start(a, t0);
+            mma_group(g, false);
+            if (dead) break;
             if (t0 == s0) {
                 const uint32_t idescb = instr_desc_bf16(NB);
                 for (int l = 0; l <= m.L && !dead; ++l) {
@@ -276,7 +335,7 @@ struct SweepEngine {
                         if (!__all_sync(0xffffffffu, mbar_wait(&sh.bempty[bbuf], ((bb_par >> bbuf) & 1u) ^ 1u, r.ctl))) { dead = true; break; }
                         tc_fence_after();
                         const uint32_t d_base = tmem_base + (uint32_t)(BASE_COL + bbuf * NB);
-                        mma_blocks(bs.kbs, d_base, idescb);
+                        mma_blocks(bs.kbs, d_base, idescb, false);
                         if (dead) break;
                         if (elect_one()) umma_commit(&sh.bfull[bbuf]);
                         bb_par ^= 1u << bbuf;
@@ -285,16 +344,9 @@ struct SweepEngine {
                 }
                 if (dead) break;
             }
-            for (int l = 0; l <= m.L && !dead; ++l) {
-                const Geo g = geo(l, t0, t1, hi);
-                if (g.nu == 0) continue;
-                const uint32_t idesc = instr_desc_bf16(g.npad);
-                const uint32_t d_tmem = tmem_base + (uint32_t)(l * NUP);
-                const int kbs = base_of(l, s0, b).kbs;
-                mma_blocks(g.kb_n - kbs, d_tmem, idesc);
-                any = any || g.kb_n > kbs;
-            }
+            mma_group(g, true);
             if (dead) break;
+            const bool any = __any_sync(0xffffffffu, g.kb_n > g.kb0);
             if (elect_one()) {
                 if (any) umma_commit(&sh.tfull);
                 else mbar_arrive(&sh.tfull);      // a group with empty prefixes (the very first positions)
@@ -303,10 +355,6 @@ struct SweepEngine {
             group_no++;
         }
     }
-
-    // row k (a source among the group's units of a[l]) of the table of weights inside the group: 32 targets
-    // as eight 16-byte chunks, chunk c stored at position c ^ (k & 7)
-    __device__ uint32_t wrow(int l, int k) const { return smem_u32(Wg) + 4u * (uint32_t)((l * NUP + k) * NUP); }
 
     __device__ void ep_sync() { asm volatile("bar.sync 1, %0;" ::"n"(NEP) : "memory"); }
 
@@ -345,40 +393,150 @@ struct SweepEngine {
         if (lane == 0) mbar_arrive(&sh.gdone);
     }
 
-    // The value of unit j of layer slot l (lane j of the running sums S) for the warp's rows, rounded like any activation, in
-    // every lane; it replaces the running sum.  Two rows travel in one shuffle.
-    __device__ __forceinline__ void complete_unit(float (&S)[RPW], int j, float (&val)[RPW]) const
+    // the encodings of the rows' symbols at position i of the group, in every lane
+    template <int RPW>
+    __device__ __forceinline__ void sample(const float (&logit)[RPW], const float (&nz)[RPW], int i, float lut0, float lut1, float (&val)[RPW]) const
+    {
+        if (r.nk == JS_NOISE_LOGISTIC) {
+#pragma unroll
+            for (int rr = 0; rr < RPW; ++rr) val[rr] = __shfl_sync(0xffffffffu, logit[rr] + nz[rr], i);      // as js_sample_binary
+#pragma unroll
+            for (int rr = 0; rr < RPW; ++rr) val[rr] = val[rr] > 0.0f ? lut1 : lut0;
+        } else {
+            uint32_t mk = symbols(logit, nz);
+            mk = __shfl_sync(0xffffffffu, mk, i);
+#pragma unroll
+            for (int rr = 0; rr < RPW; ++rr) val[rr] = (mk >> rr & 1u) ? lut1 : lut0;
+        }
+    }
+    // the symbols of this lane's position, a bit per row
+    template <int RPW>
+    __device__ __forceinline__ uint32_t symbols(const float (&logit)[RPW], const float (&nz)[RPW]) const
+    {
+        uint32_t mk = 0;
+#pragma unroll
+        for (int rr = 0; rr < RPW; ++rr) mk |= (uint32_t)js_sample_binary(r.nk, logit[rr], nz[rr]) << rr;
+        return mk;
+    }
+    // Two activations that are known, as every reader sees them: rounded to bf16.
+    template <int ACT>
+    static __device__ __forceinline__ uint32_t act2(float s0, float s1)
+    {
+        if (ACT == JS_ACT_RELU) {
+            uint32_t v;
+            asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;" : "=r"(v) : "f"(s1), "f"(s0));
+            return v;
+        }
+        return pack_bf16x2(tc_act_fn(ACT, s0), tc_act_fn(ACT, s1));
+    }
+    // The value of unit j (lane j of the running sums S, which keep it: the weights from what comes later are zero) for the
+    // warp's rows, in every lane.  Two rows travel in one shuffle.
+    template <int ACT, int RPW>
+    static __device__ __forceinline__ void complete_unit(const float (&S)[RPW], int j, float (&val)[RPW])
     {
         uint32_t p[RPW / 2];
-        if (m.act == JS_ACT_RELU) {
 #pragma unroll
-            for (int c = 0; c < RPW / 2; ++c) p[c] = pack_bf16x2(tc_act_fn(JS_ACT_RELU, S[2 * c]), tc_act_fn(JS_ACT_RELU, S[2 * c + 1]));
-        } else {
-#pragma unroll
-            for (int c = 0; c < RPW / 2; ++c) p[c] = pack_bf16x2(tc_act_fn(JS_ACT_GELU_TANH, S[2 * c]), tc_act_fn(JS_ACT_GELU_TANH, S[2 * c + 1]));
-        }
+        for (int c = 0; c < RPW / 2; ++c) p[c] = act2<ACT>(S[2 * c], S[2 * c + 1]);
 #pragma unroll
         for (int c = 0; c < RPW / 2; ++c) {
             p[c] = __shfl_sync(0xffffffffu, p[c], j);
             val[2 * c] = __uint_as_float(p[c] << 16);
             val[2 * c + 1] = __uint_as_float(p[c] & 0xffff0000u);
         }
-        if (lane == j)
-#pragma unroll
-            for (int rr = 0; rr < RPW; ++rr) S[rr] = val[rr];
     }
-    // weight from source k of a[l] to this lane's target
-    __device__ __forceinline__ float weight(int l, int k) const
+    // Units u % 32 and, with TWO, (u + 1) % 32 of S, of which as many as bits 5 and 6 of u say are complete, added to the
+    // running sums of the next layer.
+    template <int ACT, bool TWO, int RPW>
+    static __device__ __forceinline__ void complete_units(const float (&S)[RPW], uint32_t u, float (&next)[RPW], float w0, float w1)
     {
-        return lds_f(smem_u32(Wg) + 4u * (uint32_t)((l * NUP + k) * NUP + ((((lane >> 2) ^ (k & 7)) << 2) | (lane & 3))));
+        const bool one = (u & 96u) != 0u, two = (u & 64u) != 0u;
+        uint32_t p[RPW / 2], p1[RPW / 2];
+#pragma unroll
+        for (int c = 0; c < RPW / 2; ++c) p[c] = act2<ACT>(S[2 * c], S[2 * c + 1]);
+#pragma unroll
+        for (int c = 0; c < RPW / 2; ++c) {
+            if (TWO) p1[c] = __shfl_sync(0xffffffffu, p[c], (int)u + 1);
+            p[c] = __shfl_sync(0xffffffffu, p[c], (int)u);
+        }
+#pragma unroll
+        for (int c = 0; c < RPW / 2; ++c) {
+            const float n0 = one ? fmaf(w0, __uint_as_float(p[c] << 16), next[2 * c]) : next[2 * c];
+            const float n1 = one ? fmaf(w0, __uint_as_float(p[c] & 0xffff0000u), next[2 * c + 1]) : next[2 * c + 1];
+            next[2 * c] = TWO && two ? fmaf(w1, __uint_as_float(p1[c] << 16), n0) : n0;
+            next[2 * c + 1] = TWO && two ? fmaf(w1, __uint_as_float(p1[c] & 0xffff0000u), n1) : n1;
+        }
     }
+    // shared-memory address of the weight from source k of a[l] to target j
+    __device__ __forceinline__ uint32_t wat(int l, int k, int j) const { return smem_u32(Wg) + 4u * (uint32_t)((l * NUP + k) * WS + j); }
+    template <int RPW>
     static __device__ __forceinline__ void add(float (&S)[RPW], float w, const float (&val)[RPW])
     {
 #pragma unroll
         for (int rr = 0; rr < RPW; ++rr) S[rr] = fmaf(w, val[rr], S[rr]);
     }
 
-    template <int L>
+    // The positions of a group in order: S = the running sums of the warp's rows.  Afterwards every lane's S are those of its
+    // units and of its position: what comes later has weight zero there.
+    template <int L, int RPW, int ACT>
+    __device__ __forceinline__ void solve(float (&S)[L + 1][RPW], const float (&nz)[RPW], int ng, bool last) const
+    {
+        const int most = __reduce_max_sync(0xffffffffu, lane < ng ? sh.most[lane] : 0);
+        if (most <= 1) {
+            solve_few<L, RPW, ACT, false>(S, nz, ng, last);
+        } else if (most == 2) {
+            solve_few<L, RPW, ACT, true>(S, nz, ng, last);
+        } else {
+            const float lut0 = sh.lut_s[0], lut1 = sh.lut_s[1];
+            for (int i = 0; i < ng; ++i) {
+                if (last && i == ng - 1) break;
+                float val[RPW];
+                sample(S[L], nz, i, lut0, lut1, val);
+                add(S[0], lds_f(wat(0, i, lane)), val);
+#pragma unroll
+                for (int l = 0; l < L; ++l) {
+                    const int j0 = sh.cs[l + 1][i] - sh.u0[l], j1 = sh.cs[l + 1][i + 1] - sh.u0[l];
+                    for (int j = j0; j < j1; ++j) {
+                        complete_unit<ACT>(S[l], j, val);
+                        add(S[l + 1], lds_f(wat(l + 1, j, lane)), val);
+                    }
+                }
+            }
+        }
+    }
+    // The same where a position completes at most one (TWO: two) units of a layer: no branch.  With one warp per scheduler a
+    // position costs the chain of its shuffles (some 200 cycles for two layers), with four of them the instructions: 11 or 16
+    // a row and 35 besides.
+    template <int L, int RPW, int ACT, bool TWO>
+    __device__ __forceinline__ void solve_few(float (&S)[L + 1][RPW], const float (&nz)[RPW], int ng, bool last) const
+    {
+        const float lut0 = sh.lut_s[0], lut1 = sh.lut_s[1];
+        const uint32_t wl = wat(0, 0, lane), pks = smem_u32(sh.pk);
+        uint32_t pk[8];
+        lds_u4(pks, pk);
+        if (L > 4) lds_u4(pks + 16u, pk + 4);
+        for (int i = 0; i < ng; ++i) {
+            if (last && i == ng - 1) break;
+            float w[L + 1][2];                           // asked for before the symbol is known
+            w[0][0] = lds_f(wl + (uint32_t)(i * WS * 4));
+            uint32_t u[L];
+#pragma unroll
+            for (int l = 0; l < L; ++l) {
+                u[l] = pk[l];
+                w[l + 1][0] = lds_f(wl + (u[l] >> 16));
+                w[l + 1][1] = TWO ? lds_f(wl + (u[l] >> 16) + WS * 4) : 0.0f;
+            }
+            const uint32_t at = pks + 32u * (uint32_t)min(i + 1, GMAX - 1);
+            lds_u4(at, pk);
+            if (L > 4) lds_u4(at + 16u, pk + 4);
+            float val[RPW];
+            sample(S[L], nz, i, lut0, lut1, val);
+            add(S[0], w[0][0], val);
+#pragma unroll
+            for (int l = 0; l < L; ++l) complete_units<ACT, TWO>(S[l], u[l], S[l + 1], w[l + 1][0], w[l + 1][1]);
+        }
+    }
+
+    template <int L, int RPW>
     __device__ void epilogue(int rt, int slot, int a, int b, uint32_t &changed)
     {
         const int q = warp & 3, part = (warp - 2) >> 2, row = q * 32 + lane, tid = threadIdx.x - 64;
@@ -433,21 +591,22 @@ struct SweepEngine {
                 if (tid < (L + 1) * NUP && (tid & 31) < sh.nu[tid >> 5]) bv = __ldg(m.bias[tid >> 5] + sh.u0[tid >> 5] + (tid & 31));
 #pragma unroll
                 for (int l = 0; l <= L; ++l) {
-                    const uint32_t at = wrow(l, lane) + 16u * (uint32_t)((j >> 2) ^ (lane & 7)) + 4u * (uint32_t)(j & 3);
-                    sts_f(at, __bfloat162float(wv[l][0]));
-                    sts_f(at + 4u, __bfloat162float(wv[l][1]));
+                    sts_f(wat(l, lane, j), __bfloat162float(wv[l][0]));
+                    sts_f(wat(l, lane, j + 1), __bfloat162float(wv[l][1]));
                 }
                 if (tid < (L + 1) * NUP) sh.bias_s[tid >> 5][tid & 31] = bv;
                 if (tid < ng) {
-                    uint32_t pk = 0;
-                    bool one_each = L <= 4;
+                    uint32_t pk[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+                    int most = 0;
 #pragma unroll
                     for (int l = 0; l < L; ++l) {
-                        const int ca = sh.cs[l + 1][tid];
-                        one_each = one_each && sh.cs[l + 1][tid + 1] - ca == 1;
-                        if (l < 4) pk |= (uint32_t)(ca - sh.u0[l]) << (8 * l);
+                        const int n = sh.cs[l + 1][tid + 1] - sh.cs[l + 1][tid], j = (sh.cs[l + 1][tid] - sh.u0[l]) & 31;
+                        most = max(most, n);
+                        pk[l] = (uint32_t)(j | min(n, 2) << 5 | ((l + 1) * NUP + j) * WS * 4 << 16);
                     }
-                    sh.pk[tid] = one_each ? pk : ~0u;
+                    sh.pk[tid][0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                    sh.pk[tid][1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+                    sh.most[tid] = most;
                 }
             }
             ep_sync();
@@ -543,91 +702,60 @@ struct SweepEngine {
             // ---- the group's positions in order.  A value that becomes known (a sampled symbol, then the hidden units it
             // completes, layer by layer) is added at once to the running sums of everything in the group that reads it; each
             // target receives its sources in index order.
-            if (active) {
-                float S[L + 1][RPW];
+            float S[L + 1][RPW];
 #pragma unroll
-                for (int l = 0; l <= L; ++l)
+            for (int l = 0; l <= L; ++l)
 #pragma unroll
-                    for (int rr = 0; rr < RPW; ++rr) S[l][rr] = lds_f(vat(l, lane, r0 + rr));
-                uint32_t bits = 0;                       // of this lane's position: the rows' symbols
-                uint32_t pk_next = sh.pk[0];
-                for (int i = 0; i < ng; ++i) {
-                    const uint32_t pk = pk_next;
-                    const float w0 = weight(0, i);
-                    if (i + 1 < ng) pk_next = sh.pk[i + 1];
-                    uint32_t mk = 0;
-                    if (r.nk == JS_NOISE_LOGISTIC) {
-#pragma unroll
-                        for (int rr = 0; rr < RPW; ++rr) mk |= (uint32_t)js_sample_binary(JS_NOISE_LOGISTIC, S[L][rr], nz[rr]) << rr;
-                    } else {
-#pragma unroll
-                        for (int rr = 0; rr < RPW; ++rr) mk |= (uint32_t)js_sample_binary(JS_NOISE_UNIFORM_ICDF, S[L][rr], nz[rr]) << rr;
-                    }
-                    mk = __shfl_sync(0xffffffffu, mk, i);
-                    if (lane == i) bits = mk;
-                    if (t0 + i + 1 > hi) continue;
-                    float val[RPW];
-#pragma unroll
-                    for (int rr = 0; rr < RPW; ++rr) val[rr] = (mk >> rr & 1u) ? lut1 : lut0;
-                    if (pk != ~0u) {
-                        float w[L];
-#pragma unroll
-                        for (int l = 0; l < L; ++l) w[l] = weight(l + 1, (int)(pk >> (8 * (l & 3)) & 255u));
-                        add(S[0], w0, val);
-#pragma unroll
-                        for (int l = 0; l < L; ++l) {
-                            complete_unit(S[l], (int)(pk >> (8 * (l & 3)) & 255u), val);
-                            add(S[l + 1], w[l], val);
-                        }
-                    } else {
-                        add(S[0], w0, val);
-#pragma unroll
-                        for (int l = 0; l < L; ++l) {
-                            const int j0 = sh.cs[l + 1][i] - sh.u0[l], j1 = sh.cs[l + 1][i + 1] - sh.u0[l];
-                            for (int j = j0; j < j1; ++j) {
-                                complete_unit(S[l], j, val);
-                                add(S[l + 1], weight(l + 1, j), val);
-                            }
-                        }
-                    }
-                }
-                if (tid == 0) trace(5);
-                // ---- symbols that changed; the group's activations into F, for the GEMMs of the groups that follow
-                if (lane < ng)
-#pragma unroll
-                    for (int rr = 0; rr < RPW; ++rr) {
-                        const int s2 = rt * sw.rj + r0 + rr;
-                        if (s2 < r.batch && (((bits ^ xold) | xold >> 8) >> rr & 1u)) {
-                            r.x[(size_t)s2 * m.T + t0 + lane] = (uint8_t)(bits >> rr & 1u);
-                            changed |= 1u << rr;
-                        }
-                    }
-                if (t1 < b) {
-                    if (lane < ng) {
-                        __nv_bfloat16 *dst = sw.F[0] + ((size_t)slot * BM + r0) * sw.WF[0] + (t0 - kb_old[0] * BK) + lane;
-#pragma unroll
-                        for (int rr = 0; rr < RPW; ++rr) dst[(size_t)rr * sw.WF[0]] = __float2bfloat16_rn((bits >> rr & 1u) ? lut1 : lut0);
-                    }
-#pragma unroll
-                    for (int l = 1; l <= L; ++l)
-                        if (lane < sh.nin[l]) {
-                            __nv_bfloat16 *dst = sw.F[l] + ((size_t)slot * BM + r0) * sw.WF[l] + (sh.kin0[l] - kb_old[l] * BK) + lane;
-#pragma unroll
-                            for (int rr = 0; rr < RPW; ++rr) dst[(size_t)rr * sw.WF[l]] = __float2bfloat16_rn(S[l - 1][rr]);
-                        }
-                }
-            }
-            fence_proxy_async();              // F for the next group's loads, which also overwrite the running sums
+                for (int rr = 0; rr < RPW; ++rr) S[l][rr] = active ? lds_f(vat(l, lane, r0 + rr)) : 0.0f;
+            fence_proxy_async();              // the next group's loads overwrite the running sums' memory
             __syncwarp();
-            if (t1 < b && lane == 0) mbar_arrive(&sh.gdone);
+            if (t1 < b && lane == 0) mbar_arrive(&sh.vread);
+            const bool last = t0 + ng > hi;              // the block's last position completes nothing that the block reads
+            if (!active) {
+            } else if (m.act == JS_ACT_RELU) solve<L, RPW, JS_ACT_RELU>(S, nz, ng, last);
+            else solve<L, RPW, JS_ACT_GELU_TANH>(S, nz, ng, last);
+            const uint32_t bits = active ? symbols(S[L], nz) : 0u;
+            if (tid == 0) trace(5);
+            // ---- the group's activations into F, for the GEMMs of the groups that follow; symbols that changed
+            if (t1 < b) {
+                if (active && lane < ng) {
+                    __nv_bfloat16 *dst = sw.F[0] + ((size_t)slot * BM + r0) * sw.WF[0] + (t0 - kb_old[0] * BK) + lane;
+#pragma unroll
+                    for (int rr = 0; rr < RPW; ++rr) dst[(size_t)rr * sw.WF[0]] = __float2bfloat16_rn((bits >> rr & 1u) ? lut1 : lut0);
+                }
+#pragma unroll
+                for (int l = 1; l <= L; ++l)
+                    if (active && lane < sh.nin[l]) {
+                        __nv_bfloat16 *dst = sw.F[l] + ((size_t)slot * BM + r0) * sw.WF[l] + (sh.kin0[l] - kb_old[l] * BK) + lane;
+#pragma unroll
+                        for (int c = 0; c < RPW / 2; ++c) {
+                            const uint32_t v = m.act == JS_ACT_RELU ? act2<JS_ACT_RELU>(S[l - 1][2 * c], S[l - 1][2 * c + 1])
+                                                                    : act2<JS_ACT_GELU_TANH>(S[l - 1][2 * c], S[l - 1][2 * c + 1]);
+                            dst[(size_t)(2 * c) * sw.WF[l]] = __ushort_as_bfloat16((unsigned short)v);
+                            dst[(size_t)(2 * c + 1) * sw.WF[l]] = __ushort_as_bfloat16((unsigned short)(v >> 16));
+                        }
+                    }
+                fence_proxy_async();          // F for the next group's loads
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&sh.gdone);
+            }
+            if (active && lane < ng)
+#pragma unroll
+                for (int rr = 0; rr < RPW; ++rr) {
+                    const int s2 = rt * sw.rj + r0 + rr;
+                    if (s2 < r.batch && (((bits ^ xold) | xold >> 8) >> rr & 1u)) {
+                        r.x[(size_t)s2 * m.T + t0 + lane] = (uint8_t)(bits >> rr & 1u);
+                        changed |= 1u << rr;
+                    }
+                }
             if (tid == 0) trace(6);
             group_no++;
         }
     }
 };
 
-// LT = the model's number of hidden layers
-template <int LT>
+// LT = the model's number of hidden layers, RPW = sample rows per epilogue warp
+template <int LT, int RPW>
 __global__ void __launch_bounds__(NTH, 1)
 made_sweep_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ SweepDev sw, const __grid_constant__ RunArgs r)
 {
@@ -639,6 +767,7 @@ made_sweep_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ Swe
         for (int s = 0; s < MAX_STAGES; ++s) { mbar_init(&sh.full[s], 1); mbar_init(&sh.empty[s], 1); }
         mbar_init(&sh.tfull, 1);
         mbar_init(&sh.tempty, NEW);
+        mbar_init(&sh.vread, NEW);
         mbar_init(&sh.gdone, NEW);
         for (int i = 0; i < 2; ++i) { mbar_init(&sh.bfull[i], 1); mbar_init(&sh.bempty[i], NEW); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -673,7 +802,7 @@ made_sweep_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ Swe
             e.mma_issuer(a, b);
         } else {
             uint32_t changed = 0;
-            e.template epilogue<LT>(rt, blockIdx.x, a, b, changed);
+            e.template epilogue<LT, RPW>(rt, blockIdx.x, a, b, changed);
             changed = __reduce_or_sync(0xffffffffu, changed);
             if (e.lane < RPW && (changed >> e.lane & 1u)) r.smp_changed[rt * sw.rj + RPW * (warp - 2) + e.lane] = 1;
         }
@@ -750,16 +879,22 @@ static bool sweep_encode(CUtensorMap *out, const void *base, int rank, const cuu
 }
 
 typedef void (*SweepKernelFn)(const MadeDev, const SweepDev, const RunArgs);
-static SweepKernelFn sweep_kernel_of(int L)
+template <int L>
+static SweepKernelFn sweep_kernel_of(int rj_idx)
+{
+    // eight warps of four rows for 32 rows: a position costs a warp 40 instructions besides those of its rows
+    return rj_idx == 2 ? made_sweep_kernel<L, 8> : made_sweep_kernel<L, 4>;
+}
+static SweepKernelFn sweep_kernel_of(int L, int rj_idx)
 {
     switch (L) {
-    case 1: return made_sweep_kernel<1>;
-    case 2: return made_sweep_kernel<2>;
-    case 3: return made_sweep_kernel<3>;
-    case 4: return made_sweep_kernel<4>;
-    case 5: return made_sweep_kernel<5>;
-    case 6: return made_sweep_kernel<6>;
-    default: return made_sweep_kernel<7>;
+    case 1: return sweep_kernel_of<1>(rj_idx);
+    case 2: return sweep_kernel_of<2>(rj_idx);
+    case 3: return sweep_kernel_of<3>(rj_idx);
+    case 4: return sweep_kernel_of<4>(rj_idx);
+    case 5: return sweep_kernel_of<5>(rj_idx);
+    case 6: return sweep_kernel_of<6>(rj_idx);
+    default: return sweep_kernel_of<7>(rj_idx);
     }
 }
 
@@ -799,7 +934,7 @@ int js_sweep_prepare(js_model *mo)
     if (G < 1) return 0;
     s.G = G;
     const int v_bytes = (L + 1) * NUP * BM * 4;            // shares the ring's memory
-    const int fixed = (L + 1) * NUP * NUP * 4;
+    const int fixed = ((L + 1) * NUP + 1) * WS * 4;      // one row more: a pair of rows is read at the last one too
     s.n_stages = std::min(MAX_STAGES, (SMEM_DYN_MAX - 1024 - fixed) / STAGE_BYTES);
     if (s.n_stages < 2) return 0;
     s.ring_bytes = std::max(s.n_stages * STAGE_BYTES, (v_bytes + 1023) / 1024 * 1024);
@@ -882,10 +1017,11 @@ int js_sweep_prepare(js_model *mo)
         if (cudaHostAlloc((void **)&mo->h_any, sizeof(int), cudaHostAllocMapped) != cudaSuccess) return fail();
         if (cudaHostGetDevicePointer((void **)&mo->d_any, mo->h_any, 0) != cudaSuccess) return fail();
     }
-    if (cudaFuncSetAttribute(sweep_kernel_of(L), cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_DYN_MAX) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
-    }
+    for (int i = 1; i < 3; ++i)
+        if (cudaFuncSetAttribute(sweep_kernel_of(L, i), cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_DYN_MAX) != cudaSuccess) {
+            cudaGetLastError();
+            return 0;
+        }
     mo->sweep_state = 1;
     return 1;
 }
@@ -903,7 +1039,7 @@ int js_launch_made_sweep(const js_model *mo, const RunArgs &r, cudaStream_t stre
     const int njobs = (r.batch + s.rj - 1) / s.rj * nblk;
     if (njobs < 1) return (int)cudaErrorInvalidValue;
     const int grid = std::min(njobs, s.slots);
-    sweep_kernel_of(mo->made.L)<<<grid, NTH, s.smem_bytes, stream>>>(mo->made, s, r);
+    sweep_kernel_of(mo->made.L, s.rj_idx)<<<grid, NTH, s.smem_bytes, stream>>>(mo->made, s, r);
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? 0 : (int)e;
 }
