@@ -65,6 +65,21 @@ __device__ __forceinline__ void book_samples(const RunArgs &r, int parity, int k
     }
 }
 
+// After the barrier that ends an iteration: did anything change, and the first position that did.  One thread asks:
+// when all of them did, a grid's loads of the two words queued at one L2 slice for over a microsecond.
+__device__ __forceinline__ void read_changes(const JsCtl *ctl, int parity, int &any, int &minfirst)
+{
+    __shared__ int flags[2];
+    if (threadIdx.x == 0) {
+        flags[0] = ld_volatile_i32(&ctl->agg_any[parity]);
+        flags[1] = ld_volatile_i32(&ctl->agg_minfirst[parity]);
+    }
+    __syncthreads();
+    any = flags[0];
+    minfirst = flags[1];
+    __syncthreads();
+}
+
 struct DriverResult {
     int status, iterations, frontier;
     bool alive;
@@ -94,8 +109,8 @@ __device__ DriverResult made_driver(E &e, int T_, const RunArgs &r)
                     res.alive = false;
                     return res;
                 }
-                const int any = ld_volatile_i32(&ctl->agg_any[p]);
-                const int mf = ld_volatile_i32(&ctl->agg_minfirst[p]);
+                int any, mf;
+                read_changes(ctl, p, any, mf);
                 book_samples(r, p, k, k == cap, false, true);
                 reset_other_parity(r, p);
                 fin_h = max(fin_h, fin_x);
@@ -160,8 +175,8 @@ __device__ DriverResult made_driver(E &e, int T_, const RunArgs &r)
             continue;
         }
         const int cap = (r.max_iters > 0 && r.max_iters < len) ? r.max_iters : len;
-        const int any = ld_volatile_i32(&ctl->agg_any[p]);
-        const int mf = ld_volatile_i32(&ctl->agg_minfirst[p]);
+        int any, mf;
+        read_changes(ctl, p, any, mf);
         book_samples(r, p, k, k == cap, mode == KM_GS_JACOBI, mode == KM_JACOBI);
         reset_other_parity(r, p);
         fin_h = max(fin_h, min(fin_x, mode == KM_JACOBI ? T_ : bend - 1));
