@@ -12,6 +12,7 @@
 // re-encode), as in the masked-MLP kernel.  Solver loops: made_driver.cuh.
 #include <cuda.h>
 
+#include <cstring>
 #include <vector>
 
 #include "js_common.cuh"
@@ -28,7 +29,12 @@ constexpr int A_BYTES = BM * BK * 2;
 constexpr int RING_BYTES = 144 * 1024;                // cut anew for every layer: A tile + up to 256 weight rows per stage
 constexpr int MAX_STAGES = 6;                         // 64 weight rows: 24 KB; 128: 32 KB, 4 stages; 256: 48 KB, 3 stages
 constexpr int STAGING_BYTES = 32 * 1024;
-constexpr int SMEM_BYTES = RING_BYTES + STAGING_BYTES + 1024;
+constexpr int HEAD_STAGES = 2;                        // the head's ring (a tile is one or two K blocks) leaves room for the noise
+constexpr int NOISE_BUFS = 3;                         // per epilogue warp: boxes of 32 pixels x 32 classes
+constexpr int NOISE_BOX = 32 * 32 * 4;
+constexpr int NOISE_AT = HEAD_STAGES * (A_BYTES + 256 * BK * 2);      // behind the head's ring: over the rest of the layers' ring and the staging rows
+constexpr int SMEM_BYTES = NOISE_AT + 8 * NOISE_BUFS * NOISE_BOX + 1024;
+static_assert(NOISE_AT + 8 * NOISE_BUFS * NOISE_BOX >= RING_BYTES + STAGING_BYTES && NOISE_AT % 1024 == 0, "the larger of the two cuts");
 constexpr int MAX_IMAGES = 256;
 
 enum { EPI_HIDDEN = 0, EPI_LOGITS = 1, EPI_CAT = 3 };
@@ -38,7 +44,7 @@ enum { EPI_HIDDEN = 0, EPI_LOGITS = 1, EPI_CAT = 3 };
 enum { SRC_NEW = 0, SRC_OLD = 1, SRC_MIXED = 2 };
 
 struct ConvShared {
-    uint64_t full[MAX_STAGES], empty[MAX_STAGES], tfull[2], tempty[2];
+    uint64_t full[MAX_STAGES], empty[MAX_STAGES], tfull[2], tempty[2], nfull[8][NOISE_BUFS];
     uint32_t tmem_base;
     float bias_s[4][256];
     float xbest[2][4][32];    // head: the upper class half's best score and class, by tile parity and quadrant
@@ -53,6 +59,7 @@ struct ConvEngine {
     static constexpr bool has_jgs = true;
     const ConvDev &m;
     const RunArgs &r;
+    const CUtensorMap &tm_noise;
     ConvShared &sh;
     uint8_t *ring, *staging;
     unsigned epoch = 0;
@@ -66,8 +73,19 @@ struct ConvEngine {
     bool dead = false;
     uint32_t tmem_base = 0;
 
-    __device__ ConvEngine(const ConvDev &m_, const RunArgs &r_, ConvShared &sh_, uint8_t *ring_)
-        : m(m_), r(r_), sh(sh_), ring(ring_), staging(ring_ + RING_BYTES)
+    // Order of the layers of a pass.  A tile of a conv layer needs its own pixels and those of the tile above from the layer
+    // before it, so the layers of a pass are not separated by grid barriers: every tile carries a stamp, the number of the
+    // last layer that wrote it, and the loading warp waits for the two stamps (a layer of one tile per SM: 8.6 us with a
+    // barrier behind it, of which 3 us were the barrier and the way back to the first load).
+    int layer_no = 0;              // layers done by this launch, the current one included (the same in every CTA)
+    int conv_lo = 0, conv_hi = 0;  // row tiles that the conv layers of this pass recompute
+    // head: the noise boxes of this warp on their way.  Next box to ask for (tile, chunk of 32 classes), next buffer to fill and
+    // to read, parities of the buffers' next readings
+    int nz_id = 0, nz_chunk = 0, nz_fill = 0, nz_read = 0;
+    uint32_t nz_par = 0;
+
+    __device__ ConvEngine(const ConvDev &m_, const RunArgs &r_, const CUtensorMap &tm_noise_, ConvShared &sh_, uint8_t *ring_)
+        : m(m_), r(r_), tm_noise(tm_noise_), sh(sh_), ring(ring_), staging(ring_ + RING_BYTES)
     {
         warp = threadIdx.x >> 5;
         lane = threadIdx.x & 31;
@@ -110,6 +128,7 @@ struct ConvEngine {
                 r.smp_changed[i] = 0;
                 r.smp_state[i] = 0;
             }
+            for (int i = threadIdx.x; i < r.batch * m.nyt * 4; i += blockDim.x) m.stamp[i] = 0;
             if (threadIdx.x == 0) {
                 r.ctl->agg_any[0] = r.ctl->agg_any[1] = 0;
                 r.ctl->agg_minfirst[0] = r.ctl->agg_minfirst[1] = INT_MAX;
@@ -142,13 +161,46 @@ struct ConvEngine {
         return 0;
     }
 
-    // The ring is cut anew for every layer (it is drained at every phase boundary, and the parity of a stage's
-    // barriers is kept per stage).
-    __device__ void ring_for_width(int bn)
+    // The ring is cut anew for the head and behind it (the parity of a stage's barriers is kept per stage).
+    __device__ void ring_for(bool head)
     {
-        cur_stage_bytes = A_BYTES + bn * BK * 2;
-        cur_stages = min(MAX_STAGES, RING_BYTES / cur_stage_bytes);
+        const int bytes = A_BYTES + (head ? 256 : m.ch) * BK * 2;
+        if (bytes == cur_stage_bytes) return;
+        cur_stage_bytes = bytes;
+        cur_stages = head ? HEAD_STAGES : min(MAX_STAGES, RING_BYTES / bytes);
         stage = 0;
+    }
+    // the loading warp: every stage of the present cut has been read
+    __device__ bool ring_drained()
+    {
+        for (int s = 0; s < cur_stages; ++s)
+            if (!__all_sync(0xffffffffu, mbar_wait(&sh.empty[s], ((spar >> s) & 1u) ^ 1u, r.ctl))) return false;
+        return true;
+    }
+
+    // Whole warp: waits until tiles ya and yb of image n carry stamp `want` or a later one (an index outside the tiles
+    // that this pass recomputes: nothing to wait for).
+    __device__ bool wait_stamps(int n, int ya, int yb, int want)
+    {
+        const int y = lane == 0 ? ya : yb;
+        const bool look = lane < 2 && y >= conv_lo && y < conv_hi;
+        const int *st = m.stamp + 4 * (size_t)(n * m.nyt + (look ? y : 0));
+        uint64_t t0 = 0;
+        for (unsigned i = 1;; ++i) {
+            int a = want, b = want, c = want, d = want;
+            if (look) asm volatile("ld.volatile.global.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(a), "=r"(b), "=r"(c), "=r"(d) : "l"(st) : "memory");
+            if (__all_sync(0xffffffffu, min(min(a, b), min(c, d)) >= want)) break;
+            if ((i & 31u) == 0u) {
+                if (t0 == 0) t0 = global_ns();
+                if (__any_sync(0xffffffffu, ld_volatile_i32(&r.ctl->abort) != 0 || global_ns() - t0 > MBAR_WAIT_NS)) {
+                    if (lane == 0) atomicExch(&r.ctl->abort, 1);
+                    return false;
+                }
+            }
+        }
+        __threadfence();
+        fence_proxy_async();
+        return true;
     }
     __device__ uint8_t *stage_a(int s) const { return ring + (size_t)s * cur_stage_bytes; }
     __device__ uint8_t *stage_b(int s) const { return ring + (size_t)s * cur_stage_bytes + A_BYTES; }
@@ -199,33 +251,54 @@ struct ConvEngine {
         const bool head = (l == m.n_conv);
         const int per = head ? m.in_ch : 1;
         const int bn = head ? 256 : m.ch;
-        const CUtensorMap *ma_new = m.tmAct + l, *ma_old = m.tmActOld + l, *mw = m.tmW + l;
+        const CUtensorMap *mw = m.tmW + l;
         const uint32_t bytes = A_BYTES + bn * BK * 2;
         const int kcs = head ? m.ch / BK : m.cin_pad[l] / BK, kcs_log2 = kcs == 2 ? 1 : 0;       // 64 or 128 channels
         const int nkb = kblocks(l);
-        ring_for_width(bn);
+        // the head's cut lies over the layers' ring (at the start of a pass the grid barrier has drained it)
+        if (head && cur_stage_bytes != 0 && !ring_drained()) { dead = true; return; }
+        ring_for(head);
         if (lane == 0) trace(0);
         for (int id = blockIdx.x; id < ntiles && !dead; id += gridDim.x) {
             int n, yt, c;
             locate(id, nyl, yt_lo, per, n, yt, c);
             const int y0 = yt * m.R;
+            // The weights of the tile's first K blocks do not wait for the layer before.  The head writes the image, which the
+            // tile below reads in the first layer: it waits for that tile too.
+            const int ahead = min(cur_stages, nkb), s0 = stage;
             for (int kb = 0; kb < nkb;) {
-                const int run = mbar_wait_run(sh.empty, stage, cur_stages, ~spar, nkb - kb, r.ctl);
+                const int run = mbar_wait_run(sh.empty, stage, cur_stages, ~spar, (kb < ahead ? ahead : nkb) - kb, r.ctl);
                 if (run == 0) { dead = true; break; }
                 for (int i = 0; i < run; ++i, ++kb) {
-                    const int tap = kb >> kcs_log2, kc = kb & (kcs - 1);
-                    // taps in the order of the packed weights: the three of the row above, then left and centre
-                    const int dy = head || tap >= 3 ? 0 : -1, dx = head ? 0 : tap >= 3 ? tap - 4 : tap - 1;
-                    const CUtensorMap *ma = (src == SRC_OLD || (src == SRC_MIXED && dy < 0)) ? ma_old : ma_new;
                     if (elect_one()) {
                         mbar_expect_tx(&sh.full[stage], bytes);
-                        tma_load_4d(smem_u32(stage_a(stage)), ma, &sh.full[stage], kc * BK, dx, y0 + dy, n);
-                        tma_load_2d(smem_u32(stage_b(stage)), mw, &sh.full[stage], kc * BK, head ? c * 256 : tap * m.ch);
+                        tma_load_2d(smem_u32(stage_b(stage)), mw, &sh.full[stage], (kb & (kcs - 1)) * BK, head ? c * 256 : (kb >> kcs_log2) * m.ch);
+                        if (kb >= ahead) load_a(l, stage, kb, kcs, kcs_log2, src, y0, n);
                     }
                     advance_stage();
                 }
+                if (kb == ahead) {
+                    if (l > 0 && !wait_stamps(n, yt, head ? yt + 1 : yt - 1, layer_no - 1)) { dead = true; break; }
+                    if (elect_one()) {
+                        int st = s0;
+                        for (int k2 = 0; k2 < ahead; ++k2) {
+                            load_a(l, st, k2, kcs, kcs_log2, src, y0, n);
+                            if (++st == cur_stages) st = 0;
+                        }
+                    }
+                    __syncwarp();
+                }
             }
         }
+    }
+    // the pixels of K block kb: taps in the order of the packed weights, the three of the row above, then left and centre
+    __device__ void load_a(int l, int st, int kb, int kcs, int kcs_log2, int src, int y0, int n)
+    {
+        const bool head = (l == m.n_conv);
+        const int tap = kb >> kcs_log2, kc = kb & (kcs - 1);
+        const int dy = head || tap >= 3 ? 0 : -1, dx = head ? 0 : tap >= 3 ? tap - 4 : tap - 1;
+        const CUtensorMap *ma = ((src == SRC_OLD || (src == SRC_MIXED && dy < 0)) ? m.tmActOld : m.tmAct) + l;
+        tma_load_4d(smem_u32(stage_a(st)), ma, &sh.full[st], kc * BK, dx, y0 + dy, n);
     }
 
     __device__ void mma_issuer(int l, int ntiles)
@@ -233,7 +306,7 @@ struct ConvEngine {
         const bool head = (l == m.n_conv);
         const uint32_t idesc = instr_desc_bf16(head ? 256 : m.ch);
         const int nkb = kblocks(l);
-        ring_for_width(head ? 256 : m.ch);
+        ring_for(head);
         bool first = true;
         for (int id = blockIdx.x; id < ntiles && !dead; id += gridDim.x) {
             if (!__all_sync(0xffffffffu, mbar_wait(&sh.tempty[acc], aphase ^ 1u, r.ctl))) { dead = true; break; }
@@ -307,7 +380,38 @@ struct ConvEngine {
             const int prow = q * 32 + rl;
             if (prow < rows_valid && col < bn) *reinterpret_cast<uint4 *>(out + (pix0 + prow) * bn + col) = val;
         }
+        fence_proxy_async();      // read by the next layer's TMA loads
         __syncwarp();
+        if (lane == 0) {
+            __threadfence();
+            *reinterpret_cast<volatile int *>(m.stamp + 4 * (size_t)(n * m.nyt + y0 / m.R) + q) = layer_no;
+        }
+    }
+
+    // ---- head: the noise of a warp's 32 pixels and 128 classes goes through shared memory in boxes of 32 classes, so many ahead
+    // as there are buffers.  (Read by the threads, a lane per pixel, every 16-byte load of a warp touched 32 lines: 7 us per
+    // tile of 128 pixels, a quarter of a whole pass.)
+    __device__ uint8_t *noise_buf(int b) const { return ring + NOISE_AT + (size_t)((warp - 2) * NOISE_BUFS + b) * NOISE_BOX; }
+    __device__ void noise_ask(int yt_lo, int nyl, int ntiles)
+    {
+        const int q = warp & 3, half = (warp - 2) >> 2;
+        while (nz_id < ntiles) {
+            int n, yt, c;
+            locate(nz_id, nyl, yt_lo, m.in_ch, n, yt, c);
+            const int y0 = yt * m.R;
+            if (q * 32 < (min(m.height, y0 + m.R) - y0) * m.width) {      // else the quadrant lies below the image
+                if (elect_one()) {
+                    uint64_t *bar = &sh.nfull[warp - 2][nz_fill];
+                    mbar_expect_tx(bar, NOISE_BOX);
+                    tma_load_3d(smem_u32(noise_buf(nz_fill)), &tm_noise, bar, half * 128 + nz_chunk * 32, c, (n * m.height + y0) * m.width + q * 32);
+                }
+                __syncwarp();
+                if (++nz_fill == NOISE_BUFS) nz_fill = 0;
+                if (++nz_chunk == 4) { nz_chunk = 0; nz_id += gridDim.x; }
+                return;
+            }
+            nz_id += gridDim.x;
+        }
     }
 
     // Inverse CDF of the softmax from one uniform number u: the first class c with u * S < sum_{i<=c} e_i,
@@ -369,15 +473,25 @@ struct ConvEngine {
         // issue, one warp per scheduler was not enough; elsewhere it only hands the accumulator back.
         const int half = (warp - 2) >> 2;
         int tile_par = 0;
+        const bool split_head = head && kind == EPI_CAT && r.nk == JS_NOISE_GUMBEL;
         bool any_changed = false;
         int first = INT_MAX;
-        for (int id = blockIdx.x; id < ntiles && !dead; id += gridDim.x) {
+        if (split_head) {
+            // Every warp is through with its staging rows.  The layers' ring is drained: all of them have seen this CTA's
+            // last accumulator.
+            asm volatile("bar.sync 5, 256;" ::: "memory");
+            fence_proxy_async();
+            nz_id = blockIdx.x;
+            nz_chunk = 0;
+            for (int i = 0; i < NOISE_BUFS; ++i) noise_ask(yt_lo, nyl, ntiles);
+        }
+        int id = blockIdx.x;
+        for (; id < ntiles && !dead; id += gridDim.x) {
             int n, yt, c;
             locate(id, nyl, yt_lo, per, n, yt, c);
             const int y0 = yt * m.R;
-            const bool split_head = head && kind == EPI_CAT && r.nk == JS_NOISE_GUMBEL;
             if (half == 1 && !(head && (split_head || kind == EPI_LOGITS))) {
-                if (!mbar_wait(&sh.tfull[acc], aphase, r.ctl)) { dead = true; break; }
+                if (!__all_sync(0xffffffffu, mbar_wait(&sh.tfull[acc], aphase, r.ctl))) { dead = true; break; }
                 tc_fence_after();
                 release_acc();
                 advance_acc();
@@ -389,7 +503,7 @@ struct ConvEngine {
                 for (int i = lane; i < m.ch; i += 32) bs[i] = m.bias[l][i];
                 __syncwarp();
             }
-            if (!mbar_wait(&sh.tfull[acc], aphase, r.ctl)) { dead = true; break; }
+            if (!__all_sync(0xffffffffu, mbar_wait(&sh.tfull[acc], aphase, r.ctl))) { dead = true; break; }
             tc_fence_after();
             if (warp == 4 && lane == 0) trace(3);
             const uint32_t tbase = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * ACC_COLS);
@@ -417,22 +531,31 @@ struct ConvEngine {
                     float v[32];
                     __syncwarp();
                     tmem_ld32(tbase + (uint32_t)c0, v);
-                    if (!valid) continue;
                     if (kind == EPI_LOGITS) {
+                        if (!valid) continue;
 #pragma unroll
                         for (int i = 0; i < 32; ++i) zout[at * 256 + c0 + i] = v[i] + bias[c0 + i];
-                    } else {
-                        const float *gg = r.noise + at * 256 + c0;
+                    } else if (q * 32 < rows_valid) {
+                        if (!__all_sync(0xffffffffu, mbar_wait(&sh.nfull[warp - 2][nz_read], (nz_par >> nz_read) & 1u, r.ctl))) { dead = true; break; }
+                        nz_par ^= 1u << nz_read;
+                        // lane = pixel: rows of 128 bytes, their 16-byte chunks permuted by the row number (the box's swizzle)
+                        const uint32_t gg = smem_u32(noise_buf(nz_read)) + 128u * (uint32_t)lane;
                         float sc[32];
 #pragma unroll
                         for (int i = 0; i < 32; i += 4) {
                             const float4 b4 = __ldg(reinterpret_cast<const float4 *>(bias + c0 + i));
-                            const float4 g4 = __ldg(reinterpret_cast<const float4 *>(gg + i));
+                            float4 g4;
+                            asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                                         : "=f"(g4.x), "=f"(g4.y), "=f"(g4.z), "=f"(g4.w)
+                                         : "r"(gg + 16u * (uint32_t)((i >> 2) ^ (lane & 7))));
                             sc[i] = (v[i] + b4.x) + g4.x;
                             sc[i + 1] = (v[i + 1] + b4.y) + g4.y;
                             sc[i + 2] = (v[i + 2] + b4.z) + g4.z;
                             sc[i + 3] = (v[i + 3] + b4.w) + g4.w;
                         }
+                        __syncwarp();
+                        if (++nz_read == NOISE_BUFS) nz_read = 0;
+                        noise_ask(yt_lo, nyl, ntiles);
                         argmax_chunk32(sc, c0, best, bi);
                     }
                 }
@@ -475,6 +598,9 @@ struct ConvEngine {
             }
             advance_acc();
         }
+        // a warp that gave up lets its partner through the meetings it will not come to
+        if (split_head && dead)
+            for (; id < ntiles; id += gridDim.x) asm volatile("bar.arrive %0, 64;" ::"r"(1 + q) : "memory");
         if (warp == 4 && lane == 0) trace(4);
         if (flag) {
             const bool wany = __any_sync(0xffffffffu, any_changed);
@@ -488,7 +614,7 @@ struct ConvEngine {
         }
     }
 
-    __device__ bool layer_phase(int l, int kind, const Win &w, bool flag, int parity, float *zout, int src = SRC_NEW)
+    __device__ void layer_phase(int l, int kind, const Win &w, bool flag, int parity, float *zout, int src = SRC_NEW)
     {
         const bool head = (l == m.n_conv);
         int yt_lo, yt_hi;
@@ -505,8 +631,10 @@ struct ConvEngine {
                 weight_bytes += 2ull * BK * (unsigned long long)kblocks(l) * (unsigned long long)(head ? 256 * m.in_ch : m.ch);
             if (blockIdx.x == 0) skipped += (unsigned long long)(r.batch * m.nyt - sh.n_img * nyl) * (head ? m.in_ch : 1);
         }
-        if (ntiles == 0) return false;
+        if (ntiles == 0) return;
         phase_no++;
+        layer_no++;
+        if (!head) conv_lo = yt_lo, conv_hi = yt_hi;
         if (warp == 0) {
             producer(l, yt_lo, nyl, ntiles, src);
         } else if (warp == 1) {
@@ -514,19 +642,19 @@ struct ConvEngine {
         } else {
             epilogue(l, kind, w, flag, parity, zout, yt_lo, nyl, ntiles, src);
         }
-        return true;
     }
 
+    // One pass.  Inside it the tiles wait for one another by their stamps; the grid barrier at its end lets the next pass
+    // overwrite what this one read, and makes the flags complete.
     __device__ bool step(const Win &w, bool flag, int parity, float *zout, int src = SRC_NEW)
     {
+        conv_lo = conv_hi = 0;
         const int l_end = src == SRC_OLD ? m.n_conv - 1 : m.n_conv;      // the old set needs no head
         for (int l = 0; l <= l_end; ++l) {
             const bool last = (l == m.n_conv);
-            const bool did = layer_phase(l, last ? (zout ? EPI_LOGITS : EPI_CAT) : EPI_HIDDEN, w, last && flag, parity, zout, src);
-            if (did || l == l_end)
-                if (!barrier()) return false;
+            layer_phase(l, last ? (zout ? EPI_LOGITS : EPI_CAT) : EPI_HIDDEN, w, last && flag, parity, zout, src);
         }
-        return true;
+        return barrier();
     }
 
     // One outer iteration of Algorithm 2 with one-image-row blocks.  A block's sequential sweep yields the
@@ -588,7 +716,7 @@ struct ConvEngine {
 };
 
 __global__ void __launch_bounds__(NTH, 1)
-conv_tc_kernel(const __grid_constant__ ConvDev m, const __grid_constant__ RunArgs r)
+conv_tc_kernel(const __grid_constant__ ConvDev m, const __grid_constant__ RunArgs r, const __grid_constant__ CUtensorMap tm_noise)
 {
     extern __shared__ uint8_t smem_raw[];
     __shared__ ConvShared sh;
@@ -597,6 +725,8 @@ conv_tc_kernel(const __grid_constant__ ConvDev m, const __grid_constant__ RunArg
     if (threadIdx.x == 0) {
         for (int s = 0; s < MAX_STAGES; ++s) { mbar_init(&sh.full[s], 1); mbar_init(&sh.empty[s], 1); }
         for (int a = 0; a < 2; ++a) { mbar_init(&sh.tfull[a], 1); mbar_init(&sh.tempty[a], 8); }
+        for (int w = 0; w < 8; ++w)
+            for (int i = 0; i < NOISE_BUFS; ++i) mbar_init(&sh.nfull[w][i], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async();
     }
@@ -606,7 +736,7 @@ conv_tc_kernel(const __grid_constant__ ConvDev m, const __grid_constant__ RunArg
     __syncthreads();
     tc_fence_after();
 
-    ConvEngine e(m, r, sh, ring);
+    ConvEngine e(m, r, tm_noise, sh, ring);
     e.tmem_base = sh.tmem_base;
     DriverResult res = made_driver(e, m.T, r);
     if (e.dead) res.alive = false;
@@ -646,12 +776,12 @@ static EncodeTiledFn conv_encode_fn()
 }
 
 static bool encode_nd(CUtensorMap *out, const void *base, int rank, const cuuint64_t *dims, const cuuint64_t *strides,
-                      const cuuint32_t *box)
+                      const cuuint32_t *box, CUtensorMapDataType type = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16)
 {
     EncodeTiledFn fn = conv_encode_fn();
     if (!fn) return false;
     const cuuint32_t estr[4] = {1, 1, 1, 1};
-    return fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, const_cast<void *>(base), dims, strides, box, estr,
+    return fn(out, type, rank, const_cast<void *>(base), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -754,6 +884,7 @@ int js_conv_build(js_model *mo, const js_conv_desc *d)
         if (!upload<float>(mo, lut.data(), lut.size(), &ld)) return JS_ERR_CUDA;
         v.lut = ld;
     }
+    if (!upload<int>(mo, nullptr, (size_t)nb * v.nyt * 4, &v.stamp)) return JS_ERR_CUDA;
     CUtensorMap *pa = nullptr, *pw = nullptr, *pao = nullptr;
     if (!upload<CUtensorMap>(mo, mapsAold.data(), mapsAold.size(), &pao)) return JS_ERR_CUDA;
     v.tmActOld = pao;
@@ -779,7 +910,16 @@ int js_launch_conv_tc(const js_model *mo, const RunArgs &r, cudaStream_t stream)
     const ConvDev &v = mo->conv;
     const int tiles = r.batch * v.nyt * v.in_ch;
     const int grid = std::max(1, std::min(mo->conv_max_grid, tiles));
-    void *args[2] = {(void *)&v, (void *)&r};
+    CUtensorMap noise;
+    std::memset(&noise, 0, sizeof noise);
+    if (r.nk == JS_NOISE_GUMBEL && r.noise) {
+        // {class, sub-pixel, pixel}, a box per 32 pixels and 32 classes of one sub-pixel
+        const cuuint64_t dims[3] = {256, (cuuint64_t)v.in_ch, (cuuint64_t)r.batch * v.height * v.width};
+        const cuuint64_t strides[2] = {1024, (cuuint64_t)v.in_ch * 1024};
+        const cuuint32_t box[3] = {32, 1, 32};
+        if (!encode_nd(&noise, r.noise, 3, dims, strides, box, CU_TENSOR_MAP_DATA_TYPE_FLOAT32)) return (int)cudaErrorInvalidValue;
+    }
+    void *args[3] = {(void *)&v, (void *)&r, (void *)&noise};
     cudaError_t e = cudaLaunchCooperativeKernel((const void *)conv_tc_kernel, dim3(grid), dim3(NTH), args, SMEM_BYTES,
                                                 stream);
     return e == cudaSuccess ? 0 : (int)e;
