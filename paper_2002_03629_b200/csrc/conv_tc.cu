@@ -23,18 +23,22 @@
 namespace {
 
 constexpr int BM = TC_BM, BK = TC_BK;
-constexpr int NTH = 320;          // warp 0 loads, warp 1 MMA, warps 2-9 epilogue: two per tensor-memory lane quadrant
+constexpr int NTH = 352;          // warp 0 loads pixels, warp 1 MMA, warps 2-9 epilogue: two per tensor-memory lane quadrant, warp 10 loads weights
 constexpr int ACC_COLS = 256;
 constexpr int A_BYTES = BM * BK * 2;
-constexpr int RING_BYTES = 144 * 1024;                // cut anew for every layer: A tile + up to 256 weight rows per stage
-constexpr int MAX_STAGES = 6;                         // 64 weight rows: 24 KB; 128: 32 KB, 4 stages; 256: 48 KB, 3 stages
-constexpr int STAGING_BYTES = 32 * 1024;
-constexpr int HEAD_STAGES = 2;                        // the head's ring (a tile is one or two K blocks) leaves room for the noise
+// Two rings, each with a loading warp of its own: weights, which wait for nothing but room and so are there before the layer
+// in front has finished, and pixels.  A load takes about 1 us, the MMAs of a K block 0.14: with one ring of 4 stages for both,
+// filled when the pixels were there, the ten K blocks of a tile took 2.9 us.
+constexpr int W_RING = 80 * 1024;                     // 64 weight rows: 8 KB, 10 stages; 128: 5 stages; the head's 256: 2 stages
+constexpr int A_STAGES = 6;
+constexpr int MAX_STAGES = 10;
+constexpr int STAGING_BYTES = 32 * 1024;              // 4 KB per epilogue warp
+constexpr int HEAD_STAGES = 2;                        // a tile of the head is one or two K blocks: pixel stages that leave room for the noise
 constexpr int NOISE_BUFS = 3;                         // per epilogue warp: boxes of 32 pixels x 32 classes
 constexpr int NOISE_BOX = 32 * 32 * 4;
-constexpr int NOISE_AT = HEAD_STAGES * (A_BYTES + 256 * BK * 2);      // behind the head's ring: over the rest of the layers' ring and the staging rows
-constexpr int SMEM_BYTES = NOISE_AT + 8 * NOISE_BUFS * NOISE_BOX + 1024;
-static_assert(NOISE_AT + 8 * NOISE_BUFS * NOISE_BOX >= RING_BYTES + STAGING_BYTES && NOISE_AT % 1024 == 0, "the larger of the two cuts");
+constexpr int NOISE_AT = W_RING + HEAD_STAGES * A_BYTES;      // over the rest of the layers' pixel ring and the staging rows
+constexpr int SMEM_BYTES = W_RING + A_STAGES * A_BYTES + STAGING_BYTES + 1024;
+static_assert(NOISE_AT + 8 * NOISE_BUFS * NOISE_BOX <= SMEM_BYTES - 1024 && NOISE_AT % 1024 == 0, "room for the noise");
 constexpr int MAX_IMAGES = 256;
 
 enum { EPI_HIDDEN = 0, EPI_LOGITS = 1, EPI_CAT = 3 };
@@ -44,9 +48,9 @@ enum { EPI_HIDDEN = 0, EPI_LOGITS = 1, EPI_CAT = 3 };
 enum { SRC_NEW = 0, SRC_OLD = 1, SRC_MIXED = 2 };
 
 struct ConvShared {
-    uint64_t full[MAX_STAGES], empty[MAX_STAGES], tfull[2], tempty[2], nfull[8][NOISE_BUFS];
+    uint64_t wfull[MAX_STAGES], wempty[MAX_STAGES], afull[A_STAGES], aempty[A_STAGES], tfull[2], tempty[2], nfull[8][NOISE_BUFS];
     uint32_t tmem_base;
-    float bias_s[4][256];
+    float bias_s[8][64];      // of the channels of an epilogue warp
     float xbest[2][4][32];    // head: the upper class half's best score and class, by tile parity and quadrant
     int xbi[2][4][32];
     float lut_s[256];         // input encoding table
@@ -65,9 +69,10 @@ struct ConvEngine {
     unsigned epoch = 0;
     unsigned long long issued = 0, skipped = 0, mma_flops = 0, weight_bytes = 0;
     int warp, lane;
-    int stage = 0;
-    uint32_t spar = 0;             // bit s: parity of the next use of ring stage s
-    int cur_stages = 1, cur_stage_bytes = 0;      // ring geometry of the current layer
+    // the rings: stage in turn, bit s = parity of the next use of stage s, present cut
+    int wst = 0, ast = 0;
+    uint32_t wpar = 0, apar = 0;
+    int w_stages = 1, w_bytes = 0, a_stages = A_STAGES;
     int acc = 0;
     uint32_t aphase = 0;
     bool dead = false;
@@ -85,7 +90,7 @@ struct ConvEngine {
     uint32_t nz_par = 0;
 
     __device__ ConvEngine(const ConvDev &m_, const RunArgs &r_, const CUtensorMap &tm_noise_, ConvShared &sh_, uint8_t *ring_)
-        : m(m_), r(r_), tm_noise(tm_noise_), sh(sh_), ring(ring_), staging(ring_ + RING_BYTES)
+        : m(m_), r(r_), tm_noise(tm_noise_), sh(sh_), ring(ring_), staging(ring_ + W_RING + A_STAGES * A_BYTES)
     {
         warp = threadIdx.x >> 5;
         lane = threadIdx.x & 31;
@@ -128,7 +133,7 @@ struct ConvEngine {
                 r.smp_changed[i] = 0;
                 r.smp_state[i] = 0;
             }
-            for (int i = threadIdx.x; i < r.batch * m.nyt * 4; i += blockDim.x) m.stamp[i] = 0;
+            for (int i = threadIdx.x; i < r.batch * m.nyt * 8; i += blockDim.x) m.stamp[i] = 0;
             if (threadIdx.x == 0) {
                 r.ctl->agg_any[0] = r.ctl->agg_any[1] = 0;
                 r.ctl->agg_minfirst[0] = r.ctl->agg_minfirst[1] = INT_MAX;
@@ -161,35 +166,51 @@ struct ConvEngine {
         return 0;
     }
 
-    // The ring is cut anew for the head and behind it (the parity of a stage's barriers is kept per stage).
-    __device__ void ring_for(bool head)
+    // The rings are cut anew for the head and behind it (the parity of a stage's barriers is kept per stage).  At the start of a
+    // pass the grid barrier has drained them; a loading warp that goes over to the head waits until its ring is.
+    __device__ void cut_rings(bool head)
     {
-        const int bytes = A_BYTES + (head ? 256 : m.ch) * BK * 2;
-        if (bytes == cur_stage_bytes) return;
-        cur_stage_bytes = bytes;
-        cur_stages = head ? HEAD_STAGES : min(MAX_STAGES, RING_BYTES / bytes);
-        stage = 0;
+        const int bytes = (head ? 256 : m.ch) * BK * 2;
+        if (bytes != w_bytes) {
+            w_bytes = bytes;
+            w_stages = min(MAX_STAGES, W_RING / bytes);
+            wst = 0;
+        }
+        const int as = head ? HEAD_STAGES : A_STAGES;
+        if (as != a_stages) {
+            a_stages = as;
+            ast = 0;
+        }
     }
-    // the loading warp: every stage of the present cut has been read
-    __device__ bool ring_drained()
+    __device__ bool drained(uint64_t *empty, int n, uint32_t par)
     {
-        for (int s = 0; s < cur_stages; ++s)
-            if (!__all_sync(0xffffffffu, mbar_wait(&sh.empty[s], ((spar >> s) & 1u) ^ 1u, r.ctl))) return false;
+        for (int s = 0; s < n; ++s)
+            if (!__all_sync(0xffffffffu, mbar_wait(&empty[s], ((par >> s) & 1u) ^ 1u, r.ctl))) return false;
         return true;
+    }
+    __device__ uint8_t *stage_w(int s) const { return ring + (size_t)s * w_bytes; }
+    __device__ uint8_t *stage_a(int s) const { return ring + W_RING + (size_t)s * A_BYTES; }
+    __device__ void advance_w()
+    {
+        wpar ^= 1u << wst;
+        if (++wst == w_stages) wst = 0;
+    }
+    __device__ void advance_a()
+    {
+        apar ^= 1u << ast;
+        if (++ast == a_stages) ast = 0;
     }
 
     // Whole warp: waits until tiles ya and yb of image n carry stamp `want` or a later one (an index outside the tiles
-    // that this pass recomputes: nothing to wait for).
+    // that this pass recomputes: nothing to wait for).  Eight stamps per tile, one per warp that writes it.
     __device__ bool wait_stamps(int n, int ya, int yb, int want)
     {
-        const int y = lane == 0 ? ya : yb;
-        const bool look = lane < 2 && y >= conv_lo && y < conv_hi;
-        const int *st = m.stamp + 4 * (size_t)(n * m.nyt + (look ? y : 0));
+        const int y = lane < 8 ? ya : yb;
+        const bool look = lane < 16 && y >= conv_lo && y < conv_hi;
+        const int *st = m.stamp + 8 * (size_t)(n * m.nyt + (look ? y : 0)) + (lane & 7);
         uint64_t t0 = 0;
         for (unsigned i = 1;; ++i) {
-            int a = want, b = want, c = want, d = want;
-            if (look) asm volatile("ld.volatile.global.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(a), "=r"(b), "=r"(c), "=r"(d) : "l"(st) : "memory");
-            if (__all_sync(0xffffffffu, min(min(a, b), min(c, d)) >= want)) break;
+            if (__all_sync(0xffffffffu, !look || ld_volatile_i32(st) >= want)) break;
             if ((i & 31u) == 0u) {
                 if (t0 == 0) t0 = global_ns();
                 if (__any_sync(0xffffffffu, ld_volatile_i32(&r.ctl->abort) != 0 || global_ns() - t0 > MBAR_WAIT_NS)) {
@@ -201,13 +222,6 @@ struct ConvEngine {
         __threadfence();
         fence_proxy_async();
         return true;
-    }
-    __device__ uint8_t *stage_a(int s) const { return ring + (size_t)s * cur_stage_bytes; }
-    __device__ uint8_t *stage_b(int s) const { return ring + (size_t)s * cur_stage_bytes + A_BYTES; }
-    __device__ void advance_stage()
-    {
-        spar ^= 1u << stage;
-        if (++stage == cur_stages) stage = 0;
     }
     __device__ void advance_acc()
     {
@@ -246,59 +260,61 @@ struct ConvEngine {
         return l < m.n_conv ? 5 * (m.cin_pad[l] / BK) : m.ch / BK;
     }
 
-    __device__ void producer(int l, int yt_lo, int nyl, int ntiles, int src)
+    __device__ void load_weights(int l, int ntiles)
     {
         const bool head = (l == m.n_conv);
-        const int per = head ? m.in_ch : 1;
-        const int bn = head ? 256 : m.ch;
-        const CUtensorMap *mw = m.tmW + l;
-        const uint32_t bytes = A_BYTES + bn * BK * 2;
-        const int kcs = head ? m.ch / BK : m.cin_pad[l] / BK, kcs_log2 = kcs == 2 ? 1 : 0;       // 64 or 128 channels
+        const int per = head ? m.in_ch : 1, kcs = head ? m.ch / BK : m.cin_pad[l] / BK, kcs_log2 = kcs == 2 ? 1 : 0;
         const int nkb = kblocks(l);
-        // the head's cut lies over the layers' ring (at the start of a pass the grid barrier has drained it)
-        if (head && cur_stage_bytes != 0 && !ring_drained()) { dead = true; return; }
-        ring_for(head);
-        if (lane == 0) trace(0);
-        for (int id = blockIdx.x; id < ntiles && !dead; id += gridDim.x) {
-            int n, yt, c;
-            locate(id, nyl, yt_lo, per, n, yt, c);
-            const int y0 = yt * m.R;
-            // The weights of the tile's first K blocks do not wait for the layer before.  The head writes the image, which the
-            // tile below reads in the first layer: it waits for that tile too.
-            const int ahead = min(cur_stages, nkb), s0 = stage;
+        const CUtensorMap *mw = m.tmW + l;
+        if (head && w_bytes != 0 && !drained(sh.wempty, w_stages, wpar)) { dead = true; return; }
+        cut_rings(head);
+        for (int id = blockIdx.x; id < ntiles; id += gridDim.x) {
+            const int c = id % per;
             for (int kb = 0; kb < nkb;) {
-                const int run = mbar_wait_run(sh.empty, stage, cur_stages, ~spar, (kb < ahead ? ahead : nkb) - kb, r.ctl);
-                if (run == 0) { dead = true; break; }
+                const int run = mbar_wait_run(sh.wempty, wst, w_stages, ~wpar, nkb - kb, r.ctl);
+                if (run == 0) { dead = true; return; }
                 for (int i = 0; i < run; ++i, ++kb) {
                     if (elect_one()) {
-                        mbar_expect_tx(&sh.full[stage], bytes);
-                        tma_load_2d(smem_u32(stage_b(stage)), mw, &sh.full[stage], (kb & (kcs - 1)) * BK, head ? c * 256 : (kb >> kcs_log2) * m.ch);
-                        if (kb >= ahead) load_a(l, stage, kb, kcs, kcs_log2, src, y0, n);
+                        mbar_expect_tx(&sh.wfull[wst], (uint32_t)w_bytes);
+                        tma_load_2d(smem_u32(stage_w(wst)), mw, &sh.wfull[wst], (kb & (kcs - 1)) * BK, head ? c * 256 : (kb >> kcs_log2) * m.ch);
                     }
-                    advance_stage();
-                }
-                if (kb == ahead) {
-                    if (l > 0 && !wait_stamps(n, yt, head ? yt + 1 : yt - 1, layer_no - 1)) { dead = true; break; }
-                    if (elect_one()) {
-                        int st = s0;
-                        for (int k2 = 0; k2 < ahead; ++k2) {
-                            load_a(l, st, k2, kcs, kcs_log2, src, y0, n);
-                            if (++st == cur_stages) st = 0;
-                        }
-                    }
-                    __syncwarp();
+                    advance_w();
                 }
             }
         }
     }
-    // the pixels of K block kb: taps in the order of the packed weights, the three of the row above, then left and centre
-    __device__ void load_a(int l, int st, int kb, int kcs, int kcs_log2, int src, int y0, int n)
+
+    __device__ void load_pixels(int l, int yt_lo, int nyl, int ntiles, int src)
     {
         const bool head = (l == m.n_conv);
-        const int tap = kb >> kcs_log2, kc = kb & (kcs - 1);
-        const int dy = head || tap >= 3 ? 0 : -1, dx = head ? 0 : tap >= 3 ? tap - 4 : tap - 1;
-        const CUtensorMap *ma = ((src == SRC_OLD || (src == SRC_MIXED && dy < 0)) ? m.tmActOld : m.tmAct) + l;
-        tma_load_4d(smem_u32(stage_a(st)), ma, &sh.full[st], kc * BK, dx, y0 + dy, n);
+        const int per = head ? m.in_ch : 1, kcs = head ? m.ch / BK : m.cin_pad[l] / BK, kcs_log2 = kcs == 2 ? 1 : 0;       // 64 or 128 channels
+        const int nkb = kblocks(l);
+        const CUtensorMap *ma_new = m.tmAct + l, *ma_old = m.tmActOld + l;
+        if (head && w_bytes != 0 && !drained(sh.aempty, a_stages, apar)) { dead = true; return; }
+        cut_rings(head);
+        if (lane == 0) trace(0);
+        for (int id = blockIdx.x; id < ntiles; id += gridDim.x) {
+            int n, yt, c;
+            locate(id, nyl, yt_lo, per, n, yt, c);
+            const int y0 = yt * m.R;
+            // The head writes the image, which the tile below reads in the first layer: it waits for that tile too.
+            if (l > 0 && !wait_stamps(n, yt, head ? yt + 1 : yt - 1, layer_no - 1)) { dead = true; return; }
+            for (int kb = 0; kb < nkb;) {
+                const int run = mbar_wait_run(sh.aempty, ast, a_stages, ~apar, nkb - kb, r.ctl);
+                if (run == 0) { dead = true; return; }
+                for (int i = 0; i < run; ++i, ++kb) {
+                    const int tap = kb >> kcs_log2, kc = kb & (kcs - 1);
+                    // taps in the order of the packed weights: the three of the row above, then left and centre
+                    const int dy = head || tap >= 3 ? 0 : -1, dx = head ? 0 : tap >= 3 ? tap - 4 : tap - 1;
+                    const CUtensorMap *ma = (src == SRC_OLD || (src == SRC_MIXED && dy < 0)) ? ma_old : ma_new;
+                    if (elect_one()) {
+                        mbar_expect_tx(&sh.afull[ast], A_BYTES);
+                        tma_load_4d(smem_u32(stage_a(ast)), ma, &sh.afull[ast], kc * BK, dx, y0 + dy, n);
+                    }
+                    advance_a();
+                }
+            }
+        }
     }
 
     __device__ void mma_issuer(int l, int ntiles)
@@ -306,29 +322,32 @@ struct ConvEngine {
         const bool head = (l == m.n_conv);
         const uint32_t idesc = instr_desc_bf16(head ? 256 : m.ch);
         const int nkb = kblocks(l);
-        ring_for(head);
+        cut_rings(head);
         bool first = true;
         for (int id = blockIdx.x; id < ntiles && !dead; id += gridDim.x) {
             if (!__all_sync(0xffffffffu, mbar_wait(&sh.tempty[acc], aphase ^ 1u, r.ctl))) { dead = true; break; }
             tc_fence_after();
             const uint32_t d_tmem = tmem_base + (uint32_t)(acc * ACC_COLS);
             for (int kb = 0; kb < nkb;) {
-                const int run = mbar_wait_run(sh.full, stage, cur_stages, spar, nkb - kb, r.ctl);
+                int run = mbar_wait_run(sh.wfull, wst, w_stages, wpar, nkb - kb, r.ctl);
+                if (run > 0) run = mbar_wait_run(sh.afull, ast, a_stages, apar, run, r.ctl);
                 if (run == 0) { dead = true; break; }
                 tc_fence_after();
                 if (first && lane == 0) trace(1);
                 first = false;
                 for (int i = 0; i < run; ++i, ++kb) {
-                    const uint64_t adesc = smem_desc_sw128(smem_u32(stage_a(stage)));
-                    const uint64_t bdesc = smem_desc_sw128(smem_u32(stage_b(stage)));
+                    const uint64_t adesc = smem_desc_sw128(smem_u32(stage_a(ast)));
+                    const uint64_t bdesc = smem_desc_sw128(smem_u32(stage_w(wst)));
                     if (elect_one()) {
 #pragma unroll
                         for (int k = 0; k < BK / 16; ++k)
                             umma_bf16(d_tmem, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), idesc,
                                       (kb > 0 || k > 0) ? 1u : 0u);
-                        umma_commit(&sh.empty[stage]);
+                        umma_commit(&sh.aempty[ast]);
+                        umma_commit(&sh.wempty[wst]);
                     }
-                    advance_stage();
+                    advance_a();
+                    advance_w();
                 }
             }
             if (dead) break;
@@ -345,46 +364,46 @@ struct ConvEngine {
         if (lane == 0) mbar_arrive(&sh.tempty[acc]);
     }
 
-    // conv layer: ReLU(acc + bias) -> bf16, through the staging buffer so that the NHWC stores
-    // are coalesced (see the masked-MLP kernel for the layout of the staging rows)
-    __device__ void epi_hidden_tile(int l, int n, int y0, uint32_t tbase, int src)
+    // conv layer: ReLU(acc + bias) -> bf16, through the staging buffer so that the NHWC stores are coalesced.  A warp takes half
+    // the channels (64 or 32) of its quadrant's 32 pixels: rows of 128 bytes, 16-byte chunks permuted by the row number.
+    __device__ void epi_hidden_tile(int n, int y0, uint32_t tbase, int half, __nv_bfloat16 *out)
     {
-        uint8_t *stg = staging + (size_t)(warp - 2) * 8192;
+        const uint32_t stg = smem_u32(staging + (size_t)(warp - 2) * 4096);
         const float *bs = sh.bias_s[warp - 2];
-        const int bn = m.ch;
+        const int bn = m.ch, mine = bn / 2;
 #pragma unroll 1
-        for (int c0 = 0; c0 < bn; c0 += 32) {
+        for (int c0 = 0; c0 < mine; c0 += 32) {
             float v[32];
-            tmem_ld32(tbase + (uint32_t)c0, v);
-            uint32_t pk[16];
-#pragma unroll
-            for (int i = 0; i < 32; i += 2)
-                pk[i / 2] = pack_bf16x2(fmaxf(v[i] + bs[c0 + i], 0.0f), fmaxf(v[i + 1] + bs[c0 + i + 1], 0.0f));
+            tmem_ld32(tbase + (uint32_t)(half * mine + c0), v);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                const int chunk = c0 / 8 + i;
-                *reinterpret_cast<uint4 *>(stg + lane * 256 + ((chunk ^ (lane & 15)) << 4)) =
-                    make_uint4(pk[4 * i], pk[4 * i + 1], pk[4 * i + 2], pk[4 * i + 3]);
+                uint32_t pk[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int j = 8 * i + 2 * k;
+                    pk[k] = pack_bf16x2(fmaxf(v[j] + bs[c0 + j], 0.0f), fmaxf(v[j + 1] + bs[c0 + j + 1], 0.0f));
+                }
+                asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(stg + 128u * (uint32_t)lane + 16u * (uint32_t)((c0 / 8 + i) ^ (lane & 7))),
+                             "r"(pk[0]), "r"(pk[1]), "r"(pk[2]), "r"(pk[3]) : "memory");
             }
         }
         release_acc();
-        __nv_bfloat16 *out = (__nv_bfloat16 *)(src == SRC_OLD ? m.act_old[l + 1] : m.act[l + 1]);
-        const int q = warp & 3, ch = lane & 15;
-        const int col = ch * 8;
-        const int rows_valid = (min(m.height, y0 + m.R) - y0) * m.width;     // pixels of the tile inside the image
-        const size_t pix0 = (size_t)n * m.height * m.width + (size_t)y0 * m.width;
+        const int q = warp & 3, per_row = mine / 8, ch = lane & (per_row - 1);      // 8 or 4 lanes per pixel
+        const int rows_valid = (min(m.height, y0 + m.R) - y0) * m.width;            // pixels of the tile inside the image
+        __nv_bfloat16 *dst = out + ((size_t)n * m.height * m.width + (size_t)y0 * m.width) * bn + half * mine + ch * 8;
 #pragma unroll 4
-        for (int it = 0; it < 16; ++it) {
-            const int rl = it * 2 + (lane >> 4);
-            const uint4 val = *reinterpret_cast<const uint4 *>(stg + rl * 256 + ((ch ^ (rl & 15)) << 4));
-            const int prow = q * 32 + rl;
-            if (prow < rows_valid && col < bn) *reinterpret_cast<uint4 *>(out + (pix0 + prow) * bn + col) = val;
+        for (int rl = lane / per_row; rl < 32; rl += 32 / per_row) {
+            uint32_t x, y, z, w;
+            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                         : "=r"(x), "=r"(y), "=r"(z), "=r"(w)
+                         : "r"(stg + 128u * (uint32_t)rl + 16u * (uint32_t)(ch ^ (rl & 7))));
+            if (q * 32 + rl < rows_valid) *reinterpret_cast<uint4 *>(dst + (size_t)(q * 32 + rl) * bn) = make_uint4(x, y, z, w);
         }
-        fence_proxy_async();      // read by the next layer's TMA loads
+        // (The reader's proxy fence, behind its look at the stamp, orders these stores before its TMA loads.)
         __syncwarp();
         if (lane == 0) {
             __threadfence();
-            *reinterpret_cast<volatile int *>(m.stamp + 4 * (size_t)(n * m.nyt + y0 / m.R) + q) = layer_no;
+            *reinterpret_cast<volatile int *>(m.stamp + 8 * (size_t)(n * m.nyt + y0 / m.R) + warp - 2) = layer_no;
         }
     }
 
@@ -469,16 +488,16 @@ struct ConvEngine {
         const int per = head ? m.in_ch : 1;
         const int q = warp & 3;
         // Two warps share a quadrant (a warp reaches only the tensor-memory lanes of its own quadrant).  The
-        // second one takes the upper 128 classes of a 256-way head tile: the argmax is bound by instruction
-        // issue, one warp per scheduler was not enough; elsewhere it only hands the accumulator back.
+        // second one takes the upper half of the channels or of the 256 classes (the argmax is bound by instruction
+        // issue, one warp per scheduler was not enough); behind uniform noise it only hands the accumulator back.
         const int half = (warp - 2) >> 2;
         int tile_par = 0;
         const bool split_head = head && kind == EPI_CAT && r.nk == JS_NOISE_GUMBEL;
         bool any_changed = false;
         int first = INT_MAX;
         if (split_head) {
-            // Every warp is through with its staging rows.  The layers' ring is drained: all of them have seen this CTA's
-            // last accumulator.
+            // Every warp is through with its staging rows, and has seen this CTA's last accumulator: the layers' pixel ring
+            // is drained.
             asm volatile("bar.sync 5, 256;" ::: "memory");
             fence_proxy_async();
             nz_id = blockIdx.x;
@@ -490,7 +509,7 @@ struct ConvEngine {
             int n, yt, c;
             locate(id, nyl, yt_lo, per, n, yt, c);
             const int y0 = yt * m.R;
-            if (half == 1 && !(head && (split_head || kind == EPI_LOGITS))) {
+            if (half == 1 && head && !split_head && kind != EPI_LOGITS) {
                 if (!__all_sync(0xffffffffu, mbar_wait(&sh.tfull[acc], aphase, r.ctl))) { dead = true; break; }
                 tc_fence_after();
                 release_acc();
@@ -500,7 +519,7 @@ struct ConvEngine {
             if (!head) {
                 float *bs = sh.bias_s[warp - 2];
                 __syncwarp();
-                for (int i = lane; i < m.ch; i += 32) bs[i] = m.bias[l][i];
+                for (int i = lane; i < m.ch / 2; i += 32) bs[i] = m.bias[l][half * (m.ch / 2) + i];
                 __syncwarp();
             }
             if (!__all_sync(0xffffffffu, mbar_wait(&sh.tfull[acc], aphase, r.ctl))) { dead = true; break; }
@@ -508,7 +527,7 @@ struct ConvEngine {
             if (warp == 4 && lane == 0) trace(3);
             const uint32_t tbase = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * ACC_COLS);
             if (!head) {
-                epi_hidden_tile(l, n, y0, tbase, src);
+                epi_hidden_tile(n, y0, tbase, half, (__nv_bfloat16 *)(src == SRC_OLD ? m.act_old[l + 1] : m.act[l + 1]));
             } else {
                 // thread = one pixel of the tile; 256 logits of sub-pixel c
                 const int prow = q * 32 + lane;
@@ -636,9 +655,11 @@ struct ConvEngine {
         layer_no++;
         if (!head) conv_lo = yt_lo, conv_hi = yt_hi;
         if (warp == 0) {
-            producer(l, yt_lo, nyl, ntiles, src);
+            load_pixels(l, yt_lo, nyl, ntiles, src);
         } else if (warp == 1) {
             mma_issuer(l, ntiles);
+        } else if (warp == 10) {
+            load_weights(l, ntiles);
         } else {
             epilogue(l, kind, w, flag, parity, zout, yt_lo, nyl, ntiles, src);
         }
@@ -723,7 +744,8 @@ conv_tc_kernel(const __grid_constant__ ConvDev m, const __grid_constant__ RunArg
     uint8_t *ring = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const int warp = threadIdx.x >> 5;
     if (threadIdx.x == 0) {
-        for (int s = 0; s < MAX_STAGES; ++s) { mbar_init(&sh.full[s], 1); mbar_init(&sh.empty[s], 1); }
+        for (int s = 0; s < MAX_STAGES; ++s) { mbar_init(&sh.wfull[s], 1); mbar_init(&sh.wempty[s], 1); }
+        for (int s = 0; s < A_STAGES; ++s) { mbar_init(&sh.afull[s], 1); mbar_init(&sh.aempty[s], 1); }
         for (int a = 0; a < 2; ++a) { mbar_init(&sh.tfull[a], 1); mbar_init(&sh.tempty[a], 8); }
         for (int w = 0; w < 8; ++w)
             for (int i = 0; i < NOISE_BUFS; ++i) mbar_init(&sh.nfull[w][i], 1);
@@ -884,7 +906,7 @@ int js_conv_build(js_model *mo, const js_conv_desc *d)
         if (!upload<float>(mo, lut.data(), lut.size(), &ld)) return JS_ERR_CUDA;
         v.lut = ld;
     }
-    if (!upload<int>(mo, nullptr, (size_t)nb * v.nyt * 4, &v.stamp)) return JS_ERR_CUDA;
+    if (!upload<int>(mo, nullptr, (size_t)nb * v.nyt * 8, &v.stamp)) return JS_ERR_CUDA;
     CUtensorMap *pa = nullptr, *pw = nullptr, *pao = nullptr;
     if (!upload<CUtensorMap>(mo, mapsAold.data(), mapsAold.size(), &pao)) return JS_ERR_CUDA;
     v.tmActOld = pao;

@@ -93,7 +93,7 @@ struct ConvDev {
     void *act_old[JS_MAXL + 1];         // the same for the previous outer iterate (Jacobi-GS)
     const float *bias[JS_MAXL + 1];     // conv biases, head bias at [n_conv]
     const float *lut;
-    int *stamp;                         // [batch][nyt][4]: number of the last layer that wrote each quarter of a tile
+    int *stamp;                         // [batch][nyt][8]: number of the last layer that wrote each eighth of a tile
     const CUtensorMap *tmAct;           // [n_conv+1] 4-D maps {channel, x, y, image}, box 64 x width x R x 1
     const CUtensorMap *tmActOld;        // the same over act_old
     const CUtensorMap *tmW;             // [n_conv+1] 2-D maps of the packed weights
