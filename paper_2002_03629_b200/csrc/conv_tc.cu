@@ -30,14 +30,14 @@ constexpr int A_BYTES = BM * BK * 2;
 // in front has finished, and pixels.  A load takes about 1 us, the MMAs of a K block 0.14: with one ring of 4 stages for both,
 // filled when the pixels were there, the ten K blocks of a tile took 2.9 us.
 constexpr int W_RING = 80 * 1024;                     // 64 weight rows: 8 KB, 10 stages; 128: 5 stages; the head's 256: 2 stages
-constexpr int A_STAGES = 6;
+constexpr int A_RING = 120 * 1024;                    // pixels of 64 channels: 128 of them, or with the image row above them
 constexpr int MAX_STAGES = 10;
-constexpr int STAGING_BYTES = 32 * 1024;              // 4 KB per epilogue warp
+constexpr int STAGING_BYTES = 16 * 1024;              // 2 KB per epilogue warp
 constexpr int HEAD_STAGES = 2;                        // a tile of the head is one or two K blocks: pixel stages that leave room for the noise
 constexpr int NOISE_BUFS = 3;                         // per epilogue warp: boxes of 32 pixels x 32 classes
 constexpr int NOISE_BOX = 32 * 32 * 4;
 constexpr int NOISE_AT = W_RING + HEAD_STAGES * A_BYTES;      // over the rest of the layers' pixel ring and the staging rows
-constexpr int SMEM_BYTES = W_RING + A_STAGES * A_BYTES + STAGING_BYTES + 1024;
+constexpr int SMEM_BYTES = W_RING + A_RING + STAGING_BYTES + 1024;
 static_assert(NOISE_AT + 8 * NOISE_BUFS * NOISE_BOX <= SMEM_BYTES - 1024 && NOISE_AT % 1024 == 0, "room for the noise");
 constexpr int MAX_IMAGES = 256;
 
@@ -48,14 +48,13 @@ enum { EPI_HIDDEN = 0, EPI_LOGITS = 1, EPI_CAT = 3 };
 enum { SRC_NEW = 0, SRC_OLD = 1, SRC_MIXED = 2 };
 
 struct ConvShared {
-    uint64_t wfull[MAX_STAGES], wempty[MAX_STAGES], afull[A_STAGES], aempty[A_STAGES], tfull[2], tempty[2], nfull[8][NOISE_BUFS];
+    uint64_t wfull[MAX_STAGES], wempty[MAX_STAGES], afull[MAX_STAGES], aempty[MAX_STAGES], tfull[2], tempty[2], nfull[8][NOISE_BUFS];
     uint32_t tmem_base;
-    float bias_s[8][64];      // of the channels of an epilogue warp
+    alignas(16) float bias_s[8][64];      // of the channels of an epilogue warp
     float xbest[2][4][32];    // head: the upper class half's best score and class, by tile parity and quadrant
     int xbi[2][4][32];
     float lut_s[256];         // input encoding table
     int img[MAX_IMAGES];      // images still iterating
-    unsigned char keep[MAX_IMAGES];
     int n_img;
 };
 
@@ -72,7 +71,7 @@ struct ConvEngine {
     // the rings: stage in turn, bit s = parity of the next use of stage s, present cut
     int wst = 0, ast = 0;
     uint32_t wpar = 0, apar = 0;
-    int w_stages = 1, w_bytes = 0, a_stages = A_STAGES;
+    int w_stages = 1, w_bytes = 0, a_stages = 1, a_bytes = 0;
     int acc = 0;
     uint32_t aphase = 0;
     bool dead = false;
@@ -86,11 +85,11 @@ struct ConvEngine {
     int conv_lo = 0, conv_hi = 0;  // row tiles that the conv layers of this pass recompute
     // head: the noise boxes of this warp on their way.  Next box to ask for (tile, chunk of 32 classes), next buffer to fill and
     // to read, parities of the buffers' next readings
-    int nz_id = 0, nz_chunk = 0, nz_fill = 0, nz_read = 0;
+    int nz_id = 0, nz_chunk = 0, nz_fill = 0, nz_read = 0, nz_c = 0, nz_pix = 0;
     uint32_t nz_par = 0;
 
     __device__ ConvEngine(const ConvDev &m_, const RunArgs &r_, const CUtensorMap &tm_noise_, ConvShared &sh_, uint8_t *ring_)
-        : m(m_), r(r_), tm_noise(tm_noise_), sh(sh_), ring(ring_), staging(ring_ + W_RING + A_STAGES * A_BYTES)
+        : m(m_), r(r_), tm_noise(tm_noise_), sh(sh_), ring(ring_), staging(ring_ + W_RING + A_RING)
     {
         warp = threadIdx.x >> 5;
         lane = threadIdx.x & 31;
@@ -149,18 +148,30 @@ struct ConvEngine {
     // move, so nothing has to be rebuilt.  Always returns 0 (no remapping).
     __device__ int compact(int parity)
     {
-        __syncthreads();
-        // the flags are fetched by as many threads as there are images (one thread reading them one after
-        // the other paid an L2 round trip per image, 7 us per pass on a batch of 16), then one thread packs
-        for (int i = threadIdx.x; i < sh.n_img; i += blockDim.x)
-            sh.keep[i] = ld_volatile_i32(&r.smp_changed[parity * r.batch + sh.img[i]]) != 0 ? 1 : 0;
-        __syncthreads();
-        if (threadIdx.x == 0) {
+        // by one warp: the flags of all images in flight at once (read one after the other they took an L2 round trip each, 7 us
+        // per pass on a batch of 16), then a ballot per 32 images
+        if (warp == 0) {
+            const int n = sh.n_img;
+            int img[MAX_IMAGES / 32];
+            bool keep[MAX_IMAGES / 32];
+#pragma unroll
+            for (int i = 0; i < MAX_IMAGES / 32; ++i) {
+                const bool in = 32 * i + lane < n;
+                img[i] = in ? sh.img[32 * i + lane] : 0;
+                keep[i] = in && ld_volatile_i32(&r.smp_changed[parity * r.batch + img[i]]) != 0;
+            }
+            __syncwarp();
             int k = 0;
-            for (int i = 0; i < sh.n_img; ++i)
-                if (sh.keep[i]) sh.img[k++] = sh.img[i];
-            sh.n_img = k;
-            if (blockIdx.x == 0) { r.ctl->compactions += 1; r.ctl->live = k; }
+#pragma unroll
+            for (int i = 0; i < MAX_IMAGES / 32; ++i) {
+                const unsigned bal = __ballot_sync(0xffffffffu, keep[i]);
+                if (keep[i]) sh.img[k + __popc(bal & ((1u << lane) - 1u))] = img[i];
+                k += __popc(bal);
+            }
+            if (lane == 0) {
+                sh.n_img = k;
+                if (blockIdx.x == 0) { r.ctl->compactions += 1; r.ctl->live = k; }
+            }
         }
         __syncthreads();
         return 0;
@@ -176,9 +187,10 @@ struct ConvEngine {
             w_stages = min(MAX_STAGES, W_RING / bytes);
             wst = 0;
         }
-        const int as = head ? HEAD_STAGES : A_STAGES;
+        const int as = head ? HEAD_STAGES : min(MAX_STAGES, A_RING / m.stage_a);
         if (as != a_stages) {
             a_stages = as;
+            a_bytes = head ? A_BYTES : m.stage_a;
             ast = 0;
         }
     }
@@ -189,7 +201,7 @@ struct ConvEngine {
         return true;
     }
     __device__ uint8_t *stage_w(int s) const { return ring + (size_t)s * w_bytes; }
-    __device__ uint8_t *stage_a(int s) const { return ring + W_RING + (size_t)s * A_BYTES; }
+    __device__ uint8_t *stage_a(int s) const { return ring + W_RING + (size_t)s * a_bytes; }
     __device__ void advance_w()
     {
         wpar ^= 1u << wst;
@@ -284,12 +296,16 @@ struct ConvEngine {
         }
     }
 
+    // Pixel loads of a tile: a box per K block, or, where the ring holds them all (m.share), a box per horizontal shift and 64
+    // channels that has the image row above the tile too, and serves the taps of both rows.  (Not for a one-row block, which
+    // takes the two rows from different sets.)
+    __device__ bool shares(bool head, int src) const { return !head && m.share && src != SRC_MIXED; }
     __device__ void load_pixels(int l, int yt_lo, int nyl, int ntiles, int src)
     {
-        const bool head = (l == m.n_conv);
+        const bool head = (l == m.n_conv), share = shares(head, src);
         const int per = head ? m.in_ch : 1, kcs = head ? m.ch / BK : m.cin_pad[l] / BK, kcs_log2 = kcs == 2 ? 1 : 0;       // 64 or 128 channels
-        const int nkb = kblocks(l);
-        const CUtensorMap *ma_new = m.tmAct + l, *ma_old = m.tmActOld + l;
+        const int n_loads = share ? 3 * kcs : kblocks(l);
+        const CUtensorMap *ma_new = m.tmAct + l, *ma_old = m.tmActOld + l, *ma_two = (src == SRC_OLD ? m.tmActOld2 : m.tmAct2) + l;
         if (head && w_bytes != 0 && !drained(sh.aempty, a_stages, apar)) { dead = true; return; }
         cut_rings(head);
         if (lane == 0) trace(0);
@@ -299,16 +315,17 @@ struct ConvEngine {
             const int y0 = yt * m.R;
             // The head writes the image, which the tile below reads in the first layer: it waits for that tile too.
             if (l > 0 && !wait_stamps(n, yt, head ? yt + 1 : yt - 1, layer_no - 1)) { dead = true; return; }
-            for (int kb = 0; kb < nkb;) {
-                const int run = mbar_wait_run(sh.aempty, ast, a_stages, ~apar, nkb - kb, r.ctl);
+            for (int k = 0; k < n_loads;) {
+                const int run = mbar_wait_run(sh.aempty, ast, a_stages, ~apar, n_loads - k, r.ctl);
                 if (run == 0) { dead = true; return; }
-                for (int i = 0; i < run; ++i, ++kb) {
-                    const int tap = kb >> kcs_log2, kc = kb & (kcs - 1);
+                for (int i = 0; i < run; ++i, ++k) {
+                    const int tap = k >> kcs_log2, kc = k & (kcs - 1);
                     // taps in the order of the packed weights: the three of the row above, then left and centre
                     const int dy = head || tap >= 3 ? 0 : -1, dx = head ? 0 : tap >= 3 ? tap - 4 : tap - 1;
-                    const CUtensorMap *ma = (src == SRC_OLD || (src == SRC_MIXED && dy < 0)) ? ma_old : ma_new;
+                    const bool two = share && tap < 2;
+                    const CUtensorMap *ma = two ? ma_two : (src == SRC_OLD || (src == SRC_MIXED && dy < 0)) ? ma_old : ma_new;
                     if (elect_one()) {
-                        mbar_expect_tx(&sh.afull[ast], A_BYTES);
+                        mbar_expect_tx(&sh.afull[ast], two ? A_BYTES + m.width * BK * 2 : A_BYTES);
                         tma_load_4d(smem_u32(stage_a(ast)), ma, &sh.afull[ast], kc * BK, dx, y0 + dy, n);
                     }
                     advance_a();
@@ -317,44 +334,59 @@ struct ConvEngine {
         }
     }
 
-    __device__ void mma_issuer(int l, int ntiles)
+    // One thread of the warp issues everything (the ring and accumulator state of this role lives in it).  It asks for the next
+    // K block's barriers before it issues the MMAs of this one: a look at a barrier takes 150 cycles, the MMAs of a K block 256,
+    // and with look and issue one after the other a K block took 600.
+    __device__ void mma_issuer(int l, int src, int ntiles)
     {
-        const bool head = (l == m.n_conv);
+        cut_rings(l == m.n_conv);
+        __syncwarp();
+        if (elect_one()) mma_tiles(l, src, ntiles);
+        __syncwarp();
+        if (lane == 0) trace(2);
+    }
+    __device__ void mma_tiles(int l, int src, int ntiles)
+    {
+        const bool head = (l == m.n_conv), share = shares(head, src);
         const uint32_t idesc = instr_desc_bf16(head ? 256 : m.ch);
-        const int nkb = kblocks(l);
-        cut_rings(head);
+        const int nkb = kblocks(l), kcs = head ? m.ch / BK : m.cin_pad[l] / BK;
+        const int n_loads = share ? 3 * kcs : nkb;
+        const uint32_t row = (uint32_t)m.width * BK * 2;             // one image row of a stage
         bool first = true;
         for (int id = blockIdx.x; id < ntiles && !dead; id += gridDim.x) {
-            if (!__all_sync(0xffffffffu, mbar_wait(&sh.tempty[acc], aphase ^ 1u, r.ctl))) { dead = true; break; }
-            tc_fence_after();
+            if (!mbar_wait(&sh.tempty[acc], aphase ^ 1u, r.ctl)) { dead = true; break; }
             const uint32_t d_tmem = tmem_base + (uint32_t)(acc * ACC_COLS);
-            for (int kb = 0; kb < nkb;) {
-                int run = mbar_wait_run(sh.wfull, wst, w_stages, wpar, nkb - kb, r.ctl);
-                if (run > 0) run = mbar_wait_run(sh.afull, ast, a_stages, apar, run, r.ctl);
-                if (run == 0) { dead = true; break; }
+            const int a0 = ast;
+            bool w_ok = false, a_ok = false;
+            for (int kb = 0; kb < nkb; ++kb) {
+                const bool again = kb >= n_loads;
+                if (!w_ok && !mbar_wait(&sh.wfull[wst], (wpar >> wst) & 1u, r.ctl)) { dead = true; break; }
+                if (!again && !a_ok && !mbar_wait(&sh.afull[ast], (apar >> ast) & 1u, r.ctl)) { dead = true; break; }
                 tc_fence_after();
-                if (first && lane == 0) trace(1);
+                if (first) trace(1);
                 first = false;
-                for (int i = 0; i < run; ++i, ++kb) {
-                    const uint64_t adesc = smem_desc_sw128(smem_u32(stage_a(ast)));
-                    const uint64_t bdesc = smem_desc_sw128(smem_u32(stage_w(wst)));
-                    if (elect_one()) {
-#pragma unroll
-                        for (int k = 0; k < BK / 16; ++k)
-                            umma_bf16(d_tmem, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), idesc,
-                                      (kb > 0 || k > 0) ? 1u : 0u);
-                        umma_commit(&sh.aempty[ast]);
-                        umma_commit(&sh.wempty[wst]);
-                    }
-                    advance_a();
-                    advance_w();
+                // taps 3 and 4 (left, centre) of a shared load are one image row further down in the stages of taps 0 and 1
+                int a_now = again ? a0 + kb - n_loads : ast;
+                if (a_now >= a_stages) a_now -= a_stages;
+                const int w_now = wst;
+                const uint64_t adesc = smem_desc_sw128(smem_u32(stage_a(a_now)) + (again ? row : 0u));
+                const uint64_t bdesc = smem_desc_sw128(smem_u32(stage_w(w_now)));
+                advance_w();
+                if (!again) advance_a();
+                if (kb + 1 < nkb) {
+                    w_ok = mbar_test_wait(&sh.wfull[wst], (wpar >> wst) & 1u);
+                    a_ok = kb + 1 >= n_loads || mbar_test_wait(&sh.afull[ast], (apar >> ast) & 1u);
                 }
+#pragma unroll
+                for (int k = 0; k < BK / 16; ++k)
+                    umma_bf16(d_tmem, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), idesc, (kb > 0 || k > 0) ? 1u : 0u);
+                if (!share || kb >= 2 * kcs) umma_commit(&sh.aempty[a_now]);
+                umma_commit(&sh.wempty[w_now]);
             }
             if (dead) break;
-            if (elect_one()) umma_commit(&sh.tfull[acc]);
+            umma_commit(&sh.tfull[acc]);
             advance_acc();
         }
-        if (lane == 0) trace(2);
     }
 
     __device__ void release_acc()
@@ -365,42 +397,47 @@ struct ConvEngine {
     }
 
     // conv layer: ReLU(acc + bias) -> bf16, through the staging buffer so that the NHWC stores are coalesced.  A warp takes half
-    // the channels (64 or 32) of its quadrant's 32 pixels: rows of 128 bytes, 16-byte chunks permuted by the row number.
+    // the channels (64 or 32) of its quadrant's 32 pixels, 32 at a time: rows of 64 bytes, 16-byte chunks permuted by the row.
     __device__ void epi_hidden_tile(int n, int y0, uint32_t tbase, int half, __nv_bfloat16 *out)
     {
-        const uint32_t stg = smem_u32(staging + (size_t)(warp - 2) * 4096);
-        const float *bs = sh.bias_s[warp - 2];
-        const int bn = m.ch, mine = bn / 2;
+        const uint32_t stg = smem_u32(staging) + 2048u * (uint32_t)(warp - 2), bs = smem_u32(sh.bias_s[warp - 2]);
+        const int bn = m.ch, mine = bn / 2, q = warp & 3;
+        const int rows_valid = (min(m.height, y0 + m.R) - y0) * m.width;            // pixels of the tile inside the image
+        // readback: four lanes per pixel, eight pixels at once
+        const int ch = lane & 3, r0 = lane >> 2;
+        __nv_bfloat16 *dst = out + ((size_t)n * m.height * m.width + (size_t)y0 * m.width + q * 32 + r0) * bn + half * mine + ch * 8;
 #pragma unroll 1
         for (int c0 = 0; c0 < mine; c0 += 32) {
             float v[32];
             tmem_ld32(tbase + (uint32_t)(half * mine + c0), v);
+            if (c0 + 32 == mine) release_acc();
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 uint32_t pk[4];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int j = 8 * i + 2 * k;
-                    pk[k] = pack_bf16x2(fmaxf(v[j] + bs[c0 + j], 0.0f), fmaxf(v[j + 1] + bs[c0 + j + 1], 0.0f));
+                for (int k = 0; k < 2; ++k) {
+                    const int j = 8 * i + 4 * k;
+                    float4 b;
+                    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w) : "r"(bs + 4u * (uint32_t)(c0 + j)));
+                    pk[2 * k] = pack_bf16x2(fmaxf(v[j] + b.x, 0.0f), fmaxf(v[j + 1] + b.y, 0.0f));
+                    pk[2 * k + 1] = pack_bf16x2(fmaxf(v[j + 2] + b.z, 0.0f), fmaxf(v[j + 3] + b.w, 0.0f));
                 }
-                asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(stg + 128u * (uint32_t)lane + 16u * (uint32_t)((c0 / 8 + i) ^ (lane & 7))),
+                asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(stg + 64u * (uint32_t)lane + 16u * (uint32_t)(i ^ ((lane >> 1) & 3))),
                              "r"(pk[0]), "r"(pk[1]), "r"(pk[2]), "r"(pk[3]) : "memory");
             }
-        }
-        release_acc();
-        const int q = warp & 3, per_row = mine / 8, ch = lane & (per_row - 1);      // 8 or 4 lanes per pixel
-        const int rows_valid = (min(m.height, y0 + m.R) - y0) * m.width;            // pixels of the tile inside the image
-        __nv_bfloat16 *dst = out + ((size_t)n * m.height * m.width + (size_t)y0 * m.width) * bn + half * mine + ch * 8;
-#pragma unroll 4
-        for (int rl = lane / per_row; rl < 32; rl += 32 / per_row) {
-            uint32_t x, y, z, w;
-            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
-                         : "=r"(x), "=r"(y), "=r"(z), "=r"(w)
-                         : "r"(stg + 128u * (uint32_t)rl + 16u * (uint32_t)(ch ^ (rl & 7))));
-            if (q * 32 + rl < rows_valid) *reinterpret_cast<uint4 *>(dst + (size_t)(q * 32 + rl) * bn) = make_uint4(x, y, z, w);
+            __syncwarp();
+#pragma unroll
+            for (int it = 0; it < 4; ++it) {
+                const int rl = 8 * it + r0;
+                uint32_t x, y, z, w;
+                asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                             : "=r"(x), "=r"(y), "=r"(z), "=r"(w)
+                             : "r"(stg + 64u * (uint32_t)rl + 16u * (uint32_t)(ch ^ ((rl >> 1) & 3))));
+                if (q * 32 + rl < rows_valid) *reinterpret_cast<uint4 *>(dst + (size_t)(8 * it) * bn + c0) = make_uint4(x, y, z, w);
+            }
+            __syncwarp();
         }
         // (The reader's proxy fence, behind its look at the stamp, orders these stores before its TMA loads.)
-        __syncwarp();
         if (lane == 0) {
             __threadfence();
             *reinterpret_cast<volatile int *>(m.stamp + 8 * (size_t)(n * m.nyt + y0 / m.R) + warp - 2) = layer_no;
@@ -411,25 +448,33 @@ struct ConvEngine {
     // as there are buffers.  (Read by the threads, a lane per pixel, every 16-byte load of a warp touched 32 lines: 7 us per
     // tile of 128 pixels, a quarter of a whole pass.)
     __device__ uint8_t *noise_buf(int b) const { return ring + NOISE_AT + (size_t)((warp - 2) * NOISE_BUFS + b) * NOISE_BOX; }
+    // the first tile from nz_id on whose quadrant does not lie below the image
+    __device__ void noise_tile(int yt_lo, int nyl, int ntiles)
+    {
+        const int q = warp & 3;
+        for (; nz_id < ntiles; nz_id += gridDim.x) {
+            int n, yt;
+            locate(nz_id, nyl, yt_lo, m.in_ch, n, yt, nz_c);
+            const int y0 = yt * m.R;
+            nz_pix = (n * m.height + y0) * m.width + q * 32;
+            if (q * 32 < (min(m.height, y0 + m.R) - y0) * m.width) break;
+        }
+        nz_chunk = 0;
+    }
     __device__ void noise_ask(int yt_lo, int nyl, int ntiles)
     {
-        const int q = warp & 3, half = (warp - 2) >> 2;
-        while (nz_id < ntiles) {
-            int n, yt, c;
-            locate(nz_id, nyl, yt_lo, m.in_ch, n, yt, c);
-            const int y0 = yt * m.R;
-            if (q * 32 < (min(m.height, y0 + m.R) - y0) * m.width) {      // else the quadrant lies below the image
-                if (elect_one()) {
-                    uint64_t *bar = &sh.nfull[warp - 2][nz_fill];
-                    mbar_expect_tx(bar, NOISE_BOX);
-                    tma_load_3d(smem_u32(noise_buf(nz_fill)), &tm_noise, bar, half * 128 + nz_chunk * 32, c, (n * m.height + y0) * m.width + q * 32);
-                }
-                __syncwarp();
-                if (++nz_fill == NOISE_BUFS) nz_fill = 0;
-                if (++nz_chunk == 4) { nz_chunk = 0; nz_id += gridDim.x; }
-                return;
-            }
+        if (nz_id >= ntiles) return;
+        const int half = (warp - 2) >> 2;
+        if (elect_one()) {
+            uint64_t *bar = &sh.nfull[warp - 2][nz_fill];
+            mbar_expect_tx(bar, NOISE_BOX);
+            tma_load_3d(smem_u32(noise_buf(nz_fill)), &tm_noise, bar, half * 128 + nz_chunk * 32, nz_c, nz_pix);
+        }
+        __syncwarp();
+        if (++nz_fill == NOISE_BUFS) nz_fill = 0;
+        if (++nz_chunk == 4) {
             nz_id += gridDim.x;
+            noise_tile(yt_lo, nyl, ntiles);
         }
     }
 
@@ -501,7 +546,7 @@ struct ConvEngine {
             asm volatile("bar.sync 5, 256;" ::: "memory");
             fence_proxy_async();
             nz_id = blockIdx.x;
-            nz_chunk = 0;
+            noise_tile(yt_lo, nyl, ntiles);
             for (int i = 0; i < NOISE_BUFS; ++i) noise_ask(yt_lo, nyl, ntiles);
         }
         int id = blockIdx.x;
@@ -657,7 +702,7 @@ struct ConvEngine {
         if (warp == 0) {
             load_pixels(l, yt_lo, nyl, ntiles, src);
         } else if (warp == 1) {
-            mma_issuer(l, ntiles);
+            mma_issuer(l, src, ntiles);
         } else if (warp == 10) {
             load_weights(l, ntiles);
         } else {
@@ -745,7 +790,7 @@ conv_tc_kernel(const __grid_constant__ ConvDev m, const __grid_constant__ RunArg
     const int warp = threadIdx.x >> 5;
     if (threadIdx.x == 0) {
         for (int s = 0; s < MAX_STAGES; ++s) { mbar_init(&sh.wfull[s], 1); mbar_init(&sh.wempty[s], 1); }
-        for (int s = 0; s < A_STAGES; ++s) { mbar_init(&sh.afull[s], 1); mbar_init(&sh.aempty[s], 1); }
+        for (int s = 0; s < MAX_STAGES; ++s) { mbar_init(&sh.afull[s], 1); mbar_init(&sh.aempty[s], 1); }
         for (int a = 0; a < 2; ++a) { mbar_init(&sh.tfull[a], 1); mbar_init(&sh.tempty[a], 8); }
         for (int w = 0; w < 8; ++w)
             for (int i = 0; i < NOISE_BUFS; ++i) mbar_init(&sh.nfull[w][i], 1);
@@ -841,7 +886,11 @@ int js_conv_build(js_model *mo, const js_conv_desc *d)
     const size_t npix = (size_t)nb * d->height * d->width;
     auto group = [&](int k) { return (int)(((long long)d->in_ch * k) / ch); };
 
-    std::vector<CUtensorMap> mapsA(d->n_conv + 1), mapsAold(d->n_conv + 1), mapsW(d->n_conv + 1);
+    // a pixel stage with the row above the tile, if three shifts of all channels fit into the ring
+    const int two = (v.R + 1) * d->width * BK * 2;
+    v.share = 3 * (ch / BK) * two <= A_RING;
+    v.stage_a = v.share ? two : A_BYTES;
+    std::vector<CUtensorMap> mapsA(d->n_conv + 1), mapsAold(d->n_conv + 1), mapsA2(d->n_conv + 1), mapsAold2(d->n_conv + 1), mapsW(d->n_conv + 1);
     for (int l = 0; l <= d->n_conv; ++l) {
         const int c_l = l == 0 ? 64 : ch;                 // channels of act[l] (the image is padded to 64)
         if (l < d->n_conv) v.cin_pad[l] = c_l;
@@ -854,7 +903,9 @@ int js_conv_build(js_model *mo, const js_conv_desc *d)
             const cuuint64_t strides[3] = {(cuuint64_t)c_l * 2, (cuuint64_t)d->width * c_l * 2,
                                            (cuuint64_t)d->height * d->width * c_l * 2};
             const cuuint32_t box[4] = {(cuuint32_t)BK, (cuuint32_t)d->width, (cuuint32_t)v.R, 1};
+            const cuuint32_t box2[4] = {(cuuint32_t)BK, (cuuint32_t)d->width, (cuuint32_t)v.R + 1, 1};
             if (!encode_nd(set == 0 ? &mapsA[l] : &mapsAold[l], a, 4, dims, strides, box)) return JS_ERR_UNSUPPORTED;
+            if (!encode_nd(set == 0 ? &mapsA2[l] : &mapsAold2[l], a, 4, dims, strides, box2)) return JS_ERR_UNSUPPORTED;
         }
     }
     static const int tky[5] = {0, 0, 0, 1, 1}, tkx[5] = {0, 1, 2, 0, 1};
@@ -907,7 +958,11 @@ int js_conv_build(js_model *mo, const js_conv_desc *d)
         v.lut = ld;
     }
     if (!upload<int>(mo, nullptr, (size_t)nb * v.nyt * 8, &v.stamp)) return JS_ERR_CUDA;
-    CUtensorMap *pa = nullptr, *pw = nullptr, *pao = nullptr;
+    CUtensorMap *pa = nullptr, *pw = nullptr, *pao = nullptr, *pa2 = nullptr, *pao2 = nullptr;
+    if (!upload<CUtensorMap>(mo, mapsA2.data(), mapsA2.size(), &pa2)) return JS_ERR_CUDA;
+    if (!upload<CUtensorMap>(mo, mapsAold2.data(), mapsAold2.size(), &pao2)) return JS_ERR_CUDA;
+    v.tmAct2 = pa2;
+    v.tmActOld2 = pao2;
     if (!upload<CUtensorMap>(mo, mapsAold.data(), mapsAold.size(), &pao)) return JS_ERR_CUDA;
     v.tmActOld = pao;
     if (!upload<CUtensorMap>(mo, mapsA.data(), mapsA.size(), &pa)) return JS_ERR_CUDA;

@@ -96,6 +96,8 @@ struct ConvDev {
     int *stamp;                         // [batch][nyt][8]: number of the last layer that wrote each eighth of a tile
     const CUtensorMap *tmAct;           // [n_conv+1] 4-D maps {channel, x, y, image}, box 64 x width x R x 1
     const CUtensorMap *tmActOld;        // the same over act_old
+    const CUtensorMap *tmAct2, *tmActOld2;      // the same with boxes of R + 1 rows
+    int share, stage_a;                 // conv layers load R + 1 rows at once; bytes of a pixel stage
     const CUtensorMap *tmW;             // [n_conv+1] 2-D maps of the packed weights
 };
 

@@ -363,43 +363,48 @@ struct TcEngine {
         }
     }
 
+    // One thread of the warp issues everything (the ring and accumulator state of this role lives in it).  It asks for the next
+    // stage's barrier before it issues the MMAs of this one: a look at a barrier takes 150 cycles, the MMAs of a K block
+    // 2 x (tile width), and look, issue and commit one after the other came to 400 and more.
     __device__ void mma_issuer(int l, int nt_lo, int nt_hi, int MT)
+    {
+        ring_for_layer(l);
+        __syncwarp();
+        if (elect_one()) mma_units(l, nt_lo, nt_hi, MT);
+        __syncwarp();
+        if (lane == 0) trace(2);
+    }
+    __device__ void mma_units(int l, int nt_lo, int nt_hi, int MT)
     {
         const TcLayer &ly = t.lay[l];
         const uint32_t idesc = instr_desc_bf16(ly.bn);
-        ring_for_layer(l);
         int e, e_end;
         unit_list(l, MT, e, e_end);
         Unit u;
         bool first = true;
-        while (!dead && next_unit(l, e, e_end, nt_lo, nt_hi, MT, u)) {
-            if (!__all_sync(0xffffffffu, mbar_wait(&sh.tempty[acc], aphase ^ 1u, r.ctl))) { dead = true; break; }
-            tc_fence_after();
+        while (next_unit(l, e, e_end, nt_lo, nt_hi, MT, u)) {
+            if (!mbar_wait(&sh.tempty[acc], aphase ^ 1u, r.ctl)) { dead = true; return; }
             const uint32_t d_tmem = tmem_base + (uint32_t)(acc * ACC_COLS);
-            for (int kb = u.kb0; kb < u.kb1;) {
-                const int run = mbar_wait_run(sh.full, stage, cur_stages, spar, u.kb1 - kb, r.ctl);
-                if (run == 0) { dead = true; break; }
+            bool ready = false;
+            for (int kb = u.kb0; kb < u.kb1; ++kb) {
+                if (!ready && !mbar_wait(&sh.full[stage], (spar >> stage) & 1u, r.ctl)) { dead = true; return; }
                 tc_fence_after();
-                if (first && lane == 0) trace(1);
+                if (first) trace(1);
                 first = false;
-                for (int i = 0; i < run; ++i, ++kb) {
-                    const uint64_t adesc = smem_desc_sw128(smem_u32(stage_a(stage)));
-                    const uint64_t bdesc = smem_desc_sw128(smem_u32(stage_b(stage)));
-                    if (elect_one()) {
+                const int now = stage;
+                const uint64_t adesc = smem_desc_sw128(smem_u32(stage_a(now)));
+                const uint64_t bdesc = smem_desc_sw128(smem_u32(stage_b(now)));
+                advance_stage();
+                ready = mbar_test_wait(&sh.full[stage], (spar >> stage) & 1u);
 #pragma unroll
-                        for (int k = 0; k < BK / 16; ++k)       // 16 bf16 = 32 bytes per instruction along K
-                            umma_bf16(d_tmem, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), idesc,
-                                      (kb > u.kb0 || k > 0) ? 1u : 0u);
-                        umma_commit(&sh.empty[stage]);          // frees the stage once these MMAs have read it
-                    }
-                    advance_stage();
-                }
+                for (int k = 0; k < BK / 16; ++k)               // 16 bf16 = 32 bytes per instruction along K
+                    umma_bf16(d_tmem, adesc + (uint64_t)(2 * k), bdesc + (uint64_t)(2 * k), idesc,
+                              (kb > u.kb0 || k > 0) ? 1u : 0u);
+                umma_commit(&sh.empty[now]);                    // frees the stage once these MMAs have read it
             }
-            if (dead) break;
-            if (elect_one()) umma_commit(&sh.tfull[acc]);       // accumulator complete
+            umma_commit(&sh.tfull[acc]);                        // accumulator complete
             advance_acc();
         }
-        if (lane == 0) trace(2);
     }
 
     // ---- partial sums.  Layout of a slot: [column / 4][128 rows] float4, written and read with

@@ -318,9 +318,15 @@ __device__ __forceinline__ void argmax_chunk32(const float (&s)[32], int c0, flo
 #pragma unroll
         for (int i = 0; i < w; ++i) t[i] = fmaxf(t[i], t[i + w]);
     const float mx = t[0];
-    int idx = 31;
+    // four chains of eight selects, not one of 32: the chain is what a warp waits for
+    int at[4];
 #pragma unroll
-    for (int i = 30; i >= 0; --i) idx = (s[i] == mx) ? i : idx;
+    for (int g = 0; g < 4; ++g) {
+        at[g] = 32;
+#pragma unroll
+        for (int i = 7; i >= 0; --i) at[g] = (s[8 * g + i] == mx) ? 8 * g + i : at[g];
+    }
+    const int idx = min(31, min(min(at[0], at[1]), min(at[2], at[3])));
     const bool upd = mx > best;
     best = upd ? mx : best;
     bi = upd ? c0 + idx : bi;
