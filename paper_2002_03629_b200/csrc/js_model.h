@@ -35,7 +35,7 @@ struct TcDev {
     int bin_bulk;                // binary output rows are 16-byte granular: moved by bulk copies
     int grid;                    // CTAs the schedules were built for (the launch uses exactly this)
     float *partials;             // [slot][columns/4][128 rows] float4: fp32 partial sums of non-owning chunks
-    unsigned *pflags;            // [slot][4 row quadrants]: phase stamp once the partial is stored
+    unsigned *pflags;            // [slot][4 row quadrants][2 column halves]: phase stamp once the partial is stored
     int n_pflags;
 };
 

@@ -29,10 +29,15 @@ namespace {
 
 constexpr int BM = TC_BM;          // samples per tile (UMMA M)
 constexpr int BK = TC_BK;          // bf16 elements per K block
-constexpr int NTH = 192;
+// Warp 0 loads, warp 1 issues MMAs, the others do the epilogues: EH per tensor-memory lane quadrant, each with its share of a
+// tile's columns.  Two in models with binary outputs (with one, an owner's epilogue in a 4096-wide layer lasted 5.6 us and a
+// partial sum's 3.1, of a phase of 20).  One in models with 256-way outputs, whose time goes into loading the output layer's
+// weights while the epilogues of other tiles run, and whose epilogue needs the registers.
+constexpr int threads_of(int EH) { return 64 + 128 * EH; }
+constexpr int MAX_WARPS = 10;
 constexpr int ACC_COLS = 256;      // TMEM columns per accumulator slot (two slots)
 constexpr int A_BYTES = BM * BK * 2;
-constexpr int STAGING_BYTES = 32 * 1024;   // epilogue transposition buffer, 8 KB per epilogue warp
+constexpr int STAGING_BYTES = 32 * 1024;   // epilogue transposition buffer, 4 KB per epilogue warp
 constexpr int MAX_STAGES = 6;
 // binary output tiles: per sample row 128 noise values and 128 symbols, rows padded by 16 bytes
 constexpr int BIN_NZ_ROW = 512 + 16, BIN_XS_ROW = 128 + 16;
@@ -47,18 +52,20 @@ enum { EPI_HIDDEN = 0, EPI_LOGITS = 1, EPI_BINARY = 2, EPI_CAT = 3 };
 
 struct TcShared {
     uint64_t full[MAX_STAGES], empty[MAX_STAGES], tfull[2], tempty[2];
-    uint64_t nzbar[4];             // per epilogue warp: bulk copies of a binary tile's noise and symbols
+    uint64_t nzbar[8];             // per epilogue warp: bulk copies of its noise and symbols
     uint32_t tmem_base;
     int off[JS_MAXL + 1];          // start of layer l's tile metadata inside `meta`
     float lut_s[256];              // input encoding table (a lookup per committed symbol would be an L2 round trip)
-    alignas(16) float bias_s[4][256];   // per epilogue warp: bias of the current tile's columns (read as float4)
-    int wcnt[NTH / 32];            // compaction: per-warp counts
+    alignas(16) float bias_s[4][256];   // per pair of epilogue warps: bias of the current tile's columns (read as float4)
+    int wcnt[MAX_WARPS];           // compaction: per-warp counts
     int cbase;                     // compaction: rows kept so far
 };
 
 // ------------------------------------------------------------------ engine
+template <int EH>
 struct TcEngine {
     static constexpr bool has_jgs = false;
+    static constexpr int NTH = threads_of(EH);
     const MadeDev &m;
     const TcDev &t;
     const RunArgs &r;
@@ -411,13 +418,16 @@ struct TcEngine {
     // thread = row, so stores and loads are coalesced without any transposition.
     __device__ size_t tile_floats(int l) const { return (size_t)BM * t.lay[l].bn; }
 
-    // non-owning chunk: accumulator -> its slot, then raise the slot's flag for this row quadrant
+    // which share of a tile's columns is this warp's (logits: all are the first one's)
+    __device__ int half() const { return EH == 1 ? 0 : (warp - 2) >> 2; }
+
+    // non-owning chunk: accumulator -> its slot, then raise the slot's flag for this warp's rows and columns
     __device__ void store_partial(int l, int slot, uint32_t tbase)
     {
-        const int q = warp & 3, row = q * 32 + lane;
+        const int q = warp & 3, row = q * 32 + lane, w = t.lay[l].bn / EH;
         float4 *base = reinterpret_cast<float4 *>(t.partials + (size_t)slot * tile_floats(l)) + row;
 #pragma unroll 1
-        for (int c0 = 0; c0 < t.lay[l].bn; c0 += 32) {
+        for (int c0 = half() * w; c0 < (half() + 1) * w; c0 += 32) {
             uint32_t ra[32];
             tmem_ld32_issue(tbase + (uint32_t)c0, ra);
             tmem_wait_ld();
@@ -427,23 +437,23 @@ struct TcEngine {
                                                               __uint_as_float(ra[4 * i + 2]), __uint_as_float(ra[4 * i + 3]));
         }
         release_acc();
-        __threadfence();
         __syncwarp();
         if (lane == 0) {
-            unsigned *f = t.pflags + (size_t)slot * 4 + q;
+            unsigned *f = t.pflags + (size_t)slot * 8 + EH * q + half();
             asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(f), "r"(stamp) : "memory");
         }
     }
 
-    // owner: bounded wait until this warp's row quadrant of every partial of the tile is stored
-    __device__ bool wait_partials(int slot, int nparts)
+    // owner: bounded wait until this warp's rows of every partial of the tile are stored (its share of the columns, or all)
+    __device__ bool wait_partials(int slot, int nparts, bool all)
     {
         // lane p polls the flag of partial p: one round trip for all of them instead of one each
-        const int q = warp & 3;
+        const int q = warp & 3, per = all ? EH : 1, n = per * nparts;
         int ok = 1;
-        for (int p0 = 0; p0 < nparts && ok; p0 += 32) {
-            const bool mine = p0 + lane < nparts;
-            const unsigned *f = t.pflags + (size_t)(slot + p0 + (mine ? lane : 0)) * 4 + q;
+        for (int p0 = 0; p0 < n && ok; p0 += 32) {
+            const bool mine = p0 + lane < n;
+            const int p = mine ? p0 + lane : 0;
+            const unsigned *f = t.pflags + (size_t)(slot + p / per) * 8 + EH * q + (all ? p % per : half());
             uint64_t t0 = 0;
             for (unsigned i = 0;; ++i) {
                 const bool set = !mine || ld_acquire_u32(f) == stamp;
@@ -459,12 +469,38 @@ struct TcEngine {
                 }
             }
         }
-        __threadfence();
+        __syncwarp();             // the polls were acquires
         return ok != 0;
     }
 
-    // the same for 64 columns held in two register groups, with all sixteen loads of a partial in
-    // flight together (one memory latency per partial instead of two)
+    // Add the tile's partial sums, in chunk order, to accumulator columns starting at c0.  Sixteen loads are in flight together,
+    // as the registers allow: two partials of 32 columns ...
+    __device__ void add_partials(uint32_t (&ra)[32], int c0) const
+    {
+        const int row = (warp & 3) * 32 + lane;
+        const float4 *base = reinterpret_cast<const float4 *>(cur_pbase) + row + (size_t)(c0 / 4) * BM;
+        const size_t next = cur_tile_floats / 4;
+#pragma unroll 1
+        for (int p = 0; p < cur_parts; p += 2) {
+            const bool two = p + 1 < cur_parts;
+            float4 v[8], u[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                v[i] = __ldcg(base + (size_t)p * next + (size_t)i * BM);
+                u[i] = two ? __ldcg(base + (size_t)(p + 1) * next + (size_t)i * BM) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const float s[4] = {v[i].x, v[i].y, v[i].z, v[i].w}, s2[4] = {u[i].x, u[i].y, u[i].z, u[i].w};
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const float a = __uint_as_float(ra[4 * i + k]) + s[k];
+                    ra[4 * i + k] = __float_as_uint(two ? a + s2[k] : a);
+                }
+            }
+        }
+    }
+    // ... or one of 64, held in two register groups
     __device__ void add_partials64(uint32_t (&ra)[32], uint32_t (&rb)[32], int c0) const
     {
         const int row = (warp & 3) * 32 + lane;
@@ -487,23 +523,6 @@ struct TcEngine {
         }
     }
 
-    // add the tile's partial sums, in chunk order, to 32 accumulator columns starting at c0
-    __device__ void add_partials(uint32_t (&ra)[32], int c0) const
-    {
-        const int row = (warp & 3) * 32 + lane;
-        for (int p = 0; p < cur_parts; ++p) {
-            const float4 *base = reinterpret_cast<const float4 *>(cur_pbase + (size_t)p * cur_tile_floats) + row;
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const float4 v = __ldcg(base + (size_t)(c0 / 4 + i) * BM);
-                ra[4 * i] = __float_as_uint(__uint_as_float(ra[4 * i]) + v.x);
-                ra[4 * i + 1] = __float_as_uint(__uint_as_float(ra[4 * i + 1]) + v.y);
-                ra[4 * i + 2] = __float_as_uint(__uint_as_float(ra[4 * i + 2]) + v.z);
-                ra[4 * i + 3] = __float_as_uint(__uint_as_float(ra[4 * i + 3]) + v.w);
-            }
-        }
-    }
-
     // ---- chunk-wise epilogues: thread = one sample row of the tile, 32 columns at a time
     __device__ void epi_logits(float *zout, int row, int n0, int c0, const float (&v)[32])
     {
@@ -516,19 +535,18 @@ struct TcEngine {
             if (col + i < N) zout[(size_t)row * N + col + i] = v[i] + bias[col + i];
     }
 
-    // ---- whole-tile epilogues that go through shared memory so that global accesses are
-    // coalesced.  Each epilogue warp owns 32 rows of the tile and an 8 KB staging area holding
-    // 32 rows x 256 bytes; 16-byte chunk c of row r sits at chunk c ^ (r & 15) (conflict-free both
-    // for the row-per-lane writes and for the row-wise reads).
-    // (at the end of the auxiliary buffer: the part before it serves hidden layers as extra ring stages)
-    __device__ uint8_t *my_staging() const { return staging + (t.aux_bytes - STAGING_BYTES) + (size_t)(warp - 2) * 8192; }
+    // ---- hidden layers go through shared memory so that global accesses are coalesced: 4 KB per epilogue warp, 32 rows x 64
+    // activations.  (At the end of the auxiliary buffer: the part before it serves hidden layers as extra ring stages.)
+    __device__ uint32_t my_staging() const { return smem_u32(staging + (t.aux_bytes - STAGING_BYTES)) + 4096u * (uint32_t)(warp - 2); }
 
-    __device__ void load_bias_tile(int l, int n0, int bn)
+    // bias of columns [c, c + n) of the layer, for this warp alone (two warps of a quadrant share a row of 256)
+    __device__ float *my_bias() { return sh.bias_s[(warp - 2) & 3] + 256 / EH * half(); }
+    __device__ void load_bias(int l, int c, int n)
     {
-        float *bs = sh.bias_s[warp - 2];
+        float *bs = my_bias();
         const int N = m.n[l + 1];
         __syncwarp();
-        for (int i = lane; i < bn; i += 32) bs[i] = (n0 + i < N) ? m.bias[l][n0 + i] : 0.0f;
+        for (int i = lane; i < n; i += 32) bs[i] = (c + i < N) ? m.bias[l][c + i] : 0.0f;
         __syncwarp();
     }
 
@@ -539,56 +557,70 @@ struct TcEngine {
         if (lane == 0) mbar_arrive(&sh.tempty[acc]);
     }
 
-    // accumulator columns [half*64, half*64+64) of this warp's 32 rows -> staging, raw fp32,
-    // row-per-lane (thread = TMEM lane), 16-byte chunks swizzled by row
-    __device__ void stage_half(uint32_t tbase, int half)
-    {
-        uint8_t *stg = my_staging();
-        uint32_t ra[32], rb[32];
-        tmem_ld32_issue(tbase + (uint32_t)(half * 64), ra);       // two loads in flight per wait
-        tmem_ld32_issue(tbase + (uint32_t)(half * 64 + 32), rb);
-        tmem_wait_ld();
-        if (cur_parts > 0) add_partials64(ra, rb, half * 64);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            *reinterpret_cast<uint4 *>(stg + lane * 256 + ((i ^ (lane & 15)) << 4)) =
-                make_uint4(ra[4 * i], ra[4 * i + 1], ra[4 * i + 2], ra[4 * i + 3]);
-            *reinterpret_cast<uint4 *>(stg + lane * 256 + (((i + 8) ^ (lane & 15)) << 4)) =
-                make_uint4(rb[4 * i], rb[4 * i + 1], rb[4 * i + 2], rb[4 * i + 3]);
-        }
-    }
-
-    // The row-wise passes below give half a warp to each row: lane -> row pair member (lane >> 4)
-    // and 16-byte chunk (lane & 15) = four consecutive columns.  Their loops are kept rolled: these
-    // kernels are instruction-cache bound when every path is unrolled.
-
-    // hidden layer: act(acc + bias) -> bf16, 64 columns at a time
+    // hidden layer: act(acc + partial sums + bias) -> bf16, a warp's share of the columns, up to 64 at a time.  Rows of 128 bytes
+    // in the staging area, 16-byte chunks permuted by the row number: lane = row writes, eight (or four) lanes per row read.
     __device__ void epi_hidden_tile(int l, int mt, int n0, uint32_t tbase)
     {
-        uint8_t *stg = my_staging();
-        const float *bs = sh.bias_s[warp - 2];
-        const int N = m.n[l + 1];
-        __nv_bfloat16 *out = (__nv_bfloat16 *)m.a[l + 1];
-        const int q = warp & 3, ch = lane & 15, rsel = lane >> 4;
-        const int act = m.act;
-        const int halves = t.lay[l].bn / 64;
+        const uint32_t stg = my_staging(), bs = smem_u32(my_bias());
+        const int N = m.n[l + 1], q = warp & 3, w = t.lay[l].bn / EH, act = m.act;
+        const int per_row = min(w, 64) / 8, ch = lane & (per_row - 1), r0 = lane / per_row, step = 32 / per_row;
+        __nv_bfloat16 *out = (__nv_bfloat16 *)m.a[l + 1] + (size_t)(mt * BM + q * 32) * N;
 #pragma unroll 1
-        for (int half = 0; half < halves; ++half) {
-            stage_half(tbase, half);
-            if (half == halves - 1) { release_acc(); if (warp == 4 && lane == 0) trace(6); } else __syncwarp();
-            const int cb = half * 64 + ch * 4;
-            const float b0 = bs[cb], b1 = bs[cb + 1], b2 = bs[cb + 2], b3 = bs[cb + 3];
-            const int col = n0 + cb;
+        for (int c0 = 0; c0 < w; c0 += EH == 1 ? 64 : 32) {
+            const int cb = half() * w + c0;
+            uint32_t ra[32];
+            tmem_ld32_issue(tbase + (uint32_t)cb, ra);
+            if constexpr (EH == 1) {
+                uint32_t rb[32];
+                tmem_ld32_issue(tbase + (uint32_t)(cb + 32), rb);
+                tmem_wait_ld();
+                if (c0 + 64 >= w) release_acc();
+                if (cur_parts > 0) add_partials64(ra, rb, cb);
+                stage32(stg, bs + 4u * (uint32_t)(c0 + 32), 4, act, rb);
+            } else {
+                tmem_wait_ld();
+                if (c0 + 32 >= w) release_acc();
+                if (cur_parts > 0) add_partials(ra, cb);
+            }
+            if (warp == 4 && lane == 0) trace(6);
+            stage32(stg, bs + 4u * (uint32_t)c0, (c0 & 32) / 8, act, ra);
+            if (EH == 2 && (c0 & 32) == 0 && c0 + 32 < w) continue;
+            __syncwarp();
+            const int col = n0 + half() * w + (c0 & ~63) + 8 * ch;
 #pragma unroll 4
-            for (int it = 0; it < 16; ++it) {
-                const int rl = it * 2 + rsel;
-                const float4 v = *reinterpret_cast<const float4 *>(stg + rl * 256 + ((ch ^ (rl & 15)) << 4));
-                const int row = mt * BM + q * 32 + rl;
-                const uint32_t p0 = pack_bf16x2(tc_act_fn(act, v.x + b0), tc_act_fn(act, v.y + b1));
-                const uint32_t p1 = pack_bf16x2(tc_act_fn(act, v.z + b2), tc_act_fn(act, v.w + b3));
-                if (row < live && col < N) *reinterpret_cast<uint2 *>(out + (size_t)row * N + col) = make_uint2(p0, p1);
+            for (int rl = r0; rl < 32; rl += step) {
+                uint4 v;
+                asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                             : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                             : "r"(stg + 128u * (uint32_t)rl + 16u * (uint32_t)(ch ^ (rl & 7))));
+                if (mt * BM + q * 32 + rl < live && col < N) *reinterpret_cast<uint4 *>(out + (size_t)rl * N + col) = v;
             }
             __syncwarp();
+        }
+    }
+    // 32 columns of lane's row, as chunks first .. first + 3 of its staging row.  One activation's code per call: an epilogue runs
+    // once or twice per phase and fetches its instructions anew each time, so it pays for every one that stands in its way.
+    __device__ __forceinline__ void stage32(uint32_t stg, uint32_t bs, int first, int act, const uint32_t (&ra)[32])
+    {
+        if (act == JS_ACT_RELU) stage32_act<JS_ACT_RELU>(stg, bs, first, ra);
+        else stage32_act<JS_ACT_GELU_TANH>(stg, bs, first, ra);
+    }
+    template <int ACT>
+    __device__ __forceinline__ void stage32_act(uint32_t stg, uint32_t bs, int first, const uint32_t (&ra)[32])
+    {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            uint32_t pk[4];
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const int j = 8 * i + 4 * k;
+                float4 b;
+                asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w) : "r"(bs + 4u * (uint32_t)j));
+                pk[2 * k] = pack_bf16x2(tc_act_fn(ACT, __uint_as_float(ra[j]) + b.x), tc_act_fn(ACT, __uint_as_float(ra[j + 1]) + b.y));
+                pk[2 * k + 1] = pack_bf16x2(tc_act_fn(ACT, __uint_as_float(ra[j + 2]) + b.z), tc_act_fn(ACT, __uint_as_float(ra[j + 3]) + b.w));
+            }
+            asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(stg + 128u * (uint32_t)lane + 16u * (uint32_t)((first + i) ^ (lane & 7))),
+                         "r"(pk[0]), "r"(pk[1]), "r"(pk[2]), "r"(pk[3]) : "memory");
         }
     }
 
@@ -607,45 +639,46 @@ struct TcEngine {
         raised_stamp = stamp;
     }
 
-    // ---- binary output layer (128 positions per tile), thread = one sample row of the tile.
-    // The row's noise (512 bytes) and current symbols (128 bytes) are brought into shared memory by
+    // ---- binary output layer (128 positions per tile), thread = one sample row of the tile and 64 of its positions.
+    // Their noise (256 bytes) and current symbols (64 bytes) are brought into shared memory by
     // bulk copies that are issued before the accumulator is waited for, so they travel while the
     // K loop still runs; rows are padded by 16 bytes, which makes the row-per-lane 16-byte accesses
     // conflict-free.  The new symbols replace the old ones in place, the new encodings (bf16)
     // overwrite the part of the noise row that has been consumed, and a row in which something
     // changed goes back to global memory as two bulk stores.
-    __device__ uint8_t *nz_row() const { return staging + (size_t)((warp & 3) * 32 + lane) * BIN_NZ_ROW; }
-    __device__ uint8_t *xs_row() const { return staging + BIN_NZ_BYTES + (size_t)((warp & 3) * 32 + lane) * BIN_XS_ROW; }
+    __device__ uint8_t *nz_warp() const { return staging + (size_t)((warp & 3) * 32) * BIN_NZ_ROW + 256 * half(); }
+    __device__ uint8_t *xs_warp() const { return staging + BIN_NZ_BYTES + (size_t)((warp & 3) * 32) * BIN_XS_ROW + 64 * half(); }
+    __device__ uint8_t *nz_row() const { return nz_warp() + (size_t)lane * BIN_NZ_ROW; }
+    __device__ uint8_t *xs_row() const { return xs_warp() + (size_t)lane * BIN_XS_ROW; }
 
     __device__ void bin_fetch_rows(int smp, int n0, int ncols)
     {
-        const int q = warp & 3;
         bulk_wait_read();                     // this thread's earlier bulk stores no longer read the rows
         __syncwarp();
         if (t.bin_bulk) {
             const uint32_t bytes = smp >= 0 ? (uint32_t)ncols * 5u : 0u;
             const uint32_t tot = __reduce_add_sync(0xffffffffu, bytes);
-            if (lane == 0) mbar_expect_tx(&sh.nzbar[q], tot);
+            if (lane == 0) mbar_expect_tx(&sh.nzbar[warp - 2], tot);
             __syncwarp();
-            if (smp >= 0) {
+            if (smp >= 0 && ncols > 0) {
                 const size_t at = (size_t)smp * m.T + n0;
-                bulk_load(smem_u32(nz_row()), r.noise + at, (uint32_t)ncols * 4u, &sh.nzbar[q]);
-                bulk_load(smem_u32(xs_row()), r.x + at, (uint32_t)ncols, &sh.nzbar[q]);
+                bulk_load(smem_u32(nz_row()), r.noise + at, (uint32_t)ncols * 4u, &sh.nzbar[warp - 2]);
+                bulk_load(smem_u32(xs_row()), r.x + at, (uint32_t)ncols, &sh.nzbar[warp - 2]);
             }
         } else {
             // Rows that do not start on 16 bytes: the warp takes its 32 rows in turn, lane = column (coalesced whatever the
             // length of a row), four rows' loads in flight together.
-            uint8_t *nz = staging + (size_t)(q * 32) * BIN_NZ_ROW, *xs = staging + BIN_NZ_BYTES + (size_t)(q * 32) * BIN_XS_ROW;
+            uint8_t *nz = nz_warp(), *xs = xs_warp();
 #pragma unroll 1
             for (int r0 = 0; r0 < 32; r0 += 4) {
-                float nv[4][4];
-                uint8_t xv[4][4];
+                float nv[4][2];
+                uint8_t xv[4][2];
 #pragma unroll
                 for (int rr = 0; rr < 4; ++rr) {
                     const int s = __shfl_sync(0xffffffffu, smp, r0 + rr);
                     const size_t at = (size_t)max(s, 0) * m.T + n0;
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
+                    for (int k = 0; k < 2; ++k) {
                         const int c = 32 * k + lane;
                         const bool in = s >= 0 && c < ncols;
                         nv[rr][k] = in ? __ldg(r.noise + at + c) : 0.0f;
@@ -655,7 +688,7 @@ struct TcEngine {
 #pragma unroll
                 for (int rr = 0; rr < 4; ++rr)
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
+                    for (int k = 0; k < 2; ++k) {
                         *reinterpret_cast<float *>(nz + (r0 + rr) * BIN_NZ_ROW + 4 * (32 * k + lane)) = nv[rr][k];
                         xs[(r0 + rr) * BIN_XS_ROW + 32 * k + lane] = xv[rr][k];
                     }
@@ -670,13 +703,13 @@ struct TcEngine {
     __device__ bool epi_binary_tile(const Win &w, int smp, int rw, int n0, int ncols, uint32_t tbase, bool flag,
                                     int parity, bool &wany, int &wfirst)
     {
-        const float *bs = sh.bias_s[warp - 2];
+        const float *bs = my_bias();
         uint8_t *nz = nz_row(), *xs = xs_row();
         const float lut0 = sh.lut_s[0], lut1 = sh.lut_s[1];
         // columns [clo, chi) of the tile are sampled; the others keep their symbol
         const int clo = max(w.plo - n0, 0), chi = min(min(w.phi, m.T) - n0, ncols);
         if (t.bin_bulk) {
-            if (!mbar_wait(&sh.nzbar[warp & 3], nzphase, r.ctl)) return false;
+            if (!mbar_wait(&sh.nzbar[warp - 2], nzphase, r.ctl)) return false;
             nzphase ^= 1u;
         }
         uint32_t diff_any = 0, fdiff = 0;
@@ -684,61 +717,59 @@ struct TcEngine {
         const bool tr = (warp == 4 && lane == 0);
         if (tr) trace(6);
 #pragma unroll 1
-        for (int c0 = 0; c0 < BM; c0 += 32) {
+        for (int c0 = 0; c0 < BM / 2; c0 += 32) {
             uint32_t ra[32];
             __syncwarp();
-            tmem_ld32_issue(tbase + (uint32_t)c0, ra);
+            tmem_ld32_issue(tbase + (uint32_t)(64 * half() + c0), ra);
             tmem_wait_ld();
-            if (c0 == BM - 32) release_acc();
-            if (cur_parts > 0) add_partials(ra, c0);
-            if (smp >= 0 && c0 < ncols) {
-                // everything the 32 columns need is read before anything is written: the stores below
-                // go to the same rows, and a load may not overtake a store it might alias
-                float4 e4[8], b4[8];
-                uint4 xo4[2];
+            if (c0 == BM / 2 - 32) release_acc();
+            if (cur_parts > 0) add_partials(ra, 64 * half() + c0);
+            if (smp >= 0 && c0 < ncols)
 #pragma unroll
-                for (int i = 0; i < 8; ++i) e4[i] = *reinterpret_cast<const float4 *>(nz + (c0 + i * 4) * 4);
+                for (int cc = 0; cc < 32; cc += 16) {
+                    // everything the 16 columns need is read before anything is written: the stores below
+                    // go to the same rows, and a load may not overtake a store it might alias
+                    const int cq = c0 + cc;
+                    float4 e4[4];
 #pragma unroll
-                for (int i = 0; i < 2; ++i) xo4[i] = *reinterpret_cast<const uint4 *>(xs + c0 + i * 16);
+                    for (int i = 0; i < 4; ++i) e4[i] = *reinterpret_cast<const float4 *>(nz + (cq + i * 4) * 4);
+                    const uint4 xo4 = *reinterpret_cast<const uint4 *>(xs + cq);
+                    uint32_t xn[4];
+                    uint2 en[4];
 #pragma unroll
-                for (int i = 0; i < 8; ++i) b4[i] = *reinterpret_cast<const float4 *>(bs + c0 + i * 4);
-                uint32_t xn[8];
-                uint2 en[8];
+                    for (int i = 0; i < 4; ++i) {
+                        const int c = cq + i * 4;
+                        const float4 b4 = *reinterpret_cast<const float4 *>(bs + c);
+                        const uint32_t xw = i == 0 ? xo4.x : i == 1 ? xo4.y : i == 2 ? xo4.z : xo4.w;
+                        const float e[4] = {e4[i].x, e4[i].y, e4[i].z, e4[i].w};
+                        const float bb[4] = {b4.x, b4.y, b4.z, b4.w};
+                        uint32_t nw = 0;
+                        float enc[4];
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int c = c0 + i * 4;
-                    const uint32_t xw = (i & 3) == 0 ? xo4[i >> 2].x : (i & 3) == 1 ? xo4[i >> 2].y
-                                      : (i & 3) == 2 ? xo4[i >> 2].z : xo4[i >> 2].w;
-                    const float e[4] = {e4[i].x, e4[i].y, e4[i].z, e4[i].w};
-                    const float bb[4] = {b4[i].x, b4[i].y, b4[i].z, b4[i].w};
-                    uint32_t nw = 0;
-                    float enc[4];
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const uint32_t o = (xw >> (8 * k)) & 0xffu;
-                        const float z = __uint_as_float(ra[i * 4 + k]) + bb[k];
-                        const bool in = (unsigned)(c + k - clo) < (unsigned)(chi - clo);
-                        const uint32_t nv = in ? (uint32_t)js_sample_binary(NK, z, e[k]) : o;
-                        nw |= nv << (8 * k);
-                        enc[k] = nv ? lut1 : lut0;
+                        for (int k = 0; k < 4; ++k) {
+                            const uint32_t o = (xw >> (8 * k)) & 0xffu;
+                            const float z = __uint_as_float(ra[cc + i * 4 + k]) + bb[k];
+                            const bool in = (unsigned)(c + k - clo) < (unsigned)(chi - clo);
+                            const uint32_t nv = in ? (uint32_t)js_sample_binary(NK, z, e[k]) : o;
+                            nw |= nv << (8 * k);
+                            enc[k] = nv ? lut1 : lut0;
+                        }
+                        const uint32_t df = nw ^ xw;
+                        // first word with a change and its difference, by selects; the position follows below
+                        const bool newfirst = df != 0u && fword == INT_MAX;
+                        fword = newfirst ? c : fword;
+                        fdiff = newfirst ? df : fdiff;
+                        diff_any |= df;
+                        xn[i] = nw;
+                        en[i] = make_uint2(pack_bf16x2(enc[0], enc[1]), pack_bf16x2(enc[2], enc[3]));
                     }
-                    const uint32_t df = nw ^ xw;
-                    // first word with a change and its difference, by selects; the position follows below
-                    const bool newfirst = df != 0u && fword == INT_MAX;
-                    fword = newfirst ? c : fword;
-                    fdiff = newfirst ? df : fdiff;
-                    diff_any |= df;
-                    xn[i] = nw;
-                    en[i] = make_uint2(pack_bf16x2(enc[0], enc[1]), pack_bf16x2(enc[2], enc[3]));
-                }
-                // new symbols in place; encodings over noise that has been consumed (bytes [2c, 2c+8)
-                // of the row lie below the noise of column c+4 and beyond)
-                *reinterpret_cast<uint4 *>(xs + c0) = make_uint4(xn[0], xn[1], xn[2], xn[3]);
-                *reinterpret_cast<uint4 *>(xs + c0 + 16) = make_uint4(xn[4], xn[5], xn[6], xn[7]);
+                    // new symbols in place; encodings over noise that has been consumed (bytes [2c, 2c+8)
+                    // of the row lie below the noise of column c+4 and beyond)
+                    *reinterpret_cast<uint4 *>(xs + cq) = make_uint4(xn[0], xn[1], xn[2], xn[3]);
 #pragma unroll
-                for (int i = 0; i < 8; i += 2)
-                    *reinterpret_cast<uint4 *>(nz + (c0 + i * 4) * 2) = make_uint4(en[i].x, en[i].y, en[i + 1].x, en[i + 1].y);
-            }
+                    for (int i = 0; i < 4; i += 2)
+                        *reinterpret_cast<uint4 *>(nz + (cq + i * 4) * 2) = make_uint4(en[i].x, en[i].y, en[i + 1].x, en[i + 1].y);
+                }
         }
         __syncwarp();
         if (tr) trace(7);
@@ -753,16 +784,15 @@ struct TcEngine {
             }
         } else {
             // changed rows, one after the other, lane = column; the encodings' rows start on 16 bytes (n[0])
-            const uint8_t *nzw = staging + (size_t)((warp & 3) * 32) * BIN_NZ_ROW;
-            const uint8_t *xsw = staging + BIN_NZ_BYTES + (size_t)((warp & 3) * 32) * BIN_XS_ROW;
+            const uint8_t *nzw = nz_warp(), *xsw = xs_warp();
             __syncwarp();
             for (unsigned todo = __ballot_sync(0xffffffffu, changed); todo != 0u; todo &= todo - 1u) {
                 const int rr = __ffs((int)todo) - 1;
                 const int s = __shfl_sync(0xffffffffu, smp, rr), rwr = __shfl_sync(0xffffffffu, rw, rr);
 #pragma unroll
-                for (int k = 0; k < 4; ++k)
+                for (int k = 0; k < 2; ++k)
                     if (32 * k + lane < ncols) r.x[(size_t)s * m.T + n0 + 32 * k + lane] = xsw[rr * BIN_XS_ROW + 32 * k + lane];
-                if (8 * lane < ncols && lane < 16)
+                if (8 * lane < ncols && lane < 8)
                     *reinterpret_cast<uint4 *>((__nv_bfloat16 *)m.a[0] + (size_t)rwr * m.n[0] + n0 + 8 * lane) =
                         *reinterpret_cast<const uint4 *>(nzw + rr * BIN_NZ_ROW + 16 * lane);
             }
@@ -801,10 +831,10 @@ struct TcEngine {
         const int q = warp & 3;
         __syncwarp();                         // every lane is done with the previous tile's rows
         const uint32_t tot = __reduce_add_sync(0xffffffffu, sample >= 0 ? 1024u : 0u);
-        if (lane == 0) mbar_expect_tx(&sh.nzbar[q], tot);
+        if (lane == 0) mbar_expect_tx(&sh.nzbar[warp - 2], tot);
         __syncwarp();
         if (sample >= 0)
-            bulk_load(smem_u32(cat_row()), r.noise + ((size_t)sample * m.T + d) * 256, 1024u, &sh.nzbar[q]);
+            bulk_load(smem_u32(cat_row()), r.noise + ((size_t)sample * m.T + d) * 256, 1024u, &sh.nzbar[warp - 2]);
     }
     __device__ bool epi_cat_tile(int sample, int row, int d, uint32_t tbase, const Win &w, bool flag, int parity,
                                  bool &any_changed, int &first)
@@ -814,7 +844,7 @@ struct TcEngine {
         const float *gg = smem_rows ? reinterpret_cast<const float *>(cat_row())
                                     : r.noise + ((size_t)max(sample, 0) * m.T + d) * 256;
         if (smem_rows) {
-            if (!mbar_wait(&sh.nzbar[warp & 3], nzphase, r.ctl)) return false;
+            if (!mbar_wait(&sh.nzbar[warp - 2], nzphase, r.ctl)) return false;
             nzphase ^= 1u;
         }
         float best = -INFINITY;
@@ -995,13 +1025,19 @@ struct TcEngine {
         while (!dead && next_unit(l, e, e_end, nt_lo, nt_hi, MT, u)) {
             const int nt = u.nt, mt = u.mt;
             const bool owner = u.nparts >= 0;
-            if (owner && kind != EPI_LOGITS) load_bias_tile(l, nt * ly.bn, ly.bn);
+            if (owner && half() == 1 && kind == EPI_LOGITS) {
+                if (!mbar_wait(&sh.tfull[acc], aphase, r.ctl)) { dead = true; break; }
+                release_acc();
+                advance_acc();
+                continue;
+            }
+            if (owner && kind != EPI_LOGITS) load_bias(l, nt * ly.bn + half() * (ly.bn / EH), ly.bn / EH);
             int csmp = -1;
-            if (owner && kind == EPI_CAT && r.nk != JS_NOISE_GUMBEL) {
+            if (EH == 1 && owner && kind == EPI_CAT && r.nk != JS_NOISE_GUMBEL) {
                 const int rw = mt * BM + q * 32 + lane;
                 csmp = rw < live ? perm_cur()[rw] : -1;
             }
-            if (owner && kind == EPI_CAT && r.nk == JS_NOISE_GUMBEL) {
+            if (EH == 1 && owner && kind == EPI_CAT && r.nk == JS_NOISE_GUMBEL) {
                 const int rw = mt * BM + q * 32 + lane;
                 csmp = rw < live ? perm_cur()[rw] : -1;
                 if (!cat_ahead) cat_prefetch(csmp, nt);          // first tile of the phase
@@ -1016,18 +1052,18 @@ struct TcEngine {
                 }
             }
             int bsmp = -1, bcols = 0;
-            if (owner && kind == EPI_BINARY) {
+            if (EH == 2 && owner && kind == EPI_BINARY) {
                 const int rw = mt * BM + q * 32 + lane;
                 bsmp = rw < live ? perm_cur()[rw] : -1;
-                bcols = min(BM, m.T - nt * ly.bn);
-                bin_fetch_rows(bsmp, nt * ly.bn, bcols);     // in flight while the tile is still being computed
+                bcols = max(0, min(BM / 2, m.T - (nt * ly.bn + half() * (BM / 2))));
+                bin_fetch_rows(bsmp, nt * ly.bn + half() * (BM / 2), bcols);     // in flight while the tile is still being computed
             }
             if (owner) {
                 cur_parts = u.nparts;
                 cur_pbase = t.partials + (size_t)u.slot * tile_floats(l);
                 cur_tile_floats = tile_floats(l);
                 // partial sums do not depend on this CTA's accumulator: wait for them first
-                if (cur_parts > 0 && !wait_partials(u.slot, cur_parts)) { dead = true; break; }
+                if (cur_parts > 0 && !wait_partials(u.slot, cur_parts, kind == EPI_LOGITS)) { dead = true; break; }
             }
             if (!mbar_wait(&sh.tfull[acc], aphase, r.ctl)) { dead = true; break; }
             tc_fence_after();
@@ -1042,15 +1078,15 @@ struct TcEngine {
             }
             if (kind == EPI_HIDDEN) {
                 epi_hidden_tile(l, mt, n0, tbase);
-            } else if (kind == EPI_BINARY) {
+            } else if (EH == 2 && kind == EPI_BINARY) {
                 bool wany = false;
                 int wfirst = INT_MAX;
                 const bool fine = r.nk == JS_NOISE_LOGISTIC
-                    ? epi_binary_tile<JS_NOISE_LOGISTIC>(w, bsmp, row, n0, bcols, tbase, flag, parity, wany, wfirst)
-                    : epi_binary_tile<JS_NOISE_UNIFORM_ICDF>(w, bsmp, row, n0, bcols, tbase, flag, parity, wany, wfirst);
+                    ? epi_binary_tile<JS_NOISE_LOGISTIC>(w, bsmp, row, n0 + half() * (BM / 2), bcols, tbase, flag, parity, wany, wfirst)
+                    : epi_binary_tile<JS_NOISE_UNIFORM_ICDF>(w, bsmp, row, n0 + half() * (BM / 2), bcols, tbase, flag, parity, wany, wfirst);
                 if (!fine) { dead = true; break; }
                 if (wany) { any_changed = true; first = min(first, wfirst); }
-            } else if (kind == EPI_CAT) {
+            } else if (EH == 1 && kind == EPI_CAT) {
                 const bool fine = r.nk == JS_NOISE_GUMBEL ? epi_cat_tile(csmp, row, nt, tbase, w, flag, parity, any_changed, first)
                                                           : epi_icdf_tile(csmp, row, nt, tbase, w, flag, parity, any_changed, first);
                 if (!fine) { dead = true; break; }
@@ -1110,7 +1146,7 @@ struct TcEngine {
     // pipeline is instantiated once in the kernel
     __device__ bool step(const Win &w, bool flag, int parity, float *zout)
     {
-        const int out_kind = zout ? EPI_LOGITS : (m.C == 1 ? EPI_BINARY : EPI_CAT);
+        const int out_kind = zout ? EPI_LOGITS : EH == 2 ? EPI_BINARY : EPI_CAT;
         for (int l = 0; l <= m.L; ++l) {
             const bool last = (l == m.L);
             const bool did = gemm_phase(l, last ? out_kind : EPI_HIDDEN, w, last && flag, parity, zout);
@@ -1121,7 +1157,8 @@ struct TcEngine {
     }
 };
 
-__global__ void __launch_bounds__(NTH, 1)
+template <int EH>
+__global__ void __launch_bounds__(threads_of(EH), 1)
 made_tc_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ TcDev t, const __grid_constant__ RunArgs r)
 {
     extern __shared__ uint8_t smem_raw[];
@@ -1133,8 +1170,8 @@ made_tc_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ TcDev 
         r.trace[((size_t)js_trace_who(r) * JS_TRACE_PHASES) * JS_TRACE_SLOTS + 2] = global_ns();   // kernel entry
     if (threadIdx.x == 0) {
         for (int s = 0; s < MAX_STAGES; ++s) { mbar_init(&sh.full[s], 1); mbar_init(&sh.empty[s], 1); }
-        for (int a = 0; a < 2; ++a) { mbar_init(&sh.tfull[a], 1); mbar_init(&sh.tempty[a], 4); }
-        for (int a = 0; a < 4; ++a) mbar_init(&sh.nzbar[a], 1);
+        for (int a = 0; a < 2; ++a) { mbar_init(&sh.tfull[a], 1); mbar_init(&sh.tempty[a], 4 * EH); }
+        for (int a = 0; a < 8; ++a) mbar_init(&sh.nzbar[a], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async();
     }
@@ -1163,7 +1200,7 @@ made_tc_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ TcDev 
     __syncthreads();
     tc_fence_after();
 
-    TcEngine e(m, t, r, sh, ring, meta);
+    TcEngine<EH> e(m, t, r, sh, ring, meta);
     e.tmem_base = sh.tmem_base;
     if (threadIdx.x == 0) e.trace(0);
     DriverResult res = made_driver(e, m.T, r);
@@ -1186,6 +1223,10 @@ made_tc_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ TcDev 
 }
 
 }  // namespace
+
+// binary outputs: two epilogue warps per quadrant; 256-way outputs: one
+static int tc_threads(const MadeDev &v) { return threads_of(v.C == 1 ? 2 : 1); }
+static const void *tc_kernel_of(const MadeDev &v) { return v.C == 1 ? (const void *)made_tc_kernel<2> : (const void *)made_tc_kernel<1>; }
 
 // Weight layout of this kernel: K-block major, [K block][padded unit][64 inputs], so that the
 // bn x 64 box of one TMA load is one contiguous piece of memory (bn x 128 bytes) instead of bn
@@ -1500,7 +1541,7 @@ int js_tc_prepare(js_model *mo)
         if (cudaMalloc(&q, std::max<size_t>(part_floats, 4) * sizeof(float)) != cudaSuccess) return JS_ERR_CUDA;
         mo->allocs.push_back(q);
         t.partials = (float *)q;
-        t.n_pflags = std::max(max_slots, 1) * 4;
+        t.n_pflags = std::max(max_slots, 1) * 8;
         if (cudaMalloc(&q, (size_t)t.n_pflags * sizeof(unsigned)) != cudaSuccess) return JS_ERR_CUDA;
         mo->allocs.push_back(q);
         if (cudaMemset(q, 0, (size_t)t.n_pflags * sizeof(unsigned)) != cudaSuccess) return JS_ERR_CUDA;
@@ -1519,12 +1560,13 @@ int js_tc_prepare(js_model *mo)
     t.smem_bytes = 1024 + t.ring_bytes + t.aux_bytes + meta_bytes;
     // the attribute belongs to the function, not to a model: always allow the largest request
     const int smem = SMEM_DYN_MAX;
-    if (cudaFuncSetAttribute(made_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
+    const void *kernel = tc_kernel_of(v);
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
         cudaGetLastError();      // not sticky: the CUDA-core kernels will serve this model
         return 0;
     }
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, made_tc_kernel, NTH, smem) != cudaSuccess || per_sm < 1)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, tc_threads(v), smem) != cudaSuccess || per_sm < 1)
         return 0;
     mo->tc_max_grid = sms;      // one CTA per SM: each owns all 512 TMEM columns
     mo->tc_ok = 1;
@@ -1539,7 +1581,6 @@ int js_launch_made_tc(const js_model *mo, const RunArgs &r, cudaStream_t stream)
     const int grid = std::min(t.grid, mo->tc_max_grid);
     if (grid != t.grid) return (int)cudaErrorInvalidConfiguration;     // the schedules need exactly t.grid CTAs
     void *args[3] = {(void *)&v, (void *)&t, (void *)&r};
-    cudaError_t e = cudaLaunchCooperativeKernel((const void *)made_tc_kernel, dim3(grid), dim3(NTH), args,
-                                                t.smem_bytes, stream);
+    cudaError_t e = cudaLaunchCooperativeKernel(tc_kernel_of(v), dim3(grid), dim3(tc_threads(v)), args, t.smem_bytes, stream);
     return e == cudaSuccess ? 0 : (int)e;
 }
