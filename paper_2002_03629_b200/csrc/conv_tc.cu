@@ -23,7 +23,8 @@
 namespace {
 
 constexpr int BM = TC_BM, BK = TC_BK;
-constexpr int NTH = 352;          // warp 0 loads pixels, warp 1 MMA, warps 2-9 epilogue: two per tensor-memory lane quadrant, warp 10 loads weights
+// warp 0 loads pixels, warp 1 MMA, warps 2-9 epilogue: two per tensor-memory lane quadrant, warp 10 loads weights, 11 the head's noise
+constexpr int NTH = 384;
 constexpr int ACC_COLS = 256;
 constexpr int A_BYTES = BM * BK * 2;
 // Two rings, each with a loading warp of its own: weights, which wait for nothing but room and so are there before the layer
@@ -34,11 +35,11 @@ constexpr int A_RING = 120 * 1024;                    // pixels of 64 channels: 
 constexpr int MAX_STAGES = 10;
 constexpr int STAGING_BYTES = 16 * 1024;              // 2 KB per epilogue warp
 constexpr int HEAD_STAGES = 2;                        // a tile of the head is one or two K blocks: pixel stages that leave room for the noise
-constexpr int NOISE_BUFS = 3;                         // per epilogue warp: boxes of 32 pixels x 32 classes
-constexpr int NOISE_BOX = 32 * 32 * 4;
+constexpr int NOISE_BUFS = 3;                         // per half of the classes: boxes of 128 pixels x 32 classes
+constexpr int NOISE_BOX = 128 * 32 * 4;
 constexpr int NOISE_AT = W_RING + HEAD_STAGES * A_BYTES;      // over the rest of the layers' pixel ring and the staging rows
 constexpr int SMEM_BYTES = W_RING + A_RING + STAGING_BYTES + 1024;
-static_assert(NOISE_AT + 8 * NOISE_BUFS * NOISE_BOX <= SMEM_BYTES - 1024 && NOISE_AT % 1024 == 0, "room for the noise");
+static_assert(NOISE_AT + 2 * NOISE_BUFS * NOISE_BOX <= SMEM_BYTES - 1024 && NOISE_AT % 1024 == 0, "room for the noise");
 constexpr int MAX_IMAGES = 256;
 
 enum { EPI_HIDDEN = 0, EPI_LOGITS = 1, EPI_CAT = 3 };
@@ -48,9 +49,9 @@ enum { EPI_HIDDEN = 0, EPI_LOGITS = 1, EPI_CAT = 3 };
 enum { SRC_NEW = 0, SRC_OLD = 1, SRC_MIXED = 2 };
 
 struct ConvShared {
-    uint64_t wfull[MAX_STAGES], wempty[MAX_STAGES], afull[MAX_STAGES], aempty[MAX_STAGES], tfull[2], tempty[2], nfull[8][NOISE_BUFS];
+    uint64_t wfull[MAX_STAGES], wempty[MAX_STAGES], afull[MAX_STAGES], aempty[MAX_STAGES], tfull[2], tempty[2], nfull[2][NOISE_BUFS], nempty[2][NOISE_BUFS];
     uint32_t tmem_base;
-    alignas(16) float bias_s[8][64];      // of the channels of an epilogue warp
+    alignas(16) float bias_s[8][128];     // of the channels or classes of an epilogue warp
     float xbest[2][4][32];    // head: the upper class half's best score and class, by tile parity and quadrant
     int xbi[2][4][32];
     float lut_s[256];         // input encoding table
@@ -83,9 +84,8 @@ struct ConvEngine {
     // barrier behind it, of which 3 us were the barrier and the way back to the first load).
     int layer_no = 0;              // layers done by this launch, the current one included (the same in every CTA)
     int conv_lo = 0, conv_hi = 0;  // row tiles that the conv layers of this pass recompute
-    // head: the noise boxes of this warp on their way.  Next box to ask for (tile, chunk of 32 classes), next buffer to fill and
-    // to read, parities of the buffers' next readings
-    int nz_id = 0, nz_chunk = 0, nz_fill = 0, nz_read = 0, nz_c = 0, nz_pix = 0;
+    // head: next noise buffer (loaded or read by this warp), bit b = parity of buffer b's next use
+    int nz_buf = 0;
     uint32_t nz_par = 0;
 
     __device__ ConvEngine(const ConvDev &m_, const RunArgs &r_, const CUtensorMap &tm_noise_, ConvShared &sh_, uint8_t *ring_)
@@ -444,37 +444,43 @@ struct ConvEngine {
         }
     }
 
-    // ---- head: the noise of a warp's 32 pixels and 128 classes goes through shared memory in boxes of 32 classes, so many ahead
-    // as there are buffers.  (Read by the threads, a lane per pixel, every 16-byte load of a warp touched 32 lines: 7 us per
-    // tile of 128 pixels, a quarter of a whole pass.)
-    __device__ uint8_t *noise_buf(int b) const { return ring + NOISE_AT + (size_t)((warp - 2) * NOISE_BUFS + b) * NOISE_BOX; }
-    // the first tile from nz_id on whose quadrant does not lie below the image
-    __device__ void noise_tile(int yt_lo, int nyl, int ntiles)
+    static __device__ __forceinline__ float4 lds_f4(uint32_t a)
     {
-        const int q = warp & 3;
-        for (; nz_id < ntiles; nz_id += gridDim.x) {
-            int n, yt;
-            locate(nz_id, nyl, yt_lo, m.in_ch, n, yt, nz_c);
-            const int y0 = yt * m.R;
-            nz_pix = (n * m.height + y0) * m.width + q * 32;
-            if (q * 32 < (min(m.height, y0 + m.R) - y0) * m.width) break;
-        }
-        nz_chunk = 0;
+        float4 v;
+        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a));
+        return v;
     }
-    __device__ void noise_ask(int yt_lo, int nyl, int ntiles)
+
+    // ---- head: the noise of a tile goes through shared memory, from a warp of its own, in boxes of 128 pixels x 32 classes.
+    // (Read by the threads, a lane per pixel, every 16-byte load of a warp touched 32 lines: 7 us per tile, a quarter of a whole
+    // pass.  Asked for by the epilogue warps themselves, a box cost them 0.23 us each, of 0.9 per 32 classes.)
+    __device__ uint8_t *noise_buf(int half, int b) const { return ring + NOISE_AT + (size_t)(half * NOISE_BUFS + b) * NOISE_BOX; }
+    // Head, epilogue warps and the one that loads the noise: every warp is through with its staging rows and has seen this CTA's
+    // last accumulator, so the layers' pixel ring is drained too.
+    __device__ void noise_may_come()
     {
-        if (nz_id >= ntiles) return;
-        const int half = (warp - 2) >> 2;
-        if (elect_one()) {
-            uint64_t *bar = &sh.nfull[warp - 2][nz_fill];
-            mbar_expect_tx(bar, NOISE_BOX);
-            tma_load_3d(smem_u32(noise_buf(nz_fill)), &tm_noise, bar, half * 128 + nz_chunk * 32, nz_c, nz_pix);
-        }
-        __syncwarp();
-        if (++nz_fill == NOISE_BUFS) nz_fill = 0;
-        if (++nz_chunk == 4) {
-            nz_id += gridDim.x;
-            noise_tile(yt_lo, nyl, ntiles);
+        asm volatile("bar.sync 5, 288;" ::: "memory");
+        fence_proxy_async();
+    }
+    __device__ void load_noise(int yt_lo, int nyl, int ntiles)
+    {
+        for (int id = blockIdx.x; id < ntiles; id += gridDim.x) {
+            int n, yt, c;
+            locate(id, nyl, yt_lo, m.in_ch, n, yt, c);
+            const int pix = (n * m.height + yt * m.R) * m.width;
+            for (int k = 0; k < 4; ++k) {
+                for (int half = 0; half < 2; ++half) {
+                    if (!__all_sync(0xffffffffu, mbar_wait(&sh.nempty[half][nz_buf], ((nz_par >> nz_buf) & 1u) ^ 1u, r.ctl))) { dead = true; return; }
+                    if (elect_one()) {
+                        uint64_t *bar = &sh.nfull[half][nz_buf];
+                        mbar_expect_tx(bar, NOISE_BOX);
+                        tma_load_3d(smem_u32(noise_buf(half, nz_buf)), &tm_noise, bar, half * 128 + k * 32, c, pix);
+                    }
+                    __syncwarp();
+                }
+                nz_par ^= 1u << nz_buf;
+                if (++nz_buf == NOISE_BUFS) nz_buf = 0;
+            }
         }
     }
 
@@ -540,15 +546,7 @@ struct ConvEngine {
         const bool split_head = head && kind == EPI_CAT && r.nk == JS_NOISE_GUMBEL;
         bool any_changed = false;
         int first = INT_MAX;
-        if (split_head) {
-            // Every warp is through with its staging rows, and has seen this CTA's last accumulator: the layers' pixel ring
-            // is drained.
-            asm volatile("bar.sync 5, 256;" ::: "memory");
-            fence_proxy_async();
-            nz_id = blockIdx.x;
-            noise_tile(yt_lo, nyl, ntiles);
-            for (int i = 0; i < NOISE_BUFS; ++i) noise_ask(yt_lo, nyl, ntiles);
-        }
+        if (split_head) noise_may_come();
         int id = blockIdx.x;
         for (; id < ntiles && !dead; id += gridDim.x) {
             int n, yt, c;
@@ -561,10 +559,12 @@ struct ConvEngine {
                 advance_acc();
                 continue;
             }
-            if (!head) {
+            if (!head || split_head) {
+                const float *bias = head ? m.bias[l] + (size_t)c * 256 + half * 128 : m.bias[l] + half * (m.ch / 2);
                 float *bs = sh.bias_s[warp - 2];
                 __syncwarp();
-                for (int i = lane; i < m.ch / 2; i += 32) bs[i] = m.bias[l][half * (m.ch / 2) + i];
+                if (4 * lane < (head ? 128 : m.ch / 2))
+                    *reinterpret_cast<float4 *>(bs + 4 * lane) = __ldg(reinterpret_cast<const float4 *>(bias) + lane);
                 __syncwarp();
             }
             if (!__all_sync(0xffffffffu, mbar_wait(&sh.tfull[acc], aphase, r.ctl))) { dead = true; break; }
@@ -599,27 +599,24 @@ struct ConvEngine {
                         if (!valid) continue;
 #pragma unroll
                         for (int i = 0; i < 32; ++i) zout[at * 256 + c0 + i] = v[i] + bias[c0 + i];
-                    } else if (q * 32 < rows_valid) {
-                        if (!__all_sync(0xffffffffu, mbar_wait(&sh.nfull[warp - 2][nz_read], (nz_par >> nz_read) & 1u, r.ctl))) { dead = true; break; }
-                        nz_par ^= 1u << nz_read;
+                    } else {
+                        if (!__all_sync(0xffffffffu, mbar_wait(&sh.nfull[half][nz_buf], (nz_par >> nz_buf) & 1u, r.ctl))) { dead = true; break; }
                         // lane = pixel: rows of 128 bytes, their 16-byte chunks permuted by the row number (the box's swizzle)
-                        const uint32_t gg = smem_u32(noise_buf(nz_read)) + 128u * (uint32_t)lane;
+                        const uint32_t gg = smem_u32(noise_buf(half, nz_buf)) + 128u * (uint32_t)prow;
+                        const uint32_t bb = smem_u32(sh.bias_s[warp - 2]) + 4u * (uint32_t)(c0 - half * 128);
                         float sc[32];
 #pragma unroll
                         for (int i = 0; i < 32; i += 4) {
-                            const float4 b4 = __ldg(reinterpret_cast<const float4 *>(bias + c0 + i));
-                            float4 g4;
-                            asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
-                                         : "=f"(g4.x), "=f"(g4.y), "=f"(g4.z), "=f"(g4.w)
-                                         : "r"(gg + 16u * (uint32_t)((i >> 2) ^ (lane & 7))));
+                            const float4 b4 = lds_f4(bb + 4u * (uint32_t)i), g4 = lds_f4(gg + 16u * (uint32_t)((i >> 2) ^ (lane & 7)));
                             sc[i] = (v[i] + b4.x) + g4.x;
                             sc[i + 1] = (v[i + 1] + b4.y) + g4.y;
                             sc[i + 2] = (v[i + 2] + b4.z) + g4.z;
                             sc[i + 3] = (v[i + 3] + b4.w) + g4.w;
                         }
                         __syncwarp();
-                        if (++nz_read == NOISE_BUFS) nz_read = 0;
-                        noise_ask(yt_lo, nyl, ntiles);
+                        if (lane == 0) mbar_arrive(&sh.nempty[half][nz_buf]);
+                        nz_par ^= 1u << nz_buf;
+                        if (++nz_buf == NOISE_BUFS) nz_buf = 0;
                         argmax_chunk32(sc, c0, best, bi);
                     }
                 }
@@ -705,6 +702,11 @@ struct ConvEngine {
             mma_issuer(l, src, ntiles);
         } else if (warp == 10) {
             load_weights(l, ntiles);
+        } else if (warp == 11) {
+            if (head && kind == EPI_CAT && r.nk == JS_NOISE_GUMBEL) {
+                noise_may_come();
+                load_noise(yt_lo, nyl, ntiles);
+            }
         } else {
             epilogue(l, kind, w, flag, parity, zout, yt_lo, nyl, ntiles, src);
         }
@@ -792,8 +794,8 @@ conv_tc_kernel(const __grid_constant__ ConvDev m, const __grid_constant__ RunArg
         for (int s = 0; s < MAX_STAGES; ++s) { mbar_init(&sh.wfull[s], 1); mbar_init(&sh.wempty[s], 1); }
         for (int s = 0; s < MAX_STAGES; ++s) { mbar_init(&sh.afull[s], 1); mbar_init(&sh.aempty[s], 1); }
         for (int a = 0; a < 2; ++a) { mbar_init(&sh.tfull[a], 1); mbar_init(&sh.tempty[a], 8); }
-        for (int w = 0; w < 8; ++w)
-            for (int i = 0; i < NOISE_BUFS; ++i) mbar_init(&sh.nfull[w][i], 1);
+        for (int h = 0; h < 2; ++h)
+            for (int i = 0; i < NOISE_BUFS; ++i) { mbar_init(&sh.nfull[h][i], 1); mbar_init(&sh.nempty[h][i], 4); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async();
     }
@@ -990,10 +992,10 @@ int js_launch_conv_tc(const js_model *mo, const RunArgs &r, cudaStream_t stream)
     CUtensorMap noise;
     std::memset(&noise, 0, sizeof noise);
     if (r.nk == JS_NOISE_GUMBEL && r.noise) {
-        // {class, sub-pixel, pixel}, a box per 32 pixels and 32 classes of one sub-pixel
+        // {class, sub-pixel, pixel}, a box per 128 pixels and 32 classes of one sub-pixel
         const cuuint64_t dims[3] = {256, (cuuint64_t)v.in_ch, (cuuint64_t)r.batch * v.height * v.width};
         const cuuint64_t strides[2] = {1024, (cuuint64_t)v.in_ch * 1024};
-        const cuuint32_t box[3] = {32, 1, 32};
+        const cuuint32_t box[3] = {32, 1, 128};
         if (!encode_nd(&noise, r.noise, 3, dims, strides, box, CU_TENSOR_MAP_DATA_TYPE_FLOAT32)) return (int)cudaErrorInvalidValue;
     }
     void *args[3] = {(void *)&v, (void *)&r, (void *)&noise};
