@@ -626,8 +626,7 @@ struct GenericEngine {
     }
     __device__ bool barrier()
     {
-        // activations stored by threads are read by TMA after the barrier
-        if constexpr (Conf<T, JGS>::TMA) fence_proxy_async();
+        // activations stored by threads are read by TMA after the barrier: the proxy fence is on the reading side
         const bool ok = grid_barrier(r.ctl, epoch, r.spin_limit);
         if constexpr (Conf<T, JGS>::TMA) fence_proxy_async();
         return ok;

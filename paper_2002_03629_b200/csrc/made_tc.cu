@@ -4,7 +4,7 @@
 // masked network is a GEMM  D[128 samples x BN units] = A[128 x K] * W[BN x K]^T
 // on the 5th-generation tensor cores: operands arrive in shared memory by TMA
 // (128-byte swizzle, K-major), one warp issues tcgen05.mma with the
-// fp32 accumulator in tensor memory, and four epilogue warps read it back with
+// fp32 accumulator in tensor memory, and four or eight epilogue warps read it back with
 // tcgen05.ld.  Masked (all-zero) K blocks beyond a tile's last live input are
 // never loaded; adding exact zeros would not change the fp32 sum, so h_t stays
 // the same function whatever is skipped.  The output layer's epilogue is the
@@ -12,8 +12,8 @@
 // threshold or 256-way argmax, compare with the previous iterate, per-sample
 // change flags; logits never reach global memory.
 //
-// Warp roles (192 threads): warp 0 = TMA producer, warp 1 = MMA issuer and TMEM
-// owner, warps 2-5 = epilogue (TMEM lane quadrant = warp index mod 4).
+// Warp roles (192 or 320 threads): warp 0 = TMA producer, warp 1 = MMA issuer and TMEM
+// owner, the others = epilogue (TMEM lane quadrant = warp index mod 4).
 // All waits are bounded; a wait that gives up raises the abort flag, every role
 // drains, TMEM is freed and the kernel returns JS_ERR_TIMEOUT.
 #include <cuda.h>
@@ -116,8 +116,8 @@ struct TcEngine {
 
     __device__ bool barrier()
     {
-        // epilogue stores of this phase must be visible to the TMA reads of the next one
-        fence_proxy_async();
+        // One proxy fence, on the side of the TMA loads that read what threads stored before the barrier.  (One in front too made
+        // every thread wait for its stores a second time.)
         const bool ok = grid_barrier(r.ctl, epoch, r.spin_limit);
         fence_proxy_async();
         if (threadIdx.x == 0) trace(5);
@@ -707,7 +707,8 @@ struct TcEngine {
         uint8_t *nz = nz_row(), *xs = xs_row();
         const float lut0 = sh.lut_s[0], lut1 = sh.lut_s[1];
         // columns [clo, chi) of the tile are sampled; the others keep their symbol
-        const int clo = max(w.plo - n0, 0), chi = min(min(w.phi, m.T) - n0, ncols);
+        // (none of them where the window lies in the other half of the tile)
+        const int clo = max(w.plo - n0, 0), chi = max(clo, min(min(w.phi, m.T) - n0, ncols));
         if (t.bin_bulk) {
             if (!mbar_wait(&sh.nzbar[warp - 2], nzphase, r.ctl)) return false;
             nzphase ^= 1u;
