@@ -14,7 +14,7 @@
 // What bounds it: 16 images of 32 x 32 through eight layers of 128 channels (one tile per SM) take 6.7 us per layer (8.6 with a grid
 // barrier behind each): 1.7 us from a tile's stamps to its first pixels, 2.8 us of K loop (272 KB per tile at the 108 GB/s that an
 // SM takes in), 2.2 us of epilogue, half of which is the fence in front of the stamp.  A head tile takes 2.3 to 3.5 us (7 with
-// the noise read by the threads).  A call of 13 passes: 903 us, 1290 before.
+// the noise read by the threads).  A call of 13 passes: 891 us, 1290 before.
 #include <cuda.h>
 
 #include <cstring>
@@ -60,8 +60,8 @@ struct ConvShared {
     float xbest[2][4][32];    // head: the upper class half's best score and class, by tile parity and quadrant
     int xbi[2][4][32];
     float lut_s[256];         // input encoding table
-    int img[MAX_IMAGES];      // images still iterating
-    int n_img;
+    int img[2][MAX_IMAGES];   // images still iterating, by engine's icur: this pass's and, while it is being looked at, the next one's
+    int n_img[2];
 };
 
 struct ConvEngine {
@@ -104,6 +104,7 @@ struct ConvEngine {
     // phase: 0 producer starts, 1 first operands have landed, 2 last MMA issued, 3 last accumulator
     // complete, 4 epilogues done, 5 grid barrier passed
     int phase_no = 0;
+    int icur = 0;                  // which list of images is this pass's
     int raised_img = -1, raised_phase = -1;      // last (image, phase) this warp reported a change for
     __device__ void trace(int slot) const
     {
@@ -144,42 +145,42 @@ struct ConvEngine {
                 r.ctl->agg_minfirst[0] = r.ctl->agg_minfirst[1] = INT_MAX;
             }
         }
-        for (int i = threadIdx.x; i < r.batch; i += blockDim.x) sh.img[i] = i;
-        if (threadIdx.x == 0) sh.n_img = r.batch;
+        for (int i = threadIdx.x; i < r.batch; i += blockDim.x) sh.img[icur][i] = i;
+        if (threadIdx.x == 0) sh.n_img[icur] = r.batch;
         __syncthreads();
     }
 
     // Images whose iterate did not change are at their fixed point: they drop out of the
     // tile lists.  Every CTA derives the same list from the per-sample flags; rows do not
-    // move, so nothing has to be rebuilt.  Always returns 0 (no remapping).
-    __device__ int compact(int parity)
+    // move, so nothing has to be rebuilt.  The list is made by one warp while another one asks what changed at all (the two
+    // round trips to L2 and a block barrier one after the other cost 1 us per pass): the flags of all images in flight at
+    // once, then a ballot per 32 images.
+    __device__ void look_ahead(int parity)
     {
-        // by one warp: the flags of all images in flight at once (read one after the other they took an L2 round trip each, 7 us
-        // per pass on a batch of 16), then a ballot per 32 images
-        if (warp == 0) {
-            const int n = sh.n_img;
-            int img[MAX_IMAGES / 32];
-            bool keep[MAX_IMAGES / 32];
+        if (warp != 1) return;
+        const int n = sh.n_img[icur];
+        int img[MAX_IMAGES / 32];
+        bool keep[MAX_IMAGES / 32];
 #pragma unroll
-            for (int i = 0; i < MAX_IMAGES / 32; ++i) {
-                const bool in = 32 * i + lane < n;
-                img[i] = in ? sh.img[32 * i + lane] : 0;
-                keep[i] = in && ld_volatile_i32(&r.smp_changed[parity * r.batch + img[i]]) != 0;
-            }
-            __syncwarp();
-            int k = 0;
-#pragma unroll
-            for (int i = 0; i < MAX_IMAGES / 32; ++i) {
-                const unsigned bal = __ballot_sync(0xffffffffu, keep[i]);
-                if (keep[i]) sh.img[k + __popc(bal & ((1u << lane) - 1u))] = img[i];
-                k += __popc(bal);
-            }
-            if (lane == 0) {
-                sh.n_img = k;
-                if (blockIdx.x == 0) { r.ctl->compactions += 1; r.ctl->live = k; }
-            }
+        for (int i = 0; i < MAX_IMAGES / 32; ++i) {
+            const bool in = 32 * i + lane < n;
+            img[i] = in ? sh.img[icur][32 * i + lane] : 0;
+            keep[i] = in && ld_volatile_i32(&r.smp_changed[parity * r.batch + img[i]]) != 0;
         }
-        __syncthreads();
+        int k = 0;
+#pragma unroll
+        for (int i = 0; i < MAX_IMAGES / 32; ++i) {
+            const unsigned bal = __ballot_sync(0xffffffffu, keep[i]);
+            if (keep[i]) sh.img[icur ^ 1][k + __popc(bal & ((1u << lane) - 1u))] = img[i];
+            k += __popc(bal);
+        }
+        if (lane == 0) sh.n_img[icur ^ 1] = k;
+    }
+    // takes the list that look_ahead has made; always returns 0 (no remapping)
+    __device__ int compact(int)
+    {
+        icur ^= 1;
+        if (blockIdx.x == 0 && threadIdx.x == 0) { r.ctl->compactions += 1; r.ctl->live = sh.n_img[icur]; }
         return 0;
     }
 
@@ -270,7 +271,7 @@ struct ConvEngine {
         c = id % per;
         const int t2 = id / per;
         yt = yt_lo + t2 % nyl;
-        n = sh.img[t2 / nyl];
+        n = sh.img[icur][t2 / nyl];
     }
 
     __device__ int kblocks(int l) const
@@ -687,7 +688,7 @@ struct ConvEngine {
         int yt_lo, yt_hi;
         live_rows(head, w, yt_lo, yt_hi);
         const int nyl = yt_hi - yt_lo;
-        const int ntiles = sh.n_img * nyl * (head ? m.in_ch : 1);
+        const int ntiles = sh.n_img[icur] * nyl * (head ? m.in_ch : 1);
         if (threadIdx.x == 0) {
             for (int id = blockIdx.x; id < ntiles; id += gridDim.x) {
                 issued++;
@@ -696,7 +697,7 @@ struct ConvEngine {
             // a layer's packed weights serve every tile: the pass streams them once
             if (blockIdx.x == 0 && ntiles > 0)
                 weight_bytes += 2ull * BK * (unsigned long long)kblocks(l) * (unsigned long long)(head ? 256 * m.in_ch : m.ch);
-            if (blockIdx.x == 0) skipped += (unsigned long long)(r.batch * m.nyt - sh.n_img * nyl) * (head ? m.in_ch : 1);
+            if (blockIdx.x == 0) skipped += (unsigned long long)(r.batch * m.nyt - sh.n_img[icur] * nyl) * (head ? m.in_ch : 1);
         }
         if (ntiles == 0) return;
         phase_no++;

@@ -176,6 +176,7 @@ __device__ DriverResult made_driver(E &e, int T_, const RunArgs &r)
         }
         const int cap = (r.max_iters > 0 && r.max_iters < len) ? r.max_iters : len;
         int any, mf;
+        if (mode == KM_JACOBI && r.compact) e.look_ahead(p);      // for compact() below, beside the next line's round trip
         read_changes(ctl, p, any, mf);
         book_samples(r, p, k, k == cap, mode == KM_GS_JACOBI, mode == KM_JACOBI);
         reset_other_parity(r, p);

@@ -638,6 +638,7 @@ struct GenericEngine {
         else
             init_phase<T>(m, r, src);
     }
+    __device__ void look_ahead(int) {}
     __device__ int compact(int) { return 0; }      // the CUDA-core path keeps the batch as it is
     // One forward pass over the window; then either the logits go to zout (teacher forcing) or positions [w.plo, w.phi) are
     // sampled and committed: in the output tiles themselves where a position has one logit or a location and a log-scale,

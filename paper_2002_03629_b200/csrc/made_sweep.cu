@@ -24,7 +24,7 @@
 // activations then go to F, where the next group's GEMMs find them.  What those GEMMs read of earlier groups (all full K
 // blocks below the group's first unit) does not wait for that: it is loaded and multiplied while the positions are solved.
 //
-// What bounds it: the chain of the positions.  100 samples of a 784-784-784-784 model, one block (4 jobs of 32 rows): 445 us
+// What bounds it: the chain of the positions.  100 samples of a 784-784-784-784 model, one block (8 jobs of 32 rows): 431 us
 // (1117 with thread = row), per group 5.7 us of positions, 2.6 us from the operands of its late K blocks to the sums, 1.6 us to
 // store its activations.  512 samples of a 4096-wide model in 32 blocks (128 jobs of 128 rows): 1281 us for three outer
 // iterations (1613); a sweep is 230 us, of which the base GEMMs of the longest prefixes take 95 and the positions 75.
@@ -707,7 +707,7 @@ struct SweepEngine {
             for (int l = 0; l <= L; ++l)
 #pragma unroll
                 for (int rr = 0; rr < RPW; ++rr) S[l][rr] = active ? lds_f(vat(l, lane, r0 + rr)) : 0.0f;
-            fence_proxy_async();              // the next group's loads overwrite the running sums' memory
+            fence_proxy_async_smem();         // the next group's loads overwrite the running sums' memory
             __syncwarp();
             if (t1 < b && lane == 0) mbar_arrive(&sh.vread);
             const bool last = t0 + ng > hi;              // the block's last position completes nothing that the block reads

@@ -171,6 +171,7 @@ struct TcEngine {
     // is needed to agree on it.  It is adopted only when it frees at least one 128-row tile; then
     // the encoded iterate is rebuilt for the new rows and a grid barrier makes it visible.
     // Returns 1 if rows were remapped, 0 if not, -1 if the barrier gave up.
+    __device__ void look_ahead(int) {}
     __device__ int compact(int parity)
     {
         const int *pc = perm_cur();
