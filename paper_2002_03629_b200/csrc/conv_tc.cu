@@ -100,9 +100,9 @@ struct ConvEngine {
         lane = threadIdx.x & 31;
     }
 
-    // optional device timeline (JS_OPT_TRACE, js_get_trace): first and last CTA, one row of stamps per
-    // phase: 0 producer starts, 1 first operands have landed, 2 last MMA issued, 3 last accumulator
-    // complete, 4 epilogues done, 5 grid barrier passed
+    // optional device timeline (JS_OPT_TRACE, js_get_trace): first and last (or chosen) CTA, one row of stamps per
+    // layer: 0 epilogue warps start, 1 first operands have landed, 2 last MMA issued, 3 last accumulator
+    // complete, 4 epilogues done, 5 grid barrier passed (all layers but a pass's last: the CTA is through with the layer)
     int phase_no = 0;
     int icur = 0;                  // which list of images is this pass's
     int raised_img = -1, raised_phase = -1;      // last (image, phase) this warp reported a change for
@@ -315,7 +315,6 @@ struct ConvEngine {
         const CUtensorMap *ma_new = m.tmAct + l, *ma_old = m.tmActOld + l, *ma_two = (src == SRC_OLD ? m.tmActOld2 : m.tmAct2) + l;
         if (head && w_bytes != 0 && !drained(sh.aempty, a_stages, apar)) { dead = true; return; }
         cut_rings(head);
-        if (lane == 0) trace(0);
         for (int id = blockIdx.x; id < ntiles; id += gridDim.x) {
             int n, yt, c;
             locate(id, nyl, yt_lo, per, n, yt, c);
@@ -549,6 +548,7 @@ struct ConvEngine {
         // second one takes the upper half of the channels or of the 256 classes (the argmax is bound by instruction
         // issue, one warp per scheduler was not enough); behind uniform noise it only hands the accumulator back.
         const int half = (warp - 2) >> 2;
+        if (warp == 4 && lane == 0) trace(0);
         int tile_par = 0;
         const bool split_head = head && kind == EPI_CAT && r.nk == JS_NOISE_GUMBEL;
         bool any_changed = false;
@@ -670,6 +670,7 @@ struct ConvEngine {
         if (split_head && dead)
             for (; id < ntiles; id += gridDim.x) asm volatile("bar.arrive %0, 64;" ::"r"(1 + q) : "memory");
         if (warp == 4 && lane == 0) trace(4);
+        if (warp == 4 && lane == 0) trace(5);            // (a pass's last layer: overwritten behind the grid barrier)
         if (flag) {
             const bool wany = __any_sync(0xffffffffu, any_changed);
             if (wany) {

@@ -24,10 +24,10 @@
 // activations then go to F, where the next group's GEMMs find them.  What those GEMMs read of earlier groups (all full K
 // blocks below the group's first unit) does not wait for that: it is loaded and multiplied while the positions are solved.
 //
-// What bounds it: the chain of the positions.  100 samples of a 784-784-784-784 model, one block (8 jobs of 32 rows): 431 us
+// What bounds it: the chain of the positions.  256 samples of a 784-1024-1024-784 model, one block (8 jobs of 32 rows): 431 us
 // (1117 with thread = row), per group 5.7 us of positions, 2.6 us from the operands of its late K blocks to the sums, 1.6 us to
-// store its activations.  512 samples of a 4096-wide model in 32 blocks (128 jobs of 128 rows): 1281 us for three outer
-// iterations (1613); a sweep is 230 us, of which the base GEMMs of the longest prefixes take 95 and the positions 75.
+// store its activations.  512 samples of a 4096-wide model in 32 blocks (128 jobs of 128 rows): 1245 us for three outer
+// iterations (1613); a sweep is 220 us, of which the base GEMMs of the longest prefixes take 95 and the positions 75.
 //
 // Every value is a fixed function of the iterate: the split into prefix and group depends on the
 // block size and the position alone.  Waits are bounded as in the other tensor-core kernels.
