@@ -12,13 +12,13 @@
  * A Jacobi iteration evaluates the right-hand side for every t at once from the previous iterate; after n
  * iterations the last n states are exact (Proposition 1), all of them after T.
  *
- * Conventions.  Every pointer is a DEVICE pointer to fp32, row-major, owned by the caller; the calls are
- * asynchronous on `stream` (a cudaStream_t; NULL = the default stream) and allocate nothing.  Sequences of
- * a batch are independent (one thread block each).  Limits: 1 <= T <= 128, 1 <= H <= 128 with H a multiple
- * of 4, 1 <= d_in, d_out <= 16, B >= 1.  Return value: 0, RNN_ERR_INVALID (-1) for a null pointer or a size
- * outside the limits (nothing is launched), RNN_ERR_CUDA (-2) if the launch failed (rnn_last_error() names
- * the CUDA error).  Arithmetic: fp32 fused multiply-adds in a fixed order (results are reproducible run to
- * run); exp/log from the fast-math intrinsics are not used.
+ * Conventions.  Every pointer is a DEVICE pointer to fp32, row-major, owned by the caller and aligned like any float
+ * (on 16 bytes it is read and written faster); the calls are asynchronous on `stream` (a cudaStream_t; NULL = the
+ * default stream) and allocate nothing.  The sequences of a batch are independent.  Limits: 1 <= T <= 128,
+ * 1 <= H <= 128 with H a multiple of 4, 1 <= d_in, d_out <= 16, B >= 1.  Return value: 0, RNN_ERR_INVALID (-1) for a
+ * null pointer or a size outside the limits (nothing is launched), RNN_ERR_CUDA (-2) if the launch failed
+ * (rnn_last_error() names the CUDA error).  Arithmetic: fp32 fused multiply-adds in a fixed order (results are
+ * reproducible run to run); exp/log from the fast-math intrinsics are not used.
  */
 #ifndef RNN_BPTT_H
 #define RNN_BPTT_H

@@ -29,6 +29,21 @@ int launch_status()
     return RNN_ERR_CUDA;
 }
 
+// Four neighbouring floats of global memory.  VEC: every pointer of the call lies on 16 bytes (rows do then too, H being a
+// multiple of 4) and they move as one piece; otherwise (views into a larger buffer, say) one by one.
+template <bool VEC>
+__device__ __forceinline__ float4 ldg4(const float *p)
+{
+    if constexpr (VEC) return __ldg(reinterpret_cast<const float4 *>(p));
+    return make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
+}
+template <bool VEC>
+__device__ __forceinline__ void stg4(float *p, float4 v)
+{
+    if constexpr (VEC) { *reinterpret_cast<float4 *>(p) = v; return; }
+    p[0] = v.x; p[1] = v.y; p[2] = v.z; p[3] = v.w;
+}
+
 // ------------------------------------------------------------------ one step of a chain
 // A matrix-vector product with a 128 x 128 matrix in the registers of 128 threads.  Thread (warp w, lane) holds a 4 x 32
 // tile: the four outputs 4 g .. 4 g + 3, g = 8 w + lane % 8, by the inputs k = 16 m + 4 q + e (m < 8, e < 4), q = lane / 8;
@@ -84,7 +99,7 @@ __device__ __forceinline__ float scatter_sum(const float (&v)[4], int lane)
 // 0.57 us; with every warp of the second group doing a quarter of each kind of work in every iteration, 0.8 us.
 // T = 100, H = 128 (B200): batch 1 86 -> 41 us, batch 592 209 -> 140 us.
 // NS sequences per CTA: the weights in registers serve NS independent chains, whose latencies overlap.
-template <int NS>
+template <int NS, bool VEC>
 __global__ void __launch_bounds__(2 * CT, 1)
 rnn_forward_kernel(const float *__restrict__ Wh, const float *__restrict__ Wx, const float *__restrict__ b,
                    const float *__restrict__ Wo, const float *__restrict__ bo, const float *__restrict__ x,
@@ -120,8 +135,7 @@ rnn_forward_kernel(const float *__restrict__ Wh, const float *__restrict__ Wx, c
             const int k = 16 * m + 4 * q;               // H is a multiple of 4
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                const float4 v = (4 * g < H && k < H) ? __ldg(reinterpret_cast<const float4 *>(Wh + (size_t)(4 * g + u) * H + k))
-                                                      : make_float4(0, 0, 0, 0);
+                const float4 v = (4 * g < H && k < H) ? ldg4<VEC>(Wh + (size_t)(4 * g + u) * H + k) : make_float4(0, 0, 0, 0);
                 w.w[u][4 * m] = v.x; w.w[u][4 * m + 1] = v.y; w.w[u][4 * m + 2] = v.z; w.w[u][4 * m + 3] = v.w;
             }
         }
@@ -144,7 +158,7 @@ rnn_forward_kernel(const float *__restrict__ Wh, const float *__restrict__ Wx, c
     } else {
         const int j4 = 4 * lane;                         // this lane's units (H is a multiple of 4)
         const bool on = j4 < H;
-        const float4 b4 = on ? __ldg(reinterpret_cast<const float4 *>(b + j4)) : make_float4(0, 0, 0, 0);
+        const float4 b4 = on ? ldg4<VEC>(b + j4) : make_float4(0, 0, 0, 0);
         float part[NS];
         float4 hv[NS], lv[NS], nv[NS], ev[NS];           // of this warp's step: state, direct gradient, sigmoid as a fraction
 #pragma unroll
@@ -187,7 +201,7 @@ rnn_forward_kernel(const float *__restrict__ Wh, const float *__restrict__ Wx, c
                         fraction(a.y, nv[n].y, ev[n].y);
                         fraction(a.z, nv[n].z, ev[n].z);
                         fraction(a.w, nv[n].w, ev[n].w);
-                        if (on) *reinterpret_cast<float4 *>(h + o) = hv[n];
+                        if (on) stg4<VEC>(h + o, hv[n]);
                     } else if (phase == 1) {
                         lv[n] = make_float4(0, 0, 0, 0);
 #pragma unroll 1
@@ -201,8 +215,8 @@ rnn_forward_kernel(const float *__restrict__ Wh, const float *__restrict__ Wx, c
                             part[n] = fmaf(0.5f * res, res, part[n]);
                         }
                     } else if (on) {
-                        *reinterpret_cast<float4 *>(l + o) = lv[n];
-                        *reinterpret_cast<float4 *>(d + o) = make_float4(nv[n].x / ev[n].x, nv[n].y / ev[n].y, nv[n].z / ev[n].z, nv[n].w / ev[n].w);
+                        stg4<VEC>(l + o, lv[n]);
+                        stg4<VEC>(d + o, make_float4(nv[n].x / ev[n].x, nv[n].y / ev[n].y, nv[n].z / ev[n].z, nv[n].w / ev[n].w));
                     }
                 }
             }
@@ -226,13 +240,20 @@ rnn_forward_kernel(const float *__restrict__ Wh, const float *__restrict__ Wx, c
 // T = 100, H = 128 (B200): batch 1 39 -> 25 us, batch 592 110 -> 64 us.
 constexpr int SC = 16;
 
-__device__ __forceinline__ void copy16_async(float *dst, const float *src, bool in)
+template <bool VEC>
+__device__ __forceinline__ void copy4_async(float *dst, const float *src, bool in)
 {
     const uint32_t a = (uint32_t)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(a), "l"(src), "r"(in ? 16 : 0) : "memory");
+    if constexpr (VEC) {
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(a), "l"(src), "r"(in ? 16 : 0) : "memory");
+    } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(a + 4u * e), "l"(src + e), "r"(in ? 4 : 0) : "memory");
+    }
 }
 
-template <int NS>
+template <int NS, bool VEC>
 __global__ void __launch_bounds__(CT, NS == 1 ? 3 : 2)
 rnn_bptt_sequential_kernel(const float *__restrict__ Wh, const float *__restrict__ l, const float *__restrict__ d,
                            int B, int T, int H, float *__restrict__ s)
@@ -246,7 +267,7 @@ rnn_bptt_sequential_kernel(const float *__restrict__ Wh, const float *__restrict
 #pragma unroll
     for (int m = 0; m < MH / 4; ++m) {
         const int k = 16 * (m >> 2) + 4 * q + (m & 3);
-        const float4 v = (4 * g < H && k < H) ? __ldg(reinterpret_cast<const float4 *>(Wh + (size_t)k * H + 4 * g)) : make_float4(0, 0, 0, 0);
+        const float4 v = (4 * g < H && k < H) ? ldg4<VEC>(Wh + (size_t)k * H + 4 * g) : make_float4(0, 0, 0, 0);
         w.w[0][m] = v.x; w.w[1][m] = v.y; w.w[2][m] = v.z; w.w[3][m] = v.w;
     }
     auto chunk = [&](int n, int buf, int which) { return ring + (((n * 2 + buf) * 2 + which) * SC) * MH; };
@@ -257,8 +278,8 @@ rnn_bptt_sequential_kernel(const float *__restrict__ Wh, const float *__restrict
             for (int n = 0; n < NS; ++n) {
                 const bool in = t >= 0 && c < H && seq0 + n < B;
                 const size_t at = in ? ((size_t)(seq0 + n) * T + t) * H + c : 0;
-                copy16_async(chunk(n, buf, 0) + r * MH + c, l + at, in);
-                copy16_async(chunk(n, buf, 1) + r * MH + c, d + at, in);
+                copy4_async<VEC>(chunk(n, buf, 0) + r * MH + c, l + at, in);
+                copy4_async<VEC>(chunk(n, buf, 1) + r * MH + c, d + at, in);
             }
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
@@ -314,7 +335,7 @@ __device__ __forceinline__ void cluster_barrier()
 }
 __device__ __forceinline__ int vrow(int k, int VS) { return k * VS + (k & ~3); }
 
-template <int FORM, int NT>
+template <int FORM, int NT, bool VEC>
 __global__ void __launch_bounds__(NT, 1)
 rnn_bptt_jacobi_kernel(const float *__restrict__ Wh, const float *__restrict__ l, const float *__restrict__ d,
                        int B, int T, int H, int n_iters, const float *__restrict__ s0, float *__restrict__ s, int csz, int rpc)
@@ -333,7 +354,7 @@ rnn_bptt_jacobi_kernel(const float *__restrict__ Wh, const float *__restrict__ l
     for (int p = tid; p < H * 2 * NG; p += nth) {
         const int k = p / (2 * NG), g = p - k * 2 * NG;
         *reinterpret_cast<float4 *>(W + (size_t)k * MH + (g < NG ? 4 * g : 64 + 4 * (g - NG))) =
-            4 * g < H ? __ldg(reinterpret_cast<const float4 *>(Wh + (size_t)k * H + 4 * g)) : make_float4(0, 0, 0, 0);
+            4 * g < H ? ldg4<VEC>(Wh + (size_t)k * H + 4 * g) : make_float4(0, 0, 0, 0);
     }
     if (n_iters <= 0) {
         for (int n = 0; n < NSQ && seq0 + n < B; ++n)
@@ -368,7 +389,7 @@ rnn_bptt_jacobi_kernel(const float *__restrict__ Wh, const float *__restrict__ l
     }
     auto load4 = [&](const float *src, int r, int hf) {          // l or d of step t0 + r, components 4 (ig + hf NG) ..
         const int i = 4 * (ig + hf * NG);
-        return r < nr && i < H ? __ldg(reinterpret_cast<const float4 *>(src + (size_t)(t0 + r) * H + i)) : make_float4(0, 0, 0, 0);
+        return r < nr && i < H ? ldg4<VEC>(src + (size_t)(t0 + r) * H + i) : make_float4(0, 0, 0, 0);
     };
     float4 lk[2], dk[2];                                 // JAC_SPLIT: l and d of this part's row
     if (FORM == JAC_SPLIT && here)
@@ -391,7 +412,7 @@ rnn_bptt_jacobi_kernel(const float *__restrict__ Wh, const float *__restrict__ l
                 const int i = 4 * (ig + hf * NG);
                 if (i >= H) continue;
                 if (last || t == T - 1 - it)
-                    *reinterpret_cast<float4 *>(sp + (size_t)t * H + i) = make_float4(v[4 * hf], v[4 * hf + 1], v[4 * hf + 2], v[4 * hf + 3]);
+                    stg4<VEC>(sp + (size_t)t * H + i, make_float4(v[4 * hf], v[4 * hf + 1], v[4 * hf + 2], v[4 * hf + 3]));
                 if (last) continue;
                 const float dd[4] = {dv[hf].x, dv[hf].y, dv[hf].z, dv[hf].w};
                 const int row = nxt + vrow(i, VS);
@@ -466,6 +487,7 @@ rnn_bptt_jacobi_kernel(const float *__restrict__ Wh, const float *__restrict__ l
 // the right.  T = 100, H = 128 (B200): batch 1 31 -> 17 us, batch 592 191 -> 79 us (60 MB in, 39 MB out).
 constexpr int GC = 16, GN = 64, GTH = 128;
 
+template <bool VEC>
 __global__ void __launch_bounds__(GTH)
 rnn_param_grads_kernel(const float *__restrict__ s, const float *__restrict__ d, const float *__restrict__ h,
                        const float *__restrict__ x, int T, int H, int d_in, float *__restrict__ dWh,
@@ -487,15 +509,14 @@ rnn_param_grads_kernel(const float *__restrict__ s, const float *__restrict__ d,
             const int t = tc + ty / 4 + 4 * e, i = (tid & 31) * 4;
             const bool in = t < T && i < H;
             const size_t at = base + (size_t)t * H + i;
-            const float4 a = in ? __ldg(reinterpret_cast<const float4 *>(d + at)) : make_float4(0, 0, 0, 0);
-            const float4 b = in ? __ldg(reinterpret_cast<const float4 *>(s + at)) : make_float4(0, 0, 0, 0);
+            const float4 a = in ? ldg4<VEC>(d + at) : make_float4(0, 0, 0, 0);
+            const float4 b = in ? ldg4<VEC>(s + at) : make_float4(0, 0, 0, 0);
             rg[e] = make_float4(a.x * b.x, a.y * b.y, a.z * b.z, a.w * b.w);
         }
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
             const int t = tc + tid / 16 + 8 * e, i = n0 + (tid & 15) * 4;
-            rh[e] = (t >= 1 && t < T && i < H) ? __ldg(reinterpret_cast<const float4 *>(h + base + (size_t)(t - 1) * H + i))
-                                               : make_float4(0, 0, 0, 0);
+            rh[e] = (t >= 1 && t < T && i < H) ? ldg4<VEC>(h + base + (size_t)(t - 1) * H + i) : make_float4(0, 0, 0, 0);
         }
     };
     float acc[8][8], sb = 0.0f, sx[MIO];
@@ -545,8 +566,8 @@ rnn_param_grads_kernel(const float *__restrict__ s, const float *__restrict__ d,
         for (int hf = 0; hf < 2; ++hf) {
             const int i = n0 + 32 * hf + 4 * tx;
             if (i < H)
-                *reinterpret_cast<float4 *>(dWh + ((size_t)seq * H + j) * H + i) =
-                    make_float4(acc[a][4 * hf], acc[a][4 * hf + 1], acc[a][4 * hf + 2], acc[a][4 * hf + 3]);
+                stg4<VEC>(dWh + ((size_t)seq * H + j) * H + i,
+                          make_float4(acc[a][4 * hf], acc[a][4 * hf + 1], acc[a][4 * hf + 2], acc[a][4 * hf + 3]));
         }
     }
     if (extra && tid < H) {
@@ -568,7 +589,7 @@ int seqs_per_cta(int B) { return B <= 3 * 148 ? 1 : 2; }
 template <typename K>
 bool allow_smem(K kernel, size_t bytes, int which)
 {
-    static std::atomic<unsigned long long> done[3];      // bit = device
+    static std::atomic<unsigned long long> done[6];      // bit = device; one word per instance
     int dev = 0;
     if (cudaGetDevice(&dev) == cudaSuccess && dev < 64 && (done[which].load(std::memory_order_relaxed) >> dev & 1ull)) return true;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) {
@@ -577,6 +598,13 @@ bool allow_smem(K kernel, size_t bytes, int which)
     }
     if (dev < 64) done[which].fetch_or(1ull << dev);
     return true;
+}
+
+// do all these pointers lie on 16 bytes?
+template <typename... P>
+bool vectors(const P *...p)
+{
+    return ((... | reinterpret_cast<uintptr_t>(p)) & 15u) == 0;
 }
 
 }  // namespace
@@ -590,9 +618,11 @@ int rnn_forward(const float *Wh, const float *Wx, const float *b, const float *W
     if (!Wh || !Wx || !b || !Wo || !bo || !x || !r || !h || !d || !l || !loss) return RNN_ERR_INVALID;
     if (!sizes_ok(B, T, H) || d_in < 1 || d_in > MIO || d_out < 1 || d_out > MIO) return RNN_ERR_INVALID;
     const int ns = B <= 148 ? 1 : B <= 296 ? 2 : 4;          // sequences per CTA: one CTA per SM
-    auto kernel = ns == 1 ? rnn_forward_kernel<1> : ns == 2 ? rnn_forward_kernel<2> : rnn_forward_kernel<4>;
+    const bool vec = vectors(Wh, b, h, d, l);
+    auto kernel = vec ? (ns == 1 ? rnn_forward_kernel<1, true> : ns == 2 ? rnn_forward_kernel<2, true> : rnn_forward_kernel<4, true>)
+                      : (ns == 1 ? rnn_forward_kernel<1, false> : ns == 2 ? rnn_forward_kernel<2, false> : rnn_forward_kernel<4, false>);
     const size_t smem = (size_t)((d_in + d_out) * (MH + ns * T)) * sizeof(float);
-    if (!allow_smem(kernel, (size_t)(2 * MIO * (MH + 4 * MT)) * sizeof(float), ns / 2)) return RNN_ERR_CUDA;
+    if (!allow_smem(kernel, (size_t)(2 * MIO * (MH + 4 * MT)) * sizeof(float), ns / 2 + (vec ? 0 : 3))) return RNN_ERR_CUDA;
     kernel<<<(B + ns - 1) / ns, 2 * CT, smem, (cudaStream_t)stream>>>(Wh, Wx, b, Wo, bo, x, r, B, T, H, d_in, d_out, h, d, l, loss);
     return launch_status();
 }
@@ -601,9 +631,11 @@ int rnn_bptt_sequential(const float *Wh, const float *l, const float *d, int B, 
 {
     if (!Wh || !l || !d || !s || !sizes_ok(B, T, H)) return RNN_ERR_INVALID;
     const int ns = seqs_per_cta(B);
-    auto kernel = ns == 1 ? rnn_bptt_sequential_kernel<1> : rnn_bptt_sequential_kernel<2>;
+    const bool vec = vectors(Wh, l, d);
+    auto kernel = vec ? (ns == 1 ? rnn_bptt_sequential_kernel<1, true> : rnn_bptt_sequential_kernel<2, true>)
+                      : (ns == 1 ? rnn_bptt_sequential_kernel<1, false> : rnn_bptt_sequential_kernel<2, false>);
     const size_t smem = (size_t)ns * 4 * SC * MH * sizeof(float);
-    if (!allow_smem(kernel, smem, ns == 1 ? 0 : 1)) return RNN_ERR_CUDA;
+    if (!allow_smem(kernel, smem, ns - 1 + (vec ? 0 : 2))) return RNN_ERR_CUDA;
     kernel<<<(B + ns - 1) / ns, CT, smem, (cudaStream_t)stream>>>(Wh, l, d, B, T, H, s);
     return launch_status();
 }
@@ -618,9 +650,11 @@ int rnn_bptt_jacobi(const float *Wh, const float *l, const float *d, int B, int 
     const int rpc = (T + csz - 1) / csz, NG = (H + 7) / 8, VS = (rpc + 3) / 4 * 4;
     const int grp = (((rpc + 3) / 4 + 1) / 2 * 2 * NG + 31) / 32 * 32;       // threads of a sequence's share
     const int form = csz > 1 || (grp <= 128 && B <= 148) ? JAC_SPLIT : B > 148 && grp <= 416 ? JAC_PAIR : JAC_ONE;
-    auto kernel = form == JAC_PAIR ? rnn_bptt_jacobi_kernel<JAC_PAIR, 832>
-                : form == JAC_SPLIT ? rnn_bptt_jacobi_kernel<JAC_SPLIT, 512> : rnn_bptt_jacobi_kernel<JAC_ONE, 512>;
-    if (!allow_smem(kernel, JACOBI_SMEM_MAX, form)) return RNN_ERR_CUDA;
+    const bool vec = vectors(Wh, l, d, s);
+    auto kernel = form == JAC_PAIR ? (vec ? rnn_bptt_jacobi_kernel<JAC_PAIR, 832, true> : rnn_bptt_jacobi_kernel<JAC_PAIR, 832, false>)
+                : form == JAC_SPLIT ? (vec ? rnn_bptt_jacobi_kernel<JAC_SPLIT, 512, true> : rnn_bptt_jacobi_kernel<JAC_SPLIT, 512, false>)
+                                    : (vec ? rnn_bptt_jacobi_kernel<JAC_ONE, 512, true> : rnn_bptt_jacobi_kernel<JAC_ONE, 512, false>);
+    if (!allow_smem(kernel, JACOBI_SMEM_MAX, form + (vec ? 0 : 3))) return RNN_ERR_CUDA;
     const int nsq = form == JAC_PAIR ? 2 : 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)((B + nsq - 1) / nsq * csz));
@@ -641,7 +675,8 @@ int rnn_param_grads(const float *s, const float *d, const float *h, const float 
                     float *dWh, float *dWx, float *db, void *stream)
 {
     if (!s || !d || !h || !x || !dWh || !dWx || !db || !sizes_ok(B, T, H) || d_in < 1 || d_in > MIO) return RNN_ERR_INVALID;
-    rnn_param_grads_kernel<<<dim3(B, (H + GN - 1) / GN), GTH, 0, (cudaStream_t)stream>>>(s, d, h, x, T, H, d_in, dWh, dWx, db);
+    auto kernel = vectors(s, d, h, dWh) ? rnn_param_grads_kernel<true> : rnn_param_grads_kernel<false>;
+    kernel<<<dim3(B, (H + GN - 1) / GN), GTH, 0, (cudaStream_t)stream>>>(s, d, h, x, T, H, d_in, dWh, dWx, db);
     return launch_status();
 }
 
