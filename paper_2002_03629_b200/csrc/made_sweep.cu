@@ -842,8 +842,9 @@ __global__ void jgs_book_kernel(int batch, int k, int at_cap, int *changed, int 
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        *any_out = any;
+        // the host polls this word and returns when it is there: everything the block has written comes before it
         __threadfence_system();
+        *reinterpret_cast<volatile int *>(any_out) = any;
     }
 }
 
