@@ -352,7 +352,7 @@ int run_sweep_sequential(js_model *m, RunArgs &r, cudaStream_t st)
 // per-sample bookkeeping; the host looks at one word per outer iteration.  After k outer iterations
 // the first k blocks are final (proof of Proposition 2): they are not swept again, and the hidden
 // units that depend on them alone are not recomputed.
-int run_jacobi_gs_tc(js_model *m, RunArgs &r, cudaStream_t st)
+int jacobi_gs_outer(js_model *m, RunArgs &r, cudaStream_t st)
 {
     const MadeDev &v = m->made;
     const int T = v.T, B = r.block, M = (T + B - 1) / B;
@@ -415,6 +415,14 @@ int run_jacobi_gs_tc(js_model *m, RunArgs &r, cudaStream_t st)
     m->stats.final_frontier = status == JS_OK ? T : std::min(T, k * B);
     m->stats.status = status;
     return status;
+}
+
+int run_jacobi_gs_tc(js_model *m, RunArgs &r, cudaStream_t st)
+{
+    const int rc = jacobi_gs_outer(m, r, st);
+    // an error may leave launches of this iteration queued that write the caller's buffers and the model's words
+    if (rc < 0) cudaStreamSynchronize(st);
+    return rc;
 }
 
 int run_made(js_model *m, RunArgs &r, cudaStream_t st)

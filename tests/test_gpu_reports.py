@@ -35,3 +35,23 @@ def test_jacobi_gs_counts_are_there_for_another_stream():
         np.testing.assert_array_equal(got_it.cpu().numpy(), want_it)
         np.testing.assert_array_equal(got_x.cpu().numpy(), want_x)
     model.close()
+
+
+def test_jacobi_gs_leaves_nothing_queued_after_an_error():
+    """A wait that gives up ends the call with launches of the same iteration behind it: they are over when it returns."""
+    p, cfg, model, noise = binary_model()
+    out = torch.zeros((cfg.batch, cfg.D), dtype=torch.uint8, device="cuda")
+    it = torch.full((cfg.batch,), -7, dtype=torch.int32, device="cuda")
+    model.set_option(p.JS_OPT_SPIN_LIMIT, 0)
+    for _ in range(3):
+        with pytest.raises(p.JsError) as e:
+            p.jacobi_sample(model, noise, cfg.noise_kind, None, p.JS_JACOBI_GS, 16, 0, out, it)
+        assert e.value.code == p.JS_ERR_TIMEOUT
+        assert torch.cuda.current_stream().query()
+    assert int((it != -7).sum()) == 0
+    model.set_option(p.JS_OPT_SPIN_LIMIT, 1 << 22)
+    assert p.jacobi_sample(model, noise, cfg.noise_kind, None, p.JS_JACOBI_GS, 16, 0, out, it) == 0
+    ref = torch.zeros_like(out)
+    assert p.sequential_sample(model, noise, cfg.noise_kind, ref) == 0
+    assert torch.equal(out, ref) and int(it.min()) >= 1
+    model.close()
