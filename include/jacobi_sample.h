@@ -13,8 +13,16 @@
  *   - Pointers named *_dev are DEVICE pointers owned by the caller; pointers in
  *     the model descriptors are HOST pointers, read during the create call only.
  *   - Calls enqueue their work on `cuda_stream` (a cudaStream_t passed as
- *     void*, NULL = default stream) and synchronise that stream before they
- *     return, so outputs are complete and the return value is final.
+ *     void*, NULL = default stream), after what is queued there, and return
+ *     when it is done: the return value is final, and the outputs are complete
+ *     for whatever the program does next, on any stream.  Where every output
+ *     lies in plain device memory of the current GPU the call learns this from
+ *     a word that its last kernel writes, a moment before the stream itself is
+ *     idle (cudaStreamQuery may still say "not ready"), with the calling thread
+ *     spinning meanwhile.  Outputs in mapped host, managed or another GPU's
+ *     memory, or a device set to cudaDeviceScheduleBlockingSync or ...Yield,
+ *     make it synchronise the stream instead.  Errors that other work raises
+ *     on the stream are reported by whoever next synchronises it.
  *   - Return value: 0 = done and converged; JS_NOT_CONVERGED (1) = max_iters
  *     reached while some sample still changed, outputs hold the last iterate;
  *     negative = error, outputs unspecified.  No exceptions, no exit().

@@ -237,14 +237,42 @@ int prep_args(js_model *m, RunArgs &r, cudaStream_t st)
     return JS_OK;
 }
 
-// Waits for the launch and reads what the kernel reported through mapped host memory.  The kernel writes the
-// status word last, when the outputs are complete and the control block is cleared, so polling it is enough; going
-// through the driver's stream synchronisation instead costs 3.2 us more (launch + wait of an empty kernel on B200:
-// 10.1 us against 6.9 us).  The stream itself is asked now and then, for a launch that ended without reporting.
-int wait_result(js_model *m, cudaStream_t st, JsCtl &h)
+// May the end of a call be read off a word that its kernel writes, or has the stream to be synchronised?  The words come
+// behind the outputs for later work on this GPU, which is all that plain device memory needs.  Outputs that the host or
+// another GPU reaches by itself (mapped host memory, managed memory, a peer's) are only known to be complete when the
+// stream is; and a program that asked the driver to block or to yield while it waits does not want a spinning core.
+// Asked after the launch, so that it costs no time of the call.
+bool may_poll(const RunArgs &r)
 {
+    unsigned flags = 0;
+    int dev = 0;
+    if (cudaGetDeviceFlags(&flags) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess ||
+        (flags & (cudaDeviceScheduleBlockingSync | cudaDeviceScheduleYield))) {
+        cudaGetLastError();
+        return false;
+    }
+    for (const void *p : {(const void *)r.x, (const void *)r.out_iters, (const void *)r.xr, (const void *)r.logits_out}) {
+        if (!p) continue;
+        cudaPointerAttributes a;
+        if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        if (a.type != cudaMemoryTypeDevice || a.device != dev) return false;
+    }
+    return true;
+}
+
+// Waits for the launch and reads what the kernel reported through mapped host memory.  The kernel writes the
+// status word last, when the outputs are complete and the control block is cleared, so polling it is enough (see
+// may_poll); going through the driver's stream synchronisation instead costs 3.2 us more (launch + wait of an empty
+// kernel on B200: 10.1 us against 6.9 us).  The stream itself is asked now and then, for a launch that ended without
+// reporting.
+int wait_result(js_model *m, cudaStream_t st, bool poll, JsCtl &h)
+{
+    if (!poll) CU_TRY(cudaStreamSynchronize(st));
     volatile int *status = &m->h_result->status;
-    for (unsigned i = 1; *status == NOT_REPORTED; ++i) {
+    for (unsigned i = 1; poll && *status == NOT_REPORTED; ++i) {
         if ((i & 0x3fffu) == 0) {
             const cudaError_t e = cudaStreamQuery(st);
             if (e == cudaErrorNotReady) continue;
@@ -264,8 +292,9 @@ int wait_result(js_model *m, cudaStream_t st, JsCtl &h)
 }
 
 // The same for kernels whose clusters report one by one (cluster_report in made_driver.cuh).
-int wait_words(js_model *m, int n, cudaStream_t st, JsCtl &h)
+int wait_words(js_model *m, int n, cudaStream_t st, bool poll, JsCtl &h)
 {
+    if (!poll) CU_TRY(cudaStreamSynchronize(st));
     memset(&h, 0, sizeof h);
     h.frontier = INT_MAX;
     volatile unsigned long long *words = m->h_words;
@@ -335,7 +364,7 @@ int run_sweep_sequential(js_model *m, RunArgs &r, cudaStream_t st)
     const int rl = js_launch_made_sweep(m, r, st);
     if (rl != 0) return launch_failed(rl);
     JsCtl h;
-    if ((rc = wait_result(m, st, h)) != JS_OK) return rc;
+    if ((rc = wait_result(m, st, may_poll(r), h)) != JS_OK) return rc;
     fill_stats(m, h, 0);
     m->stats.iterations = 1;
     m->stats.final_frontier = m->made.T;
@@ -364,6 +393,7 @@ int jacobi_gs_outer(js_model *m, RunArgs &r, cudaStream_t st)
     CU_TRY(cudaMemsetAsync(m->sw_flags, 0, 2 * (size_t)m->rows * sizeof(int), st));
     long long flops = 0;
     int status = JS_OK, k = 0;
+    const bool poll = may_poll(r);
     for (k = 1;; ++k) {
         const int fin_blocks = m->opt_frontier_skip ? k - 1 : 0;          // blocks known final before this iteration
         RunArgs f = r;
@@ -377,7 +407,7 @@ int jacobi_gs_outer(js_model *m, RunArgs &r, cudaStream_t st)
         int rl = js_launch_made_tc(m, f, st);
         if (rl != 0) return launch_failed(rl);
         JsCtl h;
-        if ((rc = wait_result(m, st, h)) != JS_OK) return rc;
+        if ((rc = wait_result(m, st, poll, h)) != JS_OK) return rc;
         if (h.status < 0) { fill_stats(m, h, 0); return h.status; }
         flops += (long long)h.mma_flops;
         RunArgs s2 = r;
@@ -389,12 +419,13 @@ int jacobi_gs_outer(js_model *m, RunArgs &r, cudaStream_t st)
         *m->h_any = -1;
         rl = js_launch_jgs_book(m, r.batch, k, k == cap, r.out_iters, st);
         if (rl != 0) return launch_failed(rl);
-        if ((rc = wait_result(m, st, h)) != JS_OK) return rc;
+        if ((rc = wait_result(m, st, poll, h)) != JS_OK) return rc;
         flops += (long long)h.mma_flops;
         if (h.status < 0) { fill_stats(m, h, 0); return h.status; }
         // the bookkeeping kernel runs after the sweep that has just reported
+        if (!poll) CU_TRY(cudaStreamSynchronize(st));
         volatile int *any_word = m->h_any;
-        for (unsigned i = 1; *any_word < 0; ++i) {
+        for (unsigned i = 1; poll && *any_word < 0; ++i) {
             if ((i & 0x3fffu) == 0 && cudaStreamQuery(st) != cudaErrorNotReady) break;
             cpu_relax();
         }
@@ -441,7 +472,7 @@ int run_made(js_model *m, RunArgs &r, cudaStream_t st)
         const int rl = cluster ? js_launch_made_cluster(m, r, st, &clusters) : js_launch_made_small(m, r, st, &clusters);
         if (rl != 0) return launch_failed(rl);
         JsCtl h;
-        if ((rc = wait_words(m, clusters, st, h)) != JS_OK) return rc;
+        if ((rc = wait_words(m, clusters, st, may_poll(r), h)) != JS_OK) return rc;
         fill_stats(m, h, cluster ? 0 : 1);
         return h.status;
     }
@@ -475,7 +506,7 @@ int run_made(js_model *m, RunArgs &r, cudaStream_t st)
     }
     if (rc_launch != 0) return launch_failed(rc_launch);
     JsCtl h;
-    if ((rc = wait_result(m, st, h)) != JS_OK) return rc;
+    if ((rc = wait_result(m, st, may_poll(r), h)) != JS_OK) return rc;
     fill_stats(m, h, used_path);
     return h.status;
 }

@@ -269,7 +269,7 @@ __device__ __forceinline__ void driver_finish(const RunArgs &r, const DriverResu
 
 // Report of a cluster that solved its samples by itself (kernels without a grid-wide step): one 64-bit word in
 // mapped host memory per cluster, written when the cluster's outputs are complete; the host polls and combines
-// them (js_cluster_word / combine_words in api.cu).  No counter is shared on the device: summing up in the control
+// them (wait_words in api.cu).  No counter is shared on the device: summing up in the control
 // block and copying it out cost 4 us of fences and round trips at the end of a 15 us kernel.
 //   bits 0-1 state (1 done, 2 iteration cap reached, 3 a wait gave up), 2-21 iterations, 22-41 frontier, 42-63 tiles
 __device__ __forceinline__ void cluster_report(unsigned long long *words, int cluster, bool alive, int status,
@@ -279,9 +279,9 @@ __device__ __forceinline__ void cluster_report(unsigned long long *words, int cl
     const unsigned long long w = state | (unsigned long long)min(iterations, 0xfffff) << 2 |
                                  (unsigned long long)min(frontier, 0xfffff) << 22 |
                                  (unsigned long long)min(tiles, 0x3fffffu) << 42;
-    // The cluster's outputs first (its barrier made them visible to this thread).  They lie in device memory, which
-    // the host only reaches through later work on the GPU, so the device-wide fence is the one they need; the
-    // system-wide one costs 3 us here.
+    // The cluster's outputs first (its barrier made them visible to this thread).  Where the host polls this word they lie
+    // in device memory, which it only reaches through later work on the GPU, so the device-wide fence is the one they
+    // need (for other outputs it synchronises the stream, may_poll in api.cu); the system-wide one costs 3 us here.
     __threadfence();
     *reinterpret_cast<volatile unsigned long long *>(words + cluster) = w;
 }
