@@ -168,13 +168,22 @@ made_small_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ Sma
     }
     if (tid < 2) sh.first[tid] = INT_MAX;
     if (tid == 0) sh.tiles = 0u;
-    const bool alive = mbar_wait(&sh.wbar, 0, r.ctl);
+    // A CTA whose weights do not come says so where every CTA of the cluster looks for the first iteration's changes: all of
+    // them leave at the same place then.  (A spin limit of zero: the first look decides, as at the grid barriers.)
+    bool here = mbar_test_wait(&sh.wbar, 0);
+    if (!here && r.spin_limit != 0) here = mbar_wait(&sh.wbar, 0, r.ctl);
+    const bool gave_up = !__syncthreads_and(here);
+    if (gave_up && tid == 0) {
+        atomicExch(&r.ctl->abort, 1);
+        sh.first[1] = -1;
+    }
     if constexpr (CL) cluster_sync();          // every CTA of the cluster has started: its shared memory may be written
     else __syncthreads();
 
     const int cap = (r.max_iters > 0 && r.max_iters < T) ? r.max_iters : T;
     int fin_x = 0, fin_h = 0, lo = 0, k = 0, status = JS_OK;
     unsigned long long tiles = 0;
+    int mf;
     for (;;) {
         ++k;
         const int par = k & 1;
@@ -265,7 +274,8 @@ made_small_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ Sma
         // Every warp reads the flags of all CTAs of the cluster (they are kept until two iterations later, so no
         // further barrier is needed); the first keeps the samples' counts, the second clears the other parity's flags,
         // last read before the barriers of this iteration.
-        int mf = INT_MAX, any = 0;
+        int any = 0;
+        mf = INT_MAX;
         for (int rr = lane; rr < nrow; rr += 32) {
             int ch = 0;
             if constexpr (CL)
@@ -276,7 +286,7 @@ made_small_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ Sma
         }
         if (lane < CS) mf = CL ? ld_peer_i(peer_addr(smem_u32(&sh.first[par]), lane)) : sh.first[par];
         mf = __reduce_min_sync(0xffffffffu, mf);
-        any = __any_sync(0xffffffffu, any != 0);
+        any = __any_sync(0xffffffffu, any != 0 && mf >= 0);
         if (warp == 1) {
             for (int rr = lane; rr < R; rr += 32) sh.chg[par ^ 1][rr] = 0;
             if (lane == 0) sh.first[par ^ 1] = INT_MAX;
@@ -288,20 +298,23 @@ made_small_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ Sma
         if (any && cap < T) status = JS_NOT_CONVERGED;
         break;
     }
+    const bool alive = mf >= 0;
     // results: symbols or states of the own positions; counts by the first CTA of the cluster
-    for (int i = tid; i < own * nrow; i += NTH) {
+    for (int i = tid; alive && i < own * nrow; i += NTH) {
         const int rr = i / own, j = i - rr * own;
         const size_t at = (size_t)(row0 + rr) * T + c + CS * j;
         if constexpr (REAL) r.xr[at] = xs[j * RS + rr];
         else r.x[at] = (uint8_t)xs[j * RS + rr];
     }
-    if (c == 0 && r.out_iters)
+    if (c == 0 && r.out_iters && alive)
         for (int rr = tid; rr < nrow; rr += NTH) r.out_iters[row0 + rr] = sh.count[rr];
     tiles = __reduce_add_sync(0xffffffffu, lane == 0 ? (unsigned)tiles : 0u);
     if (lane == 0) {
         if constexpr (!CL) atomicAdd(&sh.tiles, (unsigned)tiles);
         else atom_peer_add(peer_addr(smem_u32(&sh.tiles), 0), (unsigned)tiles);
     }
+    if (gave_up)
+        for (int i = 0; i < 2000; ++i) __nanosleep(1000);      // weights still on their way land before shared memory goes away
     if constexpr (CL) cluster_sync();          // no CTA leaves while others may still read its flags
     else __syncthreads();
     if (tid == 0 && c == 0) cluster_report(r.words, (int)(blockIdx.x >> csh), alive, status, k, fin_x, sh.tiles);

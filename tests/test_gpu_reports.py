@@ -118,3 +118,26 @@ assert wall > 0.02 and cpu < 0.5 * wall, (cpu, wall)
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     run = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
     assert run.returncode == 0, run.stdout + run.stderr
+
+
+@pytest.mark.parametrize("T,H,batch", [(100, (512, 512), 64), (100, (96,), 8)])
+def test_weights_that_do_not_come_end_the_call(T, H, batch):
+    """Small fp32 models: no wait at all is allowed, so the CTAs' weights (up to 190 KB each) are not there at the first look.
+    Whichever CTA of a cluster gives up, the call says so, and the model works afterwards, also on the kernel with grid barriers."""
+    p, cfg, model, noise = binary_model(T, H, batch, si.PREC_F32)
+    ref = torch.zeros((batch, T), dtype=torch.uint8, device="cuda")
+    assert p.sequential_sample(model, noise, cfg.noise_kind, ref) == 0
+    out = torch.zeros_like(ref)
+    for _ in range(3):
+        model.set_option(p.JS_OPT_SPIN_LIMIT, 0)
+        try:
+            rc = p.jacobi_sample(model, noise, cfg.noise_kind, None, p.JS_JACOBI, 0, 0, out)
+        except p.JsError as e:
+            assert e.code == p.JS_ERR_TIMEOUT
+        else:                                            # (the weights may be there all the same where they are few)
+            assert rc == 0 and len(H) == 1 and torch.equal(out, ref)
+        model.set_option(p.JS_OPT_SPIN_LIMIT, 1 << 22)
+        assert p.jacobi_sample(model, noise, cfg.noise_kind, None, p.JS_GS_JACOBI, 32, 0, out) == 0 and torch.equal(out, ref)
+        out.zero_()
+        assert p.jacobi_sample(model, noise, cfg.noise_kind, None, p.JS_JACOBI, 0, 0, out) == 0 and torch.equal(out, ref)
+    model.close()
