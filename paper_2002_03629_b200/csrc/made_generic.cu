@@ -95,7 +95,9 @@ __device__ __forceinline__ void tma_tile(Smem &s, Ring &rg, int kend, int lr, in
         for (int j = 0; j < NR; ++j) acc[i][j] = 0.0f;
     const uint32_t xa = (uint32_t)(lr & 7) << 4, xb = (uint32_t)(wc & 7) << 4;       // row + 4: the piece's bit 2 flips
     for (int k0 = 0; k0 < kend; k0 += TK) {
-        if (!mbar_wait(&s.full[rg.st], rg.ph, ctl)) { rg.dead = true; return; }
+        // (A thread whose wait gives up goes on with what is there and waits no more: the warp has to stay together here and in
+        // the caller, and the grid barrier behind the layer sees the abort flag.)
+        if (!rg.dead && !mbar_wait(&s.full[rg.st], rg.ph, ctl)) rg.dead = true;
         uint32_t ra = ring_base() + (uint32_t)(rg.st * TMA_STAGE_BYTES), rb = ra + (uint32_t)(TK / BOX_K * BMt * 128 + wc * 128);
         ra += (uint32_t)(lr * 128);
         auto read = [&](int q, float4 (&a)[MR], float4 (&b)[NR]) {      // inputs 4 q .. 4 q + 3 from ra, rb on
@@ -313,8 +315,8 @@ __device__ void gemm_phase(Smem &s, Ring &rg, const MadeDev &m, const RunArgs &r
         else live = (dmax > w.hdeg_lo) && (dmin <= w.hdeg_hi);
         if (!live) { if (threadIdx.x == 0) skipped++; continue; }
         if constexpr (Conf<T, JGS>::TMA) {
-            if (rg.dead) break;
             if (loader) {
+                if (rg.dead) break;
                 tma_tile_load(s, rg, m, l, m.t_kend[l][meta], m0, n0, r.ctl);
                 continue;
             }
@@ -349,7 +351,6 @@ __device__ void gemm_phase(Smem &s, Ring &rg, const MadeDev &m, const RunArgs &r
             }
         if constexpr (Conf<T, JGS>::TMA) {
             tma_tile(s, rg, m.t_kend[l][meta], lr, wc, r.ctl, acc);
-            if (rg.dead) break;
         } else {
             gemm_tile<T, Conf<T, JGS>::STAGES, Conf<T, JGS>::STAGE_F>(Asrc, K, (const T *)m.W[l], K, N, m.t_kend[l][meta], m0, n0, lr, wc, acc);
         }
