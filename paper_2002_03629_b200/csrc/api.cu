@@ -101,8 +101,10 @@ int made_build(js_model *m, const js_made_desc *d)
         const int N = v.n[l + 1], K = v.n[l], nt = (N + JS_GT - 1) / JS_GT;
         std::vector<int> kend(nt), dmin(nt), dmax(nt);
         for (int t = 0; t < nt; ++t) {
+            // (padding units do not count: a tile with some at its end must not read inputs that its real units do not read,
+            // which may be infinite in a model of continuous states)
             int lo = INT32_MAX, hi = 0;
-            for (int i = t * JS_GT; i < std::min(N, (t + 1) * JS_GT); ++i) {
+            for (int i = t * JS_GT; i < std::min({N, wn[l + 1], (t + 1) * JS_GT}); ++i) {
                 lo = std::min(lo, deg[l + 1][i]);
                 hi = std::max(hi, deg[l + 1][i]);
             }

@@ -141,3 +141,31 @@ def test_real_entry_points_reject_symbol_models():
         p.jacobi_sample_real(m, noise, None, p.JS_JACOBI, 0, 0, 0.0, out)
     assert e.value.code == p.JS_ERR_UNSUPPORTED
     m.close()
+
+
+def states_with_one_infinite(T, H, batch, prec, mode, block, at, sign):
+    """(states, states of the same samples in the strict order with finite noise) where position `at` of every sample has
+    infinite noise."""
+    p = pkg()
+    cfg = si.MadeConfig("real_inf", 95, D=T, C=2, H=H, act=si.ACT_RELU, prec=prec, batch=batch, noise_kind=si.NOISE_LOGISTIC, w_var_scale=2.0, b_var=0.05)
+    W, b = si.made_real_weights(cfg)
+    model = p.Model.made(T, 2, list(H), cfg.act, cfg.prec, W, b, np.zeros(2, np.float32), batch)
+    noise = torch.from_numpy(si.draw_noise(cfg)).cuda()
+    seq, x = (torch.full((batch, T), 7.0, device="cuda") for _ in range(2))
+    assert p.sequential_sample_real(model, noise, seq) == 0
+    noise[:, at] = sign * float("inf")
+    p.jacobi_sample_real(model, noise, None, mode, block, 0, 0.0, x)
+    model.close()
+    return x.cpu().numpy(), seq.cpu().numpy()
+
+
+# u = 0 or 1 gives infinite logistic noise: the state is infinite, and what comes before it must not notice.  Nothing reads
+# the last state, so every other one is that of the strict order, to the bit (eps = 0 and T iterations are exact).
+@pytest.mark.parametrize("T,H,batch,prec", [(37, (101,), 3, si.PREC_F32), (37, (101,), 3, si.PREC_BF16), (200, (300, 299), 20, si.PREC_BF16)])
+@pytest.mark.parametrize("mode", ["jacobi", "gs_jacobi"])
+def test_infinite_last_state_with_ragged_widths(T, H, batch, prec, mode):
+    p = pkg()
+    jacobi = mode == "jacobi" and prec == si.PREC_BF16      # (fp32 Jacobi of this size: the small models' kernel, below)
+    x, seq = states_with_one_infinite(T, H, batch, prec, p.JS_JACOBI if jacobi else p.JS_GS_JACOBI, 0 if jacobi else T, T - 1, -1.0)
+    np.testing.assert_array_equal(x[:, :-1], seq[:, :-1])
+    assert np.all(np.isneginf(x[:, -1]))
