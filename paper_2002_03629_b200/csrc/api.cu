@@ -117,6 +117,7 @@ int made_build(js_model *m, const js_made_desc *d)
         if ((rc = dev_upload<int>(m, &v.t_dmin[l], dmin.data(), nt)) != JS_OK) return rc;
         if ((rc = dev_upload<int>(m, &v.t_dmax[l], dmax.data(), nt)) != JS_OK) return rc;
         m->host_deg = deg;
+        m->host_kend[l] = kend;
     }
 
     // weights: upload unmasked fp32, mask and round on the device

@@ -51,6 +51,8 @@ struct MadeDev {
     const float *lut;
     float *logits;                    // scratch [rows][T*C]
     const void *tma_a, *tma_w;        // fp32 models: tensor maps of a[0..L] and W[0..L] (made_generic.cu)
+    const void *tma_cut;              // the same of a[l] up to t_kend[l][tile], layer after layer
+    int cut_off[JS_MAXL + 1];         // where layer l's begin
 };
 
 struct RunArgs {

@@ -104,6 +104,7 @@ struct ConvDev {
 #define JS_MAX_CLUSTERS 4096          // most clusters a call of the cluster kernels may have
 
 struct js_model {
+    std::vector<int> host_kend[JS_MAXL + 1];       // t_kend of the device view
     int kind = 0;                 // 0 masked MLP, 1 masked-conv stack
     int max_batch = 0;
     int rows = 0;                 // max_batch rounded up to a multiple of 128
@@ -151,7 +152,7 @@ int js_small_prepare(js_model *m);
 bool js_small_serves(const js_model *m, const RunArgs &r);
 int js_launch_made_small(const js_model *m, const RunArgs &r, cudaStream_t stream, int *clusters);
 bool js_encode_map_2d(CUtensorMap *out, const void *base, int rows, int cols, int box_rows);
-bool js_encode_map_f32(CUtensorMap *out, const void *base, int rows, int cols, int box_cols, int box_rows);
+bool js_encode_map_f32(CUtensorMap *out, const void *base, int rows, int cols, int box_cols, int box_rows, int row_stride = 0);
 int js_generic_prepare(js_model *m);
 int js_cluster_prepare(js_model *m);
 bool js_cluster_serves(const js_model *m, const RunArgs &r);

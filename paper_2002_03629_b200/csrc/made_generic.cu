@@ -10,6 +10,8 @@
 // iteration (the convergence proofs need that).
 #include <limits.h>
 
+#include <algorithm>
+
 #include "js_common.cuh"
 #include "made_driver.cuh"
 #include "js_model.h"
@@ -68,9 +70,15 @@ __device__ __forceinline__ float4 lds_f4(uint32_t a)
 // behind all those the weight rows likewise, 128 bytes a row, 16-byte pieces permuted by the row number (128-byte swizzle,
 // which keeps the reads of eight rows in different banks).  cp.async, 16 bytes a lane, cost the shared-memory pipe as much
 // as the operand reads (14 wavefronts for 512 bytes).
-__device__ __forceinline__ void tma_tile_load(Smem &s, Ring &rg, const MadeDev &m, int l, int kend, int m0, int n0, JsCtl *ctl)
+__device__ __forceinline__ void tma_tile_load(Smem &s, Ring &rg, const MadeDev &m, int l, int meta, int m0, int n0, JsCtl *ctl)
 {
     const CUtensorMap *ma = (const CUtensorMap *)m.tma_a + l, *mw = (const CUtensorMap *)m.tma_w + l;
+    const int kend = m.t_kend[l][meta];
+    // Inputs from kend on are masked.  Their weights are zeros, but a continuous state may be infinite there (its noise is, or
+    // an iterate on its way), and zero times that is no zero: where a tile ends inside the four inputs that are multiplied at
+    // a time, its last box comes through a map that ends at kend too, and the copy fills the rest with zeros.  (Cutting them
+    // in the product cost 2 to 5 % of it.)
+    const CUtensorMap *mc = (kend & 3) ? (const CUtensorMap *)m.tma_cut + m.cut_off[l] + meta : ma;
     for (int k0 = 0; k0 < kend; k0 += TK) {
         if (!__all_sync(0xffffffffu, mbar_wait(&s.empty[rg.st], rg.ph ^ 1u, ctl))) { rg.dead = true; return; }
         if (elect_one()) {
@@ -78,7 +86,7 @@ __device__ __forceinline__ void tma_tile_load(Smem &s, Ring &rg, const MadeDev &
             const int boxes = min(TK / BOX_K, (kend - k0 + BOX_K - 1) / BOX_K);
             mbar_expect_tx(&s.full[rg.st], (uint32_t)(boxes * (BMt + BNt) * BOX_K * 4));
             for (int h = 0; h < boxes; ++h) {
-                tma_load_2d(base + (uint32_t)(h * BMt * 128), ma, &s.full[rg.st], k0 + h * BOX_K, m0);
+                tma_load_2d(base + (uint32_t)(h * BMt * 128), k0 + (h + 1) * BOX_K >= kend ? mc : ma, &s.full[rg.st], k0 + h * BOX_K, m0);
                 tma_load_2d(base + (uint32_t)(TK / BOX_K * BMt * 128 + h * BNt * 128), mw, &s.full[rg.st], k0 + h * BOX_K, n0);
             }
         }
@@ -317,7 +325,7 @@ __device__ void gemm_phase(Smem &s, Ring &rg, const MadeDev &m, const RunArgs &r
         if constexpr (Conf<T, JGS>::TMA) {
             if (loader) {
                 if (rg.dead) break;
-                tma_tile_load(s, rg, m, l, m.t_kend[l][meta], m0, n0, r.ctl);
+                tma_tile_load(s, rg, m, l, meta, m0, n0, r.ctl);
                 continue;
             }
         }
@@ -727,17 +735,23 @@ static int generic_smem(int prec, bool jgs)
 }
 static int generic_threads(int prec, bool jgs) { return prec == JS_BF16 || jgs ? NTHREADS : Conf<float, false>::THREADS; }
 
-// Tensor maps of an fp32 model's activations and masked weights: boxes of 32 inputs x 16 rows (activations) or 32 rows, 128-byte swizzle.
+// Tensor maps of an fp32 model's activations and masked weights: boxes of 32 inputs x 16 rows (activations) or 32 rows, 128-byte
+// swizzle; and of the activations once more for every 64-wide tile of outputs, with the inputs that it reads.
 int js_generic_prepare(js_model *mo)
 {
     MadeDev &v = mo->made;
-    v.tma_a = v.tma_w = nullptr;
+    v.tma_a = v.tma_w = v.tma_cut = nullptr;
     if (v.prec != JS_F32) return JS_OK;
     std::vector<CUtensorMap> maps(2 * (v.L + 1));
     for (int l = 0; l <= v.L; ++l) {
         if (!js_encode_map_f32(&maps[l], v.a[l], mo->rows, v.n[l], BOX_K, BMt) ||
             !js_encode_map_f32(&maps[v.L + 1 + l], v.W[l], v.n[l + 1], v.n[l], BOX_K, BNt))
             return JS_ERR_CUDA;
+        v.cut_off[l] = (int)maps.size() - 2 * (v.L + 1);
+        for (int kend : mo->host_kend[l]) {
+            maps.emplace_back();
+            if (!js_encode_map_f32(&maps.back(), v.a[l], mo->rows, std::max(kend, 1), BOX_K, BMt, v.n[l])) return JS_ERR_CUDA;
+        }
     }
     void *p = nullptr;
     if (cudaMalloc(&p, maps.size() * sizeof(CUtensorMap)) != cudaSuccess) return JS_ERR_CUDA;
@@ -745,6 +759,7 @@ int js_generic_prepare(js_model *mo)
     if (cudaMemcpy(p, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice) != cudaSuccess) return JS_ERR_CUDA;
     v.tma_a = p;
     v.tma_w = (const CUtensorMap *)p + v.L + 1;
+    v.tma_cut = (const CUtensorMap *)p + 2 * (v.L + 1);
     return JS_OK;
 }
 

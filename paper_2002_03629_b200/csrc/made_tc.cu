@@ -1280,13 +1280,14 @@ bool js_encode_map_2d(CUtensorMap *out, const void *base, int rows, int cols, in
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// 2-D fp32 row-major tensor [rows][cols] (cols a multiple of 4), box = box_cols (32: one 128-byte swizzle row) x box_rows
-bool js_encode_map_f32(CUtensorMap *out, const void *base, int rows, int cols, int box_cols, int box_rows)
+// 2-D fp32 row-major tensor [rows][cols], rows row_stride values apart (a multiple of 4; 0: cols), box = box_cols (32: one
+// 128-byte swizzle row) x box_rows
+bool js_encode_map_f32(CUtensorMap *out, const void *base, int rows, int cols, int box_cols, int box_rows, int row_stride)
 {
     EncodeTiledFn fn = get_encode_fn();
     if (!fn) return false;
     const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-    const cuuint64_t strides[1] = {(cuuint64_t)cols * 4};
+    const cuuint64_t strides[1] = {(cuuint64_t)(row_stride ? row_stride : cols) * 4};
     const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
     const cuuint32_t estr[2] = {1, 1};
     return fn(out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void *>(base), dims, strides, box, estr,

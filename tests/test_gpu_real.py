@@ -169,3 +169,13 @@ def test_infinite_last_state_with_ragged_widths(T, H, batch, prec, mode):
     x, seq = states_with_one_infinite(T, H, batch, prec, p.JS_JACOBI if jacobi else p.JS_GS_JACOBI, 0 if jacobi else T, T - 1, -1.0)
     np.testing.assert_array_equal(x[:, :-1], seq[:, :-1])
     assert np.all(np.isneginf(x[:, -1]))
+
+
+@pytest.mark.parametrize("T,H,batch", [(61, (96,), 5), (62, (96,), 5), (63, (96,), 5), (64, (96,), 5), (65, (64, 64), 5), (126, (256,), 17),
+                                       (258, (640,), 3), (131, (640, 516), 3)])
+def test_infinite_last_state_at_every_remainder(T, H, batch):
+    """The CUDA-core kernel reads inputs in fours and multiplies them in runs of 64: tiles whose inputs end anywhere in them."""
+    p = pkg()
+    x, seq = states_with_one_infinite(T, H, batch, si.PREC_F32, p.JS_GS_JACOBI, T, T - 1, 1.0)
+    np.testing.assert_array_equal(x[:, :-1], seq[:, :-1])
+    assert np.all(np.isposinf(x[:, -1]))
