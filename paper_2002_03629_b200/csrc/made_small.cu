@@ -192,7 +192,7 @@ made_small_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ Sma
             const bool out = l == L;
             const int K = m.n[l], nc = s.nc[l], ncs = s.ncs[l];
             const float *W = sm + s.w_off[l], *bias = sm + s.b_off[l];
-            const int *deg = reinterpret_cast<const int *>(sm + s.d_off[l]);
+            const uint32_t *deg = reinterpret_cast<const uint32_t *>(sm + s.d_off[l]);      // degree, inputs << 16
             const float *A = sm + lo_.a[l];
             // a warp's work: 32 own outputs of one group of RG samples
             const int nblk = (nc + 31) / 32, nrg = RS / RG;
@@ -201,28 +201,47 @@ made_small_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ Sma
                 if (rg >= nrg) break;
                 const int ib = blk * 32, i = ib + lane;
                 const bool mine = i < nc;
-                const int ii = min(i, nc - 1), dg = deg[ii];
+                const int ii = min(i, nc - 1), dg = (int)(deg[ii] & 0xffffu);
                 // live: hidden units of degree > hlo, output positions (degree - 1) >= plo
                 const bool live = mine && (out ? dg > plo : dg > hlo);
                 if (!__any_sync(0xffffffffu, live)) continue;
                 tiles++;
                 // inputs beyond the largest degree of the warp's units are masked: exact zeros
-                int kend = min(K, s.kend[l][min(ib / 32, SMALL_KENDS - 1)]);
+                const int kend = min(K, s.kend[l][min(ib / 32, SMALL_KENDS - 1)]);
+                // Inputs up to the unit's own last live one.  The warp's units lie CS apart, so the warp reads far beyond it for
+                // some; a continuous state may be infinite there (its noise is, or an iterate on its way), and a zero weight
+                // does not make that a zero.
+                const int kl = REAL ? (int)(deg[ii] >> 16) : 0;
+                const int kall = REAL ? (int)__reduce_min_sync(0xffffffffu, (unsigned)kl) : 0;
                 float acc[RG];
 #pragma unroll
                 for (int q = 0; q < RG; ++q) acc[q] = 0.0f;
                 // KS steps at a time: their loads in flight together, then the multiply-adds in order
                 const float *w = W + ii, *a = A + rg * RG;
-                for (int k0 = 0; k0 < kend; k0 += KS) {
-                    float wv[KS], av[KS][RG];
+                int k0 = 0;
+                if (RG > 1 || !REAL)
+                    for (; k0 < (REAL ? min(kend, kall / KS * KS) : kend); k0 += KS) {
+                        float wv[KS], av[KS][RG];
 #pragma unroll
-                    for (int q = 0; q < KS; ++q) wv[q] = w[(k0 + q) * ncs];
-                    load_rows<RG>(a + k0 * RS, RS, av);
+                        for (int q = 0; q < KS; ++q) wv[q] = w[(k0 + q) * ncs];
+                        load_rows<RG>(a + k0 * RS, RS, av);
 #pragma unroll
-                    for (int kk = 0; kk < KS; ++kk)
+                        for (int kk = 0; kk < KS; ++kk)
 #pragma unroll
-                        for (int q = 0; q < RG; ++q) acc[q] = fmaf(av[kk][q], wv[kk], acc[q]);
-                }
+                            for (int q = 0; q < RG; ++q) acc[q] = fmaf(av[kk][q], wv[kk], acc[q]);
+                    }
+                if constexpr (REAL)
+                    for (; k0 < kend; k0 += KS) {
+                        float wv[KS], av[KS][RG];
+#pragma unroll
+                        for (int q = 0; q < KS; ++q) wv[q] = w[(k0 + q) * ncs];
+                        load_rows<RG>(a + k0 * RS, RS, av);
+#pragma unroll
+                        for (int kk = 0; kk < KS; ++kk)
+#pragma unroll
+                            for (int q = 0; q < RG; ++q)
+                                if (k0 + kk < kl) acc[q] = fmaf(av[kk][q], wv[kk], acc[q]);
+                    }
                 const float bv = bias[ii];
 #pragma unroll
                 for (int q = 0; q < RG; ++q) {
@@ -338,8 +357,17 @@ __global__ void pack_small_weights(const MadeDev m, const SmallDev s, float *pac
         }
         for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nc; i += gridDim.x * blockDim.x) {
             dst[s.b_off[l] + i] = i < mine ? m.bias[l][unit(i)] : 0.0f;
-            // an output beyond the CTA's own ones is never live
-            reinterpret_cast<int *>(dst + s.d_off[l])[i] = i < mine ? m.deg[l + 1][unit(i)] : INT_MIN;
+            // degree and last live input (continuous states), 16 bits each: weights for more inputs do not fit a CTA.  An output
+            // beyond the CTA's own ones is never live and limits nobody.
+            uint32_t v = 0xffffu << 16;
+            if (i < mine) {
+                const int dg = m.deg[l + 1][unit(i)];
+                int ke = K;
+                if (C == 2)
+                    while (ke > 0 && !(l == m.L ? m.deg[l][ke - 1] < dg : m.deg[l][ke - 1] <= dg)) --ke;
+                v = (uint32_t)dg | (uint32_t)ke << 16;
+            }
+            reinterpret_cast<uint32_t *>(dst + s.d_off[l])[i] = v;
         }
     }
 }
@@ -401,6 +429,7 @@ int js_small_prepare(js_model *mo)
             s.d_off[l] = at; at += s.nc[l];
         }
         s.pack_floats = (at + 3) / 4 * 4;
+        static_assert(190 * 1024 / 4 < 0x10000, "degrees and inputs in 16 bits");
         if (small_layout(v, s, 1).total * 4 > SMEM_MAX || s.pack_floats * 4 > 190 * 1024) continue;
         // last live input of every block of 32 own outputs, over all CTAs of the cluster
         for (int l = 0; l <= v.L; ++l) {

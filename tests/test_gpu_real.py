@@ -179,3 +179,14 @@ def test_infinite_last_state_at_every_remainder(T, H, batch):
     x, seq = states_with_one_infinite(T, H, batch, si.PREC_F32, p.JS_GS_JACOBI, T, T - 1, 1.0)
     np.testing.assert_array_equal(x[:, :-1], seq[:, :-1])
     assert np.all(np.isposinf(x[:, -1]))
+
+
+@pytest.mark.parametrize("T,H,batch", [(16, (33,), 1), (48, (96,), 2), (100, (200, 150), 30), (130, (385,), 70)])
+@pytest.mark.parametrize("where", [0.0, 0.5, 1.0])
+def test_infinite_state_in_a_small_model(T, H, batch, where):
+    """The small models' kernel stops at every unit's own last input: nothing before an infinite state notices it."""
+    p = pkg()
+    at = int(where * (T - 1))
+    x, seq = states_with_one_infinite(T, H, batch, si.PREC_F32, p.JS_JACOBI, 0, at, 1.0)
+    np.testing.assert_array_equal(x[:, :at], seq[:, :at])
+    assert np.all(np.isposinf(x[:, at]))
