@@ -10,6 +10,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cstdio>
 
@@ -89,6 +90,11 @@ __device__ __forceinline__ float scatter_sum(const float (&v)[4], int lane)
     return (b0 ? k1 : k0) + __shfl_xor_sync(0xffffffffu, b0 ? k0 : k1, 8);
 }
 
+template <int N>
+struct Count {
+    static constexpr int value = N;
+};
+
 // ------------------------------------------------------------------ forward
 // Two groups of 128 threads.  The first carries the chain and nothing else: product, softplus, new state (0.33 us per
 // step).  The second follows it with what does not feed back.  Its four warps take the steps in turn, lane = four units,
@@ -99,7 +105,7 @@ __device__ __forceinline__ float scatter_sum(const float (&v)[4], int lane)
 // 0.57 us; with every warp of the second group doing a quarter of each kind of work in every iteration, 0.8 us.
 // T = 100, H = 128 (B200): batch 1 86 -> 41 us, batch 592 209 -> 140 us.
 // NS sequences per CTA: the weights in registers serve NS independent chains, whose latencies overlap.
-template <int NS, bool VEC>
+template <int NS, bool VEC, bool MANY>
 __global__ void __launch_bounds__(2 * CT, 1)
 rnn_forward_kernel(const float *__restrict__ Wh, const float *__restrict__ Wx, const float *__restrict__ b,
                    const float *__restrict__ Wo, const float *__restrict__ bo, const float *__restrict__ x,
@@ -167,14 +173,45 @@ rnn_forward_kernel(const float *__restrict__ Wh, const float *__restrict__ Wx, c
             return make_float4(fmaf(w.x, x, a.x), fmaf(w.y, x, a.y), fmaf(w.z, x, a.z), fmaf(w.w, x, a.w));
         };
         auto input_part = [&](int t) {
+            float4 a[NS];
 #pragma unroll
-            for (int n = 0; n < NS; ++n) {
-                float4 a = b4;
-#pragma unroll 1
-                for (int c = 0; c < d_in; ++c)
-                    a = fma4(xs[(n * T + t) * d_in + c], *reinterpret_cast<const float4 *>(wxs + c * MH + j4), a);
-                *reinterpret_cast<float4 *>(&xin[t & 1][n][j4]) = a;
+            for (int n = 0; n < NS; ++n) a[n] = b4;
+#pragma unroll MANY ? 4 : 1
+            for (int c = 0; c < d_in; ++c) {
+                const float4 wv = *reinterpret_cast<const float4 *>(wxs + c * MH + j4);
+#pragma unroll
+                for (int n = 0; n < NS; ++n) a[n] = fma4(xs[(n * T + t) * d_in + c], wv, a[n]);
             }
+#pragma unroll
+            for (int n = 0; n < NS; ++n) *reinterpret_cast<float4 *>(&xin[t & 1][n][j4]) = a[n];
+        };
+        // Outputs c .. c + G - 1 of step t for all sequences: their sums over the units go through the shuffles side by side
+        // (a shuffle's latency is 25 cycles and a sum takes five, one after the other).
+        auto outputs = [&](auto g_, int t, int c) {
+            constexpr int G = decltype(g_)::value;
+            float4 wv[G];
+            float y[NS][G];
+#pragma unroll
+            for (int g = 0; g < G; ++g) {
+                wv[g] = *reinterpret_cast<const float4 *>(wos + (c + g) * MH + j4);
+#pragma unroll
+                for (int n = 0; n < NS; ++n)
+                    y[n][g] = fmaf(wv[g].w, hv[n].w, fmaf(wv[g].z, hv[n].z, fmaf(wv[g].y, hv[n].y, wv[g].x * hv[n].x)));
+            }
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1)
+#pragma unroll
+                for (int n = 0; n < NS; ++n)
+#pragma unroll
+                    for (int g = 0; g < G; ++g) y[n][g] += __shfl_xor_sync(0xffffffffu, y[n][g], off);
+#pragma unroll
+            for (int g = 0; g < G; ++g)
+#pragma unroll
+                for (int n = 0; n < NS; ++n) {
+                    const float res = y[n][g] + bos[c + g] - rs[(n * T + t) * d_out + c + g];
+                    lv[n] = fma4(res, wv[g], lv[n]);
+                    part[n] = fmaf(0.5f * res, res, part[n]);
+                }
         };
         // derivative of softplus from the pre-activation: the exponential's argument is never positive
         auto fraction = [](float a, float &num, float &den) {
@@ -190,34 +227,39 @@ rnn_forward_kernel(const float *__restrict__ Wh, const float *__restrict__ Wx, c
             if (phase == 3) {
                 if (it + 1 < T) input_part(it + 1);
             } else if (t >= 0 && t < T) {
+                const size_t o = ((size_t)seq0 * T + t) * H + j4, next = (size_t)T * H;
+                if (phase == 0) {
 #pragma unroll
-                for (int n = 0; n < NS; ++n) {
-                    if (n >= ns) break;
-                    const size_t o = ((size_t)(seq0 + n) * T + t) * H + j4;
-                    if (phase == 0) {
+                    for (int n = 0; n < NS; ++n) {
                         hv[n] = *reinterpret_cast<const float4 *>(&hs[it & 1][n][j4]);
                         const float4 a = *reinterpret_cast<const float4 *>(&as[t & 1][n][j4]);
                         fraction(a.x, nv[n].x, ev[n].x);
                         fraction(a.y, nv[n].y, ev[n].y);
                         fraction(a.z, nv[n].z, ev[n].z);
                         fraction(a.w, nv[n].w, ev[n].w);
-                        if (on) stg4<VEC>(h + o, hv[n]);
-                    } else if (phase == 1) {
-                        lv[n] = make_float4(0, 0, 0, 0);
-#pragma unroll 1
-                        for (int c = 0; c < d_out; ++c) {
-                            const float4 wv = *reinterpret_cast<const float4 *>(wos + c * MH + j4);
-                            float y = fmaf(wv.w, hv[n].w, fmaf(wv.z, hv[n].z, fmaf(wv.y, hv[n].y, wv.x * hv[n].x)));
-#pragma unroll
-                            for (int off = 16; off > 0; off >>= 1) y += __shfl_xor_sync(0xffffffffu, y, off);
-                            const float res = y + bos[c] - rs[(n * T + t) * d_out + c];
-                            lv[n] = fma4(res, wv, lv[n]);
-                            part[n] = fmaf(0.5f * res, res, part[n]);
-                        }
-                    } else if (on) {
-                        stg4<VEC>(l + o, lv[n]);
-                        stg4<VEC>(d + o, make_float4(nv[n].x / ev[n].x, nv[n].y / ev[n].y, nv[n].z / ev[n].z, nv[n].w / ev[n].w));
+                        if (on && n < ns) stg4<VEC>(h + o + n * next, hv[n]);
                     }
+                } else if (phase == 1) {
+                    constexpr int GM = NS <= 2 ? 4 : 2;          // sums side by side: six to eight, four for one sequence
+#pragma unroll
+                    for (int n = 0; n < NS; ++n) lv[n] = make_float4(0, 0, 0, 0);
+                    int c = 0;
+                    if constexpr (MANY) {
+#pragma unroll 1
+                        for (; c + GM <= d_out; c += GM) outputs(Count<GM>(), t, c);
+                        if (GM == 4 && c + 2 <= d_out) { outputs(Count<2>(), t, c); c += 2; }
+                        if (c < d_out) outputs(Count<1>(), t, c);
+                    } else {
+#pragma unroll 1
+                        for (; c < d_out; ++c) outputs(Count<1>(), t, c);
+                    }
+                } else if (on) {
+#pragma unroll
+                    for (int n = 0; n < NS; ++n)
+                        if (n < ns) {
+                            stg4<VEC>(l + o + n * next, lv[n]);
+                            stg4<VEC>(d + o + n * next, make_float4(nv[n].x / ev[n].x, nv[n].y / ev[n].y, nv[n].z / ev[n].z, nv[n].w / ev[n].w));
+                        }
                 }
             }
             __syncthreads();
@@ -582,14 +624,28 @@ bool sizes_ok(int B, int T, int H) { return B >= 1 && T >= 1 && T <= MT && H >= 
 
 constexpr size_t JACOBI_SMEM_MAX = (size_t)(2 * MH * (MT + 1) + MH * MH) * sizeof(float);
 
+int sm_count()
+{
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) return 148;
+    return sms;
+}
+
+template <bool VEC>
+auto forward_kernel_of(int ns, bool many)
+{
+    return ns == 1 ? (many ? rnn_forward_kernel<1, VEC, true> : rnn_forward_kernel<1, VEC, false>)
+         : ns == 2 ? rnn_forward_kernel<2, VEC, true> : ns == 3 ? rnn_forward_kernel<3, VEC, true> : rnn_forward_kernel<4, VEC, true>;
+}
+
 // one sequence per CTA until three of them per SM are not enough (the most its registers allow)
-int seqs_per_cta(int B) { return B <= 3 * 148 ? 1 : 2; }
+int seqs_per_cta(int B) { return B <= 3 * sm_count() ? 1 : 2; }
 
 // A kernel's dynamic shared memory limit, raised once per device (the attribute call costs as much as a launch).
 template <typename K>
 bool allow_smem(K kernel, size_t bytes, int which)
 {
-    static std::atomic<unsigned long long> done[6];      // bit = device; one word per instance
+    static std::atomic<unsigned long long> done[10];      // bit = device; one word per instance
     int dev = 0;
     if (cudaGetDevice(&dev) == cudaSuccess && dev < 64 && (done[which].load(std::memory_order_relaxed) >> dev & 1ull)) return true;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) {
@@ -617,12 +673,12 @@ int rnn_forward(const float *Wh, const float *Wx, const float *b, const float *W
 {
     if (!Wh || !Wx || !b || !Wo || !bo || !x || !r || !h || !d || !l || !loss) return RNN_ERR_INVALID;
     if (!sizes_ok(B, T, H) || d_in < 1 || d_in > MIO || d_out < 1 || d_out > MIO) return RNN_ERR_INVALID;
-    const int ns = B <= 148 ? 1 : B <= 296 ? 2 : 4;          // sequences per CTA: one CTA per SM
+    const int sms = sm_count(), ns = std::min(4, (B + sms - 1) / sms);          // sequences per CTA: one CTA per SM, up to four
+    const bool many = d_out > 1 || d_in > 4;
     const bool vec = vectors(Wh, b, h, d, l);
-    auto kernel = vec ? (ns == 1 ? rnn_forward_kernel<1, true> : ns == 2 ? rnn_forward_kernel<2, true> : rnn_forward_kernel<4, true>)
-                      : (ns == 1 ? rnn_forward_kernel<1, false> : ns == 2 ? rnn_forward_kernel<2, false> : rnn_forward_kernel<4, false>);
+    auto kernel = vec ? forward_kernel_of<true>(ns, many) : forward_kernel_of<false>(ns, many);
     const size_t smem = (size_t)((d_in + d_out) * (MH + ns * T)) * sizeof(float);
-    if (!allow_smem(kernel, (size_t)(2 * MIO * (MH + 4 * MT)) * sizeof(float), ns / 2 + (vec ? 0 : 3))) return RNN_ERR_CUDA;
+    if (!allow_smem(kernel, (size_t)(2 * MIO * (MH + 4 * MT)) * sizeof(float), (ns == 1 && !many ? 0 : ns) + (vec ? 0 : 5))) return RNN_ERR_CUDA;
     kernel<<<(B + ns - 1) / ns, 2 * CT, smem, (cudaStream_t)stream>>>(Wh, Wx, b, Wo, bo, x, r, B, T, H, d_in, d_out, h, d, l, loss);
     return launch_status();
 }

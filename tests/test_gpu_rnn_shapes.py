@@ -49,3 +49,20 @@ def test_shapes(T, H, d_in, d_out, B):
         close(dWh[i], g[0], f"dWh[{i}]")
         close(dWx[i], g[1], f"dWx[{i}]")
         close(db[i], g[2], f"db[{i}]")
+
+
+# one to four sequences per CTA, with outputs and inputs whose sums go one, two or four at a time, and what is left of them
+@pytest.mark.parametrize("d_in,d_out,B", [(1, 1, 3), (5, 1, 3), (4, 2, 3), (2, 3, 2), (3, 7, 150), (1, 4, 299), (6, 5, 445), (16, 16, 593)])
+def test_forward_with_many_outputs(d_in, d_out, B):
+    import paper_2002_03629_b200.rnn as rnn
+    cfg = si.RnnConfig("shape", 22, T=9, H=20, d_in=d_in, d_out=d_out, batch=B)
+    Wh, Wx, b, Wo, bo = si.rnn_weights(cfg)
+    rng = np.random.default_rng(B)
+    b, bo = (rng.normal(0, 0.1, v.shape).astype(np.float32) for v in (b, bo))
+    x, r = rng.normal(size=(B, 9, d_in)).astype(np.float32), rng.normal(size=(B, 9, d_out)).astype(np.float32)
+    h, d, l, loss = rnn.rnn_forward(*dev(Wh, Wx, b, Wo, bo, x, r))
+    for i in sorted({0, 1, B // 2, B - 2, B - 1}):
+        want = ro.forward(Wh, Wx, b, Wo, bo, x[i], r[i])
+        for name, got in (("h", h), ("d", d), ("l", l)):
+            close(got[i], want[name], f"{name}[{i}]")
+        close(loss[i], np.float64(want["loss"]), f"loss[{i}]")
