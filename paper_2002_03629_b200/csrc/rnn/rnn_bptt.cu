@@ -702,10 +702,15 @@ int rnn_bptt_jacobi(const float *Wh, const float *l, const float *d, int B, int 
     if (!Wh || !l || !d || !s || !sizes_ok(B, T, H) || n_iters < 0) return RNN_ERR_INVALID;
     // CTAs per sequence: 15 clusters of 8 or 33 of 4 fit the GPU at a time, and two rounds of 4 still beat whole sequences
     // on single CTAs; shares of fewer than eight steps would be mostly barriers
+    const int sms = sm_count();
     int csz = B <= 15 && T >= 64 ? 8 : B <= 66 && T >= 32 ? 4 : 1;
     const int rpc = (T + csz - 1) / csz, NG = (H + 7) / 8, VS = (rpc + 3) / 4 * 4;
     const int grp = (((rpc + 3) / 4 + 1) / 2 * 2 * NG + 31) / 32 * 32;       // threads of a sequence's share
-    const int form = csz > 1 || (grp <= 128 && B <= 148) ? JAC_SPLIT : B > 148 && grp <= 416 ? JAC_PAIR : JAC_ONE;
+    // Pairs where an even number of rounds of one sequence per SM would be needed: a round of pairs takes 1.9 times as long
+    // (T = 100, H = 128, 20 iterations: 450 and 236 us), so that for 300 sequences two of them, 904 us, lose to three rounds
+    // of one, 705 us, and for 592 two, 900 us, win over four, 945 us.
+    const int rounds = (B + sms - 1) / sms;
+    const int form = csz > 1 || (grp <= 128 && rounds == 1) ? JAC_SPLIT : rounds % 2 == 0 && grp <= 416 ? JAC_PAIR : JAC_ONE;
     const bool vec = vectors(Wh, l, d, s);
     auto kernel = form == JAC_PAIR ? (vec ? rnn_bptt_jacobi_kernel<JAC_PAIR, 832, true> : rnn_bptt_jacobi_kernel<JAC_PAIR, 832, false>)
                 : form == JAC_SPLIT ? (vec ? rnn_bptt_jacobi_kernel<JAC_SPLIT, 512, true> : rnn_bptt_jacobi_kernel<JAC_SPLIT, 512, false>)

@@ -66,3 +66,16 @@ def test_forward_with_many_outputs(d_in, d_out, B):
         for name, got in (("h", h), ("d", d), ("l", l)):
             close(got[i], want[name], f"{name}[{i}]")
         close(loss[i], np.float64(want["loss"]), f"loss[{i}]")
+
+
+# rounds of sequences per SM: three (one per CTA), two and four (pairs), the last of them ragged
+@pytest.mark.parametrize("T,H,B", [(37, 64, 297), (37, 64, 296), (101, 128, 443), (101, 128, 445)])
+def test_rounds_of_sequences(T, H, B):
+    import paper_2002_03629_b200.rnn as rnn
+    g = torch.Generator("cuda").manual_seed(B)
+    Wh = torch.randn((H, H), generator=g, device="cuda") * 0.1
+    l, d = torch.randn((B, T, H), generator=g, device="cuda"), torch.rand((B, T, H), generator=g, device="cuda")
+    a = rnn.rnn_bptt_jacobi(Wh, l, d, 6)
+    ln, dn, W = l.cpu().double().numpy(), d.cpu().double().numpy(), Wh.cpu().numpy()
+    for i in sorted({0, 147, 148, B // 2, B - 2, B - 1}):
+        close(a[i], ro.backprop_jacobi(W, ln[i], dn[i], 6), f"jacobi[{i}]")
