@@ -499,11 +499,12 @@ int run_made(js_model *m, RunArgs &r, cudaStream_t st)
             snprintf(g_cuda_err, sizeof g_cuda_err, "occupancy query failed");
             return JS_ERR_CUDA;
         }
-        // smallest tiles of the products (16 x 32); the phases that take a warp or a thread per element
+        // tiles of the products (16 x 32, in Jacobi-GS 16 x 64); the phases that take a warp or a thread per element
+        const int width = jgs ? 64 : 32, threads = jgs ? 256 : 128;
         long long tiles = 1;
         for (int l = 0; l <= v.L; ++l)
-            tiles = std::max<long long>(tiles, (long long)((r.batch + 15) / 16) * ((v.n[l + 1] + 31) / 32));
-        const long long elems = ((long long)r.batch * v.T * (v.C > 1 ? 32 : 1) + 127) / 128;
+            tiles = std::max<long long>(tiles, (long long)((r.batch + 15) / 16) * ((v.n[l + 1] + width - 1) / width));
+        const long long elems = ((long long)r.batch * v.T * (v.C > 1 ? 32 : 1) + threads - 1) / threads;
         const int grid = (int)std::min<long long>(most, std::max(tiles, elems));
         rc_launch = js_launch_made_generic(v, r, std::max(grid, 1), st);
     }

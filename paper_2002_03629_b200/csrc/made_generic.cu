@@ -27,13 +27,17 @@ constexpr int ROWF = KC + 4;   // row stride in shared memory: the 16-byte piece
 // 784 - 1024 - 1024 - 1568, five passes: 298 us, with 16 x 64 tiles 343, with 32 x 64 552; 16 samples: 228, 309, 488.
 constexpr int MR = 2, NR = 2, BMt = 8 * MR, BNt = 16 * NR;
 // Instances: fp32 products (operands by TMA: a fifth warp loads), bf16 products (operands converted on their way through
-// registers), and for either type Jacobi-GS's, whose micro-steps are a warp per inner product and want many warps per SM.
+// registers), and for either type Jacobi-GS's, whose micro-steps are a warp per inner product and want many warps per SM
+// but few CTAs at the thousands of grid barriers between them: 256 threads, tiles of 16 x 64 (with 128 threads a call of
+// T = 784, H = 1024 x 2 in blocks of 98 took 7.56 ms for one sample, 6.41 so; T = 16, H = 64, batch 8 150 us, 133 so).
 template <typename T, bool JGS> struct Conf {
     static constexpr bool TMA = sizeof(T) == 4 && !JGS;
-    static constexpr int STAGES = JGS ? 2 : 4, STAGE_F = (BMt + BNt) * (TMA ? 2 * KC : ROWF), CTAS = JGS ? 6 : 2;
+    static constexpr int NTH = JGS ? 2 * NTHREADS : NTHREADS, BN = BNt * (NTH / NTHREADS);
+    static constexpr int STAGES = JGS ? 2 : 4, STAGE_F = (BMt + BN) * (TMA ? 2 * KC : ROWF), CTAS = JGS ? 3 : 2;
     static constexpr int SMEM_BYTES = STAGES * STAGE_F * (int)sizeof(float) + (TMA ? 1024 : 0);
-    static constexpr int THREADS = TMA ? NTHREADS + 32 : NTHREADS;
+    static constexpr int THREADS = TMA ? NTH + 32 : NTH;
 };
+constexpr int JTHREADS = Conf<float, true>::NTH;
 // TMA instance: stages of TK inputs in boxes of 32 (128-byte rows)
 constexpr int TK = 2 * KC, BOX_K = 32, TMA_STAGES = 4, TMA_STAGE_BYTES = (BMt + BNt) * TK * 4;
 
@@ -44,7 +48,7 @@ extern __shared__ __align__(16) float g_sm[];
 
 struct Smem {
     int list_n;
-    int wcnt[NTHREADS / 32];
+    int wcnt[JTHREADS / 32];
     uint64_t full[TMA_STAGES], empty[TMA_STAGES];
 };
 
@@ -165,19 +169,19 @@ __device__ __forceinline__ void tma_tile(Smem &s, Ring &rg, int kend, int lr, in
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// One tile of  out = A[rows][K] * W[N][K]^T  over k in [0, kend): 8 MR rows x 16 NR columns, 128 threads of MR x NR outputs
+// One tile of  out = A[rows][K] * W[N][K]^T  over k in [0, kend): 8 MR rows x BN columns, NT threads of MR x NR outputs
 // (row lr + 8 i, column 4 NR warp + lc + 4 j).  Operand rows are copied as they lie in memory, 16 bytes at a time, three
 // steps of 64 inputs in flight; a thread reads four inputs of a row at once, the next four while it multiplies.  lr takes bits
 // 0, 3, 4 of the lane and lc bits 1, 2: a 16-byte shared-memory load whose address does not depend on bit 0, or not on bit 1,
 // takes two cycles for a warp instead of four.  Every output is one chain of fused multiply-adds over k in ascending order.
-template <typename T, int STAGES, int STAGE_F>
+template <typename T, int STAGES, int STAGE_F, int NT, int BN>
 __device__ __forceinline__ void gemm_tile(const T *A, int lda, const T *__restrict__ W, int ldw, int N, int kend,
                                           int m0, int n0, int lr, int wc, float (&acc)[MR][NR])
 {
     constexpr int EPP = 16 / sizeof(T);      // values per 16-byte piece
-    constexpr int PPR = KC / EPP, RPE = NTHREADS / PPR;    // pieces per row, rows per round of the 128 threads
-    constexpr int EA = BMt / RPE, EW = BNt / RPE;      // rounds for the activations, for the weights
-    static_assert(BMt % RPE == 0 && BNt % RPE == 0, "a round lies in one operand");
+    constexpr int PPR = KC / EPP, RPE = NT / PPR;          // pieces per row, rows per round of the threads
+    constexpr int E = (BMt + BN + RPE - 1) / RPE;      // rounds: the activations' rows, behind them the weights'
+    constexpr bool EVEN = (BMt + BN) % RPE == 0;
     const int steps = (kend + KC - 1) / KC;
     float *tile = g_sm;
 #pragma unroll
@@ -185,16 +189,20 @@ __device__ __forceinline__ void gemm_tile(const T *A, int lda, const T *__restri
 #pragma unroll
         for (int j = 0; j < NR; ++j) acc[i][j] = 0.0f;
     const int prow = threadIdx.x / PPR, pk = (threadIdx.x % PPR) * EPP;       // this thread's piece: row (+ RPE e), inputs
-    const T *pa = A + (size_t)(m0 + prow) * lda + pk;
     const uint32_t dst0 = smem_addr(tile) + 4u * (uint32_t)(prow * ROWF + pk);
     // (weight rows beyond the last column: the last one again, their outputs are not stored)
-    auto w_src = [&](int e) { return W + (size_t)min(n0 + prow + RPE * e, N - 1) * ldw + pk; };
-    uint4 reg[sizeof(T) == 2 ? EA + EW : 1];
+    auto src_of = [&](int e) {
+        const int row = prow + RPE * e;
+        const bool act = BMt % RPE == 0 ? e < BMt / RPE : row < BMt;
+        return act ? A + (size_t)(m0 + row) * lda + pk : W + (size_t)min(n0 + row - BMt, N - 1) * ldw + pk;
+    };
+    uint4 reg[sizeof(T) == 2 ? E : 1];
     auto fetch = [&](int c, int st) {               // fp32: asynchronous copies; bf16: into registers, converted by put()
         const int vals = max(0, min(EPP, kend - (c * KC + pk))), off = vals > 0 ? c * KC : -pk;
 #pragma unroll
-        for (int e = 0; e < EA + EW; ++e) {
-            const T *src = (e < EA ? pa + (size_t)(RPE * e) * lda : w_src(e - EA)) + off;
+        for (int e = 0; e < E; ++e) {
+            if (!EVEN && prow + RPE * e >= BMt + BN) break;
+            const T *src = src_of(e) + off;
             if constexpr (sizeof(T) == 4)
                 asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst0 + 4u * (uint32_t)(st * STAGE_F + RPE * e * ROWF)),
                              "l"(src), "r"(vals * 4) : "memory");
@@ -206,7 +214,8 @@ __device__ __forceinline__ void gemm_tile(const T *A, int lda, const T *__restri
     auto put = [&](int c, int st) {
         const int vals = kend - (c * KC + pk);
 #pragma unroll
-        for (int e = 0; e < EA + EW; ++e) {
+        for (int e = 0; e < E; ++e) {
+            if (!EVEN && prow + RPE * e >= BMt + BN) break;
             const uint32_t w[4] = {reg[sizeof(T) == 2 ? e : 0].x, reg[sizeof(T) == 2 ? e : 0].y, reg[sizeof(T) == 2 ? e : 0].z, reg[sizeof(T) == 2 ? e : 0].w};
             float v[8];
 #pragma unroll
@@ -306,8 +315,10 @@ template <typename T, bool JGS>
 __device__ void gemm_phase(Smem &s, Ring &rg, const MadeDev &m, const RunArgs &r, int l, const T *Asrc, T *out, const OutArgs &oa, const Win &w,
                            unsigned long long &issued, unsigned long long &skipped)
 {
+    constexpr int BN = Conf<T, JGS>::BN;
+    static_assert(JS_GT % BN == 0, "a tile lies in one tile of the metadata");
     const int N = m.n[l + 1], K = m.n[l], batch = r.batch;
-    const int mt = (batch + BMt - 1) / BMt, nt = (N + BNt - 1) / BNt, G = (int)gridDim.x;
+    const int mt = (batch + BMt - 1) / BMt, nt = (N + BN - 1) / BN, G = (int)gridDim.x;
     const bool is_out = (l == m.L);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int lr = (lane & 1) | ((lane >> 3) << 1), wc = 4 * NR * warp + ((lane >> 1) & 3);
@@ -316,7 +327,7 @@ __device__ void gemm_phase(Smem &s, Ring &rg, const MadeDev &m, const RunArgs &r
     for (int round = 0; round * G < mt * nt; ++round) {
         const int tile = round * G + ((round & 1) ? G - 1 - (int)blockIdx.x : (int)blockIdx.x);
         if (tile >= mt * nt) continue;
-        const int tn = nt - 1 - tile / mt, tm = tile % mt, m0 = tm * BMt, n0 = tn * BNt, meta = n0 / JS_GT;
+        const int tn = nt - 1 - tile / mt, tm = tile % mt, m0 = tm * BMt, n0 = tn * BN, meta = n0 / JS_GT;
         const int dmin = m.t_dmin[l][meta], dmax = m.t_dmax[l][meta];
         bool live;
         if (is_out) live = (dmax - 1 >= w.olo) && (dmin - 1 < w.ohi);
@@ -360,7 +371,7 @@ __device__ void gemm_phase(Smem &s, Ring &rg, const MadeDev &m, const RunArgs &r
         if constexpr (Conf<T, JGS>::TMA) {
             tma_tile(s, rg, m.t_kend[l][meta], lr, wc, r.ctl, acc);
         } else {
-            gemm_tile<T, Conf<T, JGS>::STAGES, Conf<T, JGS>::STAGE_F>(Asrc, K, (const T *)m.W[l], K, N, m.t_kend[l][meta], m0, n0, lr, wc, acc);
+            gemm_tile<T, Conf<T, JGS>::STAGES, Conf<T, JGS>::STAGE_F, Conf<T, JGS>::NTH, BN>(Asrc, K, (const T *)m.W[l], K, N, m.t_kend[l][meta], m0, n0, lr, wc, acc);
         }
 #pragma unroll
         for (int i = 0; i < MR; ++i) {
@@ -515,7 +526,7 @@ __device__ void jgs_hidden_phase(Smem &s, const MadeDev &m, const RunArgs &r, in
         const int uend = min(N, ubase + 4096);
         if (threadIdx.x == 0) s.list_n = 0;
         __syncthreads();
-        for (int base = ubase; base < uend; base += NTHREADS) {
+        for (int base = ubase; base < uend; base += JTHREADS) {
             const int i = base + threadIdx.x;
             bool pred = false;
             if (i < uend) {
@@ -531,7 +542,7 @@ __device__ void jgs_hidden_phase(Smem &s, const MadeDev &m, const RunArgs &r, in
             __syncthreads();
             if (threadIdx.x == 0) {
                 int tot = 0;
-                for (int w2 = 0; w2 < NTHREADS / 32; ++w2) tot += s.wcnt[w2];
+                for (int w2 = 0; w2 < JTHREADS / 32; ++w2) tot += s.wcnt[w2];
                 s.list_n += tot;
             }
             __syncthreads();
@@ -730,10 +741,10 @@ static const void *generic_kernel_of(int prec, bool jgs)
 }
 static int generic_smem(int prec, bool jgs)
 {
-    if (jgs) return Conf<float, true>::SMEM_BYTES;
+    if (jgs) return prec == JS_BF16 ? Conf<__nv_bfloat16, true>::SMEM_BYTES : Conf<float, true>::SMEM_BYTES;
     return prec == JS_BF16 ? Conf<__nv_bfloat16, false>::SMEM_BYTES : Conf<float, false>::SMEM_BYTES;
 }
-static int generic_threads(int prec, bool jgs) { return prec == JS_BF16 || jgs ? NTHREADS : Conf<float, false>::THREADS; }
+static int generic_threads(int prec, bool jgs) { return jgs ? JTHREADS : prec == JS_BF16 ? NTHREADS : Conf<float, false>::THREADS; }
 
 // Tensor maps of an fp32 model's activations and masked weights: boxes of 32 inputs x 16 rows (activations) or 32 rows, 128-byte
 // swizzle; and of the activations once more for every 64-wide tile of outputs, with the inputs that it reads.
