@@ -835,32 +835,10 @@ conv_tc_kernel(const __grid_constant__ ConvDev m, const __grid_constant__ RunArg
 }  // namespace
 
 // --------------------------------------------------------------- host side
-typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
-                                  const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-static EncodeTiledFn conv_encode_fn()
-{
-    static EncodeTiledFn fn = nullptr;
-    if (fn) return fn;
-    void *p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess)
-        return nullptr;
-    fn = (EncodeTiledFn)p;
-    return fn;
-}
-
 static bool encode_nd(CUtensorMap *out, const void *base, int rank, const cuuint64_t *dims, const cuuint64_t *strides,
                       const cuuint32_t *box, CUtensorMapDataType type = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16)
 {
-    EncodeTiledFn fn = conv_encode_fn();
-    if (!fn) return false;
-    const cuuint32_t estr[4] = {1, 1, 1, 1};
-    return fn(out, type, rank, const_cast<void *>(base), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    return js_encode_map(out, type, base, rank, dims, strides, box);
 }
 
 template <typename T>
@@ -887,7 +865,7 @@ int js_conv_build(js_model *mo, const js_conv_desc *d)
     if (d->in_ch < 1 || d->in_ch > 8 || (d->ch != 64 && d->ch != 128)) return JS_ERR_UNSUPPORTED;
     if (d->width < 8 || d->width > 128 || (128 % d->width) != 0 || d->height < 1) return JS_ERR_UNSUPPORTED;
     if (d->n_conv < 1 || d->n_conv > JS_MAXL || d->max_batch > MAX_IMAGES) return JS_ERR_UNSUPPORTED;
-    if (!conv_encode_fn()) return JS_ERR_UNSUPPORTED;
+    if (!js_tensor_maps()) return JS_ERR_UNSUPPORTED;
     v.height = d->height; v.width = d->width; v.in_ch = d->in_ch; v.ch = d->ch; v.n_conv = d->n_conv; v.C = d->C;
     v.T = d->height * d->width * d->in_ch;
     v.R = 128 / d->width;

@@ -151,8 +151,11 @@ int js_launch_made_tc(const js_model *m, const RunArgs &r, cudaStream_t stream);
 int js_small_prepare(js_model *m);
 bool js_small_serves(const js_model *m, const RunArgs &r);
 int js_launch_made_small(const js_model *m, const RunArgs &r, cudaStream_t stream, int *clusters);
-bool js_encode_map_2d(CUtensorMap *out, const void *base, int rows, int cols, int box_rows);
-bool js_encode_map_f32(CUtensorMap *out, const void *base, int rows, int cols, int box_cols, int box_rows, int row_stride = 0);
+bool js_tensor_maps();        // can the driver encode them?
+bool js_encode_map(CUtensorMap *out, CUtensorMapDataType type, const void *base, int rank, const cuuint64_t *dims,
+                   const cuuint64_t *strides, const cuuint32_t *box);
+bool js_encode_map_2d(CUtensorMap *out, CUtensorMapDataType type, const void *base, int rows, int cols, int box_cols, int box_rows,
+                      int row_stride = 0);
 int js_generic_prepare(js_model *m);
 int js_cluster_prepare(js_model *m);
 bool js_cluster_serves(const js_model *m, const RunArgs &r);

@@ -66,26 +66,10 @@ struct ClShared {
     float bias_s[CL_MAXL + 1][MAXOWN][TM];
 };
 
-__device__ __forceinline__ uint32_t cluster_rank()
-{
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ uint32_t peer_addr(uint32_t addr, uint32_t cta)
-{
-    uint32_t p;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(p) : "r"(addr), "r"(cta));
-    return p;
-}
 __device__ __forceinline__ void copy_to_peer(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar)
 {
     asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(dst), "r"(src), "r"(bytes), "r"(bar) : "memory");
-}
-__device__ __forceinline__ void cluster_sync_all()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8])
 {
@@ -725,7 +709,7 @@ made_cluster_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ C
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (CS > 1) cluster_sync_all();          // every CTA's barriers are initialised
+    if (CS > 1) cluster_sync();          // every CTA's barriers are initialised
     if (tid == 0) mbar_arrive(&sh.go);       // the first pass
 
     int status = JS_OK, passes = 0, fin = 0;
@@ -768,7 +752,7 @@ made_cluster_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ C
         tc_fence_after();
         tmem_dealloc(sh.tmem_base, NSLOT * 2 * ACC);
     }
-    if (CS > 1) cluster_sync_all();
+    if (CS > 1) cluster_sync();
     if (tid == 64 && e.rank == 0)
         cluster_report(r.words, cluster, alive && ld_volatile_i32(&r.ctl->abort) == 0, status, passes, fin, sh.tiles * (unsigned)CS);
 }
@@ -818,7 +802,7 @@ int js_cluster_prepare(js_model *mo)
             c.tiles.dmax[l][t] = (short)hi;
         }
         c.npad[l] = mo->tc.lay[l].npad;
-        if (!js_encode_map_2d(&maps[l], mo->tc_weights[l], c.nkb[l] * c.npad[l], BK, TM)) return 0;
+        if (!js_encode_map_2d(&maps[l], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, mo->tc_weights[l], c.nkb[l] * c.npad[l], BK, BK, TM)) return 0;
     }
     c.kblocks = (c.kblocks + c.CS - 1) / c.CS;
     // Encodings may be sent before the pass has ended everywhere if each CTA's last output tile reads hidden units of every

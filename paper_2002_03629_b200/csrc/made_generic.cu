@@ -755,13 +755,13 @@ int js_generic_prepare(js_model *mo)
     if (v.prec != JS_F32) return JS_OK;
     std::vector<CUtensorMap> maps(2 * (v.L + 1));
     for (int l = 0; l <= v.L; ++l) {
-        if (!js_encode_map_f32(&maps[l], v.a[l], mo->rows, v.n[l], BOX_K, BMt) ||
-            !js_encode_map_f32(&maps[v.L + 1 + l], v.W[l], v.n[l + 1], v.n[l], BOX_K, BNt))
+        if (!js_encode_map_2d(&maps[l], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, v.a[l], mo->rows, v.n[l], BOX_K, BMt) ||
+            !js_encode_map_2d(&maps[v.L + 1 + l], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, v.W[l], v.n[l + 1], v.n[l], BOX_K, BNt))
             return JS_ERR_CUDA;
         v.cut_off[l] = (int)maps.size() - 2 * (v.L + 1);
         for (int kend : mo->host_kend[l]) {
             maps.emplace_back();
-            if (!js_encode_map_f32(&maps.back(), v.a[l], mo->rows, std::max(kend, 1), BOX_K, BMt, v.n[l])) return JS_ERR_CUDA;
+            if (!js_encode_map_2d(&maps.back(), CU_TENSOR_MAP_DATA_TYPE_FLOAT32, v.a[l], mo->rows, std::max(kend, 1), BOX_K, BMt, v.n[l])) return JS_ERR_CUDA;
         }
     }
     void *p = nullptr;

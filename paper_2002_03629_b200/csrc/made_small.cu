@@ -39,18 +39,6 @@ struct SmallShared {
     unsigned tiles;
 };
 
-__device__ __forceinline__ uint32_t cluster_rank()
-{
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ uint32_t peer_addr(uint32_t addr, uint32_t cta)
-{
-    uint32_t p;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(p) : "r"(addr), "r"(cta));
-    return p;
-}
 __device__ __forceinline__ void st_peer_f(uint32_t addr, float v)
 {
     asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
@@ -60,14 +48,6 @@ __device__ __forceinline__ int ld_peer_i(uint32_t addr)
     int v;
     asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
     return v;
-}
-__device__ __forceinline__ void atom_peer_add(uint32_t addr, unsigned v)
-{
-    asm volatile("red.shared::cluster.add.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
-}
-__device__ __forceinline__ void cluster_sync()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 // shared memory after the packed weights: activations a[l][k][RS], noise and symbols of the CTA's own positions
@@ -330,7 +310,7 @@ made_small_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ Sma
     tiles = __reduce_add_sync(0xffffffffu, lane == 0 ? (unsigned)tiles : 0u);
     if (lane == 0) {
         if constexpr (!CL) atomicAdd(&sh.tiles, (unsigned)tiles);
-        else atom_peer_add(peer_addr(smem_u32(&sh.tiles), 0), (unsigned)tiles);
+        else peer_add(peer_addr(smem_u32(&sh.tiles), 0), (unsigned)tiles);
     }
     if (gave_up)
         for (int i = 0; i < 2000; ++i) __nanosleep(1000);      // weights still on their way land before shared memory goes away

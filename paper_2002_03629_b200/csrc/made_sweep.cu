@@ -80,12 +80,6 @@ struct Base { int kbs, ub0, nb; };           // K blocks [0, kbs), units [ub0, u
 
 // shared-memory accesses by 32-bit shared address: the position loop runs on one warp per scheduler, and
 // a generic load (which is what a pointer kept in a structure compiles to) waits much longer than ld.shared
-__device__ __forceinline__ float4 lds_f4(uint32_t a)
-{
-    float4 v;
-    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a));
-    return v;
-}
 __device__ __forceinline__ void sts_f4(uint32_t a, float4 v)
 {
     asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
@@ -851,34 +845,6 @@ __global__ void jgs_book_kernel(int batch, int k, int at_cap, int *changed, int 
 }  // namespace
 
 // --------------------------------------------------------------- host side
-typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
-                                  const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-static EncodeTiledFn sweep_encode_fn()
-{
-    static EncodeTiledFn fn = nullptr;
-    if (fn) return fn;
-    void *p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess)
-        return nullptr;
-    fn = (EncodeTiledFn)p;
-    return fn;
-}
-
-static bool sweep_encode(CUtensorMap *out, const void *base, int rank, const cuuint64_t *dims, const cuuint64_t *strides,
-                         const cuuint32_t *box)
-{
-    EncodeTiledFn fn = sweep_encode_fn();
-    if (!fn) return false;
-    const cuuint32_t estr[3] = {1, 1, 1};
-    return fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, const_cast<void *>(base), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 typedef void (*SweepKernelFn)(const MadeDev, const SweepDev, const RunArgs);
 template <int L>
 static SweepKernelFn sweep_kernel_of(int rj_idx)
@@ -908,7 +874,7 @@ int js_sweep_prepare(js_model *mo)
     mo->sweep_state = -1;
     const MadeDev &v = mo->made;
     SweepDev &s = mo->sweep;
-    if (!mo->tc_ok || v.C != 1 || v.prec != JS_BF16 || !sweep_encode_fn()) return 0;
+    if (!mo->tc_ok || v.C != 1 || v.prec != JS_BF16 || !js_tensor_maps()) return 0;
     if ((v.L + 1) * NUP > BASE_COL) return 0;              // the groups' accumulators end where the base's begin
     const int L = v.L, T = v.T;
     // prefix counts; the group size is the largest one that keeps every layer's units of a group within NUP
@@ -972,15 +938,15 @@ int js_sweep_prepare(js_model *mo)
             const cuuint64_t dimsA[2] = {(cuuint64_t)v.n[l], (cuuint64_t)mo->rows}, stridesA[1] = {(cuuint64_t)v.n[l] * 2};
             for (int i = 0; i < 3; ++i) {
                 const cuuint32_t box[3] = {(cuuint32_t)BK, 32u << i, 1};
-                if (!sweep_encode(&mapsF[i * (L + 1) + l], f, 3, dims, strides, box)) return 0;
-                if (!sweep_encode(&mapsA[i * (L + 1) + l], v.a[l], 2, dimsA, stridesA, box)) return 0;
+                if (!js_encode_map(&mapsF[i * (L + 1) + l], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, f, 3, dims, strides, box)) return 0;
+                if (!js_encode_map(&mapsA[i * (L + 1) + l], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, v.a[l], 2, dimsA, stridesA, box)) return 0;
             }
         }
         for (int big = 0; big < 3; ++big) {
             const cuuint64_t dims[2] = {(cuuint64_t)v.n[l], (cuuint64_t)v.n[l + 1]};
             const cuuint64_t strides[1] = {(cuuint64_t)v.n[l] * 2};
             const cuuint32_t box[2] = {(cuuint32_t)BK, big == 2 ? (cuuint32_t)NB : 16u << big};
-            if (!sweep_encode(&mapsW[big * (L + 1) + l], v.W[l], 2, dims, strides, box)) return 0;
+            if (!js_encode_map(&mapsW[big * (L + 1) + l], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, v.W[l], 2, dims, strides, box)) return 0;
         }
     }
     void *pf = nullptr, *pw = nullptr, *pa = nullptr;

@@ -1249,52 +1249,6 @@ __global__ void tile_major_weights(const __nv_bfloat16 *__restrict__ W, __nv_bfl
 }
 
 // --------------------------------------------------------------- host side
-typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
-                                  const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-static EncodeTiledFn get_encode_fn()
-{
-    static EncodeTiledFn fn = nullptr;
-    if (fn) return fn;
-    void *p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess)
-        return nullptr;
-    fn = (EncodeTiledFn)p;
-    return fn;
-}
-
-// 2-D bf16 row-major tensor [rows][cols], box = 64 columns x box_rows rows, 128-byte swizzle
-bool js_encode_map_2d(CUtensorMap *out, const void *base, int rows, int cols, int box_rows)
-{
-    EncodeTiledFn fn = get_encode_fn();
-    if (!fn) return false;
-    const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-    const cuuint64_t strides[1] = {(cuuint64_t)cols * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)BK, (cuuint32_t)box_rows};
-    const cuuint32_t estr[2] = {1, 1};
-    return fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// 2-D fp32 row-major tensor [rows][cols], rows row_stride values apart (a multiple of 4; 0: cols), box = box_cols (32: one
-// 128-byte swizzle row) x box_rows
-bool js_encode_map_f32(CUtensorMap *out, const void *base, int rows, int cols, int box_cols, int box_rows, int row_stride)
-{
-    EncodeTiledFn fn = get_encode_fn();
-    if (!fn) return false;
-    const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-    const cuuint64_t strides[1] = {(cuuint64_t)(row_stride ? row_stride : cols) * 4};
-    const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
-    const cuuint32_t estr[2] = {1, 1};
-    return fn(out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void *>(base), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 // Builds the tensor-core view of a model.  Returns 1 if the model qualifies, 0 if it
 // does not (the CUDA-core path then serves it), negative on CUDA errors.
 int js_tc_prepare(js_model *mo)
@@ -1306,7 +1260,7 @@ int js_tc_prepare(js_model *mo)
     if (!(v.C == 1 || v.C == 256)) return 0;
     for (int l = 0; l <= v.L; ++l)
         if (v.n[l] % 8 != 0) return 0;
-    if (!get_encode_fn()) return 0;
+    if (!js_tensor_maps()) return 0;
     const int L = v.L;
     bool wide = (v.C == 256);
     t.stage_bytes = A_BYTES + (wide ? 256 : 128) * BK * 2;
@@ -1375,7 +1329,7 @@ int js_tc_prepare(js_model *mo)
         const int ring_cap = t.ring_bytes + (l < L ? t.aux_bytes - STAGING_BYTES : 0);
         t.lay[l].n_stages = std::min(MAX_STAGES, ring_cap / t.lay[l].stage_bytes);
         kb_all[l] = kb;
-        if (!js_encode_map_2d(&mapsA[l], v.a[l], mo->rows, K, BM)) return 0;
+        if (!js_encode_map_2d(&mapsA[l], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, v.a[l], mo->rows, K, BK, BM)) return 0;
         {
             const int nkb = (K + BK - 1) / BK, npad = nt * bn;
             void *wp = nullptr;
@@ -1385,7 +1339,7 @@ int js_tc_prepare(js_model *mo)
             if (cudaGetLastError() != cudaSuccess) return JS_ERR_CUDA;
             mo->tc_weights[l] = wp;
             t.lay[l].npad = npad;
-            if (!js_encode_map_2d(&mapsW[l], wp, nkb * npad, BK, bn)) return 0;
+            if (!js_encode_map_2d(&mapsW[l], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, wp, nkb * npad, BK, BK, bn)) return 0;
         }
     }
     if (cudaDeviceSynchronize() != cudaSuccess) return JS_ERR_CUDA;     // the tile-major copies are complete

@@ -49,6 +49,28 @@ __device__ __forceinline__ bool mbar_test_wait(uint64_t *bar, uint32_t parity)
         : "memory");
     return ok != 0;
 }
+// thread-block clusters: this CTA's rank, an address of this CTA's shared memory in CTA `cta`, an addition there, the barrier
+__device__ __forceinline__ uint32_t cluster_rank()
+{
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ uint32_t peer_addr(uint32_t addr, uint32_t cta)
+{
+    uint32_t p;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(p) : "r"(addr), "r"(cta));
+    return p;
+}
+__device__ __forceinline__ void peer_add(uint32_t addr, unsigned v)
+{
+    asm volatile("red.shared::cluster.add.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 __device__ __forceinline__ uint64_t global_ns()
 {
     uint64_t t;
@@ -229,32 +251,12 @@ __device__ __forceinline__ void tmem_ld32_issue(uint32_t taddr, uint32_t (&r)[32
 
 // loads that are issued where they are written (the compiler may otherwise sink a plain load down to
 // its first use, which turns a batch of independent loads into a chain of exposed latencies)
-__device__ __forceinline__ float2 ld_nc_f2_now(const float *p)
-{
-    float2 v;
-    asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
-    return v;
-}
-__device__ __forceinline__ uint32_t ld_u16_now(const uint8_t *p)
-{
-    uint16_t v;
-    asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p));
-    return (uint32_t)v;
-}
-
 __device__ __forceinline__ float4 ld_nc_f4_now(const float *p)
 {
     float4 v;
     asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
     return v;
 }
-__device__ __forceinline__ uint32_t ld_u32_now(const uint8_t *p)
-{
-    uint32_t v;
-    asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
-    return v;
-}
-
 __device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 // 32 consecutive fp32 columns of this thread's TMEM lane
