@@ -83,3 +83,27 @@ def test_host_call_argument_errors():
             p.jacobi_sample_host(model, noise, cfg.noise_kind, None, p.JS_GS_JACOBI, 0, 0, out)
     finally:
         model.close()
+
+
+def test_host_buffers_before_torch_has_touched_the_gpu():
+    """A program that only has host tensors: the binding asks for the current stream before torch has set its side up."""
+    import os
+    import subprocess
+    import sys
+    code = """
+import numpy as np
+import torch
+import paper_2002_03629_b200 as p, synth_inputs as si
+cfg = si.CONFIGS["made_tiny"]
+W, b = si.made_weights(cfg)
+m = p.Model.from_config(cfg, W, b, si.made_lut(cfg))
+noise = torch.from_numpy(si.draw_noise(cfg))
+out = torch.zeros((cfg.batch, cfg.D), dtype=torch.uint8)
+assert p.jacobi_sample_host(m, noise, cfg.noise_kind, None, p.JS_JACOBI, 0, 0, out) == 0
+import oracle
+ref = oracle.from_config(cfg, W, b, si.made_lut(cfg)).sequential_batch(noise.numpy(), cfg.noise_kind)
+assert np.array_equal(out.numpy(), ref)
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    run = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
+    assert run.returncode == 0, run.stdout + run.stderr
