@@ -196,7 +196,8 @@ typedef enum {
 } js_option;
 int js_set_option(js_model *m, int option, int value);
 
-/* counters of the most recent sampling call on this model */
+/* counters of the most recent sampling call on this model.  Where groups of samples are solved by themselves (small and
+ * ordinary binary models) iterations and final_frontier are those of the group that took most, tiles and flops all groups'. */
 typedef struct {
     int iterations;            /* forward passes executed; outer iterations for Jacobi-GS on the tensor cores (micro-steps
                                   on the CUDA-core kernels); 1 for the cached sweep */

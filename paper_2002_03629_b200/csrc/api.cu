@@ -184,7 +184,7 @@ int common_scratch(js_model *m, int T)
     if ((rc = dev_alloc<JsCtl>(m, &m->ctl, 1, true)) != JS_OK) return rc;
     CU_TRY(cudaHostAlloc((void **)&m->h_result, sizeof(JsCtl), cudaHostAllocMapped));
     CU_TRY(cudaHostGetDevicePointer((void **)&m->d_result, m->h_result, 0));
-    CU_TRY(cudaHostAlloc((void **)&m->h_words, sizeof(unsigned long long) * JS_MAX_CLUSTERS, cudaHostAllocMapped));
+    CU_TRY(cudaHostAlloc((void **)&m->h_words, 2 * sizeof(unsigned long long) * JS_MAX_CLUSTERS, cudaHostAllocMapped));
     CU_TRY(cudaHostGetDevicePointer((void **)&m->d_words, m->h_words, 0));
     if ((rc = dev_alloc<int>(m, &m->smp_changed, 2 * (size_t)m->rows, true)) != JS_OK) return rc;
     if ((rc = dev_alloc<int>(m, &m->smp_state, 2 * (size_t)m->rows, true)) != JS_OK) return rc;
@@ -294,36 +294,52 @@ int wait_result(js_model *m, cudaStream_t st, bool poll, JsCtl &h)
     return JS_OK;
 }
 
-// The same for kernels whose clusters report one by one (cluster_report in made_driver.cuh).
-int wait_words(js_model *m, int n, cudaStream_t st, bool poll, JsCtl &h)
+// The same for kernels whose clusters report one by one (cluster_report in made_driver.cuh).  The statistics are those of
+// the whole call: each cluster's passes, tiles and counts added up.
+int wait_words(js_model *m, const ClusterWork &work, bool cluster, cudaStream_t st, bool poll, JsCtl &h)
 {
     if (!poll) CU_TRY(cudaStreamSynchronize(st));
     memset(&h, 0, sizeof h);
     h.frontier = INT_MAX;
     volatile unsigned long long *words = m->h_words;
-    for (int c = 0; c < n; ++c) {
-        for (unsigned i = 1; words[c] == 0; ++i) {
-            if ((i & 0x3fffu) == 0) {
+    unsigned long long passes = 0, counts = 0, most = 0;
+    for (int i = 0; i < 2 * work.clusters; ++i) {
+        for (unsigned n = 1; words[i] == 0; ++n) {
+            if (!poll || (n & 0x3fffu) == 0) {
                 const cudaError_t e = cudaStreamQuery(st);
                 if (e == cudaErrorNotReady) continue;
                 CU_TRY(e);
-                if (words[c] == 0) {
+                if (words[i] == 0) {
                     snprintf(g_cuda_err, sizeof g_cuda_err, "the kernel ended without reporting");
                     return JS_ERR_CUDA;
                 }
             }
             cpu_relax();
         }
-        const unsigned long long w = words[c];
+        const unsigned long long w = words[i];
+        if (i & 1) {
+            h.iters_max = std::max(h.iters_max, (int)(w >> 1 & 0xfffff));
+            counts += w >> 21;
+            most = std::max(most, w >> 21);
+            continue;
+        }
         const int state = (int)(w & 3);
         if (state == 3) h.status = JS_ERR_TIMEOUT;
         else if (state == 2 && h.status == JS_OK) h.status = JS_NOT_CONVERGED;
         h.iterations = std::max(h.iterations, (int)(w >> 2 & 0xfffff));
         h.frontier = std::min(h.frontier, (int)(w >> 22 & 0xfffff));
+        passes += w >> 2 & 0xfffff;
         h.tiles_issued += w >> 42;
     }
     std::atomic_thread_fence(std::memory_order_acquire);
-    h.iters_max = h.iterations;
+    if (cluster) {           // counted: K blocks.  Every cluster streams its own weights; they are counted once per pass
+        const unsigned long long all = passes * (unsigned long long)work.tiles;
+        h.tiles_skipped = all > h.tiles_issued ? all - h.tiles_issued : 0;
+        h.mma_flops = counts * (unsigned long long)work.block_flops;
+        h.weight_bytes = most * (unsigned long long)work.block_bytes;
+    } else {
+        h.tiles_skipped = counts;
+    }
     m->ctl_clean = h.status >= 0;        // these kernels touch the control block only to give up
     return JS_OK;
 }
@@ -471,11 +487,11 @@ int run_made(js_model *m, RunArgs &r, cudaStream_t st)
     if (rc != JS_OK) return rc;
     const bool cluster = m->opt_path == 0 && js_cluster_serves(m, r);
     if (cluster || js_small_serves(m, r)) {
-        int clusters = 0;
-        const int rl = cluster ? js_launch_made_cluster(m, r, st, &clusters) : js_launch_made_small(m, r, st, &clusters);
+        ClusterWork work;
+        const int rl = cluster ? js_launch_made_cluster(m, r, st, &work) : js_launch_made_small(m, r, st, &work);
         if (rl != 0) return launch_failed(rl);
         JsCtl h;
-        if ((rc = wait_words(m, clusters, st, may_poll(r), h)) != JS_OK) return rc;
+        if ((rc = wait_words(m, work, cluster, st, may_poll(r), h)) != JS_OK) return rc;
         fill_stats(m, h, cluster ? 0 : 1);
         return h.status;
     }

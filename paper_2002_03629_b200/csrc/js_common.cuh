@@ -85,7 +85,7 @@ struct RunArgs {
     JsCtl *ctl;
     const unsigned *noise_ready;   // NULL, or a word that takes the value noise_stamp once `noise` has arrived
     unsigned noise_stamp;
-    unsigned long long *words;     // mapped host memory: one report per cluster (kernels without a grid-wide step)
+    unsigned long long *words;     // mapped host memory: two words per cluster, its report (kernels without a grid-wide step)
     JsCtl *result;            // host memory mapped into the device: the last CTA to leave copies ctl here
     unsigned long long *trace;   // [2 CTAs][JS_TRACE_PHASES][JS_TRACE_SLOTS] globaltimer stamps, or NULL
     int trace_cta;               // the second traced CTA (the first is CTA 0); < 0: the last CTA of the grid

@@ -103,6 +103,13 @@ struct ConvDev {
 
 #define JS_MAX_CLUSTERS 4096          // most clusters a call of the cluster kernels may have
 
+// What a launch of a cluster kernel consists of, for the statistics.
+struct ClusterWork {
+    int clusters;
+    int tiles;                              // output tiles of a pass, all layers (cluster kernel of bf16 models)
+    long long block_flops, block_bytes;     // of a K block: its MMAs, its weights
+};
+
 struct js_model {
     std::vector<int> host_kend[JS_MAXL + 1];       // t_kend of the device view
     int kind = 0;                 // 0 masked MLP, 1 masked-conv stack
@@ -115,7 +122,7 @@ struct js_model {
     JsCtl *ctl = nullptr;
     JsCtl *h_result = nullptr;    // pinned host memory, mapped: the kernels report here
     JsCtl *d_result = nullptr;    // the same memory as the device sees it
-    unsigned long long *h_words = nullptr, *d_words = nullptr;      // JS_MAX_CLUSTERS reports, mapped like h_result
+    unsigned long long *h_words = nullptr, *d_words = nullptr;      // JS_MAX_CLUSTERS reports of two words, mapped like h_result
     bool ctl_clean = false;       // the last call left the control block zeroed
     // host-buffer entry point: device staging, copy stream, "noise has arrived" word
     float *st_noise = nullptr;
@@ -150,7 +157,7 @@ int js_tc_prepare(js_model *m);
 int js_launch_made_tc(const js_model *m, const RunArgs &r, cudaStream_t stream);
 int js_small_prepare(js_model *m);
 bool js_small_serves(const js_model *m, const RunArgs &r);
-int js_launch_made_small(const js_model *m, const RunArgs &r, cudaStream_t stream, int *clusters);
+int js_launch_made_small(const js_model *m, const RunArgs &r, cudaStream_t stream, ClusterWork *work);
 bool js_tensor_maps();        // can the driver encode them?
 bool js_encode_map(CUtensorMap *out, CUtensorMapDataType type, const void *base, int rank, const cuuint64_t *dims,
                    const cuuint64_t *strides, const cuuint32_t *box);
@@ -159,7 +166,7 @@ bool js_encode_map_2d(CUtensorMap *out, CUtensorMapDataType type, const void *ba
 int js_generic_prepare(js_model *m);
 int js_cluster_prepare(js_model *m);
 bool js_cluster_serves(const js_model *m, const RunArgs &r);
-int js_launch_made_cluster(const js_model *m, const RunArgs &r, cudaStream_t stream, int *clusters);
+int js_launch_made_cluster(const js_model *m, const RunArgs &r, cudaStream_t stream, ClusterWork *work);
 int js_conv_build(js_model *m, const js_conv_desc *d);
 int js_launch_conv_tc(const js_model *m, const RunArgs &r, cudaStream_t stream);
 int js_sweep_prepare(js_model *m);

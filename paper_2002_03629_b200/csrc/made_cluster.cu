@@ -63,6 +63,7 @@ struct ClShared {
     int count[64];
     int issued, consumed;                    // weight loads
     unsigned tiles;
+    unsigned sums[2];                        // of the whole cluster (in its first CTA): tiles, K blocks
     float bias_s[CL_MAXL + 1][MAXOWN][TM];
 };
 
@@ -650,7 +651,7 @@ made_cluster_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ C
         mbar_init(&sh.ack, jacobi ? 2 : 3);
         sh.stop = sh.dead = 0;
         sh.issued = sh.consumed = 0;
-        sh.tiles = 0;
+        sh.tiles = sh.sums[0] = sh.sums[1] = 0;
         for (int i = 0; i < 2; ++i) { sh.chg[i][0] = sh.chg[i][1] = 0; sh.first[i] = INT_MAX; }
     }
     for (int i = tid; i < 2 * CL_TILES; i += NTH) mbar_init(&(&sh.xbar[0][0])[i], 1);
@@ -745,6 +746,10 @@ made_cluster_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ C
         if (e.rank == 0 && r.out_iters)
             for (int s = tid - 64; s < nrow; s += 128) r.out_iters[row0 + s] = sh.count[s];
     }
+    if (tid == 0) {
+        peer_add(peer_addr(smem_u32(&sh.sums[0]), 0), sh.tiles);
+        peer_add(peer_addr(smem_u32(&sh.sums[1]), 0), (unsigned)sh.consumed);
+    }
     if (!alive)
         for (int i = 0; i < 2000; ++i) __nanosleep(1000);      // copies still in flight land before shared memory goes away
     __syncthreads();
@@ -753,8 +758,13 @@ made_cluster_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ C
         tmem_dealloc(sh.tmem_base, NSLOT * 2 * ACC);
     }
     if (CS > 1) cluster_sync();
-    if (tid == 64 && e.rank == 0)
-        cluster_report(r.words, cluster, alive && ld_volatile_i32(&r.ctl->abort) == 0, status, passes, fin, sh.tiles * (unsigned)CS);
+    if (warp == 2 && e.rank == 0) {
+        int most = 0;
+        for (int s = lane; s < nrow; s += 32) most = max(most, sh.count[s]);
+        most = __reduce_max_sync(0xffffffffu, most);
+        if (lane == 0)
+            cluster_report(r.words, cluster, alive && ld_volatile_i32(&r.ctl->abort) == 0, status, passes, fin, sh.sums[0], most, sh.sums[1]);
+    }
 }
 
 }  // namespace
@@ -871,14 +881,15 @@ bool js_cluster_serves(const js_model *mo, const RunArgs &r)
     return mo->cluster.kblocks <= 230 && (r.batch + R - 1) / R <= std::min(JS_MAX_CLUSTERS, mo->cluster.max_clusters);
 }
 
-int js_launch_made_cluster(const js_model *mo, const RunArgs &r, cudaStream_t stream, int *clusters)
+int js_launch_made_cluster(const js_model *mo, const RunArgs &r, cudaStream_t stream, ClusterWork *work)
 {
     ClusterDev c = mo->cluster;
     const int R = cluster_rows(mo, r.batch, &c.n_stages);
-    *clusters = (r.batch + R - 1) / R;
-    memset(mo->h_words, 0, sizeof(unsigned long long) * (size_t)*clusters);
+    *work = ClusterWork{(r.batch + R - 1) / R, 0, 2LL * TM * BK * R, STAGE};
+    for (int l = 0; l <= mo->made.L; ++l) work->tiles += c.nt[l];
+    memset(mo->h_words, 0, 2 * sizeof(unsigned long long) * (size_t)work->clusters);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(*clusters * c.CS));
+    cfg.gridDim = dim3((unsigned)(work->clusters * c.CS));
     cfg.blockDim = dim3(NTH);
     cfg.dynamicSmemBytes = cluster_smem(c, mo->made, R, c.n_stages);
     cfg.stream = stream;

@@ -267,13 +267,14 @@ __device__ __forceinline__ void driver_finish(const RunArgs &r, const DriverResu
     ctl_report(r, res.status);     // res.status is the same in every CTA
 }
 
-// Report of a cluster that solved its samples by itself (kernels without a grid-wide step): one 64-bit word in
-// mapped host memory per cluster, written when the cluster's outputs are complete; the host polls and combines
+// Report of a cluster that solved its samples by itself (kernels without a grid-wide step): two 64-bit words in
+// mapped host memory per cluster, each complete by itself, written when the cluster's outputs are complete; the host polls and combines
 // them (wait_words in api.cu).  No counter is shared on the device: summing up in the control
 // block and copying it out cost 4 us of fences and round trips at the end of a 15 us kernel.
-//   bits 0-1 state (1 done, 2 iteration cap reached, 3 a wait gave up), 2-21 iterations, 22-41 frontier, 42-63 tiles
+//   first: bits 0-1 state (1 done, 2 iteration cap reached, 3 a wait gave up), 2-21 iterations, 22-41 frontier, 42-63 tiles
+//   second: bit 0 set, 1-20 largest iteration count of a sample, 21-63 `count` (what it counts is the kernel's own)
 __device__ __forceinline__ void cluster_report(unsigned long long *words, int cluster, bool alive, int status,
-                                               int iterations, int frontier, unsigned tiles)
+                                               int iterations, int frontier, unsigned tiles, int iters_max, unsigned count)
 {
     const unsigned long long state = !alive ? 3ull : status == JS_OK ? 1ull : 2ull;
     const unsigned long long w = state | (unsigned long long)min(iterations, 0xfffff) << 2 |
@@ -283,5 +284,7 @@ __device__ __forceinline__ void cluster_report(unsigned long long *words, int cl
     // in device memory, which it only reaches through later work on the GPU, so the device-wide fence is the one they
     // need (for other outputs it synchronises the stream, may_poll in api.cu); the system-wide one costs 3 us here.
     __threadfence();
-    *reinterpret_cast<volatile unsigned long long *>(words + cluster) = w;
+    volatile unsigned long long *to = words + 2 * cluster;
+    to[1] = 1ull | (unsigned long long)min(iters_max, 0xfffff) << 1 | (unsigned long long)count << 21;
+    to[0] = w;
 }

@@ -36,7 +36,7 @@ struct SmallShared {
     int chg[2][RMAX];                    // per parity: did the sample change in this CTA's positions
     int first[2];                        // per parity: smallest changed position of this CTA
     int done[RMAX], count[RMAX];
-    unsigned tiles;
+    unsigned tiles, skipped;
 };
 
 __device__ __forceinline__ void st_peer_f(uint32_t addr, float v)
@@ -147,7 +147,7 @@ made_small_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ Sma
         if (i < RMAX) { sh.done[i] = 0; sh.count[i] = 0; }
     }
     if (tid < 2) sh.first[tid] = INT_MAX;
-    if (tid == 0) sh.tiles = 0u;
+    if (tid == 0) sh.tiles = sh.skipped = 0u;
     // A CTA whose weights do not come says so where every CTA of the cluster looks for the first iteration's changes: all of
     // them leave at the same place then.  (A spin limit of zero: the first look decides, as at the grid barriers.)
     bool here = mbar_test_wait(&sh.wbar, 0);
@@ -162,7 +162,7 @@ made_small_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ Sma
 
     const int cap = (r.max_iters > 0 && r.max_iters < T) ? r.max_iters : T;
     int fin_x = 0, fin_h = 0, lo = 0, k = 0, status = JS_OK;
-    unsigned long long tiles = 0;
+    unsigned tiles = 0, skipped = 0;
     int mf;
     for (;;) {
         ++k;
@@ -184,7 +184,7 @@ made_small_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ Sma
                 const int ii = min(i, nc - 1), dg = (int)(deg[ii] & 0xffffu);
                 // live: hidden units of degree > hlo, output positions (degree - 1) >= plo
                 const bool live = mine && (out ? dg > plo : dg > hlo);
-                if (!__any_sync(0xffffffffu, live)) continue;
+                if (!__any_sync(0xffffffffu, live)) { skipped++; continue; }
                 tiles++;
                 // inputs beyond the largest degree of the warp's units are masked: exact zeros
                 const int kend = min(K, s.kend[l][min(ib / 32, SMALL_KENDS - 1)]);
@@ -307,16 +307,20 @@ made_small_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ Sma
     }
     if (c == 0 && r.out_iters && alive)
         for (int rr = tid; rr < nrow; rr += NTH) r.out_iters[row0 + rr] = sh.count[rr];
-    tiles = __reduce_add_sync(0xffffffffu, lane == 0 ? (unsigned)tiles : 0u);
     if (lane == 0) {
-        if constexpr (!CL) atomicAdd(&sh.tiles, (unsigned)tiles);
-        else peer_add(peer_addr(smem_u32(&sh.tiles), 0), (unsigned)tiles);
+        if constexpr (!CL) {
+            atomicAdd(&sh.tiles, tiles);
+            atomicAdd(&sh.skipped, skipped);
+        } else {
+            peer_add(peer_addr(smem_u32(&sh.tiles), 0), tiles);
+            peer_add(peer_addr(smem_u32(&sh.skipped), 0), skipped);
+        }
     }
     if (gave_up)
         for (int i = 0; i < 2000; ++i) __nanosleep(1000);      // weights still on their way land before shared memory goes away
     if constexpr (CL) cluster_sync();          // no CTA leaves while others may still read its flags
     else __syncthreads();
-    if (tid == 0 && c == 0) cluster_report(r.words, (int)(blockIdx.x >> csh), alive, status, k, fin_x, sh.tiles);
+    if (tid == 0 && c == 0) cluster_report(r.words, (int)(blockIdx.x >> csh), alive, status, k, fin_x, sh.tiles, k, sh.skipped);
 }
 
 // packed weights of CTA c: per layer [K][ncs] (column i = unit of the i-th own output), then biases, then degrees
@@ -445,14 +449,14 @@ bool js_small_serves(const js_model *mo, const RunArgs &r)
     return mo->small_ok && r.kmode == KM_JACOBI && (r.real != 0) == (mo->made.C == 2) && rows_of(mo, r.batch) > 0;
 }
 
-int js_launch_made_small(const js_model *mo, const RunArgs &r, cudaStream_t stream, int *clusters)
+int js_launch_made_small(const js_model *mo, const RunArgs &r, cudaStream_t stream, ClusterWork *work)
 {
     const SmallDev &s = mo->small;
     const int R = rows_of(mo, r.batch), rg = rows_group(R), RS = (R + rg - 1) / rg * rg;
-    *clusters = (r.batch + R - 1) / R;
-    memset(mo->h_words, 0, sizeof(unsigned long long) * (size_t)*clusters);
+    *work = ClusterWork{(r.batch + R - 1) / R, 0, 0, 0};
+    memset(mo->h_words, 0, 2 * sizeof(unsigned long long) * (size_t)work->clusters);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(*clusters * s.CS));
+    cfg.gridDim = dim3((unsigned)(work->clusters * s.CS));
     cfg.blockDim = dim3(NTH);
     cfg.dynamicSmemBytes = (size_t)small_layout(mo->made, s, RS).total * 4;
     cfg.stream = stream;

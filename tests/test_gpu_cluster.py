@@ -50,3 +50,38 @@ def test_jacobi_and_blocks(T, H, batch, skip):
         out = torch.empty((batch, T), dtype=torch.uint8, device="cuda")
         assert p.jacobi_sample(model, d_noise, cfg.noise_kind, None, p.JS_JACOBI, 0, 1, out) == p.JS_NOT_CONVERGED
     model.close()
+
+
+@pytest.mark.parametrize("T,H,batch", [(129, (191, 65), 9), (530, (513, 1025), 100), (600, (520, 776, 640), 40)])
+def test_statistics_cover_the_whole_call(T, H, batch):
+    """Counters of a call whose clusters solve their samples by themselves: what the header says, and what the same call counts
+    on the grid-wide kernel (which JS_OPT_TRACE selects), where the two are comparable."""
+    import __graft_entry__ as ge
+    ge.build()
+    import paper_2002_03629_b200 as p
+    cfg = si.MadeConfig("cluster", 65, D=T, C=1, H=H, act=si.ACT_RELU, prec=si.PREC_BF16, batch=batch, noise_kind=si.NOISE_LOGISTIC, w_var_scale=3.0, b_var=0.1)
+    W, b = si.made_weights(cfg)
+    model = p.Model.from_config(cfg, W, b, si.made_lut(cfg))
+    noise = torch.from_numpy(si.draw_noise(cfg)).cuda()
+    n = [T, *H, T]
+    deg = [np.arange(1, T + 1), *[1 + np.arange(h) * (T - 1) // h for h in H], np.arange(1, T + 1)]
+    live = [int(np.searchsorted(deg[l], deg[l + 1], side="left" if l == len(H) else "right").sum()) for l in range(len(H) + 1)]
+    out = torch.empty((batch, T), dtype=torch.uint8, device="cuda")
+    it = torch.empty(batch, dtype=torch.int32, device="cuda")
+    for mode, block in ((p.JS_JACOBI, 0), (p.JS_GS_JACOBI, T // 3)):
+        seen = []
+        for trace in (0, 1):
+            model.set_option(p.JS_OPT_TRACE, trace)
+            assert p.jacobi_sample(model, noise, cfg.noise_kind, None, mode, block, 0, out, it) == 0
+            seen.append(model.stats())
+        a, grid = seen
+        assert a.path == grid.path == 0
+        assert a.batch_iters_max == grid.batch_iters_max == int(it.max())
+        assert a.iterations <= grid.iterations and a.tiles_issued > 0
+        assert (a.tiles_skipped > 0) == (mode == p.JS_GS_JACOBI)      # Jacobi passes compute every tile here
+        passes = a.iterations if mode == p.JS_JACOBI else 1
+        assert a.weight_bytes >= 2 * sum(live) * passes
+        assert a.mma_flops >= 2 * sum(live) * int(it.sum() if mode == p.JS_JACOBI else batch)
+        assert a.mma_flops <= 2 * 64 * 64 * 64 * (a.tiles_issued * max((v + 63) // 64 for v in n))
+        assert a.tiles_issued >= sum((v + 63) // 64 for v in n[1:])
+    model.close()
