@@ -13,7 +13,7 @@
 //     the MMA reads.  A finished tile IS one K block of the layer above: it is written in place and sent to the other CTAs by
 //     one bulk copy each (cp.async.bulk to distributed shared memory, completing on the receiver's mbarrier for that block).
 //     An MMA waits for the K blocks it reads, not for a layer: there is no barrier inside a pass;
-//   - weights stream from L2 through a ring, independent of all that: the next tile's, and in Jacobi mode the next pass's,
+//   - weights stream from L2 through two rings (even and odd K blocks), independent of all that: the next tile's, and in Jacobi mode the next pass's,
 //     weights are on their way while a layer waits for its inputs;
 //   - noise, symbols and biases of the CTA's own output positions stay in shared memory.
 // A pass ends with one exchange of change masks (64 bits, one per sample) between the CTAs.
@@ -61,7 +61,7 @@ struct ClShared {
     int first[2];
     uint4 flags[2][8];                       // per pass parity and CTA: change mask, smallest changed position
     int count[64];
-    int issued, consumed;                    // weight loads
+    int issued[2], consumed[2];              // weight loads, of even and of odd K blocks
     unsigned tiles;
     unsigned sums[2];                        // of the whole cluster (in its first CTA): tiles, K blocks
     float bias_s[CL_MAXL + 1][MAXOWN][TM];
@@ -202,19 +202,24 @@ struct ClEngine {
             }
         }
     }
-    // the ring stage `off` positions on, and the parity of its use there
-    __device__ __forceinline__ void ring_at(int st, uint32_t ph, int off, int &s, uint32_t &p) const
+    // The weight ring is two: even K blocks of every tile take the stages 0, 2, 4 .., odd ones 1, 3, 5 .., in turn, because each
+    // half has a consumer of its own.  In one ring for both, a consumer could look at a stage whose former occupant, the other
+    // consumer's, had not even arrived (loads overtake one another), and a parity cannot tell that phase from the one after the
+    // next: it took the stage for full.  In its own ring it has consumed every former occupant itself.
+    // Stage `off` positions on in ring `half`, and the parity of its use there.
+    __device__ __forceinline__ void ring_at(int half, int st, uint32_t ph, int off, int &s, uint32_t &p) const
     {
-        s = st + off;
+        int q = st + off;
         p = ph;
-        while (s >= S) { s -= S; p ^= 1u; }
+        while (q >= (S >> 1)) { q -= S >> 1; p ^= 1u; }
+        s = 2 * q + half;
     }
 
     // ---------------------------------------------------------------- roles
     __device__ void producer(bool jacobi)
     {
-        int n = 0, st = 0;
-        uint32_t ph = 0;
+        int n0 = 0, n1 = 0, st0 = 0, st1 = 0;    // per ring: loads so far, next stage, parity of its use
+        uint32_t ph0 = 0, ph1 = 0;
         bool on = true;
         const uint32_t ring0 = smem_u32(ring);
         for (unsigned pass = 0; on; ++pass) {
@@ -233,24 +238,31 @@ struct ClEngine {
                     for (int kb = 0; kb < o.y;) {
                         int s;
                         uint32_t p;
-                        ring_at(st, ph, lane, s, p);
+                        const int h = (kb + lane) & 1;
+                        ring_at(h, h ? st1 : st0, h ? ph1 : ph0, lane >> 1, s, p);      // (as many of this half lie between)
                         const bool look = lane < S && kb + lane < o.y;
                         const int run = wait_run([&] { return look && mbar_test_wait(&sh.empty[s], p ^ 1u); }, jacobi);
                         if (run == 0) { on = false; break; }
                         for (int i = 0; i < run; ++i, ++kb, row += cd.npad[l]) {
+                            const int half = kb & 1, st = 2 * (half ? st1 : st0) + half;
                             if (elect_one()) {
                                 mbar_expect_tx(&sh.full[st], STAGE);
                                 tma_load_2d(ring0 + (uint32_t)st * STAGE, map, &sh.full[st], 0, row);
                             }
-                            ++n;
-                            if (++st == S) { st = 0; ph ^= 1u; }
+                            if (half) {
+                                ++n1;
+                                if (++st1 == (S >> 1)) { st1 = 0; ph1 ^= 1u; }
+                            } else {
+                                ++n0;
+                                if (++st0 == (S >> 1)) { st0 = 0; ph0 ^= 1u; }
+                            }
                         }
                     }
                 }
             }
             if (!jacobi && lane == 0) mbar_arrive(&sh.ack);
         }
-        if (lane == 0) sh.issued = n;
+        if (lane == 0) { sh.issued[0] = n0; sh.issued[1] = n1; }
     }
 
     // half 0 issues the even K blocks of every tile, half 1 the odd ones
@@ -261,7 +273,7 @@ struct ClEngine {
         uint64_t apar[CL_MAXL + 2];              // parity of the next completion of every K block's barrier; x: two sets
 #pragma unroll
         for (int l = 0; l < CL_MAXL + 2; ++l) apar[l] = 0;
-        int n = 0, slot = 0, st = 0;             // st, ph: ring position of the tile's first K block
+        int n = 0, slot = 0, st = 0;             // st, ph: position in this half's ring of its first K block of the tile
         uint32_t ph = 0, spar = 0;               // spar: parity of the accumulator slots' next use
         bool on = true;
         unsigned tiles = 0;
@@ -288,8 +300,8 @@ struct ClEngine {
                         const int lk = kb + 2 * lane;
                         int s;
                         uint32_t p;
-                        const bool look = lk < o.y && lk < kb + S;
-                        ring_at(st, ph, look ? lk : 0, s, p);
+                        const bool look = lk < o.y && lane < (S >> 1);
+                        ring_at(half, st, ph, look ? lk >> 1 : 0, s, p);
                         const bool isfresh = look && in(fr, lk);
                         uint64_t *ab = block_bar(l, look ? lk : 0, pass);
                         const uint32_t abp = (uint32_t)(ap >> (look ? lk : 0)) & 1u;
@@ -302,7 +314,7 @@ struct ClEngine {
                                 const int kc = kb + 2 * i;
                                 int cs;
                                 uint32_t cp;
-                                ring_at(st, ph, kc, cs, cp);
+                                ring_at(half, st, ph, kc >> 1, cs, cp);
                                 const uint64_t ad = ring_desc + (uint64_t)(cs * (STAGE >> 4)), bd = act_desc + (uint64_t)(kc * (int)(blk_bytes >> 4));
 #pragma unroll
                                 for (int k = 0; k < BK / 16; ++k)
@@ -315,9 +327,10 @@ struct ClEngine {
                     }
                     if (!on) break;
                     if (elect_one()) umma_commit(&sh.tfull[slot]);      // (with no K block of its own too: all its earlier MMAs are done)
-                    n += o.y;
-                    st += o.y;
-                    while (st >= S) { st -= S; ph ^= 1u; }
+                    const int mine = (o.y + 1 - half) >> 1;
+                    n += mine;
+                    st += mine;
+                    while (st >= (S >> 1)) { st -= S >> 1; ph ^= 1u; }
                     spar ^= 1u << slot;
                     slot = (slot + 1) % NSLOT;
                 }
@@ -328,9 +341,9 @@ struct ClEngine {
             }
             if (lane == 0) mbar_arrive(&sh.ack);
         }
-        if (half == 0 && lane == 0) {
-            sh.consumed = n;
-            sh.tiles = tiles;
+        if (lane == 0) {
+            sh.consumed[half] = n;
+            if (half == 0) sh.tiles = tiles;
         }
     }
 
@@ -650,7 +663,7 @@ made_cluster_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ C
         mbar_init(&sh.go, 1);
         mbar_init(&sh.ack, jacobi ? 2 : 3);
         sh.stop = sh.dead = 0;
-        sh.issued = sh.consumed = 0;
+        for (int h = 0; h < 2; ++h) sh.issued[h] = sh.consumed[h] = 0;
         sh.tiles = sh.sums[0] = sh.sums[1] = 0;
         for (int i = 0; i < 2; ++i) { sh.chg[i][0] = sh.chg[i][1] = 0; sh.first[i] = INT_MAX; }
     }
@@ -733,7 +746,9 @@ made_cluster_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ C
     __syncthreads();
     const bool alive = sh.dead == 0 && ld_volatile_i32(&r.ctl->abort) == 0;
     if (tid == 0 && alive)                   // weights that ran ahead: let them land
-        for (int n = sh.consumed; n < sh.issued; ++n) e.wait(&sh.full[n % cd.n_stages], (uint32_t)(n / cd.n_stages) & 1u);
+        for (int h = 0; h < 2; ++h)
+            for (int n = sh.consumed[h], q = cd.n_stages >> 1; n < sh.issued[h]; ++n)
+                e.wait(&sh.full[2 * (n % q) + h], (uint32_t)(n / q) & 1u);
     // results: symbols of the own positions, counts
     if (warp >= 2 && warp < 6 && alive) {
         const int u = (warp & 3) * 16 + (lane & 15);
@@ -748,7 +763,7 @@ made_cluster_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ C
     }
     if (tid == 0) {
         peer_add(peer_addr(smem_u32(&sh.sums[0]), 0), sh.tiles);
-        peer_add(peer_addr(smem_u32(&sh.sums[1]), 0), (unsigned)sh.consumed);
+        peer_add(peer_addr(smem_u32(&sh.sums[1]), 0), (unsigned)(sh.consumed[0] + sh.consumed[1]));
     }
     if (!alive)
         for (int i = 0; i < 2000; ++i) __nanosleep(1000);      // copies still in flight land before shared memory goes away
@@ -859,7 +874,7 @@ static int cluster_rows(const js_model *mo, int batch, int *n_stages)
     const ClusterDev &c = mo->cluster;
     const int want = std::min(64, ((batch + c.max_clusters - 1) / c.max_clusters + 7) / 8 * 8);
     for (int R = want; R >= 8; R -= 8)
-        for (int st = MAX_STAGES; st >= 4; --st)
+        for (int st = MAX_STAGES; st >= 4; st -= 2)            // (two rings of half as many)
             if (cluster_smem(c, mo->made, R, st) <= SMEM_MAX) {
                 *n_stages = st;
                 return R;
