@@ -235,6 +235,15 @@ def run_reference(args, cfg):
 NOMINAL = {"bf16_tflops": 2250.0, "hbm_gbs": 7700.0}      # data-sheet figures, for context beside the measured peaks
 
 
+def made_kernel_name(cfg, stats):
+    """Which kernel serves a Jacobi call of this masked MLP: the rules of the library (js_cluster_serves, js_small_serves),
+    as far as the workloads here need them."""
+    widest = max([cfg.D, *cfg.H])
+    if stats.path == 0:
+        return "made_cluster_kernel" if cfg.C == 1 and len(cfg.H) <= 3 and widest <= 1024 else "made_tc_kernel"
+    return "made_small_kernel" if cfg.prec == si.PREC_F32 and cfg.C <= 2 and widest <= 256 else "made_generic_kernel"
+
+
 def roofline_of(cfg, stats, it_np, ms_launch, peaks):
     """Roofline record of one call.  Algorithmic work counts only what the method needs: the live
     (unmasked) multiply-accumulates of a forward pass for every sample that was still iterating in that
@@ -247,7 +256,7 @@ def roofline_of(cfg, stats, it_np, ms_launch, peaks):
     noise_per_sample = cfg.D * (cfg.C if cfg.noise_kind == si.NOISE_GUMBEL else 1) * 4
     wbytes = float(stats.weight_bytes) if stats.weight_bytes > 0 else 2.0 * live * stats.iterations
     nbytes = wbytes + (noise_per_sample + 2.0 * cfg.D) * sample_passes
-    kernel_name = "conv_tc_kernel" if cfg.kind == "conv" else ("made_tc_kernel" if stats.path == 0 else "made_generic_kernel")
+    kernel_name = "conv_tc_kernel" if cfg.kind == "conv" else made_kernel_name(cfg, stats)
     ridge = peaks["bf16_tflops"] * 1e12 / (peaks["hbm_gbs"] * 1e9)
     sec = ms_launch / 1e3
     if flops / nbytes >= ridge:

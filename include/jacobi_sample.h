@@ -192,7 +192,9 @@ typedef enum {
     JS_OPT_PATH = 3,           /* 0 (default): tensor-core kernels where the model allows; 1: CUDA-core kernels only */
     JS_OPT_COMPACT = 4,        /* 1 (default): move finished samples out of the working batch */
     JS_OPT_TRACE = 5           /* 0 (default); 1: record device timestamps of the next calls (js_get_trace) for the
-                                  first and the last CTA; n >= 2: for the first CTA and CTA n - 2 */
+                                  first and the last CTA; n >= 2: for the first CTA and CTA n - 2.  Binary bf16 models that
+                                  are otherwise solved in groups of samples, a cluster each (a kernel without a timeline), go to
+                                  the grid-wide tensor-core kernel while it is on: the same samples, another time */
 } js_option;
 int js_set_option(js_model *m, int option, int value);
 

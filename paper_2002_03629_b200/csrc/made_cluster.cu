@@ -890,9 +890,9 @@ bool js_cluster_serves(const js_model *mo, const RunArgs &r)
     int st = 0;
     const int R = cluster_rows(mo, r.batch, &st);
     if (R == 0) return false;
-    // A CTA streams its share of the weights every pass, 0.22 us per K block where the ring is short of room: measured at
-    // 4 passes of T = 1936, H = 2048 x 3 (259 K blocks): 262 us against 246 us grid-wide; T = 1296, H = 2048 x 2 (150): 170
-    // against 222 us.
+    // A CTA streams its share of the weights every pass, whatever the batch.  T and H = 2048 x 3, 16 and 64 samples, us here
+    // and grid-wide: T = 1024 (204 K blocks) 132 and 162, 132 and 165; 1296 (226) 148 and 170, 149 and 174; 1600 (241) 163 and
+    // 172, 164 and 175; 1936 (264) 186 and 173, 241 and 226.
     return mo->cluster.kblocks <= 230 && (r.batch + R - 1) / R <= std::min(JS_MAX_CLUSTERS, mo->cluster.max_clusters);
 }
 

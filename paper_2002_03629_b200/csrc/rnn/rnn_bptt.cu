@@ -103,8 +103,11 @@ struct Count {
 //   2  l_t and derivative to global memory                       3  input part W_x x + b of the next step of the chain
 // One block barrier per iteration keeps the groups together.  With all of it between two steps of the chain a step took
 // 0.57 us; with every warp of the second group doing a quarter of each kind of work in every iteration, 0.8 us.
-// T = 100, H = 128 (B200): batch 1 86 -> 41 us, batch 592 209 -> 140 us.
-// NS sequences per CTA: the weights in registers serve NS independent chains, whose latencies overlap.
+// T = 100, H = 128, one input and output (B200): batch 1 86 -> 40 us, batch 592 209 -> 118 us; 16 inputs and outputs, T = 128:
+// 200 -> 132 and 613 -> 326 us.
+// NS sequences per CTA: the weights in registers serve NS independent chains, whose latencies overlap.  MANY: sums of several
+// outputs go through the shuffles side by side; for one output and few inputs the plain loop is the shorter step (T = 100,
+// batch 1: 40 us against 46; two outputs 52 against 48).
 template <int NS, bool VEC, bool MANY>
 __global__ void __launch_bounds__(2 * CT, 1)
 rnn_forward_kernel(const float *__restrict__ Wh, const float *__restrict__ Wx, const float *__restrict__ b,
