@@ -3,10 +3,8 @@
 // iterations (Algorithm 1) and the parameter gradients.  fp32 fused multiply-adds in a fixed order.
 //
 // Forward pass and back-substitution are chains of T matrix-vector products: what counts is the latency of one
-// step, so a step is spread over four threads per component (see the kernels).  A Jacobi iteration has parallel slack,
-// all T states at once, a [T x H] x [H x H] product per iteration: a register-tiled product out of shared memory in
-// which the iterate (premultiplied by the activation derivative and shifted by one step) and the weights stay; a small
-// batch shares each sequence among the CTAs of a cluster, which hand over one row per iteration.
+// step, so a step is spread over four threads per component (see the kernels).  A Jacobi iteration is a product for all T
+// states at once, [T x H] x [H x H]: it runs on the tensor cores, in pieces of bf16 that add up to fp32.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -15,6 +13,7 @@
 #include <cstdio>
 
 #include "../../../include/rnn_bptt.h"
+#include "../tc_common.cuh"
 
 namespace {
 
@@ -353,174 +352,432 @@ rnn_bptt_sequential_kernel(const float *__restrict__ Wh, const float *__restrict
 }
 
 // ------------------------------------------------------------------ Jacobi iterations
-// A sequence is solved by a cluster of csz CTAs (1 where the batch fills the GPU); CTA c owns the steps
-// [c rpc, (c + 1) rpc).  V[k][r] = d_{t+1}[k] * s_{t+1}[k] of the current iterate for t = c rpc + r (zero where t + 1 >= T
-// or k >= H), so that  s_new[t][i] = l[t][i] + sum_k V[k][r] * W_h[k][i];  the value of a CTA's first step belongs to the
-// CTA before it.  A thread owns a tile of 4 steps x 8 components.  Neighbouring lanes take the same columns and
-// neighbouring tile rows: a 16-byte shared-memory load then takes two cycles for a warp instead of the four it takes when
-// neighbouring lanes read sixteen pieces of a weight row, and the product is bound by its multiply-adds (8 cycles per
-// warp and k against 6).  Steps are laid out without padding to 128, for which 100 steps paid 28 %.  Row k of V starts at
-// vrow(k): the four floats of slack after every fourth row spread the transposed stores over the banks.
-// Three forms:
-//   JAC_PAIR   two sequences per CTA, each with its own threads and its own (named) barrier, for batches beyond one per
-//              SM: one sequence's stores and waits pass while the other multiplies, and 26 warps balance better over
-//              four schedulers than 13.  One buffer for V, refilled between two barriers.
-//   JAC_ONE    one sequence per CTA, two buffers.
-//   JAC_SPLIT  one sequence per cluster: a CTA has so few steps that the k range is cut into four parts for as many
-//              thread groups; part p adds the four sums of every tile's row p (in order) and finishes it.
-// After k iterations the last k states are final (Proposition 1), and a repeated evaluation would give the same bits:
-// they are stored when they become final and not computed again; their warps drop out.
-// Bound: issue of fp32 multiply-adds (a plain FFMA loop reaches 61 TFLOP/s on this GPU).  T = 100, H = 128, 20 iterations:
-// batch 1 285 -> 73 us (cluster of 8), batch 592 1148 -> 895 us (40 TFLOP/s of what is still computed).
-enum { JAC_PAIR = 0, JAC_ONE = 1, JAC_SPLIT = 2 };
+// On the tensor cores.  An iteration is a product with the recurrent weights for all steps at once,
+//     s_new[t][i] = l[t][i] + sum_k U[t + 1][k] * W_h[k][i],   U[t][k] = d[t][k] * s[t][k],
+// computed transposed: D[i][c] = sum_k A[i][k] * B[k][c] with A = W_h^T, 128 x 128, constant, in tensor memory, and the iterate U in
+// shared memory.  Column c of a CTA's unit is step t = c % T of its sequence c / T (a unit is one sequence, or as many whole
+// ones as 128 columns hold): as the steps of a batch lie one after another in memory, so do the columns, and U, taken as
+// zero at t = 0, keeps a sequence from reaching into the one before it.
+// fp32 values are cut into three bf16 pieces (8 + 8 + 8 bits; what is left is below 2^-26 of the value) and the six products
+// of pieces down to 2^-18 are summed.  The tensor core rounds its running sums towards zero, so the five small products
+// come first, while the sum is small, and the large one, high by high, is shared by two accumulators: four steps of full size each.
+//   warps 0-7   epilogue: thread = (component i, JC columns of each slot); l and d of these stay in registers, s = l + D, U goes back to
+//               shared memory as three pieces, eight columns (16 bytes) a store.  JC = 32; up to 64 components the rows of A lie
+//               in tensor memory twice, so that all eight warps find work: 16 columns each
+//   warps 8, 9  MMA, a slot each (their warpgroup hands its registers to the others)
+// The columns go in two slots of up to 64, each with accumulators of its own: one slot's MMAs run while the other's epilogue
+// does.  A slot's last column takes its sum from the first column of the slot behind it, which is therefore the first in every round.
+// l and d of the next unit come into shared memory (bulk copies, where the pointers lie on 16 bytes) while this one is worked on.
+// Values that three pieces cannot carry (infinities, NaN, or so large that a piece overflows) show as non-finite
+// states: such a unit is computed again with plain multiply-adds before anything of it is stored.
+// Bound: at 65 to 128 components the MMAs, 96 of 17 to 32 cycles an iteration (1.6 us of the 1.7 measured for 100 steps of 128
+// components; multiply-adds on the CUDA cores, 40 TFLOP/s, took 10); below that the way from a slot's last product to its next
+// first one (0.3 us of waits, 0.3 to 0.6 of epilogue).  T = 100, H = 128, 20 iterations: batch 1 71 -> 44 us, batch 592 894 -> 163 us;
+// T = 50, H = 64, 10 iterations, batch 300: 61 -> 28 us.  Against 64 bits the states are off by 1.0e-7 (2-norm), 1.1e-7 to 3.4e-7 before.
+constexpr int JE = 256, JTH = JE + 128;      // epilogue threads, all threads
+constexpr int J_SLOT = 64;                   // columns of a slot
+constexpr int J_PIECE = MH * J_SLOT * 2;     // bytes of one piece of a slot's operand: [128 k][64 columns], 128-byte swizzle
+constexpr size_t J_OPS = 6 * J_PIECE;        // then l and d of a unit, [columns][H] each
+constexpr uint32_t J_DCOL = 3 * (MH / 2);    // tensor memory: three pieces of A, then per slot the two accumulators
 
-__device__ __forceinline__ void cluster_barrier()
+struct JacShared {
+    uint64_t ready[2], full[2];              // the slot's operand is there; its products are
+    uint32_t tmem;
+    uint64_t staged;                         // the unit's l and d are in shared memory
+    int dead;                                // a wait gave up
+};
+
+// D[tmem] (+)= A[tmem] * B[smem], 128 x N x 16
+__device__ __forceinline__ void umma_ts_bf16(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, bool accumulate)
 {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+                 ::"r"(d), "r"(a), "l"(b), "r"(idesc), "r"((uint32_t)accumulate) : "memory");
 }
-__device__ __forceinline__ int vrow(int k, int VS) { return k * VS + (k & ~3); }
-
-template <int FORM, int NT, bool VEC>
-__global__ void __launch_bounds__(NT, 1)
-rnn_bptt_jacobi_kernel(const float *__restrict__ Wh, const float *__restrict__ l, const float *__restrict__ d,
-                       int B, int T, int H, int n_iters, const float *__restrict__ s0, float *__restrict__ s, int csz, int rpc)
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16])
 {
-    constexpr int TR = 4, KS = FORM == JAC_SPLIT ? TR : 1, NSQ = FORM == JAC_PAIR ? 2 : 1;
-    constexpr bool DB = FORM != JAC_PAIR;
-    extern __shared__ __align__(16) float sm[];
-    const int tid = threadIdx.x, nth = blockDim.x;
-    const int seq0 = blockIdx.x / csz * NSQ, c = FORM == JAC_SPLIT ? blockIdx.x % csz : 0;
-    const int NG = (H + 7) / 8, VS = (rpc + 3) / 4 * 4, VB = H * (VS + 1);      // VB: one buffer of a sequence's iterate
-    float *W = sm;                                       // [H][MH]: component 4 ig + e at 4 ig + e, 4 (ig + NG) + e at 64 + 4 ig + e
-    float *V = sm + (size_t)H * MH;                      // [NSQ][1 or 2][VB]
-    float *part = V + (size_t)(NSQ * (DB ? 2 : 1)) * VB; // JAC_SPLIT: [4 parts][4 rows][8][threads of a part]
-    const int t0 = c * rpc, nr = max(0, min(rpc, T - t0));
-    for (int p = tid; p < NSQ * (DB ? 2 : 1) * VB; p += nth) V[p] = 0.0f;
-    for (int p = tid; p < H * 2 * NG; p += nth) {
-        const int k = p / (2 * NG), g = p - k * 2 * NG;
-        *reinterpret_cast<float4 *>(W + (size_t)k * MH + (g < NG ? 4 * g : 64 + 4 * (g - NG))) =
-            4 * g < H ? ldg4<VEC>(Wh + (size_t)k * H + 4 * g) : make_float4(0, 0, 0, 0);
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
+                   "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+                 : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ uint32_t tmem_ld1(uint32_t taddr)
+{
+    uint32_t r;
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(taddr) : "memory");
+    return r;
+}
+__device__ __forceinline__ void tmem_st4(uint32_t taddr, const uint32_t (&r)[4])
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
+}
+__device__ __forceinline__ void sts4(uint32_t at, const uint32_t (&r)[4])
+{
+    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
+}
+// two values in three bf16 pieces each, packed (the first in the low half)
+__device__ __forceinline__ void cut3(float a, float b, uint32_t &h, uint32_t &m, uint32_t &l)
+{
+    h = pack_bf16x2(a, b);
+    a -= __uint_as_float(h << 16);
+    b -= __uint_as_float(h & 0xffff0000u);
+    m = pack_bf16x2(a, b);
+    a -= __uint_as_float(m << 16);
+    b -= __uint_as_float(m & 0xffff0000u);
+    l = pack_bf16x2(a, b);
+}
+// bounded: true once the barrier's phase has completed, false after 2 s or when another wait of the CTA has given up
+__device__ __forceinline__ bool jac_wait(JacShared &sh, uint64_t *bar, uint32_t parity)
+{
+    if (mbar_try_wait(bar, parity)) return true;
+    const uint64_t t0 = global_ns();
+    for (unsigned i = 1;; ++i) {
+        if (mbar_try_wait(bar, parity)) return true;
+        if ((i & 63u) == 0u && (*(volatile int *)&sh.dead || global_ns() - t0 > MBAR_WAIT_NS)) break;
     }
-    if (n_iters <= 0) {
-        for (int n = 0; n < NSQ && seq0 + n < B; ++n)
-            for (int p = tid; p < nr * H; p += nth) {
-                const size_t at = (size_t)(seq0 + n) * T * H + (size_t)t0 * H + p;
-                s[at] = s0 != nullptr ? s0[at] : 0.0f;
-            }
-        return;                                          // every CTA of the cluster leaves here
+    *(volatile int *)&sh.dead = 1;
+    return false;
+}
+// barrier of the epilogue warps: did every thread say yes?
+__device__ __forceinline__ bool jac_all(bool ok)
+{
+    int all;
+    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %1, 0;\n\tbar.red.and.pred q, 1, 256, p;\n\tselp.b32 %0, 1, 0, q;\n\t}" : "=r"(all) : "r"((int)ok) : "memory");
+    return all != 0;
+}
+
+// One sequence by plain multiply-adds, thread = component, U in shared memory.  Steps in ascending order: step t reads U[t + 1], not yet
+// overwritten, and then replaces U[t], which nobody reads any more.
+__device__ __forceinline__ void jac_plain(const float *Wh, const float *l, const float *d, int T, int H, int iters, const float *s0, float *s,
+                                          float *U, int tid)
+{
+    for (int p = tid; p < T * MH; p += JE) {
+        const int t = p / MH, k = p % MH;
+        U[p] = k < H && s0 != nullptr ? d[t * H + k] * s0[t * H + k] : 0.0f;
     }
-    // thread = (sequence n or part ks, tile row tg, column group ig); a sequence's threads are whole warps
-    const int tgs = ((rpc + TR - 1) / TR + 1) / 2 * 2, per_seq = tgs * NG;
-    const int grp = FORM == JAC_ONE ? nth : nth / (NSQ * KS), gi = FORM == JAC_ONE ? 0 : tid / grp, ti = tid - gi * grp;
-    const int n = FORM == JAC_PAIR ? gi : 0, ks = FORM == JAC_SPLIT ? gi : 0;
-    const int ig = (ti >> 1) % NG, tg = (ti >> 1) / NG * 2 + (ti & 1), r0 = tg * TR;
-    const bool here = ti < per_seq && seq0 + n < B;
-    const float *lp = l + (size_t)(seq0 + n) * T * H, *dp = d + (size_t)(seq0 + n) * T * H;
-    float *sp = s + (size_t)(seq0 + n) * T * H;
-    float *Vn = V + n * VB;
-    __syncthreads();
-    if (s0 != nullptr)
-        for (int m = 0; m < NSQ && seq0 + m < B; ++m)
-            for (int p = tid; p < nr * H; p += nth) {
-                const int r = p / H, k = p - r * H, t = t0 + r + 1;
-                const size_t at = (size_t)(seq0 + m) * T * H + (size_t)t * H + k;
-                if (t < T) V[m * VB + vrow(k, VS) + r] = d[at] * s0[at];
-            }
-    // the CTA before this one: where the value of our first step goes
-    uint32_t prev = 0;
-    if (FORM == JAC_SPLIT && c > 0) {
-        const uint32_t mine = (uint32_t)__cvta_generic_to_shared(Vn);
-        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(prev) : "r"(mine), "r"(c - 1));
-    }
-    auto load4 = [&](const float *src, int r, int hf) {          // l or d of step t0 + r, components 4 (ig + hf NG) ..
-        const int i = 4 * (ig + hf * NG);
-        return r < nr && i < H ? ldg4<VEC>(src + (size_t)(t0 + r) * H + i) : make_float4(0, 0, 0, 0);
+#pragma unroll 1
+    for (int it = 0; it < iters; ++it)
+#pragma unroll 1
+        for (int t = 0; t < T; ++t) {
+            jac_all(true);
+            if (tid >= H) continue;
+            const int at = t * H + tid;
+            float acc = l[at];
+            if (t + 1 < T)
+#pragma unroll 4
+                for (int k = 0; k < H; ++k) acc = fmaf(U[(t + 1) * MH + k], Wh[k * H + tid], acc);
+            if (it + 1 == iters) s[at] = acc;
+            else U[t * MH + tid] = d[at] * acc;
+        }
+    jac_all(true);
+}
+
+// MANY: units of several sequences
+template <int JC, bool MANY>
+__global__ void __launch_bounds__(JTH, 1)
+rnn_bptt_jacobi_kernel(const float *__restrict__ Wh, const float *l, const float *d, int B, int T, int H, int iters, const float *s0, float *s,
+                       int per_unit)
+{
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ JacShared sh;
+    uint8_t *ops = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);   // [slot][piece]
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    constexpr int ROWS = MH * JC / 32, G = J_SLOT / JC;              // rows of A before they repeat, groups of columns
+    const int row = (warp & 3) * 32 + lane;                                  // epilogue: tensor memory lane,
+    const int i = row % ROWS, g = (warp >> 2) * (G / 2) + row / ROWS;        // component, group of columns
+    const uint32_t quad = (uint32_t)((warp & 3) * 32) << 16;
+    const int width = per_unit * T;                                          // columns of a unit
+    const bool two = width > J_SLOT;
+    const int units = (B + per_unit - 1) / per_unit, nk = (H + 15) / 16;
+    // the columns of a slot that its MMAs compute
+    auto slot_columns = [&](int k) { return max(0, min(J_SLOT, width - k * J_SLOT) + 15) / 16 * 16; };
+    float *const ls = reinterpret_cast<float *>(ops + J_OPS), *const ds = ls + width * H;
+    const bool stages = ((reinterpret_cast<uintptr_t>(l) | reinterpret_cast<uintptr_t>(d)) & 15u) == 0;
+    auto stage = [&](int u) {
+        if (u >= units || !stages) return;
+        const uint32_t bytes = (uint32_t)(min(width, (B - u * per_unit) * T) * H) * 4u;
+        const size_t from = (size_t)u * per_unit * T * H;
+        mbar_expect_tx(&sh.staged, 2 * bytes);
+        bulk_load(smem_u32(ls), l + from, bytes, &sh.staged);
+        bulk_load(smem_u32(ds), d + from, bytes, &sh.staged);
     };
-    float4 lk[2], dk[2];                                 // JAC_SPLIT: l and d of this part's row
-    if (FORM == JAC_SPLIT && here)
+    if (tid == 0) {
+        for (int k = 0; k < 2; ++k) { mbar_init(&sh.ready[k], JE / 32); mbar_init(&sh.full[k], 1); }
+        mbar_init(&sh.staged, 1);
+        sh.dead = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        stage(blockIdx.x);
+    }
+    if (warp == 8) tmem_alloc(&sh.tmem, 512);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tm = sh.tmem;
+    const int nmma = iters - (s0 == nullptr ? 1 : 0);                        // from zero the first iteration gives l
+    bool fine = true;                                                        // this thread's weights are finite
+    if (warp < 8) {
+        float chk = 0.0f;
+#pragma unroll 4
+        for (int c4 = 0; c4 < 8; ++c4) {                                     // 32 words of every piece, 64 k
+            const int k0 = (warp >> 2) * 64 + c4 * 8;
+            if (k0 >= nk * 16) break;
+            uint32_t ph[4], pm[4], pl[4];
+            float w[8];
 #pragma unroll
-        for (int hf = 0; hf < 2; ++hf) { lk[hf] = load4(lp, r0 + ks, hf); dk[hf] = load4(dp, r0 + ks, hf); }
-    if (FORM == JAC_SPLIT) cluster_barrier();
-    else __syncthreads();
-    const int iters = min(n_iters, T), kc = (H / 4 + KS - 1) / KS * 4;     // k per part (H is a multiple of 4)
-    const int k0 = ks * kc, k1 = min(H, k0 + kc);
-    for (int it = 0; it < iters; ++it) {
-        const int cur = DB ? (it & 1) * VB : 0, nxt = DB ? VB - cur : 0;
-        const int live = min(nr, T - it - t0);           // steps beyond are final
-        const bool work = here && r0 < live;             // (pairs of tile rows drop out of the warps together)
-        const bool last = it + 1 == iters;
-        // a finished row: to global memory when it is final, to the next iterate unless this was the last iteration
-        auto finish = [&](int r, const float (&v)[8], const float4 (&dv)[2]) {
-            const int t = t0 + r;
-#pragma unroll
-            for (int hf = 0; hf < 2; ++hf) {
-                const int i = 4 * (ig + hf * NG);
-                if (i >= H) continue;
-                if (last || t == T - 1 - it)
-                    stg4<VEC>(sp + (size_t)t * H + i, make_float4(v[4 * hf], v[4 * hf + 1], v[4 * hf + 2], v[4 * hf + 3]));
-                if (last) continue;
-                const float dd[4] = {dv[hf].x, dv[hf].y, dv[hf].z, dv[hf].w};
-                const int row = nxt + vrow(i, VS);
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const float val = dd[e] * v[4 * hf + e];
-                    if (r >= 1) Vn[row + e * VS + r - 1] = val;
-                    else if (FORM == JAC_SPLIT && c > 0)
-                        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(prev + 4u * (uint32_t)(row + e * VS + rpc - 1)), "f"(val) : "memory");
-                }
+            for (int e = 0; e < 8; ++e) {
+                w[e] = k0 + e < H && i < H ? __ldg(Wh + (k0 + e) * H + i) : 0.0f;
+                chk = fmaf(w[e], 0.0f, chk);
             }
-        };
-        float acc[TR][8];
-        if (work) {
 #pragma unroll
-            for (int rr = 0; rr < TR; ++rr)
-#pragma unroll
-                for (int hf = 0; hf < 2; ++hf) {
-                    const float4 a = FORM == JAC_SPLIT ? make_float4(0, 0, 0, 0) : load4(lp, r0 + rr, hf);
-                    acc[rr][4 * hf] = a.x; acc[rr][4 * hf + 1] = a.y; acc[rr][4 * hf + 2] = a.z; acc[rr][4 * hf + 3] = a.w;
-                }
-            const float *vp = Vn + cur + r0 + vrow(k0, VS), *wp = W + 4 * ig + (size_t)k0 * MH;
-            for (int k = k0; k < k1; k += 4, vp += 4 * VS + 4, wp += 4 * MH)
-#pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {
-                    const float4 a = *reinterpret_cast<const float4 *>(vp + kk * VS);
-                    const float4 w0 = *reinterpret_cast<const float4 *>(wp + kk * MH);
-                    const float4 w1 = *reinterpret_cast<const float4 *>(wp + kk * MH + 64);
-                    const float av[TR] = {a.x, a.y, a.z, a.w};
-                    const float wv[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
-#pragma unroll
-                    for (int rr = 0; rr < TR; ++rr)
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) acc[rr][e] = fmaf(av[rr], wv[e], acc[rr][e]);
-                }
-            if (FORM == JAC_SPLIT)
-#pragma unroll
-                for (int e = 0; e < 32; ++e) part[(ks * 32 + e) * grp + ti] = acc[e >> 3][e & 7];
+            for (int e = 0; e < 4; ++e) cut3(w[2 * e], w[2 * e + 1], ph[e], pm[e], pl[e]);
+            const uint32_t at = tm + quad + (uint32_t)(k0 / 2);
+            tmem_st4(at, ph);
+            tmem_st4(at + MH / 2, pm);
+            tmem_st4(at + MH, pl);
         }
-        if (FORM == JAC_SPLIT) {
-            __syncthreads();                             // the parts' sums are there
-            if (work && r0 + ks < live) {
-                float v[8] = {lk[0].x, lk[0].y, lk[0].z, lk[0].w, lk[1].x, lk[1].y, lk[1].z, lk[1].w};
-#pragma unroll
-                for (int p = 0; p < KS; ++p)
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) v[e] += part[(p * 32 + ks * 8 + e) * grp + ti];
-                finish(r0 + ks, v, dk);
-            }
-            cluster_barrier();
-        } else {
-            if (FORM == JAC_PAIR) asm volatile("bar.sync %0, %1;" ::"r"(1 + n), "r"(grp) : "memory");     // V has been read
-            if (work)
-#pragma unroll
-                for (int rr = 0; rr < TR; ++rr)
-                    if (r0 + rr < live) {
-                        const float4 dv[2] = {load4(dp, r0 + rr, 0), load4(dp, r0 + rr, 1)};
-                        finish(r0 + rr, acc[rr], dv);
+        fine = chk == 0.0f;
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        tc_fence_before();
+    }
+    __syncthreads();
+    tc_fence_after();
+
+    if (warp >= 8) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");                 // 384 threads x 168 registers = 256 x 232 + 128 x 40
+        if (warp < 10) {
+            const int slot = warp - 8, cols = slot_columns(slot);
+            if (cols > 0) {
+                // B lies with neighbouring columns together ("MN-major": bit 16)
+                const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(MH >> 4) << 24) | ((uint32_t)(cols >> 3) << 17);
+                const uint32_t d0 = tm + J_DCOL + (uint32_t)(slot * 128), d1 = d0 + J_SLOT;
+                // swizzled, 64 columns a row of 128 bytes, groups of eight k rows 1024 bytes apart
+                const uint64_t bd = smem_desc_sw128(smem_u32(ops + (size_t)slot * 3 * J_PIECE)) | ((uint64_t)(1024 >> 4) << 16);
+                constexpr uint64_t PC = J_PIECE >> 4, K16 = 2048 >> 4;
+                uint32_t par = 0;
+                bool on = true;
+                for (int u = blockIdx.x; u < units && on; u += gridDim.x)
+                    for (int it = 0; it < nmma && on; ++it, par ^= 1u) {
+                        on = __all_sync(0xffffffffu, jac_wait(sh, &sh.ready[slot], par));
+                        if (!on) break;
+                        tc_fence_after();
+                        if (elect_one()) {
+                            // (rolled: straight-line code of 96 MMAs cost 10 us of instruction fetches in the first iterations)
+                            uint32_t a = tm;
+                            uint64_t b = bd;
+#pragma unroll 2
+                            for (int k = 0; k < nk; ++k, a += 8, b += K16) {
+                                umma_ts_bf16(d1, a + MH, b, idesc, k > 0);
+                                umma_ts_bf16(d1, a, b + 2 * PC, idesc, true);
+                                umma_ts_bf16(d1, a + MH / 2, b + PC, idesc, true);
+                                umma_ts_bf16(d1, a + MH / 2, b, idesc, true);
+                                umma_ts_bf16(d1, a, b + PC, idesc, true);
+                            }
+                            a = tm;
+                            b = bd;
+#pragma unroll 2
+                            for (int k = 0; k < nk; ++k, a += 8, b += K16) umma_ts_bf16(k < nk / 2 ? d1 : d0, a, b, idesc, k != nk / 2);
+                            umma_commit(&sh.full[slot]);
+                        }
+                        __syncwarp();
                     }
-            if (FORM == JAC_PAIR) asm volatile("bar.sync %0, %1;" ::"r"(1 + n), "r"(grp) : "memory");
-            else __syncthreads();
+            }
+        }
+    } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 232;");
+        uint32_t par = 0, staged_par = 0;
+        for (int u = blockIdx.x; u < units; u += gridDim.x) {
+            const int cols = min(width, (B - u * per_unit) * T);
+            const size_t base = (size_t)u * per_unit * T * H + i;
+            bool ok = true;
+            if (stages) ok = jac_wait(sh, &sh.staged, staged_par);
+            staged_par ^= 1u;
+            const float *lp = stages ? ls + i : l + base, *dp = stages ? ds + i : d + base;
+            float lv[2][JC], dv[2][JC], l0 = 0.0f;
+            uint32_t first[2];
+            // This thread's columns of slot k are 64 k + JC g + 1 + j, its operand columns one less; column 0 feeds nothing.
+            // (Row offsets are run along anew for every array: kept for all columns they would take 64 registers.)
+            auto rows = [&](int k, auto f) {
+                int step = H;
+                asm volatile("" : "+r"(step));
+                const int c0 = k * J_SLOT + g * JC + 1, left = i < H ? cols - c0 : 0;
+                int at = c0 * step;
+#pragma unroll
+                for (int j0 = 0; j0 < JC; j0 += 8) {
+                    if (j0 + 8 <= left) {
+#pragma unroll
+                        for (int j = j0; j < j0 + 8; ++j, at += step) f(j, at, true);
+                    } else {
+#pragma unroll
+                        for (int j = j0; j < j0 + 8; ++j, at += step) f(j, at, j < left);
+                    }
+                }
+            };
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                rows(k, [&](int j, int at, bool in) { lv[k][j] = in ? lp[at] : 0.0f; });
+                rows(k, [&](int j, int at, bool in) { dv[k][j] = in ? dp[at] : 0.0f; });
+                // first steps of the unit's other sequences: no U, not even of an infinite state
+                first[k] = 0;
+                if (MANY)
+                    for (int c = T; c < cols; c += T) {
+                        const int j = c - (k * J_SLOT + g * JC + 1);
+                        if (j >= 0 && j < JC) first[k] |= 1u << j;
+                    }
+            }
+            if (g == 0 && i < H) l0 = lp[0];
+            ok = jac_all(ok);                                                // everything has been read
+            if (tid == 0) stage(u + (int)gridDim.x);
+            const bool idle = (i & ~31) >= H;                                // no component of this warp's (and no k that the MMAs read)
+            // eight columns of the operand of slot k from their states: pieces of U = d s
+            auto put8 = [&](int k, int j0, const float (&v)[8]) {
+                uint32_t ph[4], pm[4], pl[4];
+                float w[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) w[e] = dv[k][j0 + e] * v[e];
+                if (MANY)
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) w[e] = first[k] >> (j0 + e) & 1u ? 0.0f : w[e];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) cut3(w[2 * e], w[2 * e + 1], ph[e], pm[e], pl[e]);
+                const uint32_t at = smem_u32(ops + (size_t)k * 3 * J_PIECE) + (uint32_t)(i * 128 + (((JC / 8 * g + (j0 >> 3)) ^ (i & 7)) << 4));
+                sts4(at, ph);
+                sts4(at + J_PIECE, pm);
+                sts4(at + 2 * J_PIECE, pl);
+            };
+            // this warp's part of the operand of slot k is written and its sums are read
+            auto hand_over = [&](int k) {
+                fence_proxy_async_smem();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&sh.ready[k]);
+            };
+            float edge = 0.0f;                                               // the last group's: column 64's sum
+            // A slot's sums to states: into the operand, or, in the last iteration, in place of l.  The last of a thread's columns is
+            // the first of the other thread's, or of the slot behind.
+            auto finish = [&](int k, bool last) {
+                const uint32_t at = tm + quad + J_DCOL + (uint32_t)(k * 128 + g * JC);
+                const int mine = slot_columns(k) - g * JC;                   // a multiple of 16
+                if (idle) return;
+                if (k == 1 && g == G - 1) {
+                    const uint32_t first = tm + quad + J_DCOL + 128u, e0 = tmem_ld1(first), e1 = tmem_ld1(first + J_SLOT);
+                    tmem_wait_ld();
+                    edge = __uint_as_float(e0) + __uint_as_float(e1);
+                }
+                if (mine <= 0) return;
+                // sixteen columns in hand, the next ones on their way
+                uint32_t a[JC / 16][16], b[JC / 16][16], an = 0, bn = 0;
+                tmem_ld16(at, a[0]);
+                tmem_ld16(at + J_SLOT, b[0]);
+                if (JC == 32) tmem_wait_ld();
+                if (JC == 32 && mine > 16) {
+                    tmem_ld16(at + 16, a[JC / 16 - 1]);
+                    tmem_ld16(at + J_SLOT + 16, b[JC / 16 - 1]);
+                }
+                if (g < G - 1 && mine > JC) { an = tmem_ld1(at + JC); bn = tmem_ld1(at + J_SLOT + JC); }
+                if (JC == 16) tmem_wait_ld();
+                auto sum = [&](int c) { return __uint_as_float(a[c >> 4][c & 15]) + __uint_as_float(b[c >> 4][c & 15]); };
+                auto beyond = [&] { return g < G - 1 ? __uint_as_float(an) + __uint_as_float(bn) : k == 0 ? edge : 0.0f; };
+                auto take = [&](int j0, float (&w)[8]) {
+                    if (last) {
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) lv[k][j0 + e] += w[e];
+                    } else {
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) w[e] += lv[k][j0 + e];
+                        put8(k, j0, w);
+                    }
+                };
+                float w[8];
+                if (g == 0 && k == 0 && last) l0 += sum(0);
+#pragma unroll
+                for (int e = 0; e < 8; ++e) w[e] = sum(1 + e);
+                take(0, w);
+#pragma unroll
+                for (int e = 0; e < 7; ++e) w[e] = sum(9 + e);
+                if constexpr (JC == 16) {
+                    w[7] = beyond();
+                    take(8, w);
+                } else {
+                    tmem_wait_ld();
+                    w[7] = mine > 16 ? sum(16) : 0.0f;                       // (a seventeenth column that is nobody's)
+                    take(8, w);
+                    if (mine > 16) {
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) w[e] = sum(17 + e);
+                        take(16, w);
+#pragma unroll
+                        for (int e = 0; e < 7; ++e) w[e] = sum(25 + e);
+                        w[7] = beyond();
+                        take(24, w);
+                    }
+                }
+            };
+            // the start: U of s0, or of the first iteration from zero, which gives l
+            if (nmma > 0) {
+#pragma unroll
+                for (int k = 1; k >= 0; --k) {
+                    if (k == 1 && !two) continue;
+                    float v[JC];
+                    if (s0 != nullptr) rows(k, [&](int j, int at, bool in) { v[j] = in ? (s0 + base)[at] : 0.0f; });
+#pragma unroll
+                    for (int j0 = 0; j0 < JC; j0 += 8) {
+                        if (idle || j0 >= slot_columns(k) - g * JC) break;
+                        float w[8];
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) w[j] = s0 != nullptr ? v[j0 + j] : lv[k][j0 + j];
+                        put8(k, j0, w);
+                    }
+                    hand_over(k);
+                }
+            }
+            for (int it = 0; it < nmma && ok; ++it, par ^= 1u) {
+                const bool last = it + 1 == nmma;
+#pragma unroll
+                for (int k = 1; k >= 0; --k) {
+                    if (k == 1 && !two) continue;
+                    ok = __all_sync(0xffffffffu, jac_wait(sh, &sh.full[k], par));
+                    if (!ok) break;
+                    tc_fence_after();
+                    finish(k, last);
+                    if (!last) hand_over(k);
+                }
+            }
+            // Non-finite anywhere?  (Whatever became non-finite on the way either shows here or has left at a first step.)
+            float chk = fine ? l0 * 0.0f : NAN;
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+#pragma unroll
+                for (int j = 0; j < JC; ++j) chk = fmaf(lv[k][j], 0.0f, chk);
+            const bool plain = !jac_all(chk == 0.0f);
+            ok = jac_all(ok);
+            if (!ok) {
+                // the MMAs did not end: nothing is known about the states
+                for (int c = g; c < cols; c += G)
+                    if (i < H) s[base + (size_t)c * H] = NAN;
+            } else if (plain) {
+                for (int q = 0; q < per_unit && u * per_unit + q < B; ++q) {
+                    const size_t o = (size_t)(u * per_unit + q) * T * H;
+                    jac_plain(Wh, l + o, d + o, T, H, iters, s0 != nullptr ? s0 + o : nullptr, s + o, reinterpret_cast<float *>(ops), tid);
+                }
+            } else if (i < H) {
+#pragma unroll
+                for (int k = 0; k < 2; ++k) rows(k, [&](int j, int at, bool in) { if (in) (s + base)[at] = lv[k][j]; });
+                if (g == 0) s[base] = l0;
+            }
         }
     }
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 8) {
+        tc_fence_after();
+        tmem_dealloc(tm, 512);
+    }
+}
+
+// n_iters == 0: the start iterate
+__global__ void rnn_copy_kernel(const float *s0, float *s, size_t n)
+{
+    for (size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (size_t)gridDim.x * blockDim.x) s[p] = s0 != nullptr ? s0[p] : 0.0f;
 }
 
 // ------------------------------------------------------------------ parameter gradients
@@ -625,8 +882,6 @@ rnn_param_grads_kernel(const float *__restrict__ s, const float *__restrict__ d,
 
 bool sizes_ok(int B, int T, int H) { return B >= 1 && T >= 1 && T <= MT && H >= 1 && H <= MH && H % 4 == 0; }
 
-constexpr size_t JACOBI_SMEM_MAX = (size_t)(2 * MH * (MT + 1) + MH * MH) * sizeof(float);
-
 int sm_count()
 {
     int dev = 0, sms = 0;
@@ -703,35 +958,20 @@ int rnn_bptt_jacobi(const float *Wh, const float *l, const float *d, int B, int 
                     float *s, void *stream)
 {
     if (!Wh || !l || !d || !s || !sizes_ok(B, T, H) || n_iters < 0) return RNN_ERR_INVALID;
-    // CTAs per sequence: 15 clusters of 8 or 33 of 4 fit the GPU at a time, and two rounds of 4 still beat whole sequences
-    // on single CTAs; shares of fewer than eight steps would be mostly barriers
     const int sms = sm_count();
-    int csz = B <= 15 && T >= 64 ? 8 : B <= 66 && T >= 32 ? 4 : 1;
-    const int rpc = (T + csz - 1) / csz, NG = (H + 7) / 8, VS = (rpc + 3) / 4 * 4;
-    const int grp = (((rpc + 3) / 4 + 1) / 2 * 2 * NG + 31) / 32 * 32;       // threads of a sequence's share
-    // Pairs where an even number of rounds of one sequence per SM would be needed: a round of pairs takes 1.9 times as long
-    // (T = 100, H = 128, 20 iterations: 450 and 236 us), so that for 300 sequences two of them, 904 us, lose to three rounds
-    // of one, 705 us, and for 592 two, 900 us, win over four, 945 us.
-    const int rounds = (B + sms - 1) / sms;
-    const int form = csz > 1 || (grp <= 128 && rounds == 1) ? JAC_SPLIT : rounds % 2 == 0 && grp <= 416 ? JAC_PAIR : JAC_ONE;
-    const bool vec = vectors(Wh, l, d, s);
-    auto kernel = form == JAC_PAIR ? (vec ? rnn_bptt_jacobi_kernel<JAC_PAIR, 832, true> : rnn_bptt_jacobi_kernel<JAC_PAIR, 832, false>)
-                : form == JAC_SPLIT ? (vec ? rnn_bptt_jacobi_kernel<JAC_SPLIT, 512, true> : rnn_bptt_jacobi_kernel<JAC_SPLIT, 512, false>)
-                                    : (vec ? rnn_bptt_jacobi_kernel<JAC_ONE, 512, true> : rnn_bptt_jacobi_kernel<JAC_ONE, 512, false>);
-    if (!allow_smem(kernel, JACOBI_SMEM_MAX, form + (vec ? 0 : 3))) return RNN_ERR_CUDA;
-    const int nsq = form == JAC_PAIR ? 2 : 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((B + nsq - 1) / nsq * csz));
-    cfg.blockDim = dim3((unsigned)(form == JAC_PAIR ? 2 * grp : form == JAC_SPLIT ? 4 * grp : grp));
-    cfg.dynamicSmemBytes = (size_t)(H * MH + 2 * H * (VS + 1) + (form == JAC_SPLIT ? 128 * grp : 0)) * sizeof(float);
-    cfg.stream = (cudaStream_t)stream;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)csz;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = csz > 1 ? 1 : 0;
-    cudaLaunchKernelEx(&cfg, kernel, Wh, l, d, B, T, H, n_iters, s0, s, csz, rpc);
+    if (n_iters == 0) {
+        const size_t n = (size_t)B * T * H;
+        rnn_copy_kernel<<<(unsigned)std::min<size_t>((n + 255) / 256, (size_t)sms * 8), 256, 0, (cudaStream_t)stream>>>(s0, s, n);
+        return launch_status();
+    }
+    // several sequences in a unit of 128 columns only where there are more of them than SMs
+    const int per_unit = std::max(1, std::min(2 * J_SLOT / T, (B + sms - 1) / sms));
+    auto kernel = per_unit > 1 ? (H > 64 ? rnn_bptt_jacobi_kernel<32, true> : rnn_bptt_jacobi_kernel<16, true>)
+                               : (H > 64 ? rnn_bptt_jacobi_kernel<32, false> : rnn_bptt_jacobi_kernel<16, false>);
+    if (!allow_smem(kernel, 1024 + J_OPS + (size_t)2 * MT * MH * sizeof(float), (H > 64) + 2 * (per_unit > 1))) return RNN_ERR_CUDA;
+    const size_t smem = 1024 + J_OPS + (size_t)2 * per_unit * T * H * sizeof(float);
+    kernel<<<std::min(sms, (B + per_unit - 1) / per_unit), JTH, smem, (cudaStream_t)stream>>>(
+        Wh, l, d, B, T, H, std::min(n_iters, T), s0, s, per_unit);
     return launch_status();
 }
 

@@ -1,0 +1,85 @@
+"""Jacobi iterations of the recurrent network on the tensor cores, where the kernel can go wrong: one and two slots of 64 columns,
+several sequences in a unit and a ragged last unit, components around 16, 64 and 128, values that bf16 pieces cannot carry."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+def reference(W, l, d, n, s0=None):
+    W, l, d = W.double(), l.double(), d.double()
+    s = torch.zeros_like(l) if s0 is None else s0.double()
+    for _ in range(n):
+        u = torch.zeros_like(l)
+        u[:, :-1] = (d * s)[:, 1:]
+        s = l + u @ W
+    return s
+
+
+def draw(B, T, H):
+    g = torch.Generator("cuda").manual_seed(1000 * B + 10 * T + H)
+    W = torch.randn((H, H), generator=g, device="cuda") * 0.1
+    return W, torch.randn((B, T, H), generator=g, device="cuda"), torch.rand((B, T, H), generator=g, device="cuda"), torch.randn(
+        (B, T, H), generator=g, device="cuda")
+
+
+# fp32 multiply-adds in any order stay within sqrt(K) rounding steps of 2^-24 in the 2-norm, K <= 128 products: 7e-7
+@pytest.mark.parametrize("B,T,H", [(1, 1, 4), (2, 2, 16), (1, 63, 20), (1, 64, 64), (1, 65, 68), (1, 80, 128), (3, 81, 112), (1, 128, 128),
+                                   (150, 64, 64), (299, 64, 128), (297, 43, 36), (451, 32, 124), (500, 31, 8), (1500, 12, 32), (149, 65, 48)])
+def test_against_64_bits(B, T, H):
+    import paper_2002_03629_b200.rnn as rnn
+    W, l, d, s0 = draw(B, T, H)
+    for n, s in ((1, None), (2, None), (3, s0), (min(T, 9), None), (T + 1, s0)):
+        got, want = rnn.rnn_bptt_jacobi(W, l, d, n, s0=s), reference(W, l, d, n, s)
+        assert ((got.double() - want).norm() / want.norm()).item() < 7e-7, n
+
+
+def plain(W, l, d, n, s0):
+    """fp32 multiply-adds, component sums in ascending order."""
+    W, l, d = W.cpu().numpy(), l.cpu().numpy(), d.cpu().numpy()
+    s = np.zeros_like(l) if s0 is None else s0.cpu().numpy()
+    with np.errstate(all="ignore"):
+        for _ in range(n):
+            new = l.copy()
+            u = d * s
+            for k in range(W.shape[0]):
+                new[:, :-1] += u[:, 1:, k, None] * W[k]
+            s = new
+    return s
+
+
+@pytest.mark.parametrize("T,H", [(20, 12), (70, 100)])
+def test_values_beyond_the_pieces(T, H):
+    """Infinities and NaN reach the steps that depend on them and no others; finite values that would round to an infinite bf16
+    number stay finite; a start iterate's infinity is forgotten after T iterations."""
+    import paper_2002_03629_b200.rnn as rnn
+    B = 300
+    W, l, d, s0 = draw(B, T, H)
+    big = l.clone()
+    big[3, T - 2, 1] = float("inf")
+    big[4, 5, 2] = float("nan")
+    big[200] *= 0
+    big[200, T - 1, 0] = 3.4e38
+    d[200] = 1.0
+    for n, start in ((1, None), (4, None), (2, s0)):
+        got, want = rnn.rnn_bptt_jacobi(W, big, d, n, s0=start).cpu().numpy(), plain(W, big, d, n, start)
+        for i in (2, 3, 4, 5, 199, 200, 201, B - 1):
+            np.testing.assert_array_equal(np.isfinite(got[i]), np.isfinite(want[i]))
+            m = np.isfinite(want[i])
+            scale = np.abs(want[i][m]).max()
+            assert np.abs(got[i][m].astype(np.float64) - want[i][m]).max() <= 1e-5 * scale, (n, i)
+    bad = s0.clone()
+    bad[7, 2, 1] = float("inf")
+    assert torch.equal(rnn.rnn_bptt_jacobi(W, l, d, T + 2, s0=bad)[:7], rnn.rnn_bptt_jacobi(W, l, d, T + 2)[:7])
+    assert torch.isfinite(rnn.rnn_bptt_jacobi(W, l, d, T, s0=bad)).all()
+
+
+def test_in_place():
+    """The states may replace the direct gradients, the derivatives or the start iterate."""
+    import paper_2002_03629_b200.rnn as rnn
+    W, l, d, s0 = draw(155, 70, 64)
+    want = rnn.rnn_bptt_jacobi(W, l, d, 6, s0=s0)
+    for which in range(3):
+        a = [l.clone(), d.clone(), s0.clone()]
+        assert torch.equal(rnn.rnn_bptt_jacobi(W, a[0], a[1], 6, s0=a[2], out=a[which]), want)
