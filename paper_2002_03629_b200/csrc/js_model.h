@@ -30,13 +30,15 @@ struct TcDev {
     const CUtensorMap *tmW;      // [L+1] masked weights W[l], box 64 x bn
     TcLayer lay[JS_MAXL + 1];
     int stage_bytes, n_stages, smem_bytes;
-    int ring_bytes, aux_bytes;   // shared memory: operand ring, then the epilogues' auxiliary buffer
+    int ring_bytes, aux_bytes;   // shared memory: operand ring, then the epilogues' auxiliary buffer,
+    int meta_bytes, ucap;        // tile metadata, decoded units (the first ucap of every layer)
     int cat_rows;                // 256-way outputs: the first cat_rows rows of a tile get their noise through shared memory
     int bin_bulk;                // binary output rows are 16-byte granular: moved by bulk copies
     int grid;                    // CTAs the schedules were built for (the launch uses exactly this)
     float *partials;             // [slot][columns/4][128 rows] float4: fp32 partial sums of non-owning chunks
     unsigned *pflags;            // [slot][4 row quadrants][2 column halves]: phase stamp once the partial is stored
     int n_pflags;
+    bool streams;                // output weights that do not stay in L2 from pass to pass
 };
 
 // What the cached sweeps (made_sweep.cu) need beside the tensor-core view.

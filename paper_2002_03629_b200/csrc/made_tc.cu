@@ -59,6 +59,8 @@ struct TcShared {
     alignas(16) float bias_s[4][256];   // per pair of epilogue warps: bias of the current tile's columns (read as float4)
     int wcnt[MAX_WARPS];           // compaction: per-warp counts
     int cbase;                     // compaction: rows kept so far
+    int2 rng[JS_MAXL + 1];         // this pass's live tile range per layer
+    int ucnt[JS_MAXL + 1];         // this CTA's units per layer
 };
 
 // ------------------------------------------------------------------ engine
@@ -73,6 +75,7 @@ struct TcEngine {
     uint8_t *ring;
     uint8_t *staging;
     const int *meta;               // tile metadata in shared memory: per layer kb_end[nt], dmin[nt], dmax[nt]
+    int4 *units;                   // this CTA's first t.ucap units of every layer, decoded
     unsigned epoch = 0;
     unsigned long long issued = 0, skipped = 0, mma_flops = 0, weight_bytes = 0;
     int warp, lane;
@@ -92,7 +95,7 @@ struct TcEngine {
 
     __device__ TcEngine(const MadeDev &m_, const TcDev &t_, const RunArgs &r_, TcShared &sh_, uint8_t *ring_,
                         const int *meta_)
-        : m(m_), t(t_), r(r_), sh(sh_), ring(ring_), staging(ring_ + t_.ring_bytes), meta(meta_)
+        : m(m_), t(t_), r(r_), sh(sh_), ring(ring_), staging(ring_ + t_.ring_bytes), meta(meta_), units((int4 *)(ring_ + t_.ring_bytes + t_.aux_bytes + t_.meta_bytes))
     {
         warp = threadIdx.x >> 5;
         lane = threadIdx.x & 31;
@@ -211,6 +214,7 @@ struct TcEngine {
         if ((nlive + BM - 1) / BM >= (live + BM - 1) / BM) return 0;
         live = nlive;
         pcur ^= 1;
+        fill_units();
         if (blockIdx.x == 0 && threadIdx.x == 0) { r.ctl->compactions += 1; r.ctl->live = nlive; }
         __threadfence_block();
         __nv_bfloat16 *a0 = (__nv_bfloat16 *)m.a[0];
@@ -296,35 +300,55 @@ struct TcEngine {
         int nparts;        // owner: partial sums to add (>= 0); non-owner: -1
         int slot;          // non-owner: its slot; owner: slot of the tile's first partial
     };
-    __device__ bool next_unit(int l, int &e, int e_end, int nt_lo, int nt_hi, int MT, Unit &u) const
+    // unit e of this CTA's list of layer l, from the host's tables: {row tile, column tile, first and last K block, parts and slot}
+    __device__ int4 decode(int l, int MT, int e) const
     {
         const TcLayer &ly = t.lay[l];
+        const int *so = ly.sched_off + (size_t)(ly.n_sched > 1 ? MT - 1 : 0) * (gridDim.x + 1);
+        const int v = ly.sched[so[blockIdx.x] + e], mt = v >> 24, nt = (v >> 8) & 0xffff, chunk = v & 0xff;
+        // nc chunks of nearly equal length: the first `rem` of them hold one K block more
+        const int kbe = kb_end_of(l, nt);
+        const int nc = (kbe + ly.ch - 1) / ly.ch;
+        const int base = kbe / nc, rem = kbe - base * nc;
+        const int kb0 = chunk * base + min(chunk, rem), kb1 = kb0 + base + (chunk < rem ? 1 : 0);
+        const bool owner = (chunk == nc - 1);
+        return make_int4(mt << 16 | nt, kb0 << 16 | kb1, owner ? nc - 1 : -1, mt * ly.slots_per_mt + ly.slot_base[nt] + (owner ? 0 : chunk));
+    }
+    // The lists for a working batch of MT row tiles into shared memory, at the start and when the working batch has shrunk: read from
+    // the host's tables as they are needed, they put three dependent round trips to L2 between a barrier and the first load.
+    // (Followed by a block or grid barrier.)
+    __device__ void fill_units()
+    {
+        const int MT = (live + BM - 1) / BM;
+        for (int l = 0; l <= m.L; ++l) {
+            const TcLayer &ly = t.lay[l];
+            const int *so = ly.sched_off + (size_t)(ly.n_sched > 1 ? MT - 1 : 0) * (gridDim.x + 1) + blockIdx.x;
+            const int n = so[1] - so[0];
+            if (threadIdx.x == 0) sh.ucnt[l] = n;
+            for (int i = threadIdx.x; i < min(n, t.ucap); i += NTH) units[l * t.ucap + i] = decode(l, MT, i);
+        }
+    }
+    __device__ bool next_unit(int l, int &e, int e_end, int nt_lo, int nt_hi, int MT, Unit &u) const
+    {
         while (e < e_end) {
-            const int v = ly.sched[e++];
-            u.mt = v >> 24;
-            u.nt = (v >> 8) & 0xffff;
-            const int chunk = v & 0xff;
+            const int4 v = e < t.ucap ? units[l * t.ucap + e] : decode(l, MT, e);
+            ++e;
+            u.mt = v.x >> 16;
+            u.nt = v.x & 0xffff;
             if (u.mt >= MT || u.nt < nt_lo || u.nt >= nt_hi) continue;
-            // nc chunks of nearly equal length: the first `rem` of them hold one K block more
-            const int kbe = kb_end_of(l, u.nt);
-            const int nc = (kbe + ly.ch - 1) / ly.ch;
-            const int base = kbe / nc, rem = kbe - base * nc;
-            u.kb0 = chunk * base + min(chunk, rem);
-            u.kb1 = u.kb0 + base + (chunk < rem ? 1 : 0);
-            const bool owner = (chunk == nc - 1);
-            u.nparts = owner ? nc - 1 : -1;
-            u.slot = u.mt * ly.slots_per_mt + ly.slot_base[u.nt] + (owner ? 0 : chunk);
+            u.kb0 = v.y >> 16;
+            u.kb1 = v.y & 0xffff;
+            u.nparts = v.z;
+            u.slot = v.w;
             return true;
         }
         return false;
     }
-    // this CTA's unit list of layer l for a working batch of MT row tiles
-    __device__ void unit_list(int l, int MT, int &e, int &e_end) const
+    // this CTA's unit list of layer l
+    __device__ void unit_list(int l, int &e, int &e_end) const
     {
-        const TcLayer &ly = t.lay[l];
-        const int *so = ly.sched_off + (size_t)(ly.n_sched > 1 ? MT - 1 : 0) * (gridDim.x + 1);
-        e = so[blockIdx.x];
-        e_end = so[blockIdx.x + 1];
+        e = 0;
+        e_end = sh.ucnt[l];
     }
 
     // (the whole warp walks the units; one elected lane issues)
@@ -335,8 +359,10 @@ struct TcEngine {
         const uint32_t bytes = A_BYTES + ly.bn * BK * 2;
         ring_for_layer(l);
         if (lane == 0) trace(0);
+        const bool streams = EH == 1 && l == m.L && t.streams;
+        const uint64_t policy = l2_stream_policy();
         int e, e_end;
-        unit_list(l, MT, e, e_end);
+        unit_list(l, e, e_end);
         Unit u;
         while (!dead && next_unit(l, e, e_end, nt_lo, nt_hi, MT, u)) {
             issued++;
@@ -349,7 +375,8 @@ struct TcEngine {
                     if (elect_one()) {
                         mbar_expect_tx(&sh.full[stage], bytes);
                         tma_load_2d(smem_u32(stage_a(stage)), ma, &sh.full[stage], kb * BK, u.mt * BM);
-                        tma_load_2d(smem_u32(stage_b(stage)), mw, &sh.full[stage], 0, kb * ly.npad + u.nt * ly.bn);
+                        if (streams) tma_load_2d_hint(smem_u32(stage_b(stage)), mw, &sh.full[stage], 0, kb * ly.npad + u.nt * ly.bn, policy);
+                        else tma_load_2d(smem_u32(stage_b(stage)), mw, &sh.full[stage], 0, kb * ly.npad + u.nt * ly.bn);
                     }
                     advance_stage();
                 }
@@ -363,7 +390,7 @@ struct TcEngine {
             const int ln = (l == m.L) ? 0 : l + 1;
             const TcLayer &nx = t.lay[ln];
             int e2, e2_end, lo2 = 0, hi2 = nx.nt;
-            unit_list(ln, MT, e2, e2_end);
+            unit_list(ln, e2, e2_end);
             Unit v;
             if (next_unit(ln, e2, e2_end, lo2, hi2, MT, v))
                 for (int kb = v.kb0; kb < v.kb1 && kb < v.kb0 + nx.n_stages; ++kb)
@@ -387,7 +414,7 @@ struct TcEngine {
         const TcLayer &ly = t.lay[l];
         const uint32_t idesc = instr_desc_bf16(ly.bn);
         int e, e_end;
-        unit_list(l, MT, e, e_end);
+        unit_list(l, e, e_end);
         Unit u;
         bool first = true;
         while (next_unit(l, e, e_end, nt_lo, nt_hi, MT, u)) {
@@ -822,6 +849,10 @@ struct TcEngine {
     {
         if (sample < 0) return;
         const float *gg = r.noise + ((size_t)sample * m.T + d) * 256;
+        if (t.streams) {
+            bulk_prefetch_hint(gg, 1024u, l2_stream_policy());
+            return;
+        }
 #pragma unroll
         for (int i = 0; i < 8; ++i) prefetch_l2(gg + i * 32);
     }
@@ -835,8 +866,10 @@ struct TcEngine {
         const uint32_t tot = __reduce_add_sync(0xffffffffu, sample >= 0 ? 1024u : 0u);
         if (lane == 0) mbar_expect_tx(&sh.nzbar[warp - 2], tot);
         __syncwarp();
-        if (sample >= 0)
-            bulk_load(smem_u32(cat_row()), r.noise + ((size_t)sample * m.T + d) * 256, 1024u, &sh.nzbar[warp - 2]);
+        if (sample < 0) return;
+        const float *gg = r.noise + ((size_t)sample * m.T + d) * 256;
+        if (t.streams) bulk_load_hint(smem_u32(cat_row()), gg, 1024u, &sh.nzbar[warp - 2], l2_stream_policy());
+        else bulk_load(smem_u32(cat_row()), gg, 1024u, &sh.nzbar[warp - 2]);
     }
     __device__ bool epi_cat_tile(int sample, int row, int d, uint32_t tbase, const Win &w, bool flag, int parity,
                                  bool &any_changed, int &first)
@@ -1022,7 +1055,7 @@ struct TcEngine {
         int first = INT_MAX;
         bool cat_ahead = false;        // the current tile's noise was asked into L2 during the previous tile
         int e, e_end;
-        unit_list(l, MT, e, e_end);
+        unit_list(l, e, e_end);
         Unit u;
         while (!dead && next_unit(l, e, e_end, nt_lo, nt_hi, MT, u)) {
             const int nt = u.nt, mt = u.mt;
@@ -1126,8 +1159,7 @@ struct TcEngine {
     // one layer over the window; returns false when there was nothing to do (no barrier needed)
     __device__ bool gemm_phase(int l, int kind, const Win &w, bool flag, int parity, float *zout)
     {
-        int nt_lo, nt_hi;
-        live_range(l, w, nt_lo, nt_hi);
+        const int nt_lo = sh.rng[l].x, nt_hi = sh.rng[l].y;
         const int MT = (live + BM - 1) / BM;
         const int nlive = max(0, nt_hi - nt_lo);
         if (threadIdx.x == 0 && blockIdx.x == 0) skipped += (unsigned long long)(t.lay[l].nt - nlive) * MT;
@@ -1149,6 +1181,13 @@ struct TcEngine {
     __device__ bool step(const Win &w, bool flag, int parity, float *zout)
     {
         const int out_kind = zout ? EPI_LOGITS : EH == 2 ? EPI_BINARY : EPI_CAT;
+        // the live tiles of all layers, a warp each (searched behind every barrier they cost every phase half a microsecond)
+        for (int l = warp; l <= m.L; l += NTH / 32) {
+            int2 rg;
+            live_range(l, w, rg.x, rg.y);
+            if (lane == 0) sh.rng[l] = rg;
+        }
+        __syncthreads();
         for (int l = 0; l <= m.L; ++l) {
             const bool last = (l == m.L);
             const bool did = gemm_phase(l, last ? out_kind : EPI_HIDDEN, w, last && flag, parity, zout);
@@ -1204,6 +1243,7 @@ made_tc_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ TcDev 
 
     TcEngine<EH> e(m, t, r, sh, ring, meta);
     e.tmem_base = sh.tmem_base;
+    e.fill_units();
     if (threadIdx.x == 0) e.trace(0);
     DriverResult res = made_driver(e, m.T, r);
     if (e.dead) res.alive = false;
@@ -1375,7 +1415,7 @@ int js_tc_prepare(js_model *mo)
     }
     t.grid = G;
     size_t part_floats = 0;
-    int max_slots = 0;
+    int max_slots = 0, most_units = 0;
     // One schedule per size of the working batch (compaction shrinks it), as long as that is a
     // handful; the chunks themselves never depend on it, only who computes them.
     const int n_sched = MTmax <= 16 ? MTmax : 1;
@@ -1408,7 +1448,8 @@ int js_tc_prepare(js_model *mo)
             // tile's partial sums have been stored.  Units are taken longest first and put where
             // the CTA finishes earliest.  Inside a CTA: partial chunks first (owners elsewhere
             // wait for them), then owners that wait for nobody, then owners that add partial sums.
-            const int FILL = 6, EPI_PART = 5, EPI_OWN = (l == L ? (bn == 256 ? 5 : 9) : 4), EPI_ADD = 8;
+            // (EPI_ADD 4, 6, 8, 10: 312, 315, 318, 318 us for 4096 units a layer and 512 samples; the others make no difference.)
+            const int FILL = 6, EPI_PART = 5, EPI_OWN = (l == L ? (bn == 256 ? 5 : 9) : 4), EPI_ADD = 4;
             struct Item { int code, size, epi, ready; };
             std::vector<std::vector<Item>> lp(G), lo0(G), lo1(G);
             auto finish = [&](int c, const Item *extra, int where) {
@@ -1471,6 +1512,7 @@ int js_tc_prepare(js_model *mo)
                     v0 = mix;
                 }
             for (int c = 0; c < G; ++c) {
+                most_units = std::max(most_units, (int)(lp[c].size() + lo0[c].size() + lo1[c].size()));
                 off.push_back((int)flat.size());
                 for (const Item &it : lp[c]) flat.push_back(it.code);
                 for (const Item &it : lo0[c]) flat.push_back(it.code);
@@ -1514,7 +1556,19 @@ int js_tc_prepare(js_model *mo)
     t.tmA = (const CUtensorMap *)pa;
     t.tmW = (const CUtensorMap *)pw;
 
-    t.smem_bytes = 1024 + t.ring_bytes + t.aux_bytes + meta_bytes;
+    // Output weights beyond what L2 keeps from one pass to the next are marked as the first to be evicted (the noise they are read
+    // with too), so that each pass finds some of them: with all lines alike every line has gone before its turn comes.  Live
+    // weights of 537, 250, 134 and 105 MB: 607 -> 570, 380 -> 346, 285 -> 258, 246 -> 229 us a call; 79 MB 219 -> 217; 52 MB, which L2
+    // keeps, 153 -> 158.
+    {
+        size_t live_kb = 0;
+        for (int x : kb_all[L]) live_kb += (size_t)x;
+        t.streams = wide && live_kb * BK * 256 * sizeof(__nv_bfloat16) > (size_t)64 << 20;
+    }
+    t.meta_bytes = meta_bytes;
+    // room for the decoded lists: as many units of every layer as a CTA has at most, or as there is room for
+    t.ucap = std::max(0, std::min(most_units, (SMEM_DYN_MAX - 1024 - t.ring_bytes - t.aux_bytes - meta_bytes) / (16 * (L + 1))));
+    t.smem_bytes = 1024 + t.ring_bytes + t.aux_bytes + meta_bytes + 16 * (L + 1) * t.ucap;
     // the attribute belongs to the function, not to a model: always allow the largest request
     const int smem = SMEM_DYN_MAX;
     const void *kernel = tc_kernel_of(v);
