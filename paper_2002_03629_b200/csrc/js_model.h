@@ -82,7 +82,7 @@ struct ClusterDev {
     int early_ok;                // encodings may be sent as soon as they are sampled
     int n_stages;
     ClTiles tiles;
-    const CUtensorMap *tmW;      // tile-major weights, box 64 x 64
+    const CUtensorMap *tmW;      // [L+1][2] tile-major weights: one K block of 64 units, two of them
 };
 
 // Device view of a masked-convolution stack (tensor-core kernel only).

@@ -13,13 +13,15 @@
 //     the MMA reads.  A finished tile IS one K block of the layer above: it is written in place and sent to the other CTAs by
 //     one bulk copy each (cp.async.bulk to distributed shared memory, completing on the receiver's mbarrier for that block).
 //     An MMA waits for the K blocks it reads, not for a layer: there is no barrier inside a pass;
-//   - weights stream from L2 through two rings (even and odd K blocks), independent of all that: the next tile's, and in Jacobi mode the next pass's,
-//     weights are on their way while a layer waits for its inputs;
+//   - weights stream from L2 through a ring, two K blocks a load, independent of all that: the next tile's, and in Jacobi mode the
+//     next pass's, weights are on their way while a layer waits for its inputs;
 //   - noise, symbols and biases of the CTA's own output positions stay in shared memory.
 // A pass ends with one exchange of change masks (64 bits, one per sample) between the CTAs.
 // What bounds it: the chain of a pass (per layer: last K block arrives -> MMAs -> epilogue -> copy), and for wide models
-// the weight stream (each cluster reads all live weights per pass).
-//
+// the weight stream (each cluster reads all live weights per pass).  784 positions, 1024 units x 2, 24 samples a cluster: 12 us a
+// pass, of which three layers at 3.2 and 1.5 from the last mask to the next pass's first MMA; 16.5 before the loads took two
+// blocks, one thread of a warp looked for weights, activations and room at once (a look is 150 cycles), and every role
+// saw the masks itself.
 // Solvers: Jacobi (Algorithm 1) and GS-Jacobi (Algorithm 3), the control logic of made_driver.cuh on the cluster's samples.
 // Warps: 0 weight loads, 1 and 7 MMA (1 owns tensor memory), 2-5 epilogue, 6 arms and drains the activation barriers.
 // All waits are bounded, as in the other tensor-core kernels.
@@ -40,16 +42,16 @@ constexpr int BK = TC_BK;
 constexpr int TM = 64;                       // units per tile
 constexpr int NTH = 256;
 constexpr int STAGE = TM * BK * 2;           // 8 KB of weights
-constexpr int MAX_STAGES = 16;
+constexpr int MAX_STAGES = 16;               // of 8 KB; they are used in pairs, an even K block and the odd one behind it
 constexpr int NSLOT = 2, ACC = 64;           // accumulator slots; columns of one accumulator (two per slot: even, odd K blocks)
 constexpr int MAXOWN = CL_TILES / 8;         // own tiles per layer (the cluster size grows with the tile count)
 constexpr int SMEM_MAX = 227 * 1024 - 11 * 1024;
 
 struct ClShared {
-    uint64_t full[MAX_STAGES], empty[MAX_STAGES], tfull[NSLOT], tempty[NSLOT];
+    uint64_t full[MAX_STAGES / 2], empty[MAX_STAGES / 2], tfull[NSLOT], tempty[NSLOT];
     uint64_t xbar[2][CL_TILES];              // K block of the encoded iterate complete in this CTA, by pass parity
     uint64_t hbar[CL_MAXL][CL_TILES];        // K block of a[l + 1] complete in this CTA
-    uint64_t pbar;                           // every CTA of the cluster has finished the pass
+    uint64_t pbar[2];                        // by pass parity: every CTA of the cluster has finished the pass, their masks are here
     uint64_t go;                             // the next pass may start (or the roles may leave)
     uint64_t ack;                            // the loading and MMA warps are done with the pass's ranges
     uint32_t tmem_base;
@@ -61,7 +63,9 @@ struct ClShared {
     int first[2];
     uint4 flags[2][8];                       // per pass parity and CTA: change mask, smallest changed position
     int count[64];
-    int issued[2], consumed[2];              // weight loads, of even and of odd K blocks
+    int issued, consumed[2];                 // weight loads; K blocks multiplied, even and odd ones
+    int consumed_loads;
+    uint64_t apar[2][CL_MAXL + 2];
     unsigned tiles;
     unsigned sums[2];                        // of the whole cluster (in its first CTA): tiles, K blocks
     float bias_s[CL_MAXL + 1][MAXOWN][TM];
@@ -71,6 +75,23 @@ __device__ __forceinline__ void copy_to_peer(uint32_t dst, uint32_t src, uint32_
 {
     asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(dst), "r"(src), "r"(bytes), "r"(bar) : "memory");
+}
+// 16 bytes into another CTA's shared memory, counted on the barrier there as they arrive
+__device__ __forceinline__ void send16(uint32_t dst, uint4 v, uint32_t bar)
+{
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
+                 ::"r"(dst), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(bar) : "memory");
+}
+// Eight columns of a warp's sixteen accumulator lanes, over all its threads: lane i gets columns 2 (i % 4) and the next of rows
+// i / 4 (r[0], r[1]) and i / 4 + 8 (r[2], r[3]).
+__device__ __forceinline__ void tmem_ld_16x8(uint32_t taddr, uint32_t (&r)[4])
+{
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(taddr) : "memory");
+}
+// two 8 x 8 blocks in that order of the threads, transposed: lane i (and i + 8) gives the address of the first (second) block's column i
+__device__ __forceinline__ void stmatrix2_trans(uint32_t addr, uint32_t a, uint32_t b)
+{
+    asm volatile("stmatrix.sync.aligned.m8n8.x2.trans.shared.b16 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
 }
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8])
 {
@@ -89,7 +110,7 @@ struct ClEngine {
     float *nz;                    // [own output tile][R][64]
     uint64_t *xs;                 // [own output tile][64]: bit s = symbol of sample s
     const int R;
-    int rank, CS, L, S, warp, lane;
+    int rank, CS, L, NP, warp, lane;          // NP: pairs in the weight ring
     uint32_t blk_bytes;           // one K block of activations: R x 128 bytes
     int a_blk[CL_MAXL + 1];       // first K block of a[l] inside `acts`
 
@@ -99,11 +120,11 @@ struct ClEngine {
         CS = cd.CS;
         rank = CS > 1 ? (int)cluster_rank() : 0;
         L = m.L;
-        S = cd.n_stages;
+        NP = cd.n_stages >> 1;
         warp = threadIdx.x >> 5;
         lane = threadIdx.x & 31;
         blk_bytes = (uint32_t)R * 128u;
-        acts = ring + (size_t)S * STAGE;
+        acts = ring + (size_t)(2 * NP) * STAGE;
         int at = 0;
 #pragma unroll
         for (int l = 0; l <= CL_MAXL; ++l) {
@@ -182,176 +203,157 @@ struct ClEngine {
         if (try_wait<CLUSTER>(bar, parity)) return true;
         return wait_slow<CLUSTER>(bar, parity);
     }
-    __device__ bool wait_all_lanes(uint64_t *bar, uint32_t parity) const
+    // May pass `pass` start?  In Jacobi mode every role sees for itself, in the masks of the pass before, whether there is another one
+    // (told by the epilogue warps, behind their bookkeeping, it came 0.9 us later); else they are told, and learn the window.
+    __device__ bool next_pass(unsigned pass, bool jacobi) const
     {
-        return __all_sync(0xffffffffu, wait(bar, parity));
+        if (pass == 0 || !jacobi) return wait(&sh.go, pass & 1) && !*(volatile int *)&sh.stop;
+        if (!wait<true>(&sh.pbar[(pass - 1) & 1], (pass - 1) >> 1 & 1)) return false;
+        uint32_t any = 0;
+        for (int i = 0; i < CS; ++i) {
+            const volatile uint4 &f = sh.flags[(pass - 1) & 1][i];
+            any |= f.x | f.y;
+        }
+        const int cap = r.max_iters > 0 && r.max_iters < m.T ? r.max_iters : m.T;
+        return any != 0 && (int)pass < cap && !*(volatile int *)&sh.dead;
     }
-    // Warp-wide: how many of the next items are ready, one after the other (lane i tests the i-th); 0: gave up, or told to
-    // stop.  (See mbar_wait_run in tc_common.cuh for why one look serves several items.)
-    template <typename F>
-    __device__ __forceinline__ int wait_run(F ready, bool stoppable) const
+    // A stage of the weight ring is a pair of K blocks, an even one and the odd one behind it, brought by one load and freed by
+    // both consumers.  (A load costs the loading thread 0.2 us, barrier and all, whatever its size: block by block, and with a
+    // ring of its own for either consumer, the weights of a pass of 45 blocks took 11 us of the pass's 16.)  Each consumer waits
+    // for every stage, also where the last pair of a tile lacks its block: so it cannot take a stage for full, or free one, in a
+    // use of it other than its own (a parity does not tell a phase from the one after the next).
+
+    // ---------------------------------------------------------------- roles
+    // (one thread)
+    __device__ bool room(uint64_t *bar, uint32_t parity, bool stoppable) const
     {
         uint64_t t0 = 0;
         for (unsigned i = 0;; ++i) {
-            const unsigned mask = __ballot_sync(0xffffffffu, ready());
-            if (mask & 1u) return mask == 0xffffffffu ? 32 : __ffs((int)~mask) - 1;
-            if (stoppable && __any_sync(0xffffffffu, *(volatile int *)&sh.stop)) return 0;
-            if (__any_sync(0xffffffffu, hopeless(i, t0))) {
-                if (lane == 0) give_up();
-                return 0;
-            }
+            if (mbar_test_wait(bar, parity)) return true;
+            if (stoppable && *(volatile int *)&sh.stop) return false;
+            if (hopeless(i, t0)) return give_up();
         }
     }
-    // The weight ring is two: even K blocks of every tile take the stages 0, 2, 4 .., odd ones 1, 3, 5 .., in turn, because each
-    // half has a consumer of its own.  In one ring for both, a consumer could look at a stage whose former occupant, the other
-    // consumer's, had not even arrived (loads overtake one another), and a parity cannot tell that phase from the one after the
-    // next: it took the stage for full.  In its own ring it has consumed every former occupant itself.
-    // Stage `off` positions on in ring `half`, and the parity of its use there.
-    __device__ __forceinline__ void ring_at(int half, int st, uint32_t ph, int off, int &s, uint32_t &p) const
-    {
-        int q = st + off;
-        p = ph;
-        while (q >= (S >> 1)) { q -= S >> 1; p ^= 1u; }
-        s = 2 * q + half;
-    }
-
-    // ---------------------------------------------------------------- roles
     __device__ void producer(bool jacobi)
     {
-        int n0 = 0, n1 = 0, st0 = 0, st1 = 0;    // per ring: loads so far, next stage, parity of its use
-        uint32_t ph0 = 0, ph1 = 0;
+        int n = 0, st = 0;
+        uint32_t ph = 1;
         bool on = true;
         const uint32_t ring0 = smem_u32(ring);
         for (unsigned pass = 0; on; ++pass) {
-            if (!jacobi) {
-                if (!wait_all_lanes(&sh.go, pass & 1)) break;
-                if (__any_sync(0xffffffffu, *(volatile int *)&sh.stop)) break;
-            }
+            if (!jacobi && !next_pass(pass, false)) break;
             for (int l = 0; l <= L && on; ++l) {
                 // in Jacobi mode every tile is computed in every pass: the stream needs no go-ahead
                 const int2 rg = jacobi ? make_int2(0, cd.nt[l]) : sh.rng[pass & 1][l];
-                const CUtensorMap *map = cd.tmW + l;
-                for (int j = 0; j < sh.nown[l] && on; ++j) {
+                const CUtensorMap *map = cd.tmW + 2 * l;
+                const int npad = cd.npad[l], own = sh.nown[l];
+                for (int j = 0; j < own && on; ++j) {
                     const int2 o = sh.own[l][j];
                     if (!in(rg, o.x)) continue;
-                    int row = o.x * TM;
-                    for (int kb = 0; kb < o.y;) {
-                        int s;
-                        uint32_t p;
-                        const int h = (kb + lane) & 1;
-                        ring_at(h, h ? st1 : st0, h ? ph1 : ph0, lane >> 1, s, p);      // (as many of this half lie between)
-                        const bool look = lane < S && kb + lane < o.y;
-                        const int run = wait_run([&] { return look && mbar_test_wait(&sh.empty[s], p ^ 1u); }, jacobi);
-                        if (run == 0) { on = false; break; }
-                        for (int i = 0; i < run; ++i, ++kb, row += cd.npad[l]) {
-                            const int half = kb & 1, st = 2 * (half ? st1 : st0) + half;
-                            if (elect_one()) {
-                                mbar_expect_tx(&sh.full[st], STAGE);
-                                tma_load_2d(ring0 + (uint32_t)st * STAGE, map, &sh.full[st], 0, row);
-                            }
-                            if (half) {
-                                ++n1;
-                                if (++st1 == (S >> 1)) { st1 = 0; ph1 ^= 1u; }
-                            } else {
-                                ++n0;
-                                if (++st0 == (S >> 1)) { st0 = 0; ph0 ^= 1u; }
-                            }
+                    for (int kb = 0; kb < o.y; kb += 2) {
+                        if (!room(&sh.empty[st], ph, jacobi)) { on = false; break; }
+                        const uint32_t to = ring0 + (uint32_t)st * (2 * STAGE);
+                        if (kb + 1 < o.y) {
+                            mbar_expect_tx(&sh.full[st], 2 * STAGE);
+                            tma_load_3d(to, map + 1, &sh.full[st], 0, o.x * TM, kb);
+                        } else {
+                            mbar_expect_tx(&sh.full[st], STAGE);
+                            tma_load_2d(to, map, &sh.full[st], 0, kb * npad + o.x * TM);
                         }
+                        ++n;
+                        if (++st == NP) { st = 0; ph ^= 1u; }
                     }
                 }
             }
-            if (!jacobi && lane == 0) mbar_arrive(&sh.ack);
+            if (!jacobi) mbar_arrive(&sh.ack);
         }
-        if (lane == 0) { sh.issued[0] = n0; sh.issued[1] = n1; }
+        sh.issued = n;
     }
 
-    // half 0 issues the even K blocks of every tile, half 1 the odd ones
-    __device__ void mma_issuer(int half)
+    // bits lo .. hi - 1
+    static __device__ uint64_t bits(const int2 &r)
+    {
+        return r.y <= r.x ? 0ull : (~0ull >> (64 - (r.y - r.x))) << r.x;
+    }
+    __device__ __noinline__ bool wait_both(uint64_t *a, uint32_t pa, uint64_t *b, uint32_t pb) const
+    {
+        return (mbar_test_wait(a, pa) || wait_slow<false>(a, pa)) && (mbar_test_wait(b, pb) || wait_slow<false>(b, pb));
+    }
+    // One thread; half 0 issues the even K blocks of every tile, half 1 the odd ones.  It looks for the next block's weights and
+    // activations (150 cycles) before it issues this one's MMAs (96).
+    __device__ void mma_issuer(int half, bool jacobi)
     {
         const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(R >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
-        const uint64_t ring_desc = smem_desc_sw128(smem_u32(ring));
-        uint64_t apar[CL_MAXL + 2];              // parity of the next completion of every K block's barrier; x: two sets
-#pragma unroll
-        for (int l = 0; l < CL_MAXL + 2; ++l) apar[l] = 0;
-        int n = 0, slot = 0, st = 0;             // st, ph: position in this half's ring of its first K block of the tile
+        const uint64_t ring_desc = smem_desc_sw128(smem_u32(ring) + (uint32_t)(half * STAGE));
+        const uint32_t blk = blk_bytes >> 4;
+        int n = 0, loads = 0, slot = 0, st = 0;  // st, ph: the ring's next stage and the parity of its use
         uint32_t ph = 0, spar = 0;               // spar: parity of the accumulator slots' next use
         bool on = true;
         unsigned tiles = 0;
         for (unsigned pass = 0; on; ++pass) {
-            if (!wait_all_lanes(&sh.go, pass & 1)) break;
-            if (__any_sync(0xffffffffu, *(volatile int *)&sh.stop)) break;
+            if (!next_pass(pass, jacobi)) break;
 #pragma unroll 1
             for (int l = 0; l <= L && on; ++l) {
                 const int2 fr = fresh(l, pass), rg = sh.rng[pass & 1][l];
-                const int set = l == 0 ? (pass & 1 ? CL_MAXL + 1 : 0) : l;
-                uint64_t ap = 0;
-#pragma unroll
-                for (int q = 0; q < CL_MAXL + 2; ++q) ap = q == set ? apar[q] : ap;
-                const uint64_t act_desc = smem_desc_sw128(smem_u32(block(l, 0)));
-                for (int j = 0; j < sh.nown[l] && on; ++j) {
+                uint64_t *const apar = &sh.apar[half][l == 0 && (pass & 1) ? CL_MAXL + 1 : l];       // parities of the K blocks' barriers; x: two sets
+                const uint64_t ap = *apar, isfresh = bits(fr);
+                const uint64_t act_desc = smem_desc_sw128(smem_u32(block(l, 0))) + (uint64_t)(half * blk);
+                uint64_t *const bars = block_bar(l, half, pass);
+#pragma unroll 1
+                for (int j = 0; j < sh.nown[l]; ++j) {
                     const int2 o = sh.own[l][j];
                     if (!in(rg, o.x)) continue;
                     ++tiles;
-                    if (!wait_all_lanes(&sh.tempty[slot], (spar >> slot & 1u) ^ 1u)) { on = false; break; }
-                    tc_fence_after();
+                    const int mine = (o.y + 1 - half) >> 1, pairs = (o.y + 1) >> 1;
                     const uint32_t d = sh.tmem_base + (uint32_t)((2 * slot + half) * ACC);
-                    for (int kb = half; kb < o.y;) {
-                        // lane i: are the weights and the activations of K block kb + 2 i here?
-                        const int lk = kb + 2 * lane;
-                        int s;
-                        uint32_t p;
-                        const bool look = lk < o.y && lane < (S >> 1);
-                        ring_at(half, st, ph, look ? lk >> 1 : 0, s, p);
-                        const bool isfresh = look && in(fr, lk);
-                        uint64_t *ab = block_bar(l, look ? lk : 0, pass);
-                        const uint32_t abp = (uint32_t)(ap >> (look ? lk : 0)) & 1u;
-                        const int run = wait_run([&] { return look && mbar_test_wait(&sh.full[s], p) && (!isfresh || mbar_test_wait(ab, abp)); }, false);
-                        if (run == 0) { on = false; break; }
-                        tc_fence_after();
-                        // (one election per run, not per K block: 200 cycles a block instead of 250)
-                        if (elect_one()) {
-                            for (int i = 0; i < run; ++i) {
-                                const int kc = kb + 2 * i;
-                                int cs;
-                                uint32_t cp;
-                                ring_at(half, st, ph, kc >> 1, cs, cp);
-                                const uint64_t ad = ring_desc + (uint64_t)(cs * (STAGE >> 4)), bd = act_desc + (uint64_t)(kc * (int)(blk_bytes >> 4));
-#pragma unroll
-                                for (int k = 0; k < BK / 16; ++k)
-                                    umma_bf16(d, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc, (kc > half || k > 0) ? 1u : 0u);
-                                umma_commit(&sh.empty[cs]);
-                            }
+                    uint64_t bd = act_desc, am = ap >> half, fm = isfresh >> half, *ab = bars;
+                    auto look = [&](int i) {         // block i of this half
+                        const bool w = mbar_test_wait(&sh.full[st], ph), a = mbar_test_wait(ab, (uint32_t)am & 1u);
+                        return w & (a | (i >= mine) | !(fm & 1ull));
+                    };
+                    bool ready = look(0);
+                    if (!wait(&sh.tempty[slot], (spar >> slot & 1u) ^ 1u)) { on = false; break; }
+#pragma unroll 1
+                    for (int i = 0; i < pairs; ++i) {
+                        if (!ready) {
+                            const bool need = i < mine && (fm & 1ull);
+                            if (!wait_both(&sh.full[st], ph, need ? ab : &sh.full[st], need ? (uint32_t)am & 1u : ph)) { on = false; break; }
                         }
-                        __syncwarp();
-                        kb += 2 * run;
+                        tc_fence_after();
+                        const int cur = st;
+                        const uint64_t ad = ring_desc + (uint64_t)(cur * (2 * STAGE >> 4)), b = bd;
+                        if (++st == NP) { st = 0; ph ^= 1u; }
+                        bd += 2 * blk;
+                        am >>= 2;
+                        fm >>= 2;
+                        ab += 2;
+                        ready = i + 1 < pairs && look(i + 1);
+                        if (i < mine)
+#pragma unroll
+                            for (int k = 0; k < BK / 16; ++k)
+                                umma_bf16(d, ad + (uint64_t)(2 * k), b + (uint64_t)(2 * k), idesc, (i > 0 || k > 0) ? 1u : 0u);
+                        umma_commit(&sh.empty[cur]);
                     }
                     if (!on) break;
-                    if (elect_one()) umma_commit(&sh.tfull[slot]);      // (with no K block of its own too: all its earlier MMAs are done)
-                    const int mine = (o.y + 1 - half) >> 1;
+                    umma_commit(&sh.tfull[slot]);      // (with no K block of its own too: all its earlier MMAs are done)
                     n += mine;
-                    st += mine;
-                    while (st >= (S >> 1)) { st -= S >> 1; ph ^= 1u; }
+                    loads += pairs;
                     spar ^= 1u << slot;
-                    slot = (slot + 1) % NSLOT;
+                    slot ^= 1;
                 }
-                uint64_t flip = 0;
-                for (int kb = fr.x; kb < fr.y; ++kb) flip |= 1ull << kb;
-#pragma unroll
-                for (int q = 0; q < CL_MAXL + 2; ++q) apar[q] ^= q == set ? flip : 0ull;
+                *apar = ap ^ isfresh;
             }
-            if (lane == 0) mbar_arrive(&sh.ack);
+            if (!jacobi) mbar_arrive(&sh.ack);
         }
-        if (lane == 0) {
-            sh.consumed[half] = n;
-            if (half == 0) sh.tiles = tiles;
-        }
+        sh.consumed[half] = n;
+        if (half == 0) { sh.tiles = tiles; sh.consumed_loads = loads; }
     }
 
     // Barrier keeper (one warp, lane = K block).  Every block another CTA sends completes its barrier once per pass in
     // which it is live: armed here with the bytes to come, and waited for before the pass may end, so that no copy is in
     // flight when its source or its barrier is used again.  (Bytes that arrive before the arming are counted all the same:
     // the phase cannot complete without it, and the phase before was waited for in the pass before.)
-    __device__ void keeper(bool early)
+    __device__ void keeper(bool early, bool jacobi)
     {
         uint64_t apar[CL_MAXL + 2];
 #pragma unroll
@@ -377,12 +379,12 @@ struct ClEngine {
             for (int q = 0; q < CL_MAXL + 2; ++q) apar[q] = q == set ? ap : apar[q];
         };
         for (unsigned pass = 0;; ++pass) {
-            on = __all_sync(0xffffffffu, wait(&sh.go, pass & 1));
-            if (!on) break;
-            if (__any_sync(0xffffffffu, *(volatile int *)&sh.stop)) {
-                if (early && *(volatile int *)&sh.dead == 0) { arm(0, pass); drain(0, pass); }    // encodings sent ahead for a pass that is not run
+            if (!__all_sync(0xffffffffu, next_pass(pass, jacobi))) {
+                if (*(volatile int *)&sh.dead) break;
+                if (early) { arm(0, pass); drain(0, pass); }         // encodings sent ahead for a pass that is not run
                 return;
             }
+            if (lane == 0) mbar_expect_tx(&sh.pbar[pass & 1], (uint32_t)(16 * CS));
             for (int l = 0; l <= L; ++l) arm(l, pass);
             for (int l = 0; l <= L; ++l) drain(l, pass);
             on = __all_sync(0xffffffffu, on);
@@ -436,24 +438,28 @@ struct ClEngine {
         tmem_ld8(tb, a);
         if (two) tmem_ld8(tb + ACC, b);
     }
+    // bias: of the tile's units.  A value goes from the thread that has it to its sample's row by a transposing store, eight samples
+    // of eight units at a time: lane = unit, with half the lanes idle and a 2-byte store per value, took 0.4 us longer.
     template <int ACT>
-    __device__ __forceinline__ void hidden_columns(uint8_t *dst, uint32_t tb, bool two, float bv, int u, bool act_lane)
+    __device__ __forceinline__ void hidden_columns(uint32_t dst, uint32_t tb, bool two, const float *bias, int q)
     {
-        uint32_t na[8], nb[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        load_sums(tb, na, nb, two);
+        const float b0 = bias[q * 16 + (lane >> 2)], b1 = bias[q * 16 + (lane >> 2) + 8];
+        uint32_t na[4], nb[4] = {0, 0, 0, 0};
+        tmem_ld_16x8(tb, na);
+        if (two) tmem_ld_16x8(tb + ACC, nb);
+        uint32_t at = dst + (uint32_t)((lane & 7) * 128 + (((2 * q + (lane >> 3 & 1)) ^ (lane & 7)) << 4));
 #pragma unroll 1
-        for (int s0 = 0; s0 < R; s0 += 8, dst += 1024) {
-            float v[8];
+        for (int s0 = 0; s0 < R; s0 += 8, at += 1024) {
+            float v[4];
             tmem_wait_ld();
 #pragma unroll
-            for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(na[i]) + __uint_as_float(nb[i]);
-            load_sums(tb + (uint32_t)min(s0 + 8, R - 8), na, nb, two);
-            if (act_lane)
-#pragma unroll
-                for (int i = 0; i < 8; ++i)
-                    *reinterpret_cast<__nv_bfloat16 *>(dst + at_block(i, u)) = __float2bfloat16_rn(tc_act_fn(ACT, v[i] + bv));
+            for (int i = 0; i < 4; ++i) v[i] = __uint_as_float(na[i]) + __uint_as_float(nb[i]);
+            if (s0 + 8 < R) {
+                tmem_ld_16x8(tb + (uint32_t)(s0 + 8), na);
+                if (two) tmem_ld_16x8(tb + ACC + (uint32_t)(s0 + 8), nb);
+            }
+            stmatrix2_trans(at, pack_bf16x2(tc_act_fn(ACT, v[0] + b0), tc_act_fn(ACT, v[1] + b0)), pack_bf16x2(tc_act_fn(ACT, v[2] + b1), tc_act_fn(ACT, v[3] + b1)));
         }
-        tmem_wait_ld();
     }
     template <int NK>
     __device__ __forceinline__ uint64_t sample_columns(const float *nzt, uint32_t tb, bool two, float bv)
@@ -506,16 +512,17 @@ struct ClEngine {
                     const int tile = sh.own[l][j].x;
                     if (!in(sh.rng[par][l], tile)) continue;
                     const bool two = sh.own[l][j].y > 1;
-                    const float bv = sh.bias_s[l][j][u];
+                    const float *bias = sh.bias_s[l][j];
                     const bool ok = __all_sync(0xffffffffu, wait(&sh.tfull[slot], spar >> slot & 1u));
                     tc_fence_after();
                     const uint32_t tb = sh.tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(2 * slot * ACC);
                     if (l < L) {
-                        uint8_t *dst = block(l + 1, tile);
-                        if (m.act == JS_ACT_RELU) hidden_columns<JS_ACT_RELU>(dst, tb, two, bv, u, act_lane);
-                        else hidden_columns<JS_ACT_GELU_TANH>(dst, tb, two, bv, u, act_lane);
+                        const uint32_t dst = smem_u32(block(l + 1, tile));
+                        if (m.act == JS_ACT_RELU) hidden_columns<JS_ACT_RELU>(dst, tb, two, bias, q);
+                        else hidden_columns<JS_ACT_GELU_TANH>(dst, tb, two, bias, q);
                     } else {
                         const int p = tile * TM + u;
+                        const float bv = bias[u];
                         const bool mine = act_lane && p >= w.plo && p < w.phi;
                         uint8_t *dst = stag + (size_t)(par * cd.own_out + j) * blk_bytes;
                         const float *nzt = nz + (size_t)j * R * TM + u;
@@ -563,14 +570,12 @@ struct ClEngine {
             if (early) send_all_x();
             // ---- end of the pass: masks to everybody, once this CTA's MMAs are done and all its copies have landed
             asm volatile("bar.sync 2, 160;" ::: "memory");
-            if (tid < CS) {
-                const uint32_t to = peer_addr(smem_u32(&sh.flags[par][rank]), tid);
-                asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(to), "r"(sh.chg[par][0]), "r"(sh.chg[par][1]),
-                             "r"(sh.first[par]), "r"(0) : "memory");
-                asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(peer_addr(smem_u32(&sh.pbar), tid)) : "memory");
-            }
-            bool fine = wait<true>(&sh.pbar, pass & 1);
-            if (tid == 0) fine = wait(&sh.ack, pass & 1) && fine;
+            // (data and signal in one: a store and a releasing arrival behind it took two trips between CTAs, 1.5 us)
+            if (tid < CS)
+                send16(peer_addr(smem_u32(&sh.flags[par][rank]), tid), make_uint4(sh.chg[par][0], sh.chg[par][1], (uint32_t)sh.first[par], 0u),
+                       peer_addr(smem_u32(&sh.pbar[par]), tid));
+            bool fine = wait<true>(&sh.pbar[par], pass >> 1 & 1);
+            if (!jacobi && tid == 0) fine = wait(&sh.ack, pass & 1) && fine;
             if (!ep_all(fine && *(volatile int *)&sh.dead == 0)) return -1;
             uint32_t clo = 0, chi = 0;
             int mf = INT_MAX;
@@ -605,11 +610,11 @@ struct ClEngine {
             }
             if (!over && !early) send_all_x();
             if (tid < 32) {
-                if (!over) {
+                if (!over && !jacobi) {
                     const int nb = min(a + B, T);
-                    const Win nw = jacobi ? w : r.frontier_skip ? make_win(fin_h, nb - 1, lo, nb) : make_win(0, T, a, nb);
+                    const Win nw = r.frontier_skip ? make_win(fin_h, nb - 1, lo, nb) : make_win(0, T, a, nb);
                     for (int l = 0; l <= L; ++l) {
-                        const int2 rg = jacobi ? sh.rng[par][l] : live_range(l, nw);
+                        const int2 rg = live_range(l, nw);
                         if (lane == 0) sh.rng[par ^ 1][l] = rg;
                     }
                 }
@@ -618,7 +623,7 @@ struct ClEngine {
                     sh.chg[par ^ 1][0] = sh.chg[par ^ 1][1] = 0;
                     sh.first[par ^ 1] = INT_MAX;
                     __threadfence_block();
-                    mbar_arrive(&sh.go);
+                    if (!jacobi) mbar_arrive(&sh.go);
                 }
             }
             if (over) break;
@@ -654,16 +659,18 @@ made_cluster_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ C
         const int bend = min(jacobi ? T : r.block, T);
         const Win w = jacobi ? make_win(0, T, 0, T) : r.frontier_skip ? make_win(0, bend - 1, 0, bend) : make_win(0, T, 0, bend);
         const int2 rg = e.live_range(l, w);
-        if (lane == 0) { sh.nown[l] = n; sh.rng[0][l] = rg; }
+        if (lane == 0) { sh.nown[l] = n; sh.rng[0][l] = sh.rng[1][l] = rg; }
     }
     if (warp == 4 && lane == 0) {
-        for (int s = 0; s < MAX_STAGES; ++s) { mbar_init(&sh.full[s], 1); mbar_init(&sh.empty[s], 1); }
+        for (int s = 0; s < MAX_STAGES / 2; ++s) { mbar_init(&sh.full[s], 1); mbar_init(&sh.empty[s], 2); }
         for (int s = 0; s < NSLOT; ++s) { mbar_init(&sh.tfull[s], 2); mbar_init(&sh.tempty[s], 1); }
-        mbar_init(&sh.pbar, CS);
+        mbar_init(&sh.pbar[0], 1);
+        mbar_init(&sh.pbar[1], 1);
         mbar_init(&sh.go, 1);
-        mbar_init(&sh.ack, jacobi ? 2 : 3);
+        mbar_init(&sh.ack, 3);
         sh.stop = sh.dead = 0;
-        for (int h = 0; h < 2; ++h) sh.issued[h] = sh.consumed[h] = 0;
+        for (int i = 0; i < 2 * (CL_MAXL + 2); ++i) (&sh.apar[0][0])[i] = 0;
+        sh.issued = sh.consumed_loads = sh.consumed[0] = sh.consumed[1] = 0;
         sh.tiles = sh.sums[0] = sh.sums[1] = 0;
         for (int i = 0; i < 2; ++i) { sh.chg[i][0] = sh.chg[i][1] = 0; sh.first[i] = INT_MAX; }
     }
@@ -728,11 +735,11 @@ made_cluster_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ C
 
     int status = JS_OK, passes = 0, fin = 0;
     if (warp == 0) {
-        e.producer(jacobi);
+        if (elect_one()) e.producer(jacobi);
     } else if (warp == 1 || warp == 7) {
-        e.mma_issuer(warp == 7);
+        if (elect_one()) e.mma_issuer(warp == 7, jacobi);
     } else if (warp == 6) {
-        e.keeper(early);
+        e.keeper(early, jacobi);
     } else {
         fin = e.epilogue(jacobi, early, nrow, status, passes);
         if (fin < 0 && tid == 64) {          // a wait gave up: the other roles must not wait for a next pass
@@ -746,9 +753,7 @@ made_cluster_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ C
     __syncthreads();
     const bool alive = sh.dead == 0 && ld_volatile_i32(&r.ctl->abort) == 0;
     if (tid == 0 && alive)                   // weights that ran ahead: let them land
-        for (int h = 0; h < 2; ++h)
-            for (int n = sh.consumed[h], q = cd.n_stages >> 1; n < sh.issued[h]; ++n)
-                e.wait(&sh.full[2 * (n % q) + h], (uint32_t)(n / q) & 1u);
+        for (int n = sh.consumed_loads, q = cd.n_stages >> 1; n < sh.issued; ++n) e.wait(&sh.full[n % q], (uint32_t)(n / q) & 1u);
     // results: symbols of the own positions, counts
     if (warp >= 2 && warp < 6 && alive) {
         const int u = (warp & 3) * 16 + (lane & 15);
@@ -811,7 +816,7 @@ int js_cluster_prepare(js_model *mo)
     c.CS = most <= 2 ? 1 : most <= 4 ? 2 : most <= 8 ? 4 : 8;
     c.cs_log2 = c.CS == 1 ? 0 : c.CS == 2 ? 1 : c.CS == 4 ? 2 : 3;
     c.own_out = (c.nt[v.L] + c.CS - 1) / c.CS;
-    std::vector<CUtensorMap> maps(v.L + 1);
+    std::vector<CUtensorMap> maps(2 * (v.L + 1));
     c.kblocks = 0;
     for (int l = 0; l <= v.L; ++l) {
         const std::vector<int> &din = mo->host_deg[l], &dout = mo->host_deg[l + 1];
@@ -827,7 +832,10 @@ int js_cluster_prepare(js_model *mo)
             c.tiles.dmax[l][t] = (short)hi;
         }
         c.npad[l] = mo->tc.lay[l].npad;
-        if (!js_encode_map_2d(&maps[l], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, mo->tc_weights[l], c.nkb[l] * c.npad[l], BK, BK, TM)) return 0;
+        if (!js_encode_map_2d(&maps[2 * l], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, mo->tc_weights[l], c.nkb[l] * c.npad[l], BK, BK, TM)) return 0;
+        const cuuint64_t dims[3] = {BK, (cuuint64_t)c.npad[l], (cuuint64_t)c.nkb[l]}, strides[2] = {BK * 2, (cuuint64_t)c.npad[l] * BK * 2};
+        const cuuint32_t box[3] = {BK, TM, 2};
+        if (!js_encode_map(&maps[2 * l + 1], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, mo->tc_weights[l], 3, dims, strides, box)) return 0;
     }
     c.kblocks = (c.kblocks + c.CS - 1) / c.CS;
     // Encodings may be sent before the pass has ended everywhere if each CTA's last output tile reads hidden units of every
