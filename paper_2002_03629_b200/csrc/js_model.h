@@ -81,6 +81,8 @@ struct ClusterDev {
     int kblocks;                 // K blocks of weights a CTA reads per pass
     int early_ok;                // encodings may be sent as soon as they are sampled
     int n_stages;
+    unsigned char need[CL_MAXL + 1][8], off[CL_MAXL + 1][8];     // per layer and CTA: K blocks of a[l] that it reads, where it keeps them
+    int blocks;                  // most K blocks of activations in a CTA
     ClTiles tiles;
     const CUtensorMap *tmW;      // [L+1][2] tile-major weights: one K block of 64 units, two of them
 };

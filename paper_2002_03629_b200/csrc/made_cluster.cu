@@ -45,7 +45,7 @@ constexpr int STAGE = TM * BK * 2;           // 8 KB of weights
 constexpr int MAX_STAGES = 16;               // of 8 KB; they are used in pairs, an even K block and the odd one behind it
 constexpr int NSLOT = 2, ACC = 64;           // accumulator slots; columns of one accumulator (two per slot: even, odd K blocks)
 constexpr int MAXOWN = CL_TILES / 8;         // own tiles per layer (the cluster size grows with the tile count)
-constexpr int SMEM_MAX = 227 * 1024 - 11 * 1024;
+constexpr int SMEM_MAX = 227 * 1024 - 4 * 1024;      // beside ClShared
 
 struct ClShared {
     uint64_t full[MAX_STAGES / 2], empty[MAX_STAGES / 2], tfull[NSLOT], tempty[NSLOT];
@@ -68,8 +68,9 @@ struct ClShared {
     uint64_t apar[2][CL_MAXL + 2];
     unsigned tiles;
     unsigned sums[2];                        // of the whole cluster (in its first CTA): tiles, K blocks
-    float bias_s[CL_MAXL + 1][MAXOWN][TM];
+    unsigned char place[CL_MAXL][MAXOWN];    // this CTA's hidden tiles: K block of a[l + 1] that it keeps them in
 };
+static_assert(sizeof(ClShared) <= 4 * 1024, "SMEM_MAX leaves this much");
 
 __device__ __forceinline__ void copy_to_peer(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar)
 {
@@ -109,10 +110,11 @@ struct ClEngine {
     uint8_t *stag;                // [pass parity][own output tile][R x 128 bytes]: encodings on their way to the CTAs
     float *nz;                    // [own output tile][R][64]
     uint64_t *xs;                 // [own output tile][64]: bit s = symbol of sample s
+    float *bias;                  // [own tile of layer 0, 1, ..][64]
     const int R;
     int rank, CS, L, NP, warp, lane;          // NP: pairs in the weight ring
     uint32_t blk_bytes;           // one K block of activations: R x 128 bytes
-    int a_blk[CL_MAXL + 1];       // first K block of a[l] inside `acts`
+    int b_off[CL_MAXL + 1];       // first own tile of layer l in `bias`
 
     __device__ ClEngine(const MadeDev &m_, const ClusterDev &cd_, const RunArgs &r_, ClShared &sh_, uint8_t *base, int R_)
         : m(m_), cd(cd_), r(r_), sh(sh_), ring(base), R(R_)
@@ -125,17 +127,22 @@ struct ClEngine {
         lane = threadIdx.x & 31;
         blk_bytes = (uint32_t)R * 128u;
         acts = ring + (size_t)(2 * NP) * STAGE;
+        stag = acts + (size_t)cd.blocks * blk_bytes;
+        nz = reinterpret_cast<float *>(stag + (size_t)(2 * cd.own_out) * blk_bytes);
+        xs = reinterpret_cast<uint64_t *>(nz + (size_t)cd.own_out * R * TM);
+        bias = reinterpret_cast<float *>(xs + (size_t)cd.own_out * TM);
         int at = 0;
 #pragma unroll
         for (int l = 0; l <= CL_MAXL; ++l) {
-            a_blk[l] = at;
-            if (l <= L) at += cd.nkb[l];
+            b_off[l] = at;
+            if (l <= L) at += (cd.nt[l] + CS - 1) >> cd.cs_log2;
         }
-        stag = acts + (size_t)at * blk_bytes;
-        nz = reinterpret_cast<float *>(stag + (size_t)(2 * cd.own_out) * blk_bytes);
-        xs = reinterpret_cast<uint64_t *>(nz + (size_t)cd.own_out * R * TM);
     }
-    __device__ uint8_t *block(int l, int kb) const { return acts + (size_t)(a_blk[l] + kb) * blk_bytes; }
+    // A CTA keeps the K blocks of a[l] that its own tiles of layer l read, cd.need of them, and behind those what it sends
+    // of its tiles beyond (js_cluster_prepare: 39 blocks instead of 45 where 784 positions meet 1024 units x 2, which leaves
+    // the weights a fourth load in flight; 112 samples with three, four and five: 71.5, 66.7 and 66.0 us).
+    __device__ uint8_t *block(int l, int kb) const { return acts + (size_t)(cd.off[l][rank] + kb) * blk_bytes; }
+    __device__ uint32_t block_in(int peer, int l, int kb) const { return peer_addr(smem_u32(acts) + (uint32_t)(cd.off[l][peer] + kb) * blk_bytes, peer); }
     __device__ uint64_t *block_bar(int l, int kb, unsigned pass) const { return l == 0 ? &sh.xbar[pass & 1][kb] : &sh.hbar[l - 1][kb]; }
 
     // Tiles are dealt largest K range first, back and forth over the CTAs, in opposite directions in neighbouring layers.
@@ -362,7 +369,7 @@ struct ClEngine {
         auto arm = [&](int l, unsigned pass) {
             const int2 fr = fresh(l, pass);
             for (int kb = lane; kb < cd.nkb[l]; kb += 32)
-                if (in(fr, kb) && (l == 0 || owner(l - 1, kb) != rank)) mbar_expect_tx(block_bar(l, kb, pass), blk_bytes);
+                if (in(fr, kb) && kb < cd.need[l][rank] && (l == 0 || owner(l - 1, kb) != rank)) mbar_expect_tx(block_bar(l, kb, pass), blk_bytes);
         };
         auto drain = [&](int l, unsigned pass) {
             const int2 fr = fresh(l, pass);
@@ -371,7 +378,7 @@ struct ClEngine {
 #pragma unroll
             for (int q = 0; q < CL_MAXL + 2; ++q) ap = q == set ? apar[q] : ap;
             for (int kb = lane; kb < cd.nkb[l]; kb += 32)
-                if (in(fr, kb)) {
+                if (in(fr, kb) && kb < cd.need[l][rank]) {
                     if (!wait(block_bar(l, kb, pass), (uint32_t)(ap >> kb) & 1u)) on = false;
                     ap ^= 1ull << kb;
                 }
@@ -403,17 +410,14 @@ struct ClEngine {
                      : "=r"(all) : "r"((int)ok) : "memory");
         return all != 0;
     }
-    // Tile `tile` of layer l - 1 lies complete in this CTA's K block of a[l]: to the others.  Each epilogue warp serves two
-    // CTAs (the copies of one warp leave one after the other, 60 cycles apart).
-    __device__ void send(int l, int tile)
+    // Tile `tile` of layer l - 1 lies complete in this CTA's K block `place` of a[l]: to the others that read it.  Each epilogue warp serves
+    // two CTAs (the copies of one warp leave one after the other, 60 cycles apart).
+    __device__ void send(int l, int tile, int place)
     {
         const int peer = (warp & 3) * 2 + lane;
-        if (lane < 2 && peer < CS) {
+        if (lane < 2 && peer < CS && tile < cd.need[l][peer]) {
             if (peer == rank) mbar_arrive(&sh.hbar[l - 1][tile]);
-            else {
-                const uint32_t a = smem_u32(block(l, tile));
-                copy_to_peer(peer_addr(a, peer), a, blk_bytes, peer_addr(smem_u32(&sh.hbar[l - 1][tile]), peer));
-            }
+            else copy_to_peer(block_in(peer, l, tile), smem_u32(block(l, place)), blk_bytes, peer_addr(smem_u32(&sh.hbar[l - 1][tile]), peer));
         }
     }
     // Encodings of output tile `tile` from their staging buffer to every CTA, this one included, for pass `next`.  (They
@@ -423,8 +427,8 @@ struct ClEngine {
     __device__ void send_x(int tile, const uint8_t *src, unsigned next)
     {
         const int peer = (warp & 3) * 2 + lane;
-        if (lane < 2 && peer < CS)
-            copy_to_peer(peer_addr(smem_u32(block(0, tile)), peer), smem_u32(src), blk_bytes,
+        if (lane < 2 && peer < CS && tile < cd.need[0][peer])
+            copy_to_peer(block_in(peer, 0, tile), smem_u32(src), blk_bytes,
                          peer_addr(smem_u32(&sh.xbar[next & 1][tile]), peer));
     }
     // byte offset of unit u (0..63) of sample s inside a K block
@@ -438,12 +442,12 @@ struct ClEngine {
         tmem_ld8(tb, a);
         if (two) tmem_ld8(tb + ACC, b);
     }
-    // bias: of the tile's units.  A value goes from the thread that has it to its sample's row by a transposing store, eight samples
+    // bt: bias of the tile's units.  A value goes from the thread that has it to its sample's row by a transposing store, eight samples
     // of eight units at a time: lane = unit, with half the lanes idle and a 2-byte store per value, took 0.4 us longer.
     template <int ACT>
-    __device__ __forceinline__ void hidden_columns(uint32_t dst, uint32_t tb, bool two, const float *bias, int q)
+    __device__ __forceinline__ void hidden_columns(uint32_t dst, uint32_t tb, bool two, const float *bt, int q)
     {
-        const float b0 = bias[q * 16 + (lane >> 2)], b1 = bias[q * 16 + (lane >> 2) + 8];
+        const float b0 = bt[q * 16 + (lane >> 2)], b1 = bt[q * 16 + (lane >> 2) + 8];
         uint32_t na[4], nb[4] = {0, 0, 0, 0};
         tmem_ld_16x8(tb, na);
         if (two) tmem_ld_16x8(tb + ACC, nb);
@@ -512,17 +516,17 @@ struct ClEngine {
                     const int tile = sh.own[l][j].x;
                     if (!in(sh.rng[par][l], tile)) continue;
                     const bool two = sh.own[l][j].y > 1;
-                    const float *bias = sh.bias_s[l][j];
+                    const float *bt = bias + (size_t)(b_off[l] + j) * TM;
                     const bool ok = __all_sync(0xffffffffu, wait(&sh.tfull[slot], spar >> slot & 1u));
                     tc_fence_after();
                     const uint32_t tb = sh.tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(2 * slot * ACC);
                     if (l < L) {
-                        const uint32_t dst = smem_u32(block(l + 1, tile));
-                        if (m.act == JS_ACT_RELU) hidden_columns<JS_ACT_RELU>(dst, tb, two, bias, q);
-                        else hidden_columns<JS_ACT_GELU_TANH>(dst, tb, two, bias, q);
+                        const uint32_t dst = smem_u32(block(l + 1, sh.place[l][j]));
+                        if (m.act == JS_ACT_RELU) hidden_columns<JS_ACT_RELU>(dst, tb, two, bt, q);
+                        else hidden_columns<JS_ACT_GELU_TANH>(dst, tb, two, bt, q);
                     } else {
                         const int p = tile * TM + u;
-                        const float bv = bias[u];
+                        const float bv = bt[u];
                         const bool mine = act_lane && p >= w.plo && p < w.phi;
                         uint8_t *dst = stag + (size_t)(par * cd.own_out + j) * blk_bytes;
                         const float *nzt = nz + (size_t)j * R * TM + u;
@@ -554,7 +558,7 @@ struct ClEngine {
                     fence_proxy_async_smem();
                     if (!ep_all(ok)) return -1;
                     if (tid == 0) mbar_arrive(&sh.tempty[slot]);
-                    if (l < L) send(l + 1, tile);
+                    if (l < L) send(l + 1, tile, sh.place[l][j]);
                     spar ^= 1u << slot;
                     slot = (slot + 1) % NSLOT;
                 }
@@ -648,13 +652,20 @@ made_cluster_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ C
     // this CTA's tiles, per layer a warp; the first pass's ranges; barriers
     if (warp <= L) {
         const int l = warp;
-        int n = 0;
+        int n = 0, beyond = 0;
+        const int need = l < L ? cd.need[l + 1][e.rank] : 0;
         for (int t0 = 0; t0 < cd.nt[l]; t0 += 32) {
             const int t = t0 + lane;
             const bool mine = t < cd.nt[l] && e.owner(l, t) == e.rank;
             const unsigned bal = __ballot_sync(0xffffffffu, mine);
-            if (mine) sh.own[l][n + __popc(bal & ((1u << lane) - 1u))] = make_int2(t, cd.tiles.kbe[l][t]);
+            const unsigned far = __ballot_sync(0xffffffffu, mine && t >= need), before = (1u << lane) - 1u;
+            if (mine) {
+                const int j = n + __popc(bal & before);
+                sh.own[l][j] = make_int2(t, cd.tiles.kbe[l][t]);
+                if (l < L) sh.place[l][j] = (unsigned char)(t < need ? t : need + beyond + __popc(far & before));
+            }
             n += __popc(bal);
+            beyond += __popc(far);
         }
         const int bend = min(jacobi ? T : r.block, T);
         const Win w = jacobi ? make_win(0, T, 0, T) : r.frontier_skip ? make_win(0, bend - 1, 0, bend) : make_win(0, T, 0, bend);
@@ -680,7 +691,7 @@ made_cluster_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ C
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     if (warp == 5) tmem_alloc(&sh.tmem_base, NSLOT * 2 * ACC);
     // activations start as zeros (padding units and samples stay finite)
-    for (int i = tid; i < (e.a_blk[L] + cd.nkb[L]) * (int)(e.blk_bytes / 16); i += NTH)
+    for (int i = tid; i < cd.blocks * (int)(e.blk_bytes / 16); i += NTH)
         reinterpret_cast<uint4 *>(e.acts)[i] = make_uint4(0, 0, 0, 0);
     __syncthreads();
     // noise of the own positions: asynchronous copies, waited for below
@@ -707,12 +718,12 @@ made_cluster_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ C
     for (int l = 0; l <= L; ++l)
         for (int i = tid; i < sh.nown[l] * TM; i += NTH) {
             const int u = sh.own[l][i / TM].x * TM + i % TM;
-            sh.bias_s[l][i / TM][i % TM] = u < m.n[l + 1] ? __ldg(m.bias[l] + u) : 0.0f;
+            e.bias[e.b_off[l] * TM + i] = u < m.n[l + 1] ? __ldg(m.bias[l] + u) : 0.0f;
         }
     {
         // the iterate's encodings, eight positions (16 bytes) at a time
         const __nv_bfloat16 e0 = __float2bfloat16_rn(m.lut[0]), e1 = __float2bfloat16_rn(m.lut[1]);
-        const int chunks = (T + 7) / 8;
+        const int chunks = min((T + 7) / 8, (int)cd.need[0][e.rank] * (TM / 8));
         for (int s = warp; s < nrow; s += NTH / 32)
             for (int c = lane; c < chunks; c += 32) {
                 const int p0 = c * 8;
@@ -792,9 +803,16 @@ made_cluster_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ C
 // --------------------------------------------------------------- host side
 static size_t cluster_smem(const ClusterDev &c, const MadeDev &v, int R, int n_stages)
 {
-    int blocks = 0;
-    for (int l = 0; l <= v.L; ++l) blocks += c.nkb[l];
-    return 1024 + (size_t)n_stages * STAGE + (size_t)(blocks + 2 * c.own_out) * R * 128 + (size_t)c.own_out * (R * TM * 4 + TM * 8);
+    int own = 0;
+    for (int l = 0; l <= v.L; ++l) own += (c.nt[l] + c.CS - 1) / c.CS;
+    return 1024 + (size_t)n_stages * STAGE + (size_t)(c.blocks + 2 * c.own_out) * R * 128 + (size_t)c.own_out * (R * TM * 4 + TM * 8) + (size_t)own * TM * 4;
+}
+
+// which CTA of a cluster has a tile (ClEngine::owner)
+static int cluster_owner(const ClusterDev &c, int l, int tile)
+{
+    const int q = c.nt[l] - 1 - tile, round = q >> c.cs_log2, pos = q & (c.CS - 1);
+    return ((round ^ l) & 1) ? c.CS - 1 - pos : pos;
 }
 
 // Builds the view of a model for this kernel: 1 if it qualifies, 0 if not, negative on CUDA errors.  Needs the tile-major
@@ -838,14 +856,28 @@ int js_cluster_prepare(js_model *mo)
         if (!js_encode_map(&maps[2 * l + 1], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, mo->tc_weights[l], 3, dims, strides, box)) return 0;
     }
     c.kblocks = (c.kblocks + c.CS - 1) / c.CS;
+    // K blocks of activations per CTA: those that its tiles read, then its own tiles beyond them
+    c.blocks = 0;
+    for (int i = 0; i < c.CS; ++i) {
+        int at = 0;
+        for (int l = 0; l <= v.L; ++l) {
+            int need = 0, own = 0;
+            for (int t = 0; t < c.nt[l]; ++t)
+                if (cluster_owner(c, l, t) == i) need = std::max(need, (int)c.tiles.kbe[l][t]);
+            for (int t = need; l > 0 && t < c.nt[l - 1]; ++t) own += cluster_owner(c, l - 1, t) == i;
+            c.off[l][i] = (unsigned char)at;
+            c.need[l][i] = (unsigned char)need;
+            at += need + own;
+        }
+        c.blocks = std::max(c.blocks, at);
+    }
     // Encodings may be sent before the pass has ended everywhere if each CTA's last output tile reads hidden units of every
     // CTA, in a layer above the first: a CTA issues its MMAs in order, so all of them have then done the first layer.
     c.early_ok = v.L >= 2 && c.nt[v.L] >= c.CS ? 1 : 0;
     for (int i = 0; i < c.CS && c.early_ok; ++i) {
         unsigned seen = 0;
         for (int kb = 0; kb < c.tiles.kbe[v.L][c.nt[v.L] - 1 - i]; ++kb) {
-            const int l = v.L - 1, q = c.nt[l] - 1 - kb, round = q >> c.cs_log2, pos = q & (c.CS - 1);
-            seen |= 1u << (((round ^ l) & 1) ? c.CS - 1 - pos : pos);
+            seen |= 1u << cluster_owner(c, v.L - 1, kb);
         }
         if (seen != (1u << c.CS) - 1u) c.early_ok = 0;
     }
