@@ -668,8 +668,8 @@ made_cluster_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ C
             beyond += __popc(far);
         }
         const int bend = min(jacobi ? T : r.block, T);
-        const Win w = jacobi ? make_win(0, T, 0, T) : r.frontier_skip ? make_win(0, bend - 1, 0, bend) : make_win(0, T, 0, bend);
-        const int2 rg = e.live_range(l, w);
+        // (the whole of every layer in Jacobi mode)
+        const int2 rg = jacobi ? make_int2(0, cd.nt[l]) : e.live_range(l, r.frontier_skip ? make_win(0, bend - 1, 0, bend) : make_win(0, T, 0, bend));
         if (lane == 0) { sh.nown[l] = n; sh.rng[0][l] = sh.rng[1][l] = rg; }
     }
     if (warp == 4 && lane == 0) {
@@ -690,9 +690,6 @@ made_cluster_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ C
     for (int i = tid; i < 64; i += NTH) sh.count[i] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     if (warp == 5) tmem_alloc(&sh.tmem_base, NSLOT * 2 * ACC);
-    // activations start as zeros (padding units and samples stay finite)
-    for (int i = tid; i < cd.blocks * (int)(e.blk_bytes / 16); i += NTH)
-        reinterpret_cast<uint4 *>(e.acts)[i] = make_uint4(0, 0, 0, 0);
     __syncthreads();
     // noise of the own positions: asynchronous copies, waited for below
     for (int j = 0; j < sh.nown[L]; ++j) {
@@ -714,24 +711,36 @@ made_cluster_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ C
             e.xs[j * TM + i] = x;
         }
     }
-    // biases of the own tiles
+    // biases of the own tiles, likewise
     for (int l = 0; l <= L; ++l)
         for (int i = tid; i < sh.nown[l] * TM; i += NTH) {
             const int u = sh.own[l][i / TM].x * TM + i % TM;
-            e.bias[e.b_off[l] * TM + i] = u < m.n[l + 1] ? __ldg(m.bias[l] + u) : 0.0f;
+            const bool in = u < m.n[l + 1];
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(e.bias + e.b_off[l] * TM + i)), "l"(m.bias[l] + (in ? u : 0)), "r"(in ? 4 : 0)
+                         : "memory");
         }
+    // In a window a tile may read K blocks that are not computed yet: zeros.
+    if (!jacobi)
+        for (int i = tid; i < cd.blocks * (int)(e.blk_bytes / 16); i += NTH) reinterpret_cast<uint4 *>(e.acts)[i] = make_uint4(0, 0, 0, 0);
     {
-        // the iterate's encodings, eight positions (16 bytes) at a time
-        const __nv_bfloat16 e0 = __float2bfloat16_rn(m.lut[0]), e1 = __float2bfloat16_rn(m.lut[1]);
-        const int chunks = min((T + 7) / 8, (int)cd.need[0][e.rank] * (TM / 8));
-        for (int s = warp; s < nrow; s += NTH / 32)
-            for (int c = lane; c < chunks; c += 32) {
+        // The iterate's encodings, eight positions (16 bytes) at a time.  From zeros the K blocks that lie inside the image are one value
+        // throughout, whatever the order of their chunks (samples that are not there included: nothing is taken from their columns);
+        // zeros behind the last position.
+        const __nv_bfloat16 e0 = __float2bfloat16_rn(m.lut[0]), e1 = __float2bfloat16_rn(m.lut[1]), z0 = __float2bfloat16_rn(0.0f);
+        const int need = cd.need[0][e.rank], whole = r.init ? 0 : min(need, T / TM);
+        if (!jacobi) __syncthreads();
+        const __nv_bfloat162 e2 = __halves2bfloat162(e0, e0);
+        const uint32_t w = *reinterpret_cast<const uint32_t *>(&e2);
+        for (int i = tid; i < whole * (int)(e.blk_bytes / 16); i += NTH) reinterpret_cast<uint4 *>(e.block(0, 0))[i] = make_uint4(w, w, w, w);
+        const int c0 = whole * (TM / 8), chunks = need * (TM / 8);
+        for (int s = warp; s < R; s += NTH / 32)
+            for (int c = c0 + lane; c < chunks; c += 32) {
                 const int p0 = c * 8;
                 alignas(16) __nv_bfloat16 v[8];
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
-                    const bool one = r.init && p0 + k < T && r.init[(size_t)(row0 + s) * T + p0 + k] != 0;
-                    v[k] = p0 + k < T ? (one ? e1 : e0) : __float2bfloat16_rn(0.0f);
+                    const bool in = s < nrow && p0 + k < T, one = in && r.init && r.init[(size_t)(row0 + s) * T + p0 + k] != 0;
+                    v[k] = in ? (one ? e1 : e0) : z0;
                 }
                 *reinterpret_cast<uint4 *>(e.block(0, p0 / TM) + ClEngine::at_block(s, p0 % TM)) = *reinterpret_cast<const uint4 *>(v);
             }
