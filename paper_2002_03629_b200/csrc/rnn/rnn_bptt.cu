@@ -414,6 +414,12 @@ __device__ __forceinline__ void sts4(uint32_t at, const uint32_t (&r)[4])
 {
     asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
 }
+// Eight columns of sixteen accumulator lanes, over all threads of a warp: lane i gets columns 2 (i % 4) and the next of rows i / 4
+// (r[0], r[1]) and i / 4 + 8 (r[2], r[3]).
+__device__ __forceinline__ void tmem_ld_16x8(uint32_t taddr, uint32_t (&r)[4])
+{
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(taddr) : "memory");
+}
 // two values in three bf16 pieces each, packed (the first in the low half)
 __device__ __forceinline__ void cut3(float a, float b, uint32_t &h, uint32_t &m, uint32_t &l)
 {
@@ -426,15 +432,15 @@ __device__ __forceinline__ void cut3(float a, float b, uint32_t &h, uint32_t &m,
     l = pack_bf16x2(a, b);
 }
 // bounded: true once the barrier's phase has completed, false after 2 s or when another wait of the CTA has given up
-__device__ __forceinline__ bool jac_wait(JacShared &sh, uint64_t *bar, uint32_t parity)
+__device__ __forceinline__ bool jac_wait(int &dead, uint64_t *bar, uint32_t parity)
 {
     if (mbar_try_wait(bar, parity)) return true;
     const uint64_t t0 = global_ns();
     for (unsigned i = 1;; ++i) {
         if (mbar_try_wait(bar, parity)) return true;
-        if ((i & 63u) == 0u && (*(volatile int *)&sh.dead || global_ns() - t0 > MBAR_WAIT_NS)) break;
+        if ((i & 63u) == 0u && (*(volatile int *)&dead || global_ns() - t0 > MBAR_WAIT_NS)) break;
     }
-    *(volatile int *)&sh.dead = 1;
+    *(volatile int *)&dead = 1;
     return false;
 }
 // barrier of the epilogue warps: did every thread say yes?
@@ -556,7 +562,7 @@ rnn_bptt_jacobi_kernel(const float *__restrict__ Wh, const float *l, const float
                 bool on = true;
                 for (int u = blockIdx.x; u < units && on; u += gridDim.x)
                     for (int it = 0; it < nmma && on; ++it, par ^= 1u) {
-                        on = __all_sync(0xffffffffu, jac_wait(sh, &sh.ready[slot], par));
+                        on = __all_sync(0xffffffffu, jac_wait(sh.dead, &sh.ready[slot], par));
                         if (!on) break;
                         tc_fence_after();
                         if (elect_one()) {
@@ -588,7 +594,7 @@ rnn_bptt_jacobi_kernel(const float *__restrict__ Wh, const float *l, const float
             const int cols = min(width, (B - u * per_unit) * T);
             const size_t base = (size_t)u * per_unit * T * H + i;
             bool ok = true;
-            if (stages) ok = jac_wait(sh, &sh.staged, staged_par);
+            if (stages) ok = jac_wait(sh.dead, &sh.staged, staged_par);
             staged_par ^= 1u;
             const float *lp = stages ? ls + i : l + base, *dp = stages ? ds + i : d + base;
             float lv[2][JC], dv[2][JC], l0 = 0.0f;
@@ -734,7 +740,7 @@ rnn_bptt_jacobi_kernel(const float *__restrict__ Wh, const float *l, const float
 #pragma unroll
                 for (int k = 1; k >= 0; --k) {
                     if (k == 1 && !two) continue;
-                    ok = __all_sync(0xffffffffu, jac_wait(sh, &sh.full[k], par));
+                    ok = __all_sync(0xffffffffu, jac_wait(sh.dead, &sh.full[k], par));
                     if (!ok) break;
                     tc_fence_after();
                     finish(k, last);
@@ -781,17 +787,199 @@ __global__ void rnn_copy_kernel(const float *s0, float *s, size_t n)
 }
 
 // ------------------------------------------------------------------ parameter gradients
-// dWh = sum_t g_t h_{t-1}^T with g_t = d_t * s_t: a [128 x T] x [T x 64] product per CTA (two CTAs per sequence), 128
-// threads with 8 x 8 outputs each (rows 4 ty.. and 64 + 4 ty.., columns 4 tx.. and 32 + 4 tx..).  The steps come in
-// chunks of GC through two small shared-memory buffers, the next chunk's loads in registers while one is multiplied, so
-// that several CTAs share an SM and one's loads and stores hide behind another's arithmetic; before, a CTA held all
-// steps (128 KB) and its three stages ran one after another.  db and dWx ride along: the same sums with 1 and x_t on
-// the right.  T = 100, H = 128 (B200): batch 1 31 -> 17 us, batch 592 191 -> 79 us (60 MB in, 39 MB out).
+// dWh = sum_t g_t h_{t-1}^T with g_t = d_t * s_t: a [128 x T] x [T x 128] product per sequence, on the tensor cores like the Jacobi
+// iterations: three bf16 pieces of either side, six products, the five small ones in an accumulator of their own.  Both operands lie
+// in shared memory as they come, components together, steps in rows (PK of them at a time, so that two CTAs share an SM and one's
+// loads and stores pass while the other multiplies).  A CTA computes `cols` columns of one sequence: all of them, or a half or a
+// quarter where there are few sequences.  db and dWx, the same sums with 1 and x_t on the right, are taken up while the operands are cut:
+// a warp sums the steps that it cuts, the warps' sums are added in order.
+// Values that the pieces cannot carry (infinities, NaN, beyond what bf16 reaches): plain multiply-adds, as in jac_plain.
+// T = 100, H = 128 (B200): batch 592 45 us (60 MB in, 39 MB out: 15 us), batch 1 11; multiply-adds on the CUDA cores took 75 and 16.  Against 64 bits
+// dWh is off by 1.1e-7 in the 2-norm, 1.8e-7 before.  Bound: a CTA's chain of loads, cutting, MMAs and stores, twice per SM.
+constexpr int PK = 64, PGT = 256;            // steps at a time, threads
+constexpr int P_PIECE = PK * MH * 2;         // bytes of a piece: [two groups of 64 components][PK steps][128 bytes, swizzled]
+constexpr size_t P_SMEM = 6 * P_PIECE + 1024;
+
+// NX: room for that many inputs
+template <bool VEC, int NX>
+__global__ void __launch_bounds__(PGT, 2)
+rnn_param_grads_kernel(const float *__restrict__ s, const float *__restrict__ d, const float *__restrict__ h,
+                       const float *__restrict__ x, int T, int H, int d_in, int cols, float *__restrict__ dWh,
+                       float *__restrict__ dWx, float *__restrict__ db)
+{
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ uint64_t done;
+    __shared__ uint32_t tmem;
+    __shared__ int dead;
+    uint8_t *ops = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);    // pieces of g, then of h
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, seq = blockIdx.x, n0 = blockIdx.y * cols;
+    const size_t base = (size_t)seq * T * H;
+    const bool extra = blockIdx.y == 0;
+    if (tid == 0) {
+        mbar_init(&done, 1);
+        dead = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) tmem_alloc(&tmem, 256);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tm = tmem;
+    const int i4 = lane * 4;
+    float sx[1 + NX][4];                                 // db, then dWx
+#pragma unroll
+    for (int c = 0; c <= NX; ++c)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) sx[c][e] = 0.0f;
+    bool fine = true, ok = true;
+    // four neighbouring components of step row r of an operand, in pieces
+    auto put = [&](uint8_t *op, int r, const float (&v)[4]) {
+        uint32_t ph[2], pm[2], pl[2];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            cut3(v[2 * e], v[2 * e + 1], ph[e], pm[e], pl[e]);
+            fine = fine && fabsf(v[2 * e]) <= 3.38e38f && fabsf(v[2 * e + 1]) <= 3.38e38f;
+        }
+        const uint32_t at = smem_u32(op) + (uint32_t)((i4 >> 6) * (PK * 128) + r * 128 + ((((i4 & 63) >> 3) ^ (r & 7)) << 4) + (i4 & 7) * 2);
+        asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(at), "r"(ph[0]), "r"(ph[1]) : "memory");
+        asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(at + P_PIECE), "r"(pm[0]), "r"(pm[1]) : "memory");
+        asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(at + 2 * P_PIECE), "r"(pl[0]), "r"(pl[1]) : "memory");
+    };
+    uint32_t par = 0;
+    for (int t0 = 0; t0 < T; t0 += PK, par ^= 1u) {
+        if (t0 > 0) {                                    // the steps before have been multiplied
+            ok = jac_wait(dead, &done, par ^ 1u);
+            if (!__syncthreads_and(ok)) { ok = false; break; }
+        }
+        const int rows = (min(PK, T - t0) + 15) / 16 * 16;
+#pragma unroll (NX <= 4 ? 4 : 2)
+        for (int r = warp; r < rows; r += PGT / 32) {
+            const int t = t0 + r;
+            const bool in = t < T && i4 < H, hin = in && t >= 1;
+            const size_t at = base + (size_t)t * H + i4;
+            const float4 a = in ? ldg4<VEC>(d + at) : make_float4(0, 0, 0, 0), b = in ? ldg4<VEC>(s + at) : make_float4(0, 0, 0, 0);
+            const float4 hv = hin ? ldg4<VEC>(h + at - H) : make_float4(0, 0, 0, 0);
+            const float gv[4] = {a.x * b.x, a.y * b.y, a.z * b.z, a.w * b.w};
+            put(ops, r, gv);
+            const float hh[4] = {hv.x, hv.y, hv.z, hv.w};
+            put(ops + 3 * P_PIECE, r, hh);
+            if (extra && t < T) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) sx[0][e] += gv[e];
+#pragma unroll
+                for (int c = 0; c < NX; ++c)
+                    if (c < d_in) {
+                        const float xv = __ldg(x + ((size_t)seq * T + t) * d_in + c);
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) sx[c + 1][e] = fmaf(gv[e], xv, sx[c + 1][e]);
+                    }
+            }
+        }
+        fence_proxy_async_smem();
+        tc_fence_before();
+        __syncthreads();
+        if (warp == 0 && elect_one()) {
+            tc_fence_after();
+            // both operands lie with neighbouring components together ("MN-major": bits 15 and 16)
+            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (3u << 15) | ((uint32_t)(MH >> 4) << 24) | ((uint32_t)(cols >> 3) << 17);
+            // groups of 64 components PK x 128 bytes apart, of eight steps 1024
+            const uint64_t lead = (uint64_t)((PK * 128 >> 4) - 1) << 16;      // (the descriptor comes with 1)
+            const uint64_t ad0 = smem_desc_sw128(smem_u32(ops)) + lead;
+            const uint64_t bd0 = smem_desc_sw128(smem_u32(ops + 3 * P_PIECE + (n0 >> 6) * (PK * 128)) + (uint32_t)((n0 & 63) * 2)) + lead;
+            constexpr uint64_t PC = P_PIECE >> 4, K16 = 2048 >> 4;
+            const uint32_t dm = tm, dc = tm + MH;
+            uint64_t a = ad0, b = bd0;
+#pragma unroll 1
+            for (int k = 0; k < rows; k += 16, a += K16, b += K16) {
+                const bool on = t0 > 0 || k > 0;
+                umma_bf16(dc, a + 2 * PC, b, idesc, on);
+                umma_bf16(dc, a, b + 2 * PC, idesc, 1u);
+                umma_bf16(dc, a + PC, b + PC, idesc, 1u);
+                umma_bf16(dc, a + PC, b, idesc, 1u);
+                umma_bf16(dc, a, b + PC, idesc, 1u);
+                umma_bf16(dm, a, b, idesc, on);
+            }
+            umma_commit(&done);
+        }
+        __syncwarp();
+    }
+    if (ok) ok = jac_wait(dead, &done, par ^ 1u);
+    ok = __syncthreads_and(ok) != 0;
+    const bool plain = !__syncthreads_and(fine);
+    tc_fence_after();
+    float *out = dWh + (size_t)seq * H * H;
+    if (!ok || plain) {
+        for (int p = tid; p < H * cols; p += PGT) {
+            const int i = p / cols, j = n0 + p % cols;
+            if (j >= H) continue;
+            float acc = ok ? 0.0f : NAN;
+            for (int t = 1; ok && t < T; ++t) {
+                const size_t at = base + (size_t)t * H;
+                acc = fmaf(d[at + i] * s[at + i], h[at - H + j], acc);
+            }
+            out[(size_t)i * H + j] = acc;
+        }
+    } else {
+        // a warp takes sixteen rows of its quadrant and half of the columns at a time: eight rows of 32 bytes a store
+        const int q = warp & 3, half = cols / 2, c0 = (warp >> 2) * half;
+#pragma unroll 1
+        for (int rr = 0; rr < 32; rr += 16)
+#pragma unroll 1
+            for (int c = c0; c < c0 + half; c += 8) {
+                const uint32_t at = tm + ((uint32_t)(q * 32 + rr) << 16) + (uint32_t)c;
+                uint32_t a[4], b[4];
+                tmem_ld_16x8(at, a);
+                tmem_ld_16x8(at + MH, b);
+                tmem_wait_ld();
+                float v[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) v[e] = __uint_as_float(a[e]) + __uint_as_float(b[e]);
+                const int j = n0 + c + 2 * (lane & 3);
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int i = q * 32 + rr + (lane >> 2) + 8 * e;
+                    if (i < H && j < H) {                // (H is even)
+                        float *to = out + (size_t)i * H + j;
+                        if constexpr (VEC) *reinterpret_cast<float2 *>(to) = make_float2(v[2 * e], v[2 * e + 1]);
+                        else { to[0] = v[2 * e]; to[1] = v[2 * e + 1]; }
+                    }
+                }
+            }
+    }
+    if (extra) {
+        // the warps' sums through the operands' memory
+        float *sums = reinterpret_cast<float *>(ops);        // [warp][1 + d_in][MH]
+        const int n = 1 + d_in;
+        if (ok)                                              // (else the MMAs may still read there)
+#pragma unroll
+            for (int c = 0; c <= NX; ++c)
+                if (c < n) *reinterpret_cast<float4 *>(sums + (warp * n + c) * MH + i4) = make_float4(sx[c][0], sx[c][1], sx[c][2], sx[c][3]);
+        __syncthreads();
+        for (int p = tid; p < n * MH; p += PGT) {
+            const int c = p / MH, i = p % MH;
+            if (i >= H) continue;
+            float t = ok ? 0.0f : NAN;
+            for (int w = 0; ok && w < PGT / 32; ++w) t += sums[(w * n + c) * MH + i];
+            if (c == 0) db[(size_t)seq * H + i] = t;
+            else dWx[((size_t)seq * H + i) * d_in + c - 1] = t;
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) {
+        tc_fence_after();
+        tmem_dealloc(tm, 256);
+    }
+}
+
+// Few steps: multiply-adds on the CUDA cores, a [128 x T] x [T x 64] product per CTA (two CTAs per sequence), 128 threads with 8 x 8 outputs
+// each (rows 4 ty.. and 64 + 4 ty.., columns 4 tx.. and 32 + 4 tx..), the steps in chunks of GC through two small shared-memory buffers, the
+// next chunk's loads in registers while one is multiplied.  db and dWx ride along: the same sums with 1 and x_t on the right.
 constexpr int GC = 16, GN = 64, GTH = 128;
 
 template <bool VEC>
 __global__ void __launch_bounds__(GTH)
-rnn_param_grads_kernel(const float *__restrict__ s, const float *__restrict__ d, const float *__restrict__ h,
+rnn_param_grads_short_kernel(const float *__restrict__ s, const float *__restrict__ d, const float *__restrict__ h,
                        const float *__restrict__ x, int T, int H, int d_in, float *__restrict__ dWh,
                        float *__restrict__ dWx, float *__restrict__ db)
 {
@@ -979,8 +1167,21 @@ int rnn_param_grads(const float *s, const float *d, const float *h, const float 
                     float *dWh, float *dWx, float *db, void *stream)
 {
     if (!s || !d || !h || !x || !dWh || !dWx || !db || !sizes_ok(B, T, H) || d_in < 1 || d_in > MIO) return RNN_ERR_INVALID;
-    auto kernel = vectors(s, d, h, dWh) ? rnn_param_grads_kernel<true> : rnn_param_grads_kernel<false>;
-    kernel<<<dim3(B, (H + GN - 1) / GN), GTH, 0, (cudaStream_t)stream>>>(s, d, h, x, T, H, d_in, dWh, dWx, db);
+    const bool vec = vectors(s, d, h, dWh);
+    // Tensor memory and operands cost a CTA about a microsecond: 12 steps, H = 32, batch 1 and 300: 4.2 and 8.2 us that way, 3.5 and 5.4 this;
+    // 13 steps, H = 92, batch 2: 4.4 and 3.9; 30 steps, H = 60, batch 592: 12.5 and 16.8; 31 steps, batch 59: 5.9 and 6.4.
+    if (T <= 24) {
+        auto few = vec ? rnn_param_grads_short_kernel<true> : rnn_param_grads_short_kernel<false>;
+        few<<<dim3(B, (H + GN - 1) / GN), GTH, 0, (cudaStream_t)stream>>>(s, d, h, x, T, H, d_in, dWh, dWx, db);
+        return launch_status();
+    }
+    auto kernel = d_in <= 4 ? (vec ? rnn_param_grads_kernel<true, 4> : rnn_param_grads_kernel<false, 4>)
+                            : (vec ? rnn_param_grads_kernel<true, MIO> : rnn_param_grads_kernel<false, MIO>);
+    // columns per CTA: all where there are sequences for all SMs, else a half, a quarter
+    const int sms = sm_count(), all = (H + 31) / 32 * 32;
+    const int cols = B >= sms ? all : B >= sms / 2 ? std::min(all, MH / 2) : std::min(all, MH / 4);
+    if (!allow_smem(kernel, P_SMEM, vec + 2 * (d_in <= 4))) return RNN_ERR_CUDA;
+    kernel<<<dim3(B, (H + cols - 1) / cols), PGT, P_SMEM, (cudaStream_t)stream>>>(s, d, h, x, T, H, d_in, cols, dWh, dWx, db);
     return launch_status();
 }
 

@@ -1,5 +1,6 @@
-"""Jacobi iterations of the recurrent network on the tensor cores, where the kernel can go wrong: one and two slots of 64 columns,
-several sequences in a unit and a ragged last unit, components around 16, 64 and 128, values that bf16 pieces cannot carry."""
+"""Jacobi iterations and parameter gradients of the recurrent network on the tensor cores, where the kernels can go wrong: one and two
+slots of 64 columns, several sequences in a unit and a ragged last unit, components around 16, 64 and 128, one and two chunks of
+steps, all, half or a quarter of the columns per CTA, values that bf16 pieces cannot carry."""
 import numpy as np
 import pytest
 import torch
@@ -83,3 +84,27 @@ def test_in_place():
     for which in range(3):
         a = [l.clone(), d.clone(), s0.clone()]
         assert torch.equal(rnn.rnn_bptt_jacobi(W, a[0], a[1], 6, s0=a[2], out=a[which]), want)
+
+
+@pytest.mark.parametrize("B,T,H,d_in", [(1, 25, 4, 1), (1, 64, 32, 3), (2, 65, 36, 4), (1, 128, 128, 16), (74, 48, 100, 1), (75, 66, 64, 5), (148, 63, 68, 2),
+                                        (300, 127, 128, 1), (2, 24, 128, 2)])
+def test_parameter_gradients_against_64_bits(B, T, H, d_in):
+    import paper_2002_03629_b200.rnn as rnn
+    _, s, d, h = draw(B, T, H)
+    x = torch.rand((B, T, d_in), device="cuda")
+    g = d.double() * s.double()
+    want = torch.einsum("bti,btj->bij", g[:, 1:], h.double()[:, :-1]), torch.einsum("bti,btc->bic", g, x.double()), g.sum(1)
+    for a, b in zip(rnn.rnn_param_grads(s, d, h, x), want):
+        assert ((a.double() - b).norm() / b.norm()).item() < 7e-7
+    # a value that the pieces cannot carry: its sequence alone, the entries that it reaches alone
+    s[0, T - 1, 1] = float("inf")
+    h[0, 0, 2] = 3.39e38
+    s[0, 1] = s[0, 1].abs() * 1e-30
+    dWh, _, db = rnn.rnn_param_grads(s, d, h, x)
+    g = d.double() * s.double()
+    row = torch.arange(H, device="cuda") != 1
+    want = torch.einsum("ti,tj->ij", g[0, 1:], h[0].double()[:-1])[row]
+    assert torch.isfinite(dWh[0, row]).all() and not torch.isfinite(dWh[0, 1]).any() and not torch.isfinite(db[0, 1])
+    assert ((dWh[0, row].double() - want).abs() <= 1e-5 * want.abs() + 1e-4).all()
+    if B > 1:
+        assert torch.isfinite(dWh[1:]).all()
