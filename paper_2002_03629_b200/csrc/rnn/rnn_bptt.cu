@@ -54,6 +54,19 @@ __device__ __forceinline__ void stg4(float *p, float4 v)
 // computed once per output.
 constexpr int CT = 128;          // threads
 
+// two fp32 values in a register pair; a multiply-add on both
+__device__ __forceinline__ unsigned long long pair(float lo, float hi)
+{
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c)
+{
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
 struct MatvecTile {
     float w[4][MH / 4];
 };
@@ -79,6 +92,27 @@ __device__ __forceinline__ void tile_dot(const MatvecTile &t, const float *v, in
 #pragma unroll
     for (int u = 0; u < 4; ++u) out[u] = c0[u] + c1[u];
 }
+// The same by packed multiply-adds, the same values: half the instructions leave the schedulers to the forward pass's second group of
+// warps (batch 1: 38 -> 35 us, 592: 116 -> 111, T = 64, H = 64, batch 30: 27 -> 23).  Back-substitution, which has the schedulers to
+// itself, is slower with them (24 -> 26, 61 -> 65 us).
+__device__ __forceinline__ void tile_dot2(const MatvecTile &t, const float *v, int q, float (&out)[4])
+{
+    const ulonglong2 *p = reinterpret_cast<const ulonglong2 *>(v) + q;
+    // eight chains, two to a packed multiply-add (inputs of even and of odd number)
+    unsigned long long c[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) c[u] = 0ull;
+#pragma unroll
+    for (int m = 0; m < MH / 16; ++m) {
+        const ulonglong2 x = p[4 * m];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) c[u] = fma2(pair(t.w[u][4 * m], t.w[u][4 * m + 1]), x.x, c[u]);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) c[u] = fma2(pair(t.w[u][4 * m + 2], t.w[u][4 * m + 3]), x.y, c[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) out[u] = __uint_as_float((uint32_t)c[u]) + __uint_as_float((uint32_t)(c[u] >> 32));
+}
 // sums over the four lanes q = 0..3 of a group; lane q keeps the sum of v[q]
 __device__ __forceinline__ float scatter_sum(const float (&v)[4], int lane)
 {
@@ -102,8 +136,8 @@ struct Count {
 //   2  l_t and derivative to global memory                       3  input part W_x x + b of the next step of the chain
 // One block barrier per iteration keeps the groups together.  With all of it between two steps of the chain a step took
 // 0.57 us; with every warp of the second group doing a quarter of each kind of work in every iteration, 0.8 us.
-// T = 100, H = 128, one input and output (B200): batch 1 86 -> 40 us, batch 592 209 -> 118 us; 16 inputs and outputs, T = 128:
-// 200 -> 132 and 613 -> 326 us.
+// T = 100, H = 128, one input and output (B200): batch 1 86 -> 35 us, batch 592 209 -> 111 us; 16 inputs and outputs, T = 128 (before
+// packed multiply-adds): 200 -> 132 and 613 -> 326 us.
 // NS sequences per CTA: the weights in registers serve NS independent chains, whose latencies overlap.  MANY: sums of several
 // outputs go through the shuffles side by side; for one output and few inputs the plain loop is the shorter step (T = 100,
 // batch 1: 40 us against 46; two outputs 52 against 48).
@@ -155,7 +189,7 @@ rnn_forward_kernel(const float *__restrict__ Wh, const float *__restrict__ Wx, c
 #pragma unroll
                 for (int n = 0; n < NS; ++n) {
                     float v[4];
-                    tile_dot(w, hs[cur][n], q, v);
+                    tile_dot2(w, hs[cur][n], q, v);
                     const float a = xin[cur][n][j] + scatter_sum(v, lane);
                     hs[cur ^ 1][n][j] = on ? fmaxf(a, 0.0f) + log1pf(expf(-fabsf(a))) : 0.0f;
                     as[cur][n][j] = a;
