@@ -509,8 +509,10 @@ int run_made(js_model *m, RunArgs &r, cudaStream_t st)
         rc_launch = js_launch_made_tc(m, r, st);
     } else {
         const bool jgs = r.kmode == KM_JACOBI_GS;
-        int &most = m->max_grid_generic[jgs];
-        if (most <= 0) most = js_made_generic_max_grid(v.prec, jgs);
+        // the sums of an fp32 model that made_small.cu serves in Jacobi mode are made as that kernel makes them
+        const bool split = !jgs && v.prec == JS_F32 && !m->small_ok;
+        int &most = m->max_grid_generic[jgs ? 1 : split ? 2 : 0];
+        if (most <= 0) most = js_made_generic_max_grid(v.prec, jgs, split);
         if (most <= 0) {
             snprintf(g_cuda_err, sizeof g_cuda_err, "occupancy query failed");
             return JS_ERR_CUDA;
@@ -522,7 +524,7 @@ int run_made(js_model *m, RunArgs &r, cudaStream_t st)
             tiles = std::max<long long>(tiles, (long long)((r.batch + 15) / 16) * ((v.n[l + 1] + width - 1) / width));
         const long long elems = ((long long)r.batch * v.T * (v.C > 1 ? 32 : 1) + threads - 1) / threads;
         const int grid = (int)std::min<long long>(most, std::max(tiles, elems));
-        rc_launch = js_launch_made_generic(v, r, std::max(grid, 1), st);
+        rc_launch = js_launch_made_generic(v, r, split, std::max(grid, 1), st);
     }
     if (rc_launch != 0) return launch_failed(rc_launch);
     JsCtl h;

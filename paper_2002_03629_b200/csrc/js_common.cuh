@@ -235,5 +235,5 @@ template <> __device__ __forceinline__ float from_f32<float>(float v) { return v
 template <> __device__ __forceinline__ __nv_bfloat16 from_f32<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
 
 // host-side launchers implemented by the kernel files
-int js_launch_made_generic(const MadeDev &m, const RunArgs &r, int grid_limit, cudaStream_t stream);
-int js_made_generic_max_grid(int prec, bool jgs);
+int js_launch_made_generic(const MadeDev &m, const RunArgs &r, bool split, int grid_limit, cudaStream_t stream);
+int js_made_generic_max_grid(int prec, bool jgs, bool split);

@@ -140,7 +140,7 @@ struct js_model {
     uint8_t *x_old = nullptr, *x_tmp = nullptr;
     unsigned long long *trace = nullptr;
     int opt_frontier_skip = 1, opt_seq_skip = 2, opt_spin_limit = 1 << 22, opt_path = 0, opt_compact = 1, opt_trace = 0;
-    int max_grid_generic[2] = {0, 0};      // of the products' instance, of Jacobi-GS's
+    int max_grid_generic[3] = {0, 0, 0};   // of the products' instance, of Jacobi-GS's, of the products with split inputs
     TcDev tc{};
     int tc_ok = 0, tc_max_grid = 0;
     const void *tc_weights[JS_MAXL + 1] = {};       // tile-major weights of the tensor-core kernels

@@ -21,6 +21,7 @@ namespace {
 
 constexpr int KC = 64;         // inputs per step of a product
 constexpr int NTHREADS = 128;
+constexpr int SUM_ROW = 40;    // row stride of partial sums: rows r .. r + 3 by columns c .. c + 7 lie in different banks
 constexpr int ROWF = KC + 4;   // row stride in shared memory: the 16-byte pieces of eight rows lie in different banks
 // The products go by tiles of 16 rows x 32 columns.  What bounds a layer is its longest tile (one chain over all inputs, with
 // every wait of a step in it), so small tiles win although they read shared memory more often: 256 samples through
@@ -30,11 +31,13 @@ constexpr int MR = 2, NR = 2, BMt = 8 * MR, BNt = 16 * NR;
 // registers), and for either type Jacobi-GS's, whose micro-steps are a warp per inner product and want many warps per SM
 // but few CTAs at the thousands of grid barriers between them: 256 threads, tiles of 16 x 64 (with 128 threads a call of
 // T = 784, H = 1024 x 2 in blocks of 98 took 7.56 ms for one sample, 6.41 so; T = 16, H = 64, batch 8 150 us, 133 so).
-template <typename T, bool JGS> struct Conf {
+// SPLIT: fp32 products with the inputs of a tile dealt to the warps, see split_tile.
+template <typename T, bool JGS, bool SPLIT = false> struct Conf {
     static constexpr bool TMA = sizeof(T) == 4 && !JGS;
     static constexpr int NTH = JGS ? 2 * NTHREADS : NTHREADS, BN = BNt * (NTH / NTHREADS);
     static constexpr int STAGES = JGS ? 2 : 4, STAGE_F = (BMt + BN) * (TMA ? 2 * KC : ROWF), CTAS = JGS ? 3 : 2;
-    static constexpr int SMEM_BYTES = STAGES * STAGE_F * (int)sizeof(float) + (TMA ? 1024 : 0);
+    static constexpr int SUMS = SPLIT ? 4 * BMt * SUM_ROW : 0;            // the warps' partial sums
+    static constexpr int SMEM_BYTES = (STAGES * STAGE_F + SUMS) * (int)sizeof(float) + (TMA ? 1024 : 0);
     static constexpr int THREADS = TMA ? NTH + 32 : NTH;
 };
 constexpr int JTHREADS = Conf<float, true>::NTH;
@@ -165,6 +168,80 @@ __device__ __forceinline__ void tma_tile(Smem &s, Ring &rg, int kend, int lr, in
         if ((threadIdx.x & 31) == 0) mbar_arrive(&s.empty[rg.st]);
         rg.advance();
     }
+}
+
+// The same with the inputs dealt to the warps, for models that only this kernel serves (made_small.cu sums like tma_tile, and the
+// solvers of one model must return the same floats): warp w takes inputs 32 w .. 32 w + 31 of every 128, all rows and columns of the
+// tile, 4 x 4 outputs a thread, and the four sums of an output are added in order.  With 2 x 2 outputs a thread the operand
+// reads (4 of 16 bytes for 16 multiply-adds, 8 for 64 here) kept the shared-memory pipe busier than the multiply-adds the
+// others.  T = 784, H = 1024 x 2, 256, 64, 16 samples and one: 279, 220, 209, 167 us, 264, 201, 190, 152 so; with tiles of 32 rows
+// 338 for 256, with stages of 64 inputs 213 for 64.
+__device__ __forceinline__ void split_tile(Smem &s, Ring &rg, int kend, int lr, int wc, JsCtl *ctl, float (&acc)[MR][NR])
+{
+    constexpr int PR = BMt / 4, PC = BNt / 8;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, r = lane & 3, c = lane >> 2;      // rows r + 4 i, columns c + 8 j
+    float p[PR][PC];
+#pragma unroll
+    for (int i = 0; i < PR; ++i)
+#pragma unroll
+        for (int j = 0; j < PC; ++j) p[i][j] = 0.0f;
+    for (int k0 = 0; k0 < kend; k0 += TK) {
+        if (!rg.dead && !mbar_wait(&s.full[rg.st], rg.ph, ctl)) rg.dead = true;       // (see tma_tile)
+        const uint32_t st = ring_base() + (uint32_t)(rg.st * TMA_STAGE_BYTES);
+        const uint32_t ra = st + (uint32_t)(warp * BMt * 128 + r * 128), rb = st + (uint32_t)(TK / BOX_K * BMt * 128 + warp * BNt * 128 + c * 128);
+        const int nq = min(BOX_K / 4, (kend - k0 - BOX_K * warp + 3) / 4);
+        auto quad = [&](int q) {                         // four inputs
+            float4 a[PR], b[PC];
+#pragma unroll
+            for (int i = 0; i < PR; ++i) a[i] = lds_f4(ra + (uint32_t)(i * 512) + (uint32_t)((q ^ (r | (i & 1) << 2)) << 4));
+#pragma unroll
+            for (int j = 0; j < PC; ++j) b[j] = lds_f4(rb + (uint32_t)(j * 1024) + (uint32_t)((q ^ c) << 4));
+#pragma unroll
+            for (int i = 0; i < PR; ++i)
+#pragma unroll
+                for (int j = 0; j < PC; ++j) p[i][j] = fmaf(a[i].x, b[j].x, p[i][j]);
+#pragma unroll
+            for (int i = 0; i < PR; ++i)
+#pragma unroll
+                for (int j = 0; j < PC; ++j) p[i][j] = fmaf(a[i].y, b[j].y, p[i][j]);
+#pragma unroll
+            for (int i = 0; i < PR; ++i)
+#pragma unroll
+                for (int j = 0; j < PC; ++j) p[i][j] = fmaf(a[i].z, b[j].z, p[i][j]);
+#pragma unroll
+            for (int i = 0; i < PR; ++i)
+#pragma unroll
+                for (int j = 0; j < PC; ++j) p[i][j] = fmaf(a[i].w, b[j].w, p[i][j]);
+        };
+        if (nq == BOX_K / 4) {
+#pragma unroll
+            for (int q = 0; q < BOX_K / 4; ++q) quad(q);
+        } else {
+#pragma unroll 1
+            for (int q = 0; q < nq; ++q) quad(q);
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&s.empty[rg.st]);
+        rg.advance();
+    }
+    const uint32_t sums = ring_base() + (uint32_t)(TMA_STAGES * TMA_STAGE_BYTES);
+#pragma unroll
+    for (int i = 0; i < PR; ++i)
+#pragma unroll
+        for (int j = 0; j < PC; ++j)
+            asm volatile("st.shared.f32 [%0], %1;" ::"r"(sums + 4u * (uint32_t)((warp * BMt + r + 4 * i) * SUM_ROW + c + 8 * j)), "f"(p[i][j]) : "memory");
+    asm volatile("bar.sync 1, 128;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < MR; ++i)
+#pragma unroll
+        for (int j = 0; j < NR; ++j) {
+            float v[4];
+#pragma unroll
+            for (int w = 0; w < 4; ++w)
+                asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v[w]) : "r"(sums + 4u * (uint32_t)((w * BMt + lr + 8 * i) * SUM_ROW + wc + 4 * j)) : "memory");
+            acc[i][j] = ((v[0] + v[1]) + v[2]) + v[3];
+        }
+    asm volatile("bar.sync 1, 128;" ::: "memory");          // the next tile's sums go to the same place
 }
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -311,7 +388,7 @@ struct Changes {
 
 // Layer l over the window: hidden layers store act(pre) into `out`; the output layer (l == L) see OutArgs.  Tiles with the
 // longest inner products first, dealt to the CTAs back and forth.
-template <typename T, bool JGS>
+template <typename T, bool JGS, bool SPLIT>
 __device__ void gemm_phase(Smem &s, Ring &rg, const MadeDev &m, const RunArgs &r, int l, const T *Asrc, T *out, const OutArgs &oa, const Win &w,
                            unsigned long long &issued, unsigned long long &skipped)
 {
@@ -368,7 +445,9 @@ __device__ void gemm_phase(Smem &s, Ring &rg, const MadeDev &m, const RunArgs &r
                     xo[i][j] = !in ? 0.0f : r.real ? r.xr[at] : (float)r.x[at];
                 }
             }
-        if constexpr (Conf<T, JGS>::TMA) {
+        if constexpr (SPLIT) {
+            split_tile(s, rg, m.t_kend[l][meta], lr, wc, r.ctl, acc);
+        } else if constexpr (Conf<T, JGS>::TMA) {
             tma_tile(s, rg, m.t_kend[l][meta], lr, wc, r.ctl, acc);
         } else {
             gemm_tile<T, Conf<T, JGS>::STAGES, Conf<T, JGS>::STAGE_F, Conf<T, JGS>::NTH, BN>(Asrc, K, (const T *)m.W[l], K, N, m.t_kend[l][meta], m0, n0, lr, wc, acc);
@@ -631,7 +710,7 @@ __device__ void jgs_copy_or_compare(const MadeDev &m, const RunArgs &r, bool com
 }
 
 // ------------------------------------------------------------------ engine
-template <typename T, bool JGS>
+template <typename T, bool JGS, bool SPLIT>
 struct GenericEngine {
     static constexpr bool has_jgs = JGS;
     Smem &s;
@@ -668,7 +747,7 @@ struct GenericEngine {
         const bool fused = !zout && (m.C == 1 || r.real);
         for (int l = 0; l <= m.L; ++l) {
             const OutArgs oa = {zout ? zout : fused ? (float *)nullptr : m.logits, fused && flag && l == m.L, parity};
-            gemm_phase<T, JGS>(s, rg, m, r, l, (const T *)m.a[l], l < m.L ? (T *)m.a[l + 1] : (T *)nullptr, oa, w, issued, skipped);
+            gemm_phase<T, JGS, SPLIT>(s, rg, m, r, l, (const T *)m.a[l], l < m.L ? (T *)m.a[l + 1] : (T *)nullptr, oa, w, issued, skipped);
             if (!barrier()) return false;
         }
         if (zout || fused) return true;
@@ -684,7 +763,7 @@ struct GenericEngine {
         // hidden activations of the previous outer iterate
         const Win w = make_win(fin_h, T_, T_, T_);
         for (int l = 0; l < m.L; ++l) {
-            gemm_phase<T, JGS>(s, rg, m, r, l, (const T *)m.a_old[l], (T *)m.a_old[l + 1], OutArgs{nullptr, false, 0}, w, issued, skipped);
+            gemm_phase<T, JGS, SPLIT>(s, rg, m, r, l, (const T *)m.a_old[l], (T *)m.a_old[l + 1], OutArgs{nullptr, false, 0}, w, issued, skipped);
             if (!barrier()) return false;
         }
         const int jmax = min(B, T_);
@@ -707,8 +786,8 @@ struct GenericEngine {
     }
 };
 
-template <typename T, bool JGS>
-__global__ void __launch_bounds__(Conf<T, JGS>::THREADS, Conf<T, JGS>::CTAS) made_generic_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ RunArgs r)
+template <typename T, bool JGS, bool SPLIT>
+__global__ void __launch_bounds__(Conf<T, JGS, SPLIT>::THREADS, Conf<T, JGS, SPLIT>::CTAS) made_generic_kernel(const __grid_constant__ MadeDev m, const __grid_constant__ RunArgs r)
 {
     __shared__ Smem s;
     if constexpr (Conf<T, JGS>::TMA) {
@@ -719,7 +798,7 @@ __global__ void __launch_bounds__(Conf<T, JGS>::THREADS, Conf<T, JGS>::CTAS) mad
         }
         __syncthreads();
     }
-    GenericEngine<T, JGS> e(s, m, r);
+    GenericEngine<T, JGS, SPLIT> e(s, m, r);
     DriverResult res = made_driver(e, m.T, r);
     if constexpr (Conf<T, JGS>::TMA) {
         // after an aborted wait copies may still be on their way into this CTA's shared memory
@@ -734,17 +813,18 @@ __global__ void __launch_bounds__(Conf<T, JGS>::THREADS, Conf<T, JGS>::CTAS) mad
 
 }  // namespace
 
-static const void *generic_kernel_of(int prec, bool jgs)
+struct GenericInstance { const void *kernel; int smem, threads; };
+template <typename T, bool JGS, bool SPLIT>
+static GenericInstance generic_instance()
 {
-    if (prec == JS_BF16) return jgs ? (const void *)made_generic_kernel<__nv_bfloat16, true> : (const void *)made_generic_kernel<__nv_bfloat16, false>;
-    return jgs ? (const void *)made_generic_kernel<float, true> : (const void *)made_generic_kernel<float, false>;
+    using CF = Conf<T, JGS, SPLIT>;
+    return {(const void *)made_generic_kernel<T, JGS, SPLIT>, CF::SMEM_BYTES, CF::THREADS};
 }
-static int generic_smem(int prec, bool jgs)
+static GenericInstance generic_of(int prec, bool jgs, bool split)
 {
-    if (jgs) return prec == JS_BF16 ? Conf<__nv_bfloat16, true>::SMEM_BYTES : Conf<float, true>::SMEM_BYTES;
-    return prec == JS_BF16 ? Conf<__nv_bfloat16, false>::SMEM_BYTES : Conf<float, false>::SMEM_BYTES;
+    if (prec == JS_BF16) return jgs ? generic_instance<__nv_bfloat16, true, false>() : generic_instance<__nv_bfloat16, false, false>();
+    return jgs ? generic_instance<float, true, false>() : split ? generic_instance<float, false, true>() : generic_instance<float, false, false>();
 }
-static int generic_threads(int prec, bool jgs) { return jgs ? JTHREADS : prec == JS_BF16 ? NTHREADS : Conf<float, false>::THREADS; }
 
 // Tensor maps of an fp32 model's activations and masked weights: boxes of 32 inputs x 16 rows (activations) or 32 rows, 128-byte
 // swizzle; and of the activations once more for every 64-wide tile of outputs, with the inputs that it reads.
@@ -775,23 +855,23 @@ int js_generic_prepare(js_model *mo)
 }
 
 // most CTAs that are resident at a time (a cooperative launch); jgs: of the instance that serves Jacobi-GS
-int js_made_generic_max_grid(int prec, bool jgs)
+int js_made_generic_max_grid(int prec, bool jgs, bool split)
 {
     static_assert(Conf<float, true>::SMEM_BYTES >= 4096 * 4, "the unit list of the micro-steps shares the stages' memory");
     int dev = 0, sms = 0, per_sm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return -1;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return -1;
-    const void *fn = generic_kernel_of(prec, jgs);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, generic_smem(prec, jgs));
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, generic_threads(prec, jgs), generic_smem(prec, jgs));
+    const GenericInstance g = generic_of(prec, jgs, split);
+    cudaError_t e = cudaFuncSetAttribute(g.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, g.smem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, g.kernel, g.threads, g.smem);
     if (e != cudaSuccess || per_sm < 1) return -1;
     return sms * per_sm;
 }
 
-int js_launch_made_generic(const MadeDev &m, const RunArgs &r, int grid, cudaStream_t stream)
+int js_launch_made_generic(const MadeDev &m, const RunArgs &r, bool split, int grid, cudaStream_t stream)
 {
     void *args[2] = {(void *)&m, (void *)&r};
-    const bool jgs = r.kmode == KM_JACOBI_GS;
-    cudaError_t e = cudaLaunchCooperativeKernel(generic_kernel_of(m.prec, jgs), dim3(grid), dim3(generic_threads(m.prec, jgs)), args, generic_smem(m.prec, jgs), stream);
+    const GenericInstance g = generic_of(m.prec, r.kmode == KM_JACOBI_GS, split);
+    cudaError_t e = cudaLaunchCooperativeKernel(g.kernel, dim3(grid), dim3(g.threads), args, g.smem, stream);
     return e == cudaSuccess ? 0 : (int)e;
 }
