@@ -6,10 +6,10 @@
 // samples through the whole solve, and nothing waits for other clusters:
 //   - a layer is cut into tiles of 64 units, dealt to the CTAs so that their K ranges even out (masks are triangular: a tile
 //     needs 1 .. all K blocks).  A tile is D[64 units x R samples] = W[64 x K] * A[R x K]^T: the weights are the M side of
-//     tcgen05.mma, so that few samples do not waste its rows.  Two warps issue, one the even K blocks into one accumulator,
-//     one the odd ones into another (the four MMAs of a K block take one warp 210 cycles to issue, whatever their size;
-//     two warps issue side by side); the epilogue adds the two;
-//   - every CTA holds the activations of all layers for its R samples in shared memory, K block by K block in the layout
+//     tcgen05.mma, so that few samples do not waste its rows.  Two threads issue, one the even K blocks into one accumulator,
+//     one the odd ones into another (the looks at a K block's barriers and its four MMAs take a thread 200 cycles, the tensor
+//     core 96); the epilogue adds the two;
+//   - every CTA holds the activations that its tiles read, for its R samples, in shared memory, K block by K block in the layout
 //     the MMA reads.  A finished tile IS one K block of the layer above: it is written in place and sent to the other CTAs by
 //     one bulk copy each (cp.async.bulk to distributed shared memory, completing on the receiver's mbarrier for that block).
 //     An MMA waits for the K blocks it reads, not for a layer: there is no barrier inside a pass;
@@ -22,6 +22,7 @@
 // pass, of which three layers at 3.2 and 1.5 from the last mask to the next pass's first MMA; 16.5 before the loads took two
 // blocks, one thread of a warp looked for weights, activations and room at once (a look is 150 cycles), and every role
 // saw the masks itself.
+//
 // Solvers: Jacobi (Algorithm 1) and GS-Jacobi (Algorithm 3), the control logic of made_driver.cuh on the cluster's samples.
 // Warps: 0 weight loads, 1 and 7 MMA (1 owns tensor memory), 2-5 epilogue, 6 arms and drains the activation barriers.
 // All waits are bounded, as in the other tensor-core kernels.
@@ -65,7 +66,7 @@ struct ClShared {
     int count[64];
     int issued, consumed[2];                 // weight loads; K blocks multiplied, even and odd ones
     int consumed_loads;
-    uint64_t apar[2][CL_MAXL + 2];
+    uint64_t apar[2][CL_MAXL + 2];           // of either MMA thread: parity of the next completion of every K block's barrier
     unsigned tiles;
     unsigned sums[2];                        // of the whole cluster (in its first CTA): tiles, K blocks
     unsigned char place[CL_MAXL][MAXOWN];    // this CTA's hidden tiles: K block of a[l + 1] that it keeps them in

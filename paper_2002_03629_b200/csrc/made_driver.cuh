@@ -35,12 +35,16 @@ __device__ __forceinline__ void note_change(const RunArgs &r, int parity, int b,
     atomicOr(&r.ctl->agg_any[parity], 1);
 }
 
-// After the barrier that ends an iteration: CTA 0 clears the other parity's flags.
+// The bookkeeping between two iterations falls to the last CTA of the grid.  Its loads take 1.5 us, for which the CTA comes late to the next
+// phase; the phase's first and longest units lie with the first CTAs, and often the last one has none.
+__device__ __forceinline__ bool keeps_books() { return blockIdx.x == gridDim.x - 1; }
+
+// After the barrier that ends an iteration: one CTA clears the other parity's flags.
 // Safe because every CTA read that parity before it passed at least one later
 // barrier, and nobody writes it again before at least one more barrier.
 __device__ __forceinline__ void reset_other_parity(const RunArgs &r, int parity)
 {
-    if (blockIdx.x != 0) return;
+    if (!keeps_books()) return;
     const int o = parity ^ 1;
     for (int i = threadIdx.x; i < r.batch; i += blockDim.x) r.smp_changed[o * r.batch + i] = 0;
     if (threadIdx.x == 0) {
@@ -49,11 +53,11 @@ __device__ __forceinline__ void reset_other_parity(const RunArgs &r, int parity)
     }
 }
 
-// CTA 0: a sample whose iterate did not change (or that hit the cap) stops counting.
+// One CTA: a sample whose iterate did not change (or that hit the cap) stops counting.
 __device__ __forceinline__ void book_samples(const RunArgs &r, int parity, int k, bool at_cap, bool add,
                                              bool final_write)
 {
-    if (blockIdx.x != 0) return;
+    if (!keeps_books()) return;
     int *done = r.smp_state, *count = r.smp_state + r.batch;
     for (int b = threadIdx.x; b < r.batch; b += blockDim.x) {
         if (!done[b] && (r.smp_changed[parity * r.batch + b] == 0 || at_cap)) {
@@ -197,7 +201,7 @@ __device__ DriverResult made_driver(E &e, int T_, const RunArgs &r)
         if (any && cap < len) res.status = JS_NOT_CONVERGED;
         if (mode == KM_JACOBI) break;
         fin_x = bend;          // positions < bend are never touched again: settled
-        if (blockIdx.x == 0)   // new block: nobody is done (same threads wrote these entries)
+        if (keeps_books())     // new block: nobody is done (same threads wrote these entries)
             for (int b = threadIdx.x; b < r.batch; b += blockDim.x) r.smp_state[b] = 0;
         a = bend;
         lo = a;
@@ -206,11 +210,11 @@ __device__ DriverResult made_driver(E &e, int T_, const RunArgs &r)
     }
     if (mode == KM_SEQ) {
         res.frontier = T_;
-        if (blockIdx.x == 0 && r.out_iters)
+        if (keeps_books() && r.out_iters)
             for (int b = threadIdx.x; b < r.batch; b += blockDim.x) r.out_iters[b] = 1;
     } else if (mode == KM_GS_JACOBI) {
         res.frontier = T_;
-        if (blockIdx.x == 0 && r.out_iters)
+        if (keeps_books() && r.out_iters)
             for (int b = threadIdx.x; b < r.batch; b += blockDim.x) r.out_iters[b] = r.smp_state[r.batch + b];
     } else if (mode == KM_JACOBI) {
         res.frontier = fin_x;

@@ -177,6 +177,7 @@ struct TcEngine {
     __device__ void look_ahead(int) {}
     __device__ int compact(int parity)
     {
+        if (live <= BM) return 0;         // one tile of rows: nothing to be had
         const int *pc = perm_cur();
         int *pn = r.perm + (size_t)(pcur ^ 1) * r.perm_stride;
         const int *chg = r.smp_changed + (size_t)parity * r.batch;
