@@ -468,13 +468,13 @@ def measure_rnn(local: int, with_oracle: bool):
             err = ((sn - exact).norm() / exact.norm()).item()
             flops = 2.0 * cfg.batch * n * cfg.T * cfg.H * cfg.H
             rec[f"backward_jacobi_{n}"] = {"ms": ms, "rel_l2_error_vs_exact": err, "tflops": flops / ms / 1e9}
-        # fp32 fused multiply-add peak: SMs x 128 lanes x 2 flop x clock
-        prop = torch.cuda.get_device_properties(local)
-        peak = prop.multi_processor_count * 128 * 2 * 1.965e9 / 1e12
+        # an fp32 product is six bf16 products on the tensor cores
+        peaks = load_peaks()
+        peak = peaks["bf16_tflops"] / 6
         j = rec[f"backward_jacobi_{cfg.T}"]
-        rec["roofline"] = {"bound": "alu", "kernel": "rnn_bptt_jacobi_kernel", "achieved": j["tflops"], "peak": peak,
+        rec["roofline"] = {"bound": "tensor", "kernel": "rnn_bptt_jacobi_kernel", "achieved": j["tflops"], "peak": peak,
                            "unit": "TFLOP/s", "frac": j["tflops"] / peak,
-                           "peak_source": "SMs x 128 fp32 lanes x 2 x 1965 MHz (nominal; derived, not measured)"}
+                           "peak_source": peaks["source"] + " burst bf16, a sixth of it"}
         rec["sequences_per_s_exact_gradient"] = cfg.batch / ((rec["forward_ms"] + rec["backward_sequential_ms"] +
                                                               rec["param_grads_ms"]) / 1e3)
         if with_oracle:
