@@ -932,18 +932,22 @@ static int cluster_rows(const js_model *mo, int batch, int *n_stages)
     return 0;
 }
 
-// Jacobi and GS-Jacobi calls whose samples fit the clusters that the GPU holds at a time; more samples would go in turns,
-// and the grid-wide kernel, which shares every weight tile among 128 samples, is the better one then.
+// Jacobi and GS-Jacobi calls whose samples go through in one round of clusters, or in two where a CTA's share of the weights is small and
+// its ring long; the grid-wide kernel shares every weight tile among 128 samples and is the better one for more.
 bool js_cluster_serves(const js_model *mo, const RunArgs &r)
 {
     if (!mo->cluster_ok || (r.kmode != KM_JACOBI && r.kmode != KM_GS_JACOBI) || mo->opt_trace) return false;
     int st = 0;
     const int R = cluster_rows(mo, r.batch, &st);
     if (R == 0) return false;
-    // A CTA streams its share of the weights every pass, whatever the batch.  T and H = 2048 x 3, 16 and 64 samples, us here
-    // and grid-wide: T = 1024 (204 K blocks) 132 and 162, 132 and 165; 1296 (226) 148 and 170, 149 and 174; 1600 (241) 163 and
-    // 172, 164 and 175; 1936 (264) 186 and 173, 241 and 226.
-    return mo->cluster.kblocks <= 230 && (r.batch + R - 1) / R <= std::min(JS_MAX_CLUSTERS, mo->cluster.max_clusters);
+    // A CTA streams its share of the weights every pass, whatever the batch.  One round, 16 and 100 samples, us here and grid-wide: T = 1600,
+    // H = 2048 x 3 (241 K blocks) 151 and 177, 163 and 197; T = 1936 (264) 175 and 191, 190 and 218; T = 2500, H = 2500 x 3 (410), 8 samples 404 and 229.
+    // Two rounds: 784, 1024 x 2, 512 samples (47 K blocks, 8 stages) 126 and 167; 1024, 1536 x 2, 480 (91, 10) 180 and 202; 1444, 1444 x 2,
+    // 300 (104, 8) 198 and 272; but 1024, 2048 x 2, 250 (136, 6) 231 and 202; 1600, 1024, 512 (55, 6) 233 and 221; 1936, 1500 x 2, 250 (138, 4)
+    // 340 and 196.
+    const int clusters = (r.batch + R - 1) / R, rounds = (clusters + mo->cluster.max_clusters - 1) / mo->cluster.max_clusters;
+    if (clusters > JS_MAX_CLUSTERS) return false;
+    return rounds == 1 ? mo->cluster.kblocks <= 270 : rounds == 2 && mo->cluster.kblocks <= 104 && st >= 8;
 }
 
 int js_launch_made_cluster(const js_model *mo, const RunArgs &r, cudaStream_t stream, ClusterWork *work)
