@@ -828,7 +828,7 @@ __global__ void rnn_copy_kernel(const float *s0, float *s, size_t n)
 // quarter where there are few sequences.  db and dWx, the same sums with 1 and x_t on the right, are taken up while the operands are cut:
 // a warp sums the steps that it cuts, the warps' sums are added in order.
 // Values that the pieces cannot carry (infinities, NaN, beyond what bf16 reaches): plain multiply-adds, as in jac_plain.
-// T = 100, H = 128 (B200): batch 592 45 us (60 MB in, 39 MB out: 15 us), batch 1 11; multiply-adds on the CUDA cores took 75 and 16.  Against 64 bits
+// T = 100, H = 128 (B200): batch 592 45 us (91 MB in, 39 MB out: 20 us), batch 1 11; multiply-adds on the CUDA cores took 75 and 16.  Against 64 bits
 // dWh is off by 1.1e-7 in the 2-norm, 1.8e-7 before.  Bound: a CTA's chain of loads, cutting, MMAs and stores, twice per SM.
 constexpr int PK = 64, PGT = 256;            // steps at a time, threads
 constexpr int P_PIECE = PK * MH * 2;         // bytes of a piece: [two groups of 64 components][PK steps][128 bytes, swizzled]
