@@ -827,7 +827,7 @@ __global__ void rnn_copy_kernel(const float *s0, float *s, size_t n)
 // loads and stores pass while the other multiplies).  A CTA computes `cols` columns of one sequence: all of them, or a half or a
 // quarter where there are few sequences.  db and dWx, the same sums with 1 and x_t on the right, are taken up while the operands are cut:
 // a warp sums the steps that it cuts, the warps' sums are added in order.
-// Values that the pieces cannot carry (infinities, NaN, beyond what bf16 reaches): plain multiply-adds, as in jac_plain.
+// Sums that are not finite (an operand beyond what bf16 reaches, or a product beyond fp32) are made again by plain multiply-adds, as in jac_plain.
 // T = 100, H = 128 (B200): batch 592 45 us (91 MB in, 39 MB out: 20 us), batch 1 11; multiply-adds on the CUDA cores took 75 and 16.  Against 64 bits
 // dWh is off by 1.1e-7 in the 2-norm, 1.8e-7 before.  Bound: a CTA's chain of loads, cutting, MMAs and stores, twice per SM.
 constexpr int PK = 64, PGT = 256;            // steps at a time, threads
@@ -865,15 +865,12 @@ rnn_param_grads_kernel(const float *__restrict__ s, const float *__restrict__ d,
     for (int c = 0; c <= NX; ++c)
 #pragma unroll
         for (int e = 0; e < 4; ++e) sx[c][e] = 0.0f;
-    bool fine = true, ok = true;
+    bool ok = true;
     // four neighbouring components of step row r of an operand, in pieces
     auto put = [&](uint8_t *op, int r, const float (&v)[4]) {
         uint32_t ph[2], pm[2], pl[2];
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            cut3(v[2 * e], v[2 * e + 1], ph[e], pm[e], pl[e]);
-            fine = fine && fabsf(v[2 * e]) <= 3.38e38f && fabsf(v[2 * e + 1]) <= 3.38e38f;
-        }
+        for (int e = 0; e < 2; ++e) cut3(v[2 * e], v[2 * e + 1], ph[e], pm[e], pl[e]);
         const uint32_t at = smem_u32(op) + (uint32_t)((i4 >> 6) * (PK * 128) + r * 128 + ((((i4 & 63) >> 3) ^ (r & 7)) << 4) + (i4 & 7) * 2);
         asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(at), "r"(ph[0]), "r"(ph[1]) : "memory");
         asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(at + P_PIECE), "r"(pm[0]), "r"(pm[1]) : "memory");
@@ -939,21 +936,10 @@ rnn_param_grads_kernel(const float *__restrict__ s, const float *__restrict__ d,
     }
     if (ok) ok = jac_wait(dead, &done, par ^ 1u);
     ok = __syncthreads_and(ok) != 0;
-    const bool plain = !__syncthreads_and(fine);
     tc_fence_after();
     float *out = dWh + (size_t)seq * H * H;
-    if (!ok || plain) {
-        for (int p = tid; p < H * cols; p += PGT) {
-            const int i = p / cols, j = n0 + p % cols;
-            if (j >= H) continue;
-            float acc = ok ? 0.0f : NAN;
-            for (int t = 1; ok && t < T; ++t) {
-                const size_t at = base + (size_t)t * H;
-                acc = fmaf(d[at + i] * s[at + i], h[at - H + j], acc);
-            }
-            out[(size_t)i * H + j] = acc;
-        }
-    } else {
+    float chk = 0.0f;                                    // non-zero (NaN): a sum that is not finite
+    if (ok) {
         // a warp takes sixteen rows of its quadrant and half of the columns at a time: eight rows of 32 bytes a store
         const int q = warp & 3, half = cols / 2, c0 = (warp >> 2) * half;
 #pragma unroll 1
@@ -976,10 +962,24 @@ rnn_param_grads_kernel(const float *__restrict__ s, const float *__restrict__ d,
                         float *to = out + (size_t)i * H + j;
                         if constexpr (VEC) *reinterpret_cast<float2 *>(to) = make_float2(v[2 * e], v[2 * e + 1]);
                         else { to[0] = v[2 * e]; to[1] = v[2 * e + 1]; }
+                        chk = fmaf(v[2 * e], 0.0f, fmaf(v[2 * e + 1], 0.0f, chk));
                     }
                 }
             }
     }
+    // Not finite: an operand that the pieces cannot carry, or a product or a sum beyond fp32, whose pieces leave with either sign.  (Whatever
+    // does not carry shows here: each operand meets every one of the other side, be it a zero.)
+    if (!__syncthreads_and(ok && chk == 0.0f))
+        for (int p = tid; p < H * cols; p += PGT) {
+            const int i = p / cols, j = n0 + p % cols;
+            if (j >= H) continue;
+            float acc = ok ? 0.0f : NAN;
+            for (int t = 1; ok && t < T; ++t) {
+                const size_t at = base + (size_t)t * H;
+                acc = fmaf(d[at + i] * s[at + i], h[at - H + j], acc);
+            }
+            out[(size_t)i * H + j] = acc;
+        }
     if (extra) {
         // the warps' sums through the operands' memory
         float *sums = reinterpret_cast<float *>(ops);        // [warp][1 + d_in][MH]

@@ -108,3 +108,27 @@ def test_parameter_gradients_against_64_bits(B, T, H, d_in):
     assert ((dWh[0, row].double() - want).abs() <= 1e-5 * want.abs() + 1e-4).all()
     if B > 1:
         assert torch.isfinite(dWh[1:]).all()
+
+
+@pytest.mark.parametrize("B,T,H", [(1, 25, 4), (2, 70, 128), (160, 40, 36)])
+def test_parameter_gradients_beyond_fp32(B, T, H):
+    """Finite operands whose products leave fp32 give what multiply-adds give: an infinity where one does, no NaN, and the sums that stay
+    finite as they are."""
+    import paper_2002_03629_b200.rnn as rnn
+    _, s, d, h = draw(B, T, H)
+    x = torch.zeros((B, T, 1), device="cuda")
+    s, h = s.sign() + s, h.sign() + h
+    d[:] = 1.0
+    # (bf16 rounds 1.003e30 and 1.9e30 up and the others down: the products of their pieces leave fp32 with either sign)
+    s[0, T - 2, 0], s[0, T - 2, 1] = 1.2345e30, 1.003e30
+    h[0, T - 3, 2], h[0, T - 3, 3] = 1.9e30, -1.3e30
+    got = rnn.rnn_param_grads(s, d, h, x)[0].cpu().numpy()
+    g, hp = s.cpu().numpy(), h.cpu().numpy()
+    with np.errstate(all="ignore"):
+        want = sum(g[:, t, :, None] * hp[:, t - 1, None, :] for t in range(1, T))
+    assert want[0, 1, 2] == np.inf and want[0, 1, 3] == -np.inf and not np.isnan(want).any()
+    m = np.isfinite(want)
+    np.testing.assert_array_equal(got[~m], want[~m])
+    # T products of 24 bits, the largest of a sum being 2e30 and summed in any order: T rounding steps of 2^-24 of the absolute sum
+    scale = sum(np.abs(g[:, t, :, None].astype(np.float64) * hp[:, t - 1, None, :]) for t in range(1, T))
+    assert (np.abs(got[m].astype(np.float64) - want[m]) <= 2 * T * 2.0 ** -24 * scale[m]).all()
