@@ -18,8 +18,9 @@
  * 1 <= H <= 128 with H a multiple of 4, 1 <= d_in, d_out <= 16, B >= 1.  Return value: 0, RNN_ERR_INVALID (-1) for a
  * null pointer or a size outside the limits (nothing is launched), RNN_ERR_CUDA (-2) if the launch failed
  * (rnn_last_error() names the CUDA error).  Arithmetic: fp32 fused multiply-adds in a fixed order; in the Jacobi iterations and in
- * the parameter gradients of more than 24 steps, products of three-piece bf16 expansions (24 bits) summed in fp32 on the tensor
- * cores, also in a fixed order (results are reproducible run to run); exp/log from the fast-math intrinsics are not used.
+ * the parameter gradients of more than 24 steps, products of three-piece bf16 expansions (24 bits, over the whole range of fp32) summed in fp32 on the tensor
+ * cores, also in a fixed order (results are reproducible run to run); what leaves the expansions' upper end, states beyond 1e24 or
+ * factors beyond 2e31, infinities and NaN among them, is computed again by multiply-adds, at a fraction of the speed; exp/log from the fast-math intrinsics are not used.
  */
 #ifndef RNN_BPTT_H
 #define RNN_BPTT_H

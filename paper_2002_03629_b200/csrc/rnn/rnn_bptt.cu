@@ -393,7 +393,8 @@ rnn_bptt_sequential_kernel(const float *__restrict__ Wh, const float *__restrict
 // ones as 128 columns hold): as the steps of a batch lie one after another in memory, so do the columns, and U, taken as
 // zero at t = 0, keeps a sequence from reaching into the one before it.
 // fp32 values are cut into three bf16 pieces (8 + 8 + 8 bits; what is left is below 2^-26 of the value) and the six products
-// of pieces down to 2^-18 are summed.  The tensor core rounds its running sums towards zero, so the five small products
+// of pieces down to 2^-18 are summed.  Both sides are cut 2^24 times as large and the sums brought back by 2^-48, both exact: the last
+// bit of any fp32 value then lies above the smallest bf16 number, where as they are the pieces of values below 6e-33 lose bits.  The tensor core rounds its running sums towards zero, so the five small products
 // come first, while the sum is small, and the large one, high by high, is shared by two accumulators: four steps of full size each.
 //   warps 0-7   epilogue: thread = (component i, JC columns of each slot); l and d of these stay in registers, s = l + D, U goes back to
 //               shared memory as three pieces, eight columns (16 bytes) a store.  JC = 32; up to 64 components the rows of A lie
@@ -402,7 +403,7 @@ rnn_bptt_sequential_kernel(const float *__restrict__ Wh, const float *__restrict
 // The columns go in two slots of up to 64, each with accumulators of its own: one slot's MMAs run while the other's epilogue
 // does.  A slot's last column takes its sum from the first column of the slot behind it, which is therefore the first in every round.
 // l and d of the next unit come into shared memory (bulk copies, where the pointers lie on 16 bytes) while this one is worked on.
-// Values that three pieces cannot carry (infinities, NaN, or so large that a piece overflows) show as non-finite
+// Values that three pieces cannot carry (infinities, NaN, states beyond 1e24, factors beyond 2e31) show as non-finite
 // states: such a unit is computed again with plain multiply-adds before anything of it is stored.
 // Bound: at 65 to 128 components the MMAs, 96 of 17 to 32 cycles an iteration (1.6 us of the 1.7 measured for 100 steps of 128
 // components; multiply-adds on the CUDA cores, 40 TFLOP/s, took 10); below that the way from a slot's last product to its next
@@ -454,6 +455,7 @@ __device__ __forceinline__ void tmem_ld_16x8(uint32_t taddr, uint32_t (&r)[4])
 {
     asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(taddr) : "memory");
 }
+constexpr float PIECES_UP = 0x1p24f, SUMS_DOWN = 0x1p-48f;      // before the cut, after the products
 // two values in three bf16 pieces each, packed (the first in the low half)
 __device__ __forceinline__ void cut3(float a, float b, uint32_t &h, uint32_t &m, uint32_t &l)
 {
@@ -556,7 +558,7 @@ rnn_bptt_jacobi_kernel(const float *__restrict__ Wh, const float *l, const float
     bool fine = true;                                                        // this thread's weights are finite
     if (warp < 8) {
         float chk = 0.0f;
-#pragma unroll 4
+#pragma unroll 2
         for (int c4 = 0; c4 < 8; ++c4) {                                     // 32 words of every piece, 64 k
             const int k0 = (warp >> 2) * 64 + c4 * 8;
             if (k0 >= nk * 16) break;
@@ -568,7 +570,7 @@ rnn_bptt_jacobi_kernel(const float *__restrict__ Wh, const float *l, const float
                 chk = fmaf(w[e], 0.0f, chk);
             }
 #pragma unroll
-            for (int e = 0; e < 4; ++e) cut3(w[2 * e], w[2 * e + 1], ph[e], pm[e], pl[e]);
+            for (int e = 0; e < 4; ++e) cut3(w[2 * e] * PIECES_UP, w[2 * e + 1] * PIECES_UP, ph[e], pm[e], pl[e]);
             const uint32_t at = tm + quad + (uint32_t)(k0 / 2);
             tmem_st4(at, ph);
             tmem_st4(at + MH / 2, pm);
@@ -654,7 +656,7 @@ rnn_bptt_jacobi_kernel(const float *__restrict__ Wh, const float *l, const float
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
                 rows(k, [&](int j, int at, bool in) { lv[k][j] = in ? lp[at] : 0.0f; });
-                rows(k, [&](int j, int at, bool in) { dv[k][j] = in ? dp[at] : 0.0f; });
+                rows(k, [&](int j, int at, bool in) { dv[k][j] = in ? dp[at] * PIECES_UP : 0.0f; });
                 // first steps of the unit's other sequences: no U, not even of an infinite state
                 first[k] = 0;
                 if (MANY)
@@ -667,7 +669,7 @@ rnn_bptt_jacobi_kernel(const float *__restrict__ Wh, const float *l, const float
             ok = jac_all(ok);                                                // everything has been read
             if (tid == 0) stage(u + (int)gridDim.x);
             const bool idle = (i & ~31) >= H;                                // no component of this warp's (and no k that the MMAs read)
-            // eight columns of the operand of slot k from their states: pieces of U = d s
+            // eight columns of the operand of slot k from their states: pieces of U = d s (d as large as they want it)
             auto put8 = [&](int k, int j0, const float (&v)[8]) {
                 uint32_t ph[4], pm[4], pl[4];
                 float w[8];
@@ -719,15 +721,15 @@ rnn_bptt_jacobi_kernel(const float *__restrict__ Wh, const float *l, const float
                 auto take = [&](int j0, float (&w)[8]) {
                     if (last) {
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) lv[k][j0 + e] += w[e];
+                        for (int e = 0; e < 8; ++e) lv[k][j0 + e] = fmaf(w[e], SUMS_DOWN, lv[k][j0 + e]);
                     } else {
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) w[e] += lv[k][j0 + e];
+                        for (int e = 0; e < 8; ++e) w[e] = fmaf(w[e], SUMS_DOWN, lv[k][j0 + e]);
                         put8(k, j0, w);
                     }
                 };
                 float w[8];
-                if (g == 0 && k == 0 && last) l0 += sum(0);
+                if (g == 0 && k == 0 && last) l0 = fmaf(sum(0), SUMS_DOWN, l0);
 #pragma unroll
                 for (int e = 0; e < 8; ++e) w[e] = sum(1 + e);
                 take(0, w);
@@ -822,12 +824,12 @@ __global__ void rnn_copy_kernel(const float *s0, float *s, size_t n)
 
 // ------------------------------------------------------------------ parameter gradients
 // dWh = sum_t g_t h_{t-1}^T with g_t = d_t * s_t: a [128 x T] x [T x 128] product per sequence, on the tensor cores like the Jacobi
-// iterations: three bf16 pieces of either side, six products, the five small ones in an accumulator of their own.  Both operands lie
+// iterations: three bf16 pieces of either side (2^24 times as large), six products, the five small ones in an accumulator of their own.  Both operands lie
 // in shared memory as they come, components together, steps in rows (PK of them at a time, so that two CTAs share an SM and one's
 // loads and stores pass while the other multiplies).  A CTA computes `cols` columns of one sequence: all of them, or a half or a
 // quarter where there are few sequences.  db and dWx, the same sums with 1 and x_t on the right, are taken up while the operands are cut:
 // a warp sums the steps that it cuts, the warps' sums are added in order.
-// Sums that are not finite (an operand beyond what bf16 reaches, or a product beyond fp32) are made again by plain multiply-adds, as in jac_plain.
+// Sums that are not finite (an operand beyond 2e31, a product beyond 1e24) are made again by plain multiply-adds, as in jac_plain.
 // T = 100, H = 128 (B200): batch 592 45 us (91 MB in, 39 MB out: 20 us), batch 1 11; multiply-adds on the CUDA cores took 75 and 16.  Against 64 bits
 // dWh is off by 1.1e-7 in the 2-norm, 1.8e-7 before.  Bound: a CTA's chain of loads, cutting, MMAs and stores, twice per SM.
 constexpr int PK = 64, PGT = 256;            // steps at a time, threads
@@ -870,7 +872,7 @@ rnn_param_grads_kernel(const float *__restrict__ s, const float *__restrict__ d,
     auto put = [&](uint8_t *op, int r, const float (&v)[4]) {
         uint32_t ph[2], pm[2], pl[2];
 #pragma unroll
-        for (int e = 0; e < 2; ++e) cut3(v[2 * e], v[2 * e + 1], ph[e], pm[e], pl[e]);
+        for (int e = 0; e < 2; ++e) cut3(v[2 * e] * PIECES_UP, v[2 * e + 1] * PIECES_UP, ph[e], pm[e], pl[e]);
         const uint32_t at = smem_u32(op) + (uint32_t)((i4 >> 6) * (PK * 128) + r * 128 + ((((i4 & 63) >> 3) ^ (r & 7)) << 4) + (i4 & 7) * 2);
         asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(at), "r"(ph[0]), "r"(ph[1]) : "memory");
         asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(at + P_PIECE), "r"(pm[0]), "r"(pm[1]) : "memory");
@@ -953,7 +955,7 @@ rnn_param_grads_kernel(const float *__restrict__ s, const float *__restrict__ d,
                 tmem_wait_ld();
                 float v[4];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) v[e] = __uint_as_float(a[e]) + __uint_as_float(b[e]);
+                for (int e = 0; e < 4; ++e) v[e] = (__uint_as_float(a[e]) + __uint_as_float(b[e])) * SUMS_DOWN;
                 const int j = n0 + c + 2 * (lane & 3);
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
@@ -967,17 +969,16 @@ rnn_param_grads_kernel(const float *__restrict__ s, const float *__restrict__ d,
                 }
             }
     }
-    // Not finite: an operand that the pieces cannot carry, or a product or a sum beyond fp32, whose pieces leave with either sign.  (Whatever
+    // Not finite: an operand that the pieces cannot carry, or a product or a sum beyond 1e24, whose pieces may leave fp32 with either sign.  (Whatever
     // does not carry shows here: each operand meets every one of the other side, be it a zero.)
     if (!__syncthreads_and(ok && chk == 0.0f))
         for (int p = tid; p < H * cols; p += PGT) {
             const int i = p / cols, j = n0 + p % cols;
             if (j >= H) continue;
+            const float *gd = d + base + i, *gs = s + base + i, *hj = h + base + j;
             float acc = ok ? 0.0f : NAN;
-            for (int t = 1; ok && t < T; ++t) {
-                const size_t at = base + (size_t)t * H;
-                acc = fmaf(d[at + i] * s[at + i], h[at - H + j], acc);
-            }
+#pragma unroll 4
+            for (int t = H; t < T * H; t += H) acc = fmaf(gd[t] * gs[t], hj[t - H], acc);
             out[(size_t)i * H + j] = acc;
         }
     if (extra) {

@@ -132,3 +132,27 @@ def test_parameter_gradients_beyond_fp32(B, T, H):
     # T products of 24 bits, the largest of a sum being 2e30 and summed in any order: T rounding steps of 2^-24 of the absolute sum
     scale = sum(np.abs(g[:, t, :, None].astype(np.float64) * hp[:, t - 1, None, :]) for t in range(1, T))
     assert (np.abs(got[m].astype(np.float64) - want[m]) <= 2 * T * 2.0 ** -24 * scale[m]).all()
+
+
+@pytest.mark.parametrize("scale", [2.0 ** -20, 2.0 ** -105, 2.0 ** -118])
+@pytest.mark.parametrize("B,T,H", [(1, 33, 8), (2, 100, 128), (300, 30, 64)])
+def test_small_values_keep_their_bits(B, T, H, scale):
+    """States and operands near the lower end of fp32 are as exact as others, relative to their own size: 7e-7 in the 2-norm as above
+    (at 2^-118 the smallest fp32 number, 2^-149, is below 2^-30 of the values' size and does not show)."""
+    import paper_2002_03629_b200.rnn as rnn
+    W, l, d, s0 = draw(B, T, H)
+    l, s0 = l * scale, s0 * scale
+    for n, s in ((2, None), (3, s0), (9, None)):
+        got, want = rnn.rnn_bptt_jacobi(W, l, d, n, s0=s), reference(W, l, d, n, s)
+        assert ((got.double() - want).norm() / want.norm()).item() < 7e-7, n
+    # a component that hears of the others by small weights alone
+    W2, l2 = W.clone(), l / scale
+    W2[:, 1] *= scale
+    l2[:, :, 1] = 0
+    got, want = rnn.rnn_bptt_jacobi(W2, l2, d, 4)[:, :, 1].double(), reference(W2, l2, d, 4)[:, :, 1]
+    assert ((got - want).norm() / want.norm().clamp_min(1e-300)).item() < 7e-7
+    h, x = torch.rand((B, T, H), device="cuda"), torch.ones((B, T, 1), device="cuda")
+    for g, hh in ((s0, h), (s0 / scale, h * scale)):
+        want = torch.einsum("bti,btj->bij", (d.double() * g.double())[:, 1:], hh.double()[:, :-1])
+        got = rnn.rnn_param_grads(g, d, hh, x)[0].double()
+        assert ((got - want).norm() / want.norm()).item() < 7e-7
