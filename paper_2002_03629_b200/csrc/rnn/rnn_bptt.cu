@@ -531,14 +531,16 @@ rnn_bptt_jacobi_kernel(const float *__restrict__ Wh, const float *l, const float
     const uint32_t quad = (uint32_t)((warp & 3) * 32) << 16;
     const int width = per_unit * T;                                          // columns of a unit
     const bool two = width > J_SLOT;
-    const int units = (B + per_unit - 1) / per_unit, nk = (H + 15) / 16;
+    const int units = (B - 1) / per_unit + 1, nk = (H + 15) / 16;
+    // the columns of unit u (B T need not fit 31 bits)
+    auto unit_columns = [&](int u) { return min(per_unit, B - u * per_unit) * T; };
     // the columns of a slot that its MMAs compute
     auto slot_columns = [&](int k) { return max(0, min(J_SLOT, width - k * J_SLOT) + 15) / 16 * 16; };
     float *const ls = reinterpret_cast<float *>(ops + J_OPS), *const ds = ls + width * H;
     const bool stages = ((reinterpret_cast<uintptr_t>(l) | reinterpret_cast<uintptr_t>(d)) & 15u) == 0;
     auto stage = [&](int u) {
         if (u >= units || !stages) return;
-        const uint32_t bytes = (uint32_t)(min(width, (B - u * per_unit) * T) * H) * 4u;
+        const uint32_t bytes = (uint32_t)(unit_columns(u) * H) * 4u;
         const size_t from = (size_t)u * per_unit * T * H;
         mbar_expect_tx(&sh.staged, 2 * bytes);
         bulk_load(smem_u32(ls), l + from, bytes, &sh.staged);
@@ -629,7 +631,7 @@ rnn_bptt_jacobi_kernel(const float *__restrict__ Wh, const float *l, const float
         asm volatile("setmaxnreg.inc.sync.aligned.u32 232;");
         uint32_t par = 0, staged_par = 0;
         for (int u = blockIdx.x; u < units; u += gridDim.x) {
-            const int cols = min(width, (B - u * per_unit) * T);
+            const int cols = unit_columns(u);
             const size_t base = (size_t)u * per_unit * T * H + i;
             bool ok = true;
             if (stages) ok = jac_wait(sh.dead, &sh.staged, staged_par);
@@ -1190,12 +1192,12 @@ int rnn_bptt_jacobi(const float *Wh, const float *l, const float *d, int B, int 
         return launch_status();
     }
     // several sequences in a unit of 128 columns only where there are more of them than SMs
-    const int per_unit = std::max(1, std::min(2 * J_SLOT / T, (B + sms - 1) / sms));
+    const int per_unit = std::max(1, std::min(2 * J_SLOT / T, (B - 1) / sms + 1));
     auto kernel = per_unit > 1 ? (H > 64 ? rnn_bptt_jacobi_kernel<32, true> : rnn_bptt_jacobi_kernel<16, true>)
                                : (H > 64 ? rnn_bptt_jacobi_kernel<32, false> : rnn_bptt_jacobi_kernel<16, false>);
     if (!allow_smem(kernel, 1024 + J_OPS + (size_t)2 * MT * MH * sizeof(float), (H > 64) + 2 * (per_unit > 1))) return RNN_ERR_CUDA;
     const size_t smem = 1024 + J_OPS + (size_t)2 * per_unit * T * H * sizeof(float);
-    kernel<<<std::min(sms, (B + per_unit - 1) / per_unit), JTH, smem, (cudaStream_t)stream>>>(
+    kernel<<<std::min(sms, (B - 1) / per_unit + 1), JTH, smem, (cudaStream_t)stream>>>(
         Wh, l, d, B, T, H, std::min(n_iters, T), s0, s, per_unit);
     return launch_status();
 }

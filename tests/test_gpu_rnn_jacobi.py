@@ -156,3 +156,21 @@ def test_small_values_keep_their_bits(B, T, H, scale):
         want = torch.einsum("bti,btj->bij", (d.double() * g.double())[:, 1:], hh.double()[:, :-1])
         got = rnn.rnn_param_grads(g, d, hh, x)[0].double()
         assert ((got - want).norm() / want.norm()).item() < 7e-7
+
+
+def test_more_than_two_to_the_31_steps():
+    """A batch whose steps, let alone its values, no 32-bit number counts, in place (34 GB): the first and the last sequences, some around
+    the 2^31st value and the 2^31st step from the end."""
+    import paper_2002_03629_b200.rnn as rnn
+    T, H = 128, 4
+    B = 2 ** 31 // T + 300
+    if torch.cuda.mem_get_info()[0] < 40 << 30:
+        pytest.skip("needs 40 GB of device memory")
+    g = torch.Generator("cuda").manual_seed(31)
+    W = torch.randn((H, H), generator=g, device="cuda") * 0.1
+    l = torch.empty((B, T, H), device="cuda").uniform_(0.25, 1.0, generator=g)       # the derivatives too: both are only read
+    some = sorted({b for c in (0, 150, 300, B // 4, B // 2, B - 1) for b in range(c - 3, c + 4) if 0 <= b < B})
+    before = l[some].clone()
+    got = rnn.rnn_bptt_jacobi(W, l, l, 5, out=l)[some]
+    want = reference(W, before, before, 5)
+    assert ((got.double() - want).norm(dim=(1, 2)) / want.norm(dim=(1, 2))).max().item() < 7e-7
