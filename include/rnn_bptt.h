@@ -21,6 +21,10 @@
  * the parameter gradients of more than 24 steps, products of three-piece bf16 expansions (24 bits, over the whole range of fp32) summed in fp32 on the tensor
  * cores, also in a fixed order (results are reproducible run to run); what leaves the expansions' upper end, states beyond 1e24 or
  * factors beyond 2e31, infinities and NaN among them, is computed again by multiply-adds, at a fraction of the speed; exp/log from the fast-math intrinsics are not used.
+ *
+ * Time-outs.  The kernels of the Jacobi iterations and of the parameter gradients wait for their own copies and tensor-core products, 2 s at
+ * most.  A wait that gives up ends its thread block's work: the outputs of that block's remaining sequences are NaN, and the context stays
+ * usable.  The call has returned RNN_OK long before; the `_bounded` forms below tell the caller on the device.
  */
 #ifndef RNN_BPTT_H
 #define RNN_BPTT_H
@@ -32,6 +36,7 @@ extern "C" {
 #define RNN_OK 0
 #define RNN_ERR_INVALID (-1)
 #define RNN_ERR_CUDA (-2)
+#define RNN_ERR_TIMEOUT (-3)
 #define RNN_MAX_T 128
 #define RNN_MAX_H 128
 #define RNN_MAX_IO 16
@@ -57,6 +62,14 @@ int rnn_bptt_jacobi(const float *Wh, const float *l, const float *d, int B, int 
  *   dWh [B][H][H] = sum_{t>=2} g_t h_{t-1}^T,  dWx [B][H][d_in] = sum_t g_t x_t^T,  db [B][H] = sum_t g_t. */
 int rnn_param_grads(const float *s, const float *d, const float *h, const float *x, int B, int T, int H, int d_in,
                     float *dWh, float *dWx, float *db, void *stream);
+
+/* The same two calls with `wait_ns` in place of the 2 s (0: a wait that does not find its data at the first look gives up) and a word that
+ * tells the caller whether one gave up: *status (device or mapped host memory; NULL: not wanted) is set to RNN_ERR_TIMEOUT in that case and
+ * not touched otherwise.  It can be read when the work on `stream` is done. */
+int rnn_bptt_jacobi_bounded(const float *Wh, const float *l, const float *d, int B, int T, int H, int n_iters, const float *s0,
+                            float *s, unsigned long long wait_ns, int *status, void *stream);
+int rnn_param_grads_bounded(const float *s, const float *d, const float *h, const float *x, int B, int T, int H, int d_in,
+                            float *dWh, float *dWx, float *db, unsigned long long wait_ns, int *status, void *stream);
 
 /* Text of the last CUDA error seen by these calls in this process ("" if none). */
 const char *rnn_last_error(void);

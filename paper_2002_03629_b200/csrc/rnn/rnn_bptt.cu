@@ -467,17 +467,31 @@ __device__ __forceinline__ void cut3(float a, float b, uint32_t &h, uint32_t &m,
     b -= __uint_as_float(m & 0xffff0000u);
     l = pack_bf16x2(a, b);
 }
-// bounded: true once the barrier's phase has completed, false after 2 s or when another wait of the CTA has given up
-__device__ __forceinline__ bool jac_wait(int &dead, uint64_t *bar, uint32_t parity)
+// The waits of a call: how long one may take, and where the caller wants to read that one gave up (or NULL).
+struct Waits {
+    unsigned long long ns;
+    int *status;
+};
+// bounded: true once the barrier's phase has completed, false when the time is over (0: at once) or another wait of the CTA has given up
+__device__ __forceinline__ bool jac_wait(int &dead, uint64_t *bar, uint32_t parity, const Waits &w)
 {
-    if (mbar_try_wait(bar, parity)) return true;
-    const uint64_t t0 = global_ns();
-    for (unsigned i = 1;; ++i) {
-        if (mbar_try_wait(bar, parity)) return true;
-        if ((i & 63u) == 0u && (*(volatile int *)&dead || global_ns() - t0 > MBAR_WAIT_NS)) break;
+    if (w.ns == 0 ? mbar_test_wait(bar, parity) : mbar_try_wait(bar, parity)) return true;
+    if (w.ns != 0) {
+        const uint64_t t0 = global_ns();
+        for (unsigned i = 1;; ++i) {
+            if (mbar_try_wait(bar, parity)) return true;
+            if ((i & 63u) == 0u && (*(volatile int *)&dead || global_ns() - t0 > w.ns)) break;
+        }
     }
     *(volatile int *)&dead = 1;
     return false;
+}
+// The end of a CTA in which a wait gave up (all threads, behind a barrier): the caller is told, and shared and tensor memory are kept until
+// the copies and MMAs that are on their way, microseconds' worth, have ended.
+__device__ __noinline__ void gave_up(const Waits &w)
+{
+    if (threadIdx.x == 0 && w.status != nullptr) *(volatile int *)w.status = RNN_ERR_TIMEOUT;
+    for (int i = 0; i < 2000; ++i) __nanosleep(1000);
 }
 // barrier of the epilogue warps: did every thread say yes?
 __device__ __forceinline__ bool jac_all(bool ok)
@@ -519,7 +533,7 @@ __device__ __forceinline__ void jac_plain(const float *Wh, const float *l, const
 template <int JC, bool MANY>
 __global__ void __launch_bounds__(JTH, 1)
 rnn_bptt_jacobi_kernel(const float *__restrict__ Wh, const float *l, const float *d, int B, int T, int H, int iters, const float *s0, float *s,
-                       int per_unit)
+                       int per_unit, const Waits waits)
 {
     extern __shared__ uint8_t smem_raw[];
     __shared__ JacShared sh;
@@ -602,7 +616,7 @@ rnn_bptt_jacobi_kernel(const float *__restrict__ Wh, const float *l, const float
                 bool on = true;
                 for (int u = blockIdx.x; u < units && on; u += gridDim.x)
                     for (int it = 0; it < nmma && on; ++it, par ^= 1u) {
-                        on = __all_sync(0xffffffffu, jac_wait(sh.dead, &sh.ready[slot], par));
+                        on = __all_sync(0xffffffffu, jac_wait(sh.dead, &sh.ready[slot], par, waits));
                         if (!on) break;
                         tc_fence_after();
                         if (elect_one()) {
@@ -633,8 +647,8 @@ rnn_bptt_jacobi_kernel(const float *__restrict__ Wh, const float *l, const float
         for (int u = blockIdx.x; u < units; u += gridDim.x) {
             const int cols = unit_columns(u);
             const size_t base = (size_t)u * per_unit * T * H + i;
-            bool ok = true;
-            if (stages) ok = jac_wait(sh.dead, &sh.staged, staged_par);
+            bool ok = *(volatile int *)&sh.dead == 0;                        // (a wait that gave up ends the CTA's work)
+            if (ok && stages) ok = jac_wait(sh.dead, &sh.staged, staged_par, waits);
             staged_par ^= 1u;
             const float *lp = stages ? ls + i : l + base, *dp = stages ? ds + i : d + base;
             float lv[2][JC], dv[2][JC], l0 = 0.0f;
@@ -671,7 +685,7 @@ rnn_bptt_jacobi_kernel(const float *__restrict__ Wh, const float *l, const float
             }
             if (g == 0 && i < H) l0 = lp[0];
             ok = jac_all(ok);                                                // everything has been read
-            if (tid == 0) stage(u + (int)gridDim.x);
+            if (tid == 0 && ok) stage(u + (int)gridDim.x);
             const bool idle = (i & ~31) >= H;                                // no component of this warp's (and no k that the MMAs read)
             // eight columns of the operand of slot k from their states: pieces of U = d s (d as large as they want it)
             auto put8 = [&](int k, int j0, const float (&v)[8]) {
@@ -780,7 +794,7 @@ rnn_bptt_jacobi_kernel(const float *__restrict__ Wh, const float *l, const float
 #pragma unroll
                 for (int k = 1; k >= 0; --k) {
                     if (k == 1 && !two) continue;
-                    ok = __all_sync(0xffffffffu, jac_wait(sh.dead, &sh.full[k], par));
+                    ok = __all_sync(0xffffffffu, jac_wait(sh.dead, &sh.full[k], par, waits));
                     if (!ok) break;
                     tc_fence_after();
                     finish(k, last);
@@ -796,7 +810,7 @@ rnn_bptt_jacobi_kernel(const float *__restrict__ Wh, const float *l, const float
             const bool plain = !jac_all(chk == 0.0f);
             ok = jac_all(ok);
             if (!ok) {
-                // the MMAs did not end: nothing is known about the states
+                // the operands did not come or the MMAs did not end: nothing is known about the states
                 for (int c = g; c < cols; c += G)
                     if (i < H) s[base + (size_t)c * H] = NAN;
             } else if (plain) {
@@ -814,6 +828,7 @@ rnn_bptt_jacobi_kernel(const float *__restrict__ Wh, const float *l, const float
     __syncwarp();
     tc_fence_before();
     __syncthreads();
+    if (sh.dead != 0) gave_up(waits);
     if (warp == 8) {
         tc_fence_after();
         tmem_dealloc(tm, 512);
@@ -845,7 +860,7 @@ template <bool VEC, int NX>
 __global__ void __launch_bounds__(PGT, 2)
 rnn_param_grads_kernel(const float *__restrict__ s, const float *__restrict__ d, const float *__restrict__ h,
                        const float *__restrict__ x, int T, int H, int d_in, int cols, float *__restrict__ dWh,
-                       float *__restrict__ dWx, float *__restrict__ db)
+                       float *__restrict__ dWx, float *__restrict__ db, const Waits waits)
 {
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t done;
@@ -885,7 +900,7 @@ rnn_param_grads_kernel(const float *__restrict__ s, const float *__restrict__ d,
     uint32_t par = 0;
     for (int t0 = 0; t0 < T; t0 += PK, par ^= 1u) {
         if (t0 > 0) {                                    // the steps before have been multiplied
-            ok = jac_wait(dead, &done, par ^ 1u);
+            ok = jac_wait(dead, &done, par ^ 1u, waits);
             if (!__syncthreads_and(ok)) { ok = false; break; }
         }
         const int rows = (min(PK, T - t0) + 15) / 16 * 16;
@@ -940,7 +955,7 @@ rnn_param_grads_kernel(const float *__restrict__ s, const float *__restrict__ d,
         }
         __syncwarp();
     }
-    if (ok) ok = jac_wait(dead, &done, par ^ 1u);
+    if (ok) ok = jac_wait(dead, &done, par ^ 1u, waits);
     ok = __syncthreads_and(ok) != 0;
     tc_fence_after();
     float *out = dWh + (size_t)seq * H * H;
@@ -1005,6 +1020,7 @@ rnn_param_grads_kernel(const float *__restrict__ s, const float *__restrict__ d,
     }
     tc_fence_before();
     __syncthreads();
+    if (dead != 0) gave_up(waits);
     if (warp == 0) {
         tc_fence_after();
         tmem_dealloc(tm, 256);
@@ -1181,8 +1197,8 @@ int rnn_bptt_sequential(const float *Wh, const float *l, const float *d, int B, 
     return launch_status();
 }
 
-int rnn_bptt_jacobi(const float *Wh, const float *l, const float *d, int B, int T, int H, int n_iters, const float *s0,
-                    float *s, void *stream)
+int rnn_bptt_jacobi_bounded(const float *Wh, const float *l, const float *d, int B, int T, int H, int n_iters, const float *s0,
+                            float *s, unsigned long long wait_ns, int *status, void *stream)
 {
     if (!Wh || !l || !d || !s || !sizes_ok(B, T, H) || n_iters < 0) return RNN_ERR_INVALID;
     const int sms = sm_count();
@@ -1198,12 +1214,18 @@ int rnn_bptt_jacobi(const float *Wh, const float *l, const float *d, int B, int 
     if (!allow_smem(kernel, 1024 + J_OPS + (size_t)2 * MT * MH * sizeof(float), (H > 64) + 2 * (per_unit > 1))) return RNN_ERR_CUDA;
     const size_t smem = 1024 + J_OPS + (size_t)2 * per_unit * T * H * sizeof(float);
     kernel<<<std::min(sms, (B - 1) / per_unit + 1), JTH, smem, (cudaStream_t)stream>>>(
-        Wh, l, d, B, T, H, std::min(n_iters, T), s0, s, per_unit);
+        Wh, l, d, B, T, H, std::min(n_iters, T), s0, s, per_unit, Waits{wait_ns, status});
     return launch_status();
 }
 
-int rnn_param_grads(const float *s, const float *d, const float *h, const float *x, int B, int T, int H, int d_in,
-                    float *dWh, float *dWx, float *db, void *stream)
+int rnn_bptt_jacobi(const float *Wh, const float *l, const float *d, int B, int T, int H, int n_iters, const float *s0,
+                    float *s, void *stream)
+{
+    return rnn_bptt_jacobi_bounded(Wh, l, d, B, T, H, n_iters, s0, s, MBAR_WAIT_NS, nullptr, stream);
+}
+
+int rnn_param_grads_bounded(const float *s, const float *d, const float *h, const float *x, int B, int T, int H, int d_in,
+                            float *dWh, float *dWx, float *db, unsigned long long wait_ns, int *status, void *stream)
 {
     if (!s || !d || !h || !x || !dWh || !dWx || !db || !sizes_ok(B, T, H) || d_in < 1 || d_in > MIO) return RNN_ERR_INVALID;
     const bool vec = vectors(s, d, h, dWh);
@@ -1220,8 +1242,14 @@ int rnn_param_grads(const float *s, const float *d, const float *h, const float 
     const int sms = sm_count(), all = (H + 31) / 32 * 32;
     const int cols = B >= sms ? all : B >= sms / 2 ? std::min(all, MH / 2) : std::min(all, MH / 4);
     if (!allow_smem(kernel, P_SMEM, vec + 2 * (d_in <= 4))) return RNN_ERR_CUDA;
-    kernel<<<dim3(B, (H + cols - 1) / cols), PGT, P_SMEM, (cudaStream_t)stream>>>(s, d, h, x, T, H, d_in, cols, dWh, dWx, db);
+    kernel<<<dim3(B, (H + cols - 1) / cols), PGT, P_SMEM, (cudaStream_t)stream>>>(s, d, h, x, T, H, d_in, cols, dWh, dWx, db, Waits{wait_ns, status});
     return launch_status();
+}
+
+int rnn_param_grads(const float *s, const float *d, const float *h, const float *x, int B, int T, int H, int d_in,
+                    float *dWh, float *dWx, float *db, void *stream)
+{
+    return rnn_param_grads_bounded(s, d, h, x, B, T, H, d_in, dWh, dWx, db, MBAR_WAIT_NS, nullptr, stream);
 }
 
 const char *rnn_last_error(void) { return g_err; }

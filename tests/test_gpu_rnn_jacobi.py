@@ -174,3 +174,28 @@ def test_more_than_two_to_the_31_steps():
     got = rnn.rnn_bptt_jacobi(W, l, l, 5, out=l)[some]
     want = reference(W, before, before, 5)
     assert ((got.double() - want).norm(dim=(1, 2)) / want.norm(dim=(1, 2))).max().item() < 7e-7
+
+
+@pytest.mark.parametrize("B,T,H", [(1, 30, 8), (3, 100, 128), (400, 70, 64), (900, 30, 20)])
+def test_waits_that_give_up(B, T, H):
+    """Without any patience every block gives up at its first wait: all outputs are NaN, the status says why, and the calls that follow
+    find shared and tensor memory as they need them.  With the usual patience the status stays as it was."""
+    import paper_2002_03629_b200.rnn as rnn
+    W, l, d, h = draw(B, T, H)
+    x = torch.rand((B, T, 2), device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    s = rnn.rnn_bptt_jacobi(W, l, d, 5, status=status)
+    grads = rnn.rnn_param_grads(s, d, h, x, status=status)
+    assert int(status) == 0
+    for _ in range(3):
+        status.zero_()
+        assert torch.isnan(rnn.rnn_bptt_jacobi(W, l, d, 5, status=status, wait_ns=0)).all() and int(status) == rnn.RNN_ERR_TIMEOUT
+        status.zero_()
+        for g in rnn.rnn_param_grads(s, d, h, x, status=status, wait_ns=0):
+            assert torch.isnan(g).all()
+        assert int(status) == rnn.RNN_ERR_TIMEOUT
+        rnn.rnn_bptt_jacobi(W, l, d, 5, wait_ns=0)
+        status.fill_(7)
+        assert torch.equal(rnn.rnn_bptt_jacobi(W, l, d, 5, status=status), s)
+        assert all(torch.equal(a, b) for a, b in zip(rnn.rnn_param_grads(s, d, h, x, status=status), grads))
+        assert int(status) == 7
