@@ -186,7 +186,7 @@ int common_scratch(js_model *m, int T)
     CU_TRY(cudaHostGetDevicePointer((void **)&m->d_result, m->h_result, 0));
     CU_TRY(cudaHostAlloc((void **)&m->h_words, 2 * sizeof(unsigned long long) * JS_MAX_CLUSTERS, cudaHostAllocMapped));
     CU_TRY(cudaHostGetDevicePointer((void **)&m->d_words, m->h_words, 0));
-    if ((rc = dev_alloc<int>(m, &m->smp_changed, 2 * (size_t)m->rows, true)) != JS_OK) return rc;
+    if ((rc = dev_alloc<int>(m, &m->smp_changed, JS_FLAG_SLOTS * (size_t)m->rows, true)) != JS_OK) return rc;
     if ((rc = dev_alloc<int>(m, &m->smp_state, 2 * (size_t)m->rows, true)) != JS_OK) return rc;
     if ((rc = dev_alloc<int>(m, &m->perm, 2 * (size_t)m->rows, true)) != JS_OK) return rc;
     if ((rc = dev_alloc<uint8_t>(m, &m->x_old, (size_t)m->rows * T, true)) != JS_OK) return rc;

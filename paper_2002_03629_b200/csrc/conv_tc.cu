@@ -135,15 +135,9 @@ struct ConvEngine {
             a0[pix * 64 + (i % m.in_ch)] = __float2bfloat16_rn(m.lut[v]);
         }
         if (blockIdx.x == 0) {
-            for (int i = threadIdx.x; i < 2 * r.batch; i += blockDim.x) {
-                r.smp_changed[i] = 0;
-                r.smp_state[i] = 0;
-            }
+            clear_flags(r);
+            for (int i = threadIdx.x; i < 2 * r.batch; i += blockDim.x) r.smp_state[i] = 0;
             for (int i = threadIdx.x; i < r.batch * m.nyt * 8; i += blockDim.x) m.stamp[i] = 0;
-            if (threadIdx.x == 0) {
-                r.ctl->agg_any[0] = r.ctl->agg_any[1] = 0;
-                r.ctl->agg_minfirst[0] = r.ctl->agg_minfirst[1] = INT_MAX;
-            }
         }
         for (int i = threadIdx.x; i < r.batch; i += blockDim.x) sh.img[icur][i] = i;
         if (threadIdx.x == 0) sh.n_img[icur] = r.batch;
@@ -155,7 +149,7 @@ struct ConvEngine {
     // move, so nothing has to be rebuilt.  The list is made by one warp while another one asks what changed at all (the two
     // round trips to L2 and a block barrier one after the other cost 1 us per pass): the flags of all images in flight at
     // once, then a ballot per 32 images.
-    __device__ void look_ahead(int parity)
+    __device__ void look_ahead(int fslot)
     {
         if (warp != 1) return;
         const int n = sh.n_img[icur];
@@ -165,7 +159,7 @@ struct ConvEngine {
         for (int i = 0; i < MAX_IMAGES / 32; ++i) {
             const bool in = 32 * i + lane < n;
             img[i] = in ? sh.img[icur][32 * i + lane] : 0;
-            keep[i] = in && ld_volatile_i32(&r.smp_changed[parity * r.batch + img[i]]) != 0;
+            keep[i] = in && ld_volatile_i32(&r.smp_changed[fslot * r.batch + img[i]]) != 0;
         }
         int k = 0;
 #pragma unroll
@@ -538,7 +532,7 @@ struct ConvEngine {
         return bi;
     }
 
-    __device__ void epilogue(int l, int kind, const Win &w, bool flag, int parity, float *zout, int yt_lo, int nyl,
+    __device__ void epilogue(int l, int kind, const Win &w, bool flag, int fslot, float *zout, int yt_lo, int nyl,
                              int ntiles, int src)
     {
         const bool head = (l == m.n_conv);
@@ -654,7 +648,7 @@ struct ConvEngine {
                     // plain store (a load to look first would be an L2 round trip per tile), and only
                     // once per image and phase
                     if (__any_sync(0xffffffffu, ch) && (raised_img != n || raised_phase != phase_no)) {
-                        if (lane == 0) r.smp_changed[parity * r.batch + n] = 1;
+                        if (lane == 0) r.smp_changed[fslot * r.batch + n] = 1;
                         raised_img = n;
                         raised_phase = phase_no;
                     }
@@ -676,14 +670,14 @@ struct ConvEngine {
             if (wany) {
                 const int wmin = __reduce_min_sync(0xffffffffu, first);
                 if (lane == 0) {
-                    atomicMin(&r.ctl->agg_minfirst[parity], wmin);
-                    atomicOr(&r.ctl->agg_any[parity], 1);
+                    atomicMin(&r.ctl->agg_minfirst[fslot], wmin);
+                    atomicOr(&r.ctl->agg_any[fslot], 1);
                 }
             }
         }
     }
 
-    __device__ void layer_phase(int l, int kind, const Win &w, bool flag, int parity, float *zout, int src = SRC_NEW)
+    __device__ void layer_phase(int l, int kind, const Win &w, bool flag, int fslot, float *zout, int src = SRC_NEW)
     {
         const bool head = (l == m.n_conv);
         int yt_lo, yt_hi;
@@ -716,19 +710,19 @@ struct ConvEngine {
                 load_noise(yt_lo, nyl, ntiles);
             }
         } else {
-            epilogue(l, kind, w, flag, parity, zout, yt_lo, nyl, ntiles, src);
+            epilogue(l, kind, w, flag, fslot, zout, yt_lo, nyl, ntiles, src);
         }
     }
 
     // One pass.  Inside it the tiles wait for one another by their stamps; the grid barrier at its end lets the next pass
     // overwrite what this one read, and makes the flags complete.
-    __device__ bool step(const Win &w, bool flag, int parity, float *zout, int src = SRC_NEW)
+    __device__ bool step(const Win &w, bool flag, int fslot, float *zout, int src = SRC_NEW)
     {
         conv_lo = conv_hi = 0;
         const int l_end = src == SRC_OLD ? m.n_conv - 1 : m.n_conv;      // the old set needs no head
         for (int l = 0; l <= l_end; ++l) {
             const bool last = (l == m.n_conv);
-            layer_phase(l, last ? (zout ? EPI_LOGITS : EPI_CAT) : EPI_HIDDEN, w, last && flag, parity, zout, src);
+            layer_phase(l, last ? (zout ? EPI_LOGITS : EPI_CAT) : EPI_HIDDEN, w, last && flag, fslot, zout, src);
         }
         return barrier();
     }
@@ -740,8 +734,8 @@ struct ConvEngine {
     // forward passes in which every layer reads the row above from the activations of x^{k-1} and its
     // own row from the working activations.  So: the hidden layers once on x^{k-1} (the "old" set),
     // then mixed passes until no symbol changes, then the comparison with x^{k-1} for the outer flags,
-    // which are left in the flag slot `parity`.
-    __device__ bool jgs_outer(int parity, int, int, int &iterations)
+    // which are left in the flag slot `fslot`.
+    __device__ bool jgs_outer(int fslot, int, int, int &iterations)
     {
         const size_t n = (size_t)r.batch * m.T;
         const size_t npix64 = (size_t)r.batch * m.height * m.width * 64 / 8;       // uint4 units of the padded image
@@ -754,39 +748,27 @@ struct ConvEngine {
                 dst[i] = src[i];
         }
         if (!barrier()) return false;
-        // every CTA has read the previous outer iteration's flags by now: both slots start clean
-        if (blockIdx.x == 0) {
-            for (int i = threadIdx.x; i < 2 * r.batch; i += blockDim.x) r.smp_changed[i] = 0;
-            if (threadIdx.x == 0) {
-                r.ctl->agg_any[0] = r.ctl->agg_any[1] = 0;
-                r.ctl->agg_minfirst[0] = r.ctl->agg_minfirst[1] = INT_MAX;
-            }
-        }
+        // every CTA has read the previous outer iteration's flags by now: all slots start clean
+        if (blockIdx.x == 0) clear_flags(r);
         const Win w = make_win(0, m.T, 0, m.T);
         if (!step(w, false, 0, nullptr, SRC_OLD)) return false;
         iterations++;
         const int cap = m.width * m.in_ch;
-        int q = parity;
+        int q = fslot;
         for (int k = 1; k <= cap; ++k) {
-            q ^= 1;
+            q = next_slot(q);
             if (!step(w, true, q, nullptr, SRC_MIXED)) return false;
             iterations++;
             const int any = ld_volatile_i32(&r.ctl->agg_any[q]);
-            reset_other_parity(r, q);
+            clear_old_slot(r, q);
             if (!barrier()) return false;
             if (!any) break;
         }
-        // both flag slots start clean, then the outer comparison fills slot `parity`
-        if (blockIdx.x == 0) {
-            for (int i = threadIdx.x; i < 2 * r.batch; i += blockDim.x) r.smp_changed[i] = 0;
-            if (threadIdx.x == 0) {
-                r.ctl->agg_any[0] = r.ctl->agg_any[1] = 0;
-                r.ctl->agg_minfirst[0] = r.ctl->agg_minfirst[1] = INT_MAX;
-            }
-        }
+        // all flag slots start clean, then the outer comparison fills slot `fslot`
+        if (blockIdx.x == 0) clear_flags(r);
         if (!barrier()) return false;
         for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-            if (r.x[i] != r.x_old[i]) note_change(r, parity, (int)(i / m.T), (int)(i % m.T));
+            if (r.x[i] != r.x_old[i]) note_change(r, fslot, (int)(i / m.T), (int)(i % m.T));
         return barrier();
     }
 };

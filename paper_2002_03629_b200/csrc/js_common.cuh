@@ -18,13 +18,15 @@
 enum { KM_JACOBI = 0, KM_SEQ = 1, KM_GS_JACOBI = 2, KM_JACOBI_GS = 3, KM_FORWARD = 4,
        KM_HIDDEN = 5 };      // KM_HIDDEN: hidden layers only, on the symbols x_in (activations for the sweeps)
 
+#define JS_FLAG_SLOTS 3   // sets of change flags, taken in turn by the iterations (see clear_old_slot in made_driver.cuh)
+
 // Control block in device memory, zeroed by the host before every launch.
 struct JsCtl {
     unsigned bar_count;     // grid barrier: monotonically increasing arrival counter; read together with `abort`
     int abort;              // set when a bounded wait gave up; every CTA then leaves
     int status;             // JS_OK / JS_NOT_CONVERGED / JS_ERR_TIMEOUT
-    int agg_any[2];         // per iteration parity: did any sample change
-    int agg_minfirst[2];    // per iteration parity: smallest changed position
+    int agg_any[JS_FLAG_SLOTS];         // per flag slot: did any sample change
+    int agg_minfirst[JS_FLAG_SLOTS];    // per flag slot: smallest changed position
     int iterations;         // forward passes executed
     int frontier;           // leading positions known final at exit
     int iters_max;
@@ -66,7 +68,7 @@ struct RunArgs {
     uint8_t *x;               // working iterate = output samples [batch][T]
     uint8_t *x_old;           // scratch [batch][T] (Jacobi-GS)
     int32_t *out_iters;       // may be NULL
-    int *smp_changed;         // [2][batch] per-sample change flags by iteration parity
+    int *smp_changed;         // [JS_FLAG_SLOTS][batch] per-sample change flags
     int *smp_state;           // [2][batch] per-sample bookkeeping (done flag, running count)
     const uint8_t *x_in;      // KM_FORWARD: symbols
     float *logits_out;        // KM_FORWARD: destination

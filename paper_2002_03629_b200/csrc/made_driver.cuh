@@ -28,24 +28,37 @@ __device__ __forceinline__ Win make_win(int hlo, int hhi, int plo, int phi)
     return w;
 }
 
-__device__ __forceinline__ void note_change(const RunArgs &r, int parity, int b, int d)
+__device__ __forceinline__ void note_change(const RunArgs &r, int slot, int b, int d)
 {
-    atomicOr(&r.smp_changed[parity * r.batch + b], 1);
-    atomicMin(&r.ctl->agg_minfirst[parity], d);
-    atomicOr(&r.ctl->agg_any[parity], 1);
+    atomicOr(&r.smp_changed[slot * r.batch + b], 1);
+    atomicMin(&r.ctl->agg_minfirst[slot], d);
+    atomicOr(&r.ctl->agg_any[slot], 1);
 }
 
 // The bookkeeping between two iterations falls to the last CTA of the grid.  Its loads take 1.5 us, for which the CTA comes late to the next
 // phase; the phase's first and longest units lie with the first CTAs, and often the last one has none.
 __device__ __forceinline__ bool keeps_books() { return blockIdx.x == gridDim.x - 1; }
 
-// After the barrier that ends an iteration: one CTA clears the other parity's flags.
-// Safe because every CTA read that parity before it passed at least one later
-// barrier, and nobody writes it again before at least one more barrier.
-__device__ __forceinline__ void reset_other_parity(const RunArgs &r, int parity)
+__device__ __forceinline__ int next_slot(int slot) { return slot == JS_FLAG_SLOTS - 1 ? 0 : slot + 1; }
+
+// All change flags, by one CTA.
+__device__ __forceinline__ void clear_flags(const RunArgs &r)
+{
+    for (int i = threadIdx.x; i < JS_FLAG_SLOTS * r.batch; i += blockDim.x) r.smp_changed[i] = 0;
+    if (threadIdx.x < JS_FLAG_SLOTS) {
+        r.ctl->agg_any[threadIdx.x] = 0;
+        r.ctl->agg_minfirst[threadIdx.x] = INT_MAX;
+    }
+}
+
+// After the barrier that ends the iteration with flag slot `slot`: one CTA clears the slot of the iteration before it, which is that of the
+// next iteration but one.  Every CTA had read it before it came to this barrier, and it is written again behind the next iteration's
+// barrier, to which this CTA comes when it has cleared.  (Of two slots the very next iteration would write the cleared one, and the
+// only barrier in between is one that a pass has where it computes hidden layers: not where they are all final, and not in convolutions.)
+__device__ __forceinline__ void clear_old_slot(const RunArgs &r, int slot)
 {
     if (!keeps_books()) return;
-    const int o = parity ^ 1;
+    const int o = next_slot(next_slot(slot));
     for (int i = threadIdx.x; i < r.batch; i += blockDim.x) r.smp_changed[o * r.batch + i] = 0;
     if (threadIdx.x == 0) {
         r.ctl->agg_any[o] = 0;
@@ -54,13 +67,13 @@ __device__ __forceinline__ void reset_other_parity(const RunArgs &r, int parity)
 }
 
 // One CTA: a sample whose iterate did not change (or that hit the cap) stops counting.
-__device__ __forceinline__ void book_samples(const RunArgs &r, int parity, int k, bool at_cap, bool add,
+__device__ __forceinline__ void book_samples(const RunArgs &r, int slot, int k, bool at_cap, bool add,
                                              bool final_write)
 {
     if (!keeps_books()) return;
     int *done = r.smp_state, *count = r.smp_state + r.batch;
     for (int b = threadIdx.x; b < r.batch; b += blockDim.x) {
-        if (!done[b] && (r.smp_changed[parity * r.batch + b] == 0 || at_cap)) {
+        if (!done[b] && (r.smp_changed[slot * r.batch + b] == 0 || at_cap)) {
             done[b] = 1;
             count[b] = add ? count[b] + k : k;
             if (final_write && r.out_iters) r.out_iters[b] = count[b];
@@ -71,12 +84,12 @@ __device__ __forceinline__ void book_samples(const RunArgs &r, int parity, int k
 
 // After the barrier that ends an iteration: did anything change, and the first position that did.  One thread asks:
 // when all of them did, a grid's loads of the two words queued at one L2 slice for over a microsecond.
-__device__ __forceinline__ void read_changes(const JsCtl *ctl, int parity, int &any, int &minfirst)
+__device__ __forceinline__ void read_changes(const JsCtl *ctl, int slot, int &any, int &minfirst)
 {
     __shared__ int flags[2];
     if (threadIdx.x == 0) {
-        flags[0] = ld_volatile_i32(&ctl->agg_any[parity]);
-        flags[1] = ld_volatile_i32(&ctl->agg_minfirst[parity]);
+        flags[0] = ld_volatile_i32(&ctl->agg_any[slot]);
+        flags[1] = ld_volatile_i32(&ctl->agg_minfirst[slot]);
     }
     __syncthreads();
     any = flags[0];
@@ -108,7 +121,7 @@ __device__ DriverResult made_driver(E &e, int T_, const RunArgs &r)
             const int cap = (r.max_iters > 0 && r.max_iters < M) ? r.max_iters : M;
             int fin_x = 0, fin_h = 0;
             for (int k = 1;; ++k) {
-                const int p = k & 1;
+                const int p = k % JS_FLAG_SLOTS;
                 if (!e.jgs_outer(p, r.frontier_skip ? fin_h : 0, r.frontier_skip ? fin_x / B : 0, res.iterations)) {
                     res.alive = false;
                     return res;
@@ -116,7 +129,7 @@ __device__ DriverResult made_driver(E &e, int T_, const RunArgs &r)
                 int any, mf;
                 read_changes(ctl, p, any, mf);
                 book_samples(r, p, k, k == cap, false, true);
-                reset_other_parity(r, p);
+                clear_old_slot(r, p);
                 fin_h = max(fin_h, fin_x);
                 // after outer iteration k the first k blocks are final (proof of Prop. 2)
                 fin_x = any ? max(min(k * B, T_), min(mf + 1, T_)) : T_;
@@ -145,7 +158,7 @@ __device__ DriverResult made_driver(E &e, int T_, const RunArgs &r)
     int a = 0;                     // start of the current block (GS-Jacobi) / position (sequential order)
     int lo = 0;                    // positions of the current block below lo are settled
     int k = 0;                     // iteration inside the current block
-    int tick = 0;                  // forward passes with change flags so far (parity of the flag buffers)
+    int tick = 0;                  // forward passes with change flags so far (they take the flag slots in turn)
     for (;;) {
         Win w;
         bool flag = false;
@@ -169,7 +182,7 @@ __device__ DriverResult made_driver(E &e, int T_, const RunArgs &r)
             w = r.frontier_skip ? make_win(fin_h, bend - 1 + (mode == KM_JACOBI), lo, bend)
                                 : make_win(0, T_, a, bend);
         }
-        const int p = tick & 1;
+        const int p = tick % JS_FLAG_SLOTS;
         if (!e.step(w, flag, p, zout)) { res.alive = false; return res; }
         res.iterations++;
 
@@ -183,7 +196,7 @@ __device__ DriverResult made_driver(E &e, int T_, const RunArgs &r)
         if (mode == KM_JACOBI && r.compact) e.look_ahead(p);      // for compact() below, beside the next line's round trip
         read_changes(ctl, p, any, mf);
         book_samples(r, p, k, k == cap, mode == KM_GS_JACOBI, mode == KM_JACOBI);
-        reset_other_parity(r, p);
+        clear_old_slot(r, p);
         fin_h = max(fin_h, min(fin_x, mode == KM_JACOBI ? T_ : bend - 1));
         lo = any ? max(lo + 1, min(mf + 1, bend)) : bend;
         fin_x = max(fin_x, lo);

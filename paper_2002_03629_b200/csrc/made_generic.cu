@@ -363,24 +363,24 @@ __device__ __forceinline__ size_t a0_at(const MadeDev &m, size_t i);
 struct OutArgs {
     float *zout;               // logits [batch][T*C], or NULL: sample
     bool flag;
-    int parity;
+    int fslot;
 };
 
 // Change flags of many positions: the per-sample word by a plain store, the batch-level words once per warp (an atomic per
 // changed position on two words for the whole batch took longer than the forward pass).
 struct Changes {
     int first = INT_MAX;
-    __device__ __forceinline__ void note(const RunArgs &r, int parity, int b, int d)
+    __device__ __forceinline__ void note(const RunArgs &r, int fslot, int b, int d)
     {
-        r.smp_changed[parity * r.batch + b] = 1;
+        r.smp_changed[fslot * r.batch + b] = 1;
         first = min(first, d);
     }
-    __device__ __forceinline__ void flush(const RunArgs &r, int parity)
+    __device__ __forceinline__ void flush(const RunArgs &r, int fslot)
     {
         const int f = __reduce_min_sync(0xffffffffu, first);
         if (f != INT_MAX && (threadIdx.x & 31) == 0) {
-            atomicMin(&r.ctl->agg_minfirst[parity], f);
-            atomicOr(&r.ctl->agg_any[parity], 1);
+            atomicMin(&r.ctl->agg_minfirst[fslot], f);
+            atomicOr(&r.ctl->agg_any[fslot], 1);
         }
         first = INT_MAX;
     }
@@ -479,19 +479,19 @@ __device__ void gemm_phase(Smem &s, Ring &rg, const MadeDev &m, const RunArgs &r
                     const float xn = fmaf(expf(scale), nz[i][j], pre);
                     r.xr[at] = xn;
                     ((T *)m.a[0])[a0_at(m, at)] = from_f32<T>(xn);
-                    if (oa.flag && !(fabsf(xn - xo[i][j]) <= r.eps)) chg.note(r, oa.parity, row, d);     // a NaN difference is a change
+                    if (oa.flag && !(fabsf(xn - xo[i][j]) <= r.eps)) chg.note(r, oa.fslot, row, d);     // a NaN difference is a change
                 } else {
                     const int xn = js_sample_binary(r.nk, pre, nz[i][j]);
                     if ((float)xn != xo[i][j]) {
                         r.x[at] = (uint8_t)xn;
                         ((T *)m.a[0])[a0_at(m, at)] = from_f32<T>(m.lut[xn]);
-                        if (oa.flag) chg.note(r, oa.parity, row, d);
+                        if (oa.flag) chg.note(r, oa.fslot, row, d);
                     }
                 }
             }
         }
     }
-    if (oa.flag && !loader) chg.flush(r, oa.parity);
+    if (oa.flag && !loader) chg.flush(r, oa.fslot);
 }
 
 // place in a[0] (rows of n[0] >= T values) of element i = sample * T + position
@@ -512,14 +512,8 @@ __device__ void init_phase(const MadeDev &m, const RunArgs &r, const uint8_t *sr
         a0[a0_at(m, i)] = from_f32<T>(m.lut[v]);
     }
     if (blockIdx.x == 0) {
-        for (int i = threadIdx.x; i < 2 * r.batch; i += blockDim.x) {
-            r.smp_changed[i] = 0;
-            r.smp_state[i] = 0;
-        }
-        if (threadIdx.x == 0) {
-            r.ctl->agg_any[0] = r.ctl->agg_any[1] = 0;
-            r.ctl->agg_minfirst[0] = r.ctl->agg_minfirst[1] = INT_MAX;
-        }
+        clear_flags(r);
+        for (int i = threadIdx.x; i < 2 * r.batch; i += blockDim.x) r.smp_state[i] = 0;
     }
 }
 
@@ -527,7 +521,7 @@ __device__ void init_phase(const MadeDev &m, const RunArgs &r, const uint8_t *sr
 // new symbol and its encoding: a warp per position.
 template <typename T>
 __device__ void sample_phase(const MadeDev &m, const RunArgs &r, const float *z, int plo, int phi, bool flag,
-                             int parity)
+                             int fslot)
 {
     const int T_ = m.T, C = m.C, np = phi - plo;
     T *a0 = (T *)m.a[0];
@@ -542,10 +536,10 @@ __device__ void sample_phase(const MadeDev &m, const RunArgs &r, const float *z,
         if (lane == 0 && bi != r.x[at]) {
             r.x[at] = (uint8_t)bi;
             a0[a0_at(m, at)] = from_f32<T>(m.lut[bi]);
-            if (flag) chg.note(r, parity, b, d);
+            if (flag) chg.note(r, fslot, b, d);
         }
     }
-    if (flag) chg.flush(r, parity);
+    if (flag) chg.flush(r, fslot);
 }
 
 // Continuous states: x = start values (or zeros), a[0] = x (rounded like any activation in a bf16 model).
@@ -560,14 +554,8 @@ __device__ void init_phase_real(const MadeDev &m, const RunArgs &r, const float 
         a0[a0_at(m, i)] = from_f32<T>(v);
     }
     if (blockIdx.x == 0) {
-        for (int i = threadIdx.x; i < 2 * r.batch; i += blockDim.x) {
-            r.smp_changed[i] = 0;
-            r.smp_state[i] = 0;
-        }
-        if (threadIdx.x == 0) {
-            r.ctl->agg_any[0] = r.ctl->agg_any[1] = 0;
-            r.ctl->agg_minfirst[0] = r.ctl->agg_minfirst[1] = INT_MAX;
-        }
+        clear_flags(r);
+        for (int i = threadIdx.x; i < 2 * r.batch; i += blockDim.x) r.smp_state[i] = 0;
     }
 }
 
@@ -694,19 +682,19 @@ __device__ void jgs_commit_phase(const MadeDev &m, const RunArgs &r, int j, int 
 // x_old = x and a_old[0] = a[0] (start of an outer iteration); or compare x with
 // x_old and raise change flags (end of an outer iteration).
 template <typename T>
-__device__ void jgs_copy_or_compare(const MadeDev &m, const RunArgs &r, bool compare, int parity)
+__device__ void jgs_copy_or_compare(const MadeDev &m, const RunArgs &r, bool compare, int fslot)
 {
     Changes chg;
     const size_t n = (size_t)r.batch * m.T;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         if (compare) {
-            if (r.x[i] != r.x_old[i]) chg.note(r, parity, (int)(i / m.T), (int)(i % m.T));
+            if (r.x[i] != r.x_old[i]) chg.note(r, fslot, (int)(i / m.T), (int)(i % m.T));
         } else {
             r.x_old[i] = r.x[i];
             ((T *)m.a_old[0])[a0_at(m, i)] = ((const T *)m.a[0])[a0_at(m, i)];
         }
     }
-    if (compare) chg.flush(r, parity);
+    if (compare) chg.flush(r, fslot);
 }
 
 // ------------------------------------------------------------------ engine
@@ -742,23 +730,23 @@ struct GenericEngine {
     // One forward pass over the window; then either the logits go to zout (teacher forcing) or positions [w.plo, w.phi) are
     // sampled and committed: in the output tiles themselves where a position has one logit or a location and a log-scale,
     // from the logits scratch where it has more.
-    __device__ bool step(const Win &w, bool flag, int parity, float *zout)
+    __device__ bool step(const Win &w, bool flag, int fslot, float *zout)
     {
         const bool fused = !zout && (m.C == 1 || r.real);
         for (int l = 0; l <= m.L; ++l) {
-            const OutArgs oa = {zout ? zout : fused ? (float *)nullptr : m.logits, fused && flag && l == m.L, parity};
+            const OutArgs oa = {zout ? zout : fused ? (float *)nullptr : m.logits, fused && flag && l == m.L, fslot};
             gemm_phase<T, JGS, SPLIT>(s, rg, m, r, l, (const T *)m.a[l], l < m.L ? (T *)m.a[l + 1] : (T *)nullptr, oa, w, issued, skipped);
             if (!barrier()) return false;
         }
         if (zout || fused) return true;
-        sample_phase<T>(m, r, m.logits, w.plo, w.phi, flag, parity);
+        sample_phase<T>(m, r, m.logits, w.plo, w.phi, flag, fslot);
         return barrier();
     }
     // one outer iteration of Algorithm 2
-    __device__ bool jgs_outer(int parity, int fin_h, int blk_lo, int &iterations)
+    __device__ bool jgs_outer(int fslot, int fin_h, int blk_lo, int &iterations)
     {
         const int B = r.block, T_ = m.T;
-        jgs_copy_or_compare<T>(m, r, false, parity);
+        jgs_copy_or_compare<T>(m, r, false, fslot);
         if (!barrier()) return false;
         // hidden activations of the previous outer iterate
         const Win w = make_win(fin_h, T_, T_, T_);
@@ -781,7 +769,7 @@ struct GenericEngine {
             }
             iterations++;
         }
-        jgs_copy_or_compare<T>(m, r, true, parity);
+        jgs_copy_or_compare<T>(m, r, true, fslot);
         return barrier();
     }
 };

@@ -157,30 +157,24 @@ struct TcEngine {
              i += (size_t)gridDim.x * blockDim.x)
             t.pflags[i] = 0u;
         if (blockIdx.x == 0) {
-            for (int i = threadIdx.x; i < 2 * r.batch; i += blockDim.x) {
-                r.smp_changed[i] = 0;
-                r.smp_state[i] = 0;
-            }
+            clear_flags(r);
+            for (int i = threadIdx.x; i < 2 * r.batch; i += blockDim.x) r.smp_state[i] = 0;
             for (int i = threadIdx.x; i < r.batch; i += blockDim.x) r.perm[i] = i;
-            if (threadIdx.x == 0) {
-                r.ctl->agg_any[0] = r.ctl->agg_any[1] = 0;
-                r.ctl->agg_minfirst[0] = r.ctl->agg_minfirst[1] = INT_MAX;
-            }
         }
     }
 
-    // Compaction of the working batch after an iteration of parity `parity`.  Every CTA computes
+    // Compaction of the working batch after an iteration with the flags of slot `slot`.  Every CTA computes
     // the same list (rows whose sample changed, in order) from the per-sample flags, so no exchange
     // is needed to agree on it.  It is adopted only when it frees at least one 128-row tile; then
     // the encoded iterate is rebuilt for the new rows and a grid barrier makes it visible.
     // Returns 1 if rows were remapped, 0 if not, -1 if the barrier gave up.
     __device__ void look_ahead(int) {}
-    __device__ int compact(int parity)
+    __device__ int compact(int slot)
     {
         if (live <= BM) return 0;         // one tile of rows: nothing to be had
         const int *pc = perm_cur();
         int *pn = r.perm + (size_t)(pcur ^ 1) * r.perm_stride;
-        const int *chg = r.smp_changed + (size_t)parity * r.batch;
+        const int *chg = r.smp_changed + (size_t)slot * r.batch;
         if (threadIdx.x == 0) sh.cbase = 0;
         __syncthreads();
         // four rows per thread and round, their loads in flight together
@@ -660,10 +654,10 @@ struct TcEngine {
     // of a thread that meets the same row in tile after tile.
     int raised_sample = -1;
     unsigned raised_stamp = 0;
-    __device__ void raise_flag(int parity, int sample)
+    __device__ void raise_flag(int fslot, int sample)
     {
         if (raised_sample == sample && raised_stamp == stamp) return;
-        r.smp_changed[parity * r.batch + sample] = 1;
+        r.smp_changed[fslot * r.batch + sample] = 1;
         raised_sample = sample;
         raised_stamp = stamp;
     }
@@ -730,7 +724,7 @@ struct TcEngine {
     // of this loop, which a single warp per scheduler runs)
     template <int NK>
     __device__ bool epi_binary_tile(const Win &w, int smp, int rw, int n0, int ncols, uint32_t tbase, bool flag,
-                                    int parity, bool &wany, int &wfirst)
+                                    int fslot, bool &wany, int &wfirst)
     {
         const float *bs = my_bias();
         uint8_t *nz = nz_row(), *xs = xs_row();
@@ -829,7 +823,7 @@ struct TcEngine {
             __syncwarp();
         }
         if (flag) {
-            if (changed) raise_flag(parity, smp);
+            if (changed) raise_flag(fslot, smp);
             if (__any_sync(0xffffffffu, changed)) {
                 wany = true;
                 wfirst = min(wfirst, __reduce_min_sync(0xffffffffu, first));
@@ -872,7 +866,7 @@ struct TcEngine {
         if (t.streams) bulk_load_hint(smem_u32(cat_row()), gg, 1024u, &sh.nzbar[warp - 2], l2_stream_policy());
         else bulk_load(smem_u32(cat_row()), gg, 1024u, &sh.nzbar[warp - 2]);
     }
-    __device__ bool epi_cat_tile(int sample, int row, int d, uint32_t tbase, const Win &w, bool flag, int parity,
+    __device__ bool epi_cat_tile(int sample, int row, int d, uint32_t tbase, const Win &w, bool flag, int fslot,
                                  bool &any_changed, int &first)
     {
         const float *bs = sh.bias_s[warp - 2];
@@ -935,7 +929,7 @@ struct TcEngine {
             ch = true;
         }
         if (flag && ch) {
-            raise_flag(parity, sample);
+            raise_flag(fslot, sample);
             any_changed = true;
             first = min(first, d);
         }
@@ -948,7 +942,7 @@ struct TcEngine {
     // maximum, the running sums (remembered at the chunk ends, which tells the chunk that holds the
     // answer), and once more for the class inside that chunk.  The running sum is carried in class
     // order with the same instructions in the second and third reading, so both see the same values.
-    __device__ bool epi_icdf_tile(int sample, int row, int d, uint32_t tbase, const Win &w, bool flag, int parity,
+    __device__ bool epi_icdf_tile(int sample, int row, int d, uint32_t tbase, const Win &w, bool flag, int fslot,
                                   bool &any_changed, int &first)
     {
         const float *bs = sh.bias_s[warp - 2];
@@ -1015,14 +1009,14 @@ struct TcEngine {
             ch = true;
         }
         if (flag && ch) {
-            raise_flag(parity, sample);
+            raise_flag(fslot, sample);
             any_changed = true;
             first = min(first, d);
         }
         return true;
     }
 
-    __device__ void epilogue(int l, int kind, const Win &w, bool flag, int parity, float *zout, int nt_lo,
+    __device__ void epilogue(int l, int kind, const Win &w, bool flag, int fslot, float *zout, int nt_lo,
                              int nt_hi, int MT)
     {
         const TcLayer &ly = t.lay[l];
@@ -1118,13 +1112,13 @@ struct TcEngine {
                 bool wany = false;
                 int wfirst = INT_MAX;
                 const bool fine = r.nk == JS_NOISE_LOGISTIC
-                    ? epi_binary_tile<JS_NOISE_LOGISTIC>(w, bsmp, row, n0 + half() * (BM / 2), bcols, tbase, flag, parity, wany, wfirst)
-                    : epi_binary_tile<JS_NOISE_UNIFORM_ICDF>(w, bsmp, row, n0 + half() * (BM / 2), bcols, tbase, flag, parity, wany, wfirst);
+                    ? epi_binary_tile<JS_NOISE_LOGISTIC>(w, bsmp, row, n0 + half() * (BM / 2), bcols, tbase, flag, fslot, wany, wfirst)
+                    : epi_binary_tile<JS_NOISE_UNIFORM_ICDF>(w, bsmp, row, n0 + half() * (BM / 2), bcols, tbase, flag, fslot, wany, wfirst);
                 if (!fine) { dead = true; break; }
                 if (wany) { any_changed = true; first = min(first, wfirst); }
             } else if (EH == 1 && kind == EPI_CAT) {
-                const bool fine = r.nk == JS_NOISE_GUMBEL ? epi_cat_tile(csmp, row, nt, tbase, w, flag, parity, any_changed, first)
-                                                          : epi_icdf_tile(csmp, row, nt, tbase, w, flag, parity, any_changed, first);
+                const bool fine = r.nk == JS_NOISE_GUMBEL ? epi_cat_tile(csmp, row, nt, tbase, w, flag, fslot, any_changed, first)
+                                                          : epi_icdf_tile(csmp, row, nt, tbase, w, flag, fslot, any_changed, first);
                 if (!fine) { dead = true; break; }
             } else {
                 for (int c0 = 0; c0 < ly.bn; c0 += 32) {
@@ -1150,15 +1144,15 @@ struct TcEngine {
             if (wany) {
                 const int wmin = __reduce_min_sync(0xffffffffu, first);
                 if (lane == 0) {
-                    atomicMin(&r.ctl->agg_minfirst[parity], wmin);
-                    atomicOr(&r.ctl->agg_any[parity], 1);
+                    atomicMin(&r.ctl->agg_minfirst[fslot], wmin);
+                    atomicOr(&r.ctl->agg_any[fslot], 1);
                 }
             }
         }
     }
 
     // one layer over the window; returns false when there was nothing to do (no barrier needed)
-    __device__ bool gemm_phase(int l, int kind, const Win &w, bool flag, int parity, float *zout)
+    __device__ bool gemm_phase(int l, int kind, const Win &w, bool flag, int fslot, float *zout)
     {
         const int nt_lo = sh.rng[l].x, nt_hi = sh.rng[l].y;
         const int MT = (live + BM - 1) / BM;
@@ -1172,14 +1166,14 @@ struct TcEngine {
         } else if (warp == 1) {
             mma_issuer(l, nt_lo, nt_hi, MT);
         } else {
-            epilogue(l, kind, w, flag, parity, zout, nt_lo, nt_hi, MT);
+            epilogue(l, kind, w, flag, fslot, zout, nt_lo, nt_hi, MT);
         }
         return true;
     }
 
     // one forward pass over the window: a single loop and a single call site, so that the whole
     // pipeline is instantiated once in the kernel
-    __device__ bool step(const Win &w, bool flag, int parity, float *zout)
+    __device__ bool step(const Win &w, bool flag, int fslot, float *zout)
     {
         const int out_kind = zout ? EPI_LOGITS : EH == 2 ? EPI_BINARY : EPI_CAT;
         // the live tiles of all layers, a warp each (searched behind every barrier they cost every phase half a microsecond)
@@ -1191,7 +1185,7 @@ struct TcEngine {
         __syncthreads();
         for (int l = 0; l <= m.L; ++l) {
             const bool last = (l == m.L);
-            const bool did = gemm_phase(l, last ? out_kind : EPI_HIDDEN, w, last && flag, parity, zout);
+            const bool did = gemm_phase(l, last ? out_kind : EPI_HIDDEN, w, last && flag, fslot, zout);
             if (did || last)
                 if (!barrier()) return false;
         }
