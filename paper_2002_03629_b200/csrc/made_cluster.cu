@@ -924,7 +924,7 @@ static int cluster_rows(const js_model *mo, int batch, int *n_stages)
     const ClusterDev &c = mo->cluster;
     const int want = std::min(64, ((batch + c.max_clusters - 1) / c.max_clusters + 7) / 8 * 8);
     for (int R = want; R >= 8; R -= 8)
-        for (int st = MAX_STAGES; st >= 4; st -= 2)            // (two rings of half as many)
+        for (int st = MAX_STAGES; st >= 4; st -= 2)            // (they are used in pairs)
             if (cluster_smem(c, mo->made, R, st) <= SMEM_MAX) {
                 *n_stages = st;
                 return R;
@@ -945,9 +945,16 @@ bool js_cluster_serves(const js_model *mo, const RunArgs &r)
     // Two rounds: 784, 1024 x 2, 512 samples (47 K blocks, 8 stages) 126 and 167; 1024, 1536 x 2, 480 (91, 10) 180 and 202; 1444, 1444 x 2,
     // 300 (104, 8) 198 and 272; but 1024, 2048 x 2, 250 (136, 6) 231 and 202; 1600, 1024, 512 (55, 6) 233 and 221; 1936, 1500 x 2, 250 (138, 4)
     // 340 and 196.
+    // One round, but so many samples a cluster that the ring holds two loads (four stages): a pass waits for weights, and the grid-wide
+    // kernel, which pays by the layer, is the better one from 45 K blocks a layer on, if it moves whole rows (widths of 16 positions).  Jacobi, 128
+    // or 200 samples, here and there: 1296, 2048 x 2 (53 a layer) 264 and 232; 1024, 2240 x 2 (53) 215 and 193; 1936, 1500 x 2 (46) 261 and 237;
+    // but 1296, 1024, 1600, 1750 (35) 165 and 185; 1936, 576, 2000 (36) 193 and 214; rows of any length: 1156, 2048 x 2 (50) 247 and 283; 1444,
+    // 2240, 1650 (52) 254 and 277.  GS-Jacobi in four blocks gains with all of them (1296, 2048 x 2: 256 and 452).  Three loads: 1024, 2048 x 2 (45),
+    // 128 and 200 samples 121 and 160, 171 and 200; 1936, 2304 (75) 254 and 262.
     const int clusters = (r.batch + R - 1) / R, rounds = (clusters + mo->cluster.max_clusters - 1) / mo->cluster.max_clusters;
     if (clusters > JS_MAX_CLUSTERS) return false;
-    return rounds == 1 ? mo->cluster.kblocks <= 270 : rounds == 2 && mo->cluster.kblocks <= 104 && st >= 8;
+    const bool starved = st < 6 && r.kmode == KM_JACOBI && mo->tc.bin_bulk;
+    return rounds == 1 ? mo->cluster.kblocks <= (starved ? std::min(270, 45 * (mo->made.L + 1)) : 270) : rounds == 2 && mo->cluster.kblocks <= 104 && st >= 8;
 }
 
 int js_launch_made_cluster(const js_model *mo, const RunArgs &r, cudaStream_t stream, ClusterWork *work)
