@@ -1,6 +1,6 @@
 """The weight rings of the cluster kernel: models whose rings are short (many units or samples per cluster), tiles of one, two, odd and
 even numbers of K blocks, more than 32 tiles in a layer.  Weights arrive in any order (cold L2 on the first pass); every call has
-to give the same samples."""
+to give the samples of small batches."""
 import pytest
 import torch
 
@@ -22,18 +22,19 @@ def test_every_call_gives_the_same(T, H, batch):
     W, b = si.made_weights(cfg)
     model = p.Model.from_config(cfg, W, b, si.made_lut(cfg))
     noise = torch.from_numpy(si.draw_noise(cfg)).cuda()
-    ref = torch.empty((batch, T), dtype=torch.uint8, device="cuda")
-    assert p.sequential_sample(model, noise, cfg.noise_kind, ref) == 0
     flush = torch.empty(160 << 20, dtype=torch.uint8, device="cuda")
     for mode, block in ((p.JS_JACOBI, 0), (p.JS_GS_JACOBI, max(1, T // 4))):
-        first = None
+        # a few samples at a time, whose rings are long: a sample's sums do not depend on who shares its cluster
+        ref = torch.empty((batch, T), dtype=torch.uint8, device="cuda")
+        for lo in range(0, batch, 8):
+            hi = min(batch, lo + 8)
+            few = torch.empty((hi - lo, T), dtype=torch.uint8, device="cuda")
+            assert p.jacobi_sample(model, noise[lo:hi].clone(), cfg.noise_kind, None, mode, block, 0, few) == 0
+            ref[lo:hi] = few
         for _ in range(12):
             flush.zero_()
             out = torch.full((batch, T), 7, dtype=torch.uint8, device="cuda")
             assert p.jacobi_sample(model, noise, cfg.noise_kind, None, mode, block, 0, out) == 0
             assert model.stats().path == 0
-            first = out if first is None else first
-            assert torch.equal(out, first)
-        # (the sweep sums in another order: a hidden unit may round the other way, which moves a decision that nearly ties)
-        assert int((first == ref).all(1).sum()) >= batch - max(1, batch // 8)
+            assert torch.equal(out, ref)
     model.close()

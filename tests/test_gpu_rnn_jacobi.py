@@ -96,6 +96,11 @@ def test_parameter_gradients_against_64_bits(B, T, H, d_in):
     want = torch.einsum("bti,btj->bij", g[:, 1:], h.double()[:, :-1]), torch.einsum("bti,btc->bic", g, x.double()), g.sum(1)
     for a, b in zip(rnn.rnn_param_grads(s, d, h, x), want):
         assert ((a.double() - b).norm() / b.norm()).item() < 7e-7
+    # Factors of one sign, as a network's states are: the running sums are rounded towards zero, eight of them at most in an accumulator, each by
+    # less than 2^-23 of its value at that time, which grows evenly to the whole (4.5 / 8 of it on average): 5e-7.
+    g, hh = d.double() * s.abs().double(), h.abs()
+    want = torch.einsum("bti,btj->bij", g[:, 1:], hh.double()[:, :-1])
+    assert ((rnn.rnn_param_grads(s.abs(), d, hh, x)[0].double() - want).norm() / want.norm()).item() < 7e-7
     # a value that the pieces cannot carry: its sequence alone, the entries that it reaches alone
     s[0, T - 1, 1] = float("inf")
     h[0, 0, 2] = 3.39e38
