@@ -84,12 +84,6 @@ __device__ __forceinline__ void send16(uint32_t dst, uint4 v, uint32_t bar)
     asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
                  ::"r"(dst), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(bar) : "memory");
 }
-// Eight columns of a warp's sixteen accumulator lanes, over all its threads: lane i gets columns 2 (i % 4) and the next of rows
-// i / 4 (r[0], r[1]) and i / 4 + 8 (r[2], r[3]).
-__device__ __forceinline__ void tmem_ld_16x8(uint32_t taddr, uint32_t (&r)[4])
-{
-    asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(taddr) : "memory");
-}
 // two 8 x 8 blocks in that order of the threads, transposed: lane i (and i + 8) gives the address of the first (second) block's column i
 __device__ __forceinline__ void stmatrix2_trans(uint32_t addr, uint32_t a, uint32_t b)
 {

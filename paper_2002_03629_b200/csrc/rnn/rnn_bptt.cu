@@ -449,12 +449,6 @@ __device__ __forceinline__ void sts4(uint32_t at, const uint32_t (&r)[4])
 {
     asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
 }
-// Eight columns of sixteen accumulator lanes, over all threads of a warp: lane i gets columns 2 (i % 4) and the next of rows i / 4
-// (r[0], r[1]) and i / 4 + 8 (r[2], r[3]).
-__device__ __forceinline__ void tmem_ld_16x8(uint32_t taddr, uint32_t (&r)[4])
-{
-    asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(taddr) : "memory");
-}
 constexpr float PIECES_UP = 0x1p24f, SUMS_DOWN = 0x1p-48f;      // before the cut, after the products
 // two values in three bf16 pieces each, packed (the first in the low half)
 __device__ __forceinline__ void cut3(float a, float b, uint32_t &h, uint32_t &m, uint32_t &l)

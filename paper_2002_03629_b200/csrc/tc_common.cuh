@@ -258,6 +258,12 @@ __device__ __forceinline__ void umma_commit(uint64_t *bar)
                  : "memory");
 }
 
+// Eight columns of a warp's sixteen accumulator lanes, over all its threads: lane i gets columns 2 (i % 4) and the next of rows
+// i / 4 (r[0], r[1]) and i / 4 + 8 (r[2], r[3]).
+__device__ __forceinline__ void tmem_ld_16x8(uint32_t taddr, uint32_t (&r)[4])
+{
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(taddr) : "memory");
+}
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // issue the load of 32 consecutive fp32 columns of this thread's TMEM lane; the values may be
