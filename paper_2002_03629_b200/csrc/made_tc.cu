@@ -1443,7 +1443,9 @@ int js_tc_prepare(js_model *mo)
             // tile's partial sums have been stored.  Units are taken longest first and put where
             // the CTA finishes earliest.  Inside a CTA: partial chunks first (owners elsewhere
             // wait for them), then owners that wait for nobody, then owners that add partial sums.
-            // (EPI_ADD 4, 6, 8, 10: 312, 315, 318, 318 us for 4096 units a layer and 512 samples; the others make no difference.)
+            // (Costs in K blocks.  EPI_ADD 8 and 4, us a call, batches of 512: 4096, 4096 x 4 411 and 404; 3136, 8192, 4096 491 and 482; 5184, 5000
+            // 566 and 562; 3072, 4096 x 3 373 and 375; 3600, 3600 x 3 343 and 344 (384 samples); 4096, 2560 x 4 364 and 366 (640).  Other values of
+            // the others make no difference.)
             const int FILL = 6, EPI_PART = 5, EPI_OWN = (l == L ? (bn == 256 ? 5 : 9) : 4), EPI_ADD = 4;
             struct Item { int code, size, epi, ready; };
             std::vector<std::vector<Item>> lp(G), lo0(G), lo1(G);
