@@ -416,11 +416,22 @@ constexpr int J_PIECE = MH * J_SLOT * 2;     // bytes of one piece of a slot's o
 constexpr size_t J_OPS = 6 * J_PIECE;        // then l and d of a unit, [columns][H] each
 constexpr uint32_t J_DCOL = 3 * (MH / 2);    // tensor memory: three pieces of A, then per slot the two accumulators
 
+// The waits of a call: how long one may take, and where the caller wants to read that one gave up (or NULL).
+struct Waits {
+    unsigned long long ns;
+    int *status;
+};
+// What the waits of a CTA share.  (The patience lies in shared memory: as a kernel argument in every wait it cost the loops registers, 170 us
+// instead of 168 for 592 sequences of 100 steps and 20 iterations.)
+struct CtaWaits {
+    unsigned long long ns;
+    int dead;                                // a wait gave up
+};
 struct JacShared {
     uint64_t ready[2], full[2];              // the slot's operand is there; its products are
     uint32_t tmem;
     uint64_t staged;                         // the unit's l and d are in shared memory
-    int dead;                                // a wait gave up
+    CtaWaits waits;
 };
 
 // D[tmem] (+)= A[tmem] * B[smem], 128 x N x 16
@@ -462,23 +473,17 @@ __device__ __forceinline__ void cut3(float a, float b, uint32_t &h, uint32_t &m,
     b -= __uint_as_float(m & 0xffff0000u);
     l = pack_bf16x2(a, b);
 }
-// The waits of a call: how long one may take, and where the caller wants to read that one gave up (or NULL).
-struct Waits {
-    unsigned long long ns;
-    int *status;
-};
 // bounded: true once the barrier's phase has completed, false when the time is over (0: at once) or another wait of the CTA has given up
-__device__ __forceinline__ bool jac_wait(int &dead, uint64_t *bar, uint32_t parity, const Waits &w)
+__device__ __forceinline__ bool jac_wait(CtaWaits &w, uint64_t *bar, uint32_t parity)
 {
-    if (w.ns == 0 ? mbar_test_wait(bar, parity) : mbar_try_wait(bar, parity)) return true;
-    if (w.ns != 0) {
-        const uint64_t t0 = global_ns();
-        for (unsigned i = 1;; ++i) {
-            if (mbar_try_wait(bar, parity)) return true;
-            if ((i & 63u) == 0u && (*(volatile int *)&dead || global_ns() - t0 > w.ns)) break;
-        }
+    if (mbar_test_wait(bar, parity)) return true;
+    const uint64_t t0 = global_ns();
+    const unsigned long long ns = *(volatile unsigned long long *)&w.ns;
+    for (unsigned i = 1; ns != 0; ++i) {
+        if (mbar_try_wait(bar, parity)) return true;
+        if ((i & 63u) == 0u && (*(volatile int *)&w.dead || global_ns() - t0 > ns)) break;
     }
-    *(volatile int *)&dead = 1;
+    *(volatile int *)&w.dead = 1;
     return false;
 }
 // The end of a CTA in which a wait gave up (all threads, behind a barrier): the caller is told, and shared and tensor memory are kept until
@@ -558,7 +563,7 @@ rnn_bptt_jacobi_kernel(const float *__restrict__ Wh, const float *l, const float
     if (tid == 0) {
         for (int k = 0; k < 2; ++k) { mbar_init(&sh.ready[k], JE / 32); mbar_init(&sh.full[k], 1); }
         mbar_init(&sh.staged, 1);
-        sh.dead = 0;
+        sh.waits = CtaWaits{waits.ns, 0};
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         stage(blockIdx.x);
     }
@@ -611,7 +616,7 @@ rnn_bptt_jacobi_kernel(const float *__restrict__ Wh, const float *l, const float
                 bool on = true;
                 for (int u = blockIdx.x; u < units && on; u += gridDim.x)
                     for (int it = 0; it < nmma && on; ++it, par ^= 1u) {
-                        on = __all_sync(0xffffffffu, jac_wait(sh.dead, &sh.ready[slot], par, waits));
+                        on = __all_sync(0xffffffffu, jac_wait(sh.waits, &sh.ready[slot], par));
                         if (!on) break;
                         tc_fence_after();
                         if (elect_one()) {
@@ -642,8 +647,8 @@ rnn_bptt_jacobi_kernel(const float *__restrict__ Wh, const float *l, const float
         for (int u = blockIdx.x; u < units; u += gridDim.x) {
             const int cols = unit_columns(u);
             const size_t base = (size_t)u * per_unit * T * H + i;
-            bool ok = *(volatile int *)&sh.dead == 0;                        // (a wait that gave up ends the CTA's work)
-            if (ok && stages) ok = jac_wait(sh.dead, &sh.staged, staged_par, waits);
+            bool ok = *(volatile int *)&sh.waits.dead == 0;                        // (a wait that gave up ends the CTA's work)
+            if (ok && stages) ok = jac_wait(sh.waits, &sh.staged, staged_par);
             staged_par ^= 1u;
             const float *lp = stages ? ls + i : l + base, *dp = stages ? ds + i : d + base;
             float lv[2][JC], dv[2][JC], l0 = 0.0f;
@@ -789,7 +794,7 @@ rnn_bptt_jacobi_kernel(const float *__restrict__ Wh, const float *l, const float
 #pragma unroll
                 for (int k = 1; k >= 0; --k) {
                     if (k == 1 && !two) continue;
-                    ok = __all_sync(0xffffffffu, jac_wait(sh.dead, &sh.full[k], par, waits));
+                    ok = __all_sync(0xffffffffu, jac_wait(sh.waits, &sh.full[k], par));
                     if (!ok) break;
                     tc_fence_after();
                     finish(k, last);
@@ -823,7 +828,7 @@ rnn_bptt_jacobi_kernel(const float *__restrict__ Wh, const float *l, const float
     __syncwarp();
     tc_fence_before();
     __syncthreads();
-    if (sh.dead != 0) gave_up(waits);
+    if (sh.waits.dead != 0) gave_up(waits);
     if (warp == 8) {
         tc_fence_after();
         tmem_dealloc(tm, 512);
@@ -860,14 +865,14 @@ rnn_param_grads_kernel(const float *__restrict__ s, const float *__restrict__ d,
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t done;
     __shared__ uint32_t tmem;
-    __shared__ int dead;
+    __shared__ CtaWaits own;
     uint8_t *ops = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);    // pieces of g, then of h
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, seq = blockIdx.x, n0 = blockIdx.y * cols;
     const size_t base = (size_t)seq * T * H;
     const bool extra = blockIdx.y == 0;
     if (tid == 0) {
         mbar_init(&done, 1);
-        dead = 0;
+        own = CtaWaits{waits.ns, 0};
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) tmem_alloc(&tmem, 256);
@@ -895,7 +900,7 @@ rnn_param_grads_kernel(const float *__restrict__ s, const float *__restrict__ d,
     uint32_t par = 0;
     for (int t0 = 0; t0 < T; t0 += PK, par ^= 1u) {
         if (t0 > 0) {                                    // the steps before have been multiplied
-            ok = jac_wait(dead, &done, par ^ 1u, waits);
+            ok = jac_wait(own, &done, par ^ 1u);
             if (!__syncthreads_and(ok)) { ok = false; break; }
         }
         const int rows = (min(PK, T - t0) + 15) / 16 * 16;
@@ -950,7 +955,7 @@ rnn_param_grads_kernel(const float *__restrict__ s, const float *__restrict__ d,
         }
         __syncwarp();
     }
-    if (ok) ok = jac_wait(dead, &done, par ^ 1u, waits);
+    if (ok) ok = jac_wait(own, &done, par ^ 1u);
     ok = __syncthreads_and(ok) != 0;
     tc_fence_after();
     float *out = dWh + (size_t)seq * H * H;
@@ -1015,7 +1020,7 @@ rnn_param_grads_kernel(const float *__restrict__ s, const float *__restrict__ d,
     }
     tc_fence_before();
     __syncthreads();
-    if (dead != 0) gave_up(waits);
+    if (own.dead != 0) gave_up(waits);
     if (warp == 0) {
         tc_fence_after();
         tmem_dealloc(tm, 256);
