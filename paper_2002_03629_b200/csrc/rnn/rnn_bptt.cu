@@ -408,7 +408,7 @@ rnn_bptt_sequential_kernel(const float *__restrict__ Wh, const float *__restrict
 // states: such a unit is computed again with plain multiply-adds before anything of it is stored.
 // Bound: at 65 to 128 components the MMAs, 96 of 17 to 32 cycles an iteration (1.6 us of the 1.7 measured for 100 steps of 128
 // components; multiply-adds on the CUDA cores, 40 TFLOP/s, took 10); below that the way from a slot's last product to its next
-// first one (0.3 us of waits, 0.3 to 0.6 of epilogue).  T = 100, H = 128, 20 iterations: batch 1 71 -> 43 us, batch 592 894 -> 163 us;
+// first one (0.3 us of waits, 0.3 to 0.6 of epilogue).  T = 100, H = 128, 20 iterations: batch 1 71 -> 43 us, batch 592 894 -> 168 us;
 // T = 50, H = 64, 10 iterations, batch 300: 61 -> 28 us.  Against 64 bits the states are off by 1.0e-7 (2-norm), 1.1e-7 to 3.4e-7 before.
 constexpr int JE = 256, JTH = JE + 128;      // epilogue threads, all threads
 constexpr int J_SLOT = 64;                   // columns of a slot
