@@ -947,7 +947,9 @@ bool js_cluster_serves(const js_model *mo, const RunArgs &r)
     // 128 and 200 samples 121 and 160, 171 and 200; 1936, 2304 (75) 254 and 262.
     const int clusters = (r.batch + R - 1) / R, rounds = (clusters + mo->cluster.max_clusters - 1) / mo->cluster.max_clusters;
     if (clusters > JS_MAX_CLUSTERS) return false;
-    const bool starved = st < 6 && r.kmode == KM_JACOBI && mo->tc.bin_bulk;
+    // (Buffers on any float boundary stay here: the grid-wide kernel does not take them, and the CUDA-core kernel is no match.)
+    const bool aligned = (((uintptr_t)r.noise | (uintptr_t)r.x) & 15u) == 0;
+    const bool starved = st < 6 && r.kmode == KM_JACOBI && mo->tc.bin_bulk && aligned;
     return rounds == 1 ? mo->cluster.kblocks <= (starved ? std::min(270, 45 * (mo->made.L + 1)) : 270) : rounds == 2 && mo->cluster.kblocks <= 104 && st >= 8;
 }
 
